@@ -406,11 +406,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
     for (uint32_t t = tid; t < kc; t += NT) {
         float lo, hi;
         keys_to_range(s_kmn[t], s_kmx[t], lo, hi);
-        const QParam qp = make_qparam(lo, hi, a.qmax);
-        GroupParam gp;
-        gp.s = qp.s;
-        gp.z = qp.z;
-        gp.r = div_is_safe(qp.s, lo, hi) ? __frcp_rn(qp.s) : 0.0f;
+        const GroupParam gp = group_param_from_range(lo, hi, a.qmax);
         s_par[t] = gp;
         if (rank == 0) {
             a.lo[c0 + t] = lo;

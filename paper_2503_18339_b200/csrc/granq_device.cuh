@@ -251,34 +251,88 @@ __device__ __forceinline__ void run_add(WarpRun& r, bool valid, uint32_t g, uint
 }
 
 // ---------------------------------------------------------------------------------------
-// Per-group parameters from the published min / max keys, and the arithmetic of one pack.
+// Per-group parameters, and the arithmetic of one pack.
 // ---------------------------------------------------------------------------------------
 struct GroupParam {
     float s, z, r;   // scale, zero-point, RN(1 / s) or 0 when the group must use IEEE division
+    float thr;       // tie threshold of the single-multiply-add rounding below: positive where no element can be
+                     // clamped, negative where the clamp is needed, 0: the sequence as defined
 };
 
-__device__ __forceinline__ GroupParam group_param_from_keys(const uint32_t* kmin, const uint32_t* kmax, uint32_t g,
-                                                            float qmax, float& lo, float& hi) {
-    keys_to_range(__ldcg(kmin + g), __ldcg(kmax + g), lo, hi);
+constexpr float kRoundMagic = 12582912.0f;               // 1.5 * 2^23: adding it rounds to an integer, ties to even
+constexpr uint32_t kRoundMagicBits = 0x4B400000u;
+
+// The rounded value r = round(x / s + z) from ONE fused multiply-add, where that is provably the same integer.
+// Only r enters the results (code = clamp(r), y = s * (code - z), mask = (r == code)); the quotient and the sum
+// are intermediates.  z is an integer, so with |z| <= 2^20 the constant mz = 1.5 * 2^23 + z is exact, and
+//     m = fma(x, RN(1 / s), mz)
+// is 1.5 * 2^23 + (x * RN(1 / s) + z rounded to an integer, ties to even): its low mantissa bits are the code, and
+// t = m - mz = code - z is exact, so that y = s * t.  Bound: let w = x * RN(1 / s), v = x / s,
+// u = RN(RN(v) + z) the sum as defined.  |w - v| and |RN(v) - v| are at most 2^-24 |v|, |u - (RN(v) + z)| at most
+// 2^-24 (|u| + 1), and where the clamp does not decide, |v| <= |z| + qmax + 2 and |u| <= qmax + 2: u and w + z differ
+// by at most 2^-24 (2 |z| + 3 qmax + 7).  d = fma(x, RN(1 / s), -t) is w - t up to 2^-26.  So |d| below
+//     thr = 0.5 - 2^-23 (|z| + 1.5 qmax + 4)
+// puts u less than 0.5 away from the integer t + z: round(u) = t + z.  An element that fails the test takes the
+// sequence as defined (one in 3e5 at 4 bits, one in 1e4 at 8).  Values beyond [-2, qmax + 2] clamp alike either way.
+__device__ __forceinline__ float tie_threshold(float rcp, float z, float qmax) {
+    if (rcp == 0.0f || !(fabsf(z) <= 1048576.0f)) return 0.0f;
+    return __fmaf_rn(-1.1920928955078125e-07f, __fadd_rn(fabsf(z), __fmaf_rn(1.5f, qmax, 4.0f)), 0.5f);
+}
+
+// u = x / s + z as defined, rounded: 1.5 * 2^23 + clamp(round(u), -1, qmax + 1), given the quotient t = RN(x / s)
+__device__ __forceinline__ float exact_round_magic(float t, float z, float qmax) {
+    const float u = __fadd_rn(t, z);
+    return __fadd_rn(fminf(fmaxf(u, -1.0f), __fadd_rn(qmax, 1.0f)), kRoundMagic);
+}
+
+// Parameters of a group whose range (lo, hi) is that of the tensor itself.  thr is positive only where no element
+// of the group is clamped: rounding is monotone in x, so it is enough that neither lo nor hi is.  (lo never is:
+// z = round(RN(-lo / s)), so u(lo) lies within [-0.5, 0.5] and rounds to 0; hi is where u(hi) reaches qmax + 0.5,
+// a tie of lo / s, as in a range with lo = -hi.)  In such a group every mask bit is set and gx = gy.
+__device__ __forceinline__ GroupParam group_param_from_range(float lo, float hi, float qmax) {
     const QParam p = make_qparam(lo, hi, qmax);
     GroupParam gp;
     gp.s = p.s;
     gp.z = p.z;
     gp.r = div_is_safe(p.s, lo, hi) ? __frcp_rn(p.s) : 0.0f;
+    gp.thr = tie_threshold(gp.r, gp.z, qmax);
+    const float rl = exact_round_magic(div_by_scale(lo, gp.s, gp.r), gp.z, qmax);
+    const float rh = exact_round_magic(div_by_scale(hi, gp.s, gp.r), gp.z, qmax);
+    if (!(rl >= kRoundMagic && rh <= __fadd_rn(kRoundMagic, qmax))) gp.thr = -gp.thr;
     return gp;
 }
+__device__ __forceinline__ GroupParam group_param_from_keys(const uint32_t* kmin, const uint32_t* kmax, uint32_t g,
+                                                            float qmax, float& lo, float& hi) {
+    keys_to_range(__ldcg(kmin + g), __ldcg(kmax + g), lo, hi);
+    return group_param_from_range(lo, hi, qmax);
+}
 
-// The rounded value r = round(x / s + z) from ONE fused multiply-add, where that is provably the same integer.
-// Only r enters the results (code = clamp(r), y = s * (code - z), mask = (r == code)); the quotient and the sum
-// are intermediates.  With rcp = RN(1 / s), up = RN(x * rcp + z) lies within E = 2^-24 * (|x / s| + |up|) of the
-// real number v = x / s + z, and so does the exactly rounded u = RN(RN(x / s) + z).  |x / s| <= |v| + |z|, and
-// values beyond the clamp range [-1, qmax + 1] round to the same clamped integer either way, so inside it
-// E <= 2^-24 * (|z| + 2 * 258) < M = 2^-23 * (|z| + 1024).  If up is farther than 2 M from every half-integer,
-// v is farther than M from it, u lies on the same side, and round(u) = round(up).  tie_threshold() returns
-// 0.5 - 2 M: an element whose distance |up - round(up)| reaches it takes the exact sequence instead (for
-// |z| >= 2^21 the threshold is <= 0 and every element does).
-__device__ __forceinline__ float tie_threshold(float z) {
-    return __fmaf_rn(-2.384185791015625e-07f, __fadd_rn(fabsf(z), 1024.0f), 0.5f);      // 0.5 - 2^-22 * (|z| + 1024)
+// What the extra outputs of one pack are made of (EXTRAS as in quantize_pack): bytes of codes and mask (1), mask
+// bits (2), strings of code_bits per code (3).  m: 1.5 * 2^23 + code of element i, in: the clamp was inactive.
+template <int V, int EXTRAS>
+__device__ __forceinline__ void pack_extras(const float (&m)[V], uint32_t in, uint32_t (&cb)[V / 4],
+                                            uint32_t (&mb)[V / 4], int code_bits) {
+#pragma unroll
+    for (int h = 0; h < V / 4; ++h) {
+        cb[h] = 0;
+        mb[h] = 0;
+    }
+    if constexpr (EXTRAS == 1 || EXTRAS == 3) {
+        // sum of (magic bits + code) << shift, less the magic bits' share: one multiply-add per code
+        const uint32_t b = EXTRAS == 3 ? (uint32_t)code_bits : 8u;
+        const uint32_t m1 = 1u << b, m2 = 1u << (2 * b), m3 = 1u << (3 * b);
+        const uint32_t off = kRoundMagicBits * (1u + m1 + m2 + m3);
+#pragma unroll
+        for (int h = 0; h < V / 4; ++h)
+            cb[h] = __float_as_uint(m[4 * h]) + __float_as_uint(m[4 * h + 1]) * m1 + __float_as_uint(m[4 * h + 2]) * m2 +
+                    __float_as_uint(m[4 * h + 3]) * m3 - off;
+    }
+    if constexpr (EXTRAS == 1) {
+#pragma unroll
+        for (int i = 0; i < V; ++i) mb[i / 4] |= ((in >> i) & 1u) << (8 * (i % 4));
+    } else if constexpr (EXTRAS == 2) {
+        mb[0] = in;
+    }
 }
 
 // Quantize one pack: elements [0, n1) belong to the group with parameters g1, the rest to
@@ -286,120 +340,132 @@ __device__ __forceinline__ float tie_threshold(float z) {
 // (one byte per element); EXTRAS = 2 leaves the codes out and returns the mask as V bits in mb[0]
 // (bit i: the clamp was inactive for element i), which is all the packed mask needs; EXTRAS = 3 returns
 // only the codes, code_bits each (cb[h] = the four codes of half h as a string of 4 * code_bits bits; bytes for
-// the default of 8), taken from the low mantissa bits of code + 2^23 instead of a float-to-integer conversion
-// (packed-code output).  SELF: the range is that of the tensor itself, so x / s + z lies within
-// [-1, qmax + 1] already (x in [lo, hi] gives RN(x / s) - round(RN(lo / s)) >= -1/2, and at most qmax plus a few
-// units in the last place of hi / s < 2^33 above that) and the clamp before the rounding can go.
+// the default of 8), taken from the low mantissa bits of code + 1.5 * 2^23 instead of a float-to-integer
+// conversion (packed-code output).  SELF: the range is that of the tensor itself and thr comes from
+// group_param_from_range(), so where it is positive nothing is clamped and the gradient passes whole; without SELF
+// it comes from tie_threshold() alone and x may lie anywhere.
+// Instructions per element, bf16 or fp32 alike: two multiply-adds, one add, half a three-way maximum and one
+// product (SELF), where rounding by add and subtract, clamp, compare and select took eleven.  Measured against that
+// form: forward-only bf16 [256,512,28,28] at 8 bits 127.6 -> 119.6 us (issue slots bind where an element is two
+// bytes), packed codes of fp32 [128,144,56,56] 150 -> 142 us, packed mask of [128,64,56,56] 63.0 -> 60.6 us.
 template <typename T, bool BWD, bool SPLIT, int EXTRAS, bool SELF = false>
 __device__ __forceinline__ void quantize_pack(const Pack<T>& px, const Pack<T>& pg, const GroupParam& g1,
                                               const GroupParam& g2, int n1, float qmax, Pack<T>& py, Pack<T>& pgx,
                                               uint32_t (&cb)[Pack<T>::V / 4], uint32_t (&mb)[Pack<T>::V / 4],
                                               int code_bits = 8) {
     constexpr int V = Pack<T>::V;
-    const float kMagic = 12582912.0f;  // 1.5 * 2^23
-#pragma unroll
-    for (int i = 0; i < V / 4; ++i) {
-        cb[i] = 0;
-        mb[i] = 0;
-    }
-    float yv[V];
-    uint32_t keep = 0;                                          // bit i: the clamp was inactive for element i
-    auto finish = [&](int i, float r, float s, float z) {      // r: the rounded value, within [-1, qmax + 1]
-        const float q = fminf(fmaxf(r, 0.0f), qmax);
-        const bool in = (r == q);
-        yv[i] = __fmul_rn(s, __fsub_rn(q, z));
-        if constexpr (BWD) {
-            if constexpr (V == 4) pgx.set(i, in ? pg.get(i) : 0.0f);      // fp32: a select per element is all it takes
-            else keep |= in ? (1u << i) : 0u;                              // bf16: on the raw halves, below
-        }
-        if constexpr (EXTRAS == 1) {
-            cb[i / 4] |= (uint32_t)q << (8 * (i % 4));
-            mb[i / 4] |= (in ? 1u : 0u) << (8 * (i % 4));
-        } else if constexpr (EXTRAS == 2) {
-            mb[0] |= in ? (1u << i) : 0u;
-        } else if constexpr (EXTRAS == 3) {
-            cb[i / 4] |= (__float_as_uint(__fadd_rn(q, 8388608.0f)) & 0xFFu) << ((i % 4) * code_bits);
-        }
-    };
-    auto exact_round = [&](float t, float z) -> float {        // t = RN(x / s): the sequence as defined
-        const float u = __fadd_rn(t, z);
-        const float uc = fminf(fmaxf(u, -1.0f), __fadd_rn(qmax, 1.0f));
-        return __fsub_rn(__fadd_rn(uc, kMagic), kMagic);
-    };
-    const bool fast = SPLIT ? (g1.r != 0.0f && g2.r != 0.0f) : (g1.r != 0.0f);
-    if (fast) {
-        const float thr1 = tie_threshold(g1.z), thr2 = SPLIT ? tie_threshold(g2.z) : thr1;
+    constexpr uint32_t kAll = (1u << V) - 1u;
+    float m[V], yv[V];
+    uint32_t in = kAll;                                         // bit i: the clamp was inactive for element i
+    const float thr = SPLIT ? fminf(fabsf(g1.thr), fabsf(g2.thr)) : fabsf(g1.thr);
+    const float top = __fadd_rn(kRoundMagic, qmax);
+    if (thr > 0.0f) {
+        const float mz1 = __fadd_rn(kRoundMagic, g1.z), mz2 = SPLIT ? __fadd_rn(kRoundMagic, g2.z) : mz1;
+        float worst = 0.0f;
 #pragma unroll
         for (int i = 0; i < V; ++i) {
             const bool first = !SPLIT || i < n1;
-            const float s = first ? g1.s : g2.s, z = first ? g1.z : g2.z, rc = first ? g1.r : g2.r;
+            const float rc = first ? g1.r : g2.r, mz = first ? mz1 : mz2;
             const float x = px.get(i);
-            float up = __fmaf_rn(x, rc, z);
-            if constexpr (!SELF) up = fminf(fmaxf(up, -1.0f), __fadd_rn(qmax, 1.0f));
-            float r = __fsub_rn(__fadd_rn(up, kMagic), kMagic);
-            if (!(fabsf(__fsub_rn(up, r)) < (first ? thr1 : thr2)))     // rare: too close to a tie for the shortcut
-                r = exact_round(div_by_scale(x, s, rc), z);
-            finish(i, r, s, z);
+            m[i] = __fmaf_rn(x, rc, mz);
+            worst = fmaxf(worst, fabsf(__fmaf_rn(x, rc, __fsub_rn(mz, m[i]))));
         }
-    } else {
+        if (!(worst < thr)) {                                   // rare: too close to a tie for the shortcut
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                const bool first = !SPLIT || i < n1;
+                const float s = first ? g1.s : g2.s, z = first ? g1.z : g2.z, rc = first ? g1.r : g2.r;
+                const float mz = first ? mz1 : mz2, x = px.get(i);
+                if (!(fabsf(__fmaf_rn(x, rc, __fsub_rn(mz, m[i]))) < thr))
+                    m[i] = exact_round_magic(SELF ? div_by_scale(x, s, rc) : __fdiv_rn(x, s), z, qmax);
+            }
+        }
+        if (!SELF || g1.thr < 0.0f || (SPLIT && g2.thr < 0.0f)) {
+            in = 0;
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                const float c = fminf(fmaxf(m[i], kRoundMagic), top);
+                in |= (m[i] == c) ? (1u << i) : 0u;
+                m[i] = c;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            const bool first = !SPLIT || i < n1;
+            yv[i] = __fmul_rn(first ? g1.s : g2.s, __fsub_rn(m[i], first ? mz1 : mz2));
+        }
+    } else {                                                    // the sequence as defined, element by element
+        in = 0;
 #pragma unroll
         for (int i = 0; i < V; ++i) {
             const bool first = !SPLIT || i < n1;
             const float s = first ? g1.s : g2.s, z = first ? g1.z : g2.z;
-            finish(i, exact_round(__fdiv_rn(px.get(i), s), z), s, z);
+            const float r = exact_round_magic(__fdiv_rn(px.get(i), s), z, qmax);
+            m[i] = fminf(fmaxf(r, kRoundMagic), top);
+            in |= (m[i] == r) ? (1u << i) : 0u;
+            yv[i] = __fmul_rn(s, __fsub_rn(__fsub_rn(m[i], kRoundMagic), z));
         }
     }
+    if constexpr (BWD) pgx.select(pg, in);
+    pack_extras<V, EXTRAS>(m, in, cb, mb, code_bits);
     py.set_all(yv);
-    if constexpr (BWD && V != 4) pgx.select(pg, keep);
 }
 
 // Quantize one pack whose V elements belong to V different groups (channels-last rows), the range being the
-// tensor's own: element i takes the parameters g[i].  Same arithmetic and shortcut as quantize_pack().
+// tensor's own: element i takes scale s[i], reciprocal r[i] and mz[i] = 1.5 * 2^23 + z; thr is the smallest of the
+// V groups' thresholds in magnitude, negative when one of them is, and where it is 0 the parameters are read again
+// from `par` (the zero-point may then be too large for mz).  Same arithmetic as quantize_pack<SELF>.
 template <typename T, bool BWD, bool EXTRAS>
-__device__ __forceinline__ void quantize_pack_each(const Pack<T>& px, const Pack<T>& pg,
-                                                   const GroupParam (&g)[Pack<T>::V], float qmax, Pack<T>& py,
+__device__ __forceinline__ void quantize_pack_each(const Pack<T>& px, const Pack<T>& pg, const float (&s)[Pack<T>::V],
+                                                   const float (&r)[Pack<T>::V], const float (&mz)[Pack<T>::V],
+                                                   float thr, const GroupParam* par, float qmax, Pack<T>& py,
                                                    Pack<T>& pgx, uint32_t (&cb)[Pack<T>::V / 4],
                                                    uint32_t (&mb)[Pack<T>::V / 4]) {
     constexpr int V = Pack<T>::V;
-    const float kMagic = 12582912.0f;  // 1.5 * 2^23
+    float m[V], yv[V];
+    uint32_t in = (1u << V) - 1u;
+    const float bound = fabsf(thr), top = __fadd_rn(kRoundMagic, qmax);
+    if (bound > 0.0f) {
+        float worst = 0.0f;
 #pragma unroll
-    for (int i = 0; i < V / 4; ++i) {
-        cb[i] = 0;
-        mb[i] = 0;
-    }
-    float yv[V];
-    uint32_t keep = 0;
+        for (int i = 0; i < V; ++i) {
+            const float x = px.get(i);
+            m[i] = __fmaf_rn(x, r[i], mz[i]);
+            worst = fmaxf(worst, fabsf(__fmaf_rn(x, r[i], __fsub_rn(mz[i], m[i]))));
+        }
+        if (!(worst < bound)) {                                   // rare: too close to a tie for the shortcut
 #pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const float s = g[i].s, z = g[i].z, rc = g[i].r, x = px.get(i);
-        float r;
-        if (rc != 0.0f) {
-            const float up = __fmaf_rn(x, rc, z);
-            r = __fsub_rn(__fadd_rn(up, kMagic), kMagic);
-            if (!(fabsf(__fsub_rn(up, r)) < tie_threshold(z))) {     // rare: too close to a tie for the shortcut
-                const float u = __fadd_rn(div_by_scale(x, s, rc), z);
-                const float uc = fminf(fmaxf(u, -1.0f), __fadd_rn(qmax, 1.0f));
-                r = __fsub_rn(__fadd_rn(uc, kMagic), kMagic);
+            for (int i = 0; i < V; ++i) {
+                const float x = px.get(i);
+                if (!(fabsf(__fmaf_rn(x, r[i], __fsub_rn(mz[i], m[i]))) < bound))
+                    m[i] = exact_round_magic(div_by_scale(x, s[i], r[i]), __fsub_rn(mz[i], kRoundMagic), qmax);
             }
-        } else {
-            const float u = __fadd_rn(__fdiv_rn(x, s), z);
-            const float uc = fminf(fmaxf(u, -1.0f), __fadd_rn(qmax, 1.0f));
-            r = __fsub_rn(__fadd_rn(uc, kMagic), kMagic);
         }
-        const float q = fminf(fmaxf(r, 0.0f), qmax);
-        const bool in = (r == q);
-        yv[i] = __fmul_rn(s, __fsub_rn(q, z));
-        if constexpr (BWD) {
-            if constexpr (V == 4) pgx.set(i, in ? pg.get(i) : 0.0f);
-            else keep |= in ? (1u << i) : 0u;
+        if (thr < 0.0f) {
+            in = 0;
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                const float c = fminf(fmaxf(m[i], kRoundMagic), top);
+                in |= (m[i] == c) ? (1u << i) : 0u;
+                m[i] = c;
+            }
         }
-        if constexpr (EXTRAS) {
-            cb[i / 4] |= (uint32_t)q << (8 * (i % 4));
-            mb[i / 4] |= (in ? 1u : 0u) << (8 * (i % 4));
+#pragma unroll
+        for (int i = 0; i < V; ++i) yv[i] = __fmul_rn(s[i], __fsub_rn(m[i], mz[i]));
+    } else {                                                    // the sequence as defined, element by element
+        in = 0;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            const GroupParam g = par[i];
+            const float q = exact_round_magic(__fdiv_rn(px.get(i), g.s), g.z, qmax);
+            m[i] = fminf(fmaxf(q, kRoundMagic), top);
+            in |= (m[i] == q) ? (1u << i) : 0u;
+            yv[i] = __fmul_rn(g.s, __fsub_rn(__fsub_rn(m[i], kRoundMagic), g.z));
         }
     }
+    if constexpr (BWD) pgx.select(pg, in);
+    pack_extras<V, EXTRAS ? 1 : 0>(m, in, cb, mb, 8);
     py.set_all(yv);
-    if constexpr (BWD && V != 4) pgx.select(pg, keep);
 }
 
 // per-lane min / max of elements [first, last) of one pack

@@ -384,11 +384,7 @@ __global__ void __launch_bounds__(kThreads) quant_flat_kernel(const T* __restric
                 } else {
                     Pack<T> py, pgx;
                     uint32_t cb[V / 4 > 0 ? V / 4 : 1], mb[V / 4 > 0 ? V / 4 : 1];
-                    // x may lie outside the given range: the short division needs |x| <= 2^60
-                    float amax = 0.0f;
-#pragma unroll
-                    for (int i = 0; i < V; ++i) amax = fmaxf(amax, fabsf(px[j].get(i)));
-                    GroupParam gp{p.s, p.z, (amax <= 1152921504606846976.0f) ? rcp : 0.0f};
+                    GroupParam gp{p.s, p.z, rcp, tie_threshold(rcp, p.z, qmax)};
                     GroupParam gp2 = gp;
                     int n1 = V;
                     if constexpr (RAGGED) {
@@ -398,13 +394,15 @@ __global__ void __launch_bounds__(kThreads) quant_flat_kernel(const T* __restric
                             if (tabled) {
                                 gp2.s = s_tab_s[q + 1];
                                 gp2.z = s_tab_z[q + 1];
-                                gp2.r = (amax <= 1152921504606846976.0f) ? s_tab_r[q + 1] : 0.0f;
+                                gp2.r = s_tab_r[q + 1];
+                                gp2.thr = tie_threshold(gp2.r, gp2.z, qmax);
                             } else {
                                 const uint32_t grp2 = group_at(g, base, q + 1);
                                 const QParam p2 = make_qparam(__fadd_rn(lo[grp2], 0.0f), __fadd_rn(hi[grp2], 0.0f), qmax);
                                 gp2.s = p2.s;
                                 gp2.z = p2.z;
                                 gp2.r = 0.0f;
+                                gp2.thr = 0.0f;
                             }
                         }
                     }

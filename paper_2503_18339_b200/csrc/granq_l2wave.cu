@@ -79,8 +79,7 @@ __global__ void __launch_bounds__(kLThreads, UPL == 2 ? 4 : 3) l2wave_kernel(con
     const uint32_t tab = ((a.cw + 15u) / 16u) * 16u;
     uint32_t* s_kmn = s_keys;
     uint32_t* s_kmx = s_keys + tab;
-    float2* s_sz = reinterpret_cast<float2*>(s_keys + 2 * tab);   // [tab] (scale, zero-point)
-    float* s_rcp = reinterpret_cast<float*>(s_sz + tab);          // [tab] RN(1 / scale), or 0 = use IEEE division
+    GroupParam* s_par = reinterpret_cast<GroupParam*>(s_keys + 2 * tab);   // [tab] scale, zero-point, reciprocal, tie threshold
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint4* xg = reinterpret_cast<const uint4*>(a.x);
     const uint4* gyg = reinterpret_cast<const uint4*>(a.gy);
@@ -202,8 +201,7 @@ __global__ void __launch_bounds__(kLThreads, UPL == 2 ? 4 : 3) l2wave_kernel(con
         for (uint32_t t = tid; t < sh.channels; t += kLThreads) {
             float lo, hi;
             const GroupParam gp = group_param_from_keys(a.kmin, a.kmax, c0 + t, qmax, lo, hi);
-            s_sz[t] = make_float2(gp.s, gp.z);
-            s_rcp[t] = gp.r;
+            s_par[t] = gp;
             if (writer) {
                 a.lo[c0 + t] = lo;
                 a.hi[c0 + t] = hi;
@@ -232,13 +230,7 @@ __global__ void __launch_bounds__(kLThreads, UPL == 2 ? 4 : 3) l2wave_kernel(con
             const uint32_t ch_first = ALIGNED ? a.div_plane.div(r0) : a.div_plane.div(r0 * V);
             const uint32_t ch_last = ALIGNED ? a.div_plane.div(last_u) : a.div_plane.div(last_u * V + (V - 1));
             const bool one_channel = ch_first == ch_last;
-            GroupParam row_g;
-            {
-                const float2 sz = s_sz[ch_first];
-                row_g.s = sz.x;
-                row_g.z = sz.y;
-                row_g.r = s_rcp[ch_first];
-            }
+            const GroupParam row_g = s_par[ch_first];
 #pragma unroll
             for (int j = 0; j < UPL; ++j) {
                 const uint32_t uo = r0 + j * 32 + lane;
@@ -256,18 +248,8 @@ __global__ void __launch_bounds__(kLThreads, UPL == 2 ? 4 : 3) l2wave_kernel(con
                         n1 = (int)min((uint32_t)V, a.inner - rem);
                         ci2 = min(ci1 + 1, sh.channels - 1);
                     }
-                    const float2 sz1 = s_sz[ci1];
-                    g1.s = sz1.x;
-                    g1.z = sz1.y;
-                    g1.r = s_rcp[ci1];
-                    if constexpr (ALIGNED) {
-                        g2 = g1;
-                    } else {
-                        const float2 sz2 = s_sz[ci2];
-                        g2.s = sz2.x;
-                        g2.z = sz2.y;
-                        g2.r = s_rcp[ci2];
-                    }
+                    g1 = s_par[ci1];
+                    g2 = ALIGNED ? g1 : s_par[ci2];
                 }
                 if (!valid) continue;
                 Pack<T> py, pgx;
@@ -380,7 +362,7 @@ L2Plan plan_l2wave(int dtype, const Geom& g, const QuantIO& io, const StagedTuni
     if ((uint64_t)p.cw * inner / V >= (1ull << 30)) return p;
     // long planes: rows of 128 units lie in one channel and amortise the row set-up; short planes: 64
     p.upl = tune.l2_upl == 4 ? 4 : (tune.l2_upl == 2 ? 2 : ((inner / V) >= 512 ? 4 : 2));
-    p.smem_bytes = 20u * (((p.cw + 15u) / 16u) * 16u);     // keys (8 B) and parameters (12 B) per group
+    p.smem_bytes = 24u * (((p.cw + 15u) / 16u) * 16u);     // keys (8 B) and parameters (16 B) per group
     p.ok = true;
     return p;
 }

@@ -141,13 +141,22 @@ __global__ void __launch_bounds__(kRThreads, 3) rows_quant_kernel(const RArgs a)
     for (uint32_t tile0 = 0; tile0 < a.ncol; tile0 += w.P) {
         const uint32_t col = tile0 + w.cin;
         if (!w.rowed || col >= a.ncol) continue;
-        GroupParam g[V];
+        float s[V], rc[V], mz[V], thr = 1.0f;
+        bool clamped = false;
 #pragma unroll
-        for (int i = 0; i < V; ++i) g[i] = r_par[col * V + i];
+        for (int i = 0; i < V; ++i) {
+            const GroupParam g = r_par[col * V + i];
+            s[i] = g.s;
+            rc[i] = g.r;
+            mz[i] = __fadd_rn(kRoundMagic, g.z);
+            thr = fminf(thr, fabsf(g.thr));
+            clamped |= g.thr < 0.0f;
+        }
+        if (clamped) thr = -thr;
         auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint64_t at) {
             Pack<T> py, pgx;
             uint32_t cb[V / 4], mb[V / 4];
-            quantize_pack_each<T, kBwd, EXTRAS>(px, pg, g, qmax, py, pgx, cb, mb);
+            quantize_pack_each<T, kBwd, EXTRAS>(px, pg, s, rc, mz, thr, r_par + col * V, qmax, py, pgx, cb, mb);
             st_stream_16(yg + at, py.raw);
             if constexpr (kBwd) st_stream_16(gxg + at, pgx.raw);
             if constexpr (EXTRAS) {
