@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
 
     // ---- quantize, clamp, dequantize from shared memory; STE backward (Eq. 1, 6, Section 2.1) ----
     const float qmax = a.qmax;
-    DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS only)
+    DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS = 4)
     dacc.reset();
     if constexpr (ASYNC && GY) k_cp_async_wait<0>();
     for (uint32_t tile0 = 0; tile0 < ncol; tile0 += P) {
@@ -456,9 +456,9 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
 #pragma unroll
                         for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.mask)[w + i] = mb[i];
                     }
-                    if (a.dist) dacc.add(px, py);
                 }
-                if (a.pmask) {
+                if constexpr (EXTRAS == 4) dacc.add(px, py);
+                if (EXTRAS != 4 && a.pmask) {
                     // the mask is written byte by byte (8 elements: two fp32 packs of neighbouring lanes, one bf16
                     // pack): the planner has made every run and slab whole bytes of mask and the rows of columns
                     // whole pairs of lanes, so both lanes of a byte are here together, in the same slab
@@ -514,9 +514,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
             qg += sstep;
         }
     }
-    if constexpr (EXTRAS == 1) {
-        if (a.dist) dacc.flush(a.dist);       // all lanes of every warp are here
-    }
+    if constexpr (EXTRAS == 4) dacc.flush(a.dist);       // every thread of the block is here
     if constexpr (BULK) {
         // Nothing of this CTA may still be in flight when it leaves: every barrier once more (a no-op unless a
         // wait above gave up early), with the built-in limit.
@@ -563,7 +561,7 @@ cudaError_t k_launch_t(const KArgs& args, const ClusterPlan& plan, uint32_t grid
         cfg.numAttrs = plan.early_launch ? 2 : 1;
         return cudaLaunchKernelEx(&cfg, kern, args);
     };
-    if constexpr (EXTRAS == 2 || EXTRAS == 3) {      // packed mask or packed codes alone: forward plans with per-thread copies or plain loads
+    if constexpr (EXTRAS >= 2) {      // packed mask, packed codes or sums alone: forward plans with per-thread copies or plain loads
         if (plan.load == K_LOAD_ASYNC_X) return launch(cluster_kernel<T, MODE, ALIGNED, EXTRAS, K_LOAD_ASYNC_X, 4, 2>);
         return launch(cluster_kernel<T, MODE, ALIGNED, EXTRAS, K_LOAD_PLAIN, 4, 2>);
     } else {
@@ -585,6 +583,8 @@ cudaError_t k_launch_mode(const KArgs& a, const ClusterPlan& p, bool aligned, in
             return aligned ? k_launch_t<T, MODE, true, 2>(a, p, grid, st) : k_launch_t<T, MODE, false, 2>(a, p, grid, st);
         if (extras == 3)
             return aligned ? k_launch_t<T, MODE, true, 3>(a, p, grid, st) : k_launch_t<T, MODE, false, 3>(a, p, grid, st);
+        if (extras == 4)
+            return aligned ? k_launch_t<T, MODE, true, 4>(a, p, grid, st) : k_launch_t<T, MODE, false, 4>(a, p, grid, st);
     }
     if (aligned)
         return extras ? k_launch_t<T, MODE, true, 1>(a, p, grid, st) : k_launch_t<T, MODE, true, 0>(a, p, grid, st);
@@ -630,6 +630,7 @@ ClusterPlan plan_cluster(int dtype, const Geom& g, const QuantIO& io, bool backw
             break;
     }
     // the two lanes that assemble a byte of mask must both be there: only the variants without a give-up path qualify
+    // (the sums, which take every thread of the block, fall back to plain loads in k_launch_t)
     if ((io.pmask || io.pcodes) && p.load != K_LOAD_ASYNC_X && p.load != K_LOAD_ASYNC_XG && p.load != K_LOAD_PLAIN) return p;
     const uint64_t tiles = (p.load == K_LOAD_BULK_XG || p.load == K_LOAD_ASYNC_XG) ? 2 : 1;   // staged tiles per CTA
     const uint32_t k0 = unit / k_gcd(inner, unit);
@@ -724,8 +725,10 @@ cudaError_t launch_cluster(const ClusterPlan& plan, const QuantIO& io, int mode,
     const uint32_t nruns = (a.C + plan.k - 1) / plan.k;
     const uint32_t grid = nruns * plan.R;
     const bool aligned = (a.inner % V) == 0;
-    // 1: codes / mask bytes / sums compiled in; 2: the packed mask alone (a leaner instantiation of the forward kernel)
-    const int extras = (io.codes != nullptr || io.mask != nullptr || io.dist != nullptr) ? 1 : (io.pmask != nullptr ? 2 : (io.pcodes != nullptr ? 3 : 0));
+    // 1: codes / mask bytes compiled in; leaner instantiations of the forward kernel for one extra output alone:
+    // 2: the packed mask, 3: the packed codes, 4: the distortion sums
+    const int extras = (io.codes != nullptr || io.mask != nullptr) ? 1
+                       : io.dist != nullptr ? 4 : io.pmask != nullptr ? 2 : io.pcodes != nullptr ? 3 : 0;
     if (dtype == 0) {
         if (mode == MODE_FWD) return k_launch_mode<float, MODE_FWD>(a, plan, aligned, extras, grid, st);
         return k_launch_mode<float, MODE_BOTH>(a, plan, aligned, extras, grid, st);

@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kCThreads, 4) colwalk_kernel(const CArgs a) {
     };
 
     uint32_t p1_items = 0;      // items this CTA has reduced so far (selects the shared-memory buffer)
-    DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS only)
+    DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS = 4)
     dacc.reset();
 
     // ---- phase 1: this CTA's items of wave w -> min / max keys, then arrive ----
@@ -328,9 +328,9 @@ __global__ void __launch_bounds__(kCThreads, 4) colwalk_kernel(const CArgs a) {
 #pragma unroll
                             for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.mask)[at * (V / 4) + i] = mb[i];
                         }
-                        if (a.dist) dacc.add(px, py);
                     }
-                    if (a.pmask) {
+                    if constexpr (EXTRAS == 4) dacc.add(px, py);
+                    if (EXTRAS != 4 && a.pmask) {
                         // the mask is written byte by byte (8 elements: two fp32 packs of neighbouring lanes, one
                         // bf16 pack); the planner has made every slab and wave whole mask words, so both lanes of a
                         // byte are here together
@@ -375,9 +375,7 @@ __global__ void __launch_bounds__(kCThreads, 4) colwalk_kernel(const CArgs a) {
         phase2(w);
     }
 
-    if constexpr (EXTRAS == 1) {
-        if (a.dist) dacc.flush(a.dist);
-    }
+    if constexpr (EXTRAS == 4) dacc.flush(a.dist);
 
     // ---- leave the workspace as it was found: the last CTA to finish clears keys and counters ----
     __syncthreads();
@@ -473,6 +471,8 @@ cudaError_t c_launch_mode(CArgs& a, bool aligned, int extras, int sms, int cap, 
             return aligned ? c_launch_t<T, MODE, true, 2>(a, sms, cap, st) : c_launch_t<T, MODE, false, 2>(a, sms, cap, st);
         if (extras == 3)       // the packed codes alone
             return aligned ? c_launch_t<T, MODE, true, 3>(a, sms, cap, st) : c_launch_t<T, MODE, false, 3>(a, sms, cap, st);
+        if (extras == 4)       // the distortion sums
+            return aligned ? c_launch_t<T, MODE, true, 4>(a, sms, cap, st) : c_launch_t<T, MODE, false, 4>(a, sms, cap, st);
     }
     if (aligned)
         return extras ? c_launch_t<T, MODE, true, 1>(a, sms, cap, st) : c_launch_t<T, MODE, true, 0>(a, sms, cap, st);
@@ -623,8 +623,9 @@ cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int
         s.div_ncol = make_fastdiv(s.ncol);
     }
     a.div_plane = make_fastdiv(aligned ? inner / V : inner);
-    // 1: codes / mask bytes / sums compiled in; 2: the packed mask alone
-    const int extras = (io.codes != nullptr || io.mask != nullptr || io.dist != nullptr) ? 1 : (io.pmask != nullptr ? 2 : (io.pcodes != nullptr ? 3 : 0));
+    // 1: codes / mask bytes compiled in; alone: 2 the packed mask, 3 the packed codes, 4 the distortion sums
+    const int extras = (io.codes != nullptr || io.mask != nullptr) ? 1
+                       : io.dist != nullptr ? 4 : io.pmask != nullptr ? 2 : io.pcodes != nullptr ? 3 : 0;
     const int cap = tune.l2_ctas_per_sm;
     if (dtype == 0) {
         if (mode == MODE_FWD) return c_launch_mode<float, MODE_FWD>(a, aligned, extras, sms, cap, st);

@@ -286,7 +286,8 @@ __device__ __forceinline__ void warp_pack_row(uint64_t mine, uint32_t nb, uint32
 }
 
 // ---- Eq. 1, clamp, Eq. 6, STE: elementwise pass with a given per-group range ----------------------
-// EXTRAS = 1: the optional codes / mask / packed-mask outputs are compiled in; 2: the packed mask alone.  The packed mask holds
+// EXTRAS = 1: the optional codes / mask / packed-mask / sums outputs are compiled in; 2: the packed mask alone; 4: the
+// distortion sums alone.  The packed mask holds
 // one bit per element (bit e % 32 of word e / 32): a warp's lanes own consecutive elements or packs
 // starting at a multiple of 32 elements, so whole words are assembled with warp shuffles.
 // PACKONLY: the packed integer codes are the only output (everything else is compiled out).  With EXTRAS = 3
@@ -410,11 +411,9 @@ __global__ void __launch_bounds__(kThreads) quant_flat_kernel(const T* __restric
                     if constexpr (EXTRAS == 3) {
                         code_string = code_string_of<V>(cb, code_bits);
                     } else if constexpr (EXTRAS != 0) {
-                        if constexpr (!PACKONLY) inside_bits = mask_bits_of<V, EXTRAS>(mb);
+                        if constexpr (!PACKONLY && EXTRAS != 4) inside_bits = mask_bits_of<V, EXTRAS>(mb);
+                        if constexpr (EXTRAS == 4) dacc.add(px[j], py);
                         if constexpr (kFwd && EXTRAS == 1) {
-                            if constexpr (!PACKONLY) {
-                                if (dist) dacc.add(px[j], py);
-                            }
                             if (PACKONLY || pcodes) {
 #pragma unroll
                                 for (int i = 0; i < V; ++i)
@@ -442,7 +441,7 @@ __global__ void __launch_bounds__(kThreads) quant_flat_kernel(const T* __restric
                     }
                 }
                 }
-                if constexpr (EXTRAS != 0 && kFwd) {
+                if constexpr (EXTRAS != 0 && EXTRAS != 4 && kFwd) {
                     if (!PACKONLY && pmask) {          // every lane of the warp is here: assemble whole 32-bit words
                         const uint32_t lane = threadIdx.x & 31;
                         const int64_t word = (e0 + k[j]) >> 5;
@@ -478,7 +477,7 @@ __global__ void __launch_bounds__(kThreads) quant_flat_kernel(const T* __restric
             }
         }
     }
-    if constexpr (EXTRAS == 1 && kFwd && !PACKONLY) {
+    if constexpr (EXTRAS == 4 || (V == 1 && EXTRAS == 1 && kFwd)) {      // the scalar form keeps all extras in one
         if (dist) dacc.flush(dist);
     }
 }
@@ -741,6 +740,19 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
                     io.code_bits, f, qmax, lo, hi);
             else
                 quant_flat_kernel<T, VF, MODE, 1, true, true><<<grid, kThreads, 0, st>>>(
+                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                    io.code_bits, f, qmax, lo, hi);
+            return cudaGetLastError();
+        }
+        const bool dist_only = io.dist != nullptr && io.y != nullptr && io.codes == nullptr && io.mask == nullptr &&
+                               io.pmask == nullptr && io.pcodes == nullptr;
+        if ((vec || ragged) && dist_only) {
+            if (vec)
+                quant_flat_kernel<T, VF, MODE, 4><<<grid, kThreads, 0, st>>>(
+                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                    io.code_bits, f, qmax, lo, hi);
+            else
+                quant_flat_kernel<T, VF, MODE, 4, false, true><<<grid, kThreads, 0, st>>>(
                     (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                     io.code_bits, f, qmax, lo, hi);
             return cudaGetLastError();
