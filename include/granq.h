@@ -43,7 +43,7 @@
  * Execution.  All work is enqueued on `cuda_stream` (a cudaStream_t passed as void*;
  * NULL = the default stream); no entry point synchronises with the host except
  * granq_fakequant_fused_host() (unless GRANQ_FLAG_HOST_ASYNC), granq_host_arena_status(),
- * granq_workspace_status() and granq_fakequant_weights() (which reads its host descriptor
+ * granq_workspace_status() and granq_fakequant_weights() (which has read its host descriptor
  * array before it returns).  Results are bit-identical from run to run, except the last bits
  * of the distortion sums, whose fp64 atomics arrive in no fixed order.  The library keeps no
  * results and no per-call state; the only process-wide state is (a) the planner overrides set with
@@ -262,10 +262,10 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
  *   descs       HOST array of n_tensors descriptors (read before the call returns); the pointers
  *               inside are DEVICE memory: x in, y out, gy_opt / gx_opt both or neither,
  *               min_out / max_out `channels` floats each (required), scale_opt / zp_opt or NULL
- *   workspace   DEVICE scratch of granq_weights_workspace_bytes(n_tensors), 256-byte aligned
- * Limits: fewer than 2^31 groups in the batch and 2^31 elements per group.  The call stages the
- * descriptors through host memory it owns only until it returns, so it cannot be recorded into a CUDA
- * graph: on a capturing stream it returns GRANQ_ERR_UNSUPPORTED and enqueues nothing.
+ *   workspace   DEVICE scratch of granq_weights_workspace_bytes(n_tensors), 256-byte aligned (checked as part
+ *               of the contract; the descriptors travel in the launch's parameters)
+ * Limits: fewer than 2^31 groups in the batch and 2^31 elements per group; lists beyond 256 tensors take one
+ * launch per 256.  On a capturing stream it returns GRANQ_ERR_UNSUPPORTED and enqueues nothing.
  */
 typedef struct granq_weight_desc {
     const void* x;

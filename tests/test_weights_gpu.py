@@ -62,6 +62,27 @@ def test_odd_shapes_constant_channels_and_one_tensor(b):
     assert same_bits(to_np(out.y).reshape(ref.y.shape), ref.y) and same_bits(to_np(out.lo), ref.lo)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("elems", [1, 160, 161, 320, 640, 644, 1280, 1281, 2560, 5120, 5128, 10240, 10248, 12001])
+def test_group_sizes_around_what_a_team_of_warps_holds(b, dtype, elems):
+    """One group per team: the last size that 1, 2, 4 and 8 warps hold in registers, and the first beyond (units of
+    16 bytes, single elements where groups are not whole units), with channel counts that leave teams of the last
+    block without a group, in a list mixed with a small tensor."""
+    rng = np.random.default_rng(elems)
+    shapes = [(9, elems), (3, 8), (1, elems)]
+    ws = [rng.standard_normal(s).astype(np.float32) for s in shapes]
+    gs = [rng.standard_normal(s).astype(np.float32) for s in shapes]
+    check_batch(b, ws, gs, 4, dtype)
+    check_batch(b, ws, None, 8, dtype)
+
+
+def test_more_tensors_than_one_launch_takes(b):
+    rng = np.random.default_rng(0)
+    ws = [rng.standard_normal((1 + i % 5, 4 + i % 7)).astype(np.float32) for i in range(260)]
+    check_batch(b, ws, ws, 3, "f32")
+    check_batch(b, ws[:33], None, 3, "f32")
+
+
 def test_weights_reject_bad_arguments(b):
     w = to_dev(np.ones((4, 8), np.float32))
     with pytest.raises(b.GranqError) as err:
