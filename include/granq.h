@@ -477,7 +477,8 @@ enum granq_knob {
                                              3 = bulk copies for x and gy                              */
     GRANQ_KNOB_CLUSTER_PREFETCH = 14,     /* cluster plan: 1 = L2 prefetch of gy, 2 = none             */
     GRANQ_KNOB_CLUSTER_KMUL = 15,         /* cluster plan: multiplier of a run's minimal channel count */
-    GRANQ_KNOB_CLUSTER_EARLY_LAUNCH = 16  /* cluster plan: 2 = launch without programmatic dependent launch */
+    GRANQ_KNOB_CLUSTER_EARLY_LAUNCH = 16, /* cluster plan: 2 = launch without programmatic dependent launch */
+    GRANQ_KNOB_COLWALK_TEAM = 17          /* column-walk plan: 2 = L2 waves only (as any set L2 knob means)    */
 };
 int granq_tune(int knob, int value);
 

@@ -26,8 +26,8 @@ PLAN_TWO_PASS, PLAN_NAIVE, PLAN_STAGED, PLAN_L2WAVE, PLAN_COLWALK, PLAN_CLUSTER,
 (KNOB_STAGED_DEPTH, KNOB_STAGED_MAX_BUF_UNITS, KNOB_STAGED_GRID, KNOB_SPIN_LIMIT, KNOB_TEST_EXTRA_ARRIVALS,
  KNOB_STAGED_CTAS_PER_SM, KNOB_L2_WAVE_KB, KNOB_L2_UPL, KNOB_L2_CTAS_PER_SM, KNOB_L2_LAG,
  KNOB_CLUSTER_TILE_KB, KNOB_CLUSTER_CTAS, KNOB_CLUSTER_THREADS, KNOB_CLUSTER_LOAD, KNOB_CLUSTER_PREFETCH,
- KNOB_CLUSTER_KMUL, KNOB_CLUSTER_EARLY_LAUNCH) = range(17)
-N_KNOBS = 17
+ KNOB_CLUSTER_KMUL, KNOB_CLUSTER_EARLY_LAUNCH, KNOB_COLWALK_TEAM) = range(18)
+N_KNOBS = 18
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = range(6)
 
 EXPORTS = [

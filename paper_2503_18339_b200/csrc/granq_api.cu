@@ -658,6 +658,7 @@ int granq_tune(int knob, int value) {
         case GRANQ_KNOB_CLUSTER_PREFETCH: g_tune.cl_prefetch = value; return GRANQ_OK;
         case GRANQ_KNOB_CLUSTER_KMUL: g_tune.cl_kmul = value; return GRANQ_OK;
         case GRANQ_KNOB_CLUSTER_EARLY_LAUNCH: g_tune.cl_pdl = value; return GRANQ_OK;
+        case GRANQ_KNOB_COLWALK_TEAM: g_tune.col_team = value; return GRANQ_OK;
         default: return GRANQ_ERR_INVALID_ARG;
     }
 }

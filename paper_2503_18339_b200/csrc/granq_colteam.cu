@@ -1,0 +1,369 @@
+// Resident column walk: every activation of a large channel group is read from HBM once.
+//
+// A channel of a large plane (1.6 MB for 56 x 56 planes at batch 128, 6.4 MB for 112 x 112) fits neither one SM nor
+// one thread-block cluster, but it fits the shared memory of a TEAM of CTAs of one cooperative launch, and the
+// whole GPU holds 18 teams of 16 such CTAs.  Each team takes one channel at a time:
+//   - its units (16 bytes each, all slabs laid end to end) are dealt out evenly over the team's CTAs; a CTA copies
+//     its share to shared memory with per-thread asynchronous copies, every thread copying exactly the units it will
+//     read, so no barrier stands between a copy and its use;
+//   - each CTA reduces its share (Eq. 4), publishes one pair of ordered keys with atomics, arrives on the channel's
+//     counter and waits (bounded) for the rest of its team - not for the grid;
+//   - scale and zero-point (Eq. 5) are worked out once per CTA and the share is quantized from shared memory (Eq. 1,
+//     clamp, Eq. 6, STE).  A unit's place in shared memory is free as soon as its thread has read it, so the same
+//     loop sends the copy of the team's NEXT channel after it: reads stay in flight through the whole write phase.
+// With a gradient gy is staged the same way as far as shared memory goes and read in place beyond that.
+//
+// Why not the L2-resident waves of colwalk_kernel: the L2 does not keep a wave (forward-only calls read x 1.4 to 2
+// times from HBM, ncu: 5-14 % L2 hits), and its phases alternate.  Why teams and not clusters of 16 CTAs: a
+// cluster must sit in one GPC, which leaves an SM in ten without one.  Measured against the waves (fp32 / bf16, us):
+// forward [128,64,56,56] 55.8 -> 45.7 / 34.7 -> 30.3, [128,96,112,112] 309 -> 264 / 174 -> 139, [256,512,28,28]
+// 219 -> 156 / 123 -> 92; with a gradient 87.5 -> 81.9 / 47.4 -> 45.6, 472 -> 469 / 258 -> 234, 332 -> 298 / 183 -> 153;
+// [256,16,32,32] 16.7 -> 14.9 and 21.9 -> 19.4.  Bound by HBM in the mix of reads and writes (4.5-5.3 TB/s) once a
+// team has several channels, by the chain of copy, hand-over and quantize when it has one.
+//
+// Two CTAs of 512 threads per SM, 113 KB of shared memory each: one transfers while the other waits for its team.
+// The kernel expects zeroed keys and counters and, when no wait ran out, leaves them zeroed (slot C of the
+// counters counts the CTAs that have finished; the last one clears).
+#include "granq_internal.h"
+
+#include <algorithm>
+#include <atomic>
+
+namespace granq {
+
+namespace {
+
+constexpr int kTThreads = 512;
+constexpr uint32_t kTWarps = kTThreads / 32;
+constexpr uint32_t kTSpinLimit = 1u << 24;   // bounded wait on a channel's counter (x ~32 ns)
+constexpr uint32_t kTStatusTimeout = 5;      // GRANQ_ERR_TIMEOUT
+constexpr uint32_t kTSmemUnits = 111u * 1024 / 16;      // staged units per CTA: two CTAs per SM, 228 KB between them
+
+struct TArgs {
+    const void* x;
+    const void* gy;
+    void* y;
+    void* gx;
+    uint32_t* pmask;       // the STE mask at one bit per element, or null
+    uint32_t* pcodes;      // the codes as a bit string of code_bits each, or null (y is then not written)
+    int code_bits;
+    double* dist;          // four running sums of Table 2's statistics, or null
+    uint32_t* status;
+    uint32_t* kmin;
+    uint32_t* kmax;
+    uint32_t* counters;
+    float* lo;
+    float* hi;
+    float* s_out;
+    float* z_out;
+    float qmax;
+    uint32_t C;            // channels
+    uint32_t plane_units;  // units of one plane
+    uint32_t units;        // units of one channel over all slabs
+    uint32_t R, teams;     // CTAs per team, teams
+    uint32_t tile_units;   // room for x in shared memory
+    uint32_t gy_units;     // of a CTA's share of gy, this many units are staged behind it
+    uint32_t spin_limit, expected;
+    uint64_t slab_units;   // units of one slab
+    FastDiv div_plane;     // units per plane
+};
+
+__device__ __forceinline__ uint32_t t_ld_acquire(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void t_arrive_release(uint32_t* p) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+// without an L2 cache hint: with one, sent from inside the (divergent) quantize walk, the kernel ended in an illegal
+// instruction on long walks
+__device__ __forceinline__ void t_cp_async_16(void* dst_smem, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void t_cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// U = units a thread handles together in the quantize walk
+template <typename T, int MODE, int EXTRAS, int U>
+__global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
+    constexpr int V = Pack<T>::V;
+    constexpr bool kBwd = (MODE & MODE_BWD) != 0;
+    extern __shared__ __align__(16) uint4 t_smem[];
+    __shared__ uint32_t s_kmn[kTWarps], s_kmx[kTWarps];
+    __shared__ GroupParam s_par;
+    __shared__ uint32_t s_ok;
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    const uint32_t team = blockIdx.x / a.R, rank = blockIdx.x - team * a.R;
+    // this CTA's share: whole runs of 8 units (128 bytes) of the channel's units laid end to end
+    const uint32_t runs = (a.units + 7) / 8;
+    const uint32_t q0 = 8 * (uint32_t)(((uint64_t)rank * runs) / a.R);
+    const uint32_t q1 = min(a.units, 8 * (uint32_t)(((uint64_t)(rank + 1) * runs) / a.R));
+    const uint32_t n = q1 - q0;
+    const uint32_t cnt = tid < n ? (n - tid + kTThreads - 1) / kTThreads : 0u;      // units of this thread
+    // where they are: unit q lies in slab q / plane_units, and the next one of this thread is kTThreads units on
+    uint32_t slab0, off0;
+    a.div_plane.divmod(q0 + min(tid, n), slab0, off0);
+    const uint64_t first = (uint64_t)slab0 * a.slab_units + off0;
+    uint32_t dslab, doff;
+    a.div_plane.divmod((uint32_t)kTThreads, dslab, doff);
+    const uint64_t dstep = (uint64_t)dslab * a.slab_units + doff, dwrap = a.slab_units - a.plane_units;
+    auto advance = [&](uint64_t& at, uint32_t& off) {
+        at += dstep;
+        off += doff;
+        if (off >= a.plane_units) {
+            off -= a.plane_units;
+            at += dwrap;
+        }
+    };
+    uint4* tile = t_smem + tid;
+    uint4* tileg = t_smem + a.tile_units + tid;
+    const uint32_t gcnt = kBwd ? (tid < a.gy_units ? min(cnt, (a.gy_units - tid + kTThreads - 1) / kTThreads) : 0u) : 0u;
+    const uint4* xg = reinterpret_cast<const uint4*>(a.x);
+    const uint4* gyg = reinterpret_cast<const uint4*>(a.gy);
+    uint4* yg = reinterpret_cast<uint4*>(a.y);
+    uint4* gxg = reinterpret_cast<uint4*>(a.gx);
+    const uint64_t drop = l2_policy_evict_first();
+    const float qmax = a.qmax;
+    DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS = 4)
+    dacc.reset();
+
+    // the first channel's copies; those of the later ones are sent from the quantize walk
+    {
+        uint64_t at = first + (uint64_t)team * a.plane_units;
+        uint32_t off = off0;
+        for (uint32_t i = 0; i < cnt; ++i) {
+            t_cp_async_16(tile + i * kTThreads, xg + at);
+            if (kBwd && i < gcnt) t_cp_async_16(tileg + i * kTThreads, gyg + at);
+            advance(at, off);
+        }
+    }
+    for (uint32_t c = team; c < a.C; c += a.teams) {
+        t_cp_async_wait_all();
+        // ---- Eq. 4: range of this CTA's share ----
+        float mn[2] = {INFINITY, INFINITY}, mx[2] = {-INFINITY, -INFINITY};
+        for (uint32_t i = 0; i < cnt; ++i) {
+            Pack<T> p;
+            p.raw = tile[i * kTThreads];
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                const float v = p.get(e);
+                mn[e & 1] = fminf(mn[e & 1], v);
+                mx[e & 1] = fmaxf(mx[e & 1], v);
+            }
+        }
+        const float m0 = fminf(mn[0], mn[1]), m1 = fmaxf(mx[0], mx[1]);
+        uint32_t ka = m0 <= m1 ? ~enc(m0) : 0u, kb = m0 <= m1 ? enc(m1) : 0u;
+        ka = __reduce_max_sync(kFullMask, ka);
+        kb = __reduce_max_sync(kFullMask, kb);
+        if (lane == 0) {
+            s_kmn[tid >> 5] = ka;
+            s_kmx[tid >> 5] = kb;
+        }
+        __syncthreads();
+        if (tid < 32) {
+            ka = __reduce_max_sync(kFullMask, lane < kTWarps ? s_kmn[lane] : 0u);
+            kb = __reduce_max_sync(kFullMask, lane < kTWarps ? s_kmx[lane] : 0u);
+            if (lane == 0) {
+                atomicMax(a.kmin + c, ka);
+                atomicMax(a.kmax + c, kb);
+                t_arrive_release(a.counters + c);
+                // ---- wait (bounded) until the whole team has published the channel; Eq. 5 ----
+                uint32_t ready = 0;
+                for (uint32_t i = 0; i < a.spin_limit; ++i) {
+                    if (t_ld_acquire(a.counters + c) >= a.expected) {
+                        ready = 1;
+                        break;
+                    }
+                    __nanosleep(32);
+                }
+                s_ok = ready;
+                if (ready) {
+                    float lo, hi;
+                    const GroupParam gp = group_param_from_keys(a.kmin, a.kmax, c, qmax, lo, hi);
+                    s_par = gp;
+                    if (rank == 0) {
+                        a.lo[c] = lo;
+                        a.hi[c] = hi;
+                        if (a.s_out) a.s_out[c] = gp.s;
+                        if (a.z_out) a.z_out[c] = gp.z;
+                    }
+                } else {
+                    atomicExch(a.status, kTStatusTimeout);
+                }
+            }
+        }
+        __syncthreads();
+        if (!s_ok) return;      // nothing is in flight: the copies of this channel have landed, the next ones are not sent
+        const GroupParam g = s_par;
+
+        // ---- Eq. 1, clamp, Eq. 6, STE from shared memory; the next channel's copies follow on the heels ----
+        const bool more = c + a.teams < a.C;
+        const uint64_t ahead = (uint64_t)a.teams * a.plane_units;
+        auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint64_t at) {
+            Pack<T> py, pgx;
+            uint32_t cb[V / 4], mb[V / 4];
+            quantize_pack<T, kBwd, false, EXTRAS, true>(px, pg, g, g, V, qmax, py, pgx, cb, mb, EXTRAS == 3 ? a.code_bits : 8);
+            if constexpr (EXTRAS == 3) {
+                store_code_bytes<V>(a.pcodes, at * V, code_string_of<V>(cb, a.code_bits), a.code_bits, lane);
+                return;
+            }
+            st_hint_16(yg + at, py.raw, drop);
+            if constexpr (kBwd) st_hint_16(gxg + at, pgx.raw, drop);
+            if constexpr (EXTRAS == 4) dacc.add(px, py);
+            if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, at * V, mask_bits_of<V, EXTRAS>(mb), lane);
+        };
+        uint64_t at = first + (uint64_t)c * a.plane_units;
+        uint32_t off = off0, i = 0;
+        for (; i + U <= cnt; i += U) {
+            Pack<T> px[U], pg[U];
+            uint64_t w[U];
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                w[j] = at;
+                if constexpr (kBwd) {
+                    if (i + j < gcnt) pg[j].raw = tileg[(i + j) * kTThreads];
+                    else pg[j].raw = ld_hint_16(gyg + at, drop);
+                }
+                px[j].raw = tile[(i + j) * kTThreads];
+                advance(at, off);
+            }
+            if (more) {
+#pragma unroll
+                for (int j = 0; j < U; ++j) {
+                    t_cp_async_16(tile + (i + j) * kTThreads, xg + w[j] + ahead);
+                    if (kBwd && i + j < gcnt) t_cp_async_16(tileg + (i + j) * kTThreads, gyg + w[j] + ahead);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < U; ++j) emit(px[j], pg[j], w[j]);
+        }
+        for (; i < cnt; ++i) {
+            Pack<T> px, pg;
+            if constexpr (kBwd) {
+                if (i < gcnt) pg.raw = tileg[i * kTThreads];
+                else pg.raw = ld_hint_16(gyg + at, drop);
+            }
+            px.raw = tile[i * kTThreads];
+            if (more) {
+                t_cp_async_16(tile + i * kTThreads, xg + at + ahead);
+                if (kBwd && i < gcnt) t_cp_async_16(tileg + i * kTThreads, gyg + at + ahead);
+            }
+            emit(px, pg, at);
+            advance(at, off);
+        }
+    }
+    if constexpr (EXTRAS == 4) dacc.flush(a.dist);
+
+    // ---- leave the workspace as it was found: the last CTA to finish clears keys and counters ----
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        s_ok = (atomicAdd(a.counters + a.C, 1u) == gridDim.x - 1) ? 1u : 0u;
+    }
+    __syncthreads();
+    if (s_ok) {
+        for (uint32_t i = tid; i < a.C; i += kTThreads) {
+            a.kmin[i] = 0;
+            a.kmax[i] = 0;
+        }
+        for (uint32_t i = tid; i <= a.C; i += kTThreads) a.counters[i] = 0;
+    }
+}
+
+template <typename T, int MODE, int EXTRAS>
+cudaError_t t_launch(const TArgs& args, uint32_t smem, cudaStream_t st) {
+    auto kern = colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2)>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    void* params[] = {(void*)&args};
+    return cudaLaunchCooperativeKernel((const void*)kern, dim3(args.R * args.teams), dim3(kTThreads), params, smem, st);
+}
+
+template <typename T>
+cudaError_t t_launch_mode(const TArgs& a, int mode, int extras, uint32_t smem, cudaStream_t st) {
+    if (mode == MODE_BOTH) return t_launch<T, MODE_BOTH, 0>(a, smem, st);
+    switch (extras) {
+        case 2: return t_launch<T, MODE_FWD, 2>(a, smem, st);
+        case 3: return t_launch<T, MODE_FWD, 3>(a, smem, st);
+        case 4: return t_launch<T, MODE_FWD, 4>(a, smem, st);
+        default: return t_launch<T, MODE_FWD, 0>(a, smem, st);
+    }
+}
+
+}  // namespace
+
+// Team size: the number of CTAs R for which rounds x (share of one CTA + what a hand-over costs) is smallest, the
+// share fitting the shared memory of one of two CTAs per SM.
+TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count) {
+    TeamPlan p{};
+    p.ok = false;
+    const uint32_t V = dtype == 0 ? 4 : 8;
+    // whole units; codes and masks are written 8 elements at a time
+    if (g.inner % V != 0 || g.C >= (1ll << 28) || g.inner >= (1ll << 28)) return p;
+    if ((io.pmask || io.pcodes) && g.inner % 8 != 0) return p;
+    if (io.codes || io.mask) return p;
+    const uint64_t units = (uint64_t)g.outer * (uint64_t)(g.inner / V);
+    const uint32_t ctas = 2u * (uint32_t)sm_count;
+    if (units >= (1ull << 30) || units > (uint64_t)ctas * (kTSmemUnits - 8)) return p;
+    const uint32_t kHandOver = 512;      // what a hand-over costs, in units one CTA moves meanwhile (8 KB)
+    const uint32_t runs = (uint32_t)((units + 7) / 8), C = (uint32_t)g.C;
+    uint64_t best = ~0ull;
+    for (uint32_t R = 1; R <= ctas && R <= runs; ++R) {
+        const uint32_t share = 8 * ((runs + R - 1) / R);
+        if (share > kTSmemUnits) continue;
+        const uint32_t teams = std::min(ctas / R, C), rounds = (C + teams - 1) / teams;
+        const uint64_t cost = (uint64_t)rounds * (share + kHandOver);
+        if (cost < best) {
+            best = cost;
+            p.R = R;
+            p.teams = teams;
+            p.tile_units = share;
+        }
+    }
+    if (best == ~0ull) return p;
+    p.gy_units = backward ? std::min(p.tile_units, kTSmemUnits - p.tile_units) : 0u;
+    p.smem_bytes = 16u * (p.tile_units + p.gy_units);
+    p.ok = true;
+    return p;
+}
+
+cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
+                           const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,
+                           const StagedTuning& tune, cudaStream_t st) {
+    const uint32_t V = dtype == 0 ? 4 : 8;
+    TArgs a{};
+    a.x = io.x;
+    a.gy = io.gy;
+    a.y = io.y;
+    a.gx = io.gx;
+    a.pmask = io.pmask;
+    a.pcodes = io.pcodes;
+    a.code_bits = io.code_bits;
+    a.dist = io.dist;
+    a.status = ws.status;
+    a.kmin = ws.kmin;
+    a.kmax = ws.kmax;
+    a.counters = ws.counters;
+    a.lo = lo;
+    a.hi = hi;
+    a.s_out = s_opt;
+    a.z_out = z_opt;
+    a.qmax = (float)((1 << bits) - 1);
+    a.C = (uint32_t)g.C;
+    a.plane_units = (uint32_t)(g.inner / V);
+    a.units = (uint32_t)((uint64_t)g.outer * a.plane_units);
+    a.slab_units = (uint64_t)a.C * a.plane_units;
+    a.R = plan.R;
+    a.teams = plan.teams;
+    a.tile_units = plan.tile_units;
+    a.gy_units = plan.gy_units;
+    a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kTSpinLimit;
+    a.expected = plan.R + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
+    a.div_plane = make_fastdiv(a.plane_units);
+    const int extras = io.dist ? 4 : io.pmask ? 2 : io.pcodes ? 3 : 0;
+    return dtype == 0 ? t_launch_mode<float>(a, mode, extras, plan.smem_bytes, st)
+                      : t_launch_mode<__nv_bfloat16>(a, mode, extras, plan.smem_bytes, st);
+}
+
+}  // namespace granq

@@ -575,6 +575,11 @@ cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    // the resident form, unless a knob of the waves is set
+    if (tune.col_team != 2 && tune.l2_wave_kb <= 0 && tune.l2_lag <= 0 && tune.l2_ctas_per_sm <= 0) {
+        const TeamPlan tp = plan_colteam(dtype, g, io, mode == MODE_BOTH, sms);
+        if (tp.ok) return launch_colteam(tp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, tune, st);
+    }
     CArgs a{};
     a.x = io.x;
     a.gy = io.gy;

@@ -141,6 +141,7 @@ struct StagedTuning {
     int cl_prefetch;      // cluster plan: 1 = ask the L2 for gy while x is loading, 2 = do not
     int cl_kmul;          // cluster plan: multiplier of the minimal channel count of a run
     int cl_pdl;           // cluster plan: 2 = no programmatic dependent launch
+    int col_team;         // column-walk plan: 2 = L2 waves only
 };
 StagedPlan plan_staged(int dtype, const Geom& g, const QuantIO& io, int device, const StagedTuning& tune);
 StagedPlan plan_staged_on(int dtype, const Geom& g, const QuantIO& io, int sm_count, int smem_optin,
@@ -163,6 +164,18 @@ cudaError_t launch_l2wave(const L2Plan& plan, const QuantIO& io, int mode, int d
                           const StagedTuning& tune, cudaStream_t st);
 
 // ---- column-walk persistent kernel (L2-resident waves, one unit column per thread) ----------
+// Where a channel fits the shared memory of a team of CTAs the walk keeps it there (granq_colteam.cu).
+struct TeamPlan {
+    bool ok;
+    uint32_t R, teams;       // CTAs per team, teams
+    uint32_t tile_units;     // 16-byte units of x one CTA holds
+    uint32_t gy_units;       // units of gy it holds beside them
+    uint32_t smem_bytes;     // dynamic shared memory per CTA
+};
+TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count);
+cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
+                           const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,
+                           const StagedTuning& tune, cudaStream_t st);
 struct ColPlan {
     bool ok;
     uint32_t cw;             // channels per wave

@@ -1,0 +1,70 @@
+"""The resident form of the column walk (a channel held in the shared memory of a team of CTAs) against the CPU
+oracle, bit for bit: teams of one CTA and of many, one round of channels and several, shares that are not whole
+runs of 8 units, planes shorter and longer than a block's stride, gy staged whole and in part - with every output
+that the form writes, between guard bands, the workspace zero again afterwards."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import assert_parity, make_case, same_bits, to_dev, to_np
+from oracle import granq_oracle as orc
+from test_parity_gpu import b, knobs  # noqa: F401
+from test_rounding_gpu import assert_same_string
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    (8, 400, 8, 8),      # one CTA per channel, two rounds
+    (13, 700, 2, 4),     # planes of one bf16 unit
+    (9, 24, 12, 12),     # several CTAs per channel, one round
+    (8, 3, 4, 4),        # fewer units than a team could share
+    (33, 310, 4, 8),     # rounds that do not come out even
+    (11, 5, 20, 22),     # planes that are no multiple of the block
+    (8, 4, 112, 112),    # planes longer than a block's stride
+    (128, 16, 56, 56),   # shares beyond half the shared memory: gy staged in part
+    (64, 300, 20, 20),   # two CTAs per channel and the next channel's copies on the heels of this one's
+]
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_resident_walk(b, knobs, shape, dtype):
+    x, gy = make_case(shape, seed=sum(shape), dtype=dtype, relu=shape[0] % 2 == 0)
+    bits = 2 + sum(shape) % 7
+    ref = orc.fused(x, bits, gy=gy)
+    xd, gyd = to_dev(x), to_dev(gy)
+    flags = b.FLAG_FORCE_COLWALK | b.FLAG_WORKSPACE_ZEROED
+    ws = b.make_workspace(xd, zeroed=True)
+    clean = lambda: b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
+    for _ in range(2):
+        got = b.granq_fakequant_fused(xd, bits, gy=gyd, out=b.FakeQuantOut(workspace=ws), want_params=True, flags=flags)
+        assert clean()
+        assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=True)
+    got = b.granq_fakequant_fused(xd, bits, out=b.FakeQuantOut(workspace=ws), flags=flags)
+    assert clean()
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    if (shape[1] * shape[2] * shape[3]) % 32 == 0:
+        got = b.granq_fakequant_fused_fwd_packmask(xd, bits, out=b.FakeQuantOut(workspace=ws), flags=flags)
+        assert clean()
+        assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+        assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+        got = b.granq_quantize_packed_fused(xd, bits, out=b.FakeQuantOut(workspace=ws), flags=flags)
+        assert clean()
+        assert_same_string(got.packed_codes, orc.pack_codes(ref.codes, bits))
+    got = b.granq_fakequant_fused_stats(xd, bits, out=b.FakeQuantOut(workspace=ws), flags=flags)
+    assert clean()
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    sums = orc.distortion_sums(x, ref.y)
+    # fp32 inside a pack, fp64 beyond: about 8 roundings of 2^-24 of a sum of same-signed terms
+    assert np.allclose(to_np(got.sums), sums, rtol=1e-6, atol=0)
+
+
+def test_a_hand_over_that_never_completes_is_reported(b, knobs):
+    x, gy = make_case((8, 24, 12, 12), seed=1)
+    knobs(extra_arrivals=1, spin_limit=500)
+    got = b.granq_fakequant_fused(to_dev(x), 4, gy=to_dev(gy), flags=b.FLAG_FORCE_COLWALK)
+    assert b.workspace_status(got.workspace) == b.ERR_TIMEOUT
+    knobs(extra_arrivals=0, spin_limit=0)
+    got = b.granq_fakequant_fused(to_dev(x), 4, gy=to_dev(gy), flags=b.FLAG_FORCE_COLWALK)
+    assert b.workspace_status(got.workspace) == b.OK
+    assert same_bits(to_np(got.y), orc.fused(x, 4, gy=gy).y)
