@@ -73,8 +73,8 @@ int choose_plan(int dtype, const Geom& g, const QuantIO& io, bool backward, uint
     ColPlan cp{};
     cp.ok = false;
     // Measured exception: forward-only bf16 tensors of 48 MB and more (a 100 KB tile then holds 51 200 elements
-    // and a CTA's chain of copy, fold and quantize is twice as long as for fp32) run 6-15 % faster on the
-    // column walk; with a gradient, and for fp32, the cluster-local kernel wins wherever it fits.
+    // and a CTA's chain of copy, fold and quantize is twice as long as for fp32) run faster on the column walk in
+    // its resident form ([256,512,28,28] 104 / 92 us); with a gradient, and for fp32, see prefer_team() below.
     const bool long_chain = dtype == 1 && !backward && !(io.codes || io.mask || io.pmask || io.dist) &&
                             (uint64_t)g.E * 2 >= (48ull << 20);
     if (kp.ok && long_chain) {
@@ -99,6 +99,30 @@ int choose_plan(int dtype, const Geom& g, const QuantIO& io, bool backward, uint
         return PLAN_L2WAVE;
     }
     return PLAN_TWO_PASS;
+}
+
+// Where the cluster-local plan takes a call by default, the form in which its channels are held: one cluster per
+// channel, or (this returns a plan) teams of CTAs of one cooperative launch.  Both read x once; the cluster starts
+// sooner (its launch overlaps the kernel ahead) and hands over faster, the team is dealt out evenly, keeps reads in
+// flight while it writes and needs no GPC with eight free CTAs.  Measured (cluster / team, us): the team from 96 MB
+// of x and 256 KB per channel on - fp32 [256,512,28,28] forward 169 / 156, with gradient 319 / 298, packed mask
+// 227 / 174, codes 276 / 202; [64,256,56,56] 89 / 81, 157 / 150, 125 / 91, codes 155 / 106; bf16 63 / 56, 86 / 84 -
+// and the cluster below: [128,192,28,28] 37 / 38, 62 / 62; [256,256,16,16] 33 / 40; [32,64,56,56] 17 / 19, and with
+// small channels: [256,1024,14,14] 87 / 88, 159 / 163.  fp32 with a gradient crosses later ([128,256,28,28], 98 MB:
+// 80 / 83).
+TeamPlan prefer_team(int dtype, const Geom& g, const QuantIO& io, bool backward, uint32_t flags) {
+    TeamPlan none{};
+    if (flags & GRANQ_FLAG_FORCE_CLUSTER) return none;
+    const StagedTuning& t = g_tune;
+    if (t.cl_tile_kb || t.cl_r || t.cl_threads || t.cl_load || t.cl_prefetch || t.cl_kmul || t.cl_pdl || t.col_team) return none;
+    const uint64_t bytes = (uint64_t)g.E * elt_size(dtype);
+    const uint64_t from = (backward && dtype == GRANQ_F32 ? 128ull : 96ull) << 20;
+    if (bytes < from || bytes / (uint64_t)g.C < (256ull << 10)) return none;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return none;
+    return plan_colteam(dtype, g, io, backward, sms);
 }
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -221,14 +245,18 @@ int granq_fakequant_fused(const void* x, const void* gy_opt, int dtype, const in
     // keep that word true for the next call, after.
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     const bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER;
+    TeamPlan tp{};
+    if (plan == PLAN_CLUSTER) tp = prefer_team(dtype, g, io, gy_opt != nullptr, flags);
     cudaError_t e = cudaSuccess;
-    if (plan == PLAN_CLUSTER) {
+    if (plan == PLAN_CLUSTER && !tp.ok) {
         if (!zeroed) e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);      // the status word
     } else if (!(zeroed && keeps_zero)) {
         e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
     }
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
-    if (plan == PLAN_CLUSTER) {
+    if (tp.ok) {
+        e = launch_colteam(tp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
+    } else if (plan == PLAN_CLUSTER) {
         e = launch_cluster(kp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else if (plan == PLAN_ROWS) {
         e = launch_rows(io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st);
@@ -322,11 +350,15 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
     Workspace ws = carve_workspace(workspace, G);
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     cudaError_t e = cudaSuccess;
+    const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     if (kp.ok) {
-        if (!zeroed) e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);      // the status word
+        if (!zeroed) e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
         // the kernel writes the mask byte by byte: the padding bits of a last, partial word are cleared here
         if (e == cudaSuccess && g.E % 32 != 0) e = cudaMemsetAsync(packed_mask + g.E / 32, 0, sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
+        if (tp.ok)
+            return cuda_status(launch_colteam(tp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt,
+                                              g_tune, st));
         return cuda_status(launch_cluster(kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt,
                                           g_tune, st));
     }
@@ -413,9 +445,13 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
     Workspace ws = carve_workspace(workspace, G);
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     cudaError_t e = cudaMemsetAsync(sums_out, 0, 4 * sizeof(double), st);
+    const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     if (e == cudaSuccess && kp.ok) {
-        if (!zeroed) e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);      // the status word
+        if (!zeroed) e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
+        if (tp.ok)
+            return cuda_status(launch_colteam(tp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt,
+                                              g_tune, st));
         return cuda_status(launch_cluster(kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt,
                                           g_tune, st));
     }
@@ -487,9 +523,13 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
     Workspace ws = carve_workspace(workspace, G);
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     cudaError_t e = cudaSuccess;
+    const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     if (kp.ok) {
-        if (!zeroed) e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);      // the status word
+        if (!zeroed) e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
+        if (tp.ok)
+            return cuda_status(launch_colteam(tp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out,
+                                              g_tune, st));
         return cuda_status(launch_cluster(kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out,
                                           g_tune, st));
     }

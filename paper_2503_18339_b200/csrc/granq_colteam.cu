@@ -306,14 +306,16 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
     const uint64_t units = (uint64_t)g.outer * (uint64_t)(g.inner / V);
     const uint32_t ctas = 2u * (uint32_t)sm_count;
     if (units >= (1ull << 30) || units > (uint64_t)ctas * (kTSmemUnits - 8)) return p;
-    const uint32_t kHandOver = 512;      // what a hand-over costs, in units one CTA moves meanwhile (8 KB)
+    // What a hand-over costs, in units that one CTA moves meanwhile: about 3 us, from sweeps over R (forward
+    // [128,64,56,56]: 4 rounds of 5576 units 47 us, 8 of 2720 60 us, 16 of 1360 85 us; with gradient 84, 90, 115 us).
+    const uint32_t hand_over = backward ? 700 : 2000;
     const uint32_t runs = (uint32_t)((units + 7) / 8), C = (uint32_t)g.C;
     uint64_t best = ~0ull;
     for (uint32_t R = 1; R <= ctas && R <= runs; ++R) {
         const uint32_t share = 8 * ((runs + R - 1) / R);
         if (share > kTSmemUnits) continue;
         const uint32_t teams = std::min(ctas / R, C), rounds = (C + teams - 1) / teams;
-        const uint64_t cost = (uint64_t)rounds * (share + kHandOver);
+        const uint64_t cost = (uint64_t)rounds * (share + hand_over);
         if (cost < best) {
             best = cost;
             p.R = R;

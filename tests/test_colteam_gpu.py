@@ -68,3 +68,24 @@ def test_a_hand_over_that_never_completes_is_reported(b, knobs):
     got = b.granq_fakequant_fused(to_dev(x), 4, gy=to_dev(gy), flags=b.FLAG_FORCE_COLWALK)
     assert b.workspace_status(got.workspace) == b.OK
     assert same_bits(to_np(got.y), orc.fused(x, 4, gy=gy).y)
+
+
+@pytest.mark.parametrize("dtype,shape", [("f32", (256, 168, 28, 28)), ("bf16", (256, 256, 28, 28))])
+def test_large_tensors_take_the_resident_form_by_default(b, dtype, shape):
+    """The first sizes that the default route hands to the resident form although a cluster would hold a channel,
+    with a workspace that is not zero on entry; forward and with a gradient, packed mask, packed codes, sums."""
+    x, gy = make_case(shape, seed=5, dtype=dtype)
+    ref = orc.fused(x, 4, gy=gy)
+    xd, gyd = to_dev(x), to_dev(gy)
+    ws = b.make_workspace(xd)
+    new = lambda: b.FakeQuantOut(workspace=ws.fill_(255))
+    assert_parity(b.granq_fakequant_fused(xd, 4, out=new()), ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert_parity(b.granq_fakequant_fused(xd, 4, gy=gyd, out=new()), ref, shape, 1, orc.GROUP_CHANNEL, backward=True)
+    got = b.granq_fakequant_fused_fwd_packmask(xd, 4, out=new())
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+    got = b.granq_quantize_packed_fused(xd, 4, out=new())
+    assert_same_string(got.packed_codes, orc.pack_codes(ref.codes, 4))
+    got = b.granq_fakequant_fused_stats(xd, 4, out=new())
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert b.workspace_status(ws) == b.OK
