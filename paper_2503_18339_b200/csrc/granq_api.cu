@@ -239,12 +239,12 @@ int granq_fakequant_fused(const void* x, const void* gy_opt, int dtype, const in
     if (plan < 0) return -plan;
 
     Workspace ws = carve_workspace(workspace, G);
-    // The column-walk kernel leaves a zeroed workspace zeroed and the cluster-local kernel writes
+    // The column-walk and channels-last kernels leave a zeroed workspace zeroed and the cluster-local kernel writes
     // nothing but the status word (and that only when a wait ran out); with the caller's word that
     // the workspace is zero on entry nothing has to be cleared.  The other plans clear before and, to
     // keep that word true for the next call, after.
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
-    const bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER;
+    const bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS;
     TeamPlan tp{};
     if (plan == PLAN_CLUSTER) tp = prefer_team(dtype, g, io, gy_opt != nullptr, flags);
     cudaError_t e = cudaSuccess;
@@ -259,7 +259,7 @@ int granq_fakequant_fused(const void* x, const void* gy_opt, int dtype, const in
     } else if (plan == PLAN_CLUSTER) {
         e = launch_cluster(kp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else if (plan == PLAN_ROWS) {
-        e = launch_rows(io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st);
+        e = launch_rows(io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else if (plan == PLAN_STAGED) {
         e = launch_staged(sp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else if (plan == PLAN_L2WAVE) {
@@ -645,8 +645,7 @@ int granq_fused_plan(int dtype, const int64_t dims[4], int channel_axis, int gro
     QuantIO io{};   // null pointers: alignment is assumed
     const int plan = choose_plan(dtype, g, io, with_backward != 0, flags, nullptr, nullptr, nullptr, nullptr);
     if (launches_out) {
-        if (plan == PLAN_STAGED || plan == PLAN_L2WAVE || plan == PLAN_COLWALK || plan == PLAN_CLUSTER) *launches_out = 1;
-        else if (plan == PLAN_ROWS) *launches_out = 2;
+        if (plan == PLAN_STAGED || plan == PLAN_L2WAVE || plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS) *launches_out = 1;
         else if (plan == PLAN_NAIVE) *launches_out = (int)(3 * g.C);
         else if (plan == PLAN_TWO_PASS) *launches_out = 3;
     }

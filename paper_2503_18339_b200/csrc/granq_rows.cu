@@ -1,17 +1,24 @@
-// Channels-last GranQ kernels: geometries whose channel is the innermost axis ([N, H, W, C] with the
+// Channels-last GranQ kernel: geometries whose channel is the innermost axis ([N, H, W, C] with the
 // channel axis last, or [N, C, 1, 1]), i.e. a row-major matrix [rows, C] with one group per column.
 //
-// Every channel is spread over the whole tensor, so nothing can be quantized before all of it has been
-// read: x is read twice (20 instead of 16 bytes per element with a gradient; the second read comes from
-// the L2 when the tensor fits), and two plain launches are the right shape - there is nothing for a
-// grid-wide hand-over to save.  What makes them fast is the mapping: a 16-byte unit holds V consecutive
-// channels of one row, so a thread keeps ONE unit column and walks it down the rows;
-//   range pass (Eq. 4):    per-element running min / max stay in registers for the whole walk, are folded
-//                          per channel in shared memory and reach global memory as one pair of atomics per
-//                          channel and CTA;
-//   quantize pass (Eq. 5, 1, 6, STE): the CTA turns the keys into a table of (s, z, 1/s) once; a thread
-//                          loads the V parameter sets of its column once and then streams.
-// Neither pass divides an index or looks anything up inside the walk.
+// Every channel is spread over the whole tensor, so nothing can be quantized before all of it has been read.  One
+// cooperative launch, two CTAs per SM.  The matrix is cut into slices of 16 .. 64 unit columns (a 16-byte unit holds V
+// consecutive channels), and a team of CTAs owns a slice: channels of different slices have nothing to do with each
+// other, so what a CTA does per channel (keys, atomics, parameters) stays small however wide the rows are, and nobody
+// waits for another slice.  The CTAs of a team take turns at blocks of rows; each keeps its blocks in shared memory
+// between the two halves of the work where all of them fit (33 MB over the GPU):
+//   range (Eq. 4):  rows that will be kept are sent for with per-thread asynchronous copies, others are read
+//                   directly; a thread keeps ONE unit column, its running min / max per channel are folded
+//                   in shared memory and reach global memory as one pair of atomics per channel and CTA;
+//   hand-over:      one arrival per CTA and a bounded wait for the team;
+//   quantize (Eq. 5, 1, 6, STE): the CTA turns the slice's keys into a table of parameters once; a thread loads the V
+//                   sets of its column and streams, from shared memory or, rows that were not kept, from memory again: the
+//                   last read first, as the likeliest to still be in the L2.
+// Neither half divides an index or looks anything up inside the walk.
+// Bound by HBM for the streams of the second half, by the hand-over (about 3 us) for small tensors.  Against a
+// range launch and a quantize launch that spread every channel over all CTAs (us, forward / with gradient): bf16
+// [128,28,28,192] 42 / 49 -> 31 / 42, [17,14,14,2048] 30 / 36 -> 19 / 23; fp32 [15,22,22,784] 30 / 38 -> 19 / 28,
+// [31,28,28,2048] 134 / 179 -> 101 / 162, [16,32,32,16] 17 / 18 -> 10 / 10; [128,112,112,64] 243 / 327 -> 208 / 336.
 #include "granq_internal.h"
 
 #include <algorithm>
@@ -20,8 +27,13 @@ namespace granq {
 
 namespace {
 
-constexpr int kRThreads = 256;
-constexpr uint32_t kRMaxChannels = 4096;      // keys / parameter table in shared memory
+// Threads of a CTA at most: two CTAs leave 72 registers per thread to fp32 and 80 to bf16 (V sets of parameters each).
+template <typename T>
+constexpr int kRMaxThreads = Pack<T>::V == 4 ? 448 : 384;
+constexpr uint32_t kRMaxChannels = 4096;      // 64 slices at most
+constexpr uint32_t kRSmemBytes = 111u * 1024; // of one of two CTAs on an SM
+constexpr uint32_t kRSpinLimit = 1u << 24;    // bounded wait on the grid (x ~32 ns)
+constexpr uint32_t kRStatusTimeout = 5;       // GRANQ_ERR_TIMEOUT
 
 struct RArgs {
     const void* x;
@@ -30,8 +42,10 @@ struct RArgs {
     void* gx;
     uint8_t* codes;
     uint8_t* mask;
+    uint32_t* status;
     uint32_t* kmin;
     uint32_t* kmax;
+    uint32_t* counters;
     float* lo;
     float* hi;
     float* s_out;
@@ -39,36 +53,62 @@ struct RArgs {
     float qmax;
     uint32_t C;          // channels
     uint32_t ncol;       // 16-byte units per row
+    uint32_t P;          // unit columns of a slice
+    uint32_t slices;
+    uint32_t team;       // CTAs per slice
+    uint32_t lanes;      // rows of threads: the rows of one block
+    uint32_t hold;       // blocks of rows a CTA keeps in shared memory
+    uint32_t lost;       // of the others, those before this one are not expected to be in the L2 when they are read again
+    uint32_t spin_limit, expected;
     uint64_t rows;
 };
 
-// the walk of thread t of CTA b: unit column tile0 + t % P, rows (b * nrows + t / P), + gridDim * nrows, ...
-struct RWalk {
-    uint32_t P, nrows, r0, cin;
-    bool rowed;
-    __device__ __forceinline__ RWalk(uint32_t ncol) {
-        P = min(ncol, (uint32_t)kRThreads);
-        nrows = kRThreads / P;
-        r0 = threadIdx.x / P;
-        cin = threadIdx.x - r0 * P;
-        rowed = r0 < nrows;
-    }
-};
+__device__ __forceinline__ uint32_t r_ld_acquire(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void r_cp_async_16(void* dst_smem, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)), "l"(src)
+                 : "memory");
+}
 
-template <typename T, int U>
-__global__ void __launch_bounds__(kRThreads, 4) rows_range_kernel(const RArgs a) {
+// U1 / U2 = rows a thread has in flight in the range / quantize walk
+template <typename T, int MODE, bool EXTRAS, int U1, int U2>
+__global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a) {
     constexpr int V = Pack<T>::V;
-    extern __shared__ uint32_t r_keys[];          // C min keys, C max keys
-    uint32_t* s_kmn = r_keys;
-    uint32_t* s_kmx = r_keys + a.C;
-    for (uint32_t t = threadIdx.x; t < 2 * a.C; t += kRThreads) r_keys[t] = 0;
+    constexpr bool kBwd = (MODE & MODE_BWD) != 0;
+    extern __shared__ __align__(16) unsigned char r_smem[];
+    // first the keys (min, max: element i of unit column c at i * P + c), later the parameter table, then the rows
+    uint32_t* s_kmn = reinterpret_cast<uint32_t*>(r_smem);
+    uint32_t* s_kmx = s_kmn + a.P * V;
+    GroupParam* s_par = reinterpret_cast<GroupParam*>(r_smem);
+    __shared__ uint32_t s_ok;
+    const uint32_t tid = threadIdx.x, NT = blockDim.x, P = a.P, L = a.lanes;
+    const uint32_t slice = blockIdx.x / a.team, rank = blockIdx.x - slice * a.team;
+    const uint32_t col0 = slice * P, width = min(P, a.ncol - col0), ch0 = col0 * V, chans = width * V;
+    const uint32_t r0 = tid / P, cin = tid - r0 * P;
+    // this thread's rows: row first + k * stride, k < n; the first `held` of them stay in shared memory
+    const uint64_t first = (uint64_t)rank * L + r0, stride = (uint64_t)a.team * L;
+    const uint32_t n = (r0 < L && cin < width && first < a.rows) ? (uint32_t)((a.rows - 1 - first) / stride) + 1 : 0u;
+    const uint32_t held = min(n, a.hold);
+    const uint64_t origin = first * a.ncol + col0 + cin;
+    const size_t step = (size_t)stride * a.ncol;
+    const uint4* xg = reinterpret_cast<const uint4*>(a.x) + origin;
+    const uint4* gyg = reinterpret_cast<const uint4*>(a.gy) + origin;
+    uint4* yg = reinterpret_cast<uint4*>(a.y) + origin;
+    uint4* gxg = reinterpret_cast<uint4*>(a.gx) + origin;
+    uint4* tile = reinterpret_cast<uint4*>(r_smem + (size_t)P * V * sizeof(GroupParam)) + r0 * P + cin;
+    const uint32_t tstep = L * P;
+    const float qmax = a.qmax;
+    const uint64_t drop = l2_policy_evict_first();
+
+    for (uint32_t k = 0; k < held; ++k) r_cp_async_16(tile + k * tstep, xg + k * step);
+    for (uint32_t t = tid; t < 2 * P * V; t += NT) s_kmn[t] = 0;
     __syncthreads();
-    const RWalk w(a.ncol);
-    const uint4* xg = reinterpret_cast<const uint4*>(a.x);
-    const uint64_t first = (uint64_t)blockIdx.x * w.nrows + w.r0, step = (uint64_t)gridDim.x * w.nrows;
-    for (uint32_t tile0 = 0; tile0 < a.ncol; tile0 += w.P) {
-        const uint32_t col = tile0 + w.cin;
-        if (!w.rowed || col >= a.ncol) continue;
+
+    // ---- Eq. 4: rows beyond the kept ones straight from memory, then the kept ones ----
+    {
         float mn[V], mx[V];
 #pragma unroll
         for (int i = 0; i < V; ++i) {
@@ -83,69 +123,81 @@ __global__ void __launch_bounds__(kRThreads, 4) rows_range_kernel(const RArgs a)
                 mx[i] = fmaxf(mx[i], v);
             }
         };
-        uint64_t r = first;
-        for (; r + (uint64_t)(U - 1) * step < a.rows; r += (uint64_t)U * step) {
-            Pack<T> v[U];
+        const uint4* src = xg + held * step;
+        for (uint32_t k = held; k < n; k += U1, src += U1 * step) {
+            Pack<T> v[U1];
 #pragma unroll
-            for (int j = 0; j < U; ++j) v[j].raw = ld_stream_16(xg + (r + (uint64_t)j * step) * a.ncol + col);
+            for (int j = 0; j < U1; ++j)
+                if (k + j < n) v[j].raw = k < a.lost ? ld_hint_16(src + j * step, drop) : __ldg(src + j * step);
 #pragma unroll
-            for (int j = 0; j < U; ++j) add(v[j]);
+            for (int j = 0; j < U1; ++j)
+                if (k + j < n) add(v[j]);
         }
-        for (; r < a.rows; r += step) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        for (uint32_t k = 0; k < held; ++k) {
             Pack<T> v;
-            v.raw = ld_stream_16(xg + r * a.ncol + col);
+            v.raw = tile[k * tstep];
             add(v);
         }
-        if (first < a.rows) {
+        if (n > 0) {
 #pragma unroll
             for (int i = 0; i < V; ++i) {
-                atomicMax(s_kmn + col * V + i, ~enc(mn[i]));
-                atomicMax(s_kmx + col * V + i, enc(mx[i]));
+                atomicMax(s_kmn + i * P + cin, mn[i] <= mx[i] ? ~enc(mn[i]) : 0u);
+                atomicMax(s_kmx + i * P + cin, mn[i] <= mx[i] ? enc(mx[i]) : 0u);
             }
         }
     }
     __syncthreads();
-    for (uint32_t t = threadIdx.x; t < a.C; t += kRThreads) {
-        const uint32_t k1 = s_kmn[t], k2 = s_kmx[t];
+    for (uint32_t t = tid; t < chans; t += NT) {           // channel t of the slice: element t % V of unit column t / V
+        const uint32_t at = (t % V) * P + t / V, k1 = s_kmn[at], k2 = s_kmx[at];
         if (k1 | k2) {
-            atomicMax(a.kmin + t, k1);
-            atomicMax(a.kmax + t, k2);
+            atomicMax(a.kmin + ch0 + t, k1);
+            atomicMax(a.kmax + ch0 + t, k2);
         }
     }
-}
-
-template <typename T, int MODE, bool EXTRAS, int U>
-__global__ void __launch_bounds__(kRThreads, 3) rows_quant_kernel(const RArgs a) {
-    constexpr int V = Pack<T>::V;
-    constexpr bool kBwd = (MODE & MODE_BWD) != 0;
-    extern __shared__ GroupParam r_par[];         // one (s, z, 1/s) per channel
-    for (uint32_t t = threadIdx.x; t < a.C; t += kRThreads) {
+    // ---- the team's hand-over (bounded) ----
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        atomicAdd(a.counters + slice, 1u);
+        uint32_t ready = 0;
+        for (uint32_t i = 0; i < a.spin_limit; ++i) {
+            if (r_ld_acquire(a.counters + slice) >= a.expected) {
+                ready = 1;
+                break;
+            }
+            __nanosleep(32);
+        }
+        s_ok = ready;
+        if (!ready) atomicExch(a.status, kRStatusTimeout);
+    }
+    __syncthreads();
+    if (!s_ok) return;
+    for (uint32_t t = tid; t < chans; t += NT) {
         float lo, hi;
-        const GroupParam gp = group_param_from_keys(a.kmin, a.kmax, t, a.qmax, lo, hi);
-        r_par[t] = gp;
-        if (blockIdx.x == 0) {
-            a.lo[t] = lo;
-            a.hi[t] = hi;
-            if (a.s_out) a.s_out[t] = gp.s;
-            if (a.z_out) a.z_out[t] = gp.z;
+        const GroupParam gp = group_param_from_keys(a.kmin, a.kmax, ch0 + t, qmax, lo, hi);
+        s_par[t] = gp;
+        if (rank == 0) {
+            a.lo[ch0 + t] = lo;
+            a.hi[ch0 + t] = hi;
+            if (a.s_out) a.s_out[ch0 + t] = gp.s;
+            if (a.z_out) a.z_out[ch0 + t] = gp.z;
         }
     }
     __syncthreads();
-    const RWalk w(a.ncol);
-    const uint4* xg = reinterpret_cast<const uint4*>(a.x);
-    const uint4* gyg = reinterpret_cast<const uint4*>(a.gy);
-    uint4* yg = reinterpret_cast<uint4*>(a.y);
-    uint4* gxg = reinterpret_cast<uint4*>(a.gx);
-    const uint64_t first = (uint64_t)blockIdx.x * w.nrows + w.r0, step = (uint64_t)gridDim.x * w.nrows;
-    const float qmax = a.qmax;
-    for (uint32_t tile0 = 0; tile0 < a.ncol; tile0 += w.P) {
-        const uint32_t col = tile0 + w.cin;
-        if (!w.rowed || col >= a.ncol) continue;
+    if (tid == 0) {          // the keys have been read; the last CTA to say so leaves the workspace zero (below)
+        __threadfence();
+        s_ok = (atomicAdd(a.counters + a.slices, 1u) == gridDim.x - 1) ? 1u : 0u;
+    }
+
+    // ---- Eq. 1, clamp, Eq. 6, STE ----
+    if (n > 0) {
+        const GroupParam* par = s_par + cin * V;
         float s[V], rc[V], mz[V], thr = 1.0f;
         bool clamped = false;
 #pragma unroll
         for (int i = 0; i < V; ++i) {
-            const GroupParam g = r_par[col * V + i];
+            const GroupParam g = par[i];
             s[i] = g.s;
             rc[i] = g.r;
             mz[i] = __fadd_rn(kRoundMagic, g.z);
@@ -153,57 +205,87 @@ __global__ void __launch_bounds__(kRThreads, 3) rows_quant_kernel(const RArgs a)
             clamped |= g.thr < 0.0f;
         }
         if (clamped) thr = -thr;
-        auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint64_t at) {
+        auto emit = [&](const Pack<T>& px, const Pack<T>& pg, size_t at) {
             Pack<T> py, pgx;
             uint32_t cb[V / 4], mb[V / 4];
-            quantize_pack_each<T, kBwd, EXTRAS>(px, pg, s, rc, mz, thr, r_par + col * V, qmax, py, pgx, cb, mb);
+            quantize_pack_each<T, kBwd, EXTRAS>(px, pg, s, rc, mz, thr, par, qmax, py, pgx, cb, mb);
             st_stream_16(yg + at, py.raw);
             if constexpr (kBwd) st_stream_16(gxg + at, pgx.raw);
             if constexpr (EXTRAS) {
+                const size_t w = (origin + at) * (V / 4);
                 if (a.codes) {
 #pragma unroll
-                    for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.codes)[at * (V / 4) + i] = cb[i];
+                    for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.codes)[w + i] = cb[i];
                 }
                 if (kBwd && a.mask) {
 #pragma unroll
-                    for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.mask)[at * (V / 4) + i] = mb[i];
+                    for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.mask)[w + i] = mb[i];
                 }
             }
         };
-        uint64_t r = first;
-        for (; r + (uint64_t)(U - 1) * step < a.rows; r += (uint64_t)U * step) {
-            Pack<T> px[U], pg[U];
+        // rows that were not kept, from the last one back
+        {
+            uint32_t left = n - held;
+            size_t at = (size_t)(n - 1) * step;
+            for (; left >= (uint32_t)U2; left -= U2, at -= U2 * step) {
+                Pack<T> px[U2], pg[U2];
 #pragma unroll
-            for (int j = 0; j < U; ++j) {
-                const uint64_t at = (r + (uint64_t)j * step) * a.ncol + col;
-                px[j].raw = ld_stream_16(xg + at);
-                if constexpr (kBwd) pg[j].raw = ld_stream_16(gyg + at);
+                for (int j = 0; j < U2; ++j) {
+                    px[j].raw = ld_stream_16(xg + (at - j * step));
+                    if constexpr (kBwd) pg[j].raw = ld_stream_16(gyg + (at - j * step));
+                }
+#pragma unroll
+                for (int j = 0; j < U2; ++j) emit(px[j], pg[j], at - j * step);
             }
-#pragma unroll
-            for (int j = 0; j < U; ++j) emit(px[j], pg[j], (r + (uint64_t)j * step) * a.ncol + col);
+            for (; left > 0; --left, at -= step) {
+                Pack<T> px, pg;
+                px.raw = ld_stream_16(xg + at);
+                if constexpr (kBwd) pg.raw = ld_stream_16(gyg + at);
+                emit(px, pg, at);
+            }
         }
-        for (; r < a.rows; r += step) {
-            const uint64_t at = r * a.ncol + col;
+        // the kept ones
+        size_t at = 0;
+        uint32_t k = 0;
+        for (; k + U2 <= held; k += U2, at += U2 * step) {
+            Pack<T> px[U2], pg[U2];
+#pragma unroll
+            for (int j = 0; j < U2; ++j)
+                if constexpr (kBwd) pg[j].raw = ld_stream_16(gyg + at + j * step);
+#pragma unroll
+            for (int j = 0; j < U2; ++j) px[j].raw = tile[(k + j) * tstep];
+#pragma unroll
+            for (int j = 0; j < U2; ++j) emit(px[j], pg[j], at + j * step);
+        }
+        for (; k < held; ++k, at += step) {
             Pack<T> px, pg;
-            px.raw = ld_stream_16(xg + at);
             if constexpr (kBwd) pg.raw = ld_stream_16(gyg + at);
+            px.raw = tile[k * tstep];
             emit(px, pg, at);
         }
+    }
+    __syncthreads();
+    if (s_ok) {
+        for (uint32_t t = tid; t < a.C; t += NT) {
+            a.kmin[t] = 0;
+            a.kmax[t] = 0;
+        }
+        for (uint32_t t = tid; t <= a.slices; t += NT) a.counters[t] = 0;
     }
 }
 
 bool r_aligned16(const void* p) { return p == nullptr || ((uintptr_t)p & 15) == 0; }
 
 template <typename T, int MODE>
-cudaError_t r_launch_quant(const RArgs& a, bool extras, int grid, cudaStream_t st) {
-    const size_t smem = (size_t)a.C * sizeof(GroupParam);
+cudaError_t r_launch(const RArgs& a, bool extras, int grid, int threads, size_t smem, cudaStream_t st) {
     auto go = [&](auto kern) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<grid, kRThreads, smem, st>>>(a);
-        return cudaGetLastError();
+        void* params[] = {(void*)&a};
+        return cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(threads), params, smem, st);
     };
-    return extras ? go(rows_quant_kernel<T, MODE, true, 2>) : go(rows_quant_kernel<T, MODE, false, 2>);
+    constexpr int U1 = Pack<T>::V == 4 ? 8 : 6;
+    return extras ? go(rows_kernel<T, MODE, true, U1, 2>) : go(rows_kernel<T, MODE, false, U1, 2>);
 }
 
 }  // namespace
@@ -219,7 +301,7 @@ bool plan_rows(int dtype, const Geom& g, const QuantIO& io) {
 }
 
 cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, int bits, const Workspace& ws,
-                        float* lo, float* hi, float* s_opt, float* z_opt, cudaStream_t st) {
+                        float* lo, float* hi, float* s_opt, float* z_opt, const StagedTuning& tune, cudaStream_t st) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -233,8 +315,10 @@ cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, i
     a.gx = io.gx;
     a.codes = io.codes;
     a.mask = io.mask;
+    a.status = ws.status;
     a.kmin = ws.kmin;
     a.kmax = ws.kmax;
+    a.counters = ws.counters;
     a.lo = lo;
     a.hi = hi;
     a.s_out = s_opt;
@@ -243,32 +327,42 @@ cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, i
     a.C = (uint32_t)g.C;
     a.ncol = (uint32_t)(g.C / V);
     a.rows = (uint64_t)g.outer;
-    // row lanes in the grid: no more CTAs than there are rows to give each row lane at least one
-    const uint32_t P = std::min<uint32_t>(a.ncol, kRThreads), nrows = kRThreads / P;
-    const uint64_t want = (a.rows + nrows - 1) / nrows;
-    const int grid_r = (int)std::min<uint64_t>(want, (uint64_t)sms * 4);
-    const int grid_q = (int)std::min<uint64_t>(want, (uint64_t)sms * 3);
-    const size_t smem_r = (size_t)a.C * 2 * sizeof(uint32_t);
-    if (dtype == 0) {
-        auto kr = rows_range_kernel<float, 4>;
-        e = cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_r);
-        if (e != cudaSuccess) return e;
-        kr<<<grid_r, kRThreads, smem_r, st>>>(a);
-    } else {
-        auto kr = rows_range_kernel<__nv_bfloat16, 4>;
-        e = cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_r);
-        if (e != cudaSuccess) return e;
-        kr<<<grid_r, kRThreads, smem_r, st>>>(a);
+    // the cut of a row into slices that leaves the fewest threads and CTAs without work (196 unit columns: 7 slices of
+    // 28, 16 rows of threads each); slices of 64 unit columns at most, of 16 at least where there are several
+    const uint32_t top = dtype == 0 ? kRMaxThreads<float> : kRMaxThreads<__nv_bfloat16>, ctas = 2u * (uint32_t)sms;
+    double best = 0.0;
+    for (uint32_t slices = (a.ncol + 63) / 64; slices <= std::max<uint32_t>(1, a.ncol / 16); ++slices) {
+        const uint32_t P = (a.ncol + slices - 1) / slices, lanes = top / P, used = (a.ncol + P - 1) / P;
+        const double eff = (double)a.ncol / (double)(used * P) * (double)(P * lanes) / top * (double)(ctas / used * used) / ctas;
+        if (eff > best + 0.02) {
+            best = eff;
+            a.P = P;
+            a.slices = used;
+            a.lanes = lanes;
+        }
     }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    const uint64_t blocks = (a.rows + a.lanes - 1) / a.lanes;      // no more CTAs than there are blocks of rows
+    a.team = (uint32_t)std::min<uint64_t>(blocks, ctas / a.slices);
+    const int grid = (int)(a.team * a.slices), threads = (int)((a.P * a.lanes + 31) / 32 * 32);
+    const size_t table = (size_t)a.P * V * sizeof(GroupParam), block = (size_t)a.P * a.lanes * 16;
+    // all of a CTA's blocks or none: loads in flight need L1, which is what shared memory leaves of 256 KB (keeping a
+    // part: fp32 [128,112,112,64] with gradient 363 us, none 343; bf16 [128,28,28,192] 38.5 MB, 85 % kept, 33.4 / 31.3)
+    const uint64_t per_cta = (blocks + a.team - 1) / a.team;
+    a.hold = per_cta <= (kRSmemBytes - table) / block ? (uint32_t)per_cta : 0u;
+    const size_t smem = table + a.hold * block;
+    // of a tensor that is read twice, the last 64 MB have a chance to still be in the L2: the rest makes way for them
+    // ([128,112,112,64] fp32 forward 217 -> 208 us)
+    const double tail = 64e6 / ((double)a.rows * a.ncol * 16);
+    a.lost = tail < 1.0 ? (uint32_t)((1.0 - tail) * (double)per_cta) : 0u;
+    a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kRSpinLimit;
+    a.expected = a.team + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
     const bool extras = io.codes != nullptr || io.mask != nullptr;
     if (dtype == 0) {
-        if (mode == MODE_FWD) return r_launch_quant<float, MODE_FWD>(a, extras, grid_q, st);
-        return r_launch_quant<float, MODE_BOTH>(a, extras, grid_q, st);
+        if (mode == MODE_FWD) return r_launch<float, MODE_FWD>(a, extras, grid, threads, smem, st);
+        return r_launch<float, MODE_BOTH>(a, extras, grid, threads, smem, st);
     }
-    if (mode == MODE_FWD) return r_launch_quant<__nv_bfloat16, MODE_FWD>(a, extras, grid_q, st);
-    return r_launch_quant<__nv_bfloat16, MODE_BOTH>(a, extras, grid_q, st);
+    if (mode == MODE_FWD) return r_launch<__nv_bfloat16, MODE_FWD>(a, extras, grid, threads, smem, st);
+    return r_launch<__nv_bfloat16, MODE_BOTH>(a, extras, grid, threads, smem, st);
 }
 
 }  // namespace granq

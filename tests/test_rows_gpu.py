@@ -86,3 +86,33 @@ def test_channels_last_at_full_size(b, index, dtype):
     if dtype == "bf16":
         x, gy = wl.to_bf16_bits(x), wl.to_bf16_bits(gy)
     run(b, x, gy, spec.bits[0], 3)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("shape", [(2, 33, 17, 4096), (3, 61, 7, 2048), (1, 41, 31, 784), (2, 149, 1, 4096), (2, 97, 103, 1000)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_rows_kept_in_shared_memory_and_not(b, shape, dtype):
+    """Several slices of a row, the last of them narrower, blocks of rows that not every CTA of a team gets, and a
+    tensor beyond what shared memory keeps (read twice); the workspace is zero again afterwards."""
+    x, gy = nhwc_case(shape, seed=sum(shape), dtype=dtype)
+    run(b, x, gy, 5, 3)
+    run(b, x, None, 8, 3)
+    xd = to_dev(x)
+    ws = b.make_workspace(xd, 3, zeroed=True)
+    for _ in range(2):
+        got = b.granq_fakequant_fused(xd, 3, gy=to_dev(gy), channel_axis=3, out=b.FakeQuantOut(workspace=ws), flags=b.FLAG_WORKSPACE_ZEROED)
+        assert b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
+        assert_parity(got, orc.fused(x, 3, gy=gy, channel_axis=3), shape, 3, orc.GROUP_CHANNEL, backward=True)
+
+
+def test_rows_hand_over_that_never_completes_is_reported(b):
+    x, gy = nhwc_case((2, 5, 7, 64), seed=1, dtype="f32")
+    try:
+        b.tune(b.KNOB_TEST_EXTRA_ARRIVALS, 1)
+        b.tune(b.KNOB_SPIN_LIMIT, 500)
+        got = b.granq_fakequant_fused(to_dev(x), 4, gy=to_dev(gy), channel_axis=3)
+        assert b.workspace_status(got.workspace) == b.ERR_TIMEOUT
+    finally:
+        b.tune(b.KNOB_TEST_EXTRA_ARRIVALS, 0)
+        b.tune(b.KNOB_SPIN_LIMIT, 0)
+    run(b, x, gy, 4, 3)
