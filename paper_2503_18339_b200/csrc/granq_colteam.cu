@@ -47,6 +47,7 @@ struct TArgs {
     uint32_t* pmask;       // the STE mask at one bit per element, or null
     uint32_t* pcodes;      // the codes as a bit string of code_bits each, or null (y is then not written)
     int code_bits;
+    uint32_t code_words;   // planes are whole runs of 32 codes: fp32 packs write them as words
     double* dist;          // four running sums of Table 2's statistics, or null
     uint32_t* status;
     uint32_t* kmin;
@@ -85,7 +86,8 @@ __device__ __forceinline__ void t_cp_async_16(void* dst_smem, const void* src) {
 __device__ __forceinline__ void t_cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // U = units a thread handles together in the quantize walk
-template <typename T, int MODE, int EXTRAS, int U>
+// BITS = bits of a code (EXTRAS = 3 only: shifts and lanes of the code string are then constants)
+template <typename T, int MODE, int EXTRAS, int U, int BITS>
 __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     constexpr int V = Pack<T>::V;
     constexpr bool kBwd = (MODE & MODE_BWD) != 0;
@@ -203,9 +205,16 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
         auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint64_t at) {
             Pack<T> py, pgx;
             uint32_t cb[V / 4], mb[V / 4];
-            quantize_pack<T, kBwd, false, EXTRAS, true>(px, pg, g, g, V, qmax, py, pgx, cb, mb, EXTRAS == 3 ? a.code_bits : 8);
+            quantize_pack<T, kBwd, false, EXTRAS, true>(px, pg, g, g, V, qmax, py, pgx, cb, mb, BITS);
             if constexpr (EXTRAS == 3) {
-                store_code_bytes<V>(a.pcodes, at * V, code_string_of<V>(cb, a.code_bits), a.code_bits, lane);
+                const uint64_t str = code_string_of<V>(cb, BITS);
+                if constexpr (V == 4) {
+                    if (a.code_words) {
+                        store_code_words<BITS>(a.pcodes, at * V, (uint32_t)str, lane);
+                        return;
+                    }
+                }
+                store_code_bytes<V>(a.pcodes, at * V, str, BITS, lane);
                 return;
             }
             st_hint_16(yg + at, py.raw, drop);
@@ -271,9 +280,9 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     }
 }
 
-template <typename T, int MODE, int EXTRAS>
+template <typename T, int MODE, int EXTRAS, int BITS = 8>
 cudaError_t t_launch(const TArgs& args, uint32_t smem, cudaStream_t st) {
-    auto kern = colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2)>;
+    auto kern = colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2), BITS>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void* params[] = {(void*)&args};
@@ -285,7 +294,17 @@ cudaError_t t_launch_mode(const TArgs& a, int mode, int extras, uint32_t smem, c
     if (mode == MODE_BOTH) return t_launch<T, MODE_BOTH, 0>(a, smem, st);
     switch (extras) {
         case 2: return t_launch<T, MODE_FWD, 2>(a, smem, st);
-        case 3: return t_launch<T, MODE_FWD, 3>(a, smem, st);
+        case 3:
+            switch (a.code_bits) {
+                case 1: return t_launch<T, MODE_FWD, 3, 1>(a, smem, st);
+                case 2: return t_launch<T, MODE_FWD, 3, 2>(a, smem, st);
+                case 3: return t_launch<T, MODE_FWD, 3, 3>(a, smem, st);
+                case 4: return t_launch<T, MODE_FWD, 3, 4>(a, smem, st);
+                case 5: return t_launch<T, MODE_FWD, 3, 5>(a, smem, st);
+                case 6: return t_launch<T, MODE_FWD, 3, 6>(a, smem, st);
+                case 7: return t_launch<T, MODE_FWD, 3, 7>(a, smem, st);
+                default: return t_launch<T, MODE_FWD, 3, 8>(a, smem, st);
+            }
         case 4: return t_launch<T, MODE_FWD, 4>(a, smem, st);
         default: return t_launch<T, MODE_FWD, 0>(a, smem, st);
     }
@@ -342,6 +361,7 @@ cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, in
     a.pmask = io.pmask;
     a.pcodes = io.pcodes;
     a.code_bits = io.code_bits;
+    a.code_words = g.inner % 32 == 0 ? 1u : 0u;
     a.dist = io.dist;
     a.status = ws.status;
     a.kmin = ws.kmin;

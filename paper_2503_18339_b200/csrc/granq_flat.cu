@@ -606,7 +606,81 @@ __global__ void __launch_bounds__(kThreads) distortion_kernel(const T* __restric
 }
 
 // ---- Eq. 6 from the packed integer codes: y = s * (code - z) --------------------------------------
-// V = elements per thread and step (a 16-byte pack of y when E and the pointer allow it, else 1).
+// Eight codes (BITS bytes of the bit string) per thread and step, two such strings in flight: two or three words of
+// codes, one pair of divisions for the channel, shifts that are constants, and 32 bytes of fp32 (16 of bf16) stored at
+// once.  Planes of at least 8 elements; where they are no multiple of 8 (RAGGED) a string may reach into the next
+// plane.  Bound by the stores: [128,144,56,56], 231 MB written from 36 MB of 5-bit codes, 92 -> 45 us
+// (5.9 TB/s; a thread per 16 bytes with two 32-bit divisions took 171 instructions for 4 elements).
+template <typename T, int BITS, bool RAGGED>
+__global__ void __launch_bounds__(kThreads) dequant_strings_kernel(const uint32_t* __restrict__ pcodes, T* __restrict__ y,
+                                                                   uint32_t nstrings, uint32_t last_word, uint32_t inner,
+                                                                   FastDiv div_inner, FastDiv div_C,
+                                                                   const float* __restrict__ s, const float* __restrict__ z) {
+    constexpr uint32_t kField = (1u << BITS) - 1u;
+    constexpr int kFly = 2;
+    for (uint32_t t0 = blockIdx.x * (kThreads * kFly) + threadIdx.x; t0 < nstrings; t0 += gridDim.x * (kThreads * kFly)) {
+        uint32_t w[kFly][3];
+#pragma unroll
+        for (int f = 0; f < kFly; ++f) {
+            const uint32_t t = t0 + f * kThreads;
+            if (t >= nstrings) break;
+            const uint32_t w0 = (uint32_t)(((uint64_t)t * BITS) >> 2);              // 8 * BITS bits per string
+            w[f][0] = __ldg(pcodes + w0);
+            if constexpr (BITS > 1) w[f][1] = __ldg(pcodes + min(w0 + 1, last_word));
+            if constexpr (BITS == 6 || BITS == 7) w[f][2] = __ldg(pcodes + min(w0 + 2, last_word));
+        }
+#pragma unroll
+        for (int f = 0; f < kFly; ++f) {
+            const uint32_t t = t0 + f * kThreads;
+            if (t >= nstrings) break;
+            const uint32_t sh = (t * (8u * BITS)) & 31u;                            // 0, 8, 16 or 24
+            uint32_t lo, hi = 0;
+            if constexpr (BITS == 1) lo = w[f][0] >> sh;
+            else lo = __funnelshift_r(w[f][0], w[f][1], sh);
+            if constexpr (BITS == 8) hi = w[f][1];
+            else if constexpr (BITS == 6 || BITS == 7) hi = __funnelshift_r(w[f][1], w[f][2], sh);
+            else if constexpr (BITS == 5) hi = w[f][1] >> sh;
+            uint32_t plane, rem, q, g1;
+            div_inner.divmod(t * 8u, plane, rem);
+            div_C.divmod(plane, q, g1);
+            const float s1 = __ldg(s + g1), z1 = __ldg(z + g1);
+            float s2 = s1, z2 = z1;
+            const uint32_t n1 = inner - rem;                                        // elements left in this plane
+            if constexpr (RAGGED) {
+                if (n1 < 8) {
+                    const uint32_t g2 = g1 + 1 == div_C.d ? 0u : g1 + 1;
+                    s2 = __ldg(s + g2);
+                    z2 = __ldg(z + g2);
+                }
+            }
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                constexpr uint32_t kTwo23 = 0x4B000000u;                            // 2^23: the code becomes the low mantissa
+                const int pos = i * BITS;
+                uint32_t c;
+                if (pos + BITS <= 32) c = lo >> pos;
+                else if (pos >= 32) c = hi >> (pos - 32);
+                else c = __funnelshift_r(lo, hi, pos);
+                const float code = __fsub_rn(__uint_as_float((c & kField) | kTwo23), 8388608.0f);
+                const bool first = !RAGGED || (uint32_t)i < n1;
+                v[i] = __fmul_rn(first ? s1 : s2, __fsub_rn(code, first ? z1 : z2));
+            }
+            T* out = y + (size_t)t * 8;
+            if constexpr (Pack<T>::V == 8) {
+                Pack<T> p;
+                p.set_all(v);
+                st_stream_16(out, p.raw);
+            } else {
+                asm volatile("st.global.L1::no_allocate.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(out), "f"(v[0]), "f"(v[1]),
+                             "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                             : "memory");
+            }
+        }
+    }
+}
+
+// Any geometry: V = elements per thread and step (a 16-byte pack of y when E and the pointer allow it, else 1).
 template <typename T, int V>
 __global__ void __launch_bounds__(kThreads) dequant_packed_kernel(const uint32_t* __restrict__ pcodes,
                                                                   T* __restrict__ y, int64_t E, int64_t inner,
@@ -812,6 +886,35 @@ cudaError_t naive_t(const QuantIO& io, const Geom& g, int bits, uint32_t* kmin, 
     return cudaSuccess;
 }
 
+template <typename T, int BITS>
+cudaError_t dequant_strings_bits(const uint32_t* pcodes, T* y, const Geom& g, const float* s, const float* z, int sms,
+                                 cudaStream_t st) {
+    const uint32_t n = (uint32_t)(g.E / 8), last = (uint32_t)((g.E * BITS - 1) >> 5);
+    const uint32_t per_cta = kThreads * 2, want = (n + per_cta - 1) / per_cta, cap = (uint32_t)sms * 8;
+    const uint32_t grid = want < cap ? want : cap;
+    const FastDiv di = make_fastdiv((uint32_t)g.inner), dc = make_fastdiv((uint32_t)g.C);
+    if (g.inner % 8 == 0)
+        dequant_strings_kernel<T, BITS, false><<<grid, kThreads, 0, st>>>(pcodes, y, n, last, (uint32_t)g.inner, di, dc, s, z);
+    else
+        dequant_strings_kernel<T, BITS, true><<<grid, kThreads, 0, st>>>(pcodes, y, n, last, (uint32_t)g.inner, di, dc, s, z);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t dequant_strings(const uint32_t* pcodes, T* y, const Geom& g, int bits, const float* s, const float* z, int sms,
+                            cudaStream_t st) {
+    switch (bits) {
+        case 1: return dequant_strings_bits<T, 1>(pcodes, y, g, s, z, sms, st);
+        case 2: return dequant_strings_bits<T, 2>(pcodes, y, g, s, z, sms, st);
+        case 3: return dequant_strings_bits<T, 3>(pcodes, y, g, s, z, sms, st);
+        case 4: return dequant_strings_bits<T, 4>(pcodes, y, g, s, z, sms, st);
+        case 5: return dequant_strings_bits<T, 5>(pcodes, y, g, s, z, sms, st);
+        case 6: return dequant_strings_bits<T, 6>(pcodes, y, g, s, z, sms, st);
+        case 7: return dequant_strings_bits<T, 7>(pcodes, y, g, s, z, sms, st);
+        default: return dequant_strings_bits<T, 8>(pcodes, y, g, s, z, sms, st);
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_range_flat(const void* x, int dtype, const Geom& g, uint32_t* kmin, uint32_t* kmax,
@@ -910,6 +1013,11 @@ cudaError_t launch_dequant_packed(const uint32_t* pcodes, void* y, int dtype, co
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // strings of 8 codes: planes of at least 8 elements, a whole number of strings, 32-byte (fp32) stores
+    if (g.E % 8 == 0 && g.E < (1ll << 31) && g.inner >= 8 && g.inner < (1ll << 30) && g.C < (1ll << 30) &&
+        ((uintptr_t)y & (dtype == 0 ? 31 : 15)) == 0)
+        return dtype == 0 ? dequant_strings<float>(pcodes, (float*)y, g, bits, s, z, sms, st)
+                          : dequant_strings<__nv_bfloat16>(pcodes, (__nv_bfloat16*)y, g, bits, s, z, sms, st);
     const int VF = dtype == 0 ? 4 : 8;
     const bool vec = aligned16(y) && (g.E % VF == 0);
     const int64_t units = vec ? g.E / VF : g.E;

@@ -116,3 +116,28 @@ def test_quantize_packed_fused_full_size(b, spec):
         assert b.workspace_status(got.workspace) == b.OK
         assert np.array_equal(got.packed_codes.cpu().numpy().view(np.uint8)[:want.size], want)
         assert same_bits(to_np(got.s), ref.s) and same_bits(to_np(got.z), ref.z)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("bits", [1, 2, 3, 4, 5, 6, 7, 8])
+def test_codes_written_as_words_and_expanded_eight_at_a_time(b, bits, dtype):
+    """Planes of whole runs of 32 codes (the resident column walk writes words), planes of whole and of broken runs of
+    8, a last word that is not full, strings of 8 that reach into the next plane and from the last channel into the
+    first, planes shorter than a string."""
+    for shape in ((8, 12, 8, 8), (9, 24, 16, 16), (8, 24, 12, 12), (8, 5, 7, 7), (8, 3, 3, 3), (2, 4, 3, 5), (16, 2, 2, 2)):
+        x, _ = make_case(shape, seed=bits + sum(shape), dtype=dtype)
+        ref = orc.fused(x, bits)
+        packed = orc.pack_codes(ref.codes, bits)
+        xd = to_dev(x)
+        for flags in (0, b.FLAG_FORCE_COLWALK):
+            try:
+                got = b.granq_quantize_packed_fused(xd, bits, flags=flags)
+            except b.GranqError as err:
+                assert flags and err.status == b.ERR_UNSUPPORTED
+                continue
+            words = got.packed_codes.cpu().numpy().view(np.uint8)
+            flat = np.ascontiguousarray(packed).view(np.uint8).reshape(-1)
+            assert np.array_equal(words[:flat.size], flat)
+        y = b.granq_dequantize_packed(got.packed_codes, shape, xd.dtype, bits,
+                                      to_dev(ref.s), to_dev(ref.z))
+        assert same_bits(to_np(y), ref.y), (shape, bits)
