@@ -368,8 +368,8 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
  *   flags              0, or GRANQ_FLAG_FORCE_TWO_PASS for the kernel with one pixel tile per CTA instead of the
  *                      persistent one (which is taken whenever the weight halves of all channels fit in shared
  *                      memory, and holds all of an SM's tensor memory while it runs)
- * Two launches on `cuda_stream` (weights, then expansion + contraction + epilogue) after a 4-byte clear of the
- * status word.
+ * Two launches on `cuda_stream` (weights, then expansion + contraction + epilogue); the first
+ * clears the status word.
  * Result: within (2^-17 + C * 2^-22) * sum_c |w s_c| (code + |z_c|) + 2^-21 * (|bias| + |y|) of the exact sum
  * (the split of the scaled weights, fp32 accumulation of the C products of each half in any order, the sum of
  * the two halves, one rounding each of bias and y).

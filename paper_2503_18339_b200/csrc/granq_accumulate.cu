@@ -803,8 +803,9 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
 // bias[o] = sum_c (hi + lo)[o][c] * z_c in fp64 (the matrix that is really multiplied), rounded once to fp32.
 __global__ void accumulate_weights_kernel(const float* __restrict__ w, const float* __restrict__ s,
                                           const float* __restrict__ z, int C, int Cpad, __nv_bfloat16* hi,
-                                          __nv_bfloat16* lo, float* bias) {
+                                          __nv_bfloat16* lo, float* bias, uint32_t* status) {
     const int o = blockIdx.x;
+    if (o == 0 && threadIdx.x == 0) *status = 0;      // the call's status word; the contraction comes after this kernel
     double acc = 0.0;
     for (int c = threadIdx.x; c < Cpad; c += blockDim.x) {
         float h = 0.0f, l = 0.0f;
@@ -950,10 +951,8 @@ extern "C" int granq_accumulate_codes(const uint32_t* packed_codes, const int64_
         !a_make_map(encode, &ml, lo, (uint64_t)out_channels, (uint64_t)L.Cpad, (uint32_t)BN))
         return GRANQ_ERR_CUDA;
 
-    cudaError_t e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);       // the status word
-    if (e != cudaSuccess) return GRANQ_ERR_CUDA;
     accumulate_weights_kernel<<<(unsigned)out_channels, 128, 0, st>>>(weights, scale, zp, (int)L.C, (int)L.Cpad, hi, lo,
-                                                                    bias);
+                                                                    bias, (uint32_t*)workspace);
     if (cudaGetLastError() != cudaSuccess) return GRANQ_ERR_CUDA;
     AArgs args{};
     args.y = y;
@@ -970,6 +969,7 @@ extern "C" int granq_accumulate_codes(const uint32_t* packed_codes, const int64_
     args.spin_limit = kASpin;
     args.stages = std::min(args.kblocks, 2);
     const bool persistent = !one_tile_per_cta && resident(BN);
+    cudaError_t e = cudaSuccess;
     if (persistent) {
         if (channel_axis == 3)
             e = BN == 64 ? p_launch<64, true>(mh, ml, args, st) : p_launch<128, true>(mh, ml, args, st);

@@ -240,7 +240,7 @@ int granq_fakequant_fused(const void* x, const void* gy_opt, int dtype, const in
 
     Workspace ws = carve_workspace(workspace, G);
     // The column-walk and channels-last kernels leave a zeroed workspace zeroed and the cluster-local kernel writes
-    // nothing but the status word (and that only when a wait ran out); with the caller's word that
+    // nothing but the status word (0, or that a wait on its bulk copies ran out); with the caller's word that
     // the workspace is zero on entry nothing has to be cleared.  The other plans clear before and, to
     // keep that word true for the next call, after.
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
@@ -249,7 +249,7 @@ int granq_fakequant_fused(const void* x, const void* gy_opt, int dtype, const in
     if (plan == PLAN_CLUSTER) tp = prefer_team(dtype, g, io, gy_opt != nullptr, flags);
     cudaError_t e = cudaSuccess;
     if (plan == PLAN_CLUSTER && !tp.ok) {
-        if (!zeroed) e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);      // the status word
+        if (!zeroed && !kp.clears_status) e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);      // the status word
     } else if (!(zeroed && keeps_zero)) {
         e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
     }
@@ -352,7 +352,9 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
     cudaError_t e = cudaSuccess;
     const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     if (kp.ok) {
-        if (!zeroed) e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
+        // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
+        if (!zeroed && (tp.ok || !kp.clears_status))
+            e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
         // the kernel writes the mask byte by byte: the padding bits of a last, partial word are cleared here
         if (e == cudaSuccess && g.E % 32 != 0) e = cudaMemsetAsync(packed_mask + g.E / 32, 0, sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
@@ -447,7 +449,9 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
     cudaError_t e = cudaMemsetAsync(sums_out, 0, 4 * sizeof(double), st);
     const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     if (e == cudaSuccess && kp.ok) {
-        if (!zeroed) e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
+        // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
+        if (!zeroed && (tp.ok || !kp.clears_status))
+            e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
         if (tp.ok)
             return cuda_status(launch_colteam(tp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt,
@@ -525,7 +529,9 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
     cudaError_t e = cudaSuccess;
     const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     if (kp.ok) {
-        if (!zeroed) e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
+        // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
+        if (!zeroed && (tp.ok || !kp.clears_status))
+            e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
         if (tp.ok)
             return cuda_status(launch_colteam(tp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out,

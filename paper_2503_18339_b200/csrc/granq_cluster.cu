@@ -261,6 +261,10 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
     // waits for that kernel's memory; dependents of this grid may start their own preamble from here on.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // the call's status: only bulk copies can run out of a wait, and their caller clears the word ahead of the launch
+    if constexpr (!BULK) {
+        if (blockIdx.x == 0 && tid == 0) *a.status = 0;
+    }
 
     // ---- stage x (and gy) ----
     if constexpr (BULK) {
@@ -686,6 +690,7 @@ ClusterPlan plan_cluster(int dtype, const Geom& g, const QuantIO& io, bool backw
     }
     p.prefetch_gy = tune.cl_prefetch != 2;
     p.early_launch = tune.cl_pdl != 2;
+    p.clears_status = p.load != K_LOAD_BULK_X && p.load != K_LOAD_BULK_XG;
     p.ok = true;
     return p;
 }

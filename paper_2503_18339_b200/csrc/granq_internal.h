@@ -203,6 +203,7 @@ struct ClusterPlan {
     int load;                // 0 = plain loads, 1 = x staged by bulk copies, 2 = x and gy staged by bulk copies
     bool prefetch_gy;
     bool early_launch;       // programmatic dependent launch: set the grid up while the kernel ahead drains
+    bool clears_status;      // the kernel itself writes status 0 (no wait in it can run out)
 };
 ClusterPlan plan_cluster(int dtype, const Geom& g, const QuantIO& io, bool backward, const StagedTuning& tune);
 cudaError_t launch_cluster(const ClusterPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
