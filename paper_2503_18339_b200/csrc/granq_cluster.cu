@@ -61,6 +61,7 @@ struct KArgs {
     uint32_t tile_bytes;   // shared-memory bytes of the staged tile (keys and parameters follow)
     uint32_t spin_limit;
     uint32_t prefetch_gy;  // ask the L2 for gy while x is on its way
+    uint32_t late_wait;    // wait for the kernels ahead only at the end (see below)
     uint32_t test_stall;   // test hook: after a tile has landed, wait (bounded) for a phase that never completes
     FastDiv div_inner;     // elements per plane
 };
@@ -259,7 +260,11 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
     // Everything above touched only this CTA's own state.  When the launch allows this grid to start before
     // the kernel ahead of it in the stream has finished (programmatic dependent launch), this is where it
     // waits for that kernel's memory; dependents of this grid may start their own preamble from here on.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // In a list of tensors that share no memory the wait moves to the end of the kernel: it then runs beside the kernels
+    // ahead of it and still does not complete before they do, so whatever comes after the list needs to know its last
+    // kernel only.  (It starts when every CTA of the kernel ahead has come past this line, so after the one wait of the
+    // list's first kernel.)
+    if (!a.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the call's status: only bulk copies can run out of a wait, and their caller clears the word ahead of the launch
     if constexpr (!BULK) {
@@ -529,6 +534,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
         }
         __syncthreads();
     }
+    if (a.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 bool k_aligned16(const void* p) { return p == nullptr || ((uintptr_t)p & 15) == 0; }
@@ -725,6 +731,7 @@ cudaError_t launch_cluster(const ClusterPlan& plan, const QuantIO& io, int mode,
     a.tile_bytes = plan.tile_bytes;
     a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kKSpinLimit;
     a.prefetch_gy = plan.prefetch_gy ? 1u : 0u;
+    a.late_wait = plan.late_wait && plan.early_launch ? 1u : 0u;
     a.test_stall = tune.extra_arrivals > 0 ? 1u : 0u;
     a.div_inner = make_fastdiv(a.inner);
     const uint32_t nruns = (a.C + plan.k - 1) / plan.k;

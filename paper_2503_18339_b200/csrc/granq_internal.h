@@ -204,6 +204,8 @@ struct ClusterPlan {
     bool prefetch_gy;
     bool early_launch;       // programmatic dependent launch: set the grid up while the kernel ahead drains
     bool clears_status;      // the kernel itself writes status 0 (no wait in it can run out)
+    bool late_wait;          // it shares no memory with the kernels ahead of it that may still run: it need not wait for
+                             // them before it starts, only before it ends
 };
 ClusterPlan plan_cluster(int dtype, const Geom& g, const QuantIO& io, bool backward, const StagedTuning& tune);
 cudaError_t launch_cluster(const ClusterPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,

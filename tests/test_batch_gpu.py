@@ -64,3 +64,32 @@ def test_batch_stops_at_the_bad_descriptor(b):
     torch.cuda.synchronize()
     assert same_bits(to_np(batch.outs[2].y), before)
     assert same_bits(to_np(batch.outs[0].y), orc.fused(to_np(xs[0]), 4).y)
+
+
+def test_batch_tensors_that_run_beside_one_another_and_tensors_that_depend(b):
+    """More tensors than run together, in which some read what an earlier one of the list wrote (next to it and further
+    back), one writes what an earlier one read, and two share a workspace: as if made one after the other."""
+    shape = (16, 16, 14, 14)
+    n = 24
+    cases = [make_case(shape, seed=50 + i) for i in range(n)]
+    src = [x for x, _ in cases]
+    xs = [to_dev(x) for x in src]
+    gys = [to_dev(gy) for _, gy in cases]
+    outs = [b.FakeQuantOut(y=torch.empty_like(x), gx=torch.empty_like(x), workspace=b.make_workspace(x, zeroed=True)) for x in xs]
+    reads = {3: 2, 9: 5, 17: 16, 18: 17}                   # tensor i quantizes what tensor reads[i] wrote
+    for i, k in reads.items():
+        xs[i] = outs[k].y
+    outs[13].y = xs[11]                                    # tensor 13 overwrites what tensor 11 has read
+    outs[21].workspace = outs[20].workspace
+    batch = b.FusedBatch(list(zip(xs, [4] * n, gys)), outs=outs, zeroed=True)
+    for _ in range(3):
+        xs[11].copy_(to_dev(src[11]))
+        batch.run()
+        torch.cuda.synchronize()
+        ys = []
+        for i in range(n):
+            ref = orc.fused(ys[reads[i]] if i in reads else src[i], 4, gy=cases[i][1])
+            ys.append(ref.y)
+            assert b.workspace_status(outs[i].workspace) == b.OK
+            assert same_bits(to_np(outs[i].y), ref.y) and same_bits(to_np(outs[i].gx), ref.gx), f"tensor {i}"
+            assert same_bits(to_np(outs[i].lo), ref.lo) and same_bits(to_np(outs[i].hi), ref.hi)
