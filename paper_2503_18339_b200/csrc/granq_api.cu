@@ -169,8 +169,8 @@ int granq_range(const void* x, int dtype, const int64_t dims[4], int channel_axi
     cudaStream_t st = (cudaStream_t)cuda_stream;
     Workspace ws = carve_workspace(workspace, G);
     cudaError_t e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
-    if (e == cudaSuccess) e = launch_range_flat(x, dtype, g, ws.kmin, ws.kmax, st);
-    if (e == cudaSuccess) e = launch_finalize_range(ws.kmin, ws.kmax, G, min_out, max_out, 0, nullptr, nullptr, st);
+    if (e == cudaSuccess)
+        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, 0, nullptr, nullptr, st);
     return cuda_status(e);
 }
 
@@ -274,9 +274,7 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
         if (e == cudaSuccess && (scale_opt || zp_opt))
             e = launch_params(min_out, max_out, G, bits, scale_opt, zp_opt, st);
     } else {
-        e = launch_range_flat(x, dtype, g, ws.kmin, ws.kmax, st);
-        if (e == cudaSuccess)
-            e = launch_finalize_range(ws.kmin, ws.kmax, G, min_out, max_out, bits, scale_opt, zp_opt, st);
+        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, st);
         if (e == cudaSuccess) e = launch_quant_flat(io, mode, dtype, g, bits, min_out, max_out, st);
     }
     if (e == cudaSuccess && zeroed && !keeps_zero)
@@ -380,9 +378,7 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {
-        e = launch_range_flat(x, dtype, g, ws.kmin, ws.kmax, st);
-        if (e == cudaSuccess)
-            e = launch_finalize_range(ws.kmin, ws.kmax, G, min_out, max_out, bits, scale_opt, zp_opt, st);
+        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, st);
         if (e == cudaSuccess) e = launch_quant_flat(io, MODE_FWD, dtype, g, bits, min_out, max_out, st);
         if (e == cudaSuccess && zeroed)
             e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);
@@ -521,9 +517,7 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {
-        e = launch_range_flat(x, dtype, g, ws.kmin, ws.kmax, st);
-        if (e == cudaSuccess)
-            e = launch_finalize_range(ws.kmin, ws.kmax, G, min_out, max_out, bits, scale_opt, zp_opt, st);
+        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, st);
         if (e == cudaSuccess) e = launch_quant_flat(io, MODE_FWD, dtype, g, bits, min_out, max_out, st);
         if (e == cudaSuccess && zeroed)
             e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);
@@ -601,9 +595,7 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, g_tune, st);
     } else {
-        e = launch_range_flat(x, dtype, g, ws.kmin, ws.kmax, st);
-        if (e == cudaSuccess)
-            e = launch_finalize_range(ws.kmin, ws.kmax, G, min_out, max_out, bits, scale_out, zp_out, st);
+        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_out, zp_out, st);
         if (e == cudaSuccess) e = launch_quant_flat(io, MODE_FWD, dtype, g, bits, min_out, max_out, st);
         if (e == cudaSuccess && zeroed)
             e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);
@@ -710,7 +702,7 @@ int granq_fused_plan(int dtype, const int64_t dims[4], int channel_axis, int gro
     if (launches_out) {
         if (plan == PLAN_STAGED || plan == PLAN_L2WAVE || plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS) *launches_out = 1;
         else if (plan == PLAN_NAIVE) *launches_out = (int)(3 * g.C);
-        else if (plan == PLAN_TWO_PASS) *launches_out = 3;
+        else if (plan == PLAN_TWO_PASS) *launches_out = g.C <= 4096 ? 2 : 3;
     }
     return plan;
 }

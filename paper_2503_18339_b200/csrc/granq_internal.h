@@ -88,12 +88,10 @@ struct QuantIO {
 };
 
 // ---- generic ("flat") kernels: any geometry, any alignment --------------------------------
-// keys must be zero on entry; accumulates ordered min/max keys per group
-cudaError_t launch_range_flat(const void* x, int dtype, const Geom& g, uint32_t* kmin, uint32_t* kmax,
-                              cudaStream_t st);
-// keys -> lo / hi (and s / z when bits > 0 and the pointers are given)
-cudaError_t launch_finalize_range(const uint32_t* kmin, const uint32_t* kmax, int64_t G, float* lo, float* hi,
-                                  int bits, float* s_opt, float* z_opt, cudaStream_t st);
+// Range of every group (Eq. 4) into lo / hi, and s / z when bits > 0 and the pointers are given (Eq. 5).  The keys and,
+// where one is given, the counter must be zero on entry; with a counter the range launch finishes by itself.
+cudaError_t launch_range(const void* x, int dtype, const Geom& g, uint32_t* kmin, uint32_t* kmax, uint32_t* counter,
+                         float* lo, float* hi, int bits, float* s_opt, float* z_opt, cudaStream_t st);
 // lo / hi -> s / z
 cudaError_t launch_params(const float* lo, const float* hi, int64_t G, int bits, float* s_opt, float* z_opt,
                           cudaStream_t st);
