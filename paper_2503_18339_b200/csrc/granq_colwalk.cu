@@ -566,6 +566,10 @@ ColPlan plan_colwalk(int dtype, const Geom& g, const QuantIO& io, const StagedTu
     return p;
 }
 
+static uint32_t team_rounds(int64_t channels, const TeamPlan& tp) {
+    return (uint32_t)((channels + tp.teams - 1) / tp.teams);
+}
+
 cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
                            const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,
                            const StagedTuning& tune, cudaStream_t st) {
@@ -578,7 +582,10 @@ cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int
     // the resident form, unless a knob of the waves is set
     if (tune.col_team != 2 && tune.l2_wave_kb <= 0 && tune.l2_lag <= 0 && tune.l2_ctas_per_sm <= 0) {
         const TeamPlan tp = plan_colteam(dtype, g, io, mode == MODE_BOTH, sms);
-        if (tp.ok) return launch_colteam(tp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, tune, st);
+        // a hand-over costs a team as much as 2000 units: where the rounds are several and shorter than that (small
+        // channels) the waves are faster (forward bf16 [12,2048,33,32], 7 rounds of 1584 units: 48 us, waves 43)
+        if (tp.ok && (tp.tile_units >= 2500 || team_rounds(g.C, tp) == 1))
+            return launch_colteam(tp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, tune, st);
     }
     CArgs a{};
     a.x = io.x;
