@@ -243,10 +243,11 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
 
     Workspace ws = carve_workspace(workspace, G);
     // The column-walk and channels-last kernels leave a zeroed workspace zeroed and the cluster-local kernel writes
-    // nothing but the status word (0, or that a wait on its bulk copies ran out); with the caller's word that
-    // the workspace is zero on entry nothing has to be cleared.  The other plans clear before and, to
+    // nothing but the status word (0 where the caller did not vouch for it, or that a wait on its bulk copies ran
+    // out); with the caller's word that the workspace is zero on entry nothing has to be cleared.  The other plans clear before and, to
     // keep that word true for the next call, after.
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
+    kp.zero_status = !zeroed && kp.clears_status;
     const bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS;
     TeamPlan tp{};
     if (plan == PLAN_CLUSTER) tp = prefer_team(dtype, g, io, gy_opt != nullptr, flags);
@@ -358,6 +359,7 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
     if ((flags & GRANQ_FLAG_FORCE_COLWALK) && !cp.ok) return GRANQ_ERR_UNSUPPORTED;
     Workspace ws = carve_workspace(workspace, G);
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
+    kp.zero_status = !zeroed && kp.clears_status;
     cudaError_t e = cudaSuccess;
     const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     if (kp.ok) {
@@ -499,6 +501,7 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
     if ((flags & GRANQ_FLAG_FORCE_COLWALK) && !cp.ok) return GRANQ_ERR_UNSUPPORTED;
     Workspace ws = carve_workspace(workspace, G);
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
+    kp.zero_status = !zeroed && kp.clears_status;
     cudaError_t e = cudaMemsetAsync(sums_out, 0, 4 * sizeof(double), st);
     const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     if (e == cudaSuccess && kp.ok) {
@@ -577,6 +580,7 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
     if ((flags & GRANQ_FLAG_FORCE_COLWALK) && !cp.ok) return GRANQ_ERR_UNSUPPORTED;
     Workspace ws = carve_workspace(workspace, G);
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
+    kp.zero_status = !zeroed && kp.clears_status;
     cudaError_t e = cudaSuccess;
     const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     if (kp.ok) {

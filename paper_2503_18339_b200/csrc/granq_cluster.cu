@@ -62,6 +62,7 @@ struct KArgs {
     uint32_t spin_limit;
     uint32_t prefetch_gy;  // ask the L2 for gy while x is on its way
     uint32_t late_wait;    // wait for the kernels ahead only at the end (see below)
+    uint32_t zero_status;  // write status 0 (no wait of this kernel can run out, and the caller has not vouched for the word)
     uint32_t test_stall;   // test hook: after a tile has landed, wait (bounded) for a phase that never completes
     FastDiv div_inner;     // elements per plane
 };
@@ -266,9 +267,10 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
     // list's first kernel.)
     if (!a.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // the call's status: only bulk copies can run out of a wait, and their caller clears the word ahead of the launch
+    // the call's status: only bulk copies can run out of a wait, and their caller clears the word ahead of the launch.
+    // A workspace handed over as zero is left alone: what an earlier call on it reported has to stay readable.
     if constexpr (!BULK) {
-        if (blockIdx.x == 0 && tid == 0) *a.status = 0;
+        if (a.zero_status && blockIdx.x == 0 && tid == 0) *a.status = 0;
     }
 
     // ---- stage x (and gy) ----
@@ -732,6 +734,7 @@ cudaError_t launch_cluster(const ClusterPlan& plan, const QuantIO& io, int mode,
     a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kKSpinLimit;
     a.prefetch_gy = plan.prefetch_gy ? 1u : 0u;
     a.late_wait = plan.late_wait && plan.early_launch ? 1u : 0u;
+    a.zero_status = plan.zero_status ? 1u : 0u;
     a.test_stall = tune.extra_arrivals > 0 ? 1u : 0u;
     a.div_inner = make_fastdiv(a.inner);
     const uint32_t nruns = (a.C + plan.k - 1) / plan.k;

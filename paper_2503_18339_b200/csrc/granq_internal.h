@@ -201,7 +201,8 @@ struct ClusterPlan {
     int load;                // 0 = plain loads, 1 = x staged by bulk copies, 2 = x and gy staged by bulk copies
     bool prefetch_gy;
     bool early_launch;       // programmatic dependent launch: set the grid up while the kernel ahead drains
-    bool clears_status;      // the kernel itself writes status 0 (no wait in it can run out)
+    bool clears_status;      // the kernel can write status 0 itself (no wait in it can run out)
+    bool zero_status;        // and is to do so: not where the caller vouched for a zero workspace (set by the caller)
     bool late_wait;          // it shares no memory with the kernels ahead of it that may still run: it need not wait for
                              // them before it starts, only before it ends
 };

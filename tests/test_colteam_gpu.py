@@ -89,3 +89,29 @@ def test_large_tensors_take_the_resident_form_by_default(b, dtype, shape):
     got = b.granq_fakequant_fused_stats(xd, 4, out=new())
     assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
     assert b.workspace_status(ws) == b.OK
+
+
+def test_a_reported_timeout_outlives_later_calls_on_the_same_zeroed_workspace(b, knobs):
+    """A call on a workspace handed over as zero whose hand-over never completes leaves keys and counters behind;
+    a cluster-local call on the same workspace clears none of them, so it must not clear the report either."""
+    shape = (8, 24, 12, 12)
+    x, gy = make_case(shape, seed=2)
+    xd, gyd = to_dev(x), to_dev(gy)
+    ws = b.make_workspace(xd, zeroed=True)
+    knobs(extra_arrivals=1, spin_limit=500)
+    b.granq_fakequant_fused(xd, 4, gy=gyd, out=b.FakeQuantOut(workspace=ws), flags=b.FLAG_FORCE_COLWALK | b.FLAG_WORKSPACE_ZEROED)
+    assert b.workspace_status(ws) == b.ERR_TIMEOUT
+    knobs(extra_arrivals=0, spin_limit=0)
+    zeroed = b.FLAG_FORCE_CLUSTER | b.FLAG_WORKSPACE_ZEROED
+    new = lambda: b.FakeQuantOut(workspace=ws)
+    for call in (lambda: b.granq_fakequant_fused(xd, 4, gy=gyd, out=new(), flags=zeroed),
+                 lambda: b.granq_fakequant_fused(xd, 4, out=new(), flags=zeroed),
+                 lambda: b.granq_fakequant_fused_fwd_packmask(xd, 4, out=new(), flags=b.FLAG_WORKSPACE_ZEROED),
+                 lambda: b.granq_quantize_packed_fused(xd, 4, out=new(), flags=b.FLAG_WORKSPACE_ZEROED),
+                 lambda: b.granq_fakequant_fused_stats(xd, 4, out=new(), flags=b.FLAG_WORKSPACE_ZEROED)):
+        got = call()
+        assert b.workspace_status(ws) == b.ERR_TIMEOUT
+        assert same_bits(to_np(got.lo), orc.fused(x, 4).lo)
+    got = b.granq_fakequant_fused(xd, 4, gy=gyd, out=new(), flags=b.FLAG_FORCE_CLUSTER)      # clears the word itself
+    assert b.workspace_status(ws) == b.OK
+    assert same_bits(to_np(got.y), orc.fused(x, 4, gy=gy).y)
