@@ -279,6 +279,13 @@ __device__ __forceinline__ float tie_threshold(float rcp, float z, float qmax) {
     return __fmaf_rn(-1.1920928955078125e-07f, __fadd_rn(fabsf(z), __fmaf_rn(1.5f, qmax, 4.0f)), 0.5f);
 }
 
+// the larger of two values, NaN if either is (fmaxf drops it)
+__device__ __forceinline__ float max_or_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
 // u = x / s + z as defined, rounded: 1.5 * 2^23 + clamp(round(u), -1, qmax + 1), given the quotient t = RN(x / s)
 __device__ __forceinline__ float exact_round_magic(float t, float z, float qmax) {
     const float u = __fadd_rn(t, z);
@@ -343,7 +350,8 @@ __device__ __forceinline__ void pack_extras(const float (&m)[V], uint32_t in, ui
 // the default of 8), taken from the low mantissa bits of code + 1.5 * 2^23 instead of a float-to-integer
 // conversion (packed-code output); EXTRAS = 4 returns neither (the caller adds up the distortion).  SELF: the range is that of the tensor itself and thr comes from
 // group_param_from_range(), so where it is positive nothing is clamped and the gradient passes whole; without SELF
-// it comes from tie_threshold() alone and x may lie anywhere.
+// it comes from tie_threshold() alone and x may lie anywhere.  A NaN element fails the tie test and takes the clamp:
+// code 0 and no gradient, as in the sequence as defined, whatever its neighbours are.
 // Instructions per element, bf16 or fp32 alike: two multiply-adds, one add, half a three-way maximum and one
 // product (SELF), where rounding by add and subtract, clamp, compare and select took eleven.  Measured against that
 // form: forward-only bf16 [256,512,28,28] at 8 bits 127.6 -> 119.6 us (issue slots bind where an element is two
@@ -368,9 +376,11 @@ __device__ __forceinline__ void quantize_pack(const Pack<T>& px, const Pack<T>& 
             const float rc = first ? g1.r : g2.r, mz = first ? mz1 : mz2;
             const float x = px.get(i);
             m[i] = __fmaf_rn(x, rc, mz);
-            worst = fmaxf(worst, fabsf(__fmaf_rn(x, rc, __fsub_rn(mz, m[i]))));
+            worst = max_or_nan(worst, fabsf(__fmaf_rn(x, rc, __fsub_rn(mz, m[i]))));
         }
-        if (!(worst < thr)) {                                   // rare: too close to a tie for the shortcut
+        bool clamp = !SELF || g1.thr < 0.0f || (SPLIT && g2.thr < 0.0f);
+        if (!(worst < thr)) {                                   // rare: too close to a tie for the shortcut, or NaN
+            clamp = clamp || worst != worst;                    // which the clamp turns into code 0 without a gradient
 #pragma unroll
             for (int i = 0; i < V; ++i) {
                 const bool first = !SPLIT || i < n1;
@@ -380,7 +390,7 @@ __device__ __forceinline__ void quantize_pack(const Pack<T>& px, const Pack<T>& 
                     m[i] = exact_round_magic(SELF ? div_by_scale(x, s, rc) : __fdiv_rn(x, s), z, qmax);
             }
         }
-        if (!SELF || g1.thr < 0.0f || (SPLIT && g2.thr < 0.0f)) {
+        if (clamp) {
             in = 0;
 #pragma unroll
             for (int i = 0; i < V; ++i) {
@@ -431,9 +441,11 @@ __device__ __forceinline__ void quantize_pack_each(const Pack<T>& px, const Pack
         for (int i = 0; i < V; ++i) {
             const float x = px.get(i);
             m[i] = __fmaf_rn(x, r[i], mz[i]);
-            worst = fmaxf(worst, fabsf(__fmaf_rn(x, r[i], __fsub_rn(mz[i], m[i]))));
+            worst = max_or_nan(worst, fabsf(__fmaf_rn(x, r[i], __fsub_rn(mz[i], m[i]))));
         }
-        if (!(worst < bound)) {                                   // rare: too close to a tie for the shortcut
+        bool clamp = thr < 0.0f;
+        if (!(worst < bound)) {                                   // rare: too close to a tie for the shortcut, or NaN
+            clamp = clamp || worst != worst;                      // which the clamp turns into code 0 without a gradient
 #pragma unroll
             for (int i = 0; i < V; ++i) {
                 const float x = px.get(i);
@@ -441,7 +453,7 @@ __device__ __forceinline__ void quantize_pack_each(const Pack<T>& px, const Pack
                     m[i] = exact_round_magic(div_by_scale(x, s[i], r[i]), __fsub_rn(mz[i], kRoundMagic), qmax);
             }
         }
-        if (thr < 0.0f) {
+        if (clamp) {
             in = 0;
 #pragma unroll
             for (int i = 0; i < V; ++i) {

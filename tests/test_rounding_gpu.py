@@ -4,8 +4,9 @@ for bit: elements on a tie and one unit in the last place beside it, groups whos
 the short division, constant groups - through every kernel that quantizes."""
 import numpy as np
 import pytest
+import torch
 
-from gpu_util import assert_parity, to_dev
+from gpu_util import assert_parity, same_bits, to_dev, to_np
 from oracle import granq_oracle as orc
 from paper_2503_18339_b200 import workloads as wl
 
@@ -106,3 +107,60 @@ def test_hard_groups_with_a_range_narrower_than_the_tensor(b, dtype, bits):
     assert_parity(fwd, ref, shape, 1, orc.GROUP_CHANNEL, backward=False, exact=True)
     bwd = b.granq_fakequant_bwd(to_dev(gy), to_dev(x), bits, lod, hid, want_mask=True)
     assert_parity(bwd, ref, shape, 1, orc.GROUP_CHANNEL, backward=True)
+
+
+@pytest.mark.parametrize("layout,shape,axis", LAYOUTS, ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("where", ["scattered", "clamped"])
+def test_a_nan_is_code_zero_without_a_gradient_and_spoils_no_neighbour(b, layout, shape, axis, dtype, where):
+    """NaN is outside the contract, but what it gives is the same from every kernel: it does not enter the range, its
+    code is 0, no gradient passes, and every other element is as without it.  Groups where nothing is clamped, and
+    (values on the ties of lo = -hi) groups where the top element is."""
+    bits = 4
+    n = int(np.prod(shape)) // 16
+    rng = np.random.default_rng(n)
+    rows = rng.standard_normal((16, n)).astype(np.float32)
+    if where == "clamped":
+        rows = np.clip(rows, -1.5, 1.5)
+        rows[:, 0], rows[:, 1] = -1.5, 1.5
+    others = tuple(d for i, d in enumerate(shape) if i != axis)
+    x = np.ascontiguousarray(np.moveaxis(rows.reshape((16,) + others), 0, axis))
+    gy = rng.standard_normal(shape).astype(np.float32)
+    nan = rng.random((16, n)) < 0.05
+    nan[:, :2] = False
+    nan[3:6, 5] = True
+    nan = np.ascontiguousarray(np.moveaxis(nan.reshape((16,) + others), 0, axis))
+    x[nan] = 0.0                                # inside every group's range: the oracle takes no NaN
+    bad = x.copy()
+    bad[nan] = np.nan
+    if dtype == "bf16":
+        x, gy = wl.to_bf16_bits(x), wl.to_bf16_bits(gy)
+    ref = orc.fused(x, bits, gy=gy, channel_axis=axis)
+    badd = torch.from_numpy(bad).cuda().to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    view = [1] * 4
+    view[axis] = 16
+    zero_code = torch.from_numpy((ref.s * (np.float32(0) - ref.z)).reshape(view)).expand(shape)
+    zero_code = to_np(zero_code.to(badd.dtype).contiguous())
+    ref.y[nan], ref.codes[nan], ref.mask[nan], ref.gx[nan] = zero_code[nan], 0, 0, 0
+    gyd = to_dev(gy)
+    for flags in (0, b.FLAG_FORCE_CLUSTER, b.FLAG_FORCE_COLWALK, b.FLAG_FORCE_L2WAVE, b.FLAG_FORCE_TWO_PASS):
+        if axis == 3 and flags:          # two passes read such a tensor one element at a time: a NaN is then the maximum
+            continue
+        try:
+            for extras in (False, True):
+                got = b.granq_fakequant_fused(badd, bits, gy=gyd, channel_axis=axis, want_codes=extras, want_mask=extras,
+                                              want_params=True, flags=flags)
+                assert_parity(got, ref, shape, axis, orc.GROUP_CHANNEL, backward=True)
+            if axis == 1 and flags != b.FLAG_FORCE_L2WAVE:
+                got = b.granq_fakequant_fused_fwd_packmask(badd, bits, channel_axis=axis, flags=flags)
+                assert_parity(got, ref, shape, axis, orc.GROUP_CHANNEL, backward=False)
+                assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+                got = b.granq_quantize_packed_fused(badd, bits, channel_axis=axis, flags=flags)
+                assert_same_string(got.packed_codes, orc.pack_codes(ref.codes, bits))
+        except b.GranqError as err:         # a forced plan need not take every geometry
+            assert flags and err.status == b.ERR_UNSUPPORTED
+    if axis == 3:
+        return
+    out = b.WeightBatch([badd.movedim(1, 0).contiguous()], bits, [gyd.movedim(1, 0).contiguous()]).run()[0]
+    first = lambda a: np.ascontiguousarray(np.moveaxis(a, 1, 0))
+    assert same_bits(to_np(out.y), first(ref.y)) and same_bits(to_np(out.gx), first(ref.gx))
