@@ -442,6 +442,14 @@ int granq_cluster_geometry(int dtype, const int64_t dims[4], int channel_axis, i
                            int64_t out[8]);
 
 /*
+ * Host-only query: how the channels-last plan would cut this tensor on a device with `sm_count` SMs.
+ * out = { 16-byte unit columns of a slice, slices, rows of one block, CTAs per slice }.
+ * Returns GRANQ_ERR_UNSUPPORTED when the geometry does not qualify or the device holds fewer CTAs at once than
+ * there would be slices (a call then takes two passes).
+ */
+int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int sm_count, int64_t out[4]);
+
+/*
  * Device self-test (no counterpart in the paper).  The staged kernel divides by the
  * per-group scale with a product and two exact-residual corrections from the correctly
  * rounded reciprocal; this runs `pairs` generated (x, s) pairs, hard cases included,
@@ -478,7 +486,10 @@ enum granq_knob {
     GRANQ_KNOB_CLUSTER_PREFETCH = 14,     /* cluster plan: 1 = L2 prefetch of gy, 2 = none             */
     GRANQ_KNOB_CLUSTER_KMUL = 15,         /* cluster plan: multiplier of a run's minimal channel count */
     GRANQ_KNOB_CLUSTER_EARLY_LAUNCH = 16, /* cluster plan: 2 = launch without programmatic dependent launch */
-    GRANQ_KNOB_COLWALK_TEAM = 17          /* column-walk plan: 2 = L2 waves only (as any set L2 knob means)    */
+    GRANQ_KNOB_COLWALK_TEAM = 17,         /* column-walk plan: 2 = L2 waves only (as any set L2 knob means)    */
+    GRANQ_KNOB_TEST_COOP_CTAS = 18        /* test hook: the cooperative launches that have a plan to fall back on
+                                             (channels-last, resident column walk) count as refused by the driver
+                                             where they have more CTAs than this                             */
 };
 int granq_tune(int knob, int value);
 

@@ -27,8 +27,8 @@ PLAN_TWO_PASS, PLAN_NAIVE, PLAN_STAGED, PLAN_L2WAVE, PLAN_COLWALK, PLAN_CLUSTER,
 (KNOB_STAGED_DEPTH, KNOB_STAGED_MAX_BUF_UNITS, KNOB_STAGED_GRID, KNOB_SPIN_LIMIT, KNOB_TEST_EXTRA_ARRIVALS,
  KNOB_STAGED_CTAS_PER_SM, KNOB_L2_WAVE_KB, KNOB_L2_UPL, KNOB_L2_CTAS_PER_SM, KNOB_L2_LAG,
  KNOB_CLUSTER_TILE_KB, KNOB_CLUSTER_CTAS, KNOB_CLUSTER_THREADS, KNOB_CLUSTER_LOAD, KNOB_CLUSTER_PREFETCH,
- KNOB_CLUSTER_KMUL, KNOB_CLUSTER_EARLY_LAUNCH, KNOB_COLWALK_TEAM) = range(18)
-N_KNOBS = 18
+ KNOB_CLUSTER_KMUL, KNOB_CLUSTER_EARLY_LAUNCH, KNOB_COLWALK_TEAM, KNOB_TEST_COOP_CTAS) = range(19)
+N_KNOBS = 19
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = range(6)
 
 EXPORTS = [
@@ -41,7 +41,7 @@ EXPORTS = [
     "granq_weights_workspace_bytes", "granq_fakequant_weights", "granq_packed_codes_bytes",
     "granq_quantize_packed", "granq_dequantize_packed", "granq_cluster_geometry", "granq_distortion_stats",
     "granq_accumulate_workspace_bytes", "granq_accumulate_codes", "granq_fakequant_fused_batch",
-    "granq_quantize_packed_fused",
+    "granq_quantize_packed_fused", "granq_rows_geometry",
 ]
 NOALLOC_MAX_GROUPS = 32768
 
@@ -121,6 +121,8 @@ def lib() -> ctypes.CDLL:
         L.granq_accumulate_codes.argtypes = [vp, i64p, ci, ci, vp, vp, vp, ctypes.c_int64, vp, vp, sz, u32, vp]
         L.granq_cluster_geometry.restype = ci
         L.granq_cluster_geometry.argtypes = [ci, i64p, ci, ci, ci, i64p]
+        L.granq_rows_geometry.restype = ci
+        L.granq_rows_geometry.argtypes = [ci, i64p, ci, ci, ci, i64p]
         L.granq_selftest_division.restype = ci
         L.granq_selftest_division.argtypes = [ctypes.c_uint64, ctypes.c_uint64, vp, vp]
         L.granq_range_noalloc.restype = ci
@@ -300,6 +302,16 @@ def cluster_geometry(dtype: int, shape, channel_axis: int = 1, group: int = GROU
     _check(rc, "granq_cluster_geometry")
     keys = ["grid", "threads", "cluster", "smem_bytes", "tile_bytes", "channels_per_run", "staging", "prefetch_gy"]
     return dict(zip(keys, [int(v) for v in out]))
+
+
+def rows_geometry(dtype: int, shape, channel_axis: int = 3, group: int = GROUP_CHANNEL, sm_count: int = 148):
+    """Host-only: the cut of the channels-last plan on a GPU with `sm_count` SMs, or None where it has none."""
+    out = (ctypes.c_int64 * 4)()
+    rc = lib().granq_rows_geometry(dtype, _dims(shape), channel_axis, group, sm_count, out)
+    if rc == ERR_UNSUPPORTED:
+        return None
+    _check(rc, "granq_rows_geometry")
+    return dict(zip(["columns", "slices", "lanes", "team"], [int(v) for v in out]))
 
 
 @dataclass

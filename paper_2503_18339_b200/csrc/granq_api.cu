@@ -125,6 +125,17 @@ TeamPlan prefer_team(int dtype, const Geom& g, const QuantIO& io, bool backward,
     return plan_colteam(dtype, g, io, backward, sms);
 }
 
+// The call with its channels held on chip, in the form chosen; where the GPU does not hold that many CTAs at once, by
+// the cluster, which needs no cooperative launch.
+cudaError_t launch_held(const TeamPlan& tp, const ClusterPlan& kp, const QuantIO& io, int mode, int dtype, const Geom& g,
+                        int bits, const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt, cudaStream_t st) {
+    if (tp.ok) {
+        const cudaError_t e = launch_colteam(tp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, g_tune, st);
+        if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+    }
+    return launch_cluster(kp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, g_tune, st);
+}
+
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -248,7 +259,7 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
     // keep that word true for the next call, after.
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     kp.zero_status = !zeroed && kp.clears_status;
-    const bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS;
+    bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS;
     TeamPlan tp{};
     if (plan == PLAN_CLUSTER) tp = prefer_team(dtype, g, io, gy_opt != nullptr, flags);
     cudaError_t e = cudaSuccess;
@@ -258,12 +269,19 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
         e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
     }
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
-    if (tp.ok) {
-        e = launch_colteam(tp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
-    } else if (plan == PLAN_CLUSTER) {
-        e = launch_cluster(kp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
+    // two passes over x by ordinary launches: any geometry, any GPU
+    auto two_pass = [&]() -> cudaError_t {
+        cudaError_t r = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, st);
+        return r == cudaSuccess ? launch_quant_flat(io, mode, dtype, g, bits, min_out, max_out, st) : r;
+    };
+    if (plan == PLAN_CLUSTER) {
+        e = launch_held(tp, kp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st);
     } else if (plan == PLAN_ROWS) {
         e = launch_rows(io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {
+            keeps_zero = false;
+            e = two_pass();
+        }
     } else if (plan == PLAN_STAGED) {
         e = launch_staged(sp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else if (plan == PLAN_L2WAVE) {
@@ -275,8 +293,7 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
         if (e == cudaSuccess && (scale_opt || zp_opt))
             e = launch_params(min_out, max_out, G, bits, scale_opt, zp_opt, st);
     } else {
-        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, st);
-        if (e == cudaSuccess) e = launch_quant_flat(io, mode, dtype, g, bits, min_out, max_out, st);
+        e = two_pass();
     }
     if (e == cudaSuccess && zeroed && !keeps_zero)
         e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);
@@ -369,11 +386,7 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
         // the kernel writes the mask byte by byte: the padding bits of a last, partial word are cleared here
         if (e == cudaSuccess && g.E % 32 != 0) e = cudaMemsetAsync(packed_mask + g.E / 32, 0, sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
-        if (tp.ok)
-            return cuda_status(launch_colteam(tp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt,
-                                              g_tune, st));
-        return cuda_status(launch_cluster(kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt,
-                                          g_tune, st));
+        return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     }
     if (!(zeroed && cp.ok)) e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
@@ -509,11 +522,7 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
         if (!zeroed && (tp.ok || !kp.clears_status))
             e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
-        if (tp.ok)
-            return cuda_status(launch_colteam(tp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt,
-                                              g_tune, st));
-        return cuda_status(launch_cluster(kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt,
-                                          g_tune, st));
+        return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     }
     if (e == cudaSuccess && !(zeroed && cp.ok)) e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
@@ -588,11 +597,7 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
         if (!zeroed && (tp.ok || !kp.clears_status))
             e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
-        if (tp.ok)
-            return cuda_status(launch_colteam(tp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out,
-                                              g_tune, st));
-        return cuda_status(launch_cluster(kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out,
-                                          g_tune, st));
+        return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, st));
     }
     if (!(zeroed && cp.ok)) e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
@@ -737,6 +742,18 @@ int granq_cluster_geometry(int dtype, const int64_t dims[4], int channel_axis, i
     return GRANQ_OK;
 }
 
+int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int sm_count, int64_t out[4]) {
+    Geom g;
+    int64_t G;
+    if (!out || !dtype_ok(dtype) || sm_count < 1 || !make_geom(dims, channel_axis, group, g, G)) return GRANQ_ERR_INVALID_ARG;
+    const QuantIO io{};
+    RowsCut cut{};
+    if (!plan_rows(dtype, g, io) || !cut_rows(dtype, g, 2u * (uint32_t)sm_count, cut)) return GRANQ_ERR_UNSUPPORTED;
+    const int64_t v[4] = {cut.P, cut.slices, cut.lanes, cut.team};
+    for (int i = 0; i < 4; ++i) out[i] = v[i];
+    return GRANQ_OK;
+}
+
 int granq_tune(int knob, int value) {
     switch (knob) {
         case GRANQ_KNOB_STAGED_DEPTH: g_tune.depth = value; return GRANQ_OK;
@@ -757,6 +774,7 @@ int granq_tune(int knob, int value) {
         case GRANQ_KNOB_CLUSTER_KMUL: g_tune.cl_kmul = value; return GRANQ_OK;
         case GRANQ_KNOB_CLUSTER_EARLY_LAUNCH: g_tune.cl_pdl = value; return GRANQ_OK;
         case GRANQ_KNOB_COLWALK_TEAM: g_tune.col_team = value; return GRANQ_OK;
+        case GRANQ_KNOB_TEST_COOP_CTAS: g_tune.coop_ctas = value; return GRANQ_OK;
         default: return GRANQ_ERR_INVALID_ARG;
     }
 }

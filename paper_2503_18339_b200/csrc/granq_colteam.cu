@@ -281,32 +281,32 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
 }
 
 template <typename T, int MODE, int EXTRAS, int BITS = 8>
-cudaError_t t_launch(const TArgs& args, uint32_t smem, cudaStream_t st) {
+cudaError_t t_launch(const TArgs& args, uint32_t smem, const StagedTuning& tune, cudaStream_t st) {
     auto kern = colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2), BITS>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void* params[] = {(void*)&args};
-    return cudaLaunchCooperativeKernel((const void*)kern, dim3(args.R * args.teams), dim3(kTThreads), params, smem, st);
+    return launch_cooperative((const void*)kern, args.R * args.teams, kTThreads, params, smem, tune, st);
 }
 
 template <typename T>
-cudaError_t t_launch_mode(const TArgs& a, int mode, int extras, uint32_t smem, cudaStream_t st) {
-    if (mode == MODE_BOTH) return t_launch<T, MODE_BOTH, 0>(a, smem, st);
+cudaError_t t_launch_mode(const TArgs& a, int mode, int extras, uint32_t smem, const StagedTuning& tune, cudaStream_t st) {
+    if (mode == MODE_BOTH) return t_launch<T, MODE_BOTH, 0>(a, smem, tune, st);
     switch (extras) {
-        case 2: return t_launch<T, MODE_FWD, 2>(a, smem, st);
+        case 2: return t_launch<T, MODE_FWD, 2>(a, smem, tune, st);
         case 3:
             switch (a.code_bits) {
-                case 1: return t_launch<T, MODE_FWD, 3, 1>(a, smem, st);
-                case 2: return t_launch<T, MODE_FWD, 3, 2>(a, smem, st);
-                case 3: return t_launch<T, MODE_FWD, 3, 3>(a, smem, st);
-                case 4: return t_launch<T, MODE_FWD, 3, 4>(a, smem, st);
-                case 5: return t_launch<T, MODE_FWD, 3, 5>(a, smem, st);
-                case 6: return t_launch<T, MODE_FWD, 3, 6>(a, smem, st);
-                case 7: return t_launch<T, MODE_FWD, 3, 7>(a, smem, st);
-                default: return t_launch<T, MODE_FWD, 3, 8>(a, smem, st);
+                case 1: return t_launch<T, MODE_FWD, 3, 1>(a, smem, tune, st);
+                case 2: return t_launch<T, MODE_FWD, 3, 2>(a, smem, tune, st);
+                case 3: return t_launch<T, MODE_FWD, 3, 3>(a, smem, tune, st);
+                case 4: return t_launch<T, MODE_FWD, 3, 4>(a, smem, tune, st);
+                case 5: return t_launch<T, MODE_FWD, 3, 5>(a, smem, tune, st);
+                case 6: return t_launch<T, MODE_FWD, 3, 6>(a, smem, tune, st);
+                case 7: return t_launch<T, MODE_FWD, 3, 7>(a, smem, tune, st);
+                default: return t_launch<T, MODE_FWD, 3, 8>(a, smem, tune, st);
             }
-        case 4: return t_launch<T, MODE_FWD, 4>(a, smem, st);
-        default: return t_launch<T, MODE_FWD, 0>(a, smem, st);
+        case 4: return t_launch<T, MODE_FWD, 4>(a, smem, tune, st);
+        default: return t_launch<T, MODE_FWD, 0>(a, smem, tune, st);
     }
 }
 
@@ -384,8 +384,8 @@ cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, in
     a.expected = plan.R + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
     a.div_plane = make_fastdiv(a.plane_units);
     const int extras = io.dist ? 4 : io.pmask ? 2 : io.pcodes ? 3 : 0;
-    return dtype == 0 ? t_launch_mode<float>(a, mode, extras, plan.smem_bytes, st)
-                      : t_launch_mode<__nv_bfloat16>(a, mode, extras, plan.smem_bytes, st);
+    return dtype == 0 ? t_launch_mode<float>(a, mode, extras, plan.smem_bytes, tune, st)
+                      : t_launch_mode<__nv_bfloat16>(a, mode, extras, plan.smem_bytes, tune, st);
 }
 
 }  // namespace granq

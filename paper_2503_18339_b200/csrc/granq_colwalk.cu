@@ -584,8 +584,10 @@ cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int
         const TeamPlan tp = plan_colteam(dtype, g, io, mode == MODE_BOTH, sms);
         // a hand-over costs a team as much as 2000 units: where the rounds are several and shorter than that (small
         // channels) the waves are faster (forward bf16 [12,2048,33,32], 7 rounds of 1584 units: 48 us, waves 43)
-        if (tp.ok && (tp.tile_units >= 2500 || team_rounds(g.C, tp) == 1))
-            return launch_colteam(tp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, tune, st);
+        if (tp.ok && (tp.tile_units >= 2500 || team_rounds(g.C, tp) == 1)) {
+            e = launch_colteam(tp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, tune, st);
+            if (e != cudaErrorCooperativeLaunchTooLarge) return e;      // else the waves, whose grid follows the occupancy
+        }
     }
     CArgs a{};
     a.x = io.x;

@@ -140,7 +140,18 @@ struct StagedTuning {
     int cl_kmul;          // cluster plan: multiplier of the minimal channel count of a run
     int cl_pdl;           // cluster plan: 2 = no programmatic dependent launch
     int col_team;         // column-walk plan: 2 = L2 waves only
+    int coop_ctas;        // test hook: launch_cooperative() refuses more CTAs than this
 };
+// A cooperative launch that may be refused: every CTA has to be resident at once, and where the GPU is shared out (a
+// partition, a limit on the SMs of a process) fewer are than its attributes say.  cudaErrorCooperativeLaunchTooLarge,
+// with nothing enqueued and no error left behind, tells the caller to take a plan that needs no such launch.
+inline cudaError_t launch_cooperative(const void* kern, uint32_t grid, uint32_t threads, void** params, size_t smem,
+                                      const StagedTuning& tune, cudaStream_t st) {
+    if (tune.coop_ctas > 0 && grid > (uint32_t)tune.coop_ctas) return cudaErrorCooperativeLaunchTooLarge;
+    const cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), params, smem, st);
+    if (e == cudaErrorCooperativeLaunchTooLarge) (void)cudaGetLastError();
+    return e;
+}
 StagedPlan plan_staged(int dtype, const Geom& g, const QuantIO& io, int device, const StagedTuning& tune);
 StagedPlan plan_staged_on(int dtype, const Geom& g, const QuantIO& io, int sm_count, int smem_optin,
                           const StagedTuning& tune);
@@ -171,6 +182,7 @@ struct TeamPlan {
     uint32_t smem_bytes;     // dynamic shared memory per CTA
 };
 TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count);
+// may be refused: launch_cooperative()
 cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
                            const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,
                            const StagedTuning& tune, cudaStream_t st);
@@ -187,6 +199,14 @@ cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int
 
 // ---- channels-last kernels (the channel is the innermost axis: one 16-byte unit holds V channels of a row) ----
 bool plan_rows(int dtype, const Geom& g, const QuantIO& io);
+struct RowsCut {
+    uint32_t P, slices;      // unit columns of a slice, slices
+    uint32_t lanes;          // rows of threads: the rows of one block
+    uint32_t team;           // CTAs per slice
+};
+// false where the GPU holds too few CTAs at once for any cut (ctas: how many)
+bool cut_rows(int dtype, const Geom& g, uint32_t ctas, RowsCut& cut);
+// may be refused: launch_cooperative()
 cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, int bits, const Workspace& ws,
                         float* lo, float* hi, float* s_opt, float* z_opt, const StagedTuning& tune, cudaStream_t st);
 

@@ -277,12 +277,12 @@ __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a)
 bool r_aligned16(const void* p) { return p == nullptr || ((uintptr_t)p & 15) == 0; }
 
 template <typename T, int MODE>
-cudaError_t r_launch(const RArgs& a, bool extras, int grid, int threads, size_t smem, cudaStream_t st) {
+cudaError_t r_launch(const RArgs& a, bool extras, int grid, int threads, size_t smem, const StagedTuning& tune, cudaStream_t st) {
     auto go = [&](auto kern) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         void* params[] = {(void*)&a};
-        return cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(threads), params, smem, st);
+        return launch_cooperative((const void*)kern, (uint32_t)grid, (uint32_t)threads, params, smem, tune, st);
     };
     constexpr int U1 = Pack<T>::V == 4 ? 8 : 6;
     return extras ? go(rows_kernel<T, MODE, true, U1, 2>) : go(rows_kernel<T, MODE, false, U1, 2>);
@@ -297,6 +297,28 @@ bool plan_rows(int dtype, const Geom& g, const QuantIO& io) {
     if (g.inner != 1 || g.C < V || g.C % V != 0 || g.C > (int64_t)kRMaxChannels || g.outer < 1) return false;
     if (!r_aligned16(io.x) || !r_aligned16(io.gy) || !r_aligned16(io.y) || !r_aligned16(io.gx)) return false;
     if (((uintptr_t)io.codes & 3) || ((uintptr_t)io.mask & 3)) return false;
+    return true;
+}
+
+// The cut of a row into slices that leaves the fewest threads and CTAs without work (196 unit columns: 7 slices of 28,
+// 16 rows of threads each); slices of 64 unit columns at most, of 16 at least where there are several.
+bool cut_rows(int dtype, const Geom& g, uint32_t ctas, RowsCut& cut) {
+    const uint32_t V = dtype == 0 ? 4 : 8, ncol = (uint32_t)(g.C / V);
+    const uint32_t top = dtype == 0 ? kRMaxThreads<float> : kRMaxThreads<__nv_bfloat16>;
+    double best = 0.0;
+    for (uint32_t slices = (ncol + 63) / 64; slices <= std::max<uint32_t>(1, ncol / 16); ++slices) {
+        const uint32_t P = (ncol + slices - 1) / slices, lanes = top / P, used = (ncol + P - 1) / P;
+        const double eff = (double)ncol / (double)(used * P) * (double)(P * lanes) / top * (double)(ctas / used * used) / ctas;
+        if (eff > best + 0.02) {
+            best = eff;
+            cut.P = P;
+            cut.slices = used;
+            cut.lanes = lanes;
+        }
+    }
+    if (best == 0.0) return false;
+    const uint64_t blocks = ((uint64_t)g.outer + cut.lanes - 1) / cut.lanes;      // no more CTAs than there are blocks of rows
+    cut.team = (uint32_t)std::min<uint64_t>(blocks, ctas / cut.slices);
     return true;
 }
 
@@ -327,22 +349,13 @@ cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, i
     a.C = (uint32_t)g.C;
     a.ncol = (uint32_t)(g.C / V);
     a.rows = (uint64_t)g.outer;
-    // the cut of a row into slices that leaves the fewest threads and CTAs without work (196 unit columns: 7 slices of
-    // 28, 16 rows of threads each); slices of 64 unit columns at most, of 16 at least where there are several
-    const uint32_t top = dtype == 0 ? kRMaxThreads<float> : kRMaxThreads<__nv_bfloat16>, ctas = 2u * (uint32_t)sms;
-    double best = 0.0;
-    for (uint32_t slices = (a.ncol + 63) / 64; slices <= std::max<uint32_t>(1, a.ncol / 16); ++slices) {
-        const uint32_t P = (a.ncol + slices - 1) / slices, lanes = top / P, used = (a.ncol + P - 1) / P;
-        const double eff = (double)a.ncol / (double)(used * P) * (double)(P * lanes) / top * (double)(ctas / used * used) / ctas;
-        if (eff > best + 0.02) {
-            best = eff;
-            a.P = P;
-            a.slices = used;
-            a.lanes = lanes;
-        }
-    }
-    const uint64_t blocks = (a.rows + a.lanes - 1) / a.lanes;      // no more CTAs than there are blocks of rows
-    a.team = (uint32_t)std::min<uint64_t>(blocks, ctas / a.slices);
+    RowsCut cut{};
+    if (!cut_rows(dtype, g, 2u * (uint32_t)sms, cut)) return cudaErrorCooperativeLaunchTooLarge;
+    a.P = cut.P;
+    a.slices = cut.slices;
+    a.lanes = cut.lanes;
+    a.team = cut.team;
+    const uint64_t blocks = (a.rows + a.lanes - 1) / a.lanes;
     const int grid = (int)(a.team * a.slices), threads = (int)((a.P * a.lanes + 31) / 32 * 32);
     const size_t table = (size_t)a.P * V * sizeof(GroupParam), block = (size_t)a.P * a.lanes * 16;
     // all of a CTA's blocks or none: loads in flight need L1, which is what shared memory leaves of 256 KB (keeping a
@@ -358,11 +371,11 @@ cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, i
     a.expected = a.team + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
     const bool extras = io.codes != nullptr || io.mask != nullptr;
     if (dtype == 0) {
-        if (mode == MODE_FWD) return r_launch<float, MODE_FWD>(a, extras, grid, threads, smem, st);
-        return r_launch<float, MODE_BOTH>(a, extras, grid, threads, smem, st);
+        if (mode == MODE_FWD) return r_launch<float, MODE_FWD>(a, extras, grid, threads, smem, tune, st);
+        return r_launch<float, MODE_BOTH>(a, extras, grid, threads, smem, tune, st);
     }
-    if (mode == MODE_FWD) return r_launch<__nv_bfloat16, MODE_FWD>(a, extras, grid, threads, smem, st);
-    return r_launch<__nv_bfloat16, MODE_BOTH>(a, extras, grid, threads, smem, st);
+    if (mode == MODE_FWD) return r_launch<__nv_bfloat16, MODE_FWD>(a, extras, grid, threads, smem, tune, st);
+    return r_launch<__nv_bfloat16, MODE_BOTH>(a, extras, grid, threads, smem, tune, st);
 }
 
 }  // namespace granq

@@ -248,3 +248,27 @@ def test_cluster_plan_cuts_within_its_limits(lib):
         for k in range(b.N_KNOBS):
             b.tune(k, 0)
     assert planned > 300
+
+
+def test_rows_plan_cuts_within_what_the_gpu_holds(lib):
+    """Host-only: every cut of the channels-last planner covers the row, keeps a block of rows within the threads of a
+    CTA and asks for no more CTAs than are resident at once; a GPU (or a part of one) with fewer SMs than there would
+    be slices gets no cut instead of an empty one."""
+    from paper_2503_18339_b200 import binding as b
+    rnd = random.Random(12)
+    refused = 0
+    for _ in range(4000):
+        dt, sms = rnd.choice([0, 1]), rnd.choice([1, 2, 3, 4, 8, 16, 66, 132, 148])
+        V, top = (4, 448) if dt == 0 else (8, 384)
+        C = V * rnd.randint(1, 4096 // V)
+        rows = rnd.choice([1, 7, 128, 40_000])
+        geo = b.rows_geometry(dt, (rows, rnd.choice([1, 3]), 2, C), sm_count=sms)
+        ncol, ctas = C // V, 2 * sms
+        if geo is None:
+            refused += 1
+            assert (ncol + 63) // 64 > ctas
+            continue
+        assert 1 <= geo["columns"] <= 64 and geo["columns"] * geo["slices"] >= ncol > geo["columns"] * (geo["slices"] - 1)
+        assert geo["lanes"] >= 1 and geo["columns"] * geo["lanes"] <= top
+        assert geo["team"] >= 1 and geo["team"] * geo["slices"] <= ctas
+    assert refused

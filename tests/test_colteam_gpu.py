@@ -115,3 +115,29 @@ def test_a_reported_timeout_outlives_later_calls_on_the_same_zeroed_workspace(b,
     got = b.granq_fakequant_fused(xd, 4, gy=gyd, out=new(), flags=b.FLAG_FORCE_CLUSTER)      # clears the word itself
     assert b.workspace_status(ws) == b.OK
     assert same_bits(to_np(got.y), orc.fused(x, 4, gy=gy).y)
+
+
+@pytest.mark.parametrize("dtype,shape,forced", [("f32", (256, 168, 28, 28), False), ("bf16", (256, 256, 28, 28), False),
+                                                ("f32", (9, 24, 12, 12), True), ("bf16", (9, 24, 12, 12), True)])
+def test_a_refused_cooperative_launch_falls_back(b, knobs, dtype, shape, forced):
+    """A GPU that is shared out holds fewer CTAs at once than its attributes say: where a cluster holds a channel the
+    call takes the cluster, else the waves (whose grid follows the occupancy)."""
+    x, gy = make_case(shape, seed=6, dtype=dtype)
+    ref = orc.fused(x, 4, gy=gy)
+    xd, gyd = to_dev(x), to_dev(gy)
+    ws = b.make_workspace(xd)
+    new = lambda: b.FakeQuantOut(workspace=ws.fill_(255))
+    flags = b.FLAG_FORCE_COLWALK if forced else 0
+    b.tune(b.KNOB_TEST_COOP_CTAS, 1)
+    assert_parity(b.granq_fakequant_fused(xd, 4, out=new(), flags=flags), ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert b.workspace_status(ws) == b.OK
+    assert_parity(b.granq_fakequant_fused(xd, 4, gy=gyd, out=new(), flags=flags), ref, shape, 1, orc.GROUP_CHANNEL, backward=True)
+    assert b.workspace_status(ws) == b.OK
+    got = b.granq_fakequant_fused_fwd_packmask(xd, 4, out=new(), flags=flags)
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+    got = b.granq_quantize_packed_fused(xd, 4, out=new(), flags=flags)
+    assert_same_string(got.packed_codes, orc.pack_codes(ref.codes, 4))
+    got = b.granq_fakequant_fused_stats(xd, 4, out=new(), flags=flags)
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert b.workspace_status(ws) == b.OK

@@ -116,3 +116,30 @@ def test_rows_hand_over_that_never_completes_is_reported(b):
         b.tune(b.KNOB_TEST_EXTRA_ARRIVALS, 0)
         b.tune(b.KNOB_SPIN_LIMIT, 0)
     run(b, x, gy, 4, 3)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_channels_last_where_the_cooperative_launch_is_refused(b, dtype):
+    """A GPU that is shared out holds fewer CTAs at once than its attributes say: the call then takes two passes, and a
+    workspace that was zero is zero afterwards."""
+    shape = (6, 9, 8, 40)
+    x, gy = make_case(shape, seed=4, dtype=dtype)
+    ref = orc.fused(x, 5, gy=gy, channel_axis=3)
+    xd, gyd = to_dev(x), to_dev(gy)
+    ws = b.make_workspace(xd, channel_axis=3, zeroed=True)
+    assert b.fused_plan(b.BF16 if dtype == "bf16" else b.F32, shape, channel_axis=3)[0] == b.PLAN_ROWS
+    b.tune(b.KNOB_TEST_COOP_CTAS, 1)
+    try:
+        for flags in (b.FLAG_WORKSPACE_ZEROED, 0, b.FLAG_WORKSPACE_ZEROED):
+            if not flags:
+                ws.fill_(255)
+            got = b.granq_fakequant_fused(xd, 5, gy=gyd, channel_axis=3, want_codes=True, want_mask=True, want_params=True,
+                                          out=b.FakeQuantOut(workspace=ws), flags=flags)
+            assert b.workspace_status(ws) == b.OK
+            assert_parity(got, ref, shape, 3, orc.GROUP_CHANNEL, backward=True)
+            if flags:
+                assert int(ws.view(torch.int32).abs().sum().item()) == 0
+            else:
+                ws.zero_()
+    finally:
+        b.tune(b.KNOB_TEST_COOP_CTAS, 0)
