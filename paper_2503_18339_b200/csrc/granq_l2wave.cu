@@ -297,6 +297,9 @@ inline uint32_t l_gcd(uint32_t a, uint32_t b) {
 bool l_aligned16(const void* p) { return p == nullptr || ((uintptr_t)p & 15) == 0; }
 
 // CTAs of one instantiation that fit on an SM (queried once per kernel and shared-memory size class)
+// shared memory of a wave of `channels`: keys (8 B) and parameters (16 B) per group
+constexpr uint32_t l_smem_bytes(uint32_t channels) { return 24u * (((channels + 15u) / 16u) * 16u); }
+
 template <typename K>
 int resident_ctas(K kern, uint32_t smem) {
     int n = 0;
@@ -307,8 +310,9 @@ int resident_ctas(K kern, uint32_t smem) {
 template <typename T, int MODE, bool ALIGNED, bool EXTRAS, int UPL>
 cudaError_t l_launch_upl(const L2Plan& plan, LArgs& args, int sm_count, int cta_cap, cudaStream_t st) {
     auto kern = l2wave_kernel<T, MODE, ALIGNED, EXTRAS, UPL>;
-    if (plan.smem_bytes > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
+    // waves of close to kLTabMax channels: with the static part they pass the 48 KB that need no asking for
+    if (plan.smem_bytes > 32 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l_smem_bytes(kLTabMax));
         if (e != cudaSuccess) return e;
     }
     int per_sm = resident_ctas(kern, plan.smem_bytes);
@@ -362,7 +366,7 @@ L2Plan plan_l2wave(int dtype, const Geom& g, const QuantIO& io, const StagedTuni
     if ((uint64_t)p.cw * inner / V >= (1ull << 30)) return p;
     // long planes: rows of 128 units lie in one channel and amortise the row set-up; short planes: 64
     p.upl = tune.l2_upl == 4 ? 4 : (tune.l2_upl == 2 ? 2 : ((inner / V) >= 512 ? 4 : 2));
-    p.smem_bytes = 24u * (((p.cw + 15u) / 16u) * 16u);     // keys (8 B) and parameters (16 B) per group
+    p.smem_bytes = l_smem_bytes(p.cw);
     p.ok = true;
     return p;
 }

@@ -220,6 +220,17 @@ def test_l2wave_multiwave(b, knobs, shape, upl, dtype):
         assert_parity(got, ref_f, shape, 1, orc.GROUP_CHANNEL, backward=False)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_l2wave_of_as_many_channels_as_a_wave_takes(b, dtype):
+    """A wave of 2048 channels: its tables and the kernel's static shared memory together exceed 48 KB."""
+    shape = (3, 4096, 4, 4)
+    x, gy = make_case(shape, seed=11, dtype=dtype)
+    ref = orc.fused(x, 4, gy=gy)
+    got = b.granq_fakequant_fused(to_dev(x), 4, gy=to_dev(gy), want_params=True, flags=b.FLAG_FORCE_L2WAVE)
+    assert b.workspace_status(got.workspace) == b.OK
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=True)
+
+
 def test_l2wave_bounded_wait_reports_timeout(b, knobs):
     shape = (4, 16, 14, 14)
     x, gy = make_case(shape, seed=2)
