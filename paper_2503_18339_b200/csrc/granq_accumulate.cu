@@ -36,6 +36,7 @@ namespace {
 constexpr int kABm = 128;                 // pixels per tile (rows of the accumulator = tensor-memory lanes)
 constexpr int kABk = 64;                  // channels per stage: 64 bf16 = one 128-byte swizzle row
 constexpr int kAMaxStages = 4;         // the ring is as deep as the K blocks need, at most this
+constexpr int kAStages = 2;               // operand stages of the form with one pixel tile per CTA
 constexpr int kAThreads = 128;            // all four warps expand codes and run the epilogue; thread 0 loads the
                                           // weights, thread 32 issues the MMAs
 constexpr uint32_t kASpin = 1u << 22;     // bounded mbarrier wait
@@ -879,7 +880,7 @@ cudaError_t a_launch(const CUtensorMap& mh, const CUtensorMap& ml, const AArgs& 
     // a short ring leaves room for several CTAs per SM, whose load / multiply / store chains then overlap
     const size_t smem = (size_t)args.stages * (kABm * kABk * 2 + 2 * BN * kABk * 2) + 1024;
     auto kern = accumulate_kernel<BN, NHWC>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, (size_t)kAStages * (kABm * kABk * 2 + 2 * BN * kABk * 2) + 1024);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)((args.rows + kABm - 1) / kABm), (unsigned)((args.O + BN - 1) / BN));
     kern<<<grid, kAThreads, smem, st>>>(mh, ml, args);
@@ -891,7 +892,7 @@ template <int BN, bool NHWC>
 cudaError_t p_launch(const CUtensorMap& mh, const CUtensorMap& ml, const AArgs& args, cudaStream_t st) {
     const size_t smem = (size_t)kPStages * kABm * kABk * 2 + (size_t)args.kblocks * 2 * BN * kABk * 2 + 1024;
     auto kern = accumulate_persistent_kernel<BN, NHWC>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, (size_t)kPStages * kABm * kABk * 2 + kPWeightBytes - (NHWC ? 16 * 1024 : 0) + 1024);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -967,7 +968,7 @@ extern "C" int granq_accumulate_codes(const uint32_t* packed_codes, const int64_
     args.bits = bits;
     args.kblocks = kblocks;
     args.spin_limit = kASpin;
-    args.stages = std::min(args.kblocks, 2);
+    args.stages = std::min(args.kblocks, kAStages);
     const bool persistent = !one_tile_per_cta && resident(BN);
     cudaError_t e = cudaSuccess;
     if (persistent) {

@@ -34,6 +34,8 @@ constexpr int kKBars = 8;                    // mbarriers per tile: the range wa
 constexpr uint32_t kKSpinLimit = 1u << 22;   // bounded wait on a bulk-copy barrier
 constexpr uint32_t kKStatusTimeout = 5;      // GRANQ_ERR_TIMEOUT
 constexpr uint32_t kKMaxRunChannels = 2048;  // channels of one run (keys and parameters live in shared memory)
+constexpr uint32_t kKTileBytes = 112u * 1024;      // staged tiles of one CTA: two CTAs per SM
+constexpr uint32_t kKSmemBytes = kKTileBytes + kKMaxRunChannels * (2 * sizeof(uint32_t) + sizeof(GroupParam));
 
 struct KArgs {
     const void* x;
@@ -553,7 +555,7 @@ uint32_t k_gcd(uint32_t a, uint32_t b) {
 template <typename T, int MODE, bool ALIGNED, int EXTRAS>
 cudaError_t k_launch_t(const KArgs& args, const ClusterPlan& plan, uint32_t grid, cudaStream_t st) {
     auto launch = [&](auto kern) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
+        const cudaError_t e = allow_smem(kern, std::max(plan.smem_bytes, kKSmemBytes));      // more only where a knob asks
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(grid);
@@ -627,7 +629,7 @@ ClusterPlan plan_cluster(int dtype, const Geom& g, const QuantIO& io, bool backw
     // 4 = per-thread asynchronous copies for x, 5 = for x and gy.  Default: asynchronous copies; gy is staged
     // too for fp32 tensors with a gradient when that still fits a portable cluster (measured faster there;
     // bf16 halves the bytes per element, and reading gy in the quantize walk measured faster).
-    const uint64_t limit = tune.cl_tile_kb > 0 ? (uint64_t)tune.cl_tile_kb * 1024 : 112ull * 1024;   // two CTAs per SM
+    const uint64_t limit = tune.cl_tile_kb > 0 ? (uint64_t)tune.cl_tile_kb * 1024 : kKTileBytes;
     // a run is whole 16-byte units; with a packed mask also whole bytes of mask (8 elements)
     const uint32_t unit = (io.pmask || io.pcodes) ? 8u : V;
     const uint64_t group_bytes = (uint64_t)g.outer * (unit / k_gcd((uint32_t)g.inner, unit)) * g.inner * esize;

@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
 template <typename T, int MODE, int EXTRAS, int BITS = 8>
 cudaError_t t_launch(const TArgs& args, uint32_t smem, const StagedTuning& tune, cudaStream_t st) {
     auto kern = colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2), BITS>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, kTSmemUnits * 16);
     if (e != cudaSuccess) return e;
     void* params[] = {(void*)&args};
     return launch_cooperative((const void*)kern, args.R * args.teams, kTThreads, params, smem, tune, st);

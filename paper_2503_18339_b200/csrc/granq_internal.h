@@ -87,6 +87,14 @@ struct QuantIO {
     int code_bits;
 };
 
+// Room for dynamic shared memory.  The attribute belongs to the kernel, not to the launch: every call states the same
+// value, the most the kernel's plans ask for, so that calls of different sizes from several threads cannot take it
+// from one another between stating it and launching.  (What a launch really takes of an SM is its own size.)
+template <typename K>
+inline cudaError_t allow_smem(K kern, size_t most) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // ---- generic ("flat") kernels: any geometry, any alignment --------------------------------
 // Range of every group (Eq. 4) into lo / hi, and s / z when bits > 0 and the pointers are given (Eq. 5).  The keys and,
 // where one is given, the counter must be zero on entry; with a counter the range launch finishes by itself.

@@ -312,7 +312,7 @@ cudaError_t l_launch_upl(const L2Plan& plan, LArgs& args, int sm_count, int cta_
     auto kern = l2wave_kernel<T, MODE, ALIGNED, EXTRAS, UPL>;
     // waves of close to kLTabMax channels: with the static part they pass the 48 KB that need no asking for
     if (plan.smem_bytes > 32 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l_smem_bytes(kLTabMax));
+        cudaError_t e = allow_smem(kern, l_smem_bytes(kLTabMax));
         if (e != cudaSuccess) return e;
     }
     int per_sm = resident_ctas(kern, plan.smem_bytes);

@@ -279,7 +279,7 @@ bool r_aligned16(const void* p) { return p == nullptr || ((uintptr_t)p & 15) == 
 template <typename T, int MODE>
 cudaError_t r_launch(const RArgs& a, bool extras, int grid, int threads, size_t smem, const StagedTuning& tune, cudaStream_t st) {
     auto go = [&](auto kern) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(kern, kRSmemBytes);
         if (e != cudaSuccess) return e;
         void* params[] = {(void*)&a};
         return launch_cooperative((const void*)kern, (uint32_t)grid, (uint32_t)threads, params, smem, tune, st);

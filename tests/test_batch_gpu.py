@@ -1,5 +1,7 @@
 """granq_fakequant_fused_batch: a list of tensors in one host call.  Every tensor must come out bit for bit as the
 oracle computes it (and as the single call does); a bad descriptor stops the batch at its index."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -93,3 +95,36 @@ def test_batch_tensors_that_run_beside_one_another_and_tensors_that_depend(b):
             assert b.workspace_status(outs[i].workspace) == b.OK
             assert same_bits(to_np(outs[i].y), ref.y) and same_bits(to_np(outs[i].gx), ref.gx), f"tensor {i}"
             assert same_bits(to_np(outs[i].lo), ref.lo) and same_bits(to_np(outs[i].hi), ref.hi)
+
+
+@pytest.mark.parametrize("axis,big,small,forced", [(1, (128, 16, 56, 56), (8, 16, 8, 8), "FORCE_COLWALK"), (3, (9, 14, 14, 2048), (4, 4, 4, 16), None),
+                                                   (1, (32, 48, 28, 28), (4, 16, 8, 8), "FORCE_CLUSTER")],
+                         ids=["resident column walk", "channels-last", "cluster-local"])
+def test_calls_of_different_sizes_from_several_threads(b, axis, big, small, forced):
+    """Threads with a stream each whose calls take the same kernel with much and with little shared memory."""
+    flags = getattr(b, "FLAG_" + forced) if forced else 0
+    errors, outs = [], {}
+
+    def work(name, x, stream):
+        try:
+            out = b.FakeQuantOut(y=torch.empty_like(x), workspace=b.make_workspace(x, axis),
+                                 **{k: torch.empty(x.shape[axis], device="cuda") for k in ("lo", "hi")})
+            for _ in range(400):
+                b.granq_fakequant_fused(x, 4, channel_axis=axis, out=out, flags=flags, stream=stream)
+            outs[name] = out
+        except Exception as err:
+            errors.append(err)
+
+    cases = {f"{k} {i}": make_case(s, seed=i)[0] for k, s in (("big", big), ("small", small)) for i in range(2)}
+    xs = {name: to_dev(x) for name, x in cases.items()}
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(name, x, torch.cuda.Stream())) for name, x in xs.items()]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    for name, x in cases.items():
+        assert b.workspace_status(outs[name].workspace) == b.OK
+        assert same_bits(to_np(outs[name].y), orc.fused(x, 4, channel_axis=axis).y)
