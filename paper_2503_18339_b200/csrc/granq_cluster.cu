@@ -119,6 +119,15 @@ __device__ __forceinline__ void k_red_max_peer(const uint32_t* local, uint32_t r
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(k_smem_u32(local)), "r"(rank));
     asm volatile("red.relaxed.cluster.shared::cluster.max.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
+// 16-byte load that reads the L2 whatever the L1 holds, L2 eviction hint: see late_wait in the kernel
+__device__ __forceinline__ uint4 k_ld_l2_16(const void* p, uint64_t policy) {
+    uint4 v;
+    asm volatile("ld.relaxed.gpu.global.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p), "l"(policy)
+                 : "memory");
+    return v;
+}
 // per-thread asynchronous 16-byte copy global -> shared (both 16-byte aligned), L2 eviction hint
 __device__ __forceinline__ void k_cp_async_16(void* dst_smem, const void* src, uint64_t policy) {
     asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(k_smem_u32(dst_smem)), "l"(src),
@@ -265,8 +274,13 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
     // waits for that kernel's memory; dependents of this grid may start their own preamble from here on.
     // In a list of tensors that share no memory the wait moves to the end of the kernel: it then runs beside the kernels
     // ahead of it and still does not complete before they do, so whatever comes after the list needs to know its last
-    // kernel only.  (It starts when every CTA of the kernel ahead has come past this line, so after the one wait of the
-    // list's first kernel.)
+    // kernel only.  What it reads was written before the list, by kernels that its own wait would come too late for:
+    //   - it starts when every CTA of the kernel ahead has come past this line, so - that kernel having started the same
+    //     way - after every CTA of the list's first kernel has come past its wait.  By then what was written before the
+    //     list is performed at the L2, for all of the GPU;
+    //   - x and gy are read from the L2 and nowhere nearer: cp.async.cg and the relaxed GPU-scope load pass the L1 by, in
+    //     which an SM may hold lines of the same addresses from before they were written.
+    // No other memory is read; what it writes is nobody's before the list has ended.
     if (!a.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the call's status: only bulk copies can run out of a wait, and their caller clears the word ahead of the launch.
@@ -367,7 +381,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
                 for (; s + (U1 - 1) * nrows < nl; s += U1 * nrows) {
                     Pack<T> v[U1];
 #pragma unroll
-                    for (int j = 0; j < U1; ++j) v[j].raw = ld_hint_16(p + (size_t)j * gstep, drop);
+                    for (int j = 0; j < U1; ++j) v[j].raw = k_ld_l2_16(p + (size_t)j * gstep, drop);
 #pragma unroll
                     for (int j = 0; j < U1; ++j) {
                         acc.add(v[j]);
@@ -380,7 +394,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
                     Pack<T> v[U1 - 1];
 #pragma unroll
                     for (int j = 0; j < U1 - 1; ++j)
-                        if (s + j * nrows < nl) v[j].raw = ld_hint_16(p + (size_t)j * gstep, drop);
+                        if (s + j * nrows < nl) v[j].raw = k_ld_l2_16(p + (size_t)j * gstep, drop);
 #pragma unroll
                     for (int j = 0; j < U1 - 1; ++j)
                         if (s + j * nrows < nl) {
@@ -502,7 +516,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
 #pragma unroll
             for (int j = 0; j < U2; ++j) {
                 if constexpr (GY) pg[j].raw = qg[(size_t)j * sstep];
-                else if constexpr (kBwd) pg[j].raw = ld_hint_16(gyg + gu + (size_t)j * gstep, drop);
+                else if constexpr (kBwd) pg[j].raw = k_ld_l2_16(gyg + gu + (size_t)j * gstep, drop);
             }
 #pragma unroll
             for (int j = 0; j < U2; ++j) px[j].raw = q[(size_t)j * sstep];
@@ -518,7 +532,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
                 if (!gy_ready(s)) break;
                 pg.raw = *qg;
             } else if constexpr (kBwd) {
-                pg.raw = ld_hint_16(gyg + gu, drop);
+                pg.raw = k_ld_l2_16(gyg + gu, drop);
             }
             px.raw = *q;
             emit(px, pg, gu);

@@ -97,6 +97,34 @@ def test_batch_tensors_that_run_beside_one_another_and_tensors_that_depend(b):
             assert same_bits(to_np(outs[i].lo), ref.lo) and same_bits(to_np(outs[i].hi), ref.hi)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_batch_reads_what_was_written_just_before_it(b, dtype):
+    """The inputs of all tensors of a list are rewritten by the kernel ahead of it, in place, round after round: the
+    tensors that start beside the first one must see the new values (bf16 reads gy in the quantize walk)."""
+    shape, n = (16, 64, 14, 14), 9
+    src = [make_case(shape, seed=90 + i, dtype=dtype) for i in range(3)]
+    t = torch.bfloat16 if dtype == "bf16" else torch.float32
+    X, GY = (torch.empty((n,) + shape, dtype=t, device="cuda") for _ in range(2))
+    outs = [b.FakeQuantOut(y=torch.empty(shape, dtype=t, device="cuda"), gx=torch.empty(shape, dtype=t, device="cuda")) for _ in range(n)]
+    batch = b.FusedBatch([(X[i], 4, GY[i]) for i in range(n)], outs=outs, zeroed=True)
+    srcd = [(to_dev(x), to_dev(gy)) for x, gy in src]
+    refs = [orc.fused(x, 4, gy=gy) for x, gy in src]
+    kept = [(torch.empty((n,) + shape, dtype=t, device="cuda"), torch.empty((n,) + shape, dtype=t, device="cuda")) for _ in range(6)]
+    torch.cuda.synchronize()
+    for r, (ys, gxs) in enumerate(kept):
+        x, gy = srcd[r % 3]
+        GY.copy_(gy.expand_as(GY))
+        X.copy_(x.expand_as(X))
+        batch.run()
+        for i in range(n):
+            ys[i].copy_(outs[i].y)
+            gxs[i].copy_(outs[i].gx)
+    torch.cuda.synchronize()
+    for r, (ys, gxs) in enumerate(kept):
+        for i in range(n):
+            assert same_bits(to_np(ys[i]), refs[r % 3].y) and same_bits(to_np(gxs[i]), refs[r % 3].gx), f"round {r}, tensor {i}"
+
+
 @pytest.mark.parametrize("axis,big,small,forced", [(1, (128, 16, 56, 56), (8, 16, 8, 8), "FORCE_COLWALK"), (3, (9, 14, 14, 2048), (4, 4, 4, 16), None),
                                                    (1, (32, 48, 28, 28), (4, 16, 8, 8), "FORCE_CLUSTER")],
                          ids=["resident column walk", "channels-last", "cluster-local"])
