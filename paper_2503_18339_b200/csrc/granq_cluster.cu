@@ -128,11 +128,9 @@ __device__ __forceinline__ uint4 k_ld_l2_16(const void* p, uint64_t policy) {
                  : "memory");
     return v;
 }
-// per-thread asynchronous 16-byte copy global -> shared (both 16-byte aligned), L2 eviction hint
-__device__ __forceinline__ void k_cp_async_16(void* dst_smem, const void* src, uint64_t policy) {
-    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(k_smem_u32(dst_smem)), "l"(src),
-                 "l"(policy)
-                 : "memory");
+// per-thread asynchronous 16-byte copy global -> shared (both 16-byte aligned)
+__device__ __forceinline__ void k_cp_async_16(void* dst_smem, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(k_smem_u32(dst_smem)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void k_cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -308,7 +306,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
             for (uint32_t col = cin; col < ncol; col += P) {
                 const uint4* p = xg + (size_t)r0 * slab + col;
                 uint4* q = tile + (size_t)r0 * ncol + col;
-                for (uint32_t s = r0; s < nl; s += nrows, p += gstep, q += sstep) k_cp_async_16(q, p, drop);
+                for (uint32_t s = r0; s < nl; s += nrows, p += gstep, q += sstep) k_cp_async_16(q, p);
             }
         }
         k_cp_async_commit();
@@ -317,7 +315,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
                 for (uint32_t col = cin; col < ncol; col += P) {
                     const uint4* p = gyg + (size_t)r0 * slab + col;
                     uint4* q = tileg + (size_t)r0 * ncol + col;
-                    for (uint32_t s = r0; s < nl; s += nrows, p += gstep, q += sstep) k_cp_async_16(q, p, drop);
+                    for (uint32_t s = r0; s < nl; s += nrows, p += gstep, q += sstep) k_cp_async_16(q, p);
                 }
             }
             k_cp_async_commit();

@@ -125,7 +125,6 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     const uint4* gyg = reinterpret_cast<const uint4*>(a.gy);
     uint4* yg = reinterpret_cast<uint4*>(a.y);
     uint4* gxg = reinterpret_cast<uint4*>(a.gx);
-    const uint64_t drop = l2_policy_evict_first();
     const float qmax = a.qmax;
     DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS = 4)
     dacc.reset();
@@ -217,8 +216,8 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
                 store_code_bytes<V>(a.pcodes, at * V, str, BITS, lane);
                 return;
             }
-            st_hint_16(yg + at, py.raw, drop);
-            if constexpr (kBwd) st_hint_16(gxg + at, pgx.raw, drop);
+            st_stream_16(yg + at, py.raw);
+            if constexpr (kBwd) st_stream_16(gxg + at, pgx.raw);
             if constexpr (EXTRAS == 4) dacc.add(px, py);
             if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, at * V, mask_bits_of<V, EXTRAS>(mb), lane);
         };
@@ -232,7 +231,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
                 w[j] = at;
                 if constexpr (kBwd) {
                     if (i + j < gcnt) pg[j].raw = tileg[(i + j) * kTThreads];
-                    else pg[j].raw = ld_hint_16(gyg + at, drop);
+                    else pg[j].raw = ld_stream_16(gyg + at);
                 }
                 px[j].raw = tile[(i + j) * kTThreads];
                 advance(at, off);
@@ -251,7 +250,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
             Pack<T> px, pg;
             if constexpr (kBwd) {
                 if (i < gcnt) pg.raw = tileg[i * kTThreads];
-                else pg.raw = ld_hint_16(gyg + at, drop);
+                else pg.raw = ld_stream_16(gyg + at);
             }
             px.raw = tile[i * kTThreads];
             if (more) {
