@@ -442,6 +442,17 @@ int granq_cluster_geometry(int dtype, const int64_t dims[4], int channel_axis, i
                            int64_t out[8]);
 
 /*
+ * Host-only query: how the resident form of the column walk (a channel held by a team of CTAs) would cut this tensor on
+ * a device with `sm_count` SMs.
+ * out = { CTAs per team, teams, 16-byte units of x that one CTA holds, channels that a team takes one after the other,
+ *         1 if the column-walk plan takes this form for it rather than the L2 waves }.
+ * Returns GRANQ_ERR_UNSUPPORTED when a channel does not fit or planes are no whole 16-byte units.  Calls with byte codes
+ * or masks take the waves whatever the answer.
+ */
+int granq_team_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward, int sm_count,
+                        int64_t out[5]);
+
+/*
  * Host-only query: how the channels-last plan would cut this tensor on a device with `sm_count` SMs.
  * out = { 16-byte unit columns of a slice, slices, rows of one block, CTAs per slice }.
  * Returns GRANQ_ERR_UNSUPPORTED when the geometry does not qualify or the device holds fewer CTAs at once than
@@ -486,7 +497,8 @@ enum granq_knob {
     GRANQ_KNOB_CLUSTER_PREFETCH = 14,     /* cluster plan: 1 = L2 prefetch of gy, 2 = none             */
     GRANQ_KNOB_CLUSTER_KMUL = 15,         /* cluster plan: multiplier of a run's minimal channel count */
     GRANQ_KNOB_CLUSTER_EARLY_LAUNCH = 16, /* cluster plan: 2 = launch without programmatic dependent launch */
-    GRANQ_KNOB_COLWALK_TEAM = 17,         /* column-walk plan: 2 = L2 waves only (as any set L2 knob means)    */
+    GRANQ_KNOB_COLWALK_TEAM = 17,         /* column-walk plan: 1 = resident form wherever it fits, 2 = L2 waves
+                                             only (as any set L2 knob means, unless this one is 1)           */
     GRANQ_KNOB_TEST_COOP_CTAS = 18        /* test hook: the cooperative launches that have a plan to fall back on
                                              (channels-last, resident column walk) count as refused by the driver
                                              where they have more CTAs than this                             */

@@ -41,7 +41,7 @@ EXPORTS = [
     "granq_weights_workspace_bytes", "granq_fakequant_weights", "granq_packed_codes_bytes",
     "granq_quantize_packed", "granq_dequantize_packed", "granq_cluster_geometry", "granq_distortion_stats",
     "granq_accumulate_workspace_bytes", "granq_accumulate_codes", "granq_fakequant_fused_batch",
-    "granq_quantize_packed_fused", "granq_rows_geometry",
+    "granq_quantize_packed_fused", "granq_rows_geometry", "granq_team_geometry",
 ]
 NOALLOC_MAX_GROUPS = 32768
 
@@ -121,6 +121,8 @@ def lib() -> ctypes.CDLL:
         L.granq_accumulate_codes.argtypes = [vp, i64p, ci, ci, vp, vp, vp, ctypes.c_int64, vp, vp, sz, u32, vp]
         L.granq_cluster_geometry.restype = ci
         L.granq_cluster_geometry.argtypes = [ci, i64p, ci, ci, ci, i64p]
+        L.granq_team_geometry.restype = ci
+        L.granq_team_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, i64p]
         L.granq_rows_geometry.restype = ci
         L.granq_rows_geometry.argtypes = [ci, i64p, ci, ci, ci, i64p]
         L.granq_selftest_division.restype = ci
@@ -302,6 +304,18 @@ def cluster_geometry(dtype: int, shape, channel_axis: int = 1, group: int = GROU
     _check(rc, "granq_cluster_geometry")
     keys = ["grid", "threads", "cluster", "smem_bytes", "tile_bytes", "channels_per_run", "staging", "prefetch_gy"]
     return dict(zip(keys, [int(v) for v in out]))
+
+
+def team_geometry(dtype: int, shape, channel_axis: int = 1, group: int = GROUP_CHANNEL, with_backward: bool = True,
+                  sm_count: int = 148):
+    """Host-only: the cut of the column walk's resident form on a GPU with `sm_count` SMs and whether the column-walk
+    plan takes that form ("taken"), or None if the geometry does not qualify for it."""
+    out = (ctypes.c_int64 * 5)()
+    rc = lib().granq_team_geometry(dtype, _dims(shape), channel_axis, group, int(with_backward), sm_count, out)
+    if rc == ERR_UNSUPPORTED:
+        return None
+    _check(rc, "granq_team_geometry")
+    return dict(zip(["ctas", "teams", "units", "rounds", "taken"], [int(v) for v in out]))
 
 
 def rows_geometry(dtype: int, shape, channel_axis: int = 3, group: int = GROUP_CHANNEL, sm_count: int = 148):

@@ -114,7 +114,7 @@ TeamPlan prefer_team(int dtype, const Geom& g, const QuantIO& io, bool backward,
     TeamPlan none{};
     if (flags & GRANQ_FLAG_FORCE_CLUSTER) return none;
     const StagedTuning& t = g_tune;
-    if (t.cl_tile_kb || t.cl_r || t.cl_threads || t.cl_load || t.cl_prefetch || t.cl_kmul || t.cl_pdl || t.col_team) return none;
+    if (t.cl_tile_kb || t.cl_r || t.cl_threads || t.cl_load || t.cl_prefetch || t.cl_kmul || t.cl_pdl || t.col_team == 2) return none;
     const uint64_t bytes = (uint64_t)g.E * elt_size(dtype);
     const uint64_t from = (backward && dtype == GRANQ_F32 ? 128ull : 96ull) << 20;
     if (bytes < from || bytes / (uint64_t)g.C < (256ull << 10)) return none;
@@ -751,6 +751,18 @@ int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
     if (!plan_rows(dtype, g, io) || !cut_rows(dtype, g, 2u * (uint32_t)sm_count, cut)) return GRANQ_ERR_UNSUPPORTED;
     const int64_t v[4] = {cut.P, cut.slices, cut.lanes, cut.team};
     for (int i = 0; i < 4; ++i) out[i] = v[i];
+    return GRANQ_OK;
+}
+
+int granq_team_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward, int sm_count,
+                        int64_t out[5]) {
+    Geom g;
+    int64_t G;
+    if (!out || !dtype_ok(dtype) || sm_count < 1 || !make_geom(dims, channel_axis, group, g, G)) return GRANQ_ERR_INVALID_ARG;
+    const TeamPlan p = plan_colteam(dtype, g, QuantIO{}, with_backward != 0, sm_count);
+    if (!p.ok) return GRANQ_ERR_UNSUPPORTED;
+    const int64_t v[5] = {p.R, p.teams, p.tile_units, (g.C + p.teams - 1) / p.teams, team_over_waves(p, g, g_tune) ? 1 : 0};
+    for (int i = 0; i < 5; ++i) out[i] = v[i];
     return GRANQ_OK;
 }
 

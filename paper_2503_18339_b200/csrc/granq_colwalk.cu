@@ -566,8 +566,14 @@ ColPlan plan_colwalk(int dtype, const Geom& g, const QuantIO& io, const StagedTu
     return p;
 }
 
-static uint32_t team_rounds(int64_t channels, const TeamPlan& tp) {
-    return (uint32_t)((channels + tp.teams - 1) / tp.teams);
+// The resident form, unless a knob of the waves is set.  A hand-over costs a team as much as 2000 units: where the rounds
+// are several and shorter than that (small channels) the waves are faster (forward bf16 [12,2048,33,32], 7 rounds of 1584
+// units: 48 us, waves 43).
+bool team_over_waves(const TeamPlan& plan, const Geom& g, const StagedTuning& tune) {
+    if (!plan.ok || tune.col_team == 2) return false;
+    if (tune.col_team == 1) return true;
+    if (tune.l2_wave_kb > 0 || tune.l2_lag > 0 || tune.l2_ctas_per_sm > 0) return false;
+    return plan.tile_units >= 2500 || (g.C + plan.teams - 1) / plan.teams == 1;
 }
 
 cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
@@ -579,15 +585,10 @@ cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    // the resident form, unless a knob of the waves is set
-    if (tune.col_team != 2 && tune.l2_wave_kb <= 0 && tune.l2_lag <= 0 && tune.l2_ctas_per_sm <= 0) {
-        const TeamPlan tp = plan_colteam(dtype, g, io, mode == MODE_BOTH, sms);
-        // a hand-over costs a team as much as 2000 units: where the rounds are several and shorter than that (small
-        // channels) the waves are faster (forward bf16 [12,2048,33,32], 7 rounds of 1584 units: 48 us, waves 43)
-        if (tp.ok && (tp.tile_units >= 2500 || team_rounds(g.C, tp) == 1)) {
-            e = launch_colteam(tp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, tune, st);
-            if (e != cudaErrorCooperativeLaunchTooLarge) return e;      // else the waves, whose grid follows the occupancy
-        }
+    const TeamPlan tp = plan_colteam(dtype, g, io, mode == MODE_BOTH, sms);
+    if (team_over_waves(tp, g, tune)) {
+        e = launch_colteam(tp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, tune, st);
+        if (e != cudaErrorCooperativeLaunchTooLarge) return e;      // else the waves, whose grid follows the occupancy
     }
     CArgs a{};
     a.x = io.x;

@@ -147,7 +147,7 @@ struct StagedTuning {
     int cl_prefetch;      // cluster plan: 1 = ask the L2 for gy while x is loading, 2 = do not
     int cl_kmul;          // cluster plan: multiplier of the minimal channel count of a run
     int cl_pdl;           // cluster plan: 2 = no programmatic dependent launch
-    int col_team;         // column-walk plan: 2 = L2 waves only
+    int col_team;         // column-walk plan: 1 = resident form wherever it can, 2 = L2 waves only
     int coop_ctas;        // test hook: launch_cooperative() refuses more CTAs than this
 };
 // A cooperative launch that may be refused: every CTA has to be resident at once, and where the GPU is shared out (a
@@ -190,6 +190,8 @@ struct TeamPlan {
     uint32_t smem_bytes;     // dynamic shared memory per CTA
 };
 TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count);
+// does the column walk take this form rather than the waves?
+bool team_over_waves(const TeamPlan& plan, const Geom& g, const StagedTuning& tune);
 // may be refused: launch_cooperative()
 cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
                            const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,

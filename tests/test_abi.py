@@ -272,3 +272,38 @@ def test_rows_plan_cuts_within_what_the_gpu_holds(lib):
         assert geo["lanes"] >= 1 and geo["columns"] * geo["lanes"] <= top
         assert geo["team"] >= 1 and geo["team"] * geo["slices"] <= ctas
     assert refused
+
+
+def test_team_plan_cuts_within_its_limits_and_takes_over_where_it_should(lib):
+    """Host-only: a team's shares cover a channel and fit half an SM's shared memory, teams take every channel; the form
+    is taken with one round or long shares, the knob forces or forbids it, a knob of the waves keeps them."""
+    from paper_2503_18339_b200 import binding as b
+    rnd = random.Random(13)
+    seen = set()
+    try:
+        for _ in range(3000):
+            dt, bwd, sms = rnd.choice([0, 1]), rnd.choice([False, True]), rnd.choice([8, 132, 148])
+            shape = (rnd.choice([8, 13, 64, 128, 256]), rnd.randint(1, 1200), rnd.choice([1, 4, 8, 14, 28, 56, 112]), rnd.choice([4, 7, 8, 28, 56]))
+            for k in (b.KNOB_COLWALK_TEAM, b.KNOB_L2_WAVE_KB):
+                b.tune(k, 0)
+            geo = b.team_geometry(dt, shape, with_backward=bwd, sm_count=sms)
+            V, C = (4, 8)[dt], shape[1]
+            if geo is None:
+                continue
+            units = shape[0] * shape[2] * shape[3] // V
+            assert geo["ctas"] * geo["units"] >= units and geo["units"] <= 111 * 1024 // 16
+            assert geo["ctas"] * geo["teams"] <= 2 * sms and geo["teams"] <= C
+            assert geo["rounds"] == -(-C // geo["teams"])
+            rule = geo["units"] >= 2500 or geo["rounds"] == 1
+            assert geo["taken"] == rule
+            seen.add(rule)
+            b.tune(b.KNOB_L2_WAVE_KB, 64)
+            assert b.team_geometry(dt, shape, with_backward=bwd, sm_count=sms)["taken"] == 0
+            b.tune(b.KNOB_COLWALK_TEAM, 1)
+            assert b.team_geometry(dt, shape, with_backward=bwd, sm_count=sms)["taken"] == 1
+            b.tune(b.KNOB_COLWALK_TEAM, 2)
+            assert b.team_geometry(dt, shape, with_backward=bwd, sm_count=sms)["taken"] == 0
+        assert seen == {False, True}
+    finally:
+        for k in range(b.N_KNOBS):
+            b.tune(k, 0)

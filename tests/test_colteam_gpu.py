@@ -1,7 +1,7 @@
-"""The resident form of the column walk (a channel held in the shared memory of a team of CTAs) against the CPU
+"""The two forms of the column walk on aligned planes, mostly the resident one (a channel held in the shared memory of a team of CTAs) against the CPU
 oracle, bit for bit: teams of one CTA and of many, one round of channels and several, shares that are not whole
 runs of 8 units, planes shorter and longer than a block's stride, gy staged whole and in part - with every output
-that the form writes, between guard bands, the workspace zero again afterwards."""
+that the form writes, between guard bands, the workspace zero again afterwards; and the waves on the same shapes."""
 import numpy as np
 import pytest
 import torch
@@ -24,6 +24,7 @@ SHAPES = [
     (128, 16, 56, 56),   # shares beyond half the shared memory: gy staged in part
     (64, 300, 20, 20),   # two CTAs per channel and the next channel's copies on the heels of this one's
 ]
+SEVERAL_ROUNDS = [(8, 400, 8, 8), (13, 700, 2, 4), (33, 310, 4, 8), (64, 300, 20, 20)]
 
 
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
@@ -34,6 +35,10 @@ def test_resident_walk(b, knobs, shape, dtype):
     ref = orc.fused(x, bits, gy=gy)
     xd, gyd = to_dev(x), to_dev(gy)
     flags = b.FLAG_FORCE_COLWALK | b.FLAG_WORKSPACE_ZEROED
+    knobs(col_team=1)          # also where the waves are the faster form
+    for backward in (False, True):
+        form = b.team_geometry(b.BF16 if dtype == "bf16" else b.F32, shape, with_backward=backward)
+        assert form["taken"] == 1 and (form["rounds"] > 1) == (shape in SEVERAL_ROUNDS)
     ws = b.make_workspace(xd, zeroed=True)
     clean = lambda: b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
     for _ in range(2):
@@ -59,8 +64,42 @@ def test_resident_walk(b, knobs, shape, dtype):
     assert np.allclose(to_np(got.sums), sums, rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_waves_on_aligned_planes(b, knobs, shape, dtype):
+    """The form that the resident one stands in for, with its own cut of the waves: every output it writes."""
+    x, gy = make_case(shape, seed=sum(shape) + 1, dtype=dtype, relu=shape[0] % 2 == 1)
+    ref = orc.fused(x, 5, gy=gy)
+    xd, gyd = to_dev(x), to_dev(gy)
+    knobs(col_team=2)
+    assert b.team_geometry(b.BF16 if dtype == "bf16" else b.F32, shape)["taken"] == 0
+    flags = b.FLAG_FORCE_COLWALK | b.FLAG_WORKSPACE_ZEROED
+    ws = b.make_workspace(xd, zeroed=True)
+    new = lambda: b.FakeQuantOut(workspace=ws)
+    clean = lambda: b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
+    assert_parity(b.granq_fakequant_fused(xd, 5, gy=gyd, out=new(), want_params=True, flags=flags), ref, shape, 1,
+                  orc.GROUP_CHANNEL, backward=True)
+    assert clean()
+    assert_parity(b.granq_fakequant_fused(xd, 5, out=new(), flags=flags), ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert clean()
+    got = b.granq_fakequant_fused_stats(xd, 5, out=new(), flags=flags)
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    # fp32 inside a pack, fp64 beyond: about 8 roundings of 2^-24 of a sum of same-signed terms
+    assert clean() and np.allclose(to_np(got.sums), orc.distortion_sums(x, ref.y), rtol=1e-6, atol=0)
+    if (shape[1] * shape[2] * shape[3]) % 32 == 0:
+        got = b.granq_fakequant_fused_fwd_packmask(xd, 5, out=new(), flags=flags)
+        assert clean()
+        assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+        assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+        for bits in range(1, 9):
+            got = b.granq_quantize_packed_fused(xd, bits, out=new(), flags=flags)
+            assert clean()
+            assert_same_string(got.packed_codes, orc.pack_codes(orc.fused(x, bits).codes, bits))
+
+
 def test_a_hand_over_that_never_completes_is_reported(b, knobs):
     x, gy = make_case((8, 24, 12, 12), seed=1)
+    assert b.team_geometry(b.F32, x.shape)["taken"] == 1
     knobs(extra_arrivals=1, spin_limit=500)
     got = b.granq_fakequant_fused(to_dev(x), 4, gy=to_dev(gy), flags=b.FLAG_FORCE_COLWALK)
     assert b.workspace_status(got.workspace) == b.ERR_TIMEOUT
@@ -95,6 +134,7 @@ def test_a_reported_timeout_outlives_later_calls_on_the_same_zeroed_workspace(b,
     """A call on a workspace handed over as zero whose hand-over never completes leaves keys and counters behind;
     a cluster-local call on the same workspace clears none of them, so it must not clear the report either."""
     shape = (8, 24, 12, 12)
+    assert b.team_geometry(b.F32, shape)["taken"] == 1
     x, gy = make_case(shape, seed=2)
     xd, gyd = to_dev(x), to_dev(gy)
     ws = b.make_workspace(xd, zeroed=True)

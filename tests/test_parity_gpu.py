@@ -34,7 +34,8 @@ def knobs(b):
         names = {"depth": b.KNOB_STAGED_DEPTH, "max_buf_units": b.KNOB_STAGED_MAX_BUF_UNITS,
                  "grid": b.KNOB_STAGED_GRID, "spin_limit": b.KNOB_SPIN_LIMIT,
                  "extra_arrivals": b.KNOB_TEST_EXTRA_ARRIVALS, "l2_wave_kb": b.KNOB_L2_WAVE_KB,
-                 "l2_upl": b.KNOB_L2_UPL, "l2_ctas_per_sm": b.KNOB_L2_CTAS_PER_SM, "l2_lag": b.KNOB_L2_LAG}
+                 "l2_upl": b.KNOB_L2_UPL, "l2_ctas_per_sm": b.KNOB_L2_CTAS_PER_SM, "l2_lag": b.KNOB_L2_LAG,
+                 "col_team": b.KNOB_COLWALK_TEAM}
         for k, v in kw.items():
             b.tune(names[k], v)
     yield set_
@@ -304,7 +305,7 @@ def test_colwalk_workspace_stays_zeroed(b, knobs):
 def test_colwalk_bounded_wait_reports_timeout(b, knobs):
     shape = (8, 16, 14, 14)
     x, gy = make_case(shape, seed=2)
-    knobs(extra_arrivals=1, spin_limit=2000)
+    knobs(extra_arrivals=1, spin_limit=2000, col_team=2)          # the waves
     got = b.granq_fakequant_fused(to_dev(x), 4, gy=to_dev(gy), flags=b.FLAG_FORCE_COLWALK)
     assert b.workspace_status(got.workspace) == b.ERR_TIMEOUT
     knobs(extra_arrivals=0, spin_limit=0)

@@ -1,5 +1,5 @@
 """Channels-last tensors ([N, H, W, C], channel_axis = 3) and planes of one element ([N, C, 1, 1]) through the
-plan made for them (a range launch and a quantize launch, one 16-byte unit column per thread) against the CPU
+plan made for them (one cooperative launch, one 16-byte unit column per thread) against the CPU
 oracle: small and adversarial shapes, and two tensors of the benchmark's activation sets transposed to
 channels-last at full size; every output between guard bands."""
 import numpy as np
