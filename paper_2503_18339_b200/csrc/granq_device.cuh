@@ -314,6 +314,24 @@ __device__ __forceinline__ GroupParam group_param_from_keys(const uint32_t* kmin
     return group_param_from_range(lo, hi, qmax);
 }
 
+template <int H>
+struct PartAt {
+    static constexpr int value = H;
+};
+
+// Clamp the rounded values m[H .. H + W) = 1.5 * 2^23 + r to codes.  The bits of `in` of elements that were beyond: taken
+// out (where a clamp is the exception, `in` starts full), or the others put in (where it is the rule, from none).
+template <int H, int W, bool RULE, int V>
+__device__ __forceinline__ void clamp_codes(float (&m)[V], float top, uint32_t& in) {
+#pragma unroll
+    for (int i = H; i < H + W; ++i) {
+        const float c = fminf(fmaxf(m[i], kRoundMagic), top);
+        if (RULE) in |= (m[i] == c) ? (1u << i) : 0u;
+        else in &= (m[i] == c) ? 0xFFFFFFFFu : ~(1u << i);
+        m[i] = c;
+    }
+}
+
 // What the extra outputs of one pack are made of (EXTRAS as in quantize_pack): bytes of codes and mask (1), mask
 // bits (2), strings of code_bits per code (3).  m: 1.5 * 2^23 + code of element i, in: the clamp was inactive.
 template <int V, int EXTRAS>
@@ -348,62 +366,80 @@ __device__ __forceinline__ void pack_extras(const float (&m)[V], uint32_t in, ui
 // (bit i: the clamp was inactive for element i), which is all the packed mask needs; EXTRAS = 3 returns
 // only the codes, code_bits each (cb[h] = the four codes of half h as a string of 4 * code_bits bits; bytes for
 // the default of 8), taken from the low mantissa bits of code + 1.5 * 2^23 instead of a float-to-integer
-// conversion (packed-code output); EXTRAS = 4 returns neither (the caller adds up the distortion).  SELF: the range is that of the tensor itself and thr comes from
-// group_param_from_range(), so where it is positive nothing is clamped and the gradient passes whole; without SELF
-// it comes from tie_threshold() alone and x may lie anywhere.  A NaN element fails the tie test and takes the clamp:
-// code 0 and no gradient, as in the sequence as defined, whatever its neighbours are.
+// conversion (packed-code output); EXTRAS = 4 returns neither (the caller adds up the distortion).  SELF: the range is
+// that of the tensor itself and thr comes from group_param_from_range(), so where it is positive nothing is clamped and the
+// gradient passes whole; without SELF it comes from tie_threshold() alone and x may lie anywhere.  A NaN element takes the
+// clamp - without SELF it always does, with it the tie test fails - and becomes code 0 without a gradient, as in the
+// sequence as defined, whatever its neighbours are.  PARTS: see W.
 // Instructions per element, bf16 or fp32 alike: two multiply-adds, one add, half a three-way maximum and one
 // product (SELF), where rounding by add and subtract, clamp, compare and select took eleven.  Measured against that
 // form: forward-only bf16 [256,512,28,28] at 8 bits 127.6 -> 119.6 us (issue slots bind where an element is two
 // bytes), packed codes of fp32 [128,144,56,56] 150 -> 142 us, packed mask of [128,64,56,56] 63.0 -> 60.6 us.
-template <typename T, bool BWD, bool SPLIT, int EXTRAS, bool SELF = false>
+template <typename T, bool BWD, bool SPLIT, int EXTRAS, bool SELF = false, bool PARTS = true>
 __device__ __forceinline__ void quantize_pack(const Pack<T>& px, const Pack<T>& pg, const GroupParam& g1,
                                               const GroupParam& g2, int n1, float qmax, Pack<T>& py, Pack<T>& pgx,
                                               uint32_t (&cb)[Pack<T>::V / 4], uint32_t (&mb)[Pack<T>::V / 4],
                                               int code_bits = 8) {
     constexpr int V = Pack<T>::V;
-    constexpr uint32_t kAll = (1u << V) - 1u;
+    // Elements worked on together.  Eight at a time, with the two sets of parameters of a pack that straddles groups or
+    // with the clamp in the main line, take 74 to 99 registers in kernels that want 64: bf16 then takes four at a time.
+    constexpr int W = (V == 8 && PARTS && (SPLIT || !SELF)) ? 4 : V;
+    // ... and the elements that miss the shortcut share their branch with the groups that have none
+    constexpr bool kOneBranch = !SELF && W < V;
     float m[V], yv[V];
-    uint32_t in = kAll;                                         // bit i: the clamp was inactive for element i
+    uint32_t in = SELF ? (1u << V) - 1u : 0u;                   // bit i: the clamp was inactive for element i
     const float thr = SPLIT ? fminf(fabsf(g1.thr), fabsf(g2.thr)) : fabsf(g1.thr);
     const float top = __fadd_rn(kRoundMagic, qmax);
-    if (thr > 0.0f) {
+    if (kOneBranch || thr > 0.0f) {
         const float mz1 = __fadd_rn(kRoundMagic, g1.z), mz2 = SPLIT ? __fadd_rn(kRoundMagic, g2.z) : mz1;
-        float worst = 0.0f;
+        auto part = [&](auto at) {
+            constexpr int H = decltype(at)::value;
+            float worst = 0.0f;
 #pragma unroll
-        for (int i = 0; i < V; ++i) {
-            const bool first = !SPLIT || i < n1;
-            const float rc = first ? g1.r : g2.r, mz = first ? mz1 : mz2;
-            const float x = px.get(i);
-            m[i] = __fmaf_rn(x, rc, mz);
-            worst = max_or_nan(worst, fabsf(__fmaf_rn(x, rc, __fsub_rn(mz, m[i]))));
-        }
-        bool clamp = !SELF || g1.thr < 0.0f || (SPLIT && g2.thr < 0.0f);
-        if (!(worst < thr)) {                                   // rare: too close to a tie for the shortcut, or NaN
-            clamp = clamp || worst != worst;                    // which the clamp turns into code 0 without a gradient
-#pragma unroll
-            for (int i = 0; i < V; ++i) {
+            for (int i = H; i < H + W; ++i) {
                 const bool first = !SPLIT || i < n1;
-                const float s = first ? g1.s : g2.s, z = first ? g1.z : g2.z, rc = first ? g1.r : g2.r;
-                const float mz = first ? mz1 : mz2, x = px.get(i);
-                if (!(fabsf(__fmaf_rn(x, rc, __fsub_rn(mz, m[i]))) < thr))
-                    m[i] = exact_round_magic(SELF ? div_by_scale(x, s, rc) : __fdiv_rn(x, s), z, qmax);
+                const float rc = first ? g1.r : g2.r, mz = first ? mz1 : mz2;
+                const float x = px.get(i);
+                m[i] = __fmaf_rn(x, rc, mz);
+                const float d = fabsf(__fmaf_rn(x, rc, __fsub_rn(mz, m[i])));
+                worst = SELF ? max_or_nan(worst, d) : fmaxf(worst, d);
             }
-        }
-        if (clamp) {
-            in = 0;
+            bool clamp = !SELF || g1.thr < 0.0f || (SPLIT && g2.thr < 0.0f);
+            if (!(worst < thr)) {                               // rare: too close to a tie for the shortcut, or NaN
 #pragma unroll
-            for (int i = 0; i < V; ++i) {
-                const float c = fminf(fmaxf(m[i], kRoundMagic), top);
-                in |= (m[i] == c) ? (1u << i) : 0u;
-                m[i] = c;
+                for (int i = H; i < H + W; ++i) {
+                    const bool first = !SPLIT || i < n1;
+                    const float s = first ? g1.s : g2.s, z = first ? g1.z : g2.z, rc = first ? g1.r : g2.r;
+                    const float mz = first ? mz1 : mz2, x = px.get(i);
+                    if (!(fabsf(__fmaf_rn(x, rc, __fsub_rn(mz, m[i]))) < thr))
+                        m[i] = exact_round_magic(SELF ? div_by_scale(x, s, rc) : __fdiv_rn(x, s), z, qmax);
+                }
+                // NaN: in a place of its own, so that the condition below stays one that the walk around this need not look
+                // at again ([256,960,7,7] fp32 with a gradient 50.9 -> 47.0 us); beside byte codes it is the other way
+                // round (54.9 / 61.2)
+                if constexpr (SELF && W == V && EXTRAS != 1) {
+                    if (worst != worst) clamp_codes<H, W, !SELF>(m, top, in);
+                } else if constexpr (SELF) {
+                    clamp = clamp || worst != worst;
+                }
             }
-        }
+            if (clamp) clamp_codes<H, W, !SELF>(m, top, in);
+            if (!kOneBranch || thr > 0.0f) {
 #pragma unroll
-        for (int i = 0; i < V; ++i) {
-            const bool first = !SPLIT || i < n1;
-            yv[i] = __fmul_rn(first ? g1.s : g2.s, __fsub_rn(m[i], first ? mz1 : mz2));
-        }
+                for (int i = H; i < H + W; ++i) {
+                    const bool first = !SPLIT || i < n1;
+                    yv[i] = __fmul_rn(first ? g1.s : g2.s, __fsub_rn(m[i], first ? mz1 : mz2));
+                }
+            } else {                                            // the zero-point may be too large for mz
+#pragma unroll
+                for (int i = H; i < H + W; ++i) {
+                    const bool first = !SPLIT || i < n1;
+                    yv[i] = __fmul_rn(first ? g1.s : g2.s, __fsub_rn(__fsub_rn(m[i], kRoundMagic), first ? g1.z : g2.z));
+                }
+            }
+        };
+        part(PartAt<0>{});
+        if constexpr (W < V) part(PartAt<W>{});
     } else {                                                    // the sequence as defined, element by element
         in = 0;
 #pragma unroll
@@ -453,15 +489,7 @@ __device__ __forceinline__ void quantize_pack_each(const Pack<T>& px, const Pack
                     m[i] = exact_round_magic(div_by_scale(x, s[i], r[i]), __fsub_rn(mz[i], kRoundMagic), qmax);
             }
         }
-        if (clamp) {
-            in = 0;
-#pragma unroll
-            for (int i = 0; i < V; ++i) {
-                const float c = fminf(fmaxf(m[i], kRoundMagic), top);
-                in |= (m[i] == c) ? (1u << i) : 0u;
-                m[i] = c;
-            }
-        }
+        if (clamp) clamp_codes<0, V, false>(m, top, in);
 #pragma unroll
         for (int i = 0; i < V; ++i) yv[i] = __fmul_rn(s[i], __fsub_rn(m[i], mz[i]));
     } else {                                                    // the sequence as defined, element by element

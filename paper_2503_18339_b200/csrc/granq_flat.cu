@@ -108,7 +108,7 @@ __device__ __forceinline__ void finish_range(const RangeEnd& e) {
 // ---- Eq. 4: range ------------------------------------------------------------------------------
 // V = elements per load: a 16-byte pack when planes and pointers allow it, else 1.
 template <typename T, int V>
-__global__ void __launch_bounds__(kThreads) range_flat_kernel(const T* __restrict__ x, FlatGeom g,
+__global__ void __launch_bounds__(kThreads, 8) range_flat_kernel(const T* __restrict__ x, FlatGeom g,
                                                               uint32_t* __restrict__ kmin,
                                                               uint32_t* __restrict__ kmax, RangeEnd end) {
     __shared__ TileBase s_base;
@@ -426,6 +426,16 @@ __device__ __forceinline__ void warp_pack_row(uint64_t mine, uint32_t nb, uint32
     }
 }
 
+// bf16 where a pack straddles planes, and wherever there is a gradient: four elements of a pack at a time, compiled for
+// four blocks per SM; eight at a time take 73 to 99 registers, which costs one or two of them.  Backward [256,512,28,28]
+// 147 -> 118 us, range and both directions there 207 -> 188; on ragged planes [256,1024,14,14] forward 82 -> 66, backward
+// 92 -> 70, range and both 147 -> 129.  Forward on whole packs is faster the other way (138 / 144).
+template <int V, int MODE, int EXTRAS, bool RAGGED>
+constexpr bool kFlatParts = V == 8 && (MODE == MODE_BOTH ? EXTRAS == 0 : RAGGED || MODE == MODE_BWD);
+// blocks per SM the kernel is compiled for; 0: left to the compiler
+template <int V, int MODE, int EXTRAS, bool PACKONLY, bool RAGGED>
+constexpr int kFlatBlocks = !kFlatParts<V, MODE, EXTRAS, RAGGED> ? 0 : MODE == MODE_FWD && EXTRAS == 1 ? (PACKONLY ? 3 : 0) : 4;
+
 // ---- Eq. 1, clamp, Eq. 6, STE: elementwise pass with a given per-group range ----------------------
 // EXTRAS = 1: the optional codes / mask / packed-mask / sums outputs are compiled in; 2: the packed mask alone; 4: the
 // distortion sums alone.  The packed mask holds
@@ -437,7 +447,8 @@ __device__ __forceinline__ void warp_pack_row(uint64_t mine, uint32_t nb, uint32
 // RAGGED: planes are not whole 16-byte packs (7x7 planes), so a pack may straddle two planes and takes the
 // parameters of both (planes of at least one pack: never more than two).
 template <typename T, int V, int MODE, int EXTRAS, bool PACKONLY = false, bool RAGGED = false>
-__global__ void __launch_bounds__(kThreads) quant_flat_kernel(const T* __restrict__ x, const T* __restrict__ gy,
+__global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKONLY, RAGGED>))
+                                            quant_flat_kernel(const T* __restrict__ x, const T* __restrict__ gy,
                                                               T* __restrict__ y, T* __restrict__ gx,
                                                               uint8_t* __restrict__ codes,
                                                               uint8_t* __restrict__ mask,
@@ -449,6 +460,7 @@ __global__ void __launch_bounds__(kThreads) quant_flat_kernel(const T* __restric
                                                               const float* __restrict__ hi) {
     __shared__ TileBase s_base;
     __shared__ float s_tab_s[kTableMax], s_tab_z[kTableMax], s_tab_r[kTableMax];
+    constexpr bool kParts = kFlatParts<V, MODE, EXTRAS, RAGGED>;
     constexpr bool kFwd = (MODE & MODE_FWD) != 0, kBwd = (MODE & MODE_BWD) != 0;
     DistAcc dacc;
     dacc.reset();
@@ -548,7 +560,7 @@ __global__ void __launch_bounds__(kThreads) quant_flat_kernel(const T* __restric
                             }
                         }
                     }
-                    quantize_pack<T, kBwd, RAGGED, EXTRAS>(px[j], pg[j], gp, gp2, n1, qmax, py, pgx, cb, mb, EXTRAS == 3 ? code_bits : 8);
+                    quantize_pack<T, kBwd, RAGGED, EXTRAS, false, kParts>(px[j], pg[j], gp, gp2, n1, qmax, py, pgx, cb, mb, EXTRAS == 3 ? code_bits : 8);
                     if constexpr (EXTRAS == 3) {
                         code_string = code_string_of<V>(cb, code_bits);
                     } else if constexpr (EXTRAS != 0) {
