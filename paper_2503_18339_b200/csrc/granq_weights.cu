@@ -25,7 +25,8 @@ namespace {
 
 constexpr int kWThreads = 256;
 constexpr uint32_t kWWarps = kWThreads / 32;
-constexpr uint32_t kWHold = 5;          // units (or elements) of a group one lane holds
+constexpr int kWHold = 5;               // units (or elements) of a group one lane holds at most
+constexpr int kWTail = 4;               // units in flight per lane where a group is more than its team holds
 
 struct WDesc {
     const void* x;
@@ -49,8 +50,9 @@ struct WTable {
     WDesc d[N];
 };
 
-template <typename T, bool GRAD, int N>
-__global__ void __launch_bounds__(kWThreads, GRAD ? 3 : 4) weights_kernel(const __grid_constant__ WTable<N> tab, uint32_t n) {
+// HOLD = units (or elements) of a group one lane holds
+template <typename T, bool GRAD, int N, int HOLD>
+__global__ void __launch_bounds__(kWThreads, HOLD == 1 ? (GRAD ? 5 : 6) : GRAD ? 3 : 4) weights_kernel(const __grid_constant__ WTable<N> tab, uint32_t n) {
     constexpr int V = Pack<T>::V;
     __shared__ float s_mn[kWWarps], s_mx[kWWarps];
     // the tensor of this block: last descriptor with first_block <= blockIdx.x
@@ -72,38 +74,43 @@ __global__ void __launch_bounds__(kWThreads, GRAD ? 3 : 4) weights_kernel(const 
     T* gx = reinterpret_cast<T*>(d.gx) + at;
     const bool grad = GRAD && d.gy != nullptr;
     const uint32_t units = valid ? (d.vec ? ge / V : ge) : 0;
-    const uint32_t held = kWHold * stride;
+    const uint32_t held = HOLD * stride;          // with one unit a lane: the whole group
 
     // ---- Eq. 4: the group's range; the group stays in registers ----
-    Pack<T> px[kWHold], pg[GRAD ? kWHold : 1];
-    float sx[kWHold], sg[GRAD ? kWHold : 1];
+    Pack<T> px[HOLD], pg[GRAD ? HOLD : 1];
+    float sx[HOLD], sg[GRAD ? HOLD : 1];
     float mn = INFINITY, mx = -INFINITY;
     if (d.vec) {
 #pragma unroll
-        for (int j = 0; j < (int)kWHold; ++j) {
+        for (int j = 0; j < HOLD; ++j) {
             const uint32_t u = tl + j * stride;
             if (u < units) px[j].raw = ld_stream_16(x + (size_t)u * V);
         }
         if constexpr (GRAD) {
             if (grad) {
 #pragma unroll
-                for (int j = 0; j < (int)kWHold; ++j) {
+                for (int j = 0; j < HOLD; ++j) {
                     const uint32_t u = tl + j * stride;
                     if (u < units) pg[j].raw = ld_stream_16(gy + (size_t)u * V);
                 }
             }
         }
 #pragma unroll
-        for (int j = 0; j < (int)kWHold; ++j)
+        for (int j = 0; j < HOLD; ++j)
             if (tl + j * stride < units) pack_minmax(px[j], 0, V, mn, mx);
-        for (uint32_t u = held + tl; u < units; u += stride) {
-            Pack<T> p;
-            p.raw = *reinterpret_cast<const uint4*>(x + (size_t)u * V);
-            pack_minmax(p, 0, V, mn, mx);
-        }
+        if constexpr (HOLD > 1)
+            for (uint32_t u = held + tl; u < units; u += kWTail * stride) {
+                Pack<T> p[kWTail];
+#pragma unroll
+                for (int j = 0; j < kWTail; ++j)
+                    if (u + j * stride < units) p[j].raw = *reinterpret_cast<const uint4*>(x + (size_t)(u + j * stride) * V);
+#pragma unroll
+                for (int j = 0; j < kWTail; ++j)
+                    if (u + j * stride < units) pack_minmax(p[j], 0, V, mn, mx);
+            }
     } else {
 #pragma unroll
-        for (int j = 0; j < (int)kWHold; ++j) {
+        for (int j = 0; j < HOLD; ++j) {
             const uint32_t e = tl + j * stride;
             if (e < units) {
                 sx[j] = load_scalar(x + e);
@@ -113,16 +120,17 @@ __global__ void __launch_bounds__(kWThreads, GRAD ? 3 : 4) weights_kernel(const 
             }
         }
 #pragma unroll
-        for (int j = 0; j < (int)kWHold; ++j)
+        for (int j = 0; j < HOLD; ++j)
             if (tl + j * stride < units) {
                 mn = fminf(mn, sx[j]);
                 mx = fmaxf(mx, sx[j]);
             }
-        for (uint32_t e = held + tl; e < units; e += stride) {
-            const float v = load_scalar(x + e);
-            mn = fminf(mn, v);
-            mx = fmaxf(mx, v);
-        }
+        if constexpr (HOLD > 1)
+            for (uint32_t e = held + tl; e < units; e += stride) {
+                const float v = load_scalar(x + e);
+                mn = fminf(mn, v);
+                mx = fmaxf(mx, v);
+            }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -163,18 +171,25 @@ __global__ void __launch_bounds__(kWThreads, GRAD ? 3 : 4) weights_kernel(const 
             }
         };
 #pragma unroll
-        for (int j = 0; j < (int)kWHold; ++j) {
+        for (int j = 0; j < HOLD; ++j) {
             const uint32_t u = tl + j * stride;
             if (u < units) emit(px[j], pg[GRAD ? j : 0], u);
         }
-        for (uint32_t u = held + tl; u < units; u += stride) {
-            Pack<T> p, g;
-            p.raw = *reinterpret_cast<const uint4*>(x + (size_t)u * V);
-            if constexpr (GRAD) {
-                if (grad) g.raw = *reinterpret_cast<const uint4*>(gy + (size_t)u * V);
+        if constexpr (HOLD > 1)
+            for (uint32_t u = held + tl; u < units; u += 2 * stride) {
+                const bool two = u + stride < units;
+                Pack<T> p[2], g[2];
+                p[0].raw = *reinterpret_cast<const uint4*>(x + (size_t)u * V);
+                if (two) p[1].raw = *reinterpret_cast<const uint4*>(x + (size_t)(u + stride) * V);
+                if constexpr (GRAD) {
+                    if (grad) {
+                        g[0].raw = *reinterpret_cast<const uint4*>(gy + (size_t)u * V);
+                        if (two) g[1].raw = *reinterpret_cast<const uint4*>(gy + (size_t)(u + stride) * V);
+                    }
+                }
+                emit(p[0], g[0], u);
+                if (two) emit(p[1], g[1], u + stride);
             }
-            emit(p, g, u);
-        }
     } else {
         const QParam qp{gp.s, gp.z};
         auto emit = [&](float v, float g, uint32_t e) {
@@ -187,22 +202,31 @@ __global__ void __launch_bounds__(kWThreads, GRAD ? 3 : 4) weights_kernel(const 
             }
         };
 #pragma unroll
-        for (int j = 0; j < (int)kWHold; ++j) {
+        for (int j = 0; j < HOLD; ++j) {
             const uint32_t e = tl + j * stride;
             if (e < units) emit(sx[j], sg[GRAD ? j : 0], e);
         }
-        for (uint32_t e = held + tl; e < units; e += stride)
-            emit(load_scalar(x + e), grad ? load_scalar(gy + e) : 0.0f, e);
+        if constexpr (HOLD > 1)
+            for (uint32_t e = held + tl; e < units; e += stride)
+                emit(load_scalar(x + e), grad ? load_scalar(gy + e) : 0.0f, e);
     }
 }
 
 constexpr int kWSmallTable = 32, kWTable = 256;      // descriptors of one launch (2.9 KB / 23 KB of parameters)
 
+// Launches whose groups are at most a warp's lanes (depthwise kernels, small first layers) hold one unit per lane: fewer
+// registers and twice the blocks per SM, which is all such groups are bound by.
 template <typename T, bool GRAD, int N>
 cudaError_t w_launch_n(const WDesc* descs, int n, uint32_t blocks, cudaStream_t st) {
+    constexpr uint32_t V = Pack<T>::V;
     WTable<N> tab;
-    for (int i = 0; i < n; ++i) tab.d[i] = descs[i];
-    weights_kernel<T, GRAD, N><<<blocks, kWThreads, 0, st>>>(tab, (uint32_t)n);
+    bool small = true;
+    for (int i = 0; i < n; ++i) {
+        tab.d[i] = descs[i];
+        small = small && (descs[i].vec ? descs[i].group_elems / V : descs[i].group_elems) <= 32;
+    }
+    if (small) weights_kernel<T, GRAD, N, 1><<<blocks, kWThreads, 0, st>>>(tab, (uint32_t)n);
+    else weights_kernel<T, GRAD, N, kWHold><<<blocks, kWThreads, 0, st>>>(tab, (uint32_t)n);
     return cudaGetLastError();
 }
 
