@@ -458,7 +458,8 @@ int granq_team_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
  * Returns GRANQ_ERR_UNSUPPORTED when the geometry does not qualify or the device holds fewer CTAs at once than
  * there would be slices (a call then takes two passes).
  */
-int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int sm_count, int64_t out[4]);
+int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward, int sm_count,
+                        int64_t out[4]);
 
 /*
  * Device self-test (no counterpart in the paper).  The staged kernel divides by the

@@ -124,7 +124,7 @@ def lib() -> ctypes.CDLL:
         L.granq_team_geometry.restype = ci
         L.granq_team_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, i64p]
         L.granq_rows_geometry.restype = ci
-        L.granq_rows_geometry.argtypes = [ci, i64p, ci, ci, ci, i64p]
+        L.granq_rows_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, i64p]
         L.granq_selftest_division.restype = ci
         L.granq_selftest_division.argtypes = [ctypes.c_uint64, ctypes.c_uint64, vp, vp]
         L.granq_range_noalloc.restype = ci
@@ -318,10 +318,11 @@ def team_geometry(dtype: int, shape, channel_axis: int = 1, group: int = GROUP_C
     return dict(zip(["ctas", "teams", "units", "rounds", "taken"], [int(v) for v in out]))
 
 
-def rows_geometry(dtype: int, shape, channel_axis: int = 3, group: int = GROUP_CHANNEL, sm_count: int = 148):
+def rows_geometry(dtype: int, shape, channel_axis: int = 3, group: int = GROUP_CHANNEL, with_backward: bool = True,
+                  sm_count: int = 148):
     """Host-only: the cut of the channels-last plan on a GPU with `sm_count` SMs, or None where it has none."""
     out = (ctypes.c_int64 * 4)()
-    rc = lib().granq_rows_geometry(dtype, _dims(shape), channel_axis, group, sm_count, out)
+    rc = lib().granq_rows_geometry(dtype, _dims(shape), channel_axis, group, int(with_backward), sm_count, out)
     if rc == ERR_UNSUPPORTED:
         return None
     _check(rc, "granq_rows_geometry")

@@ -742,13 +742,14 @@ int granq_cluster_geometry(int dtype, const int64_t dims[4], int channel_axis, i
     return GRANQ_OK;
 }
 
-int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int sm_count, int64_t out[4]) {
+int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward, int sm_count,
+                        int64_t out[4]) {
     Geom g;
     int64_t G;
     if (!out || !dtype_ok(dtype) || sm_count < 1 || !make_geom(dims, channel_axis, group, g, G)) return GRANQ_ERR_INVALID_ARG;
     const QuantIO io{};
     RowsCut cut{};
-    if (!plan_rows(dtype, g, io) || !cut_rows(dtype, g, 2u * (uint32_t)sm_count, cut)) return GRANQ_ERR_UNSUPPORTED;
+    if (!plan_rows(dtype, g, io) || !cut_rows(dtype, g, with_backward != 0, 2u * (uint32_t)sm_count, cut)) return GRANQ_ERR_UNSUPPORTED;
     const int64_t v[4] = {cut.P, cut.slices, cut.lanes, cut.team};
     for (int i = 0; i < 4; ++i) out[i] = v[i];
     return GRANQ_OK;

@@ -215,7 +215,7 @@ struct RowsCut {
     uint32_t team;           // CTAs per slice
 };
 // false where the GPU holds too few CTAs at once for any cut (ctas: how many)
-bool cut_rows(int dtype, const Geom& g, uint32_t ctas, RowsCut& cut);
+bool cut_rows(int dtype, const Geom& g, bool backward, uint32_t ctas, RowsCut& cut);
 // may be refused: launch_cooperative()
 cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, int bits, const Workspace& ws,
                         float* lo, float* hi, float* s_opt, float* z_opt, const StagedTuning& tune, cudaStream_t st);

@@ -302,14 +302,27 @@ bool plan_rows(int dtype, const Geom& g, const QuantIO& io) {
 
 // The cut of a row into slices that leaves the fewest threads and CTAs without work (196 unit columns: 7 slices of 28,
 // 16 rows of threads each); slices of 64 unit columns at most, of 16 at least where there are several.
-bool cut_rows(int dtype, const Geom& g, uint32_t ctas, RowsCut& cut) {
+// Where a slice ends inside a 32-byte sector or a 128-byte line, two CTAs write the two parts of it at different times.
+// A tensor that stays on chip is small enough for the L2 to join the sectors up; of a larger one they go to memory in
+// pieces, so its slices are whole lines.  fp32 with a gradient (us): [40,100,100,200] two slices of 25 columns 315, of 26
+// 279, one slice of 50 257; [64,56,56,264] 33 columns 192, 24 columns 181; [20,56,56,784] 49 columns 183, 40 columns 169;
+// bf16 [40,100,100,400] 324, one slice 297.  On chip: [8,30,30,520] 26 columns 21.0, 48 columns 21.6; bf16 [16,28,28,408]
+// 17 columns 21.7, one slice of 51 23.0.
+// Threads: all that fit, 448 or 384; with an fp32 gradient beyond 200 MB 400, which is what loads in flight of two
+// streams take there ([128,112,112,64] 334 / 327 us, [128,112,112,96] 503 / 491, [64,112,112,128] 333 / 326; 320 threads
+// 325, 522, 325; but [128,28,28,192], 77 MB, 63.6 / 64.8).
+bool cut_rows(int dtype, const Geom& g, bool backward, uint32_t ctas, RowsCut& cut) {
     const uint32_t V = dtype == 0 ? 4 : 8, ncol = (uint32_t)(g.C / V);
-    const uint32_t top = dtype == 0 ? kRMaxThreads<float> : kRMaxThreads<__nv_bfloat16>;
+    const uint64_t bytes = (uint64_t)g.outer * ncol * 16;
+    const uint32_t most = dtype == 0 ? kRMaxThreads<float> : kRMaxThreads<__nv_bfloat16>;
+    const uint32_t top = dtype == 0 && backward && bytes > (200ull << 20) ? 400 : most;
+    const uint32_t whole = bytes > (uint64_t)ctas * kRSmemBytes ? 8 : ncol % 2 == 0 ? 2 : 1;      // unit columns
     double best = 0.0;
     for (uint32_t slices = (ncol + 63) / 64; slices <= std::max<uint32_t>(1, ncol / 16); ++slices) {
-        const uint32_t P = (ncol + slices - 1) / slices, lanes = top / P, used = (ncol + P - 1) / P;
+        const uint32_t share = (ncol + slices - 1) / slices, P = slices > 1 ? (share + whole - 1) / whole * whole : share;
+        const uint32_t lanes = top / P, used = (ncol + P - 1) / P;
         const double eff = (double)ncol / (double)(used * P) * (double)(P * lanes) / top * (double)(ctas / used * used) / ctas;
-        if (eff > best + 0.02) {
+        if (eff > best + (whole == 8 ? 0.05 : 0.02)) {
             best = eff;
             cut.P = P;
             cut.slices = used;
@@ -350,7 +363,7 @@ cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, i
     a.ncol = (uint32_t)(g.C / V);
     a.rows = (uint64_t)g.outer;
     RowsCut cut{};
-    if (!cut_rows(dtype, g, 2u * (uint32_t)sms, cut)) return cudaErrorCooperativeLaunchTooLarge;
+    if (!cut_rows(dtype, g, mode != MODE_FWD, 2u * (uint32_t)sms, cut)) return cudaErrorCooperativeLaunchTooLarge;
     a.P = cut.P;
     a.slices = cut.slices;
     a.lanes = cut.lanes;

@@ -261,8 +261,8 @@ def test_rows_plan_cuts_within_what_the_gpu_holds(lib):
         dt, sms = rnd.choice([0, 1]), rnd.choice([1, 2, 3, 4, 8, 16, 66, 132, 148])
         V, top = (4, 448) if dt == 0 else (8, 384)
         C = V * rnd.randint(1, 4096 // V)
-        rows = rnd.choice([1, 7, 128, 40_000])
-        geo = b.rows_geometry(dt, (rows, rnd.choice([1, 3]), 2, C), sm_count=sms)
+        shape = (rnd.choice([1, 7, 128, 40_000]), rnd.choice([1, 3]), 2, C)
+        geo = b.rows_geometry(dt, shape, with_backward=rnd.choice([False, True]), sm_count=sms)
         ncol, ctas = C // V, 2 * sms
         if geo is None:
             refused += 1
@@ -271,6 +271,9 @@ def test_rows_plan_cuts_within_what_the_gpu_holds(lib):
         assert 1 <= geo["columns"] <= 64 and geo["columns"] * geo["slices"] >= ncol > geo["columns"] * (geo["slices"] - 1)
         assert geo["lanes"] >= 1 and geo["columns"] * geo["lanes"] <= top
         assert geo["team"] >= 1 and geo["team"] * geo["slices"] <= ctas
+        if geo["slices"] > 1:                    # no slice ends inside a line, or, of a tensor that stays on chip, a sector
+            beyond = shape[0] * shape[1] * 2 * ncol * 16 > ctas * 111 * 1024
+            assert geo["columns"] % (8 if beyond else 2 if ncol % 2 == 0 else 1) == 0
     assert refused
 
 

@@ -143,3 +143,15 @@ def test_channels_last_where_the_cooperative_launch_is_refused(b, dtype):
                 ws.zero_()
     finally:
         b.tune(b.KNOB_TEST_COOP_CTAS, 0)
+
+
+@pytest.mark.parametrize("dtype,shape", [("f32", (36, 30, 30, 264)), ("bf16", (36, 30, 30, 520)), ("f32", (20, 45, 47, 204)),
+                                         ("f32", (120, 112, 112, 36))], ids=str)
+def test_channels_last_beyond_what_the_chip_holds(b, dtype, shape):
+    """Read twice, in slices of whole lines (a last one that is narrower, one slice of an odd number of columns); the
+    last shape is large enough for the smaller blocks of threads."""
+    x, gy = nhwc_case(shape, seed=sum(shape), dtype=dtype)
+    geo = b.rows_geometry(b.BF16 if dtype == "bf16" else b.F32, shape)
+    assert x.nbytes > 296 * 111 * 1024 and (geo["slices"] == 1 or geo["columns"] % 8 == 0)
+    run(b, x, gy, 4, 3)
+    run(b, x, None, 7, 3)
