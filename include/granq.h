@@ -173,11 +173,12 @@ int granq_fakequant_bwd(const void* gy, const void* x, int dtype, const int64_t 
 /*
  * The whole path in one call (Algorithm 1, range step through pre-scale step, plus the
  * backward): range of x itself -> scale / zero-point -> y, and gx when gy_opt is given.
- * The default plan stages a run of adjacent channels once in the shared memory of one thread-block
- * cluster where their group fits (x is then read from HBM exactly once); larger groups are processed
- * in waves of channel groups that stay in the L2 cache between the range pass and the quantize pass, so
- * x is read from HBM (about) once; channels-last geometries (channel_axis = 3, or planes of one element)
- * take a range launch and a quantize launch with one 16-byte unit column per thread.
+ * The default plan holds x in shared memory between the range and the quantize step, so that it is read from
+ * HBM once: a run of adjacent channels in one thread-block cluster where their group fits, a channel of a large
+ * plane in a team of CTAs.  What neither holds (byte codes or masks beside large planes, planes that are no whole
+ * 16-byte units) goes in waves of channel groups meant to stay in the L2 between the two steps.  Channels-last
+ * geometries (channel_axis = 3, or planes of one element) take one launch in which a thread keeps one 16-byte unit
+ * column; up to 33 MB of x stay in shared memory, more is read twice.
  *   x                 in   E elements          gy_opt   in   E elements or NULL (forward only)
  *   y                 out  E elements          gx_opt   out  E elements (required iff gy_opt)
  *   min_out, max_out  out  G floats each (required)
@@ -414,8 +415,9 @@ int granq_host_arena_status(int dtype, const int64_t dims[4], int channel_axis, 
 /*
  * Plan that granq_fakequant_fused() would take for this geometry and flags on the current
  * device: 0 = two-pass, 1 = naive per-channel loop, 2 = on-chip staged, 3 = L2-resident waves,
- * 4 = column walk, 5 = cluster-local, 6 = channels-last rows (range launch + quantize launch with one
- * 16-byte unit column per thread); negative = -status.
+ * 4 = column walk, 5 = cluster-local, 6 = channels-last rows; negative = -status.  Plan 4 covers two kernels, the
+ * resident form and the waves: granq_team_geometry() tells which.  The resident form also runs in place of plan 5
+ * for x of 96 MB and more (128 MB for fp32 with a gradient) in channels of at least 256 KB.
  * `launches_out` (HOST, may be NULL) receives the number of kernel launches of that plan.
  */
 int granq_fused_plan(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward,

@@ -128,7 +128,8 @@ __device__ __forceinline__ uint4 k_ld_l2_16(const void* p, uint64_t policy) {
                  : "memory");
     return v;
 }
-// per-thread asynchronous 16-byte copy global -> shared (both 16-byte aligned)
+// per-thread asynchronous 16-byte copy global -> shared (both 16-byte aligned); without an L2 policy, which is worth
+// nothing here and is under suspicion on this instruction (granq_colteam.cu)
 __device__ __forceinline__ void k_cp_async_16(void* dst_smem, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(k_smem_u32(dst_smem)), "l"(src) : "memory");
 }

@@ -77,8 +77,10 @@ __device__ __forceinline__ uint32_t t_ld_acquire(const uint32_t* p) {
 __device__ __forceinline__ void t_arrive_release(uint32_t* p) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
-// without an L2 cache hint: with one, sent from inside the (divergent) quantize walk, the kernel ended in an illegal
-// instruction on long walks
+// No L2 policy operand here, nor on any access of this kernel: a form that gave the copies sent from the quantize walk one
+// ended in an illegal instruction on [128,64,56,56], forward.  The cause was not found: operand widths, the policy's
+// lifetime, addresses, sizes and trip counts were in order, and the same instruction in loops of unequal trip counts ran
+// elsewhere without fault.  Without the operand, with streaming loads and stores: the same times.
 __device__ __forceinline__ void t_cp_async_16(void* dst_smem, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)), "l"(src)
                  : "memory");

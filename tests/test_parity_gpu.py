@@ -268,6 +268,26 @@ def test_colwalk_multiwave(b, knobs, shape, dtype):
         assert_parity(got, ref_f, shape, 1, orc.GROUP_CHANNEL, backward=False)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_outputs_that_the_binding_allocates_as_users_get_them(b, monkeypatch, dtype):
+    """The allocation path without the guard bands that the other tests put around every output."""
+    monkeypatch.setattr(b, "_new", b._plain_new)
+    shape = (6, 10, 9, 8)
+    x, gy = make_case(shape, seed=17, dtype=dtype)
+    ref = orc.fused(x, 4, gy=gy)
+    xd, gyd = to_dev(x), to_dev(gy)
+    got = b.granq_fakequant_fused(xd, 4, gy=gyd, want_codes=True, want_mask=True, want_params=True)
+    for t in (got.y, got.gx, got.codes, got.mask):
+        assert t.shape == xd.shape and t.is_contiguous() and t.device == xd.device
+    assert got.y.dtype == got.gx.dtype == xd.dtype
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=True)
+    fwd = b.granq_fakequant_fused_fwd_packmask(xd, 4)
+    assert_parity(fwd, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert same_bits(to_np(b.granq_fakequant_bwd_packmask(gyd, fwd.packed_mask)), ref.gx)
+    one = xd.view(6 * 10, 1, 9, 8)                     # a dimension of one: contiguous in more than one layout
+    assert b.granq_fakequant_fused(one, 4).y.stride() == one.stride()
+
+
 def test_colwalk_needs_slabs_to_walk(b):
     """Too few slabs (or the sample-channel / tensor views, which have one): left to the other plans."""
     with pytest.raises(b.GranqError) as err:
