@@ -63,7 +63,7 @@ def measured_peak():
         return FALLBACK_HBM_GBS, "fallback (6.65 TB/s, earlier measurement on this pool)"
 
 
-DOMINANT_KERNEL_SOURCES = ("granq_colwalk.cu", "granq_device.cuh")
+DOMINANT_KERNEL_SOURCES = ("granq_colteam.cu", "granq_device.cuh")
 
 
 def kernel_source_hash() -> str:
@@ -79,7 +79,7 @@ def kernel_source_hash() -> str:
 def recorded_traffic():
     """DRAM bytes per launch of the dominant kernel from the committed ncu summary, or None
     when there is none or the kernel sources have changed since it was taken."""
-    path = os.path.join(ROOT, "profiles", "colwalk_kernel_traffic.txt")
+    path = os.path.join(ROOT, "profiles", "colteam_kernel_traffic.txt")
     try:
         with open(path) as fh:
             rec = json.load(fh)
@@ -306,7 +306,7 @@ def main():
                 "l2_lag": b.KNOB_L2_LAG, "cl_tile_kb": b.KNOB_CLUSTER_TILE_KB, "cl_ctas": b.KNOB_CLUSTER_CTAS,
                 "cl_threads": b.KNOB_CLUSTER_THREADS, "cl_load": b.KNOB_CLUSTER_LOAD,
                 "cl_prefetch": b.KNOB_CLUSTER_PREFETCH, "cl_kmul": b.KNOB_CLUSTER_KMUL,
-                "cl_early_launch": b.KNOB_CLUSTER_EARLY_LAUNCH}
+                "cl_early_launch": b.KNOB_CLUSTER_EARLY_LAUNCH, "col_team": b.KNOB_COLWALK_TEAM}
     for item in filter(None, args.tune.split(",")):
         name, val = item.split("=")
         b.tune(knob_ids[name], int(val))
@@ -462,15 +462,18 @@ def main():
     # ---- per-call device times inside the timed region -> roofline of the dominant kernel ----
     per_call_ms = [statistics.mean(ev[k][ci].elapsed_time(ev[k][ci + 1]) for k in range(event_steps))
                    for ci in range(len(calls))]
-    # dominant kernel: the column-walk instantiation for planes that are whole 16-byte packs
-    dominant = [ci for ci, (i, _) in enumerate(calls) if (specs[i].shape[2] * specs[i].shape[3]) % 4 == 0
-                and plans[ci][0] == b.PLAN_COLWALK]
+    # dominant kernel: the resident form of the column walk
+    def resident(shape):
+        form = b.team_geometry(b.F32, shape)
+        return form is not None and form["taken"] == 1
+
+    dominant = [ci for ci, (i, _) in enumerate(calls) if plans[ci][0] == b.PLAN_COLWALK and resident(specs[i].shape)]
     dom_bytes = sum(specs[calls[ci][0]].numel for ci in dominant) * bpe
     dom_ms = sum(per_call_ms[ci] for ci in dominant)
     achieved = dom_bytes / (dom_ms * 1e-3) / 1e9 if dominant else None
     rec = recorded_traffic()
     roofline = {
-        "bound": "hbm", "kernel": "colwalk_kernel<float, fwd+bwd, aligned planes>",
+        "bound": "hbm", "kernel": "colteam_kernel<float, fwd+bwd>",
         "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": (achieved / peak) if achieved else None,
         "peak_source": peak_src, "frac_of_nominal_8TBs": (achieved / NOMINAL_HBM_GBS) if achieved else None,
         "launches_per_step": len(dominant),

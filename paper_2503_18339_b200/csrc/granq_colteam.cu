@@ -13,8 +13,8 @@
 //     loop sends the copy of the team's NEXT channel after it: reads stay in flight through the whole write phase.
 // With a gradient gy is staged the same way as far as shared memory goes and read in place beyond that.
 //
-// Why not the L2-resident waves of colwalk_kernel: the L2 does not keep a wave (forward-only calls read x 1.4 to 2
-// times from HBM, ncu: 5-14 % L2 hits), and its phases alternate.  Why teams and not clusters of 16 CTAs: a
+// Why not the L2-resident waves of colwalk_kernel: the L2 does not keep a wave (forward-only calls read x 1.4
+// times from HBM, ncu: 9-15 % L2 hits), and its phases alternate.  Why teams and not clusters of 16 CTAs: a
 // cluster must sit in one GPC, which leaves an SM in ten without one.  Measured against the waves (fp32 / bf16, us):
 // forward [128,64,56,56] 55.8 -> 45.7 / 34.7 -> 30.3, [128,96,112,112] 309 -> 264 / 174 -> 139, [256,512,28,28]
 // 219 -> 156 / 123 -> 92; with a gradient 87.5 -> 81.9 / 47.4 -> 45.6, 472 -> 469 / 258 -> 234, 332 -> 298 / 183 -> 153;
