@@ -461,6 +461,9 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
     __shared__ TileBase s_base;
     __shared__ float s_tab_s[kTableMax], s_tab_z[kTableMax], s_tab_r[kTableMax];
     constexpr bool kParts = kFlatParts<V, MODE, EXTRAS, RAGGED>;
+    // The first loads before the parameters, not where their registers cost a block per SM or are spilled, nor in the
+    // backward pass on ragged planes ([256,960,7,7] bf16 21.4 -> 22.6 us).
+    constexpr bool kEarly = EXTRAS != 1 && !(V == 8 && MODE == MODE_BOTH) && !(RAGGED && MODE == MODE_BWD);
     constexpr bool kFwd = (MODE & MODE_FWD) != 0, kBwd = (MODE & MODE_BWD) != 0;
     DistAcc dacc;
     dacc.reset();
@@ -469,6 +472,25 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
     for (int64_t tile = blockIdx.x; tile < g.ntiles; tile += gridDim.x) {
         const int64_t e0 = tile * (int64_t)kTile;
         const uint32_t ne = (uint32_t)min((int64_t)kTile, g.E - e0);
+        uint32_t k[kUnroll];
+        Pack<T> px[kUnroll], pg[kUnroll];
+        float sx[kUnroll], sg[kUnroll];
+        auto fetch = [&](uint32_t k0) {
+#pragma unroll
+            for (int j = 0; j < kUnroll; ++j) {
+                k[j] = k0 + (j * kThreads + threadIdx.x) * V;
+                if (k[j] < ne) {
+                    if constexpr (V == 1) {
+                        sx[j] = load_scalar(x + e0 + k[j]);
+                        if constexpr (kBwd) sg[j] = load_scalar(gy + e0 + k[j]);
+                    } else {
+                        px[j].raw = ld_stream_16(x + e0 + k[j]);
+                        if constexpr (kBwd) pg[j].raw = ld_stream_16(gy + e0 + k[j]);
+                    }
+                }
+            }
+        };
+        if constexpr (kEarly) fetch(0);            // under way while the table is made
         __syncthreads();
         if (threadIdx.x == 0) s_base = tile_base(g, e0);
         __syncthreads();
@@ -486,22 +508,7 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
             __syncthreads();
         }
         for (uint32_t k0 = 0; k0 < ne; k0 += kThreads * V * kUnroll) {
-            uint32_t k[kUnroll];
-            Pack<T> px[kUnroll], pg[kUnroll];
-            float sx[kUnroll], sg[kUnroll];
-#pragma unroll
-            for (int j = 0; j < kUnroll; ++j) {
-                k[j] = k0 + (j * kThreads + threadIdx.x) * V;
-                if (k[j] < ne) {
-                    if constexpr (V == 1) {
-                        sx[j] = load_scalar(x + e0 + k[j]);
-                        if constexpr (kBwd) sg[j] = load_scalar(gy + e0 + k[j]);
-                    } else {
-                        px[j].raw = ld_stream_16(x + e0 + k[j]);
-                        if constexpr (kBwd) pg[j].raw = ld_stream_16(gy + e0 + k[j]);
-                    }
-                }
-            }
+            if (!kEarly || k0 > 0) fetch(k0);
 #pragma unroll
             for (int j = 0; j < kUnroll; ++j) {
                 const bool valid = k[j] < ne;
@@ -687,38 +694,37 @@ __global__ void __launch_bounds__(kThreads) naive_quant_kernel(const T* __restri
 }
 
 // ---- STE backward from the packed mask alone (Section 2.1): gx = gy where the element's bit is set ----
+// A stream, bound by HBM: a block per 1024 units, in the order of memory ([128,96,112,112] 200 -> 185 us against a
+// persistent grid).
 // V = elements per thread and step: a 16-byte pack when E and the pointers allow it, else 1.
 template <typename T, int V>
 __global__ void __launch_bounds__(kThreads) bwd_packmask_kernel(const T* __restrict__ gy,
                                                                 const uint32_t* __restrict__ pmask,
                                                                 T* __restrict__ gx, int64_t E) {
-    const int64_t nunits = E / V;
-    const int64_t stride = (int64_t)gridDim.x * kThreads * kUnroll;
-    for (int64_t u0 = (int64_t)blockIdx.x * kThreads * kUnroll; u0 < nunits; u0 += stride) {
-        int64_t e[kUnroll];
-        Pack<T> pg[kUnroll];
-        float sg[kUnroll];
-        uint32_t w[kUnroll];
+    const int64_t u0 = (int64_t)blockIdx.x * kThreads * kUnroll;
+    int64_t e[kUnroll];
+    Pack<T> pg[kUnroll];
+    float sg[kUnroll];
+    uint32_t w[kUnroll];
 #pragma unroll
-        for (int j = 0; j < kUnroll; ++j) {
-            e[j] = (u0 + j * kThreads + threadIdx.x) * V;
-            if (e[j] < E) {
-                if constexpr (V == 1) sg[j] = load_scalar(gy + e[j]);
-                else pg[j].raw = ld_stream_16(gy + e[j]);
-                w[j] = __ldg(pmask + (e[j] >> 5));
-            }
+    for (int j = 0; j < kUnroll; ++j) {
+        e[j] = (u0 + j * kThreads + threadIdx.x) * V;
+        if (e[j] < E) {
+            if constexpr (V == 1) sg[j] = load_scalar(gy + e[j]);
+            else pg[j].raw = ld_stream_16(gy + e[j]);
+            w[j] = __ldg(pmask + (e[j] >> 5));
         }
+    }
 #pragma unroll
-        for (int j = 0; j < kUnroll; ++j) {
-            if (e[j] >= E) continue;
-            const uint32_t bits = w[j] >> (uint32_t)(e[j] & 31);
-            if constexpr (V == 1) {
-                store_scalar(gx + e[j], (bits & 1u) ? sg[j] : 0.0f);
-            } else {
-                Pack<T> out;
-                out.select(pg[j], bits);
-                st_stream_16(gx + e[j], out.raw);
-            }
+    for (int j = 0; j < kUnroll; ++j) {
+        if (e[j] >= E) continue;
+        const uint32_t bits = w[j] >> (uint32_t)(e[j] & 31);
+        if constexpr (V == 1) {
+            store_scalar(gx + e[j], (bits & 1u) ? sg[j] : 0.0f);
+        } else {
+            Pack<T> out;
+            out.select(pg[j], bits);
+            st_stream_16(gx + e[j], out.raw);
         }
     }
 }
@@ -763,7 +769,8 @@ __global__ void __launch_bounds__(kThreads) distortion_kernel(const T* __restric
 // codes, one pair of divisions for the channel, shifts that are constants, and 32 bytes of fp32 (16 of bf16) stored at
 // once.  Planes of at least 8 elements; where they are no multiple of 8 (RAGGED) a string may reach into the next
 // plane.  Bound by the stores: [128,144,56,56], 231 MB written from 36 MB of 5-bit codes, 92 -> 45 us
-// (5.9 TB/s; a thread per 16 bytes with two 32-bit divisions took 171 instructions for 4 elements).
+// (5.9 TB/s; a thread per 16 bytes with two 32-bit divisions took 171 instructions for 4 elements).  A block per 512
+// strings rather than a persistent grid, so that the stores go out in the order of memory: [128,96,112,112] 133 -> 110 us.
 template <typename T, int BITS, bool RAGGED>
 __global__ void __launch_bounds__(kThreads) dequant_strings_kernel(const uint32_t* __restrict__ pcodes, T* __restrict__ y,
                                                                    uint32_t nstrings, uint32_t last_word, uint32_t inner,
@@ -771,64 +778,63 @@ __global__ void __launch_bounds__(kThreads) dequant_strings_kernel(const uint32_
                                                                    const float* __restrict__ s, const float* __restrict__ z) {
     constexpr uint32_t kField = (1u << BITS) - 1u;
     constexpr int kFly = 2;
-    for (uint32_t t0 = blockIdx.x * (kThreads * kFly) + threadIdx.x; t0 < nstrings; t0 += gridDim.x * (kThreads * kFly)) {
-        uint32_t w[kFly][3];
+    const uint32_t t0 = blockIdx.x * (kThreads * kFly) + threadIdx.x;
+    uint32_t w[kFly][3];
 #pragma unroll
-        for (int f = 0; f < kFly; ++f) {
-            const uint32_t t = t0 + f * kThreads;
-            if (t >= nstrings) break;
-            const uint32_t w0 = (uint32_t)(((uint64_t)t * BITS) >> 2);              // 8 * BITS bits per string
-            w[f][0] = __ldg(pcodes + w0);
-            if constexpr (BITS > 1) w[f][1] = __ldg(pcodes + min(w0 + 1, last_word));
-            if constexpr (BITS == 6 || BITS == 7) w[f][2] = __ldg(pcodes + min(w0 + 2, last_word));
+    for (int f = 0; f < kFly; ++f) {
+        const uint32_t t = t0 + f * kThreads;
+        if (t >= nstrings) break;
+        const uint32_t w0 = (uint32_t)(((uint64_t)t * BITS) >> 2);              // 8 * BITS bits per string
+        w[f][0] = __ldg(pcodes + w0);
+        if constexpr (BITS > 1) w[f][1] = __ldg(pcodes + min(w0 + 1, last_word));
+        if constexpr (BITS == 6 || BITS == 7) w[f][2] = __ldg(pcodes + min(w0 + 2, last_word));
+    }
+#pragma unroll
+    for (int f = 0; f < kFly; ++f) {
+        const uint32_t t = t0 + f * kThreads;
+        if (t >= nstrings) break;
+        const uint32_t sh = (t * (8u * BITS)) & 31u;                            // 0, 8, 16 or 24
+        uint32_t lo, hi = 0;
+        if constexpr (BITS == 1) lo = w[f][0] >> sh;
+        else lo = __funnelshift_r(w[f][0], w[f][1], sh);
+        if constexpr (BITS == 8) hi = w[f][1];
+        else if constexpr (BITS == 6 || BITS == 7) hi = __funnelshift_r(w[f][1], w[f][2], sh);
+        else if constexpr (BITS == 5) hi = w[f][1] >> sh;
+        uint32_t plane, rem, q, g1;
+        div_inner.divmod(t * 8u, plane, rem);
+        div_C.divmod(plane, q, g1);
+        const float s1 = __ldg(s + g1), z1 = __ldg(z + g1);
+        float s2 = s1, z2 = z1;
+        const uint32_t n1 = inner - rem;                                        // elements left in this plane
+        if constexpr (RAGGED) {
+            if (n1 < 8) {
+                const uint32_t g2 = g1 + 1 == div_C.d ? 0u : g1 + 1;
+                s2 = __ldg(s + g2);
+                z2 = __ldg(z + g2);
+            }
         }
+        float v[8];
 #pragma unroll
-        for (int f = 0; f < kFly; ++f) {
-            const uint32_t t = t0 + f * kThreads;
-            if (t >= nstrings) break;
-            const uint32_t sh = (t * (8u * BITS)) & 31u;                            // 0, 8, 16 or 24
-            uint32_t lo, hi = 0;
-            if constexpr (BITS == 1) lo = w[f][0] >> sh;
-            else lo = __funnelshift_r(w[f][0], w[f][1], sh);
-            if constexpr (BITS == 8) hi = w[f][1];
-            else if constexpr (BITS == 6 || BITS == 7) hi = __funnelshift_r(w[f][1], w[f][2], sh);
-            else if constexpr (BITS == 5) hi = w[f][1] >> sh;
-            uint32_t plane, rem, q, g1;
-            div_inner.divmod(t * 8u, plane, rem);
-            div_C.divmod(plane, q, g1);
-            const float s1 = __ldg(s + g1), z1 = __ldg(z + g1);
-            float s2 = s1, z2 = z1;
-            const uint32_t n1 = inner - rem;                                        // elements left in this plane
-            if constexpr (RAGGED) {
-                if (n1 < 8) {
-                    const uint32_t g2 = g1 + 1 == div_C.d ? 0u : g1 + 1;
-                    s2 = __ldg(s + g2);
-                    z2 = __ldg(z + g2);
-                }
-            }
-            float v[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                constexpr uint32_t kTwo23 = 0x4B000000u;                            // 2^23: the code becomes the low mantissa
-                const int pos = i * BITS;
-                uint32_t c;
-                if (pos + BITS <= 32) c = lo >> pos;
-                else if (pos >= 32) c = hi >> (pos - 32);
-                else c = __funnelshift_r(lo, hi, pos);
-                const float code = __fsub_rn(__uint_as_float((c & kField) | kTwo23), 8388608.0f);
-                const bool first = !RAGGED || (uint32_t)i < n1;
-                v[i] = __fmul_rn(first ? s1 : s2, __fsub_rn(code, first ? z1 : z2));
-            }
-            T* out = y + (size_t)t * 8;
-            if constexpr (Pack<T>::V == 8) {
-                Pack<T> p;
-                p.set_all(v);
-                st_stream_16(out, p.raw);
-            } else {
-                asm volatile("st.global.L1::no_allocate.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(out), "f"(v[0]), "f"(v[1]),
-                             "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
-                             : "memory");
-            }
+        for (int i = 0; i < 8; ++i) {
+            constexpr uint32_t kTwo23 = 0x4B000000u;                            // 2^23: the code becomes the low mantissa
+            const int pos = i * BITS;
+            uint32_t c;
+            if (pos + BITS <= 32) c = lo >> pos;
+            else if (pos >= 32) c = hi >> (pos - 32);
+            else c = __funnelshift_r(lo, hi, pos);
+            const float code = __fsub_rn(__uint_as_float((c & kField) | kTwo23), 8388608.0f);
+            const bool first = !RAGGED || (uint32_t)i < n1;
+            v[i] = __fmul_rn(first ? s1 : s2, __fsub_rn(code, first ? z1 : z2));
+        }
+        T* out = y + (size_t)t * 8;
+        if constexpr (Pack<T>::V == 8) {
+            Pack<T> p;
+            p.set_all(v);
+            st_stream_16(out, p.raw);
+        } else {
+            asm volatile("st.global.L1::no_allocate.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(out), "f"(v[0]), "f"(v[1]),
+                         "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                         : "memory");
         }
     }
 }
@@ -949,7 +955,13 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
     constexpr int VF = Pack<T>::V;
     bool vec = (g.inner % VF == 0) && aligned16(io.x) && aligned16(io.gy) && aligned16(io.y) && aligned16(io.gx) &&
                ((uintptr_t)io.codes % 4 == 0) && ((uintptr_t)io.mask % 4 == 0);
-    int grid = flat_grid(f);
+    // A block per tile: blocks are then started in the order of memory, while the blocks of a persistent grid drift apart and
+    // DRAM sees more open pages (two reads and two writes of 617 MB: 5.9 to 6.3 TB/s persistent, 6.9 in order).  Given range,
+    // us: forward [128,96,112,112] 207 -> 182, [256,512,28,28] 138 -> 121, bf16 97 -> 90; backward from x, channels-last
+    // bf16 [40,100,100,200] 348 -> 281.  With the distortion sums a few tiles each, as every block ends in atomics on one
+    // sector, and so the scalar form below four rounds of blocks ([32,56,56,256] channels-last 115 / 119).
+    const int few = flat_grid(f);
+    const unsigned grid = io.dist || (!vec && f.ntiles < 4 * (int64_t)few) ? (unsigned)few : (unsigned)f.ntiles;
     float qmax = (float)((1 << bits) - 1);
     const bool extras = io.codes != nullptr || io.mask != nullptr || io.pmask != nullptr || io.dist != nullptr ||
                         io.pcodes != nullptr;
@@ -1055,11 +1067,10 @@ cudaError_t naive_t(const QuantIO& io, const Geom& g, int bits, uint32_t* kmin, 
 }
 
 template <typename T, int BITS>
-cudaError_t dequant_strings_bits(const uint32_t* pcodes, T* y, const Geom& g, const float* s, const float* z, int sms,
+cudaError_t dequant_strings_bits(const uint32_t* pcodes, T* y, const Geom& g, const float* s, const float* z,
                                  cudaStream_t st) {
     const uint32_t n = (uint32_t)(g.E / 8), last = (uint32_t)((g.E * BITS - 1) >> 5);
-    const uint32_t per_cta = kThreads * 2, want = (n + per_cta - 1) / per_cta, cap = (uint32_t)sms * 8;
-    const uint32_t grid = want < cap ? want : cap;
+    const uint32_t per_cta = kThreads * 2, grid = (n + per_cta - 1) / per_cta;
     const FastDiv di = make_fastdiv((uint32_t)g.inner), dc = make_fastdiv((uint32_t)g.C);
     if (g.inner % 8 == 0)
         dequant_strings_kernel<T, BITS, false><<<grid, kThreads, 0, st>>>(pcodes, y, n, last, (uint32_t)g.inner, di, dc, s, z);
@@ -1069,17 +1080,16 @@ cudaError_t dequant_strings_bits(const uint32_t* pcodes, T* y, const Geom& g, co
 }
 
 template <typename T>
-cudaError_t dequant_strings(const uint32_t* pcodes, T* y, const Geom& g, int bits, const float* s, const float* z, int sms,
-                            cudaStream_t st) {
+cudaError_t dequant_strings(const uint32_t* pcodes, T* y, const Geom& g, int bits, const float* s, const float* z, cudaStream_t st) {
     switch (bits) {
-        case 1: return dequant_strings_bits<T, 1>(pcodes, y, g, s, z, sms, st);
-        case 2: return dequant_strings_bits<T, 2>(pcodes, y, g, s, z, sms, st);
-        case 3: return dequant_strings_bits<T, 3>(pcodes, y, g, s, z, sms, st);
-        case 4: return dequant_strings_bits<T, 4>(pcodes, y, g, s, z, sms, st);
-        case 5: return dequant_strings_bits<T, 5>(pcodes, y, g, s, z, sms, st);
-        case 6: return dequant_strings_bits<T, 6>(pcodes, y, g, s, z, sms, st);
-        case 7: return dequant_strings_bits<T, 7>(pcodes, y, g, s, z, sms, st);
-        default: return dequant_strings_bits<T, 8>(pcodes, y, g, s, z, sms, st);
+        case 1: return dequant_strings_bits<T, 1>(pcodes, y, g, s, z, st);
+        case 2: return dequant_strings_bits<T, 2>(pcodes, y, g, s, z, st);
+        case 3: return dequant_strings_bits<T, 3>(pcodes, y, g, s, z, st);
+        case 4: return dequant_strings_bits<T, 4>(pcodes, y, g, s, z, st);
+        case 5: return dequant_strings_bits<T, 5>(pcodes, y, g, s, z, st);
+        case 6: return dequant_strings_bits<T, 6>(pcodes, y, g, s, z, st);
+        case 7: return dequant_strings_bits<T, 7>(pcodes, y, g, s, z, st);
+        default: return dequant_strings_bits<T, 8>(pcodes, y, g, s, z, st);
     }
 }
 
@@ -1128,16 +1138,11 @@ cudaError_t launch_naive(const QuantIO& io, int mode, int dtype, const Geom& g, 
 
 cudaError_t launch_bwd_packmask(const void* gy, const uint32_t* pmask, void* gx, int dtype, int64_t E,
                                 cudaStream_t st) {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int VF = dtype == 0 ? 4 : 8;
     const bool vec = aligned16(gy) && aligned16(gx) && (E % VF == 0);
     const int64_t units = vec ? E / VF : E;
     const int64_t per_cta = (int64_t)kThreads * kUnroll;
-    int64_t ctas = (units + per_cta - 1) / per_cta;
-    const int64_t cap = (int64_t)sms * 16;
-    const int grid = (int)(ctas < 1 ? 1 : (ctas < cap ? ctas : cap));
+    const unsigned grid = (unsigned)((units + per_cta - 1) / per_cta);
     if (dtype == 0) {
         if (vec) bwd_packmask_kernel<float, 4><<<grid, kThreads, 0, st>>>((const float*)gy, pmask, (float*)gx, E);
         else bwd_packmask_kernel<float, 1><<<grid, kThreads, 0, st>>>((const float*)gy, pmask, (float*)gx, E);
@@ -1178,17 +1183,17 @@ cudaError_t launch_distortion(const void* x, const void* q, int dtype, int64_t E
 
 cudaError_t launch_dequant_packed(const uint32_t* pcodes, void* y, int dtype, const Geom& g, int bits,
                                   const float* s, const float* z, cudaStream_t st) {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // strings of 8 codes: planes of at least 8 elements, a whole number of strings, 32-byte (fp32) stores
     if (g.E % 8 == 0 && g.E < (1ll << 31) && g.inner >= 8 && g.inner < (1ll << 30) && g.C < (1ll << 30) &&
         ((uintptr_t)y & (dtype == 0 ? 31 : 15)) == 0)
-        return dtype == 0 ? dequant_strings<float>(pcodes, (float*)y, g, bits, s, z, sms, st)
-                          : dequant_strings<__nv_bfloat16>(pcodes, (__nv_bfloat16*)y, g, bits, s, z, sms, st);
+        return dtype == 0 ? dequant_strings<float>(pcodes, (float*)y, g, bits, s, z, st)
+                          : dequant_strings<__nv_bfloat16>(pcodes, (__nv_bfloat16*)y, g, bits, s, z, st);
     const int VF = dtype == 0 ? 4 : 8;
     const bool vec = aligned16(y) && (g.E % VF == 0);
     const int64_t units = vec ? g.E / VF : g.E;
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t ctas = (units + kThreads - 1) / kThreads, cap = (int64_t)sms * 16;
     const int grid = (int)(ctas < 1 ? 1 : (ctas < cap ? ctas : cap));
     if (dtype == 0) {
