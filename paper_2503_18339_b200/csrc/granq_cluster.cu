@@ -139,40 +139,6 @@ __device__ __forceinline__ void k_cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// per-element running min / max of one unit column
-template <typename T>
-struct KRange {
-    float mn[Pack<T>::V], mx[Pack<T>::V];
-    __device__ __forceinline__ void reset() {
-#pragma unroll
-        for (int i = 0; i < Pack<T>::V; ++i) {
-            mn[i] = INFINITY;
-            mx[i] = -INFINITY;
-        }
-    }
-    __device__ __forceinline__ void add(const Pack<T>& p) {
-#pragma unroll
-        for (int i = 0; i < Pack<T>::V; ++i) {
-            const float v = p.get(i);
-            mn[i] = fminf(mn[i], v);
-            mx[i] = fmaxf(mx[i], v);
-        }
-    }
-    // ordered keys of elements [first, last); (0, 0) when that range is empty or nothing was added
-    __device__ __forceinline__ void keys(int first, int last, uint32_t& kmn, uint32_t& kmx) const {
-        float a = INFINITY, b = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < Pack<T>::V; ++i) {
-            if (i >= first && i < last) {
-                a = fminf(a, mn[i]);
-                b = fmaxf(b, mx[i]);
-            }
-        }
-        kmn = (a <= b) ? ~enc(a) : 0u;
-        kmx = (a <= b) ? enc(b) : 0u;
-    }
-};
-
 // All 32 lanes: fold the lanes' (channel, keys) into the keys in shared memory - of this CTA and of
 // every other CTA of its cluster - with one pair of atomics per distinct channel of the warp and CTA.
 __device__ __forceinline__ void k_warp_fold(bool valid, uint32_t ch, uint32_t ka, uint32_t kb, uint32_t* s_kmn,
@@ -354,7 +320,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
     for (uint32_t tile0 = 0; tile0 < ncol; tile0 += P) {
         const uint32_t col = tile0 + cin;
         const bool valid = rowed && col < ncol;
-        KRange<T> acc;
+        RangeColumn<T> acc;
         acc.reset();
         if (valid) {
             if constexpr (LOAD != K_LOAD_PLAIN) {
@@ -411,11 +377,11 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
         int ne = V;
         if (valid) column(col, ch, ne);
         uint32_t ka, kb;
-        acc.keys(0, ne, ka, kb);
+        column_keys(acc, 0, ne, ka, kb);
         k_warp_fold(valid, ch, ka, kb, s_kmn, s_kmx, R);
         if constexpr (!ALIGNED) {
             uint32_t kc2, kd2;
-            acc.keys(ne, V, kc2, kd2);
+            column_keys(acc, ne, V, kc2, kd2);
             k_warp_fold(valid && ne < V, ch + 1, kc2, kd2, s_kmn, s_kmx, R);
         }
     }
@@ -462,7 +428,9 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
         auto emit = [&](const Pack<T>& px, const Pack<T>& pg, size_t at) {
             Pack<T> py, pgx;
             uint32_t cb[V / 4], mb[V / 4];
-            quantize_pack<T, kBwd, !ALIGNED, EXTRAS, true>(px, pg, g1, g2, ne, qmax, py, pgx, cb, mb, EXTRAS == 3 ? a.code_bits : 8);
+            const int code_bits = EXTRAS == 3 ? a.code_bits : 8;
+            if constexpr (ALIGNED) quantize_own<T, kBwd, EXTRAS>(px, pg, g1, qmax, py, pgx, cb, mb, code_bits);
+            else quantize_pack<T, kBwd, true, EXTRAS, true>(px, pg, g1, g2, ne, qmax, py, pgx, cb, mb, code_bits);
             if constexpr (EXTRAS == 3) {
                 // the packed codes are the only output: 8 codes = b bytes per pair of fp32 lanes (per bf16 lane); the
                 // planner has made every run and slab whole groups of 8 elements, so both lanes of a pair are here

@@ -144,18 +144,14 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     for (uint32_t c = team; c < a.C; c += a.teams) {
         t_cp_async_wait_all();
         // ---- Eq. 4: range of this CTA's share ----
-        float mn[2] = {INFINITY, INFINITY}, mx[2] = {-INFINITY, -INFINITY};
+        RangeFold<T> fold;
         for (uint32_t i = 0; i < cnt; ++i) {
             Pack<T> p;
             p.raw = tile[i * kTThreads];
-#pragma unroll
-            for (int e = 0; e < V; ++e) {
-                const float v = p.get(e);
-                mn[e & 1] = fminf(mn[e & 1], v);
-                mx[e & 1] = fmaxf(mx[e & 1], v);
-            }
+            fold.add(p);
         }
-        const float m0 = fminf(mn[0], mn[1]), m1 = fmaxf(mx[0], mx[1]);
+        float m0, m1;
+        fold.result(m0, m1);
         uint32_t ka = m0 <= m1 ? ~enc(m0) : 0u, kb = m0 <= m1 ? enc(m1) : 0u;
         ka = __reduce_max_sync(kFullMask, ka);
         kb = __reduce_max_sync(kFullMask, kb);
@@ -206,7 +202,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
         auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint64_t at) {
             Pack<T> py, pgx;
             uint32_t cb[V / 4], mb[V / 4];
-            quantize_pack<T, kBwd, false, EXTRAS, true>(px, pg, g, g, V, qmax, py, pgx, cb, mb, BITS);
+            quantize_own<T, kBwd, EXTRAS>(px, pg, g, qmax, py, pgx, cb, mb, BITS);
             if constexpr (EXTRAS == 3) {
                 const uint64_t str = code_string_of<V>(cb, BITS);
                 if constexpr (V == 4) {

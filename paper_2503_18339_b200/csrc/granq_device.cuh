@@ -457,6 +457,85 @@ __device__ __forceinline__ void quantize_pack(const Pack<T>& px, const Pack<T>& 
     py.set_all(yv);
 }
 
+// Two floats side by side: the fp32 pipe takes both with one instruction (fma, add, multiply; each rounded as its scalar
+// form), which is half the issue slots.
+struct F2 {
+    uint64_t v;
+};
+__device__ __forceinline__ F2 f2(float lo, float hi) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_split(F2 a, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+
+// Quantize one fp32 pack of one group whose range is that of the tensor itself (thr from group_param_from_range()); bf16 goes
+// on to quantize_pack(), which also says what the outputs are.  In the main line nothing is clamped and the gradient passes
+// whole: w = fma(x, 1 / s, mz) rounds, e = mz - w = -(code - z) exactly, fma(x, 1 / s, e) is the distance from the integer,
+// and y = s * (code - z) is fma(-s, e, +0), whose +0 keeps a zero from coming out as -0: four packed instructions for two
+// elements.  A pack with an element too close to a tie or a NaN (which becomes code 0 without a gradient, as in the sequence
+// as defined), or of a group without a shortcut, is worked out again element by element; groups that may be clamped clamp.
+// Against the scalar form, geometric mean over 26 shapes: forward 0.98, with sums 0.98, weights 0.96 of the time.  bf16, whose
+// elements have to be moved into pairs of registers first, is 3 to 10 % slower this way.
+template <typename T, bool BWD, int EXTRAS>
+__device__ __forceinline__ void quantize_own(const Pack<T>& px, const Pack<T>& pg, const GroupParam& g, float qmax, Pack<T>& py,
+                                             Pack<T>& pgx, uint32_t (&cb)[Pack<T>::V / 4], uint32_t (&mb)[Pack<T>::V / 4],
+                                             int code_bits = 8) {
+    constexpr int V = Pack<T>::V;
+    if constexpr (V == 8) {
+        quantize_pack<T, BWD, false, EXTRAS, true>(px, pg, g, g, V, qmax, py, pgx, cb, mb, code_bits);
+    } else {
+        const float mz = __fadd_rn(kRoundMagic, g.z), top = __fadd_rn(kRoundMagic, qmax);
+        const F2 r2 = f2(g.r, g.r), mz2 = f2(mz, mz), ns2 = f2(-g.s, -g.s), zero = {0};
+        float m[V], yv[V], worst = 0.0f;
+        uint32_t in = (1u << V) - 1u;
+#pragma unroll
+        for (int k = 0; k < V; k += 2) {
+            const F2 x = f2(px.get(k), px.get(k + 1)), w = f2_fma(x, r2, mz2), e = f2_sub(mz2, w);
+            float d0, d1;
+            f2_split(f2_fma(x, r2, e), d0, d1);
+            worst = max_or_nan(max_or_nan(worst, fabsf(d0)), fabsf(d1));
+            f2_split(f2_fma(ns2, e, zero), yv[k], yv[k + 1]);
+            f2_split(w, m[k], m[k + 1]);
+        }
+        if constexpr (BWD) pgx.raw = pg.raw;
+        if (!(worst < fabsf(g.thr))) {
+            in = 0;
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                const float x = px.get(i);
+                float r = __fmaf_rn(x, g.r, mz);
+                if (g.thr == 0.0f) r = exact_round_magic(__fdiv_rn(x, g.s), g.z, qmax);
+                else if (!(fabsf(__fmaf_rn(x, g.r, __fsub_rn(mz, r))) < fabsf(g.thr))) r = exact_round_magic(div_by_scale(x, g.s, g.r), g.z, qmax);
+                m[i] = fminf(fmaxf(r, kRoundMagic), top);
+                in |= (m[i] == r) ? (1u << i) : 0u;
+                yv[i] = __fmul_rn(g.s, __fsub_rn(__fsub_rn(m[i], kRoundMagic), g.z));
+            }
+            if constexpr (BWD) pgx.select(pg, in);
+        } else if (g.thr < 0.0f) {
+            clamp_codes<0, V, false>(m, top, in);
+#pragma unroll
+            for (int k = 0; k < V; k += 2)
+                f2_split(f2_fma(ns2, f2_sub(mz2, f2(m[k], m[k + 1])), zero), yv[k], yv[k + 1]);
+            if constexpr (BWD) pgx.select(pg, in);
+        }
+        pack_extras<V, EXTRAS>(m, in, cb, mb, code_bits);
+        py.set_all(yv);
+    }
+}
+
 // Quantize one pack whose V elements belong to V different groups (channels-last rows), the range being the
 // tensor's own: element i takes scale s[i], reciprocal r[i] and mz[i] = 1.5 * 2^23 + z; thr is the smallest of the
 // V groups' thresholds in magnitude, negative when one of them is, and where it is 0 the parameters are read again
@@ -506,6 +585,102 @@ __device__ __forceinline__ void quantize_pack_each(const Pack<T>& px, const Pack
     if constexpr (BWD) pgx.select(pg, in);
     pack_extras<V, EXTRAS ? 1 : 0>(m, in, cb, mb, 8);
     py.set_all(yv);
+}
+
+// Smallest and largest of any number of packs (NaN left out, as by fminf / fmaxf); two independent chains.
+template <typename T>
+struct RangeFold;
+template <>
+struct RangeFold<float> {
+    float mn[2] = {INFINITY, INFINITY}, mx[2] = {-INFINITY, -INFINITY};
+    __device__ __forceinline__ void add(const Pack<float>& p) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            mn[e & 1] = fminf(mn[e & 1], p.get(e));
+            mx[e & 1] = fmaxf(mx[e & 1], p.get(e));
+        }
+    }
+    __device__ __forceinline__ void result(float& lo, float& hi) const {
+        lo = fminf(mn[0], mn[1]);
+        hi = fmaxf(mx[0], mx[1]);
+    }
+};
+// bf16 two at a time as they are stored: half an instruction per element and side, nothing to widen
+template <>
+struct RangeFold<__nv_bfloat16> {
+    uint32_t mn[2] = {0x7F807F80u, 0x7F807F80u}, mx[2] = {0xFF80FF80u, 0xFF80FF80u};
+    __device__ __forceinline__ static void min2(uint32_t& a, uint32_t b) { asm("min.bf16x2 %0, %0, %1;" : "+r"(a) : "r"(b)); }
+    __device__ __forceinline__ static void max2(uint32_t& a, uint32_t b) { asm("max.bf16x2 %0, %0, %1;" : "+r"(a) : "r"(b)); }
+    __device__ __forceinline__ void add(const Pack<__nv_bfloat16>& p) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            min2(mn[k & 1], (&p.raw.x)[k]);
+            max2(mx[k & 1], (&p.raw.x)[k]);
+        }
+    }
+    __device__ __forceinline__ void result(float& lo, float& hi) const {
+        uint32_t a = mn[0], b = mx[0];
+        min2(a, mn[1]);
+        max2(b, mx[1]);
+        lo = fminf(__uint_as_float(a << 16), __uint_as_float(a & 0xFFFF0000u));
+        hi = fmaxf(__uint_as_float(b << 16), __uint_as_float(b & 0xFFFF0000u));
+    }
+};
+
+// Smallest and largest per element of a pack, over any number of packs: a unit column, whose element i belongs to the same
+// channel all the way down.
+template <typename T>
+struct RangeColumn;
+template <>
+struct RangeColumn<float> {
+    float mn[4], mx[4];
+    __device__ __forceinline__ void reset() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            mn[i] = INFINITY;
+            mx[i] = -INFINITY;
+        }
+    }
+    __device__ __forceinline__ void add(const Pack<float>& p) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            mn[i] = fminf(mn[i], p.get(i));
+            mx[i] = fmaxf(mx[i], p.get(i));
+        }
+    }
+    __device__ __forceinline__ float lo(int i) const { return mn[i]; }
+    __device__ __forceinline__ float hi(int i) const { return mx[i]; }
+};
+template <>
+struct RangeColumn<__nv_bfloat16> {
+    Pack<__nv_bfloat16> mn, mx;         // as they are stored, two to a word (RangeFold)
+    __device__ __forceinline__ void reset() {
+        mn.raw = make_uint4(0x7F807F80u, 0x7F807F80u, 0x7F807F80u, 0x7F807F80u);
+        mx.raw = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+    }
+    __device__ __forceinline__ void add(const Pack<__nv_bfloat16>& p) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            RangeFold<__nv_bfloat16>::min2((&mn.raw.x)[k], (&p.raw.x)[k]);
+            RangeFold<__nv_bfloat16>::max2((&mx.raw.x)[k], (&p.raw.x)[k]);
+        }
+    }
+    __device__ __forceinline__ float lo(int i) const { return mn.get(i); }
+    __device__ __forceinline__ float hi(int i) const { return mx.get(i); }
+};
+// ordered keys of elements [first, last) of a column; (0, 0) when that range is empty or nothing was added
+template <typename T>
+__device__ __forceinline__ void column_keys(const RangeColumn<T>& c, int first, int last, uint32_t& kmn, uint32_t& kmx) {
+    float a = INFINITY, b = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < Pack<T>::V; ++i) {
+        if (i >= first && i < last) {
+            a = fminf(a, c.lo(i));
+            b = fmaxf(b, c.hi(i));
+        }
+    }
+    kmn = (a <= b) ? ~enc(a) : 0u;
+    kmx = (a <= b) ? enc(b) : 0u;
 }
 
 // per-lane min / max of elements [first, last) of one pack

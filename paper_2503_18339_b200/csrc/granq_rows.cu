@@ -109,20 +109,8 @@ __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a)
 
     // ---- Eq. 4: rows beyond the kept ones straight from memory, then the kept ones ----
     {
-        float mn[V], mx[V];
-#pragma unroll
-        for (int i = 0; i < V; ++i) {
-            mn[i] = INFINITY;
-            mx[i] = -INFINITY;
-        }
-        auto add = [&](const Pack<T>& p) {
-#pragma unroll
-            for (int i = 0; i < V; ++i) {
-                const float v = p.get(i);
-                mn[i] = fminf(mn[i], v);
-                mx[i] = fmaxf(mx[i], v);
-            }
-        };
+        RangeColumn<T> acc;
+        acc.reset();
         const uint4* src = xg + held * step;
         for (uint32_t k = held; k < n; k += U1, src += U1 * step) {
             Pack<T> v[U1];
@@ -131,19 +119,21 @@ __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a)
                 if (k + j < n) v[j].raw = k < a.lost ? ld_hint_16(src + j * step, drop) : __ldg(src + j * step);
 #pragma unroll
             for (int j = 0; j < U1; ++j)
-                if (k + j < n) add(v[j]);
+                if (k + j < n) acc.add(v[j]);
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         for (uint32_t k = 0; k < held; ++k) {
             Pack<T> v;
             v.raw = tile[k * tstep];
-            add(v);
+            acc.add(v);
         }
         if (n > 0) {
 #pragma unroll
             for (int i = 0; i < V; ++i) {
-                atomicMax(s_kmn + i * P + cin, mn[i] <= mx[i] ? ~enc(mn[i]) : 0u);
-                atomicMax(s_kmx + i * P + cin, mn[i] <= mx[i] ? enc(mx[i]) : 0u);
+                uint32_t ka, kb;
+                column_keys(acc, i, i + 1, ka, kb);
+                atomicMax(s_kmn + i * P + cin, ka);
+                atomicMax(s_kmx + i * P + cin, kb);
             }
         }
     }

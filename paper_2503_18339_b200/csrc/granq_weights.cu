@@ -164,7 +164,8 @@ __global__ void __launch_bounds__(kWThreads, HOLD == 1 ? (GRAD ? 5 : 6) : GRAD ?
         auto emit = [&](const Pack<T>& p, const Pack<T>& g, uint32_t u) {
             Pack<T> py, pgx;
             uint32_t cb[V / 4], mb[V / 4];
-            quantize_pack<T, GRAD, false, 0, true>(p, g, gp, gp, V, qmax, py, pgx, cb, mb);
+            if constexpr (GRAD) quantize_pack<T, GRAD, false, 0, true>(p, g, gp, gp, V, qmax, py, pgx, cb, mb);
+            else quantize_own<T, GRAD, 0>(p, g, gp, qmax, py, pgx, cb, mb);
             st_stream_16(y + (size_t)u * V, py.raw);
             if constexpr (GRAD) {
                 if (grad) st_stream_16(gx + (size_t)u * V, pgx.raw);
