@@ -65,7 +65,7 @@ struct TArgs {
     uint32_t tile_units;   // room for x in shared memory
     uint32_t gy_units;     // of a CTA's share of gy, this many units are staged behind it
     uint32_t spin_limit, expected;
-    uint64_t slab_units;   // units of one slab
+    uint32_t slab_units;   // units of one slab
     FastDiv div_plane;     // units per plane
 };
 
@@ -277,33 +277,216 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     }
 }
 
+// The same with a gradient where a team has several rounds of channels: two channels side by side in shared memory, gy read in
+// place.  The range of channel t is taken and handed to the team before channel t - 1 is quantized, so that the hand-over has
+// that whole walk to complete in; a warp that holds no units does it.  (Forward calls lose by it: their walk is half as long,
+// and twice the rounds cost more than the hand-over: [256,512,28,28] 151 / 163 us.)
+constexpr uint32_t kTWork = kTThreads - 32;
+
+template <typename T, int U>
+__global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a) {
+    constexpr int V = Pack<T>::V;
+    constexpr uint32_t depth = 2;
+    extern __shared__ __align__(16) uint4 t_smem[];
+    __shared__ uint32_t s_kmn[2][kTWarps], s_kmx[2][kTWarps];
+    __shared__ GroupParam s_par[2];
+    __shared__ uint32_t s_bad, s_last;      // the job whose hand-over ran out of its wait; is this the last CTA?
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t team = blockIdx.x / a.R, rank = blockIdx.x - team * a.R;
+    const uint32_t jobs = (a.C - team + a.teams - 1) / a.teams;      // channels of this team: team, team + teams, ...
+    // this CTA's share: whole runs of 8 units (128 bytes) of the channel's units laid end to end
+    const uint32_t runs = (a.units + 7) / 8;
+    const uint32_t q0 = 8 * (uint32_t)(((uint64_t)rank * runs) / a.R);
+    const uint32_t q1 = min(a.units, 8 * (uint32_t)(((uint64_t)(rank + 1) * runs) / a.R));
+    const uint32_t n = q1 - q0;
+    const uint32_t cnt = tid < min(n, (uint32_t)kTWork) ? (n - tid + kTWork - 1) / kTWork : 0u;      // units of this thread
+    // where they are: unit q lies in slab q / plane_units, and the next one of this thread is kTWork units on
+    uint32_t slab0, off0;
+    a.div_plane.divmod(q0 + min(tid, n), slab0, off0);
+    const uint32_t first = slab0 * a.slab_units + off0;
+    uint32_t dslab, doff;
+    a.div_plane.divmod((uint32_t)kTWork, dslab, doff);
+    const uint32_t dstep = dslab * a.slab_units + doff, dwrap = a.slab_units - a.plane_units;
+    auto advance = [&](uint32_t& at, uint32_t& off) {
+        at += dstep;
+        off += doff;
+        if (off >= a.plane_units) {
+            off -= a.plane_units;
+            at += dwrap;
+        }
+    };
+    const uint4* xg = reinterpret_cast<const uint4*>(a.x);
+    const uint4* gyg = reinterpret_cast<const uint4*>(a.gy);
+    uint4* yg = reinterpret_cast<uint4*>(a.y);
+    uint4* gxg = reinterpret_cast<uint4*>(a.gx);
+    const float qmax = a.qmax;
+
+    // ---- Eq. 4: range of this CTA's share of job j, from its tile to the warps' keys ----
+    auto reduce = [&](uint32_t j, const uint4* tile) {
+        RangeFold<T> fold;
+        for (uint32_t i = 0; i < cnt; ++i) {
+            Pack<T> p;
+            p.raw = tile[i * kTWork];
+            fold.add(p);
+        }
+        float m0, m1;
+        fold.result(m0, m1);
+        uint32_t ka = m0 <= m1 ? ~enc(m0) : 0u, kb = m0 <= m1 ? enc(m1) : 0u;
+        ka = __reduce_max_sync(kFullMask, ka);
+        kb = __reduce_max_sync(kFullMask, kb);
+        if (lane == 0) {
+            s_kmn[j & 1][warp] = ka;
+            s_kmx[j & 1][warp] = kb;
+        }
+    };
+    // ---- the last warp: publish job j's keys, wait (bounded) until the whole team has; Eq. 5 ----
+    auto hand_over = [&](uint32_t j) {
+        const uint32_t c = team + j * a.teams;
+        const uint32_t ka = __reduce_max_sync(kFullMask, lane < kTWork / 32 ? s_kmn[j & 1][lane] : 0u);
+        const uint32_t kb = __reduce_max_sync(kFullMask, lane < kTWork / 32 ? s_kmx[j & 1][lane] : 0u);
+        if (lane != 0) return;
+        atomicMax(a.kmin + c, ka);
+        atomicMax(a.kmax + c, kb);
+        t_arrive_release(a.counters + c);
+        uint32_t ready = 0;
+        for (uint32_t i = 0; i < a.spin_limit; ++i) {
+            if (t_ld_acquire(a.counters + c) >= a.expected) {
+                ready = 1;
+                break;
+            }
+            __nanosleep(32);
+        }
+        if (!ready) {
+            s_bad = j;
+            atomicExch(a.status, kTStatusTimeout);
+            return;
+        }
+        float lo, hi;
+        const GroupParam gp = group_param_from_keys(a.kmin, a.kmax, c, qmax, lo, hi);
+        s_par[j & 1] = gp;
+        if (rank == 0) {
+            a.lo[c] = lo;
+            a.hi[c] = hi;
+            if (a.s_out) a.s_out[c] = gp.s;
+            if (a.z_out) a.z_out[c] = gp.z;
+        }
+    };
+    // ---- Eq. 1, clamp, Eq. 6, STE of job j from its tile; the copies of job j + depth follow on the heels ----
+    auto quantize = [&](uint32_t j, uint4* tile) {
+        const GroupParam g = s_par[j & 1];
+        const bool more = j + depth < jobs;
+        const uint32_t ahead = depth * a.teams * a.plane_units;
+        auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint32_t at) {
+            Pack<T> py, pgx;
+            uint32_t cb[V / 4], mb[V / 4];
+            quantize_own<T, true, 0>(px, pg, g, qmax, py, pgx, cb, mb);
+            st_stream_16(yg + at, py.raw);
+            st_stream_16(gxg + at, pgx.raw);
+        };
+        uint32_t at = first + (team + j * a.teams) * a.plane_units, off = off0, i = 0;
+        for (; i + U <= cnt; i += U) {
+            Pack<T> px[U], pg[U];
+            uint32_t w[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                w[k] = at;
+                pg[k].raw = ld_stream_16(gyg + at);
+                px[k].raw = tile[(i + k) * kTWork];
+                advance(at, off);
+            }
+            if (more) {
+#pragma unroll
+                for (int k = 0; k < U; ++k) t_cp_async_16(tile + (i + k) * kTWork, xg + (w[k] + ahead));
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) emit(px[k], pg[k], w[k]);
+        }
+        for (; i < cnt; ++i) {
+            Pack<T> px, pg;
+            pg.raw = ld_stream_16(gyg + at);
+            px.raw = tile[i * kTWork];
+            if (more) t_cp_async_16(tile + i * kTWork, xg + (at + ahead));
+            emit(px, pg, at);
+            advance(at, off);
+        }
+    };
+
+    if (tid == 0) s_bad = 0xFFFFFFFFu;
+    // the first copies; those of the later jobs are sent from the quantize walk
+    for (uint32_t j = 0; j < depth; ++j) {
+        uint4* tile = t_smem + j * a.tile_units + tid;
+        uint32_t at = first + (team + j * a.teams) * a.plane_units, off = off0;
+        if (j < jobs) {
+            for (uint32_t i = 0; i < cnt; ++i) {
+                t_cp_async_16(tile + i * kTWork, xg + at);
+                advance(at, off);
+            }
+        }
+    }
+    for (uint32_t t = 0; t <= jobs; ++t) {
+        if (t < jobs) {
+            t_cp_async_wait_all();
+            if (warp < kTWork / 32) reduce(t, t_smem + (t & 1) * a.tile_units + tid);
+        }
+        __syncthreads();
+        // job t's wait may run out while a slow warp is still here: it looks at the jobs before
+        if (t > 0 && *(volatile uint32_t*)&s_bad < t) break;
+        if (t < jobs && warp == kTWork / 32) hand_over(t);
+        if (t > 0) quantize(t - 1, t_smem + ((t - 1) & 1) * a.tile_units + tid);
+    }
+    if (*(volatile uint32_t*)&s_bad < jobs) {      // a wait has run out: nothing may be in flight when the CTA leaves
+        t_cp_async_wait_all();
+        return;
+    }
+
+    // ---- leave the workspace as it was found: the last CTA to finish clears keys and counters ----
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        s_last = (atomicAdd(a.counters + a.C, 1u) == gridDim.x - 1) ? 1u : 0u;
+    }
+    __syncthreads();
+    if (s_last) {
+        for (uint32_t i = tid; i < a.C; i += kTThreads) {
+            a.kmin[i] = 0;
+            a.kmax[i] = 0;
+        }
+        for (uint32_t i = tid; i <= a.C; i += kTThreads) a.counters[i] = 0;
+    }
+}
+
 template <typename T, int MODE, int EXTRAS, int BITS = 8>
-cudaError_t t_launch(const TArgs& args, uint32_t smem, const StagedTuning& tune, cudaStream_t st) {
-    auto kern = colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2), BITS>;
-    const cudaError_t e = allow_smem(kern, kTSmemUnits * 16);
-    if (e != cudaSuccess) return e;
-    void* params[] = {(void*)&args};
-    return launch_cooperative((const void*)kern, args.R * args.teams, kTThreads, params, smem, tune, st);
+cudaError_t t_launch(const TArgs& args, const TeamPlan& p, const StagedTuning& tune, cudaStream_t st) {
+    auto launch = [&](auto kern) -> cudaError_t {
+        const cudaError_t e = allow_smem(kern, kTSmemUnits * 16);
+        if (e != cudaSuccess) return e;
+        void* params[] = {(void*)&args};
+        return launch_cooperative((const void*)kern, args.R * args.teams, kTThreads, params, p.smem_bytes, tune, st);
+    };
+    if constexpr (MODE == MODE_BOTH) {
+        if (p.lag) return launch(colteam_lag_kernel<T, 2>);
+    }
+    return launch(colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2), BITS>);
 }
 
 template <typename T>
-cudaError_t t_launch_mode(const TArgs& a, int mode, int extras, uint32_t smem, const StagedTuning& tune, cudaStream_t st) {
-    if (mode == MODE_BOTH) return t_launch<T, MODE_BOTH, 0>(a, smem, tune, st);
+cudaError_t t_launch_mode(const TArgs& a, int mode, int extras, const TeamPlan& p, const StagedTuning& tune, cudaStream_t st) {
+    if (mode == MODE_BOTH) return t_launch<T, MODE_BOTH, 0>(a, p, tune, st);
     switch (extras) {
-        case 2: return t_launch<T, MODE_FWD, 2>(a, smem, tune, st);
+        case 2: return t_launch<T, MODE_FWD, 2>(a, p, tune, st);
         case 3:
             switch (a.code_bits) {
-                case 1: return t_launch<T, MODE_FWD, 3, 1>(a, smem, tune, st);
-                case 2: return t_launch<T, MODE_FWD, 3, 2>(a, smem, tune, st);
-                case 3: return t_launch<T, MODE_FWD, 3, 3>(a, smem, tune, st);
-                case 4: return t_launch<T, MODE_FWD, 3, 4>(a, smem, tune, st);
-                case 5: return t_launch<T, MODE_FWD, 3, 5>(a, smem, tune, st);
-                case 6: return t_launch<T, MODE_FWD, 3, 6>(a, smem, tune, st);
-                case 7: return t_launch<T, MODE_FWD, 3, 7>(a, smem, tune, st);
-                default: return t_launch<T, MODE_FWD, 3, 8>(a, smem, tune, st);
+                case 1: return t_launch<T, MODE_FWD, 3, 1>(a, p, tune, st);
+                case 2: return t_launch<T, MODE_FWD, 3, 2>(a, p, tune, st);
+                case 3: return t_launch<T, MODE_FWD, 3, 3>(a, p, tune, st);
+                case 4: return t_launch<T, MODE_FWD, 3, 4>(a, p, tune, st);
+                case 5: return t_launch<T, MODE_FWD, 3, 5>(a, p, tune, st);
+                case 6: return t_launch<T, MODE_FWD, 3, 6>(a, p, tune, st);
+                case 7: return t_launch<T, MODE_FWD, 3, 7>(a, p, tune, st);
+                default: return t_launch<T, MODE_FWD, 3, 8>(a, p, tune, st);
             }
-        case 4: return t_launch<T, MODE_FWD, 4>(a, smem, tune, st);
-        default: return t_launch<T, MODE_FWD, 0>(a, smem, tune, st);
+        case 4: return t_launch<T, MODE_FWD, 4>(a, p, tune, st);
+        default: return t_launch<T, MODE_FWD, 0>(a, p, tune, st);
     }
 }
 
@@ -322,26 +505,35 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
     const uint64_t units = (uint64_t)g.outer * (uint64_t)(g.inner / V);
     const uint32_t ctas = 2u * (uint32_t)sm_count;
     if (units >= (1ull << 30) || units > (uint64_t)ctas * (kTSmemUnits - 8)) return p;
+    if (units * (uint64_t)g.C >= (1ull << 32)) return p;      // 32-bit unit indexes
     // What a hand-over costs, in units that one CTA moves meanwhile: about 3 us, from sweeps over R (forward
-    // [128,64,56,56]: 4 rounds of 5576 units 47 us, 8 of 2720 60 us, 16 of 1360 85 us; with gradient 84, 90, 115 us).
-    const uint32_t hand_over = backward ? 700 : 2000;
+    // [128,64,56,56]: 4 rounds of 5576 units 47 us, 8 of 2720 60 us, 16 of 1360 85 us; with gradient 84, 90, 115 us).  With a
+    // gradient and several rounds, two channels side by side hide most of it: [256,512,28,28] 32 rounds of 2792 units 283 us, 29
+    // of 3136 291, 43 of 2096 293, one channel at a time 14 of 6272 300; [128,96,112,112] 48 of 2720 433, 24 of 5432 476;
+    // [128,64,56,56] 8 of 2720 78, 4 of 6272 84; bf16 [128,96,112,112] 24 of 2720 218, 20 of 3408 222, 12 of 5432 242.
     const uint32_t runs = (uint32_t)((units + 7) / 8), C = (uint32_t)g.C;
     uint64_t best = ~0ull;
-    for (uint32_t R = 1; R <= ctas && R <= runs; ++R) {
-        const uint32_t share = 8 * ((runs + R - 1) / R);
-        if (share > kTSmemUnits) continue;
-        const uint32_t teams = std::min(ctas / R, C), rounds = (C + teams - 1) / teams;
-        const uint64_t cost = (uint64_t)rounds * (share + hand_over);
-        if (cost < best) {
-            best = cost;
-            p.R = R;
-            p.teams = teams;
-            p.tile_units = share;
+    bool one_round = false;
+    for (int depth = 1; depth <= (backward ? 2 : 1) && !one_round; ++depth) {
+        const uint32_t hand_over = depth == 2 ? 250 : backward ? 700 : 2000;
+        for (uint32_t R = 1; R <= ctas && R <= runs; ++R) {
+            const uint32_t share = 8 * ((runs + R - 1) / R);
+            if (depth * share > kTSmemUnits) continue;
+            const uint32_t teams = std::min(ctas / R, C), rounds = (C + teams - 1) / teams;
+            one_round |= rounds == 1;
+            const uint64_t cost = (uint64_t)rounds * (share + hand_over);
+            if (cost < best) {
+                best = cost;
+                p.R = R;
+                p.teams = teams;
+                p.tile_units = share;
+                p.lag = depth == 2;
+            }
         }
     }
     if (best == ~0ull) return p;
-    p.gy_units = backward ? std::min(p.tile_units, kTSmemUnits - p.tile_units) : 0u;
-    p.smem_bytes = 16u * (p.tile_units + p.gy_units);
+    p.gy_units = backward && !p.lag ? std::min(p.tile_units, kTSmemUnits - p.tile_units) : 0u;
+    p.smem_bytes = 16u * ((p.lag ? 2 : 1) * p.tile_units + p.gy_units);
     p.ok = true;
     return p;
 }
@@ -372,7 +564,7 @@ cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, in
     a.C = (uint32_t)g.C;
     a.plane_units = (uint32_t)(g.inner / V);
     a.units = (uint32_t)((uint64_t)g.outer * a.plane_units);
-    a.slab_units = (uint64_t)a.C * a.plane_units;
+    a.slab_units = (uint32_t)((uint64_t)a.C * a.plane_units);
     a.R = plan.R;
     a.teams = plan.teams;
     a.tile_units = plan.tile_units;
@@ -381,8 +573,8 @@ cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, in
     a.expected = plan.R + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
     a.div_plane = make_fastdiv(a.plane_units);
     const int extras = io.dist ? 4 : io.pmask ? 2 : io.pcodes ? 3 : 0;
-    return dtype == 0 ? t_launch_mode<float>(a, mode, extras, plan.smem_bytes, tune, st)
-                      : t_launch_mode<__nv_bfloat16>(a, mode, extras, plan.smem_bytes, tune, st);
+    return dtype == 0 ? t_launch_mode<float>(a, mode, extras, plan, tune, st)
+                      : t_launch_mode<__nv_bfloat16>(a, mode, extras, plan, tune, st);
 }
 
 }  // namespace granq

@@ -185,7 +185,8 @@ cudaError_t launch_l2wave(const L2Plan& plan, const QuantIO& io, int mode, int d
 struct TeamPlan {
     bool ok;
     uint32_t R, teams;       // CTAs per team, teams
-    uint32_t tile_units;     // 16-byte units of x one CTA holds
+    bool lag;                // two channels side by side, the hand-over of one behind the quantize walk of the other
+    uint32_t tile_units;     // 16-byte units of x one CTA holds of each
     uint32_t gy_units;       // units of gy it holds beside them
     uint32_t smem_bytes;     // dynamic shared memory per CTA
 };
