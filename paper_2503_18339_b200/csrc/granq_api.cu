@@ -437,6 +437,49 @@ static bool batch_conflict(const granq_fused_desc& a, const granq_fused_desc& b,
     return false;
 }
 
+// Tensors of a list from `first` on that one launch of the resident walk takes together: with a gradient, of the same dims, on
+// workspaces handed over as zero, sharing no memory.  0: none, each is a call of its own.
+static int batch_together(const granq_fused_desc* descs, int first, int n_tensors, int dtype, int channel_axis, int group,
+                          uint32_t flags, void* cuda_stream) {
+    const StagedTuning& t = g_tune;
+    if (flags != GRANQ_FLAG_WORKSPACE_ZEROED || !dtype_ok(dtype) || t.cl_tile_kb || t.cl_r || t.cl_threads || t.cl_load ||
+        t.cl_prefetch || t.cl_kmul || t.cl_pdl || t.col_team == 2)
+        return 0;
+    Geom g;
+    int64_t G;
+    if (!make_geom(descs[first].dims, channel_axis, group, g, G) || G >= (1ll << 28)) return 0;
+    const size_t nb = (size_t)g.E * elt_size(dtype);
+    // bf16 gains nothing (seven of [256,16,32,32] 51.9 / 56.1, three of [16,64,56,56] 21.1 / 21.3)
+    if (dtype != GRANQ_F32 || nb < (8u << 20)) return 0;
+    TeamTensor tensors[kTeamListMax];
+    int n = 0;
+    for (; first + n < n_tensors && n < (int)kTeamListMax; ++n) {
+        const granq_fused_desc& d = descs[first + n];
+        bool fits = d.x && d.gy_opt && d.y && d.gx_opt && d.min_out && d.max_out && d.bits >= 1 && d.bits <= 8 &&
+                    !(((uintptr_t)d.x | (uintptr_t)d.gy_opt | (uintptr_t)d.y | (uintptr_t)d.gx_opt) & 15) &&
+                    check_workspace(d.workspace, d.workspace_bytes, G) == GRANQ_OK &&
+                    !(overlaps(d.x, nb, d.y, nb) || overlaps(d.x, nb, d.gx_opt, nb) || overlaps(d.gy_opt, nb, d.y, nb) ||
+                      overlaps(d.gy_opt, nb, d.gx_opt, nb) || overlaps(d.y, nb, d.gx_opt, nb));
+        for (int k = 0; fits && k < 4; ++k) fits = d.dims[k] == descs[first].dims[k];
+        for (int k = 0; fits && k < n; ++k) fits = !batch_conflict(descs[first + k], d, dtype, channel_axis, group);
+        if (!fits) break;
+        tensors[n] = {QuantIO{d.x, d.gy_opt, d.y, d.gx_opt}, d.bits, carve_workspace(d.workspace, G), d.min_out, d.max_out,
+                      d.scale_opt, d.zp_opt};
+    }
+    int dev = 0, sms = 0;
+    // From 12 MB of x on (two of [256,16,32,32], 16 MB, 37.5 / 27.7; three of [16,64,56,56], 12 MB, 41.9 / 31.6), or 8 MB where
+    // there are 48 MB of them ([256,32,16,16]: six 46.4 / 42.0, three 22.2 / 22.3): of smaller ones the cluster-local kernels run
+    // beside one another and have no hand-over over the GPU (six of [256,64,8,8], 4 MB, 20.2 / 23.3).
+    if (n < 2 || (nb < (12u << 20) && n * nb < (48u << 20)) || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    const TeamPlan p = plan_colteam(dtype, g, tensors[0].io, true, sms, (uint32_t)n);
+    if (!p.ok || !p.lag) return 0;
+    const cudaError_t e = launch_colteam_list(p, tensors, (uint32_t)n, dtype, g, g_tune, (cudaStream_t)cuda_stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) return 0;
+    return e == cudaSuccess ? n : -1;
+}
+
 // Calls that share no memory may run beside one another (their kernels are chained so that the last one's completion is
 // everyone's): a kernel of a few MB is a chain of latencies that leaves most of the chip idle.  Every eighth call, and
 // one that shares memory with a call since, waits for those ahead of it as a call of its own would.  The 19 activations
@@ -449,6 +492,16 @@ int granq_fakequant_fused_batch(const granq_fused_desc* descs, int n_tensors, in
     int first = 0;                 // the calls since the last one that waited, itself included, are [first, i)
     for (int i = 0; i < n_tensors; ++i) {
         const granq_fused_desc& d = descs[i];
+        const int together = batch_together(descs, i, n_tensors, dtype, channel_axis, group, flags, cuda_stream);
+        if (together) {
+            if (together < 0) {
+                if (failed_opt) *failed_opt = i;
+                return GRANQ_ERR_CUDA;
+            }
+            i += together - 1;
+            first = i + 1;
+            continue;
+        }
         bool independent = i > first && i - first < kTogether && dtype_ok(dtype);
         for (int k = first; independent && k < i; ++k)
             if (batch_conflict(descs[k], d, dtype, channel_axis, group)) independent = false;

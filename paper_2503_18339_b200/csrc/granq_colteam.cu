@@ -281,10 +281,33 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
 // place.  The range of channel t is taken and handed to the team before channel t - 1 is quantized, so that the hand-over has
 // that whole walk to complete in; a warp that holds no units does it.  (Forward calls lose by it: their walk is half as long,
 // and twice the rounds cost more than the hand-over: [256,512,28,28] 151 / 163 us.)
+// The channels may be those of a list of tensors of the same dims that share no memory: they follow one another without a
+// launch or a wait between them (fp32, seven of [256,16,32,32] 143.9 -> 90.6 us, six of [128,64,56,56] 475.7 -> 418.6).
 constexpr uint32_t kTWork = kTThreads - 32;
 
-template <typename T, int U>
-__global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a) {
+struct TTensor {
+    const void* x;
+    const void* gy;
+    void* y;
+    void* gx;
+    uint32_t* status;
+    uint32_t* kmin;
+    uint32_t* kmax;
+    uint32_t* counters;
+    float* lo;
+    float* hi;
+    float* s_out;
+    float* z_out;
+    float qmax;
+};
+struct TList {
+    uint32_t n;
+    FastDiv div_C;
+    TTensor t[kTeamListMax];
+};
+
+template <typename T, int U, bool LIST>
+__global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a, const __grid_constant__ TList list) {
     constexpr int V = Pack<T>::V;
     constexpr uint32_t depth = 2;
     extern __shared__ __align__(16) uint4 t_smem[];
@@ -293,7 +316,8 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
     __shared__ uint32_t s_bad, s_last;      // the job whose hand-over ran out of its wait; is this the last CTA?
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t team = blockIdx.x / a.R, rank = blockIdx.x - team * a.R;
-    const uint32_t jobs = (a.C - team + a.teams - 1) / a.teams;      // channels of this team: team, team + teams, ...
+    // channels of this team: team, team + teams, ... of all tensors' channels one after the other
+    const uint32_t total = LIST ? list.n * a.C : a.C, jobs = team < total ? (total - team + a.teams - 1) / a.teams : 0u;
     // this CTA's share: whole runs of 8 units (128 bytes) of the channel's units laid end to end
     const uint32_t runs = (a.units + 7) / 8;
     const uint32_t q0 = 8 * (uint32_t)(((uint64_t)rank * runs) / a.R);
@@ -315,11 +339,11 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
             at += dwrap;
         }
     };
-    const uint4* xg = reinterpret_cast<const uint4*>(a.x);
-    const uint4* gyg = reinterpret_cast<const uint4*>(a.gy);
-    uint4* yg = reinterpret_cast<uint4*>(a.y);
-    uint4* gxg = reinterpret_cast<uint4*>(a.gx);
-    const float qmax = a.qmax;
+    auto job = [&](uint32_t j, uint32_t& t, uint32_t& c) {
+        t = 0;
+        c = team + j * a.teams;
+        if constexpr (LIST) list.div_C.divmod(c, t, c);
+    };
 
     // ---- Eq. 4: range of this CTA's share of job j, from its tile to the warps' keys ----
     auto reduce = [&](uint32_t j, const uint4* tile) {
@@ -341,16 +365,18 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
     };
     // ---- the last warp: publish job j's keys, wait (bounded) until the whole team has; Eq. 5 ----
     auto hand_over = [&](uint32_t j) {
-        const uint32_t c = team + j * a.teams;
+        uint32_t ti, c;
+        job(j, ti, c);
+        const TTensor& t = list.t[ti];
         const uint32_t ka = __reduce_max_sync(kFullMask, lane < kTWork / 32 ? s_kmn[j & 1][lane] : 0u);
         const uint32_t kb = __reduce_max_sync(kFullMask, lane < kTWork / 32 ? s_kmx[j & 1][lane] : 0u);
         if (lane != 0) return;
-        atomicMax(a.kmin + c, ka);
-        atomicMax(a.kmax + c, kb);
-        t_arrive_release(a.counters + c);
+        atomicMax(t.kmin + c, ka);
+        atomicMax(t.kmax + c, kb);
+        t_arrive_release(t.counters + c);
         uint32_t ready = 0;
         for (uint32_t i = 0; i < a.spin_limit; ++i) {
-            if (t_ld_acquire(a.counters + c) >= a.expected) {
+            if (t_ld_acquire(t.counters + c) >= a.expected) {
                 ready = 1;
                 break;
             }
@@ -358,24 +384,32 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
         }
         if (!ready) {
             s_bad = j;
-            atomicExch(a.status, kTStatusTimeout);
+            for (uint32_t k = 0; k < list.n; ++k) atomicExch(list.t[k].status, kTStatusTimeout);
             return;
         }
         float lo, hi;
-        const GroupParam gp = group_param_from_keys(a.kmin, a.kmax, c, qmax, lo, hi);
+        const GroupParam gp = group_param_from_keys(t.kmin, t.kmax, c, t.qmax, lo, hi);
         s_par[j & 1] = gp;
         if (rank == 0) {
-            a.lo[c] = lo;
-            a.hi[c] = hi;
-            if (a.s_out) a.s_out[c] = gp.s;
-            if (a.z_out) a.z_out[c] = gp.z;
+            t.lo[c] = lo;
+            t.hi[c] = hi;
+            if (t.s_out) t.s_out[c] = gp.s;
+            if (t.z_out) t.z_out[c] = gp.z;
         }
     };
     // ---- Eq. 1, clamp, Eq. 6, STE of job j from its tile; the copies of job j + depth follow on the heels ----
     auto quantize = [&](uint32_t j, uint4* tile) {
         const GroupParam g = s_par[j & 1];
         const bool more = j + depth < jobs;
-        const uint32_t ahead = depth * a.teams * a.plane_units;
+        uint32_t ti, c;
+        job(more ? j + depth : j, ti, c);
+        const uint4* xn = reinterpret_cast<const uint4*>(list.t[ti].x) + (size_t)c * a.plane_units;
+        job(j, ti, c);
+        const size_t base = (size_t)c * a.plane_units;
+        const uint4* gyg = reinterpret_cast<const uint4*>(list.t[ti].gy) + base;
+        uint4* yg = reinterpret_cast<uint4*>(list.t[ti].y) + base;
+        uint4* gxg = reinterpret_cast<uint4*>(list.t[ti].gx) + base;
+        const float qmax = list.t[ti].qmax;
         auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint32_t at) {
             Pack<T> py, pgx;
             uint32_t cb[V / 4], mb[V / 4];
@@ -383,7 +417,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
             st_stream_16(yg + at, py.raw);
             st_stream_16(gxg + at, pgx.raw);
         };
-        uint32_t at = first + (team + j * a.teams) * a.plane_units, off = off0, i = 0;
+        uint32_t at = first, off = off0, i = 0;
         for (; i + U <= cnt; i += U) {
             Pack<T> px[U], pg[U];
             uint32_t w[U];
@@ -396,7 +430,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
             }
             if (more) {
 #pragma unroll
-                for (int k = 0; k < U; ++k) t_cp_async_16(tile + (i + k) * kTWork, xg + (w[k] + ahead));
+                for (int k = 0; k < U; ++k) t_cp_async_16(tile + (i + k) * kTWork, xn + w[k]);
             }
 #pragma unroll
             for (int k = 0; k < U; ++k) emit(px[k], pg[k], w[k]);
@@ -405,7 +439,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
             Pack<T> px, pg;
             pg.raw = ld_stream_16(gyg + at);
             px.raw = tile[i * kTWork];
-            if (more) t_cp_async_16(tile + i * kTWork, xg + (at + ahead));
+            if (more) t_cp_async_16(tile + i * kTWork, xn + at);
             emit(px, pg, at);
             advance(at, off);
         }
@@ -413,14 +447,15 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
 
     if (tid == 0) s_bad = 0xFFFFFFFFu;
     // the first copies; those of the later jobs are sent from the quantize walk
-    for (uint32_t j = 0; j < depth; ++j) {
+    for (uint32_t j = 0; j < depth && j < jobs; ++j) {
+        uint32_t ti, c;
+        job(j, ti, c);
+        const uint4* xg = reinterpret_cast<const uint4*>(list.t[ti].x) + (size_t)c * a.plane_units;
         uint4* tile = t_smem + j * a.tile_units + tid;
-        uint32_t at = first + (team + j * a.teams) * a.plane_units, off = off0;
-        if (j < jobs) {
-            for (uint32_t i = 0; i < cnt; ++i) {
-                t_cp_async_16(tile + i * kTWork, xg + at);
-                advance(at, off);
-            }
+        uint32_t at = first, off = off0;
+        for (uint32_t i = 0; i < cnt; ++i) {
+            t_cp_async_16(tile + i * kTWork, xg + at);
+            advance(at, off);
         }
     }
     for (uint32_t t = 0; t <= jobs; ++t) {
@@ -439,34 +474,43 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
         return;
     }
 
-    // ---- leave the workspace as it was found: the last CTA to finish clears keys and counters ----
+    // ---- leave the workspaces as they were found: the last CTA to finish clears keys and counters ----
     __syncthreads();
     if (tid == 0) {
         __threadfence();
-        s_last = (atomicAdd(a.counters + a.C, 1u) == gridDim.x - 1) ? 1u : 0u;
+        s_last = (atomicAdd(list.t[0].counters + a.C, 1u) == gridDim.x - 1) ? 1u : 0u;
     }
     __syncthreads();
     if (s_last) {
-        for (uint32_t i = tid; i < a.C; i += kTThreads) {
-            a.kmin[i] = 0;
-            a.kmax[i] = 0;
-        }
-        for (uint32_t i = tid; i <= a.C; i += kTThreads) a.counters[i] = 0;
+        for (uint32_t t = 0; t < list.n; ++t)
+            for (uint32_t i = tid; i <= a.C; i += kTThreads) {
+                if (i < a.C) list.t[t].kmin[i] = list.t[t].kmax[i] = 0;
+                list.t[t].counters[i] = 0;
+            }
     }
 }
 
 template <typename T, int MODE, int EXTRAS, int BITS = 8>
 cudaError_t t_launch(const TArgs& args, const TeamPlan& p, const StagedTuning& tune, cudaStream_t st) {
+    auto kern = colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2), BITS>;
+    const cudaError_t e = allow_smem(kern, kTSmemUnits * 16);
+    if (e != cudaSuccess) return e;
+    void* params[] = {(void*)&args};
+    return launch_cooperative((const void*)kern, args.R * args.teams, kTThreads, params, p.smem_bytes, tune, st);
+}
+
+template <typename T>
+cudaError_t t_launch_lag(const TArgs& args, const TList& list, const TeamPlan& p, const StagedTuning& tune, cudaStream_t st) {
     auto launch = [&](auto kern) -> cudaError_t {
         const cudaError_t e = allow_smem(kern, kTSmemUnits * 16);
         if (e != cudaSuccess) return e;
-        void* params[] = {(void*)&args};
+        void* params[] = {(void*)&args, (void*)&list};
         return launch_cooperative((const void*)kern, args.R * args.teams, kTThreads, params, p.smem_bytes, tune, st);
     };
-    if constexpr (MODE == MODE_BOTH) {
-        if (p.lag) return launch(colteam_lag_kernel<T, 2>);
+    if constexpr (sizeof(T) == 4) {
+        if (list.n > 1) return launch(colteam_lag_kernel<T, 2, true>);
     }
-    return launch(colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2), BITS>);
+    return list.n == 1 ? launch(colteam_lag_kernel<T, 2, false>) : cudaErrorInvalidValue;      // lists are fp32
 }
 
 template <typename T>
@@ -494,12 +538,12 @@ cudaError_t t_launch_mode(const TArgs& a, int mode, int extras, const TeamPlan& 
 
 // Team size: the number of CTAs R for which rounds x (share of one CTA + what a hand-over costs) is smallest, the
 // share fitting the shared memory of one of two CTAs per SM.
-TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count) {
+TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count, uint32_t tensors) {
     TeamPlan p{};
     p.ok = false;
     const uint32_t V = dtype == 0 ? 4 : 8;
     // whole units; codes and masks are written 8 elements at a time
-    if (g.inner % V != 0 || g.C >= (1ll << 28) || g.inner >= (1ll << 28)) return p;
+    if (g.inner % V != 0 || g.C * tensors >= (1ll << 28) || g.inner >= (1ll << 28)) return p;
     if ((io.pmask || io.pcodes) && g.inner % 8 != 0) return p;
     if (io.codes || io.mask) return p;
     const uint64_t units = (uint64_t)g.outer * (uint64_t)(g.inner / V);
@@ -510,12 +554,13 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
     // [128,64,56,56]: 4 rounds of 5576 units 47 us, 8 of 2720 60 us, 16 of 1360 85 us; with gradient 84, 90, 115 us).  With a
     // gradient and several rounds, two channels side by side hide most of it: [256,512,28,28] 32 rounds of 2792 units 283 us, 29
     // of 3136 291, 43 of 2096 293, one channel at a time 14 of 6272 300; [128,96,112,112] 48 of 2720 433, 24 of 5432 476;
-    // [128,64,56,56] 8 of 2720 78, 4 of 6272 84; bf16 [128,96,112,112] 24 of 2720 218, 20 of 3408 222, 12 of 5432 242.
-    const uint32_t runs = (uint32_t)((units + 7) / 8), C = (uint32_t)g.C;
+    // [128,64,56,56] 8 of 2720 78, 4 of 6272 84; bf16 [128,96,112,112] 24 of 2720 218, 20 of 3408 222, 12 of 5432 242, but
+    // [256,512,28,28] 16 of 2792 163, one channel at a time 7 of 6272 158.
+    const uint32_t runs = (uint32_t)((units + 7) / 8), C = tensors * (uint32_t)g.C;
     uint64_t best = ~0ull;
     bool one_round = false;
     for (int depth = 1; depth <= (backward ? 2 : 1) && !one_round; ++depth) {
-        const uint32_t hand_over = depth == 2 ? 250 : backward ? 700 : 2000;
+        const uint32_t hand_over = depth == 2 ? (dtype == 0 ? 250 : 340) : backward ? 700 : 2000;
         for (uint32_t R = 1; R <= ctas && R <= runs; ++R) {
             const uint32_t share = 8 * ((runs + R - 1) / R);
             if (depth * share > kTSmemUnits) continue;
@@ -538,10 +583,38 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
     return p;
 }
 
+cudaError_t launch_colteam_list(const TeamPlan& plan, const TeamTensor* tensors, uint32_t n, int dtype, const Geom& g,
+                                const StagedTuning& tune, cudaStream_t st) {
+    TArgs a{};
+    a.C = (uint32_t)g.C;
+    a.plane_units = (uint32_t)(g.inner / (dtype == 0 ? 4 : 8));
+    a.units = (uint32_t)((uint64_t)g.outer * a.plane_units);
+    a.slab_units = (uint32_t)((uint64_t)a.C * a.plane_units);
+    a.R = plan.R;
+    a.teams = plan.teams;
+    a.tile_units = plan.tile_units;
+    a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kTSpinLimit;
+    a.expected = plan.R + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
+    a.div_plane = make_fastdiv(a.plane_units);
+    TList list{};
+    list.n = n;
+    list.div_C = make_fastdiv(a.C);
+    for (uint32_t i = 0; i < n; ++i) {
+        const TeamTensor& t = tensors[i];
+        list.t[i] = {t.io.x, t.io.gy, t.io.y, t.io.gx, t.ws.status, t.ws.kmin, t.ws.kmax, t.ws.counters, t.lo, t.hi,
+                     t.s_opt, t.z_opt, (float)((1 << t.bits) - 1)};
+    }
+    return dtype == 0 ? t_launch_lag<float>(a, list, plan, tune, st) : t_launch_lag<__nv_bfloat16>(a, list, plan, tune, st);
+}
+
 cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
                            const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,
                            const StagedTuning& tune, cudaStream_t st) {
     const uint32_t V = dtype == 0 ? 4 : 8;
+    if (plan.lag) {
+        const TeamTensor one{io, bits, ws, lo, hi, s_opt, z_opt};
+        return launch_colteam_list(plan, &one, 1, dtype, g, tune, st);
+    }
     TArgs a{};
     a.x = io.x;
     a.gy = io.gy;

@@ -190,13 +190,25 @@ struct TeamPlan {
     uint32_t gy_units;       // units of gy it holds beside them
     uint32_t smem_bytes;     // dynamic shared memory per CTA
 };
-TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count);
+// tensors: that many of these dims in one launch
+TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count, uint32_t tensors = 1);
 // does the column walk take this form rather than the waves?
 bool team_over_waves(const TeamPlan& plan, const Geom& g, const StagedTuning& tune);
 // may be refused: launch_cooperative()
 cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
                            const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,
                            const StagedTuning& tune, cudaStream_t st);
+// a list of fp32 tensors of the same dims that share no memory, with a gradient (or one tensor of either type); the plan has to
+// be one with `lag`
+constexpr uint32_t kTeamListMax = 16;
+struct TeamTensor {
+    QuantIO io;
+    int bits;
+    Workspace ws;
+    float *lo, *hi, *s_opt, *z_opt;
+};
+cudaError_t launch_colteam_list(const TeamPlan& plan, const TeamTensor* tensors, uint32_t n, int dtype, const Geom& g,
+                                const StagedTuning& tune, cudaStream_t st);
 struct ColPlan {
     bool ok;
     uint32_t cw;             // channels per wave
