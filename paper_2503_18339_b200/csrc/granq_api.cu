@@ -136,6 +136,18 @@ cudaError_t launch_held(const TeamPlan& tp, const ClusterPlan& kp, const QuantIO
     return launch_cluster(kp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, g_tune, st);
 }
 
+// Where a call would take two passes or the L2-resident waves, not because it asked to: one launch that holds the tensor on
+// chip (what it gains stands at the kernel).
+HoldPlan prefer_hold(int dtype, const Geom& g, const QuantIO& io, uint32_t flags) {
+    HoldPlan none{};
+    if (flags & GRANQ_FLAG_FORCE_TWO_PASS) return none;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return none;
+    return plan_hold(dtype, g, io, sms);
+}
+
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -259,7 +271,9 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
     // keep that word true for the next call, after.
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     kp.zero_status = !zeroed && kp.clears_status;
-    bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS;
+    const HoldPlan hp = plan == PLAN_TWO_PASS || (plan == PLAN_L2WAVE && !(flags & GRANQ_FLAG_FORCE_L2WAVE))
+                            ? prefer_hold(dtype, g, io, flags) : HoldPlan{};
+    bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS || hp.ok;
     TeamPlan tp{};
     if (plan == PLAN_CLUSTER) tp = prefer_team(dtype, g, io, gy_opt != nullptr, flags);
     cudaError_t e = cudaSuccess;
@@ -284,7 +298,11 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
         }
     } else if (plan == PLAN_STAGED) {
         e = launch_staged(sp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
+    } else if (hp.ok && (e = launch_hold(hp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st)) !=
+                            cudaErrorCooperativeLaunchTooLarge) {
+        // done
     } else if (plan == PLAN_L2WAVE) {
+        keeps_zero = false;
         e = launch_l2wave(lp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else if (plan == PLAN_COLWALK) {
         e = launch_colwalk(cp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
@@ -293,6 +311,7 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
         if (e == cudaSuccess && (scale_opt || zp_opt))
             e = launch_params(min_out, max_out, G, bits, scale_opt, zp_opt, st);
     } else {
+        keeps_zero = false;
         e = two_pass();
     }
     if (e == cudaSuccess && zeroed && !keeps_zero)
@@ -577,8 +596,14 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
         return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     }
-    if (e == cudaSuccess && !(zeroed && cp.ok)) e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
+    const HoldPlan hp = cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
+    if (e == cudaSuccess && !(zeroed && (cp.ok || hp.ok))) e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
+    if (hp.ok) {
+        e = launch_hold(hp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
+        if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_status(e);
+        e = cudaSuccess;
+    }
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {

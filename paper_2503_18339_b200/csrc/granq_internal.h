@@ -220,6 +220,18 @@ cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int
                            const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,
                            const StagedTuning& tune, cudaStream_t st);
 
+// ---- range and quantization of a tensor held in shared memory piece by piece (granq_hold.cu) ----
+struct HoldPlan {
+    bool ok;
+    uint32_t ctas, share;    // CTAs, 16-byte units of one
+    uint32_t held, planes;   // of those, kept in shared memory; planes it can cut through
+};
+HoldPlan plan_hold(int dtype, const Geom& g, const QuantIO& io, int sm_count);
+// may be refused: launch_cooperative()
+cudaError_t launch_hold(const HoldPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
+                        const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt, const StagedTuning& tune,
+                        cudaStream_t st);
+
 // ---- channels-last kernels (the channel is the innermost axis: one 16-byte unit holds V channels of a row) ----
 bool plan_rows(int dtype, const Geom& g, const QuantIO& io);
 struct RowsCut {

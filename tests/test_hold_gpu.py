@@ -1,0 +1,92 @@
+"""The kernel that holds a tensor on chip piece by piece (planes and slabs that are not whole 16-byte units, one group over the
+whole tensor) against the CPU oracle, bit for bit: pieces that begin and end inside planes, planes shorter than a thread's run
+and longer than a piece, units that straddle two planes, fewer units than threads, one group that stays on chip and one of
+which a part is read again - forward, with a gradient, with the distortion sums; the workspace zero again afterwards."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import assert_parity, make_case, to_dev, to_np
+from oracle import granq_oracle as orc
+from test_parity_gpu import b, knobs  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+# dims, group mode; the number of elements is a multiple of 8
+CASES = [
+    ((8, 3, 3, 3), 0),          # fewer units than one CTA has threads
+    ((8, 75, 5, 7), 0),         # planes shorter than a thread's run of units, an odd number of channels
+    ((8, 301, 7, 7), 0),        # several planes to a thread
+    ((16, 5, 27, 27), 0),       # planes of several runs
+    ((8, 3, 111, 111), 0),      # a plane over many pieces
+    ((24, 75, 27, 27), 0),      # several units to a thread
+    ((3, 7, 9, 24), 2),         # one group, fewer units than one CTA has threads
+    ((5, 11, 40, 50), 2),       # one group, pieces that do not come out even
+    ((32, 128, 28, 29), 2),     # one group over several units a thread
+    ((3, 2, 256, 256), 1),      # planes of whole units, too long for a cluster to hold
+]
+
+
+@pytest.mark.parametrize("shape,mode", CASES, ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else f"g{v}")
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_held_tensor(b, shape, mode, dtype):
+    x, gy = make_case(shape, seed=sum(shape), dtype=dtype, relu=shape[0] % 2 == 0)
+    bits = 2 + sum(shape) % 7
+    ref = orc.fused(x, bits, gy=gy, group_mode=mode)
+    xd, gyd = to_dev(x), to_dev(gy)
+    ws = b.make_workspace(xd, group=mode, zeroed=True)
+    new = lambda: b.FakeQuantOut(workspace=ws)
+    clean = lambda: b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
+    for _ in range(2):
+        got = b.granq_fakequant_fused(xd, bits, gy=gyd, group=mode, out=new(), want_params=True, flags=b.FLAG_WORKSPACE_ZEROED)
+        assert clean()
+        assert_parity(got, ref, shape, 1, mode, backward=True)
+    got = b.granq_fakequant_fused(xd, bits, group=mode, out=new(), flags=b.FLAG_WORKSPACE_ZEROED)
+    assert clean()
+    assert_parity(got, ref, shape, 1, mode, backward=False)
+    got = b.granq_fakequant_fused_stats(xd, bits, group=mode, out=new(), flags=b.FLAG_WORKSPACE_ZEROED)
+    assert clean()
+    assert_parity(got, ref, shape, 1, mode, backward=False)
+    # fp32 inside a pack, fp64 beyond: about 8 roundings of 2^-24 of a sum of same-signed terms
+    assert np.allclose(to_np(got.sums), orc.distortion_sums(x, ref.y), rtol=1e-6, atol=0)
+    dirty = b.FakeQuantOut(workspace=b.make_workspace(xd, group=mode).fill_(255))
+    assert_parity(b.granq_fakequant_fused(xd, bits, gy=gyd, group=mode, out=dirty), ref, shape, 1, mode, backward=True)
+
+
+@pytest.mark.parametrize("dtype,shape", [("f32", (96, 128, 28, 28)), ("bf16", (192, 128, 28, 28))])
+def test_one_group_beyond_what_stays_on_chip(b, dtype, shape):
+    x, gy = make_case(shape, seed=3, dtype=dtype)
+    ref = orc.fused(x, 4, gy=gy, group_mode=2)
+    xd, gyd = to_dev(x), to_dev(gy)
+    assert_parity(b.granq_fakequant_fused(xd, 4, gy=gyd, group=2), ref, shape, 1, 2, backward=True)
+    assert_parity(b.granq_fakequant_fused(xd, 4, group=2), ref, shape, 1, 2, backward=False)
+    got = b.granq_fakequant_fused_stats(xd, 4, group=2)
+    assert_parity(got, ref, shape, 1, 2, backward=False)
+    assert np.allclose(to_np(got.sums), orc.distortion_sums(x, ref.y), rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("stats", [False, True])
+def test_a_hand_over_that_never_completes_is_reported(b, knobs, stats):
+    x, _ = make_case((8, 75, 5, 7), seed=1)
+    xd = to_dev(x)
+    call = b.granq_fakequant_fused_stats if stats else b.granq_fakequant_fused
+    knobs(extra_arrivals=1, spin_limit=500)
+    assert b.workspace_status(call(xd, 4).workspace) == b.ERR_TIMEOUT
+    knobs(extra_arrivals=0, spin_limit=0)
+    got = call(xd, 4)
+    assert b.workspace_status(got.workspace) == b.OK
+    assert_parity(got, orc.fused(x, 4), x.shape, 1, 0, backward=False)
+
+
+@pytest.mark.parametrize("shape,mode", [((24, 75, 27, 27), 0), ((5, 11, 40, 50), 2), ((3, 2, 256, 256), 1)])
+def test_a_refused_cooperative_launch_falls_back(b, knobs, shape, mode):
+    x, gy = make_case(shape, seed=6)
+    ref = orc.fused(x, 4, gy=gy, group_mode=mode)
+    xd, gyd = to_dev(x), to_dev(gy)
+    ws = b.make_workspace(xd, group=mode, zeroed=True)
+    b.tune(b.KNOB_TEST_COOP_CTAS, 1)
+    got = b.granq_fakequant_fused(xd, 4, gy=gyd, group=mode, out=b.FakeQuantOut(workspace=ws), flags=b.FLAG_WORKSPACE_ZEROED)
+    assert_parity(got, ref, shape, 1, mode, backward=True)
+    got = b.granq_fakequant_fused_stats(xd, 4, group=mode, out=b.FakeQuantOut(workspace=ws), flags=b.FLAG_WORKSPACE_ZEROED)
+    assert_parity(got, ref, shape, 1, mode, backward=False)
+    assert b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
