@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     const float qmax = a.qmax;
     DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS = 4)
     dacc.reset();
+    let_the_kernel_behind_start();
 
     // the first channel's copies; those of the later ones are sent from the quantize walk
     {
@@ -446,6 +447,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
     };
 
     if (tid == 0) s_bad = 0xFFFFFFFFu;
+    let_the_kernel_behind_start();
     // the first copies; those of the later jobs are sent from the quantize walk
     for (uint32_t j = 0; j < depth && j < jobs; ++j) {
         uint32_t ti, c;

@@ -111,6 +111,7 @@ template <typename T, int V>
 __global__ void __launch_bounds__(kThreads, 8) range_flat_kernel(const T* __restrict__ x, FlatGeom g,
                                                               uint32_t* __restrict__ kmin,
                                                               uint32_t* __restrict__ kmax, RangeEnd end) {
+    after_the_kernel_ahead();
     __shared__ TileBase s_base;
     WarpRun run{kNoGroup, 0u, 0u};
     for (int64_t tile = blockIdx.x; tile < g.ntiles; tile += gridDim.x) {
@@ -167,6 +168,7 @@ __global__ void __launch_bounds__(kThreads) range_rows_kernel(const uint4* __res
                                                               uint32_t inner, FastDiv div_plane, FastDiv div_C,
                                                               uint32_t groups, uint32_t* __restrict__ kmin,
                                                               uint32_t* __restrict__ kmax, RangeEnd end) {
+    after_the_kernel_ahead();
     constexpr int V = Pack<T>::V;
     __shared__ uint32_t s_kmn[kRangeSmemGroups], s_kmx[kRangeSmemGroups];
     const bool combine = groups <= kRangeSmemGroups;       // else: straight to the global keys
@@ -275,6 +277,7 @@ __global__ void __launch_bounds__(kThreads) range_cols_kernel(const uint4* __res
                                                               uint32_t outer, uint32_t chunks, FastDiv div_ncol,
                                                               FastDiv div_plane, uint32_t* __restrict__ kmin,
                                                               uint32_t* __restrict__ kmax, RangeEnd end) {
+    after_the_kernel_ahead();
     constexpr int V = Pack<T>::V;
     __shared__ uint32_t s_kmn[kColTab], s_kmx[kColTab];
     for (uint32_t t = threadIdx.x; t < kColTab; t += kThreads) {
@@ -369,12 +372,14 @@ __global__ void __launch_bounds__(kThreads) range_cols_kernel(const uint4* __res
 __global__ void finalize_range_kernel(const uint32_t* __restrict__ kmin, const uint32_t* __restrict__ kmax,
                                       int64_t G, float* __restrict__ lo, float* __restrict__ hi, int bits,
                                       float* __restrict__ s_opt, float* __restrict__ z_opt) {
+    after_the_kernel_ahead();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < G) finalize_group(kmin, kmax, i, lo, hi, bits, s_opt, z_opt);
 }
 
 __global__ void params_kernel(const float* __restrict__ lo, const float* __restrict__ hi, int64_t G, int bits,
                               float* __restrict__ s_opt, float* __restrict__ z_opt) {
+    after_the_kernel_ahead();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= G) return;
     QParam p = make_qparam(__fadd_rn(lo[i], 0.0f), __fadd_rn(hi[i], 0.0f), (float)((1 << bits) - 1));
@@ -458,6 +463,7 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
                                                               FlatGeom g, float qmax,
                                                               const float* __restrict__ lo,
                                                               const float* __restrict__ hi) {
+    after_the_kernel_ahead();
     __shared__ TileBase s_base;
     __shared__ float s_tab_s[kTableMax], s_tab_z[kTableMax], s_tab_r[kTableMax];
     constexpr bool kParts = kFlatParts<V, MODE, EXTRAS, RAGGED>;
@@ -701,6 +707,7 @@ template <typename T, int V>
 __global__ void __launch_bounds__(kThreads) bwd_packmask_kernel(const T* __restrict__ gy,
                                                                 const uint32_t* __restrict__ pmask,
                                                                 T* __restrict__ gx, int64_t E) {
+    after_the_kernel_ahead();
     const int64_t u0 = (int64_t)blockIdx.x * kThreads * kUnroll;
     int64_t e[kUnroll];
     Pack<T> pg[kUnroll];
@@ -733,6 +740,7 @@ __global__ void __launch_bounds__(kThreads) bwd_packmask_kernel(const T* __restr
 template <typename T, int V>
 __global__ void __launch_bounds__(kThreads) distortion_kernel(const T* __restrict__ x, const T* __restrict__ q,
                                                               int64_t E, double* __restrict__ sums) {
+    after_the_kernel_ahead();
     DistAcc acc;
     acc.reset();
     const int64_t nunits = E / V;
@@ -776,6 +784,7 @@ __global__ void __launch_bounds__(kThreads) dequant_strings_kernel(const uint32_
                                                                    uint32_t nstrings, uint32_t last_word, uint32_t inner,
                                                                    FastDiv div_inner, FastDiv div_C,
                                                                    const float* __restrict__ s, const float* __restrict__ z) {
+    after_the_kernel_ahead();
     constexpr uint32_t kField = (1u << BITS) - 1u;
     constexpr int kFly = 2;
     const uint32_t t0 = blockIdx.x * (kThreads * kFly) + threadIdx.x;
@@ -846,6 +855,7 @@ __global__ void __launch_bounds__(kThreads) dequant_packed_kernel(const uint32_t
                                                                   int64_t C, int bits,
                                                                   const float* __restrict__ s,
                                                                   const float* __restrict__ z) {
+    after_the_kernel_ahead();
     const int64_t nunits = E / V;
     const uint32_t field = (1u << bits) - 1u;
     for (int64_t u = (int64_t)blockIdx.x * kThreads + threadIdx.x; u < nunits; u += (int64_t)gridDim.x * kThreads) {
@@ -922,29 +932,27 @@ cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t*
         const uint32_t chunks = std::max<uint32_t>(1, std::min<uint32_t>((2 * cap + ncol - 1) / ncol, outer / 4));
         constexpr int U = VF == 4 ? 8 : 4;
         if (vec)
-            range_cols_kernel<T, true, U><<<ncol * chunks, kThreads, 0, st>>>(
-                (const uint4*)x, slab_units, outer, chunks, make_fastdiv(ncol), make_fastdiv((uint32_t)(g.inner / VF)), kmin,
+            launch_after(range_cols_kernel<T, true, U>, ncol * chunks, kThreads, 0, st, (const uint4*)x, slab_units, outer, chunks, make_fastdiv(ncol), make_fastdiv((uint32_t)(g.inner / VF)), kmin,
                 kmax, end);
         else
-            range_cols_kernel<T, false, U><<<ncol * chunks, kThreads, 0, st>>>(
-                (const uint4*)x, slab_units, outer, chunks, make_fastdiv(ncol), make_fastdiv((uint32_t)g.inner), kmin, kmax, end);
+            launch_after(range_cols_kernel<T, false, U>, ncol * chunks, kThreads, 0, st, (const uint4*)x, slab_units, outer, chunks, make_fastdiv(ncol), make_fastdiv((uint32_t)g.inner), kmin, kmax, end);
     } else if (rows_ok) {
         const uint32_t n_units = (uint32_t)(g.E / VF);
         int64_t rows = ((int64_t)n_units + 127) / 128, ctas = (rows + 2 * (kThreads / 32) - 1) / (2 * (kThreads / 32));
         const int64_t cap = (int64_t)range_rows_ctas();                 // 4 resident CTAs per SM at 64 registers
         int rgrid = (int)(ctas < cap ? ctas : cap);
         if (vec)
-            range_rows_kernel<T, true><<<rgrid, kThreads, 0, st>>>((const uint4*)x, n_units, (uint32_t)g.inner,
+            launch_after(range_rows_kernel<T, true>, rgrid, kThreads, 0, st, (const uint4*)x, n_units, (uint32_t)g.inner,
                                                                    make_fastdiv((uint32_t)(g.inner / VF)),
                                                                    make_fastdiv((uint32_t)g.C), (uint32_t)g.C, kmin, kmax, end);
         else
-            range_rows_kernel<T, false><<<rgrid, kThreads, 0, st>>>((const uint4*)x, n_units, (uint32_t)g.inner,
+            launch_after(range_rows_kernel<T, false>, rgrid, kThreads, 0, st, (const uint4*)x, n_units, (uint32_t)g.inner,
                                                                     make_fastdiv((uint32_t)g.inner),
                                                                     make_fastdiv((uint32_t)g.C), (uint32_t)g.C, kmin, kmax, end);
     } else if (vec)
-        range_flat_kernel<T, VF><<<grid, kThreads, 0, st>>>((const T*)x, f, kmin, kmax, end);
+        launch_after(range_flat_kernel<T, VF>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end);
     else
-        range_flat_kernel<T, 1><<<grid, kThreads, 0, st>>>((const T*)x, f, kmin, kmax, end);
+        launch_after(range_flat_kernel<T, 1>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end);
     return cudaGetLastError();
 }
 
@@ -978,23 +986,19 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
     if constexpr (MODE == MODE_FWD) {
         if ((vec || ragged) && pack_only && g.E % 32 == 0) {       // whole words of codes: the byte-wise writer
             if (vec)
-                quant_flat_kernel<T, VF, MODE, 3, true><<<grid, kThreads, 0, st>>>(
-                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                launch_after(quant_flat_kernel<T, VF, MODE, 3, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                     io.code_bits, f, qmax, lo, hi);
             else
-                quant_flat_kernel<T, VF, MODE, 3, true, true><<<grid, kThreads, 0, st>>>(
-                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                launch_after(quant_flat_kernel<T, VF, MODE, 3, true, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                     io.code_bits, f, qmax, lo, hi);
             return cudaGetLastError();
         }
         if ((vec || ragged) && pack_only) {
             if (vec)
-                quant_flat_kernel<T, VF, MODE, 1, true><<<grid, kThreads, 0, st>>>(
-                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                launch_after(quant_flat_kernel<T, VF, MODE, 1, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                     io.code_bits, f, qmax, lo, hi);
             else
-                quant_flat_kernel<T, VF, MODE, 1, true, true><<<grid, kThreads, 0, st>>>(
-                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                launch_after(quant_flat_kernel<T, VF, MODE, 1, true, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                     io.code_bits, f, qmax, lo, hi);
             return cudaGetLastError();
         }
@@ -1002,46 +1006,40 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
                                io.pmask == nullptr && io.pcodes == nullptr;
         if ((vec || ragged) && dist_only) {
             if (vec)
-                quant_flat_kernel<T, VF, MODE, 4><<<grid, kThreads, 0, st>>>(
-                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                launch_after(quant_flat_kernel<T, VF, MODE, 4>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                     io.code_bits, f, qmax, lo, hi);
             else
-                quant_flat_kernel<T, VF, MODE, 4, false, true><<<grid, kThreads, 0, st>>>(
-                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                launch_after(quant_flat_kernel<T, VF, MODE, 4, false, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                     io.code_bits, f, qmax, lo, hi);
             return cudaGetLastError();
         }
         if ((vec || ragged) && pmask_only) {
             if (vec)
-                quant_flat_kernel<T, VF, MODE, 2><<<grid, kThreads, 0, st>>>(
-                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                launch_after(quant_flat_kernel<T, VF, MODE, 2>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                     io.code_bits, f, qmax, lo, hi);
             else
-                quant_flat_kernel<T, VF, MODE, 2, false, true><<<grid, kThreads, 0, st>>>(
-                    (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+                launch_after(quant_flat_kernel<T, VF, MODE, 2, false, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                     io.code_bits, f, qmax, lo, hi);
             return cudaGetLastError();
         }
     }
     if (ragged) {
         if (extras)
-            quant_flat_kernel<T, VF, MODE, 1, false, true><<<grid, kThreads, 0, st>>>(
-                (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+            launch_after(quant_flat_kernel<T, VF, MODE, 1, false, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                 io.code_bits, f, qmax, lo, hi);
         else
-            quant_flat_kernel<T, VF, MODE, 0, false, true><<<grid, kThreads, 0, st>>>(
-                (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
+            launch_after(quant_flat_kernel<T, VF, MODE, 0, false, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
                 io.code_bits, f, qmax, lo, hi);
         return cudaGetLastError();
     }
     if (vec && extras)
-        quant_flat_kernel<T, VF, MODE, 1><<<grid, kThreads, 0, st>>>((const T*)io.x, (const T*)io.gy, (T*)io.y,
+        launch_after(quant_flat_kernel<T, VF, MODE, 1>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y,
                                                                         (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes, io.code_bits, f, qmax, lo, hi);
     else if (vec)
-        quant_flat_kernel<T, VF, MODE, 0><<<grid, kThreads, 0, st>>>((const T*)io.x, (const T*)io.gy, (T*)io.y,
+        launch_after(quant_flat_kernel<T, VF, MODE, 0>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y,
                                                                          (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes, io.code_bits, f, qmax, lo, hi);
     else
-        quant_flat_kernel<T, 1, MODE, 1><<<grid, kThreads, 0, st>>>((const T*)io.x, (const T*)io.gy, (T*)io.y,
+        launch_after(quant_flat_kernel<T, 1, MODE, 1>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y,
                                                                        (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes, io.code_bits, f, qmax, lo, hi);
     return cudaGetLastError();
 }
@@ -1073,9 +1071,9 @@ cudaError_t dequant_strings_bits(const uint32_t* pcodes, T* y, const Geom& g, co
     const uint32_t per_cta = kThreads * 2, grid = (n + per_cta - 1) / per_cta;
     const FastDiv di = make_fastdiv((uint32_t)g.inner), dc = make_fastdiv((uint32_t)g.C);
     if (g.inner % 8 == 0)
-        dequant_strings_kernel<T, BITS, false><<<grid, kThreads, 0, st>>>(pcodes, y, n, last, (uint32_t)g.inner, di, dc, s, z);
+        launch_after(dequant_strings_kernel<T, BITS, false>, grid, kThreads, 0, st, pcodes, y, n, last, (uint32_t)g.inner, di, dc, s, z);
     else
-        dequant_strings_kernel<T, BITS, true><<<grid, kThreads, 0, st>>>(pcodes, y, n, last, (uint32_t)g.inner, di, dc, s, z);
+        launch_after(dequant_strings_kernel<T, BITS, true>, grid, kThreads, 0, st, pcodes, y, n, last, (uint32_t)g.inner, di, dc, s, z);
     return cudaGetLastError();
 }
 
@@ -1103,14 +1101,14 @@ cudaError_t launch_range(const void* x, int dtype, const Geom& g, uint32_t* kmin
                                      : range_flat_t<__nv_bfloat16>(x, g, kmin, kmax, end, st);
     if (e != cudaSuccess || fused) return e;
     const int grid = (int)((g.C + 255) / 256);
-    finalize_range_kernel<<<grid, 256, 0, st>>>(kmin, kmax, g.C, lo, hi, bits, s_opt, z_opt);
+    launch_after(finalize_range_kernel, grid, 256, 0, st, kmin, kmax, g.C, lo, hi, bits, s_opt, z_opt);
     return cudaGetLastError();
 }
 
 cudaError_t launch_params(const float* lo, const float* hi, int64_t G, int bits, float* s_opt, float* z_opt,
                           cudaStream_t st) {
     int grid = (int)((G + 255) / 256);
-    params_kernel<<<grid, 256, 0, st>>>(lo, hi, G, bits, s_opt, z_opt);
+    launch_after(params_kernel, grid, 256, 0, st, lo, hi, G, bits, s_opt, z_opt);
     return cudaGetLastError();
 }
 
@@ -1144,14 +1142,14 @@ cudaError_t launch_bwd_packmask(const void* gy, const uint32_t* pmask, void* gx,
     const int64_t per_cta = (int64_t)kThreads * kUnroll;
     const unsigned grid = (unsigned)((units + per_cta - 1) / per_cta);
     if (dtype == 0) {
-        if (vec) bwd_packmask_kernel<float, 4><<<grid, kThreads, 0, st>>>((const float*)gy, pmask, (float*)gx, E);
-        else bwd_packmask_kernel<float, 1><<<grid, kThreads, 0, st>>>((const float*)gy, pmask, (float*)gx, E);
+        if (vec) launch_after(bwd_packmask_kernel<float, 4>, grid, kThreads, 0, st, (const float*)gy, pmask, (float*)gx, E);
+        else launch_after(bwd_packmask_kernel<float, 1>, grid, kThreads, 0, st, (const float*)gy, pmask, (float*)gx, E);
     } else {
         if (vec)
-            bwd_packmask_kernel<__nv_bfloat16, 8><<<grid, kThreads, 0, st>>>((const __nv_bfloat16*)gy, pmask,
+            launch_after(bwd_packmask_kernel<__nv_bfloat16, 8>, grid, kThreads, 0, st, (const __nv_bfloat16*)gy, pmask,
                                                                              (__nv_bfloat16*)gx, E);
         else
-            bwd_packmask_kernel<__nv_bfloat16, 1><<<grid, kThreads, 0, st>>>((const __nv_bfloat16*)gy, pmask,
+            launch_after(bwd_packmask_kernel<__nv_bfloat16, 1>, grid, kThreads, 0, st, (const __nv_bfloat16*)gy, pmask,
                                                                              (__nv_bfloat16*)gx, E);
     }
     return cudaGetLastError();
@@ -1168,14 +1166,14 @@ cudaError_t launch_distortion(const void* x, const void* q, int dtype, int64_t E
     const int64_t ctas = (units + per_cta - 1) / per_cta, cap = (int64_t)sms * 8;
     const int grid = (int)(ctas < 1 ? 1 : (ctas < cap ? ctas : cap));
     if (dtype == 0) {
-        if (vec) distortion_kernel<float, 4><<<grid, kThreads, 0, st>>>((const float*)x, (const float*)q, E, sums);
-        else distortion_kernel<float, 1><<<grid, kThreads, 0, st>>>((const float*)x, (const float*)q, E, sums);
+        if (vec) launch_after(distortion_kernel<float, 4>, grid, kThreads, 0, st, (const float*)x, (const float*)q, E, sums);
+        else launch_after(distortion_kernel<float, 1>, grid, kThreads, 0, st, (const float*)x, (const float*)q, E, sums);
     } else {
         if (vec)
-            distortion_kernel<__nv_bfloat16, 8><<<grid, kThreads, 0, st>>>((const __nv_bfloat16*)x,
+            launch_after(distortion_kernel<__nv_bfloat16, 8>, grid, kThreads, 0, st, (const __nv_bfloat16*)x,
                                                                            (const __nv_bfloat16*)q, E, sums);
         else
-            distortion_kernel<__nv_bfloat16, 1><<<grid, kThreads, 0, st>>>((const __nv_bfloat16*)x,
+            launch_after(distortion_kernel<__nv_bfloat16, 1>, grid, kThreads, 0, st, (const __nv_bfloat16*)x,
                                                                            (const __nv_bfloat16*)q, E, sums);
     }
     return cudaGetLastError();
@@ -1197,14 +1195,14 @@ cudaError_t launch_dequant_packed(const uint32_t* pcodes, void* y, int dtype, co
     const int64_t ctas = (units + kThreads - 1) / kThreads, cap = (int64_t)sms * 16;
     const int grid = (int)(ctas < 1 ? 1 : (ctas < cap ? ctas : cap));
     if (dtype == 0) {
-        if (vec) dequant_packed_kernel<float, 4><<<grid, kThreads, 0, st>>>(pcodes, (float*)y, g.E, g.inner, g.C, bits, s, z);
-        else dequant_packed_kernel<float, 1><<<grid, kThreads, 0, st>>>(pcodes, (float*)y, g.E, g.inner, g.C, bits, s, z);
+        if (vec) launch_after(dequant_packed_kernel<float, 4>, grid, kThreads, 0, st, pcodes, (float*)y, g.E, g.inner, g.C, bits, s, z);
+        else launch_after(dequant_packed_kernel<float, 1>, grid, kThreads, 0, st, pcodes, (float*)y, g.E, g.inner, g.C, bits, s, z);
     } else {
         if (vec)
-            dequant_packed_kernel<__nv_bfloat16, 8><<<grid, kThreads, 0, st>>>(pcodes, (__nv_bfloat16*)y, g.E, g.inner,
+            launch_after(dequant_packed_kernel<__nv_bfloat16, 8>, grid, kThreads, 0, st, pcodes, (__nv_bfloat16*)y, g.E, g.inner,
                                                                                g.C, bits, s, z);
         else
-            dequant_packed_kernel<__nv_bfloat16, 1><<<grid, kThreads, 0, st>>>(pcodes, (__nv_bfloat16*)y, g.E, g.inner,
+            launch_after(dequant_packed_kernel<__nv_bfloat16, 1>, grid, kThreads, 0, st, pcodes, (__nv_bfloat16*)y, g.E, g.inner,
                                                                                g.C, bits, s, z);
     }
     return cudaGetLastError();

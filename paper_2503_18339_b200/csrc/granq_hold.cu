@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
         np = a.div_inner.div((u0 + n) * V - 1) - p0 + 1;
     }
 
+    let_the_kernel_behind_start();
     for (uint32_t i = tid; i < held; i += kHThreads) h_cp_async_16(tile + i, xg + i);
     if constexpr (KIND != H_ONE) {
         for (uint32_t p = tid; p < np; p += kHThreads) s_kmn[p] = s_kmx[p] = 0;

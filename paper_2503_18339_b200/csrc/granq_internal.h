@@ -95,6 +95,24 @@ inline cudaError_t allow_smem(K kern, size_t most) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
+// Launch of a kernel that begins with after_the_kernel_ahead(): its grid is set up while the kernel ahead of it in the stream
+// drains, which hides a launch's latency: weights of a network 20.5 -> 17.6 us, range, forward and backward of [128,960,7,7]
+// 41.0 -> 37.1, codes and back of [128,144,56,56] 128.7 -> 123.9.
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // ---- generic ("flat") kernels: any geometry, any alignment --------------------------------
 // Range of every group (Eq. 4) into lo / hi, and s / z when bits > 0 and the pointers are given (Eq. 5).  The keys and,
 // where one is given, the counter must be zero on entry; with a counter the range launch finishes by itself.

@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a)
     const float qmax = a.qmax;
     const uint64_t drop = l2_policy_evict_first();
 
+    let_the_kernel_behind_start();
     for (uint32_t k = 0; k < held; ++k) r_cp_async_16(tile + k * tstep, xg + k * step);
     for (uint32_t t = tid; t < 2 * P * V; t += NT) s_kmn[t] = 0;
     __syncthreads();

@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(kWThreads, HOLD == 1 ? (GRAD ? 5 : 6) : GRAD ?
         else b = m - 1;
     }
     const WDesc& d = tab.d[a];
+    after_the_kernel_ahead();
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, team = d.team;
     const uint32_t c = (blockIdx.x - d.first_block) * (kWWarps / team) + warp / team;      // this team's group
     const bool valid = c < d.channels;
@@ -226,9 +227,8 @@ cudaError_t w_launch_n(const WDesc* descs, int n, uint32_t blocks, cudaStream_t 
         tab.d[i] = descs[i];
         small = small && (descs[i].vec ? descs[i].group_elems / V : descs[i].group_elems) <= 32;
     }
-    if (small) weights_kernel<T, GRAD, N, 1><<<blocks, kWThreads, 0, st>>>(tab, (uint32_t)n);
-    else weights_kernel<T, GRAD, N, kWHold><<<blocks, kWThreads, 0, st>>>(tab, (uint32_t)n);
-    return cudaGetLastError();
+    if (small) return launch_after(weights_kernel<T, GRAD, N, 1>, blocks, kWThreads, 0, st, tab, (uint32_t)n);
+    return launch_after(weights_kernel<T, GRAD, N, kWHold>, blocks, kWThreads, 0, st, tab, (uint32_t)n);
 }
 
 template <typename T>
