@@ -191,7 +191,7 @@ int granq_range(const void* x, int dtype, const int64_t dims[4], int channel_axi
     if (int rc = check_workspace(workspace, workspace_bytes, G)) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     Workspace ws = carve_workspace(workspace, G);
-    cudaError_t e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
+    cudaError_t e = launch_clear(workspace, ws.clear_bytes, nullptr, st);
     if (e == cudaSuccess)
         e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, 0, nullptr, nullptr, st);
     return cuda_status(e);
@@ -280,7 +280,8 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
     if (plan == PLAN_CLUSTER && !tp.ok) {
         if (!zeroed && !kp.clears_status) e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);      // the status word
     } else if (!(zeroed && keeps_zero)) {
-        e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
+        e = launch_clear(workspace, ws.clear_bytes, nullptr, st);
+        ws.cleared = true;
     }
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
     // two passes over x by ordinary launches: any geometry, any GPU
@@ -401,13 +402,17 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
     if (kp.ok) {
         // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
         if (!zeroed && (tp.ok || !kp.clears_status))
-            e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
+            e = launch_clear(workspace, tp.ok ? ws.clear_bytes : sizeof(uint32_t), nullptr, st);
+        ws.cleared = !zeroed && tp.ok;
         // the kernel writes the mask byte by byte: the padding bits of a last, partial word are cleared here
         if (e == cudaSuccess && g.E % 32 != 0) e = cudaMemsetAsync(packed_mask + g.E / 32, 0, sizeof(uint32_t), st);
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
         return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     }
-    if (!(zeroed && cp.ok)) e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
+    if (!(zeroed && cp.ok)) {
+        e = launch_clear(workspace, ws.clear_bytes, nullptr, st);
+        ws.cleared = true;
+    }
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
@@ -545,7 +550,7 @@ int granq_distortion(const void* x, const void* q, int dtype, const int64_t dims
         ((uintptr_t)sums_out & 7))
         return GRANQ_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    cudaError_t e = cudaMemsetAsync(sums_out, 0, 4 * sizeof(double), st);
+    cudaError_t e = launch_clear(nullptr, 0, sums_out, st);
     if (e == cudaSuccess) e = launch_distortion(x, q, dtype, g.E, sums_out, st);
     return cuda_status(e);
 }
@@ -587,18 +592,16 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
     Workspace ws = carve_workspace(workspace, G);
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     kp.zero_status = !zeroed && kp.clears_status;
-    cudaError_t e = cudaMemsetAsync(sums_out, 0, 4 * sizeof(double), st);
     const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
-    if (e == cudaSuccess && kp.ok) {
-        // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
-        if (!zeroed && (tp.ok || !kp.clears_status))
-            e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
-        if (e != cudaSuccess) return GRANQ_ERR_CUDA;
-        return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
-    }
-    const HoldPlan hp = cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
-    if (e == cudaSuccess && !(zeroed && (cp.ok || hp.ok))) e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
+    const HoldPlan hp = kp.ok || cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
+    // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
+    const size_t clear = zeroed && (kp.ok || cp.ok || hp.ok) ? 0
+                         : !kp.ok || tp.ok ? ws.clear_bytes : kp.clears_status ? 0 : sizeof(uint32_t);
+    cudaError_t e = launch_clear(workspace, clear, sums_out, st);
+    ws.cleared = true;
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
+    if (kp.ok)
+        return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     if (hp.ok) {
         e = launch_hold(hp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
         if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_status(e);
@@ -673,11 +676,15 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
     if (kp.ok) {
         // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
         if (!zeroed && (tp.ok || !kp.clears_status))
-            e = cudaMemsetAsync(workspace, 0, tp.ok ? ws.clear_bytes : sizeof(uint32_t), st);
+            e = launch_clear(workspace, tp.ok ? ws.clear_bytes : sizeof(uint32_t), nullptr, st);
+        ws.cleared = !zeroed && tp.ok;
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
         return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, st));
     }
-    if (!(zeroed && cp.ok)) e = cudaMemsetAsync(workspace, 0, ws.clear_bytes, st);
+    if (!(zeroed && cp.ok)) {
+        e = launch_clear(workspace, ws.clear_bytes, nullptr, st);
+        ws.cleared = true;
+    }
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, g_tune, st);

@@ -65,6 +65,7 @@ struct TArgs {
     uint32_t tile_units;   // room for x in shared memory
     uint32_t gy_units;     // of a CTA's share of gy, this many units are staged behind it
     uint32_t spin_limit, expected;
+    uint32_t early;        // x and gy may be read before the kernel ahead has completed: it only clears the workspace
     uint32_t slab_units;   // units of one slab
     FastDiv div_plane;     // units per plane
 };
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     const float qmax = a.qmax;
     DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS = 4)
     dacc.reset();
-    let_the_kernel_behind_start();
+    if (!a.early) after_the_kernel_ahead();
 
     // the first channel's copies; those of the later ones are sent from the quantize walk
     {
@@ -142,6 +143,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
             advance(at, off);
         }
     }
+    if (a.early) after_the_kernel_ahead();
     for (uint32_t c = team; c < a.C; c += a.teams) {
         t_cp_async_wait_all();
         // ---- Eq. 4: range of this CTA's share ----
@@ -447,7 +449,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
     };
 
     if (tid == 0) s_bad = 0xFFFFFFFFu;
-    let_the_kernel_behind_start();
+    if (!a.early) after_the_kernel_ahead();
     // the first copies; those of the later jobs are sent from the quantize walk
     for (uint32_t j = 0; j < depth && j < jobs; ++j) {
         uint32_t ti, c;
@@ -460,6 +462,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
             advance(at, off);
         }
     }
+    if (a.early) after_the_kernel_ahead();
     for (uint32_t t = 0; t <= jobs; ++t) {
         if (t < jobs) {
             t_cp_async_wait_all();
@@ -597,6 +600,7 @@ cudaError_t launch_colteam_list(const TeamPlan& plan, const TeamTensor* tensors,
     a.tile_units = plan.tile_units;
     a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kTSpinLimit;
     a.expected = plan.R + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
+    a.early = n == 1 && tensors[0].ws.cleared ? 1u : 0u;
     a.div_plane = make_fastdiv(a.plane_units);
     TList list{};
     list.n = n;
@@ -646,6 +650,7 @@ cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, in
     a.gy_units = plan.gy_units;
     a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kTSpinLimit;
     a.expected = plan.R + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
+    a.early = ws.cleared ? 1u : 0u;
     a.div_plane = make_fastdiv(a.plane_units);
     const int extras = io.dist ? 4 : io.pmask ? 2 : io.pcodes ? 3 : 0;
     return dtype == 0 ? t_launch_mode<float>(a, mode, extras, plan, tune, st)

@@ -253,10 +253,13 @@ __device__ __forceinline__ void run_add(WarpRun& r, bool valid, uint32_t g, uint
 // The kernel behind this one in the stream may be set up; it waits for this one's end, memory included, by itself.
 __device__ __forceinline__ void let_the_kernel_behind_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// The kernel ahead in the stream has completed and its memory is there.
+__device__ __forceinline__ void wait_for_the_kernel_ahead() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // First thing in a kernel launched by launch_after(): the kernel ahead of it in the stream has completed and its memory is
 // there; the kernel behind it may be set up (it waits in the same way).
 __device__ __forceinline__ void after_the_kernel_ahead() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_the_kernel_ahead();
     let_the_kernel_behind_start();
 }
 

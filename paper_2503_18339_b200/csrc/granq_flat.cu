@@ -377,6 +377,12 @@ __global__ void finalize_range_kernel(const uint32_t* __restrict__ kmin, const u
     if (i < G) finalize_group(kmin, kmax, i, lo, hi, bits, s_opt, z_opt);
 }
 
+__global__ void __launch_bounds__(kThreads) clear_kernel(uint32_t* __restrict__ p, uint32_t words, double* __restrict__ sums) {
+    after_the_kernel_ahead();
+    for (uint32_t i = blockIdx.x * kThreads + threadIdx.x; i < words; i += gridDim.x * kThreads) p[i] = 0;
+    if (sums && blockIdx.x == 0 && threadIdx.x < 4) sums[threadIdx.x] = 0.0;
+}
+
 __global__ void params_kernel(const float* __restrict__ lo, const float* __restrict__ hi, int64_t G, int bits,
                               float* __restrict__ s_opt, float* __restrict__ z_opt) {
     after_the_kernel_ahead();
@@ -1103,6 +1109,12 @@ cudaError_t launch_range(const void* x, int dtype, const Geom& g, uint32_t* kmin
     const int grid = (int)((g.C + 255) / 256);
     launch_after(finalize_range_kernel, grid, 256, 0, st, kmin, kmax, g.C, lo, hi, bits, s_opt, z_opt);
     return cudaGetLastError();
+}
+
+cudaError_t launch_clear(void* workspace, size_t bytes, double* sums_opt, cudaStream_t st) {
+    const size_t words = bytes / 4, blocks = (words + 4 * kThreads - 1) / (4 * kThreads);
+    return launch_after(clear_kernel, (unsigned)std::max<size_t>(1, std::min<size_t>(blocks, 256)), kThreads, 0, st,
+                        (uint32_t*)workspace, (uint32_t)words, sums_opt);
 }
 
 cudaError_t launch_params(const float* lo, const float* hi, int64_t G, int bits, float* s_opt, float* z_opt,

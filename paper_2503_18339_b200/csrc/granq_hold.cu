@@ -50,6 +50,7 @@ struct HArgs {
     uint32_t inner;        // elements of one plane
     uint32_t groups;
     uint32_t spin_limit, expected;
+    uint32_t early;        // x may be read before the kernel ahead has completed: it only clears the workspace
     FastDiv div_inner, div_groups;
 };
 
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
         np = a.div_inner.div((u0 + n) * V - 1) - p0 + 1;
     }
 
-    let_the_kernel_behind_start();
+    if (!a.early) after_the_kernel_ahead();
     for (uint32_t i = tid; i < held; i += kHThreads) h_cp_async_16(tile + i, xg + i);
     if constexpr (KIND != H_ONE) {
         for (uint32_t p = tid; p < np; p += kHThreads) s_kmn[p] = s_kmx[p] = 0;
@@ -123,6 +124,7 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
             s_one[0][tid >> 5] = ka;
             s_one[1][tid >> 5] = kb;
         }
+        if (a.early) after_the_kernel_ahead();
         __syncthreads();
         if (tid < 32) {
             ka = __reduce_max_sync(kFullMask, lane < kHWarps ? s_one[0][lane] : 0u);
@@ -170,6 +172,7 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
             }
             flush();
         }
+        if (a.early) after_the_kernel_ahead();
         __syncthreads();
         for (uint32_t t = tid; t < np; t += kHThreads) {
             const uint32_t c = p0 + t - a.div_groups.div(p0 + t) * a.groups, k1 = s_kmn[t], k2 = s_kmx[t];
@@ -354,6 +357,7 @@ cudaError_t launch_hold(const HoldPlan& plan, const QuantIO& io, int mode, int d
     a.groups = (uint32_t)g.C;
     a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kHSpinLimit;
     a.expected = plan.ctas + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
+    a.early = ws.cleared ? 1u : 0u;
     a.div_inner = make_fastdiv(a.inner);
     a.div_groups = make_fastdiv(a.groups);
     const int kind = g.C == 1 && g.outer == 1 ? H_ONE : g.inner % V == 0 ? H_PLANES : H_RAGGED;

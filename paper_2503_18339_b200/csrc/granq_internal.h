@@ -56,6 +56,7 @@ struct Workspace {
     uint32_t* kmax;
     uint32_t* counters;
     size_t clear_bytes;  // bytes from the start that must be zero before a launch
+    bool cleared;        // the kernel ahead of the launch is launch_clear()'s
 };
 inline size_t workspace_bytes_for(int64_t G) {
     size_t b = kWsHeaderBytes + (size_t)G * 8 + ((size_t)G + 1) * 4;
@@ -69,6 +70,7 @@ inline Workspace carve_workspace(void* ws, int64_t G) {
     w.kmax = w.kmin + G;
     w.counters = w.kmax + G;
     w.clear_bytes = kWsHeaderBytes + (size_t)G * 8 + ((size_t)G + 1) * 4;
+    w.cleared = false;
     return w;
 }
 
@@ -112,6 +114,10 @@ inline cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned thre
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
+
+// Zero `bytes` of a workspace (a multiple of 4) and, where given, four sums: a kernel in place of one memset or two, which a
+// cooperative launch behind it need not wait for to read its inputs (a memset and the launch behind it 7.2 us, this 4.7).
+cudaError_t launch_clear(void* workspace, size_t bytes, double* sums_opt, cudaStream_t st);
 
 // ---- generic ("flat") kernels: any geometry, any alignment --------------------------------
 // Range of every group (Eq. 4) into lo / hi, and s / z when bits > 0 and the pointers are given (Eq. 5).  The keys and,
@@ -171,10 +177,25 @@ struct StagedTuning {
 // A cooperative launch that may be refused: every CTA has to be resident at once, and where the GPU is shared out (a
 // partition, a limit on the SMs of a process) fewer are than its attributes say.  cudaErrorCooperativeLaunchTooLarge,
 // with nothing enqueued and no error left behind, tells the caller to take a plan that needs no such launch.
+// The grid is set up while the kernel ahead drains; the kernel waits for that one's memory itself: before it reads anything, or,
+// where the kernel ahead only clears its workspace (Workspace::cleared; that one has waited for all before it), between
+// reading its inputs and touching anything else.
 inline cudaError_t launch_cooperative(const void* kern, uint32_t grid, uint32_t threads, void** params, size_t smem,
                                       const StagedTuning& tune, cudaStream_t st) {
     if (tune.coop_ctas > 0 && grid > (uint32_t)tune.coop_ctas) return cudaErrorCooperativeLaunchTooLarge;
-    const cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), params, smem, st);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, kern, params);
     if (e == cudaErrorCooperativeLaunchTooLarge) (void)cudaGetLastError();
     return e;
 }

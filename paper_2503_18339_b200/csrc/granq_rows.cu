@@ -60,6 +60,7 @@ struct RArgs {
     uint32_t hold;       // blocks of rows a CTA keeps in shared memory
     uint32_t lost;       // of the others, those before this one are not expected to be in the L2 when they are read again
     uint32_t spin_limit, expected;
+    uint32_t early;      // x may be read before the kernel ahead has completed: it only clears the workspace
     uint64_t rows;
 };
 
@@ -103,7 +104,7 @@ __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a)
     const float qmax = a.qmax;
     const uint64_t drop = l2_policy_evict_first();
 
-    let_the_kernel_behind_start();
+    if (!a.early) after_the_kernel_ahead();
     for (uint32_t k = 0; k < held; ++k) r_cp_async_16(tile + k * tstep, xg + k * step);
     for (uint32_t t = tid; t < 2 * P * V; t += NT) s_kmn[t] = 0;
     __syncthreads();
@@ -138,6 +139,7 @@ __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a)
             }
         }
     }
+    if (a.early) after_the_kernel_ahead();
     __syncthreads();
     for (uint32_t t = tid; t < chans; t += NT) {           // channel t of the slice: element t % V of unit column t / V
         const uint32_t at = (t % V) * P + t / V, k1 = s_kmn[at], k2 = s_kmx[at];
@@ -373,6 +375,7 @@ cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, i
     a.lost = tail < 1.0 ? (uint32_t)((1.0 - tail) * (double)per_cta) : 0u;
     a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kRSpinLimit;
     a.expected = a.team + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
+    a.early = ws.cleared ? 1u : 0u;
     const bool extras = io.codes != nullptr || io.mask != nullptr;
     if (dtype == 0) {
         if (mode == MODE_FWD) return r_launch<float, MODE_FWD>(a, extras, grid, threads, smem, tune, st);
