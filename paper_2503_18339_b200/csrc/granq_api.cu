@@ -409,11 +409,16 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
         return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     }
-    if (!(zeroed && cp.ok)) {
+    const HoldPlan hp = cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
+    if (!(zeroed && (cp.ok || hp.ok))) {
         e = launch_clear(workspace, ws.clear_bytes, nullptr, st);
         ws.cleared = true;
     }
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
+    if (hp.ok) {
+        e = launch_hold(hp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
+        if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_status(e);
+    }
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {
@@ -681,11 +686,16 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
         return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, st));
     }
-    if (!(zeroed && cp.ok)) {
+    const HoldPlan hp = cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
+    if (!(zeroed && (cp.ok || hp.ok))) {
         e = launch_clear(workspace, ws.clear_bytes, nullptr, st);
         ws.cleared = true;
     }
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
+    if (hp.ok) {
+        e = launch_hold(hp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, g_tune, st);
+        if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_status(e);
+    }
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, g_tune, st);
     } else {
@@ -794,7 +804,8 @@ int granq_fused_plan(int dtype, const int64_t dims[4], int channel_axis, int gro
     QuantIO io{};   // null pointers: alignment is assumed
     const int plan = choose_plan(dtype, g, io, with_backward != 0, flags, nullptr, nullptr, nullptr, nullptr);
     if (launches_out) {
-        if (plan == PLAN_STAGED || plan == PLAN_L2WAVE || plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS) *launches_out = 1;
+        const bool held = plan == PLAN_TWO_PASS && prefer_hold(dtype, g, io, flags).ok;
+        if (held || plan == PLAN_STAGED || plan == PLAN_L2WAVE || plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS) *launches_out = 1;
         else if (plan == PLAN_NAIVE) *launches_out = (int)(3 * g.C);
         else if (plan == PLAN_TWO_PASS) *launches_out = g.C <= 4096 ? 2 : 3;
     }

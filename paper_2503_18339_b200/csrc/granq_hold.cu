@@ -33,6 +33,9 @@ struct HArgs {
     const void* gy;
     void* y;
     void* gx;
+    uint32_t* pmask;       // the STE mask at one bit per element, or null
+    uint32_t* pcodes;      // the codes as a bit string of code_bits each, or null (y is then not written)
+    int code_bits;
     double* dist;          // four running sums of Table 2's statistics, or null
     uint32_t* status;
     uint32_t* kmin;
@@ -225,22 +228,30 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
     auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint32_t i) {
         Pack<T> py, pgx;
         uint32_t cb[V / 4], mb[V / 4];
+        const int code_bits = EXTRAS == 3 ? a.code_bits : 8;
         if constexpr (KIND == H_ONE) {
-            quantize_own<T, kBwd, EXTRAS>(px, pg, one, qmax, py, pgx, cb, mb);
+            quantize_own<T, kBwd, EXTRAS>(px, pg, one, qmax, py, pgx, cb, mb, code_bits);
         } else {
             uint32_t p, rem;
             a.div_inner.divmod(rem0 + i * V, p, rem);
             if constexpr (KIND == H_PLANES) {
-                quantize_own<T, kBwd, EXTRAS>(px, pg, s_par[p], qmax, py, pgx, cb, mb);
+                quantize_own<T, kBwd, EXTRAS>(px, pg, s_par[p], qmax, py, pgx, cb, mb, code_bits);
             } else {
                 const int n1 = (int)min((uint32_t)V, a.inner - rem);
                 const GroupParam g1 = s_par[p];
-                if (n1 == V) quantize_own<T, kBwd, EXTRAS>(px, pg, g1, qmax, py, pgx, cb, mb);
-                else quantize_pack<T, kBwd, true, EXTRAS, true>(px, pg, g1, s_par[p + 1], n1, qmax, py, pgx, cb, mb);
+                if (n1 == V) quantize_own<T, kBwd, EXTRAS>(px, pg, g1, qmax, py, pgx, cb, mb, code_bits);
+                else quantize_pack<T, kBwd, true, EXTRAS, true>(px, pg, g1, s_par[p + 1], n1, qmax, py, pgx, cb, mb, code_bits);
             }
+        }
+        // masks and codes 8 elements at a time: the tensor is a multiple of 32 elements and a piece begins on a multiple of 8
+        // units, so both lanes of a pair of fp32 units are here
+        if constexpr (EXTRAS == 3) {
+            store_code_bytes<V>(a.pcodes, (size_t)(u0 + i) * V, code_string_of<V>(cb, code_bits), code_bits, lane);
+            return;
         }
         st_stream_16(yg + i, py.raw);
         if constexpr (kBwd) st_stream_16(gxg + i, pgx.raw);
+        if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, (size_t)(u0 + i) * V, mask_bits_of<V, EXTRAS>(mb), lane);
         if constexpr (EXTRAS == 4) dacc.add(px, py);
     };
     // what did not stay, from the end back; n - 1 - (held ...) keeps neighbouring lanes on neighbouring units
@@ -313,7 +324,8 @@ HoldPlan plan_hold(int dtype, const Geom& g, const QuantIO& io, int sm_count) {
     HoldPlan p{};
     p.ok = false;
     const int64_t V = dtype == 0 ? 4 : 8;
-    if (io.codes || io.mask || io.pmask || io.pcodes) return p;
+    if (io.codes || io.mask) return p;
+    if ((io.pmask || io.pcodes) && (g.E % 32 != 0 || io.gy)) return p;
     if (g.E % V != 0 || g.inner < V || g.E >= (1ll << 31) || g.C >= (1ll << 28)) return p;
     if (!h_aligned16(io.x) || !h_aligned16(io.gy) || !h_aligned16(io.y) || !h_aligned16(io.gx)) return p;
     const uint64_t units = (uint64_t)(g.E / V), most = 2ull * (uint64_t)sm_count;
@@ -339,6 +351,9 @@ cudaError_t launch_hold(const HoldPlan& plan, const QuantIO& io, int mode, int d
     a.gy = io.gy;
     a.y = io.y;
     a.gx = io.gx;
+    a.pmask = io.pmask;
+    a.pcodes = io.pcodes;
+    a.code_bits = io.code_bits;
     a.dist = io.dist;
     a.status = ws.status;
     a.kmin = ws.kmin;
@@ -361,13 +376,15 @@ cudaError_t launch_hold(const HoldPlan& plan, const QuantIO& io, int mode, int d
     a.div_inner = make_fastdiv(a.inner);
     a.div_groups = make_fastdiv(a.groups);
     const int kind = g.C == 1 && g.outer == 1 ? H_ONE : g.inner % V == 0 ? H_PLANES : H_RAGGED;
-    if (dtype == 0) {
-        if (mode != MODE_FWD) return h_launch<float, MODE_BOTH, 0>(a, plan, kind, tune, st);
-        return io.dist ? h_launch<float, MODE_FWD, 4>(a, plan, kind, tune, st) : h_launch<float, MODE_FWD, 0>(a, plan, kind, tune, st);
-    }
-    if (mode != MODE_FWD) return h_launch<__nv_bfloat16, MODE_BOTH, 0>(a, plan, kind, tune, st);
-    return io.dist ? h_launch<__nv_bfloat16, MODE_FWD, 4>(a, plan, kind, tune, st)
-                   : h_launch<__nv_bfloat16, MODE_FWD, 0>(a, plan, kind, tune, st);
+    auto go = [&](auto zero) -> cudaError_t {
+        using T = decltype(zero);
+        if (mode != MODE_FWD) return h_launch<T, MODE_BOTH, 0>(a, plan, kind, tune, st);
+        if (io.dist) return h_launch<T, MODE_FWD, 4>(a, plan, kind, tune, st);
+        if (io.pmask) return h_launch<T, MODE_FWD, 2>(a, plan, kind, tune, st);
+        if (io.pcodes) return h_launch<T, MODE_FWD, 3>(a, plan, kind, tune, st);
+        return h_launch<T, MODE_FWD, 0>(a, plan, kind, tune, st);
+    };
+    return dtype == 0 ? go(0.0f) : go(__nv_bfloat16());
 }
 
 }  // namespace granq

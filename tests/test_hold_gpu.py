@@ -1,7 +1,8 @@
 """The kernel that holds a tensor on chip piece by piece (planes and slabs that are not whole 16-byte units, one group over the
 whole tensor) against the CPU oracle, bit for bit: pieces that begin and end inside planes, planes shorter than a thread's run
 and longer than a piece, units that straddle two planes, fewer units than threads, one group that stays on chip and one of
-which a part is read again - forward, with a gradient, with the distortion sums; the workspace zero again afterwards."""
+which a part is read again - forward, with a gradient, with the distortion sums, packed
+mask and packed codes; the workspace zero again afterwards."""
 import numpy as np
 import pytest
 import torch
@@ -9,6 +10,7 @@ import torch
 from gpu_util import assert_parity, make_case, to_dev, to_np
 from oracle import granq_oracle as orc
 from test_parity_gpu import b, knobs  # noqa: F401
+from test_rounding_gpu import assert_same_string
 
 pytestmark = pytest.mark.gpu
 
@@ -18,6 +20,7 @@ CASES = [
     ((8, 75, 5, 7), 0),         # planes shorter than a thread's run of units, an odd number of channels
     ((8, 301, 7, 7), 0),        # several planes to a thread
     ((16, 5, 27, 27), 0),       # planes of several runs
+    ((32, 5, 27, 27), 0),       # whole words of mask and codes
     ((8, 3, 111, 111), 0),      # a plane over many pieces
     ((24, 75, 27, 27), 0),      # several units to a thread
     ((3, 7, 9, 24), 2),         # one group, fewer units than one CTA has threads
@@ -49,6 +52,14 @@ def test_held_tensor(b, shape, mode, dtype):
     assert_parity(got, ref, shape, 1, mode, backward=False)
     # fp32 inside a pack, fp64 beyond: about 8 roundings of 2^-24 of a sum of same-signed terms
     assert np.allclose(to_np(got.sums), orc.distortion_sums(x, ref.y), rtol=1e-6, atol=0)
+    got = b.granq_fakequant_fused_fwd_packmask(xd, bits, group=mode, out=new(), flags=b.FLAG_WORKSPACE_ZEROED)
+    assert clean()
+    assert_parity(got, ref, shape, 1, mode, backward=False)
+    assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+    for code_bits in (1, 3, 4, 5, 8):
+        got = b.granq_quantize_packed_fused(xd, code_bits, group=mode, out=new(), flags=b.FLAG_WORKSPACE_ZEROED)
+        assert clean()
+        assert_same_string(got.packed_codes, orc.pack_codes(orc.fused(x, code_bits, group_mode=mode).codes, code_bits))
     dirty = b.FakeQuantOut(workspace=b.make_workspace(xd, group=mode).fill_(255))
     assert_parity(b.granq_fakequant_fused(xd, bits, gy=gyd, group=mode, out=dirty), ref, shape, 1, mode, backward=True)
 
