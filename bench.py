@@ -473,7 +473,7 @@ def main():
     achieved = dom_bytes / (dom_ms * 1e-3) / 1e9 if dominant else None
     rec = recorded_traffic()
     roofline = {
-        "bound": "hbm", "kernel": "colteam_kernel<float, fwd+bwd>",
+        "bound": "hbm", "kernel": "colteam_lag_kernel<float>",
         "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": (achieved / peak) if achieved else None,
         "peak_source": peak_src, "frac_of_nominal_8TBs": (achieved / NOMINAL_HBM_GBS) if achieved else None,
         "launches_per_step": len(dominant),

@@ -220,7 +220,8 @@ int granq_fakequant_bwd_packmask(const void* gy, const uint32_t* packed_mask, in
 /* The forward half of the whole path in one call (Algorithm 1, range step through pre-scale step):
  * range of x itself -> scale / zero-point -> y and the packed mask.  Takes the cluster-local plan
  * where a run of channels that is whole bytes of mask fits one cluster, the column-walk plan when slabs
- * and waves are whole mask words, else a range pass followed by an elementwise pass
+ * and waves are whole mask words, a launch that holds the tensor on chip piece by piece where it fits and is whole
+ * 32-element words, else a range pass followed by an elementwise pass
  * (GRANQ_FLAG_FORCE_TWO_PASS / GRANQ_FLAG_FORCE_COLWALK / GRANQ_FLAG_FORCE_CLUSTER select one;
  * GRANQ_FLAG_WORKSPACE_ZEROED as for granq_fakequant_fused()).
  *   min_out, max_out out G floats each (required);  scale_opt, zp_opt G floats or NULL */
@@ -333,7 +334,8 @@ int granq_fakequant_fused_batch(const granq_fused_desc* descs, int n_tensors, in
  *                            through quantize step): range of x itself -> scale / zero-point -> packed codes; x is
  *                            read from HBM once where a single-read plan fits (cluster-local kernel, column
  *                            walk: groups of 8 codes must not straddle slabs and the tensor is a multiple of 32
- *                            elements), else a range pass, the parameters and an elementwise pass.  The codes
+ *                            elements; a tensor held on chip piece by piece), else a range pass, the parameters
+ *                            and an elementwise pass.  The codes
  *                            are bit for bit those of granq_range() + granq_quantize_packed().  workspace and
  *                            flags (GRANQ_FLAG_WORKSPACE_ZEROED, GRANQ_FLAG_FORCE_TWO_PASS / _COLWALK / _CLUSTER) as
  *                            for granq_fakequant_fused().
@@ -503,7 +505,7 @@ enum granq_knob {
     GRANQ_KNOB_COLWALK_TEAM = 17,         /* column-walk plan: 1 = resident form wherever it fits, 2 = L2 waves
                                              only (as any set L2 knob means, unless this one is 1)           */
     GRANQ_KNOB_TEST_COOP_CTAS = 18        /* test hook: the cooperative launches that have a plan to fall back on
-                                             (channels-last, resident column walk) count as refused by the driver
+                                             (channels-last, resident column walk, held tensors, lists) count as refused by the driver
                                              where they have more CTAs than this                             */
 };
 int granq_tune(int knob, int value);

@@ -11,15 +11,20 @@
 //   - scale and zero-point (Eq. 5) are worked out once per CTA and the share is quantized from shared memory (Eq. 1,
 //     clamp, Eq. 6, STE).  A unit's place in shared memory is free as soon as its thread has read it, so the same
 //     loop sends the copy of the team's NEXT channel after it: reads stay in flight through the whole write phase.
-// With a gradient gy is staged the same way as far as shared memory goes and read in place beyond that.
+// With a gradient gy is staged the same way as far as shared memory goes and read in place beyond that; where a team then
+// has several rounds of channels, colteam_lag_kernel below holds two of them at a time instead.
 //
 // Why not the L2-resident waves of colwalk_kernel: the L2 does not keep a wave (forward-only calls read x 1.4
 // times from HBM, ncu: 9-15 % L2 hits), and its phases alternate.  Why teams and not clusters of 16 CTAs: a
 // cluster must sit in one GPC, which leaves an SM in ten without one.  Measured against the waves (fp32 / bf16, us):
 // forward [128,64,56,56] 55.8 -> 45.7 / 34.7 -> 30.3, [128,96,112,112] 309 -> 264 / 174 -> 139, [256,512,28,28]
 // 219 -> 156 / 123 -> 92; with a gradient 87.5 -> 81.9 / 47.4 -> 45.6, 472 -> 469 / 258 -> 234, 332 -> 298 / 183 -> 153;
-// [256,16,32,32] 16.7 -> 14.9 and 21.9 -> 19.4.  Bound by HBM in the mix of reads and writes (4.5-5.3 TB/s) once a
-// team has several channels, by the chain of copy, hand-over and quantize when it has one.
+// [256,16,32,32] 16.7 -> 14.9 and 21.9 -> 19.4.  Bound by the chain of copy, hand-over and quantize when a team has one
+// channel.  With several it moves 4.5 to 5.7 TB/s where plain copies in blocks that come in order move 6.7: about 70
+// instructions per unit, sixteen wavefronts for an asynchronous copy of a warp, and equal shares, of which half of
+// the SMs move 21 KB/us and the other half 37 when nothing holds them together.  Chunks dealt out by a counter even the SMs
+// out but publish, poll and fetch keys per chunk: 10 us of residence against the 10 us that 33 MB last at full rate; with a
+// gradient they reached 425 us where two channels side by side take 433, forward 183 where this form takes 151.
 //
 // Two CTAs of 512 threads per SM, 113 KB of shared memory each: one transfers while the other waits for its team.
 // The kernel expects zeroed keys and counters and, when no wait ran out, leaves them zeroed (slot C of the
