@@ -243,8 +243,8 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
                 else quantize_pack<T, kBwd, true, EXTRAS, true>(px, pg, g1, s_par[p + 1], n1, qmax, py, pgx, cb, mb, code_bits);
             }
         }
-        // masks and codes 8 elements at a time: the tensor is a multiple of 32 elements and a piece begins on a multiple of 8
-        // units, so both lanes of a pair of fp32 units are here
+        // masks and codes 8 elements at a time, a pair of fp32 units by the two lanes of a pair, the first of them by the even one: the
+        // tensor is a multiple of 32 elements, a piece begins on a multiple of 8 units, and both walks give an even lane an even unit
         if constexpr (EXTRAS == 3) {
             store_code_bytes<V>(a.pcodes, (size_t)(u0 + i) * V, code_string_of<V>(cb, code_bits), code_bits, lane);
             return;
@@ -254,23 +254,26 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
         if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, (size_t)(u0 + i) * V, mask_bits_of<V, EXTRAS>(mb), lane);
         if constexpr (EXTRAS == 4) dacc.add(px, py);
     };
-    // what did not stay, from the end back; n - 1 - (held ...) keeps neighbouring lanes on neighbouring units
+    // what did not stay, a block of units at a time from the end back; inside a block forward from an even unit (masks and codes:
+    // n and held are even), so that the even lane of a pair has its first unit there too
     if constexpr (KIND == H_ONE) {
-        for (uint32_t b = 0; b < n - held; b += U * kHThreads) {
+        for (uint32_t end = n; end > held;) {
+            const uint32_t len = min((uint32_t)(U * kHThreads), end - held), start = end - len;
             Pack<T> px[U], pg[U];
 #pragma unroll
             for (int k = 0; k < U; ++k) {
-                const uint32_t i = b + k * kHThreads + tid;
-                if (i < n - held) {
-                    px[k].raw = ld_stream_16(xg + (n - 1 - i));
-                    if constexpr (kBwd) pg[k].raw = ld_stream_16(gyg + (n - 1 - i));
+                const uint32_t i = k * kHThreads + tid;
+                if (i < len) {
+                    px[k].raw = ld_stream_16(xg + start + i);
+                    if constexpr (kBwd) pg[k].raw = ld_stream_16(gyg + start + i);
                 }
             }
 #pragma unroll
             for (int k = 0; k < U; ++k) {
-                const uint32_t i = b + k * kHThreads + tid;
-                if (i < n - held) emit(px[k], pg[k], n - 1 - i);
+                const uint32_t i = k * kHThreads + tid;
+                if (i < len) emit(px[k], pg[k], start + i);
             }
+            end = start;
         }
     }
     for (uint32_t b = 0; b < held; b += U * kHThreads) {
@@ -336,7 +339,7 @@ HoldPlan plan_hold(int dtype, const Geom& g, const QuantIO& io, int sm_count) {
     if (planes * kHPlaneBytes >= kHSmemBytes / 2) return p;
     p.planes = (uint32_t)planes;
     const uint32_t room = (kHSmemBytes - (p.planes * kHPlaneBytes + 15) / 16 * 16) / 16;
-    p.held = std::min(p.share, room);
+    p.held = std::min(p.share, room / 2 * 2);             // whole pairs of fp32 units, which lanes write masks and codes of together
     if (p.held < p.share && !(one && p.share <= 2 * room && (dtype == 1 || !io.gy))) return p;
     p.ok = true;
     return p;

@@ -9,6 +9,7 @@ import torch
 
 from gpu_util import assert_parity, make_case, to_dev, to_np
 from oracle import granq_oracle as orc
+from paper_2503_18339_b200 import workloads as wl
 from test_parity_gpu import b, knobs  # noqa: F401
 from test_rounding_gpu import assert_same_string
 
@@ -74,6 +75,34 @@ def test_one_group_beyond_what_stays_on_chip(b, dtype, shape):
     got = b.granq_fakequant_fused_stats(xd, 4, group=2)
     assert_parity(got, ref, shape, 1, 2, backward=False)
     assert np.allclose(to_np(got.sums), orc.distortion_sums(x, ref.y), rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("dtype,shape", [
+    ("f32", (96, 128, 28, 28)),
+    ("f32", (128, 128, 28, 28)),
+    ("f32", (32, 315, 1667, 1)),      # next to twice what stays, the last piece a sixth shorter than the others
+    ("bf16", (192, 128, 28, 28)),
+], ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else v)
+def test_packed_outputs_of_one_group_beyond_what_stays_on_chip(b, dtype, shape):
+    """Mask and codes of the part that is read again.  At 4 bits lo = -hi = -7.5 makes s = 1 and z = 8: the elements at the
+    top, one in ten, land on 16 and get no gradient, so that a bit in the wrong place shows in the mask too."""
+    x = np.clip(6.0 * np.random.default_rng(17).standard_normal(shape, dtype=np.float32), -7.5, 7.5)
+    x = wl.to_bf16_bits(x) if dtype == "bf16" else x
+    xd = to_dev(x)
+    zeroed = b.make_workspace(xd, group=2, zeroed=True)
+    for code_bits in (1, 3, 4, 5, 8):
+        ref = orc.fused(x, code_bits, group_mode=2)
+        for ws, flags in ((b.make_workspace(xd, group=2).fill_(255), 0), (zeroed, b.FLAG_WORKSPACE_ZEROED)):
+            got = b.granq_quantize_packed_fused(xd, code_bits, group=2, out=b.FakeQuantOut(workspace=ws), flags=flags)
+            assert b.workspace_status(ws) == b.OK
+            assert_same_string(got.packed_codes, orc.pack_codes(ref.codes, code_bits))
+            if code_bits == 4:
+                got = b.granq_fakequant_fused_fwd_packmask(xd, 4, group=2, out=b.FakeQuantOut(workspace=ws), flags=flags)
+                assert b.workspace_status(ws) == b.OK
+                assert_parity(got, ref, shape, 1, 2, backward=False)
+                assert 0.05 < 1 - ref.mask.mean() < 0.2
+                assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+    assert int(zeroed.view(torch.int32).abs().sum().item()) == 0
 
 
 @pytest.mark.parametrize("stats", [False, True])
