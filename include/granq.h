@@ -448,7 +448,8 @@ int granq_cluster_geometry(int dtype, const int64_t dims[4], int channel_axis, i
 /*
  * Host-only query: how the resident form of the column walk (a channel held by a team of CTAs) would cut this tensor on
  * a device with `sm_count` SMs.
- * out = { CTAs per team, teams, 16-byte units of x that one CTA holds, channels that a team takes one after the other,
+ * out = { CTAs per team, teams, 16-byte units of x that one CTA holds (of both channels, where it holds two side by side as
+ *         calls with a gradient do), channels that a team takes one after the other,
  *         1 if the column-walk plan takes this form for it rather than the L2 waves }.
  * Returns GRANQ_ERR_UNSUPPORTED when a channel does not fit or planes are no whole 16-byte units.  Calls with byte codes
  * or masks take the waves whatever the answer.

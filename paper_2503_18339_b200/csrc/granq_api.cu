@@ -122,7 +122,7 @@ TeamPlan prefer_team(int dtype, const Geom& g, const QuantIO& io, bool backward,
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return none;
-    return plan_colteam(dtype, g, io, backward, sms);
+    return plan_colteam(dtype, g, io, backward, sms, g_tune);
 }
 
 // The call with its channels held on chip, in the form chosen; where the GPU does not hold that many CTAs at once, by
@@ -502,7 +502,7 @@ static int batch_together(const granq_fused_desc* descs, int first, int n_tensor
     if (n < 2 || (nb < (12u << 20) && n * nb < (48u << 20)) || cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return 0;
-    const TeamPlan p = plan_colteam(dtype, g, tensors[0].io, true, sms, (uint32_t)n);
+    const TeamPlan p = plan_colteam(dtype, g, tensors[0].io, true, sms, g_tune, (uint32_t)n);
     if (!p.ok || !p.lag) return 0;
     const cudaError_t e = launch_colteam_list(p, tensors, (uint32_t)n, dtype, g, g_tune, (cudaStream_t)cuda_stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) return 0;
@@ -856,9 +856,9 @@ int granq_team_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
     Geom g;
     int64_t G;
     if (!out || !dtype_ok(dtype) || sm_count < 1 || !make_geom(dims, channel_axis, group, g, G)) return GRANQ_ERR_INVALID_ARG;
-    const TeamPlan p = plan_colteam(dtype, g, QuantIO{}, with_backward != 0, sm_count);
+    const TeamPlan p = plan_colteam(dtype, g, QuantIO{}, with_backward != 0, sm_count, g_tune);
     if (!p.ok) return GRANQ_ERR_UNSUPPORTED;
-    const int64_t v[5] = {p.R, p.teams, p.tile_units, (g.C + p.teams - 1) / p.teams, team_over_waves(p, g, g_tune) ? 1 : 0};
+    const int64_t v[5] = {p.R, p.teams, (p.lag ? 2 : 1) * p.tile_units, (g.C + p.teams - 1) / p.teams, team_over_waves(p, g, g_tune) ? 1 : 0};
     for (int i = 0; i < 5; ++i) out[i] = v[i];
     return GRANQ_OK;
 }

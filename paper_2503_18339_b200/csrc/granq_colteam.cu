@@ -43,6 +43,7 @@ constexpr uint32_t kTWarps = kTThreads / 32;
 constexpr uint32_t kTSpinLimit = 1u << 24;   // bounded wait on a channel's counter (x ~32 ns)
 constexpr uint32_t kTStatusTimeout = 5;      // GRANQ_ERR_TIMEOUT
 constexpr uint32_t kTSmemUnits = 111u * 1024 / 16;      // staged units per CTA: two CTAs per SM, 228 KB between them
+constexpr uint32_t kTLagUnits = 1700;                   // smallest share of each of two channels side by side
 
 struct TArgs {
     const void* x;
@@ -550,7 +551,8 @@ cudaError_t t_launch_mode(const TArgs& a, int mode, int extras, const TeamPlan& 
 
 // Team size: the number of CTAs R for which rounds x (share of one CTA + what a hand-over costs) is smallest, the
 // share fitting the shared memory of one of two CTAs per SM.
-TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count, uint32_t tensors) {
+TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count, const StagedTuning& tune,
+                      uint32_t tensors) {
     TeamPlan p{};
     p.ok = false;
     const uint32_t V = dtype == 0 ? 4 : 8;
@@ -568,14 +570,20 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
     // of 3136 291, 43 of 2096 293, one channel at a time 14 of 6272 300; [128,96,112,112] 48 of 2720 433, 24 of 5432 476;
     // [128,64,56,56] 8 of 2720 78, 4 of 6272 84; bf16 [128,96,112,112] 24 of 2720 218, 20 of 3408 222, 12 of 5432 242, but
     // [256,512,28,28] 16 of 2792 163, one channel at a time 7 of 6272 158.
+    // Two channels side by side halve the share, and many short rounds lose all the same: from 1700 units each on (one / two channels /
+    // waves, us: f32 [140,7,96,97] at 1104 units 36 / 42 / 40, [92,11,128,127] at 1264 58 / 66 / 65, [11,90,96,96] at 1584 33.1 / 35.1 /
+    // 35.3, then [166,31,40,40] at 1800 32.7 / 32.0 / 34.7, [212,366,40,40] at 2296 346 / 341 / 400, [112,111,56,56] at 2376 120 / 112 /
+    // 131; bf16 [91,31,112,112] at 1936 63 / 59 / 70).  Where that leaves none it is one channel, or the waves.  For a list the
+    // other side is separate calls, and whoever plans it weighs those.
     const uint32_t runs = (uint32_t)((units + 7) / 8), C = tensors * (uint32_t)g.C;
+    const uint32_t least = tensors > 1 || tune.col_team == 1 ? 0u : kTLagUnits;
     uint64_t best = ~0ull;
     bool one_round = false;
     for (int depth = 1; depth <= (backward ? 2 : 1) && !one_round; ++depth) {
         const uint32_t hand_over = depth == 2 ? (dtype == 0 ? 250 : 340) : backward ? 700 : 2000;
         for (uint32_t R = 1; R <= ctas && R <= runs; ++R) {
             const uint32_t share = 8 * ((runs + R - 1) / R);
-            if (depth * share > kTSmemUnits) continue;
+            if (depth * share > kTSmemUnits || (depth == 2 && share < least)) continue;
             const uint32_t teams = std::min(ctas / R, C), rounds = (C + teams - 1) / teams;
             one_round |= rounds == 1;
             const uint64_t cost = (uint64_t)rounds * (share + hand_over);

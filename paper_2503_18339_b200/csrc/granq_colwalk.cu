@@ -566,15 +566,16 @@ ColPlan plan_colwalk(int dtype, const Geom& g, const QuantIO& io, const StagedTu
     return p;
 }
 
-// The resident form, unless a knob of the waves is set.  A hand-over costs a team several microseconds: where the rounds
-// are several and short (small channels) the waves are faster.  Measured over 20 shapes of 2 to 7 rounds (resident form /
+// The resident form, unless a knob of the waves is set.  Two channels side by side hide their hand-overs and are only planned
+// with shares that beat the waves (plan_colteam()).  One channel at a time, a hand-over costs a team several microseconds: where the
+// rounds are several and short (small channels) the waves are faster.  Measured over 20 shapes of 2 to 7 rounds (resident form /
 // waves): shares of 256 to 1600 units 1.17 to 1.01 forward, 1.16 to 0.98 with a gradient; 2000 to 2400 0.98 and 1.12 to
 // 0.93; from 2900 on 1.07 to 0.70 (3200 units in 3 rounds 1.07, in 6 0.85) and 1.04 to 0.85, so one line serves both.
 bool team_over_waves(const TeamPlan& plan, const Geom& g, const StagedTuning& tune) {
     if (!plan.ok || tune.col_team == 2) return false;
     if (tune.col_team == 1) return true;
     if (tune.l2_wave_kb > 0 || tune.l2_lag > 0 || tune.l2_ctas_per_sm > 0) return false;
-    return plan.tile_units >= 2500 || (g.C + plan.teams - 1) / plan.teams == 1;
+    return plan.lag || plan.tile_units >= 2500 || (g.C + plan.teams - 1) / plan.teams == 1;
 }
 
 cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
@@ -586,7 +587,7 @@ cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const TeamPlan tp = plan_colteam(dtype, g, io, mode == MODE_BOTH, sms);
+    const TeamPlan tp = plan_colteam(dtype, g, io, mode == MODE_BOTH, sms, tune);
     if (team_over_waves(tp, g, tune)) {
         e = launch_colteam(tp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, tune, st);
         if (e != cudaErrorCooperativeLaunchTooLarge) return e;      // else the waves, whose grid follows the occupancy

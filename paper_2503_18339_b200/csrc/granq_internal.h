@@ -230,7 +230,8 @@ struct TeamPlan {
     uint32_t smem_bytes;     // dynamic shared memory per CTA
 };
 // tensors: that many of these dims in one launch
-TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count, uint32_t tensors = 1);
+TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count, const StagedTuning& tune,
+                      uint32_t tensors = 1);
 // does the column walk take this form rather than the waves?
 bool team_over_waves(const TeamPlan& plan, const Geom& g, const StagedTuning& tune);
 // may be refused: launch_cooperative()

@@ -310,3 +310,29 @@ def test_team_plan_cuts_within_its_limits_and_takes_over_where_it_should(lib):
     finally:
         for k in range(b.N_KNOBS):
             b.tune(k, 0)
+
+
+def test_no_channel_that_a_team_would_take_alone_is_left_to_the_waves(lib):
+    """Host-only: where one channel at a time has one round or long shares, the plan with a gradient is taken too, be it that
+    one or two channels side by side; the shapes named are ones whose two-channel shares are short."""
+    from paper_2503_18339_b200 import binding as b
+    rnd = random.Random(14)
+
+    def one_channel(units, C, ctas):
+        runs = -(-units // 8)
+        cuts = [(-(-C // min(ctas // R, C)), 8 * -(-runs // R)) for R in range(1, min(ctas, runs) + 1)]
+        return min((rounds * (share + 700), rounds, share) for rounds, share in cuts if share <= 111 * 1024 // 16)[1:]
+
+    named = [(0, (222, 96, 80, 80)), (0, (112, 111, 56, 56)), (0, (212, 366, 40, 40)), (0, (143, 15, 64, 64)), (0, (143, 7, 96, 96)),
+             (1, (69, 56, 96, 96)), (1, (45, 328, 128, 127)), (0, (11, 90, 96, 96))]
+    drawn = [(rnd.choice([0, 1]), (rnd.randint(8, 256), rnd.randint(3, 500), rnd.choice([28, 40, 56, 96, 112]), rnd.choice([28, 48, 56, 80])))
+             for _ in range(400)]
+    two = 0
+    for dt, shape in named + drawn:
+        geo = b.team_geometry(dt, shape)
+        if geo is None:
+            continue
+        rounds, share = one_channel(shape[0] * shape[2] * shape[3] // (4, 8)[dt], shape[1], 296)
+        assert geo["taken"] == 1 or (rounds > 1 and share < 2500), (dt, shape)
+        two += geo["rounds"] > rounds
+    assert two > 100
