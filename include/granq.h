@@ -467,6 +467,13 @@ int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
                         int64_t out[4]);
 
 /*
+ * Host-only query: how many of the first tensors of a list of `n_tensors` of these dims granq_fakequant_fused_batch() would launch
+ * together on a device with `sm_count` SMs - with gradients, 16-byte aligned, sharing no memory, all workspaces handed over as
+ * zero.  0: each is a call of its own; negative = -status.
+ */
+int granq_batch_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int n_tensors, int sm_count);
+
+/*
  * Device self-test (no counterpart in the paper).  The staged kernel divides by the
  * per-group scale with a product and two exact-residual corrections from the correctly
  * rounded reciprocal; this runs `pairs` generated (x, s) pairs, hard cases included,

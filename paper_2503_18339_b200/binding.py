@@ -41,7 +41,7 @@ EXPORTS = [
     "granq_weights_workspace_bytes", "granq_fakequant_weights", "granq_packed_codes_bytes",
     "granq_quantize_packed", "granq_dequantize_packed", "granq_cluster_geometry", "granq_distortion_stats",
     "granq_accumulate_workspace_bytes", "granq_accumulate_codes", "granq_fakequant_fused_batch",
-    "granq_quantize_packed_fused", "granq_rows_geometry", "granq_team_geometry",
+    "granq_quantize_packed_fused", "granq_rows_geometry", "granq_team_geometry", "granq_batch_geometry",
 ]
 NOALLOC_MAX_GROUPS = 32768
 
@@ -123,6 +123,8 @@ def lib() -> ctypes.CDLL:
         L.granq_cluster_geometry.argtypes = [ci, i64p, ci, ci, ci, i64p]
         L.granq_team_geometry.restype = ci
         L.granq_team_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, i64p]
+        L.granq_batch_geometry.restype = ci
+        L.granq_batch_geometry.argtypes = [ci, i64p, ci, ci, ci, ci]
         L.granq_rows_geometry.restype = ci
         L.granq_rows_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, i64p]
         L.granq_selftest_division.restype = ci
@@ -328,6 +330,14 @@ def rows_geometry(dtype: int, shape, channel_axis: int = 3, group: int = GROUP_C
         return None
     _check(rc, "granq_rows_geometry")
     return dict(zip(["columns", "slices", "lanes", "team"], [int(v) for v in out]))
+
+
+def batch_geometry(dtype: int, shape, n_tensors: int, channel_axis: int = 1, group: int = GROUP_CHANNEL, sm_count: int = 148):
+    """Host-only: how many tensors at the head of a list of `n_tensors` of this shape go in one launch; 0 where none do."""
+    n = lib().granq_batch_geometry(dtype, _dims(shape), channel_axis, group, n_tensors, sm_count)
+    if n < 0:
+        raise GranqError(-n, "granq_batch_geometry")
+    return n
 
 
 @dataclass

@@ -466,8 +466,30 @@ static bool batch_conflict(const granq_fused_desc& a, const granq_fused_desc& b,
     return false;
 }
 
-// Tensors of a list from `first` on that one launch of the resident walk takes together: with a gradient, of the same dims, on
-// workspaces handed over as zero, sharing no memory.  0: none, each is a call of its own.
+// How many of the first tensors of a list of `count` of these dims, each with a gradient and sharing no memory, one launch of the
+// resident walk takes together; 0: none, each is a call of its own.  bf16 gains nothing (seven of [256,16,32,32] 51.9 / 56.1 us, three
+// of [16,64,56,56] 21.1 / 21.3).  Where no cluster holds a channel, the separate calls are resident walks one after the other and
+// together takes 0.53 to 0.97 of their time (two to sixteen tensors of 6 to 40 MB).  Where one does, they are cluster-local kernels that
+// run beside one another, and together pays only for many CTAs: of channels of 220 KB and more, whose tiles leave a cluster few
+// neighbours, or of few slabs, which a cluster cannot share out evenly.  Of 1400 lists, separate / together, us: six of
+// [232,32,16,16] 46 / 42, but of [214,32,16,16] 33 / 39, and four of [256,32,16,16] 33 / 33; six of [160,16,32,32] 51 / 55; three of
+// [8,72,80,80] 72 / 40; two of [70,256,14,14] 25 / 31.  Those that pass: 0.52 to 1.02, mean 0.85.  Of the others many would be up to
+// 1.5 times as slow; some long lists would gain a fifth.
+static int list_takes(int dtype, const Geom& g, int count, int sms, TeamPlan& plan) {
+    count = count < (int)kTeamListMax ? count : (int)kTeamListMax;
+    if (dtype != GRANQ_F32 || count < 2 || g.C >= (1ll << 28)) return 0;
+    const ClusterPlan kp = plan_cluster(dtype, g, QuantIO{}, true, g_tune);      // null pointers: alignment is assumed
+    if (kp.ok) {
+        const int64_t ctas = count * ((g.C + kp.k - 1) / kp.k * kp.R);
+        const bool large = g.E / g.C >= (220 << 10) / 4, few_slabs = g.outer <= 3 * (int64_t)kp.R;
+        if (!(large && ctas >= 9ll * sms) && !(few_slabs && ctas >= 5ll * sms)) return 0;
+    }
+    plan = plan_colteam(dtype, g, QuantIO{}, true, sms, g_tune, (uint32_t)count);
+    return plan.ok && plan.lag ? count : 0;
+}
+
+// Tensors of a list from `first` on that are launched together (list_takes()): on workspaces handed over as zero.  0: none; -1: the
+// launch failed.
 static int batch_together(const granq_fused_desc* descs, int first, int n_tensors, int dtype, int channel_axis, int group,
                           uint32_t flags, void* cuda_stream) {
     const StagedTuning& t = g_tune;
@@ -476,35 +498,36 @@ static int batch_together(const granq_fused_desc* descs, int first, int n_tensor
         return 0;
     Geom g;
     int64_t G;
-    if (!make_geom(descs[first].dims, channel_axis, group, g, G) || G >= (1ll << 28)) return 0;
+    int dev = 0, sms = 0;
+    if (!make_geom(descs[first].dims, channel_axis, group, g, G) || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    auto like_first = [&](int k) {
+        for (int i = 0; i < 4; ++i)
+            if (descs[first + k].dims[i] != descs[first].dims[i]) return false;
+        return true;
+    };
+    int alike = 1;
+    while (first + alike < n_tensors && alike < (int)kTeamListMax && like_first(alike)) ++alike;
+    TeamPlan plan{};
+    if (list_takes(dtype, g, alike, sms, plan) == 0) return 0;
     const size_t nb = (size_t)g.E * elt_size(dtype);
-    // bf16 gains nothing (seven of [256,16,32,32] 51.9 / 56.1, three of [16,64,56,56] 21.1 / 21.3)
-    if (dtype != GRANQ_F32 || nb < (8u << 20)) return 0;
     TeamTensor tensors[kTeamListMax];
     int n = 0;
-    for (; first + n < n_tensors && n < (int)kTeamListMax; ++n) {
+    for (; n < alike; ++n) {
         const granq_fused_desc& d = descs[first + n];
         bool fits = d.x && d.gy_opt && d.y && d.gx_opt && d.min_out && d.max_out && d.bits >= 1 && d.bits <= 8 &&
                     !(((uintptr_t)d.x | (uintptr_t)d.gy_opt | (uintptr_t)d.y | (uintptr_t)d.gx_opt) & 15) &&
                     check_workspace(d.workspace, d.workspace_bytes, G) == GRANQ_OK &&
                     !(overlaps(d.x, nb, d.y, nb) || overlaps(d.x, nb, d.gx_opt, nb) || overlaps(d.gy_opt, nb, d.y, nb) ||
                       overlaps(d.gy_opt, nb, d.gx_opt, nb) || overlaps(d.y, nb, d.gx_opt, nb));
-        for (int k = 0; fits && k < 4; ++k) fits = d.dims[k] == descs[first].dims[k];
         for (int k = 0; fits && k < n; ++k) fits = !batch_conflict(descs[first + k], d, dtype, channel_axis, group);
         if (!fits) break;
         tensors[n] = {QuantIO{d.x, d.gy_opt, d.y, d.gx_opt}, d.bits, carve_workspace(d.workspace, G), d.min_out, d.max_out,
                       d.scale_opt, d.zp_opt};
     }
-    int dev = 0, sms = 0;
-    // From 12 MB of x on (two of [256,16,32,32], 16 MB, 37.5 / 27.7; three of [16,64,56,56], 12 MB, 41.9 / 31.6), or 8 MB where
-    // there are 48 MB of them ([256,32,16,16]: six 46.4 / 42.0, three 22.2 / 22.3): of smaller ones the cluster-local kernels run
-    // beside one another and have no hand-over over the GPU (six of [256,64,8,8], 4 MB, 20.2 / 23.3).
-    if (n < 2 || (nb < (12u << 20) && n * nb < (48u << 20)) || cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 0;
-    const TeamPlan p = plan_colteam(dtype, g, tensors[0].io, true, sms, g_tune, (uint32_t)n);
-    if (!p.ok || !p.lag) return 0;
-    const cudaError_t e = launch_colteam_list(p, tensors, (uint32_t)n, dtype, g, g_tune, (cudaStream_t)cuda_stream);
+    if (n < alike && list_takes(dtype, g, n, sms, plan) == 0) return 0;
+    const cudaError_t e = launch_colteam_list(plan, tensors, (uint32_t)n, dtype, g, g_tune, (cudaStream_t)cuda_stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) return 0;
     return e == cudaSuccess ? n : -1;
 }
@@ -861,6 +884,14 @@ int granq_team_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
     const int64_t v[5] = {p.R, p.teams, (p.lag ? 2 : 1) * p.tile_units, (g.C + p.teams - 1) / p.teams, team_over_waves(p, g, g_tune) ? 1 : 0};
     for (int i = 0; i < 5; ++i) out[i] = v[i];
     return GRANQ_OK;
+}
+
+int granq_batch_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int n_tensors, int sm_count) {
+    Geom g;
+    int64_t G;
+    if (!dtype_ok(dtype) || n_tensors < 0 || sm_count < 1 || !make_geom(dims, channel_axis, group, g, G)) return -GRANQ_ERR_INVALID_ARG;
+    TeamPlan plan{};
+    return list_takes(dtype, g, n_tensors, sm_count, plan);
 }
 
 int granq_tune(int knob, int value) {

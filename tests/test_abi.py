@@ -336,3 +336,18 @@ def test_no_channel_that_a_team_would_take_alone_is_left_to_the_waves(lib):
         assert geo["taken"] == 1 or (rounds > 1 and share < 2500), (dt, shape)
         two += geo["rounds"] > rounds
     assert two > 100
+
+
+def test_lists_go_together_where_that_is_the_faster_way(lib):
+    """Host-only: lists that measured slower in one launch than as separate calls are separate, those that measured faster
+    go together, and neighbouring batch sizes take the same way."""
+    from paper_2503_18339_b200 import binding as b
+    for shape, n in (((70, 256, 14, 14), 2), ((488, 128, 7, 8), 12), ((854, 64, 8, 8), 4), ((70, 64, 28, 28), 6), ((183, 16, 32, 32), 6),
+                     ((160, 16, 32, 32), 7), ((256, 32, 16, 16), 4), ((200, 32, 16, 16), 6), ((10, 128, 32, 32), 4), ((256, 64, 8, 8), 6),
+                     ((256, 16, 32, 32), 1)):
+        assert b.batch_geometry(b.F32, shape, n) == 0, (shape, n)
+    for shape, n in (((256, 32, 16, 16), 6), ((255, 32, 16, 16), 6), ((232, 32, 16, 16), 6), ((256, 16, 32, 32), 7), ((255, 16, 32, 32), 2),
+                     ((17, 144, 56, 56), 2), ((8, 72, 80, 80), 3), ((977, 64, 8, 8), 6), ((249, 72, 16, 16), 12), ((128, 64, 56, 56), 6)):
+        assert b.batch_geometry(b.F32, shape, n) == n, (shape, n)
+    assert b.batch_geometry(b.F32, (256, 16, 32, 32), 40) == 16
+    assert b.batch_geometry(b.BF16, (256, 32, 32, 32), 8) == 0
