@@ -72,7 +72,7 @@ struct TArgs {
     uint32_t gy_units;     // of a CTA's share of gy, this many units are staged behind it
     uint32_t spin_limit, expected;
     uint32_t early;        // x and gy may be read before the kernel ahead has completed: it only clears the workspace
-    uint32_t slab_units;   // units of one slab
+    uint64_t slab_units;   // units of one slab
     FastDiv div_plane;     // units per plane
 };
 
@@ -338,10 +338,10 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
     // where they are: unit q lies in slab q / plane_units, and the next one of this thread is kTWork units on
     uint32_t slab0, off0;
     a.div_plane.divmod(q0 + min(tid, n), slab0, off0);
-    const uint32_t first = slab0 * a.slab_units + off0;
+    const uint32_t slab_units = (uint32_t)a.slab_units, first = slab0 * slab_units + off0;      // a tensor has less than 2^32 units
     uint32_t dslab, doff;
     a.div_plane.divmod((uint32_t)kTWork, dslab, doff);
-    const uint32_t dstep = dslab * a.slab_units + doff, dwrap = a.slab_units - a.plane_units;
+    const uint32_t dstep = dslab * slab_units + doff, dwrap = slab_units - a.plane_units;
     auto advance = [&](uint32_t& at, uint32_t& off) {
         at += dstep;
         off += doff;
@@ -563,7 +563,6 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
     const uint64_t units = (uint64_t)g.outer * (uint64_t)(g.inner / V);
     const uint32_t ctas = 2u * (uint32_t)sm_count;
     if (units >= (1ull << 30) || units > (uint64_t)ctas * (kTSmemUnits - 8)) return p;
-    if (units * (uint64_t)g.C >= (1ull << 32)) return p;      // 32-bit unit indexes
     // What a hand-over costs, in units that one CTA moves meanwhile: about 3 us, from sweeps over R (forward
     // [128,64,56,56]: 4 rounds of 5576 units 47 us, 8 of 2720 60 us, 16 of 1360 85 us; with gradient 84, 90, 115 us).  With a
     // gradient and several rounds, two channels side by side hide most of it: [256,512,28,28] 32 rounds of 2792 units 283 us, 29
@@ -579,7 +578,8 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
     const uint32_t least = tensors > 1 || tune.col_team == 1 ? 0u : kTLagUnits;
     uint64_t best = ~0ull;
     bool one_round = false;
-    for (int depth = 1; depth <= (backward ? 2 : 1) && !one_round; ++depth) {
+    const int most = backward && units * (uint64_t)g.C < (1ull << 32) ? 2 : 1;      // two channels: 32-bit unit indexes
+    for (int depth = 1; depth <= most && !one_round; ++depth) {
         const uint32_t hand_over = depth == 2 ? (dtype == 0 ? 250 : 340) : backward ? 700 : 2000;
         for (uint32_t R = 1; R <= ctas && R <= runs; ++R) {
             const uint32_t share = 8 * ((runs + R - 1) / R);
@@ -609,7 +609,7 @@ cudaError_t launch_colteam_list(const TeamPlan& plan, const TeamTensor* tensors,
     a.C = (uint32_t)g.C;
     a.plane_units = (uint32_t)(g.inner / (dtype == 0 ? 4 : 8));
     a.units = (uint32_t)((uint64_t)g.outer * a.plane_units);
-    a.slab_units = (uint32_t)((uint64_t)a.C * a.plane_units);
+    a.slab_units = (uint64_t)a.C * a.plane_units;
     a.R = plan.R;
     a.teams = plan.teams;
     a.tile_units = plan.tile_units;
@@ -658,7 +658,7 @@ cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, in
     a.C = (uint32_t)g.C;
     a.plane_units = (uint32_t)(g.inner / V);
     a.units = (uint32_t)((uint64_t)g.outer * a.plane_units);
-    a.slab_units = (uint32_t)((uint64_t)a.C * a.plane_units);
+    a.slab_units = (uint64_t)a.C * a.plane_units;
     a.R = plan.R;
     a.teams = plan.teams;
     a.tile_units = plan.tile_units;

@@ -351,3 +351,12 @@ def test_lists_go_together_where_that_is_the_faster_way(lib):
         assert b.batch_geometry(b.F32, shape, n) == n, (shape, n)
     assert b.batch_geometry(b.F32, (256, 16, 32, 32), 40) == 16
     assert b.batch_geometry(b.BF16, (256, 32, 32, 32), 8) == 0
+
+
+def test_teams_take_tensors_of_more_than_2_32_units(lib):
+    """Host-only: 64 GB and more (one channel at a time: two side by side count units in 32 bits)."""
+    from paper_2503_18339_b200 import binding as b
+    for dt, shape in ((0, (2048, 6000, 32, 48)), (1, (2048, 6000, 64, 48))):
+        for bwd in (False, True):
+            geo = b.team_geometry(dt, shape, with_backward=bwd)
+            assert geo["taken"] == 1 and geo["ctas"] * geo["units"] >= 2048 * 32 * 48 // 4
