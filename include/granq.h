@@ -419,7 +419,8 @@ int granq_host_arena_status(int dtype, const int64_t dims[4], int channel_axis, 
  * device: 0 = two-pass, 1 = naive per-channel loop, 2 = on-chip staged, 3 = L2-resident waves,
  * 4 = column walk, 5 = cluster-local, 6 = channels-last rows; negative = -status.  Plan 4 covers two kernels, the
  * resident form and the waves: granq_team_geometry() tells which.  The resident form also runs in place of plan 5
- * for x of 96 MB and more (128 MB for fp32 with a gradient) in channels of at least 256 KB.
+ * for x of 96 MB and more (128 MB for fp32 with a gradient) in channels of at least 256 KB.  Where granq_hold_geometry() says
+ * so, plans 0 and 3 run as one launch that holds the tensor on chip piece by piece.
  * `launches_out` (HOST, may be NULL) receives the number of kernel launches of that plan.
  */
 int granq_fused_plan(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward,
@@ -464,6 +465,16 @@ int granq_team_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
  * there would be slices (a call then takes two passes).
  */
 int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward, int sm_count,
+                        int64_t out[4]);
+
+/*
+ * Host-only query: how the launch that holds a tensor on chip piece by piece would cut this tensor on a device with `sm_count` SMs;
+ * `packed`: for packed masks and packed codes (forward only) rather than for y and gx.
+ * out = { CTAs, 16-byte units of one CTA, of those kept in shared memory (the others are read again), 1 if
+ *         granq_fakequant_fused() / granq_fakequant_fused_fwd_packmask() and granq_quantize_packed_fused() take it by default }.
+ * Returns GRANQ_ERR_UNSUPPORTED when the geometry does not qualify.
+ */
+int granq_hold_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward, int packed, int sm_count,
                         int64_t out[4]);
 
 /*

@@ -42,6 +42,7 @@ EXPORTS = [
     "granq_quantize_packed", "granq_dequantize_packed", "granq_cluster_geometry", "granq_distortion_stats",
     "granq_accumulate_workspace_bytes", "granq_accumulate_codes", "granq_fakequant_fused_batch",
     "granq_quantize_packed_fused", "granq_rows_geometry", "granq_team_geometry", "granq_batch_geometry",
+    "granq_hold_geometry",
 ]
 NOALLOC_MAX_GROUPS = 32768
 
@@ -123,6 +124,8 @@ def lib() -> ctypes.CDLL:
         L.granq_cluster_geometry.argtypes = [ci, i64p, ci, ci, ci, i64p]
         L.granq_team_geometry.restype = ci
         L.granq_team_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, i64p]
+        L.granq_hold_geometry.restype = ci
+        L.granq_hold_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, ci, i64p]
         L.granq_batch_geometry.restype = ci
         L.granq_batch_geometry.argtypes = [ci, i64p, ci, ci, ci, ci]
         L.granq_rows_geometry.restype = ci
@@ -330,6 +333,18 @@ def rows_geometry(dtype: int, shape, channel_axis: int = 3, group: int = GROUP_C
         return None
     _check(rc, "granq_rows_geometry")
     return dict(zip(["columns", "slices", "lanes", "team"], [int(v) for v in out]))
+
+
+def hold_geometry(dtype: int, shape, channel_axis: int = 1, group: int = GROUP_CHANNEL, with_backward: bool = True,
+                  packed: bool = False, sm_count: int = 148):
+    """Host-only: the cut of the launch that holds a tensor on chip piece by piece, for y and gx or (`packed`) packed masks and
+    codes, and whether calls take it by default ("taken"); None if the geometry does not qualify."""
+    out = (ctypes.c_int64 * 4)()
+    rc = lib().granq_hold_geometry(dtype, _dims(shape), channel_axis, group, int(with_backward), int(packed), sm_count, out)
+    if rc == ERR_UNSUPPORTED:
+        return None
+    _check(rc, "granq_hold_geometry")
+    return dict(zip(["ctas", "units", "kept", "taken"], [int(v) for v in out]))
 
 
 def batch_geometry(dtype: int, shape, n_tensors: int, channel_axis: int = 1, group: int = GROUP_CHANNEL, sm_count: int = 148):

@@ -136,11 +136,14 @@ cudaError_t launch_held(const TeamPlan& tp, const ClusterPlan& kp, const QuantIO
     return launch_cluster(kp, io, mode, dtype, g, bits, ws, lo, hi, s_opt, z_opt, g_tune, st);
 }
 
-// Where a call would take two passes or the L2-resident waves, not because it asked to: one launch that holds the tensor on
-// chip (what it gains stands at the kernel).
+// Where a call would take two passes or the L2-resident waves, not because it or a knob of the waves asked for them: one launch that
+// holds the tensor on chip (what it gains stands at the kernel).
+bool hold_allowed(uint32_t flags) {
+    return !(flags & (GRANQ_FLAG_FORCE_TWO_PASS | GRANQ_FLAG_FORCE_L2WAVE)) && !g_tune.l2_wave_kb && !g_tune.l2_upl && !g_tune.l2_ctas_per_sm;
+}
 HoldPlan prefer_hold(int dtype, const Geom& g, const QuantIO& io, uint32_t flags) {
     HoldPlan none{};
-    if (flags & GRANQ_FLAG_FORCE_TWO_PASS) return none;
+    if (!hold_allowed(flags)) return none;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -271,8 +274,7 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
     // keep that word true for the next call, after.
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     kp.zero_status = !zeroed && kp.clears_status;
-    const HoldPlan hp = plan == PLAN_TWO_PASS || (plan == PLAN_L2WAVE && !(flags & GRANQ_FLAG_FORCE_L2WAVE))
-                            ? prefer_hold(dtype, g, io, flags) : HoldPlan{};
+    const HoldPlan hp = plan == PLAN_TWO_PASS || plan == PLAN_L2WAVE ? prefer_hold(dtype, g, io, flags) : HoldPlan{};
     bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS || hp.ok;
     TeamPlan tp{};
     if (plan == PLAN_CLUSTER) tp = prefer_team(dtype, g, io, gy_opt != nullptr, flags);
@@ -819,12 +821,22 @@ int granq_host_arena_status(int dtype, const int64_t dims[4], int channel_axis, 
     return granq_workspace_status(ws, cuda_stream);
 }
 
+// Stand-ins for a call's arrays, 16-byte aligned, for what a query asks of a plan.
+static QuantIO aligned_io(bool backward, bool packed) {
+    QuantIO io{};
+    void* const some = (void*)256;
+    io.x = io.y = some;
+    if (backward) io.gy = io.gx = some;
+    if (packed) io.pmask = (uint32_t*)some;
+    return io;
+}
+
 int granq_fused_plan(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward,
                      uint32_t flags, int* launches_out) {
     Geom g;
     int64_t G;
     if (!dtype_ok(dtype) || !make_geom(dims, channel_axis, group, g, G)) return -GRANQ_ERR_INVALID_ARG;
-    QuantIO io{};   // null pointers: alignment is assumed
+    const QuantIO io = aligned_io(with_backward != 0, false);
     const int plan = choose_plan(dtype, g, io, with_backward != 0, flags, nullptr, nullptr, nullptr, nullptr);
     if (launches_out) {
         const bool held = plan == PLAN_TWO_PASS && prefer_hold(dtype, g, io, flags).ok;
@@ -883,6 +895,24 @@ int granq_team_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
     if (!p.ok) return GRANQ_ERR_UNSUPPORTED;
     const int64_t v[5] = {p.R, p.teams, (p.lag ? 2 : 1) * p.tile_units, (g.C + p.teams - 1) / p.teams, team_over_waves(p, g, g_tune) ? 1 : 0};
     for (int i = 0; i < 5; ++i) out[i] = v[i];
+    return GRANQ_OK;
+}
+
+int granq_hold_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward, int packed, int sm_count,
+                        int64_t out[4]) {
+    Geom g;
+    int64_t G;
+    if (!out || !dtype_ok(dtype) || sm_count < 1 || (with_backward && packed) || !make_geom(dims, channel_axis, group, g, G))
+        return GRANQ_ERR_INVALID_ARG;
+    const bool backward = with_backward != 0;
+    const QuantIO io = aligned_io(backward, packed != 0);
+    const HoldPlan p = plan_hold(dtype, g, io, sm_count);
+    if (!p.ok) return GRANQ_ERR_UNSUPPORTED;
+    const int plan = packed ? (plan_cluster(dtype, g, io, false, g_tune).ok || plan_colwalk(dtype, g, io, g_tune).ok ? PLAN_COLWALK : PLAN_TWO_PASS)
+                            : choose_plan(dtype, g, io, backward, 0, nullptr, nullptr, nullptr, nullptr);
+    const bool taken = (plan == PLAN_TWO_PASS || plan == PLAN_L2WAVE) && hold_allowed(0);
+    const int64_t v[4] = {p.ctas, p.share, p.held, taken ? 1 : 0};
+    for (int i = 0; i < 4; ++i) out[i] = v[i];
     return GRANQ_OK;
 }
 

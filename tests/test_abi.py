@@ -360,3 +360,38 @@ def test_teams_take_tensors_of_more_than_2_32_units(lib):
         for bwd in (False, True):
             geo = b.team_geometry(dt, shape, with_backward=bwd)
             assert geo["taken"] == 1 and geo["ctas"] * geo["units"] >= 2048 * 32 * 48 // 4
+
+
+def test_held_form_cuts_within_its_limits_and_leaves_the_waves_to_their_knobs(lib):
+    """Host-only: pieces cover the tensor and fit half an SM's shared memory; more is read again of one group only, of fp32
+    with a gradient nothing; a knob of the L2-resident waves keeps one group on them."""
+    from paper_2503_18339_b200 import binding as b
+    rnd = random.Random(15)
+    again = 0
+    try:
+        for _ in range(3000):
+            dt, sms = rnd.choice([0, 1]), rnd.choice([8, 132, 148])
+            bwd = rnd.choice([False, True])
+            packed = not bwd and rnd.choice([False, True])
+            mode = rnd.choice([0, 1, 2])
+            shape = (rnd.choice([1, 8, 13, 64, 128]), rnd.randint(1, 300), rnd.choice([5, 7, 14, 27, 56]), rnd.choice([4, 7, 15, 28, 56]))
+            geo = b.hold_geometry(dt, shape, group=mode, with_backward=bwd, packed=packed, sm_count=sms)
+            if geo is None:
+                continue
+            V, E = (4, 8)[dt], shape[0] * shape[1] * shape[2] * shape[3]
+            assert E % (32 if packed else V) == 0 and geo["ctas"] <= 2 * sms
+            assert geo["ctas"] * geo["units"] >= E // V > (geo["ctas"] - 1) * geo["units"] and geo["units"] % 8 == 0
+            assert geo["kept"] % 2 == 0 and geo["kept"] * 16 <= 111 * 1024 and geo["kept"] <= geo["units"] <= 2 * geo["kept"] + 4
+            if geo["kept"] < geo["units"]:
+                again += 1
+                assert (mode == 2 or shape[1] == 1 and shape[0] == 1) and (dt == 1 or not bwd)
+        assert again > 20
+        one_group = dict(group=2, with_backward=False)
+        assert b.hold_geometry(0, (64, 64, 28, 28), **one_group)["taken"] == 1
+        for k in (b.KNOB_L2_WAVE_KB, b.KNOB_L2_UPL, b.KNOB_L2_CTAS_PER_SM):
+            b.tune(k, 2)
+            assert b.hold_geometry(0, (64, 64, 28, 28), **one_group)["taken"] == 0
+            b.tune(k, 0)
+    finally:
+        for k in range(b.N_KNOBS):
+            b.tune(k, 0)

@@ -24,11 +24,17 @@ CASES = [
     ((32, 5, 27, 27), 0),       # whole words of mask and codes
     ((8, 3, 111, 111), 0),      # a plane over many pieces
     ((24, 75, 27, 27), 0),      # several units to a thread
-    ((3, 7, 9, 24), 2),         # one group, fewer units than one CTA has threads
+    ((3, 7, 9, 24), 2),         # one group that a cluster holds instead
     ((5, 11, 40, 50), 2),       # one group, pieces that do not come out even
     ((32, 128, 28, 29), 2),     # one group over several units a thread
     ((3, 2, 256, 256), 1),      # planes of whole units, too long for a cluster to hold
 ]
+
+
+def takes(b, dtype, shape, mode, with_backward=False, packed=False):
+    """Does the call take the held form?"""
+    geo = b.hold_geometry(b.BF16 if dtype == "bf16" else b.F32, shape, group=mode, with_backward=with_backward, packed=packed)
+    return geo is not None and geo["taken"] == 1
 
 
 @pytest.mark.parametrize("shape,mode", CASES, ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else f"g{v}")
@@ -38,6 +44,8 @@ def test_held_tensor(b, shape, mode, dtype):
     bits = 2 + sum(shape) % 7
     ref = orc.fused(x, bits, gy=gy, group_mode=mode)
     xd, gyd = to_dev(x), to_dev(gy)
+    assert takes(b, dtype, shape, mode) == (x.size > 8192 or mode != 2)
+    assert takes(b, dtype, shape, mode, packed=True) == (x.size % 32 == 0)
     ws = b.make_workspace(xd, group=mode, zeroed=True)
     new = lambda: b.FakeQuantOut(workspace=ws)
     clean = lambda: b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
@@ -70,6 +78,7 @@ def test_one_group_beyond_what_stays_on_chip(b, dtype, shape):
     x, gy = make_case(shape, seed=3, dtype=dtype)
     ref = orc.fused(x, 4, gy=gy, group_mode=2)
     xd, gyd = to_dev(x), to_dev(gy)
+    assert takes(b, dtype, shape, 2) and takes(b, dtype, shape, 2, with_backward=True) == (dtype == "bf16")
     assert_parity(b.granq_fakequant_fused(xd, 4, gy=gyd, group=2), ref, shape, 1, 2, backward=True)
     assert_parity(b.granq_fakequant_fused(xd, 4, group=2), ref, shape, 1, 2, backward=False)
     got = b.granq_fakequant_fused_stats(xd, 4, group=2)
@@ -89,6 +98,8 @@ def test_packed_outputs_of_one_group_beyond_what_stays_on_chip(b, dtype, shape):
     x = np.clip(6.0 * np.random.default_rng(17).standard_normal(shape, dtype=np.float32), -7.5, 7.5)
     x = wl.to_bf16_bits(x) if dtype == "bf16" else x
     xd = to_dev(x)
+    geo = b.hold_geometry(b.BF16 if dtype == "bf16" else b.F32, shape, group=2, with_backward=False, packed=True)
+    assert geo["taken"] == 1 and geo["kept"] < geo["units"]
     zeroed = b.make_workspace(xd, group=2, zeroed=True)
     for code_bits in (1, 3, 4, 5, 8):
         ref = orc.fused(x, code_bits, group_mode=2)
@@ -108,6 +119,7 @@ def test_packed_outputs_of_one_group_beyond_what_stays_on_chip(b, dtype, shape):
 @pytest.mark.parametrize("stats", [False, True])
 def test_a_hand_over_that_never_completes_is_reported(b, knobs, stats):
     x, _ = make_case((8, 75, 5, 7), seed=1)
+    assert takes(b, "f32", x.shape, 0)
     xd = to_dev(x)
     call = b.granq_fakequant_fused_stats if stats else b.granq_fakequant_fused
     knobs(extra_arrivals=1, spin_limit=500)
@@ -121,6 +133,7 @@ def test_a_hand_over_that_never_completes_is_reported(b, knobs, stats):
 @pytest.mark.parametrize("shape,mode", [((24, 75, 27, 27), 0), ((5, 11, 40, 50), 2), ((3, 2, 256, 256), 1)])
 def test_a_refused_cooperative_launch_falls_back(b, knobs, shape, mode):
     x, gy = make_case(shape, seed=6)
+    assert takes(b, "f32", shape, mode) and takes(b, "f32", shape, mode, with_backward=True)
     ref = orc.fused(x, 4, gy=gy, group_mode=mode)
     xd, gyd = to_dev(x), to_dev(gy)
     ws = b.make_workspace(xd, group=mode, zeroed=True)
