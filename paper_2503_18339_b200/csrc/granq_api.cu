@@ -270,8 +270,8 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
     Workspace ws = carve_workspace(workspace, G);
     // The column-walk and channels-last kernels leave a zeroed workspace zeroed and the cluster-local kernel writes
     // nothing but the status word (0 where the caller did not vouch for it, or that a wait on its bulk copies ran
-    // out); with the caller's word that the workspace is zero on entry nothing has to be cleared.  The other plans clear before and, to
-    // keep that word true for the next call, after.
+    // out); with the caller's word that the workspace is zero on entry nothing has to be cleared.  The other plans, to keep that word
+    // true for the next call, clear after themselves.
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     kp.zero_status = !zeroed && kp.clears_status;
     const HoldPlan hp = plan == PLAN_TWO_PASS || plan == PLAN_L2WAVE ? prefer_hold(dtype, g, io, flags) : HoldPlan{};
@@ -281,7 +281,7 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
     cudaError_t e = cudaSuccess;
     if (plan == PLAN_CLUSTER && !tp.ok) {
         if (!zeroed && !kp.clears_status) e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);      // the status word
-    } else if (!(zeroed && keeps_zero)) {
+    } else if (!zeroed) {
         e = launch_clear(workspace, ws.clear_bytes, nullptr, st);
         ws.cleared = true;
     }
@@ -412,7 +412,7 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
         return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     }
     const HoldPlan hp = cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
-    if (!(zeroed && (cp.ok || hp.ok))) {
+    if (!zeroed) {
         e = launch_clear(workspace, ws.clear_bytes, nullptr, st);
         ws.cleared = true;
     }
@@ -625,8 +625,7 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
     const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     const HoldPlan hp = kp.ok || cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
     // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
-    const size_t clear = zeroed && (kp.ok || cp.ok || hp.ok) ? 0
-                         : !kp.ok || tp.ok ? ws.clear_bytes : kp.clears_status ? 0 : sizeof(uint32_t);
+    const size_t clear = zeroed ? 0 : !kp.ok || tp.ok ? ws.clear_bytes : kp.clears_status ? 0 : sizeof(uint32_t);
     cudaError_t e = launch_clear(workspace, clear, sums_out, st);
     ws.cleared = true;
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
@@ -712,7 +711,7 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
         return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, st));
     }
     const HoldPlan hp = cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
-    if (!(zeroed && (cp.ok || hp.ok))) {
+    if (!zeroed) {
         e = launch_clear(workspace, ws.clear_bytes, nullptr, st);
         ws.cleared = true;
     }
