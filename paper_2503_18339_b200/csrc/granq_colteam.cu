@@ -72,7 +72,7 @@ struct TArgs {
     uint32_t gy_units;     // of a CTA's share of gy, this many units are staged behind it
     uint32_t spin_limit, expected;
     uint32_t early;        // x and gy may be read before the kernel ahead has completed: it only clears the workspace
-    uint64_t slab_units;   // units of one slab
+    uint32_t slab_units;   // units of one slab (where there is more than one)
     FastDiv div_plane;     // units per plane
 };
 
@@ -338,10 +338,10 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
     // where they are: unit q lies in slab q / plane_units, and the next one of this thread is kTWork units on
     uint32_t slab0, off0;
     a.div_plane.divmod(q0 + min(tid, n), slab0, off0);
-    const uint32_t slab_units = (uint32_t)a.slab_units, first = slab0 * slab_units + off0;      // a tensor has less than 2^32 units
+    const uint32_t first = slab0 * a.slab_units + off0;
     uint32_t dslab, doff;
     a.div_plane.divmod((uint32_t)kTWork, dslab, doff);
-    const uint32_t dstep = dslab * slab_units + doff, dwrap = slab_units - a.plane_units;
+    const uint32_t dstep = dslab * a.slab_units + doff, dwrap = a.slab_units - a.plane_units;
     auto advance = [&](uint32_t& at, uint32_t& off) {
         at += dstep;
         off += doff;
@@ -561,6 +561,7 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
     if ((io.pmask || io.pcodes) && g.inner % 8 != 0) return p;
     if (io.codes || io.mask) return p;
     const uint64_t units = (uint64_t)g.outer * (uint64_t)(g.inner / V);
+    if (g.outer > 1 && (uint64_t)g.C * (uint64_t)(g.inner / V) >= (1ull << 32)) return p;      // the stride of slabs is 32 bits
     const uint32_t ctas = 2u * (uint32_t)sm_count;
     if (units >= (1ull << 30) || units > (uint64_t)ctas * (kTSmemUnits - 8)) return p;
     // What a hand-over costs, in units that one CTA moves meanwhile: about 3 us, from sweeps over R (forward
@@ -609,7 +610,7 @@ cudaError_t launch_colteam_list(const TeamPlan& plan, const TeamTensor* tensors,
     a.C = (uint32_t)g.C;
     a.plane_units = (uint32_t)(g.inner / (dtype == 0 ? 4 : 8));
     a.units = (uint32_t)((uint64_t)g.outer * a.plane_units);
-    a.slab_units = (uint64_t)a.C * a.plane_units;
+    a.slab_units = (uint32_t)((uint64_t)a.C * a.plane_units);
     a.R = plan.R;
     a.teams = plan.teams;
     a.tile_units = plan.tile_units;
@@ -658,7 +659,7 @@ cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, in
     a.C = (uint32_t)g.C;
     a.plane_units = (uint32_t)(g.inner / V);
     a.units = (uint32_t)((uint64_t)g.outer * a.plane_units);
-    a.slab_units = (uint64_t)a.C * a.plane_units;
+    a.slab_units = (uint32_t)((uint64_t)a.C * a.plane_units);
     a.R = plan.R;
     a.teams = plan.teams;
     a.tile_units = plan.tile_units;
