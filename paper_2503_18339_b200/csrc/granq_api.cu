@@ -157,7 +157,7 @@ HoldPlan prefer_hold(int dtype, const Geom& g, const QuantIO& io, uint32_t flags
 // being captured, takes the memset: up to `host_bound` elements, where the two cross.  Kernel / memset, us: channels-last fp32 of
 // 0.5 MB 10.8 / 9.5, 1.5 MB 10.8 / 10.5, 2 MB 11.3 / 12.3, bf16 of 0.5 MB 11.0 / 10.5, 1.5 MB 12.6 / 13.8; one group of 0.5 MB 10.9 / 9.9; range of
 // 4 MB fp32 14.3 / 13.6, ragged of 12 MB 14.8 / 16.5, of bf16 6 MB 14.7 / 16.6.
-constexpr int64_t kHostBoundHeld = 400'000, kHostBoundRange = 2'000'000;
+constexpr int64_t kHostBoundHeld = 1 << 18, kHostBoundRange = 2'000'000;
 cudaError_t clear_workspace(Workspace& ws, const Geom& g, int64_t host_bound, cudaStream_t st) {
     if (g.E <= host_bound) {
         cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
