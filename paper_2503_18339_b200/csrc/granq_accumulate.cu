@@ -968,8 +968,8 @@ extern "C" int granq_accumulate_codes(const uint32_t* packed_codes, const int64_
         !a_make_map(encode, &ml, lo, (uint64_t)out_channels, (uint64_t)L.Cpad, (uint32_t)BN))
         return GRANQ_ERR_CUDA;
 
-    if (launch_after(accumulate_weights_kernel, (unsigned)out_channels, 128, 0, st, weights, scale, zp, (int)L.C, (int)L.Cpad, hi,
-                     lo, bias, (uint32_t*)workspace) != cudaSuccess)
+    if (launch_after(kAnyLayout, accumulate_weights_kernel, (unsigned)out_channels, 128, 0, st, weights, scale, zp, (int)L.C,
+                     (int)L.Cpad, hi, lo, bias, (uint32_t*)workspace) != cudaSuccess)
         return GRANQ_ERR_CUDA;
     AArgs args{};
     args.y = y;

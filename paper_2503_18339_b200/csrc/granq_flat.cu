@@ -906,19 +906,20 @@ __global__ void __launch_bounds__(kThreads) dequant_packed_kernel(const uint32_t
 
 bool aligned16(const void* p) { return p == nullptr || ((uintptr_t)p & 15) == 0; }
 
-int flat_grid(const FlatGeom& f) {
+int sm_count() {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int64_t cap = (int64_t)sms * 8;
+    return sms;
+}
+
+int flat_grid(const FlatGeom& f) {
+    const int64_t cap = (int64_t)sm_count() * 8;
     return (int)(f.ntiles < cap ? f.ntiles : cap);
 }
 
 int range_rows_ctas() {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms * 4;
+    return sm_count() * 4;
 }
 
 template <typename T>
@@ -937,29 +938,25 @@ cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t*
         // chunks of slabs: enough blocks to fill the chip twice over, walks of at least 4 slabs
         const uint32_t chunks = std::max<uint32_t>(1, std::min<uint32_t>((2 * cap + ncol - 1) / ncol, outer / 4));
         constexpr int U = VF == 4 ? 8 : 4;
-        if (vec)
-            launch_after(range_cols_kernel<T, true, U>, ncol * chunks, kThreads, 0, st, (const uint4*)x, slab_units, outer, chunks, make_fastdiv(ncol), make_fastdiv((uint32_t)(g.inner / VF)), kmin,
-                kmax, end);
-        else
-            launch_after(range_cols_kernel<T, false, U>, ncol * chunks, kThreads, 0, st, (const uint4*)x, slab_units, outer, chunks, make_fastdiv(ncol), make_fastdiv((uint32_t)g.inner), kmin, kmax, end);
-    } else if (rows_ok) {
+        auto cols = [&](auto kern, uint32_t plane) {
+            return launch_after(kAnyLayout, kern, ncol * chunks, kThreads, 0, st, (const uint4*)x, slab_units, outer, chunks,
+                                make_fastdiv(ncol), make_fastdiv(plane), kmin, kmax, end);
+        };
+        return vec ? cols(range_cols_kernel<T, true, U>, (uint32_t)(g.inner / VF)) : cols(range_cols_kernel<T, false, U>, (uint32_t)g.inner);
+    }
+    if (rows_ok) {
         const uint32_t n_units = (uint32_t)(g.E / VF);
         int64_t rows = ((int64_t)n_units + 127) / 128, ctas = (rows + 2 * (kThreads / 32) - 1) / (2 * (kThreads / 32));
         const int64_t cap = (int64_t)range_rows_ctas();                 // 4 resident CTAs per SM at 64 registers
         int rgrid = (int)(ctas < cap ? ctas : cap);
-        if (vec)
-            launch_after(range_rows_kernel<T, true>, rgrid, kThreads, 0, st, (const uint4*)x, n_units, (uint32_t)g.inner,
-                                                                   make_fastdiv((uint32_t)(g.inner / VF)),
-                                                                   make_fastdiv((uint32_t)g.C), (uint32_t)g.C, kmin, kmax, end);
-        else
-            launch_after(range_rows_kernel<T, false>, rgrid, kThreads, 0, st, (const uint4*)x, n_units, (uint32_t)g.inner,
-                                                                    make_fastdiv((uint32_t)g.inner),
-                                                                    make_fastdiv((uint32_t)g.C), (uint32_t)g.C, kmin, kmax, end);
-    } else if (vec)
-        launch_after(range_flat_kernel<T, VF>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end);
-    else
-        launch_after(range_flat_kernel<T, 1>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end);
-    return cudaGetLastError();
+        auto by_rows = [&](auto kern, uint32_t plane) {
+            return launch_after(kAnyLayout, kern, rgrid, kThreads, 0, st, (const uint4*)x, n_units, (uint32_t)g.inner, make_fastdiv(plane),
+                                make_fastdiv((uint32_t)g.C), (uint32_t)g.C, kmin, kmax, end);
+        };
+        return vec ? by_rows(range_rows_kernel<T, true>, (uint32_t)(g.inner / VF)) : by_rows(range_rows_kernel<T, false>, (uint32_t)g.inner);
+    }
+    return vec ? launch_after(kAnyLayout, range_flat_kernel<T, VF>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end)
+               : launch_after(kAnyLayout, range_flat_kernel<T, 1>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end);
 }
 
 template <typename T, int MODE>
@@ -989,65 +986,27 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
     const bool ragged = !vec && g.inner >= VF && g.inner % VF != 0 && g.E % VF == 0 && !f.inner_big && aligned16(io.x) &&
                         aligned16(io.gy) && aligned16(io.y) && aligned16(io.gx) && ((uintptr_t)io.codes % 4 == 0) &&
                         ((uintptr_t)io.mask % 4 == 0);
+    // five blocks of a table each fill an SM
+    const int layout = sm_layout(100, (uint64_t)g.E * sizeof(T));
+    auto go = [&](auto kern) {
+        return launch_after(layout, kern, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask,
+                            io.pmask, io.dist, io.pcodes, io.code_bits, f, qmax, lo, hi);
+    };
     if constexpr (MODE == MODE_FWD) {
-        if ((vec || ragged) && pack_only && g.E % 32 == 0) {       // whole words of codes: the byte-wise writer
-            if (vec)
-                launch_after(quant_flat_kernel<T, VF, MODE, 3, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                    io.code_bits, f, qmax, lo, hi);
-            else
-                launch_after(quant_flat_kernel<T, VF, MODE, 3, true, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                    io.code_bits, f, qmax, lo, hi);
-            return cudaGetLastError();
-        }
-        if ((vec || ragged) && pack_only) {
-            if (vec)
-                launch_after(quant_flat_kernel<T, VF, MODE, 1, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                    io.code_bits, f, qmax, lo, hi);
-            else
-                launch_after(quant_flat_kernel<T, VF, MODE, 1, true, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                    io.code_bits, f, qmax, lo, hi);
-            return cudaGetLastError();
-        }
         const bool dist_only = io.dist != nullptr && io.y != nullptr && io.codes == nullptr && io.mask == nullptr &&
                                io.pmask == nullptr && io.pcodes == nullptr;
-        if ((vec || ragged) && dist_only) {
-            if (vec)
-                launch_after(quant_flat_kernel<T, VF, MODE, 4>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                    io.code_bits, f, qmax, lo, hi);
-            else
-                launch_after(quant_flat_kernel<T, VF, MODE, 4, false, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                    io.code_bits, f, qmax, lo, hi);
-            return cudaGetLastError();
-        }
-        if ((vec || ragged) && pmask_only) {
-            if (vec)
-                launch_after(quant_flat_kernel<T, VF, MODE, 2>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                    io.code_bits, f, qmax, lo, hi);
-            else
-                launch_after(quant_flat_kernel<T, VF, MODE, 2, false, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                    io.code_bits, f, qmax, lo, hi);
-            return cudaGetLastError();
-        }
+        if ((vec || ragged) && pack_only && g.E % 32 == 0)         // whole words of codes: the byte-wise writer
+            return vec ? go(quant_flat_kernel<T, VF, MODE, 3, true>) : go(quant_flat_kernel<T, VF, MODE, 3, true, true>);
+        if ((vec || ragged) && pack_only)
+            return vec ? go(quant_flat_kernel<T, VF, MODE, 1, true>) : go(quant_flat_kernel<T, VF, MODE, 1, true, true>);
+        if ((vec || ragged) && dist_only)
+            return vec ? go(quant_flat_kernel<T, VF, MODE, 4>) : go(quant_flat_kernel<T, VF, MODE, 4, false, true>);
+        if ((vec || ragged) && pmask_only)
+            return vec ? go(quant_flat_kernel<T, VF, MODE, 2>) : go(quant_flat_kernel<T, VF, MODE, 2, false, true>);
     }
-    if (ragged) {
-        if (extras)
-            launch_after(quant_flat_kernel<T, VF, MODE, 1, false, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                io.code_bits, f, qmax, lo, hi);
-        else
-            launch_after(quant_flat_kernel<T, VF, MODE, 0, false, true>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes,
-                io.code_bits, f, qmax, lo, hi);
-        return cudaGetLastError();
-    }
-    if (vec && extras)
-        launch_after(quant_flat_kernel<T, VF, MODE, 1>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y,
-                                                                        (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes, io.code_bits, f, qmax, lo, hi);
-    else if (vec)
-        launch_after(quant_flat_kernel<T, VF, MODE, 0>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y,
-                                                                         (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes, io.code_bits, f, qmax, lo, hi);
-    else
-        launch_after(quant_flat_kernel<T, 1, MODE, 1>, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y,
-                                                                       (T*)io.gx, io.codes, io.mask, io.pmask, io.dist, io.pcodes, io.code_bits, f, qmax, lo, hi);
-    return cudaGetLastError();
+    if (ragged) return extras ? go(quant_flat_kernel<T, VF, MODE, 1, false, true>) : go(quant_flat_kernel<T, VF, MODE, 0, false, true>);
+    if (vec) return extras ? go(quant_flat_kernel<T, VF, MODE, 1>) : go(quant_flat_kernel<T, VF, MODE, 0>);
+    return go(quant_flat_kernel<T, 1, MODE, 1>);
 }
 
 template <typename T, int MODE>
@@ -1076,11 +1035,11 @@ cudaError_t dequant_strings_bits(const uint32_t* pcodes, T* y, const Geom& g, co
     const uint32_t n = (uint32_t)(g.E / 8), last = (uint32_t)((g.E * BITS - 1) >> 5);
     const uint32_t per_cta = kThreads * 2, grid = (n + per_cta - 1) / per_cta;
     const FastDiv di = make_fastdiv((uint32_t)g.inner), dc = make_fastdiv((uint32_t)g.C);
-    if (g.inner % 8 == 0)
-        launch_after(dequant_strings_kernel<T, BITS, false>, grid, kThreads, 0, st, pcodes, y, n, last, (uint32_t)g.inner, di, dc, s, z);
-    else
-        launch_after(dequant_strings_kernel<T, BITS, true>, grid, kThreads, 0, st, pcodes, y, n, last, (uint32_t)g.inner, di, dc, s, z);
-    return cudaGetLastError();
+    auto go = [&](auto kern) {
+        return launch_after(sm_layout(0, (uint64_t)g.E * sizeof(T)), kern, grid, kThreads, 0, st, pcodes, y, n, last, (uint32_t)g.inner,
+                            di, dc, s, z);
+    };
+    return g.inner % 8 == 0 ? go(dequant_strings_kernel<T, BITS, false>) : go(dequant_strings_kernel<T, BITS, true>);
 }
 
 template <typename T>
@@ -1107,21 +1066,19 @@ cudaError_t launch_range(const void* x, int dtype, const Geom& g, uint32_t* kmin
                                      : range_flat_t<__nv_bfloat16>(x, g, kmin, kmax, end, st);
     if (e != cudaSuccess || fused) return e;
     const int grid = (int)((g.C + 255) / 256);
-    launch_after(finalize_range_kernel, grid, 256, 0, st, kmin, kmax, g.C, lo, hi, bits, s_opt, z_opt);
-    return cudaGetLastError();
+    return launch_after(kAnyLayout, finalize_range_kernel, grid, 256, 0, st, kmin, kmax, g.C, lo, hi, bits, s_opt, z_opt);
 }
 
 cudaError_t launch_clear(void* workspace, size_t bytes, double* sums_opt, cudaStream_t st) {
     const size_t words = bytes / 4, blocks = (words + 4 * kThreads - 1) / (4 * kThreads);
-    return launch_after(clear_kernel, (unsigned)std::max<size_t>(1, std::min<size_t>(blocks, 256)), kThreads, 0, st,
+    return launch_after(kAnyLayout, clear_kernel, (unsigned)std::max<size_t>(1, std::min<size_t>(blocks, 256)), kThreads, 0, st,
                         (uint32_t*)workspace, (uint32_t)words, sums_opt);
 }
 
 cudaError_t launch_params(const float* lo, const float* hi, int64_t G, int bits, float* s_opt, float* z_opt,
                           cudaStream_t st) {
     int grid = (int)((G + 255) / 256);
-    launch_after(params_kernel, grid, 256, 0, st, lo, hi, G, bits, s_opt, z_opt);
-    return cudaGetLastError();
+    return launch_after(kAnyLayout, params_kernel, grid, 256, 0, st, lo, hi, G, bits, s_opt, z_opt);
 }
 
 cudaError_t launch_quant_flat(const QuantIO& io, int mode, int dtype, const Geom& g, int bits, const float* lo,
@@ -1153,18 +1110,13 @@ cudaError_t launch_bwd_packmask(const void* gy, const uint32_t* pmask, void* gx,
     const int64_t units = vec ? E / VF : E;
     const int64_t per_cta = (int64_t)kThreads * kUnroll;
     const unsigned grid = (unsigned)((units + per_cta - 1) / per_cta);
-    if (dtype == 0) {
-        if (vec) launch_after(bwd_packmask_kernel<float, 4>, grid, kThreads, 0, st, (const float*)gy, pmask, (float*)gx, E);
-        else launch_after(bwd_packmask_kernel<float, 1>, grid, kThreads, 0, st, (const float*)gy, pmask, (float*)gx, E);
-    } else {
-        if (vec)
-            launch_after(bwd_packmask_kernel<__nv_bfloat16, 8>, grid, kThreads, 0, st, (const __nv_bfloat16*)gy, pmask,
-                                                                             (__nv_bfloat16*)gx, E);
-        else
-            launch_after(bwd_packmask_kernel<__nv_bfloat16, 1>, grid, kThreads, 0, st, (const __nv_bfloat16*)gy, pmask,
-                                                                             (__nv_bfloat16*)gx, E);
-    }
-    return cudaGetLastError();
+    auto go = [&](auto kern, auto zero) {
+        using T = decltype(zero);
+        return launch_after(sm_layout(0, (uint64_t)E * sizeof(T)), kern, grid, kThreads, 0, st, (const T*)gy, pmask, (T*)gx, E);
+    };
+    if (dtype == 0) return vec ? go(bwd_packmask_kernel<float, 4>, 0.0f) : go(bwd_packmask_kernel<float, 1>, 0.0f);
+    const __nv_bfloat16 zero{};
+    return vec ? go(bwd_packmask_kernel<__nv_bfloat16, 8>, zero) : go(bwd_packmask_kernel<__nv_bfloat16, 1>, zero);
 }
 
 cudaError_t launch_distortion(const void* x, const void* q, int dtype, int64_t E, double* sums, cudaStream_t st) {
@@ -1177,18 +1129,13 @@ cudaError_t launch_distortion(const void* x, const void* q, int dtype, int64_t E
     const int64_t per_cta = (int64_t)kThreads * 2;
     const int64_t ctas = (units + per_cta - 1) / per_cta, cap = (int64_t)sms * 8;
     const int grid = (int)(ctas < 1 ? 1 : (ctas < cap ? ctas : cap));
-    if (dtype == 0) {
-        if (vec) launch_after(distortion_kernel<float, 4>, grid, kThreads, 0, st, (const float*)x, (const float*)q, E, sums);
-        else launch_after(distortion_kernel<float, 1>, grid, kThreads, 0, st, (const float*)x, (const float*)q, E, sums);
-    } else {
-        if (vec)
-            launch_after(distortion_kernel<__nv_bfloat16, 8>, grid, kThreads, 0, st, (const __nv_bfloat16*)x,
-                                                                           (const __nv_bfloat16*)q, E, sums);
-        else
-            launch_after(distortion_kernel<__nv_bfloat16, 1>, grid, kThreads, 0, st, (const __nv_bfloat16*)x,
-                                                                           (const __nv_bfloat16*)q, E, sums);
-    }
-    return cudaGetLastError();
+    auto go = [&](auto kern, auto zero) {
+        using T = decltype(zero);
+        return launch_after(sm_layout(16, (uint64_t)E * sizeof(T)), kern, grid, kThreads, 0, st, (const T*)x, (const T*)q, E, sums);
+    };
+    if (dtype == 0) return vec ? go(distortion_kernel<float, 4>, 0.0f) : go(distortion_kernel<float, 1>, 0.0f);
+    const __nv_bfloat16 zero{};
+    return vec ? go(distortion_kernel<__nv_bfloat16, 8>, zero) : go(distortion_kernel<__nv_bfloat16, 1>, zero);
 }
 
 cudaError_t launch_dequant_packed(const uint32_t* pcodes, void* y, int dtype, const Geom& g, int bits,
@@ -1206,18 +1153,13 @@ cudaError_t launch_dequant_packed(const uint32_t* pcodes, void* y, int dtype, co
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t ctas = (units + kThreads - 1) / kThreads, cap = (int64_t)sms * 16;
     const int grid = (int)(ctas < 1 ? 1 : (ctas < cap ? ctas : cap));
-    if (dtype == 0) {
-        if (vec) launch_after(dequant_packed_kernel<float, 4>, grid, kThreads, 0, st, pcodes, (float*)y, g.E, g.inner, g.C, bits, s, z);
-        else launch_after(dequant_packed_kernel<float, 1>, grid, kThreads, 0, st, pcodes, (float*)y, g.E, g.inner, g.C, bits, s, z);
-    } else {
-        if (vec)
-            launch_after(dequant_packed_kernel<__nv_bfloat16, 8>, grid, kThreads, 0, st, pcodes, (__nv_bfloat16*)y, g.E, g.inner,
-                                                                               g.C, bits, s, z);
-        else
-            launch_after(dequant_packed_kernel<__nv_bfloat16, 1>, grid, kThreads, 0, st, pcodes, (__nv_bfloat16*)y, g.E, g.inner,
-                                                                               g.C, bits, s, z);
-    }
-    return cudaGetLastError();
+    auto go = [&](auto kern, auto zero) {
+        using T = decltype(zero);
+        return launch_after(sm_layout(0, (uint64_t)g.E * sizeof(T)), kern, grid, kThreads, 0, st, pcodes, (T*)y, g.E, g.inner, g.C, bits, s, z);
+    };
+    if (dtype == 0) return vec ? go(dequant_packed_kernel<float, 4>, 0.0f) : go(dequant_packed_kernel<float, 1>, 0.0f);
+    const __nv_bfloat16 zero{};
+    return vec ? go(dequant_packed_kernel<__nv_bfloat16, 8>, zero) : go(dequant_packed_kernel<__nv_bfloat16, 1>, zero);
 }
 
 }  // namespace granq

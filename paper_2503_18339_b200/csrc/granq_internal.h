@@ -100,18 +100,30 @@ inline cudaError_t allow_smem(K kern, size_t most) {
 // Launch of a kernel that begins with after_the_kernel_ahead(): its grid is set up while the kernel ahead of it in the stream
 // drains, which hides a launch's latency: weights of a network 20.5 -> 17.6 us, range, forward and backward of [128,960,7,7]
 // 41.0 -> 37.1, codes and back of [128,144,56,56] 128.7 -> 123.9.
+// smem_kb: the shared memory that an SM full of its blocks takes, or kAnyLayout.  Stating it keeps blocks off an SM that is still laid
+// out for the shared memory of the kernel ahead; once on it, one after the other would read through what that layout leaves of
+// the L1 until the last is done.  Worth it from 16 MB on (sm_layout()); below, starting early on any SM is worth more.  Stated / not, us:
+// packed mask and backward of fp32 [128,144,56,56] 173.1 / 184.9 and [41,1896,15,16] 60.7 / 64.8, fused call and backward from x of
+// [116,1240,16,15] 110.7 / 125.3, fused call and weights of a network 113.0 / 114.9; bf16 [212,568,7,8], 13 MB, fused call and backward 25.2 /
+// 23.9.
+constexpr int kAnyLayout = -1;
+inline int sm_layout(int smem_kb, uint64_t bytes) { return bytes >= (16ull << 20) ? smem_kb : kAnyLayout; }
 template <typename... P, typename... A>
-inline cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
+inline cudaError_t launch_after(int smem_kb, void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
+                                A&&... args) {
+    constexpr int kSmemKB = 228;           // of an SM; the attribute is a percentage of it
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = smem_kb < 0 ? 0u : (unsigned)(smem_kb * 100 / kSmemKB);
+    cfg.attrs = attr;
+    cfg.numAttrs = smem_kb == kAnyLayout ? 1 : 2;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 

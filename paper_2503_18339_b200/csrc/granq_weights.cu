@@ -223,12 +223,15 @@ cudaError_t w_launch_n(const WDesc* descs, int n, uint32_t blocks, cudaStream_t 
     constexpr uint32_t V = Pack<T>::V;
     WTable<N> tab;
     bool small = true;
+    uint64_t bytes = 0;
     for (int i = 0; i < n; ++i) {
         tab.d[i] = descs[i];
+        bytes += (uint64_t)descs[i].channels * descs[i].group_elems * sizeof(T);
         small = small && (descs[i].vec ? descs[i].group_elems / V : descs[i].group_elems) <= 32;
     }
-    if (small) return launch_after(weights_kernel<T, GRAD, N, 1>, blocks, kWThreads, 0, st, tab, (uint32_t)n);
-    return launch_after(weights_kernel<T, GRAD, N, kWHold>, blocks, kWThreads, 0, st, tab, (uint32_t)n);
+    const int layout = sm_layout(0, bytes);
+    if (small) return launch_after(layout, weights_kernel<T, GRAD, N, 1>, blocks, kWThreads, 0, st, tab, (uint32_t)n);
+    return launch_after(layout, weights_kernel<T, GRAD, N, kWHold>, blocks, kWThreads, 0, st, tab, (uint32_t)n);
 }
 
 template <typename T>
