@@ -707,13 +707,15 @@ __global__ void __launch_bounds__(kThreads) naive_quant_kernel(const T* __restri
 
 // ---- STE backward from the packed mask alone (Section 2.1): gx = gy where the element's bit is set ----
 // A stream, bound by HBM: a block per 1024 units, in the order of memory ([128,96,112,112] 200 -> 185 us against a
-// persistent grid).
+// persistent grid).  The kernel behind is not let start beside it: that is mostly one that takes an SM's shared memory (the next
+// layer's), which a stream of a wave or two is slower beside (packed mask and backward, us, with / without: bf16 [128,960,7,7] 26.0 / 21.2,
+// fp32 [25,856,14,14] 21.6 / 19.2, [41,1896,15,16] 60.8 / 60.3; 26 shapes 0.98).
 // V = elements per thread and step: a 16-byte pack when E and the pointers allow it, else 1.
 template <typename T, int V>
 __global__ void __launch_bounds__(kThreads) bwd_packmask_kernel(const T* __restrict__ gy,
                                                                 const uint32_t* __restrict__ pmask,
                                                                 T* __restrict__ gx, int64_t E) {
-    after_the_kernel_ahead();
+    wait_for_the_kernel_ahead();      // and no word to the kernel behind
     const int64_t u0 = (int64_t)blockIdx.x * kThreads * kUnroll;
     int64_t e[kUnroll];
     Pack<T> pg[kUnroll];
