@@ -214,7 +214,7 @@ int granq_range(const void* x, int dtype, const int64_t dims[4], int channel_axi
     Workspace ws = carve_workspace(workspace, G);
     cudaError_t e = clear_workspace(ws, g, kHostBoundRange, st);
     if (e == cudaSuccess)
-        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, 0, nullptr, nullptr, st);
+        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, 0, nullptr, nullptr, ws.cleared, st);
     return cuda_status(e);
 }
 
@@ -305,7 +305,7 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
     // two passes over x by ordinary launches: any geometry, any GPU
     auto two_pass = [&]() -> cudaError_t {
-        cudaError_t r = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, st);
+        cudaError_t r = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, ws.cleared, st);
         return r == cudaSuccess ? launch_quant_flat(io, mode, dtype, g, bits, min_out, max_out, st) : r;
     };
     if (plan == PLAN_CLUSTER) {
@@ -438,7 +438,7 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {
-        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, st);
+        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, ws.cleared, st);
         if (e == cudaSuccess) e = launch_quant_flat(io, MODE_FWD, dtype, g, bits, min_out, max_out, st);
         if (e == cudaSuccess && zeroed)
             e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);
@@ -653,7 +653,7 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {
-        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, st);
+        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, ws.cleared, st);
         if (e == cudaSuccess) e = launch_quant_flat(io, MODE_FWD, dtype, g, bits, min_out, max_out, st);
         if (e == cudaSuccess && zeroed)
             e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);
@@ -734,7 +734,7 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, g_tune, st);
     } else {
-        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_out, zp_out, st);
+        e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_out, zp_out, ws.cleared, st);
         if (e == cudaSuccess) e = launch_quant_flat(io, MODE_FWD, dtype, g, bits, min_out, max_out, st);
         if (e == cudaSuccess && zeroed)
             e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);

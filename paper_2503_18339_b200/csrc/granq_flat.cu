@@ -925,7 +925,7 @@ int range_rows_ctas() {
 }
 
 template <typename T>
-cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t* kmax, const RangeEnd& end, cudaStream_t st) {
+cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t* kmax, const RangeEnd& end, int layout, cudaStream_t st) {
     FlatGeom f = make_flat(g);
     constexpr int VF = Pack<T>::V;
     bool vec = aligned16(x) && (g.inner % VF == 0);
@@ -941,7 +941,7 @@ cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t*
         const uint32_t chunks = std::max<uint32_t>(1, std::min<uint32_t>((2 * cap + ncol - 1) / ncol, outer / 4));
         constexpr int U = VF == 4 ? 8 : 4;
         auto cols = [&](auto kern, uint32_t plane) {
-            return launch_after(kAnyLayout, kern, ncol * chunks, kThreads, 0, st, (const uint4*)x, slab_units, outer, chunks,
+            return launch_after(layout, kern, ncol * chunks, kThreads, 0, st, (const uint4*)x, slab_units, outer, chunks,
                                 make_fastdiv(ncol), make_fastdiv(plane), kmin, kmax, end);
         };
         return vec ? cols(range_cols_kernel<T, true, U>, (uint32_t)(g.inner / VF)) : cols(range_cols_kernel<T, false, U>, (uint32_t)g.inner);
@@ -952,13 +952,13 @@ cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t*
         const int64_t cap = (int64_t)range_rows_ctas();                 // 4 resident CTAs per SM at 64 registers
         int rgrid = (int)(ctas < cap ? ctas : cap);
         auto by_rows = [&](auto kern, uint32_t plane) {
-            return launch_after(kAnyLayout, kern, rgrid, kThreads, 0, st, (const uint4*)x, n_units, (uint32_t)g.inner, make_fastdiv(plane),
+            return launch_after(layout, kern, rgrid, kThreads, 0, st, (const uint4*)x, n_units, (uint32_t)g.inner, make_fastdiv(plane),
                                 make_fastdiv((uint32_t)g.C), (uint32_t)g.C, kmin, kmax, end);
         };
         return vec ? by_rows(range_rows_kernel<T, true>, (uint32_t)(g.inner / VF)) : by_rows(range_rows_kernel<T, false>, (uint32_t)g.inner);
     }
-    return vec ? launch_after(kAnyLayout, range_flat_kernel<T, VF>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end)
-               : launch_after(kAnyLayout, range_flat_kernel<T, 1>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end);
+    return vec ? launch_after(layout, range_flat_kernel<T, VF>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end)
+               : launch_after(layout, range_flat_kernel<T, 1>, grid, kThreads, 0, st, (const T*)x, f, kmin, kmax, end);
 }
 
 template <typename T, int MODE>
@@ -988,8 +988,13 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
     const bool ragged = !vec && g.inner >= VF && g.inner % VF != 0 && g.E % VF == 0 && !f.inner_big && aligned16(io.x) &&
                         aligned16(io.gy) && aligned16(io.y) && aligned16(io.gx) && ((uintptr_t)io.codes % 4 == 0) &&
                         ((uintptr_t)io.mask % 4 == 0);
-    // five blocks of a table each fill an SM
-    const int layout = sm_layout(100, (uint64_t)g.E * sizeof(T));
+    // Five blocks of a table each fill an SM.  The scalar form is bound by its instructions: where one grid fits the GPU but two do
+    // not, blocks that start before the kernel ahead has ended crowd on the SMs that have room first, four to an SM or, backward,
+    // seven.  Alone / set up early, us: backward bf16 [100,75,27,27], 668 blocks, 31.1 / 34.4, of [33,41,51,51], 430, 25.0 / 23.7; forward of the
+    // latter 22.9 / 24.2, of [101,75,27,27] 39.3 / 38.2; codes and back of the latter but one 82.7 / 91.6.
+    const int64_t slots = (int64_t)sm_count() * (MODE == MODE_BWD ? 7 : 4);
+    const bool crowded = !vec && !ragged && f.ntiles <= slots && 2 * f.ntiles > slots;
+    const int layout = crowded ? kAlone : sm_layout(100, (uint64_t)g.E * sizeof(T));
     auto go = [&](auto kern) {
         return launch_after(layout, kern, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask,
                             io.pmask, io.dist, io.pcodes, io.code_bits, f, qmax, lo, hi);
@@ -1061,11 +1066,12 @@ cudaError_t dequant_strings(const uint32_t* pcodes, T* y, const Geom& g, int bit
 }  // namespace
 
 cudaError_t launch_range(const void* x, int dtype, const Geom& g, uint32_t* kmin, uint32_t* kmax, uint32_t* counter,
-                         float* lo, float* hi, int bits, float* s_opt, float* z_opt, cudaStream_t st) {
+                         float* lo, float* hi, int bits, float* s_opt, float* z_opt, bool behind_clear, cudaStream_t st) {
     const bool fused = counter != nullptr && g.C <= 4096;       // the last block's share: 16 groups per thread
     const RangeEnd end{fused ? counter : nullptr, kmin, kmax, lo, hi, s_opt, z_opt, (uint32_t)g.C, bits};
-    const cudaError_t e = dtype == 0 ? range_flat_t<float>(x, g, kmin, kmax, end, st)
-                                     : range_flat_t<__nv_bfloat16>(x, g, kmin, kmax, end, st);
+    const int layout = behind_clear ? kAnyLayout : kAlone;
+    const cudaError_t e = dtype == 0 ? range_flat_t<float>(x, g, kmin, kmax, end, layout, st)
+                                     : range_flat_t<__nv_bfloat16>(x, g, kmin, kmax, end, layout, st);
     if (e != cudaSuccess || fused) return e;
     const int grid = (int)((g.C + 255) / 256);
     return launch_after(kAnyLayout, finalize_range_kernel, grid, 256, 0, st, kmin, kmax, g.C, lo, hi, bits, s_opt, z_opt);

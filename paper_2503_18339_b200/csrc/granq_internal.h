@@ -106,7 +106,8 @@ inline cudaError_t allow_smem(K kern, size_t most) {
 // packed mask and backward of fp32 [128,144,56,56] 173.1 / 184.9 and [41,1896,15,16] 60.7 / 64.8, fused call and backward from x of
 // [116,1240,16,15] 110.7 / 125.3, fused call and weights of a network 113.0 / 114.9; bf16 [212,568,7,8], 13 MB, fused call and backward 25.2 /
 // 23.9.
-constexpr int kAnyLayout = -1;
+// kAlone: not before the kernel ahead has ended.
+constexpr int kAnyLayout = -1, kAlone = -2;
 inline int sm_layout(int smem_kb, uint64_t bytes) { return bytes >= (16ull << 20) ? smem_kb : kAnyLayout; }
 template <typename... P, typename... A>
 inline cudaError_t launch_after(int smem_kb, void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
@@ -123,7 +124,7 @@ inline cudaError_t launch_after(int smem_kb, void (*kern)(P...), unsigned grid, 
     attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
     attr[1].val.sharedMemCarveout = smem_kb < 0 ? 0u : (unsigned)(smem_kb * 100 / kSmemKB);
     cfg.attrs = attr;
-    cfg.numAttrs = smem_kb == kAnyLayout ? 1 : 2;
+    cfg.numAttrs = smem_kb == kAlone ? 0 : smem_kb == kAnyLayout ? 1 : 2;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
@@ -134,8 +135,10 @@ cudaError_t launch_clear(void* workspace, size_t bytes, double* sums_opt, cudaSt
 // ---- generic ("flat") kernels: any geometry, any alignment --------------------------------
 // Range of every group (Eq. 4) into lo / hi, and s / z when bits > 0 and the pointers are given (Eq. 5).  The keys and,
 // where one is given, the counter must be zero on entry; with a counter the range launch finishes by itself.
+// behind_clear: the kernel ahead is launch_clear()'s.  The range launch is set up beside that one only: beside another its blocks, about
+// a wave of them, crowd on the SMs that have room first (fused call on a zeroed workspace and forward, [33,41,51,51] 64 us / 68).
 cudaError_t launch_range(const void* x, int dtype, const Geom& g, uint32_t* kmin, uint32_t* kmax, uint32_t* counter,
-                         float* lo, float* hi, int bits, float* s_opt, float* z_opt, cudaStream_t st);
+                         float* lo, float* hi, int bits, float* s_opt, float* z_opt, bool behind_clear, cudaStream_t st);
 // lo / hi -> s / z
 cudaError_t launch_params(const float* lo, const float* hi, int64_t G, int bits, float* s_opt, float* z_opt,
                           cudaStream_t st);

@@ -64,6 +64,6 @@ extern "C" int granq_range_noalloc(const void* x, int dtype, const int64_t dims[
     // the array keeps the previous call's keys: both halves must start at the identity (0)
     e = cudaMemsetAsync(kmin, 0, (size_t)G * sizeof(uint32_t), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(kmax, 0, (size_t)G * sizeof(uint32_t), st);
-    if (e == cudaSuccess) e = launch_range(x, dtype, g, kmin, kmax, nullptr, min_out, max_out, 0, nullptr, nullptr, st);
+    if (e == cudaSuccess) e = launch_range(x, dtype, g, kmin, kmax, nullptr, min_out, max_out, 0, nullptr, nullptr, false, st);
     return e == cudaSuccess ? GRANQ_OK : GRANQ_ERR_CUDA;
 }
