@@ -493,11 +493,13 @@ static bool batch_conflict(const granq_fused_desc& a, const granq_fused_desc& b,
 // 1.5 times as slow; some long lists would gain a fifth.
 static int list_takes(int dtype, const Geom& g, int count, int sms, TeamPlan& plan) {
     count = count < (int)kTeamListMax ? count : (int)kTeamListMax;
-    if (dtype != GRANQ_F32 || count < 2 || g.C >= (1ll << 28)) return 0;
+    const bool large = g.E / g.C >= (220 << 10) / 4;
+    // most lists go no further: of small channels, and more slabs than a cluster of eight has too few of
+    if (dtype != GRANQ_F32 || count < 2 || (!large && g.outer > 24) || g.C >= (1ll << 28)) return 0;
     const ClusterPlan kp = plan_cluster(dtype, g, QuantIO{}, true, g_tune);      // null pointers: alignment is assumed
     if (kp.ok) {
         const int64_t ctas = count * ((g.C + kp.k - 1) / kp.k * kp.R);
-        const bool large = g.E / g.C >= (220 << 10) / 4, few_slabs = g.outer <= 3 * (int64_t)kp.R;
+        const bool few_slabs = g.outer <= 3 * (int64_t)kp.R;
         if (!(large && ctas >= 9ll * sms) && !(few_slabs && ctas >= 5ll * sms)) return 0;
     }
     plan = plan_colteam(dtype, g, QuantIO{}, true, sms, g_tune, (uint32_t)count);
@@ -514,10 +516,7 @@ static int batch_together(const granq_fused_desc* descs, int first, int n_tensor
         return 0;
     Geom g;
     int64_t G;
-    int dev = 0, sms = 0;
-    if (!make_geom(descs[first].dims, channel_axis, group, g, G) || cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 0;
+    if (!make_geom(descs[first].dims, channel_axis, group, g, G)) return 0;
     auto like_first = [&](int k) {
         for (int i = 0; i < 4; ++i)
             if (descs[first + k].dims[i] != descs[first].dims[i]) return false;
@@ -525,8 +524,11 @@ static int batch_together(const granq_fused_desc* descs, int first, int n_tensor
     };
     int alike = 1;
     while (first + alike < n_tensors && alike < (int)kTeamListMax && like_first(alike)) ++alike;
+    int dev = 0, sms = 0;
     TeamPlan plan{};
-    if (list_takes(dtype, g, alike, sms, plan) == 0) return 0;
+    if (alike < 2 || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || list_takes(dtype, g, alike, sms, plan) == 0)
+        return 0;
     const size_t nb = (size_t)g.E * elt_size(dtype);
     TeamTensor tensors[kTeamListMax];
     int n = 0;

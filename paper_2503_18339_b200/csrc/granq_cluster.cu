@@ -128,11 +128,6 @@ __device__ __forceinline__ uint4 k_ld_l2_16(const void* p, uint64_t policy) {
                  : "memory");
     return v;
 }
-// per-thread asynchronous 16-byte copy global -> shared (both 16-byte aligned); without an L2 policy, which is worth
-// nothing here and is under suspicion on this instruction (granq_colteam.cu)
-__device__ __forceinline__ void k_cp_async_16(void* dst_smem, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(k_smem_u32(dst_smem)), "l"(src) : "memory");
-}
 __device__ __forceinline__ void k_cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void k_cp_async_wait() {
@@ -273,7 +268,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
             for (uint32_t col = cin; col < ncol; col += P) {
                 const uint4* p = xg + (size_t)r0 * slab + col;
                 uint4* q = tile + (size_t)r0 * ncol + col;
-                for (uint32_t s = r0; s < nl; s += nrows, p += gstep, q += sstep) k_cp_async_16(q, p);
+                for (uint32_t s = r0; s < nl; s += nrows, p += gstep, q += sstep) cp_async_16(q, p);
             }
         }
         k_cp_async_commit();
@@ -282,7 +277,7 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
                 for (uint32_t col = cin; col < ncol; col += P) {
                     const uint4* p = gyg + (size_t)r0 * slab + col;
                     uint4* q = tileg + (size_t)r0 * ncol + col;
-                    for (uint32_t s = r0; s < nl; s += nrows, p += gstep, q += sstep) k_cp_async_16(q, p);
+                    for (uint32_t s = r0; s < nl; s += nrows, p += gstep, q += sstep) cp_async_16(q, p);
                 }
             }
             k_cp_async_commit();

@@ -76,11 +76,6 @@ struct TArgs {
     FastDiv div_plane;     // units per plane
 };
 
-__device__ __forceinline__ uint32_t t_ld_acquire(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ void t_arrive_release(uint32_t* p) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
@@ -88,10 +83,6 @@ __device__ __forceinline__ void t_arrive_release(uint32_t* p) {
 // ended in an illegal instruction on [128,64,56,56], forward.  The cause was not found: operand widths, the policy's
 // lifetime, addresses, sizes and trip counts were in order, and the same instruction in loops of unequal trip counts ran
 // elsewhere without fault.  Without the operand, with streaming loads and stores: the same times.
-__device__ __forceinline__ void t_cp_async_16(void* dst_smem, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)), "l"(src)
-                 : "memory");
-}
 __device__ __forceinline__ void t_cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // U = units a thread handles together in the quantize walk
@@ -144,8 +135,8 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
         uint64_t at = first + (uint64_t)team * a.plane_units;
         uint32_t off = off0;
         for (uint32_t i = 0; i < cnt; ++i) {
-            t_cp_async_16(tile + i * kTThreads, xg + at);
-            if (kBwd && i < gcnt) t_cp_async_16(tileg + i * kTThreads, gyg + at);
+            cp_async_16(tile + i * kTThreads, xg + at);
+            if (kBwd && i < gcnt) cp_async_16(tileg + i * kTThreads, gyg + at);
             advance(at, off);
         }
     }
@@ -179,7 +170,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
                 // ---- wait (bounded) until the whole team has published the channel; Eq. 5 ----
                 uint32_t ready = 0;
                 for (uint32_t i = 0; i < a.spin_limit; ++i) {
-                    if (t_ld_acquire(a.counters + c) >= a.expected) {
+                    if (ld_acquire(a.counters + c) >= a.expected) {
                         ready = 1;
                         break;
                     }
@@ -248,8 +239,8 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
             if (more) {
 #pragma unroll
                 for (int j = 0; j < U; ++j) {
-                    t_cp_async_16(tile + (i + j) * kTThreads, xg + w[j] + ahead);
-                    if (kBwd && i + j < gcnt) t_cp_async_16(tileg + (i + j) * kTThreads, gyg + w[j] + ahead);
+                    cp_async_16(tile + (i + j) * kTThreads, xg + w[j] + ahead);
+                    if (kBwd && i + j < gcnt) cp_async_16(tileg + (i + j) * kTThreads, gyg + w[j] + ahead);
                 }
             }
 #pragma unroll
@@ -263,8 +254,8 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
             }
             px.raw = tile[i * kTThreads];
             if (more) {
-                t_cp_async_16(tile + i * kTThreads, xg + at + ahead);
-                if (kBwd && i < gcnt) t_cp_async_16(tileg + i * kTThreads, gyg + at + ahead);
+                cp_async_16(tile + i * kTThreads, xg + at + ahead);
+                if (kBwd && i < gcnt) cp_async_16(tileg + i * kTThreads, gyg + at + ahead);
             }
             emit(px, pg, at);
             advance(at, off);
@@ -387,7 +378,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
         t_arrive_release(t.counters + c);
         uint32_t ready = 0;
         for (uint32_t i = 0; i < a.spin_limit; ++i) {
-            if (t_ld_acquire(t.counters + c) >= a.expected) {
+            if (ld_acquire(t.counters + c) >= a.expected) {
                 ready = 1;
                 break;
             }
@@ -441,7 +432,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
             }
             if (more) {
 #pragma unroll
-                for (int k = 0; k < U; ++k) t_cp_async_16(tile + (i + k) * kTWork, xn + w[k]);
+                for (int k = 0; k < U; ++k) cp_async_16(tile + (i + k) * kTWork, xn + w[k]);
             }
 #pragma unroll
             for (int k = 0; k < U; ++k) emit(px[k], pg[k], w[k]);
@@ -450,7 +441,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
             Pack<T> px, pg;
             pg.raw = ld_stream_16(gyg + at);
             px.raw = tile[i * kTWork];
-            if (more) t_cp_async_16(tile + i * kTWork, xn + at);
+            if (more) cp_async_16(tile + i * kTWork, xn + at);
             emit(px, pg, at);
             advance(at, off);
         }
@@ -466,7 +457,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
         uint4* tile = t_smem + j * a.tile_units + tid;
         uint32_t at = first, off = off0;
         for (uint32_t i = 0; i < cnt; ++i) {
-            t_cp_async_16(tile + i * kTWork, xg + at);
+            cp_async_16(tile + i * kTWork, xg + at);
             advance(at, off);
         }
     }

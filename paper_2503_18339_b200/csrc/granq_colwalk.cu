@@ -77,12 +77,6 @@ struct CArgs {
     FastDiv div_plane;     // units per plane (aligned planes) or elements per plane
 };
 
-__device__ __forceinline__ uint32_t c_ld_acquire(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // per-element running min / max of one unit column
 template <typename T>
 struct ColRange {
@@ -265,7 +259,7 @@ __global__ void __launch_bounds__(kCThreads, 4) colwalk_kernel(const CArgs a) {
         if (tid == 0) {
             uint32_t ready = 0;
             for (uint32_t i = 0; i < a.spin_limit; ++i) {
-                if (c_ld_acquire(a.counters + w) >= a.expected) {
+                if (ld_acquire(a.counters + w) >= a.expected) {
                     ready = 1;
                     break;
                 }

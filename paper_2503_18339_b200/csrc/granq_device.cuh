@@ -250,6 +250,19 @@ __device__ __forceinline__ void run_add(WarpRun& r, bool valid, uint32_t g, uint
     }
 }
 
+// A 16-byte unit from global to shared memory (both aligned), past the L1, without waiting; without an L2 policy, which is worth nothing
+// here and is under suspicion on this instruction (granq_colteam.cu).
+__device__ __forceinline__ void cp_async_16(void* dst_smem, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)), "l"(src)
+                 : "memory");
+}
+// a word that another CTA released
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // The kernel behind this one in the stream may be set up; it waits for this one's end, memory included, by itself.
 __device__ __forceinline__ void let_the_kernel_behind_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -8,9 +8,12 @@
 // read again, the last of it first, most of it from the L2.
 // Bound by the chain copy, fold, hand-over, quantize.  Against range pass and quantize pass (us, with gradient / forward / with
 // sums): [100,75,27,27] fp32, 21.9 MB, 37.9 / 31.6 / 36.7 -> 25.0 / 18.7 / 21.4; [200,301,7,7] bf16 38.5 / 34.0 / 37.9 -> 17.6 /
-// 16.6 / 19.8; one group: [128,128,28,28] fp32, 51 MB, sums 39.9 -> 29.2; [128,64,28,28] bf16, 13 MB, sums 24.5 -> 17.5.  Against
-// the L2-resident waves, one group: bf16 [128,192,28,28], 38.5 MB, 38.9 / 30.8 -> 35.4 / 24.7; fp32 [128,64,28,28] 26.6 / 18.8 ->
-// 26.2 / 18.0.
+// 16.6 / 19.8; one group: [128,128,28,28] fp32, 51 MB, sums 39.9 -> 29.2; [128,64,28,28] bf16, 13 MB, sums 24.5 -> 17.5.  Packed mask,
+// 4-bit and 5-bit codes of one group: [128,128,28,28] fp32, a third of it read again, 33.9 / 37.0 / 38.7 -> 32.3 / 32.9 / 33.6; [96,128,28,28]
+// fp32 27.0 / 28.8 / 29.9 -> 26.6 / 26.5 / 27.2; bf16 20.8 / 22.3 / 22.6 -> 16.6 / 20.7 / 20.8.  Against the L2-resident waves, one group:
+// bf16 [128,192,28,28], 38.5 MB, 38.9 / 30.8 -> 35.4 / 24.7; fp32 [128,64,28,28] 26.6 / 18.8 -> 26.2 / 18.0.  There is no smallest size: a tensor
+// of 80 KB, [8,75,5,7], takes 5.8 us from a graph and 11.9 eagerly where two passes took 23.1 and 25.4, one group of 0.5 MB 6.0 and 9.9 where the
+// waves took 12.4 and 9.8.
 #include "granq_internal.h"
 
 #include <algorithm>
@@ -57,16 +60,6 @@ struct HArgs {
     FastDiv div_inner, div_groups;
 };
 
-__device__ __forceinline__ void h_cp_async_16(void* dst_smem, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ uint32_t h_ld_acquire(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // U = units a thread handles together in the quantize walk
 template <typename T, int MODE, int EXTRAS, int KIND, int U>
 __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
@@ -94,7 +87,7 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
     }
 
     if (!a.early) after_the_kernel_ahead();
-    for (uint32_t i = tid; i < held; i += kHThreads) h_cp_async_16(tile + i, xg + i);
+    for (uint32_t i = tid; i < held; i += kHThreads) cp_async_16(tile + i, xg + i);
     if constexpr (KIND != H_ONE) {
         for (uint32_t p = tid; p < np; p += kHThreads) s_kmn[p] = s_kmx[p] = 0;
     }
@@ -192,7 +185,7 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
         atomicAdd(a.counters, 1u);
         uint32_t ready = 0;
         for (uint32_t i = 0; i < a.spin_limit; ++i) {
-            if (h_ld_acquire(a.counters) >= a.expected) {
+            if (ld_acquire(a.counters) >= a.expected) {
                 ready = 1;
                 break;
             }

@@ -63,12 +63,6 @@ struct LArgs {
     FastDiv div_plane;     // units per plane (aligned planes) or elements per plane
 };
 
-__device__ __forceinline__ uint32_t l_ld_acquire(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // UPL = 16-byte units per lane and step; a warp handles rows of 32 * UPL consecutive units
 template <typename T, int MODE, bool ALIGNED, bool EXTRAS, int UPL>
 __global__ void __launch_bounds__(kLThreads, UPL == 2 ? 4 : 3) l2wave_kernel(const LArgs a) {
@@ -176,7 +170,7 @@ __global__ void __launch_bounds__(kLThreads, UPL == 2 ? 4 : 3) l2wave_kernel(con
         if (tid == 0) {
             uint32_t ready = 0;
             for (uint32_t i = 0; i < a.spin_limit; ++i) {
-                if (l_ld_acquire(a.counters + w) >= a.expected) {
+                if (ld_acquire(a.counters + w) >= a.expected) {
                     ready = 1;
                     break;
                 }
@@ -282,8 +276,6 @@ __global__ void __launch_bounds__(kLThreads, UPL == 2 ? 4 : 3) l2wave_kernel(con
         phase2(w);
     }
 }
-
-
 
 inline uint32_t l_gcd(uint32_t a, uint32_t b) {
     while (b) {
@@ -426,6 +418,5 @@ cudaError_t launch_l2wave(const L2Plan& plan, const QuantIO& io, int mode, int d
     if (mode == MODE_FWD) return l_launch_mode<__nv_bfloat16, MODE_FWD>(plan, a, aligned, extras, sms, cap, st);
     return l_launch_mode<__nv_bfloat16, MODE_BOTH>(plan, a, aligned, extras, sms, cap, st);
 }
-
 
 }  // namespace granq

@@ -64,16 +64,6 @@ struct RArgs {
     uint64_t rows;
 };
 
-__device__ __forceinline__ uint32_t r_ld_acquire(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void r_cp_async_16(void* dst_smem, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)), "l"(src)
-                 : "memory");
-}
-
 // U1 / U2 = rows a thread has in flight in the range / quantize walk
 template <typename T, int MODE, bool EXTRAS, int U1, int U2>
 __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a) {
@@ -105,7 +95,7 @@ __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a)
     const uint64_t drop = l2_policy_evict_first();
 
     if (!a.early) after_the_kernel_ahead();
-    for (uint32_t k = 0; k < held; ++k) r_cp_async_16(tile + k * tstep, xg + k * step);
+    for (uint32_t k = 0; k < held; ++k) cp_async_16(tile + k * tstep, xg + k * step);
     for (uint32_t t = tid; t < 2 * P * V; t += NT) s_kmn[t] = 0;
     __syncthreads();
 
@@ -155,7 +145,7 @@ __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a)
         atomicAdd(a.counters + slice, 1u);
         uint32_t ready = 0;
         for (uint32_t i = 0; i < a.spin_limit; ++i) {
-            if (r_ld_acquire(a.counters + slice) >= a.expected) {
+            if (ld_acquire(a.counters + slice) >= a.expected) {
                 ready = 1;
                 break;
             }

@@ -64,6 +64,28 @@ def test_resident_walk(b, knobs, shape, dtype):
     assert np.allclose(to_np(got.sums), sums, rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("dtype,shape", [
+    ("f32", (143, 15, 64, 64)),      # three rounds, shares that do not come out even
+    ("f32", (232, 3, 112, 112)),     # a channel over all SMs, one team
+    ("f32", (90, 40, 60, 44)),       # ten teams, four rounds
+    ("bf16", (65, 28, 96, 96)),      # shares next to the smallest that are planned
+    ("bf16", (69, 33, 96, 96)),
+], ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else v)
+def test_two_channels_side_by_side_by_default(b, dtype, shape):
+    x, gy = make_case(shape, seed=sum(shape), dtype=dtype, relu=shape[0] % 2 == 0)
+    form = b.team_geometry(b.BF16 if dtype == "bf16" else b.F32, shape)
+    units = shape[0] * shape[2] * shape[3] // (8 if dtype == "bf16" else 4)
+    assert form["taken"] == 1 and form["rounds"] > 1 and form["ctas"] * form["units"] >= 2 * units      # of both channels
+    ref = orc.fused(x, 5, gy=gy)
+    xd, gyd = to_dev(x), to_dev(gy)
+    dirty, zeroed = b.make_workspace(xd).fill_(255), b.make_workspace(xd, zeroed=True)
+    for ws, flags in ((dirty, 0), (zeroed, b.FLAG_WORKSPACE_ZEROED), (zeroed, b.FLAG_WORKSPACE_ZEROED)):
+        got = b.granq_fakequant_fused(xd, 5, gy=gyd, out=b.FakeQuantOut(workspace=ws), want_params=True, flags=flags)
+        assert b.workspace_status(ws) == b.OK
+        assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=True)
+    assert int(zeroed.view(torch.int32).abs().sum().item()) == 0
+
+
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_waves_on_aligned_planes(b, knobs, shape, dtype):
