@@ -988,12 +988,13 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
     const bool ragged = !vec && g.inner >= VF && g.inner % VF != 0 && g.E % VF == 0 && !f.inner_big && aligned16(io.x) &&
                         aligned16(io.gy) && aligned16(io.y) && aligned16(io.gx) && ((uintptr_t)io.codes % 4 == 0) &&
                         ((uintptr_t)io.mask % 4 == 0);
-    // Five blocks of a table each fill an SM.  The scalar form is bound by its instructions: where one grid fits the GPU but two do
-    // not, blocks that start before the kernel ahead has ended crowd on the SMs that have room first, four to an SM or, backward,
-    // seven.  Alone / set up early, us: backward bf16 [100,75,27,27], 668 blocks, 31.1 / 34.4, of [33,41,51,51], 430, 25.0 / 23.7; forward of the
-    // latter 22.9 / 24.2, of [101,75,27,27] 39.3 / 38.2; codes and back of the latter but one 82.7 / 91.6.
-    const int64_t slots = (int64_t)sm_count() * (MODE == MODE_BWD ? 7 : 4);
-    const bool crowded = !vec && !ragged && f.ntiles <= slots && 2 * f.ntiles > slots;
+    // Five blocks of a table each fill an SM.  The scalar form is bound by its instructions, and its grids of up to a wave - four blocks
+    // to an SM or, backward, seven - are spread evenly only over an empty GPU: blocks that start before the kernel ahead has
+    // ended crowd on the SMs that have room first, unless two grids leave SMs free.  Alone / set up early, us: backward f32 [75,31,41,41], 477
+    // blocks, 24.8 / 31.5, of [33,41,51,51], 430, 22.8 / 20.5; fused call of bf16 [37,532,7,7], 118, 41.4 / 49.5, of [37,133,7,7], 30, 39.3 / 37.3;
+    // forward [33,41,51,51] 22.8 / 24.1, [101,75,27,27], 674, 39.3 / 38.2.
+    const int64_t sms = sm_count(), slots = sms * (MODE == MODE_BWD ? 7 : 4);
+    const bool crowded = !vec && !ragged && 2 * f.ntiles > sms && f.ntiles <= slots;
     const int layout = crowded ? kAlone : sm_layout(100, (uint64_t)g.E * sizeof(T));
     auto go = [&](auto kern) {
         return launch_after(layout, kern, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask,
