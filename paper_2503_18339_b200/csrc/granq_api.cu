@@ -212,7 +212,8 @@ int granq_range(const void* x, int dtype, const int64_t dims[4], int channel_axi
     if (int rc = check_workspace(workspace, workspace_bytes, G)) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     Workspace ws = carve_workspace(workspace, G);
-    cudaError_t e = clear_workspace(ws, g, kHostBoundRange, st);
+    // (tensors that are no whole 16-byte units keep the GPU longer than the host: [37,133,7,7] 21.9 by a memset, 19.2)
+    cudaError_t e = clear_workspace(ws, g, g.E * (int64_t)elt_size(dtype) % 16 == 0 ? kHostBoundRange : 0, st);
     if (e == cudaSuccess)
         e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, 0, nullptr, nullptr, ws.cleared, st);
     return cuda_status(e);
