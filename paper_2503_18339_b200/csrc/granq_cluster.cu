@@ -408,9 +408,16 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
     const float qmax = a.qmax;
     DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS = 4)
     dacc.reset();
+    constexpr bool kPairs = V == 4 && (EXTRAS == 2 || EXTRAS == 3);      // written by neighbouring lanes together
+    const uint32_t lane = tid & 31;
+    // slabs of this thread; of every thread of its warp that walks
+    const uint32_t mine = kPairs && r0 < nl ? (nl - r0 + nrows - 1) / nrows : 0u;
+    const uint32_t whole = kPairs ? __reduce_min_sync(kFullMask, rowed ? mine : 0xFFFFFFFFu) : 0u;
     if constexpr (ASYNC && GY) k_cp_async_wait<0>();
     for (uint32_t tile0 = 0; tile0 < ncol; tile0 += P) {
         const uint32_t col = tile0 + cin;
+        // the lanes of this warp that walk a column
+        const uint32_t walkers = kPairs ? __ballot_sync(kFullMask, rowed && col < ncol) : 0u;
         if (!(rowed && col < ncol) || !ok) continue;
         uint32_t ch;
         int ne;
@@ -420,44 +427,80 @@ __global__ void __launch_bounds__(kKMaxThreads, 2) cluster_kernel(const KArgs a)
         if constexpr (!ALIGNED) {
             if (ne < V) g2 = s_par[ch + 1];
         }
-        auto emit = [&](const Pack<T>& px, const Pack<T>& pg, size_t at) {
+        auto quantize = [&](const Pack<T>& px, const Pack<T>& pg, size_t at, uint32_t (&cb)[V / 4], uint32_t (&mb)[V / 4]) {
             Pack<T> py, pgx;
-            uint32_t cb[V / 4], mb[V / 4];
             const int code_bits = EXTRAS == 3 ? a.code_bits : 8;
             if constexpr (ALIGNED) quantize_own<T, kBwd, EXTRAS>(px, pg, g1, qmax, py, pgx, cb, mb, code_bits);
             else quantize_pack<T, kBwd, true, EXTRAS, true>(px, pg, g1, g2, ne, qmax, py, pgx, cb, mb, code_bits);
-            if constexpr (EXTRAS == 3) {
-                // the packed codes are the only output: 8 codes = b bytes per pair of fp32 lanes (per bf16 lane); the
-                // planner has made every run and slab whole groups of 8 elements, so both lanes of a pair are here
-                store_code_bytes<V>(a.pcodes, (gbase + at) * V, code_string_of<V>(cb, a.code_bits), a.code_bits, tid & 31);
-                return;
-            }
-            st_hint_16(yg + at, py.raw, drop);
+            if constexpr (EXTRAS != 3) st_hint_16(yg + at, py.raw, drop);      // packed codes are the only output
             if constexpr (kBwd) st_hint_16(gxg + at, pgx.raw, drop);
-            if constexpr (EXTRAS != 0) {
-                if constexpr (EXTRAS == 1) {
-                    const size_t w = (gbase + at) * (V / 4);
-                    if (a.codes) {
+            if constexpr (EXTRAS == 4) dacc.add(px, py);
+        };
+        auto store_extra = [&](const uint32_t (&cb)[V / 4], const uint32_t (&mb)[V / 4], size_t at, uint32_t lanes) {
+            if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, (gbase + at) * V, mb[0], lane, lanes);
+            if constexpr (EXTRAS == 3)
+                store_code_bytes<V>(a.pcodes, (gbase + at) * V, code_string_of<V>(cb, a.code_bits), a.code_bits, lane, lanes);
+        };
+        auto emit = [&](const Pack<T>& px, const Pack<T>& pg, size_t at) {
+            uint32_t cb[V / 4], mb[V / 4];
+            quantize(px, pg, at, cb, mb);
+            if constexpr (EXTRAS == 1) {
+                const size_t w = (gbase + at) * (V / 4);
+                if (a.codes) {
 #pragma unroll
-                        for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.codes)[w + i] = cb[i];
-                    }
-                    if (kBwd && a.mask) {
+                    for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.codes)[w + i] = cb[i];
+                }
+                if (kBwd && a.mask) {
 #pragma unroll
-                        for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.mask)[w + i] = mb[i];
-                    }
+                    for (int i = 0; i < V / 4; ++i) reinterpret_cast<uint32_t*>(a.mask)[w + i] = mb[i];
                 }
-                if constexpr (EXTRAS == 4) dacc.add(px, py);
-                if (EXTRAS != 4 && a.pmask) {
-                    // the mask is written byte by byte (8 elements: two fp32 packs of neighbouring lanes, one bf16
-                    // pack): the planner has made every run and slab whole bytes of mask and the rows of columns
-                    // whole pairs of lanes, so both lanes of a byte are here together, in the same slab
-                    store_mask_byte<V>(a.pmask, (gbase + at) * V, mask_bits_of<V, EXTRAS>(mb), tid & 31);
-                }
+                if (a.pmask) store_mask_byte<V>(a.pmask, (gbase + at) * V, mask_bits_of<V, EXTRAS>(mb), lane, 3u << (lane & ~1u));
+            } else {
+                store_extra(cb, mb, at, kFullMask);
             }
         };
         size_t gu = (size_t)r0 * slab + col;
         const uint4* q = tile + (size_t)r0 * ncol + col;
         const uint4* qg = tileg + (size_t)r0 * ncol + col;
+        if constexpr (kPairs) {
+            // The planner has made every run and slab whole groups of 8 elements and the rows of columns whole pairs of lanes, so
+            // both lanes of a group are here together, in the same slab.
+            uint32_t i = 0;
+            for (; i + 2 <= whole; i += 2) {
+                Pack<T> px[2];
+                uint32_t cb[2][V / 4], mb[2][V / 4];
+                px[0].raw = q[0];
+                px[1].raw = q[sstep];
+                quantize(px[0], px[0], gu, cb[0], mb[0]);
+                quantize(px[1], px[1], gu + gstep, cb[1], mb[1]);
+                if (walkers == kFullMask) {
+                    const size_t at = gbase + gu + (lane & 1 ? gstep : 0);
+                    if constexpr (EXTRAS == 2) {
+                        const uint32_t bits[2] = {mb[0][0], mb[1][0]};
+                        reinterpret_cast<uint8_t*>(a.pmask)[at >> 1] = (uint8_t)pair_up_mask<2>(bits, lane);
+                    } else {
+                        store_eight_codes(a.pcodes, at >> 1, pair_up_codes(cb[0][0], cb[1][0], a.code_bits, lane), a.code_bits);
+                    }
+                } else {
+                    store_extra(cb[0], mb[0], gu, walkers);
+                    store_extra(cb[1], mb[1], gu + gstep, walkers);
+                }
+                gu += 2 * gstep;
+                q += 2 * sstep;
+            }
+            for (uint32_t lanes; (lanes = __ballot_sync(walkers, i < mine)) != 0; ++i) {
+                if (i < mine) {
+                    Pack<T> px;
+                    uint32_t cb[V / 4], mb[V / 4];
+                    px.raw = *q;
+                    quantize(px, px, gu, cb, mb);
+                    store_extra(cb, mb, gu, lanes);
+                    gu += gstep;
+                    q += sstep;
+                }
+            }
+            continue;
+        }
         uint32_t s = r0;
         // the staged gy of slabs up to `last` has landed (bounded wait; false when it ran out)
         auto gy_ready = [&](uint32_t last) -> bool {

@@ -54,7 +54,7 @@ struct TArgs {
     uint32_t* pmask;       // the STE mask at one bit per element, or null
     uint32_t* pcodes;      // the codes as a bit string of code_bits each, or null (y is then not written)
     int code_bits;
-    uint32_t code_words;   // planes are whole runs of 32 codes: fp32 packs write them as words
+    uint32_t code_words;   // planes are whole runs of 32 codes: they are written as words
     double* dist;          // four running sums of Table 2's statistics, or null
     uint32_t* status;
     uint32_t* kmin;
@@ -88,7 +88,8 @@ __device__ __forceinline__ void t_cp_async_wait_all() { asm volatile("cp.async.w
 
 // U = units a thread handles together in the quantize walk
 // BITS = bits of a code (EXTRAS = 3 only: shifts and lanes of the code string are then constants)
-template <typename T, int MODE, int EXTRAS, int U, int BITS>
+// At = index of a unit of the tensor: 32 bits below 64 GB
+template <typename T, int MODE, int EXTRAS, int U, int BITS, typename At>
 __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     constexpr int V = Pack<T>::V;
     constexpr bool kBwd = (MODE & MODE_BWD) != 0;
@@ -107,11 +108,11 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     // where they are: unit q lies in slab q / plane_units, and the next one of this thread is kTThreads units on
     uint32_t slab0, off0;
     a.div_plane.divmod(q0 + min(tid, n), slab0, off0);
-    const uint64_t first = (uint64_t)slab0 * a.slab_units + off0;
+    const At first = (At)slab0 * a.slab_units + off0;
     uint32_t dslab, doff;
     a.div_plane.divmod((uint32_t)kTThreads, dslab, doff);
-    const uint64_t dstep = (uint64_t)dslab * a.slab_units + doff, dwrap = a.slab_units - a.plane_units;
-    auto advance = [&](uint64_t& at, uint32_t& off) {
+    const At dstep = (At)dslab * a.slab_units + doff, dwrap = a.slab_units - a.plane_units;
+    auto advance = [&](At& at, uint32_t& off) {
         at += dstep;
         off += doff;
         if (off >= a.plane_units) {
@@ -119,6 +120,9 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
             at += dwrap;
         }
     };
+    // words of codes and fp32 masks take neighbouring lanes together: units that every lane of the warp has (the first lanes may have one more)
+    constexpr bool kPairs = EXTRAS == 3 || (EXTRAS == 2 && V == 4);
+    const uint32_t whole = kPairs ? __shfl_sync(kFullMask, cnt, 31) : cnt;
     uint4* tile = t_smem + tid;
     uint4* tileg = t_smem + a.tile_units + tid;
     const uint32_t gcnt = kBwd ? (tid < a.gy_units ? min(cnt, (a.gy_units - tid + kTThreads - 1) / kTThreads) : 0u) : 0u;
@@ -133,7 +137,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
 
     // the first channel's copies; those of the later ones are sent from the quantize walk
     {
-        uint64_t at = first + (uint64_t)team * a.plane_units;
+        At at = first + (At)team * a.plane_units;
         uint32_t off = off0;
         for (uint32_t i = 0; i < cnt; ++i) {
             cp_async_16(tile + i * kTThreads, xg + at);
@@ -199,36 +203,25 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
 
         // ---- Eq. 1, clamp, Eq. 6, STE from shared memory; the next channel's copies follow on the heels ----
         const bool more = c + a.teams < a.C;
-        const uint64_t ahead = (uint64_t)a.teams * a.plane_units;
-        auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint64_t at) {
+        const At ahead = (At)a.teams * a.plane_units;
+        auto quantize = [&](const Pack<T>& px, const Pack<T>& pg, At at, uint32_t (&cb)[V / 4], uint32_t (&mb)[V / 4]) {
             Pack<T> py, pgx;
-            uint32_t cb[V / 4], mb[V / 4];
             // with a gradient the scalar form: f32 [190,4,96,97] 28.0 us, in packed pairs 29.5; [112,126,56,56] 132.7 / 137.3
             if constexpr (kBwd) quantize_pack<T, kBwd, false, EXTRAS, true>(px, pg, g, g, V, qmax, py, pgx, cb, mb);
             else quantize_own<T, kBwd, EXTRAS>(px, pg, g, qmax, py, pgx, cb, mb, BITS);
-            if constexpr (EXTRAS == 3) {
-                const uint64_t str = code_string_of<V>(cb, BITS);
-                if constexpr (V == 4) {
-                    if (a.code_words) {
-                        store_code_words<BITS>(a.pcodes, at * V, (uint32_t)str, lane);
-                        return;
-                    }
-                }
-                store_code_bytes<V>(a.pcodes, at * V, str, BITS, lane);
-                return;
-            }
-            st_stream_16(yg + at, py.raw);
+            if constexpr (EXTRAS != 3) st_stream_16(yg + at, py.raw);
             if constexpr (kBwd) st_stream_16(gxg + at, pgx.raw);
             if constexpr (EXTRAS == 4) dacc.add(px, py);
-            if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, at * V, mask_bits_of<V, EXTRAS>(mb), lane);
         };
-        uint64_t at = first + (uint64_t)c * a.plane_units;
+        At at = first + (At)c * a.plane_units;
         uint32_t off = off0, i = 0;
-        for (; i + U <= cnt; i += U) {
-            Pack<T> px[U], pg[U];
-            uint64_t w[U];
+        // N units of every lane of the warp
+        auto together = [&](auto number) {
+            constexpr int N = decltype(number)::value;
+            Pack<T> px[N], pg[N];
+            At w[N];
 #pragma unroll
-            for (int j = 0; j < U; ++j) {
+            for (int j = 0; j < N; ++j) {
                 w[j] = at;
                 if constexpr (kBwd) {
                     if (i + j < gcnt) pg[j].raw = tileg[(i + j) * kTThreads];
@@ -239,15 +232,42 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
             }
             if (more) {
 #pragma unroll
-                for (int j = 0; j < U; ++j) {
-                    cp_async_16(tile + (i + j) * kTThreads, xg + w[j] + ahead);
-                    if (kBwd && i + j < gcnt) cp_async_16(tileg + (i + j) * kTThreads, gyg + w[j] + ahead);
+                for (int j = 0; j < N; ++j) {
+                    cp_async_16(tile + (i + j) * kTThreads, xg + (w[j] + ahead));
+                    if (kBwd && i + j < gcnt) cp_async_16(tileg + (i + j) * kTThreads, gyg + (w[j] + ahead));
                 }
             }
+            i += N;
+            uint32_t cb[N][V / 4], mb[N][V / 4];
 #pragma unroll
-            for (int j = 0; j < U; ++j) emit(px[j], pg[j], w[j]);
-        }
-        for (; i < cnt; ++i) {
+            for (int j = 0; j < N; ++j) {
+                quantize(px[j], pg[j], w[j], cb[j], mb[j]);
+                if constexpr (EXTRAS == 2 && V == 8) reinterpret_cast<uint8_t*>(a.pmask)[w[j]] = (uint8_t)mb[j][0];
+                if constexpr (EXTRAS == 3 && V == 8) {
+                    const uint64_t str = code_string_of<V>(cb[j], BITS);
+                    if (a.code_words) store_code_words<BITS, 1>(a.pcodes, w[j], str, lane & 3u, lane);
+                    else store_eight_codes(a.pcodes, w[j], str, BITS);
+                }
+            }
+            if constexpr (EXTRAS == 2 && V == 4) {
+                uint32_t bits[N];
+#pragma unroll
+                for (int j = 0; j < N; ++j) bits[j] = mb[j][0];
+                const uint32_t bytes = pair_up_mask<N>(bits, lane);
+#pragma unroll
+                for (int j = 0; j < N; j += 2)
+                    reinterpret_cast<uint8_t*>(a.pmask)[(lane & 1 ? w[j + 1] : w[j]) >> 1] = (uint8_t)(bytes >> (4 * j));
+            } else if constexpr (EXTRAS == 3 && V == 4) {
+#pragma unroll
+                for (int j = 0; j < N; j += 2) {
+                    const uint64_t str = pair_up_codes(cb[j][0], cb[j + 1][0], BITS, lane);
+                    const At eight = (lane & 1 ? w[j + 1] : w[j]) >> 1;
+                    if (a.code_words) store_code_words<BITS, 2>(a.pcodes, eight, str, (lane >> 1) & 3u, lane);
+                    else store_eight_codes(a.pcodes, eight, str, BITS);
+                }
+            }
+        };
+        auto alone = [&](uint32_t lanes) {
             Pack<T> px, pg;
             if constexpr (kBwd) {
                 if (i < gcnt) pg.raw = tileg[i * kTThreads];
@@ -255,11 +275,24 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
             }
             px.raw = tile[i * kTThreads];
             if (more) {
-                cp_async_16(tile + i * kTThreads, xg + at + ahead);
-                if (kBwd && i < gcnt) cp_async_16(tileg + i * kTThreads, gyg + at + ahead);
+                cp_async_16(tile + i * kTThreads, xg + (at + ahead));
+                if (kBwd && i < gcnt) cp_async_16(tileg + i * kTThreads, gyg + (at + ahead));
             }
-            emit(px, pg, at);
+            uint32_t cb[V / 4], mb[V / 4];
+            quantize(px, pg, at, cb, mb);
+            if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, (size_t)at * V, mask_bits_of<V, EXTRAS>(mb), lane, lanes);
+            if constexpr (EXTRAS == 3) store_code_bytes<V>(a.pcodes, (size_t)at * V, code_string_of<V>(cb, BITS), BITS, lane, lanes);
             advance(at, off);
+            ++i;
+        };
+        while (i + U <= whole) together(PartAt<U>{});
+        if constexpr (kPairs && U > 2) {
+            if (i + 2 <= whole) together(PartAt<2>{});
+        }
+        while (i < whole) alone(kFullMask);
+        if constexpr (kPairs) {
+            const uint32_t lanes = __ballot_sync(kFullMask, i < cnt);
+            if (i < cnt) alone(lanes);
         }
     }
     if constexpr (EXTRAS == 4) dacc.flush(a.dist);
@@ -497,11 +530,15 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_lag_kernel(const TArgs a
 
 template <typename T, int MODE, int EXTRAS, int BITS = 8>
 cudaError_t t_launch(const TArgs& args, const TeamPlan& p, const StagedTuning& tune, cudaStream_t st) {
-    auto kern = colteam_kernel<T, MODE, EXTRAS, (MODE == MODE_FWD ? 4 : 2), BITS>;
-    const cudaError_t e = allow_smem(kern, kTSmemUnits * 16);
-    if (e != cudaSuccess) return e;
-    void* params[] = {(void*)&args};
-    return launch_cooperative((const void*)kern, args.R * args.teams, kTThreads, params, p.smem_bytes, tune, st);
+    constexpr int U = MODE == MODE_FWD ? 4 : 2;
+    auto go = [&](auto kern) -> cudaError_t {
+        const cudaError_t e = allow_smem(kern, kTSmemUnits * 16);
+        if (e != cudaSuccess) return e;
+        void* params[] = {(void*)&args};
+        return launch_cooperative((const void*)kern, args.R * args.teams, kTThreads, params, p.smem_bytes, tune, st);
+    };
+    return (uint64_t)args.units * args.C < (1ull << 32) ? go(colteam_kernel<T, MODE, EXTRAS, U, BITS, uint32_t>)
+                                                        : go(colteam_kernel<T, MODE, EXTRAS, U, BITS, uint64_t>);
 }
 
 template <typename T>

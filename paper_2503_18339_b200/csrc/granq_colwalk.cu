@@ -291,6 +291,7 @@ __global__ void __launch_bounds__(kCThreads, 4) colwalk_kernel(const CArgs a) {
         }
         for (uint32_t item = first_item(w); item < sh.nitems; item += gridDim.x) {
             const Item it = make_item(sh, item);
+            const uint32_t lanes = V == 4 && EXTRAS != 0 ? __ballot_sync(kFullMask, it.valid) : 0u;      // they walk the same slabs
             if (!it.valid) continue;
             size_t gu = (size_t)it.n0 * slab + base + it.u;
             // the channel's parameters (Eq. 5), once per walk
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(kCThreads, 4) colwalk_kernel(const CArgs a) {
                 if constexpr (EXTRAS == 3) {
                     // the packed codes are the only output: 8 codes = b bytes per pair of fp32 lanes (per bf16 lane);
                     // the planner has made every slab and wave whole groups of 8 elements
-                    store_code_bytes<V>(a.pcodes, at * V, code_string_of<V>(cb, a.code_bits), a.code_bits, lane);
+                    store_code_bytes<V>(a.pcodes, at * V, code_string_of<V>(cb, a.code_bits), a.code_bits, lane, lanes);
                     return;
                 }
                 st_hint_16(yg + at, py.raw, drop);
@@ -328,7 +329,7 @@ __global__ void __launch_bounds__(kCThreads, 4) colwalk_kernel(const CArgs a) {
                         // the mask is written byte by byte (8 elements: two fp32 packs of neighbouring lanes, one
                         // bf16 pack); the planner has made every slab and wave whole mask words, so both lanes of a
                         // byte are here together
-                        store_mask_byte<V>(a.pmask, at * V, mask_bits_of<V, EXTRAS>(mb), lane);
+                        store_mask_byte<V>(a.pmask, at * V, mask_bits_of<V, EXTRAS>(mb), lane, lanes);
                     }
                 }
             };

@@ -735,13 +735,21 @@ __device__ __forceinline__ uint32_t mask_bits_of(const uint32_t (&mb)[V / 4]) {
     }
 }
 
+// Masks and codes are written 8 elements at a time, which takes two neighbouring lanes of fp32 packs, and words of codes
+// eight.  `lanes` are the lanes of the warp that are here, whole groups of them, and the same value in every lane: with a mask
+// per group the warp goes through a shuffle group by group (forward with packed mask [128,64,56,56] 50.4 -> 45.6 us, 4-bit codes of
+// [128,256,14,14] 20.3 -> 16.6).
+__device__ __forceinline__ uint32_t from_lane(uint32_t lanes, uint32_t v, uint32_t src) {
+    return lanes == kFullMask ? __shfl_sync(kFullMask, v, (int)src) : __shfl_sync(lanes, v, (int)src);
+}
+
 // Store the packed mask one byte (8 elements) at a time: `bits` are the V mask bits of the pack that starts at
 // element `first` (a multiple of V; for V = 4 the even lane of a pair holds the low half of a byte, and both
 // lanes of the pair must call this together with neighbouring packs).
 template <int V>
-__device__ __forceinline__ void store_mask_byte(uint32_t* pmask, size_t first, uint32_t bits, uint32_t lane) {
+__device__ __forceinline__ void store_mask_byte(uint32_t* pmask, size_t first, uint32_t bits, uint32_t lane, uint32_t lanes) {
     if constexpr (V == 4) {
-        const uint32_t other = __shfl_xor_sync(3u << (lane & ~1u), bits, 1);
+        const uint32_t other = from_lane(lanes, bits, lane ^ 1u);
         if (!(lane & 1)) reinterpret_cast<uint8_t*>(pmask)[first >> 3] = (uint8_t)(bits | (other << 4));
     } else {
         static_assert(V == 8, "a pack is 4 or 8 elements");
@@ -757,57 +765,79 @@ __device__ __forceinline__ uint64_t code_string_of(const uint32_t (&cb)[V / 4], 
     return str;
 }
 
-// Store the packed codes 8 codes = b bytes at a time: `str` is the code string of the pack that starts at element
-// `first` (a multiple of V); byte (first / 8) * b of the bit string is where the 8 codes of an aligned group of 8
-// elements begin.  For V = 4 the even lane of a pair holds the first half and stores; both lanes of the pair must
-// call this together with neighbouring packs.  The buffer is only known to be 4-byte aligned.
-template <int V>
-__device__ __forceinline__ void store_code_bytes(uint32_t* pcodes, size_t first, uint64_t str, int code_bits, uint32_t lane) {
-    uint64_t eight = str;
-    if constexpr (V == 4) {
-        const uint32_t other = __shfl_xor_sync(3u << (lane & ~1u), (uint32_t)str, 1);
-        if (lane & 1) return;
-        eight |= (uint64_t)other << (4 * code_bits);
-    }
-    uint8_t* dst = reinterpret_cast<uint8_t*>(pcodes) + (first >> 3) * (size_t)code_bits;
+// b bytes: the codes of the elements 8 * eight ... of the bit string.  The buffer is only known to be 4-byte aligned.
+__device__ __forceinline__ void store_eight_codes(uint32_t* pcodes, size_t eight, uint64_t str, int code_bits) {
+    uint8_t* dst = reinterpret_cast<uint8_t*>(pcodes) + eight * (size_t)code_bits;
     switch (code_bits) {
         case 8:
-            reinterpret_cast<uint32_t*>(dst)[0] = (uint32_t)eight;
-            reinterpret_cast<uint32_t*>(dst)[1] = (uint32_t)(eight >> 32);
+            reinterpret_cast<uint32_t*>(dst)[0] = (uint32_t)str;
+            reinterpret_cast<uint32_t*>(dst)[1] = (uint32_t)(str >> 32);
             break;
-        case 4: *reinterpret_cast<uint32_t*>(dst) = (uint32_t)eight; break;
-        case 2: *reinterpret_cast<uint16_t*>(dst) = (uint16_t)eight; break;
+        case 4: *reinterpret_cast<uint32_t*>(dst) = (uint32_t)str; break;
+        case 2: *reinterpret_cast<uint16_t*>(dst) = (uint16_t)str; break;
         case 6:
-            reinterpret_cast<uint16_t*>(dst)[0] = (uint16_t)eight;
-            reinterpret_cast<uint16_t*>(dst)[1] = (uint16_t)(eight >> 16);
-            reinterpret_cast<uint16_t*>(dst)[2] = (uint16_t)(eight >> 32);
+            reinterpret_cast<uint16_t*>(dst)[0] = (uint16_t)str;
+            reinterpret_cast<uint16_t*>(dst)[1] = (uint16_t)(str >> 16);
+            reinterpret_cast<uint16_t*>(dst)[2] = (uint16_t)(str >> 32);
             break;
         default:
-            for (int t = 0; t < code_bits; ++t) dst[t] = (uint8_t)(eight >> (8 * t));
+            for (int t = 0; t < code_bits; ++t) dst[t] = (uint8_t)(str >> (8 * t));
             break;
     }
 }
 
-// Store the packed codes of fp32 packs as whole words: 8 neighbouring lanes hold 32 consecutive codes = BITS whole words
-// of the bit string, the first of them an element whose index is a multiple of 32; lane k < BITS assembles word k from
-// the lanes whose strings reach into it.  All 8 lanes must call together.  One coalesced store in place of BITS single
-// bytes per pair of lanes, each of which rewrote part of a sector in the L2: 5-bit codes of [128,144,56,56] 104 -> 86 us
-// with the shifts as constants (with BITS a variable the assembly costs more than it saves: 136 us; and bf16, whose
-// lanes hold 8 codes and need 64-bit shuffles, is faster with bytes: 54 against 80 us).
-template <int BITS>
-__device__ __forceinline__ void store_code_words(uint32_t* pcodes, size_t first, uint32_t str, uint32_t lane) {
-    constexpr uint32_t NB = 4 * BITS;                          // bits of one lane's string
-    constexpr uint32_t kMost = (30 + 2 * NB) / NB < 8 ? (30 + 2 * NB) / NB : 8;      // lanes that can reach into one word
-    const uint32_t sub = lane & 7u, group = lane & ~7u, mask = 0xFFu << group;
-    const uint32_t from = (32u * sub) / NB;                    // the first of them
-    uint32_t word = 0;
-#pragma unroll
-    for (uint32_t k = 0; k < kMost; ++k) {
-        const uint32_t v = __shfl_sync(mask, str, group + ((from + k) & 7u));
-        const int off = (int)((from + k) * NB) - (int)(32u * sub);               // where its string begins in the word
-        if (from + k < 8 && off < 32) word |= off >= 0 ? (v << off) : (v >> -off);
+// Store the packed codes 8 codes = b bytes at a time: `str` is the code string of the pack that starts at element
+// `first` (a multiple of V).  For V = 4 the even lane of a pair holds the first half and stores; both lanes of the pair must
+// call this together with neighbouring packs.
+template <int V>
+__device__ __forceinline__ void store_code_bytes(uint32_t* pcodes, size_t first, uint64_t str, int code_bits, uint32_t lane, uint32_t lanes) {
+    uint64_t eight = str;
+    if constexpr (V == 4) {
+        const uint32_t other = from_lane(lanes, (uint32_t)str, lane ^ 1u);
+        if (lane & 1) return;
+        eight |= (uint64_t)other << (4 * code_bits);
     }
-    if (sub < (uint32_t)BITS) pcodes[(first >> 5) * (size_t)BITS + sub] = word;
+    store_eight_codes(pcodes, first >> 3, eight, code_bits);
+}
+
+// Two fp32 packs of every lane of a warp at once: the strings s0 and s1 (4 * b bits) of this lane's packs, the lane beside it
+// holding their neighbours.  The even lane of a pair leaves with the eight codes of the first, the odd lane with those of the
+// second: one shuffle and, behind it, one store for two packs of a lane.
+__device__ __forceinline__ uint64_t pair_up_codes(uint32_t s0, uint32_t s1, int code_bits, uint32_t lane) {
+    const bool odd = lane & 1u;
+    const uint32_t got = __shfl_xor_sync(kFullMask, odd ? s0 : s1, 1);
+    return (odd ? got : s0) | ((uint64_t)(odd ? s1 : got) << (4 * code_bits));
+}
+// The same for the mask: 4 bits of each of U packs, U / 2 bytes of every lane for one shuffle, byte k that of pack 2 k (even lane)
+// or 2 k + 1 (odd lane).
+template <int U>
+__device__ __forceinline__ uint32_t pair_up_mask(const uint32_t (&bits)[U], uint32_t lane) {
+    static_assert(U == 2 || U == 4, "one byte or two of every lane");
+    const uint32_t a = U == 4 ? bits[0] | (bits[U - 2] << 8) : bits[0], b = U == 4 ? bits[1] | (bits[U - 1] << 8) : bits[1];
+    const bool odd = lane & 1u;
+    const uint32_t got = __shfl_xor_sync(kFullMask, odd ? a : b, 1);
+    return (odd ? got : a) | ((odd ? b : got) << 4);
+}
+
+// Store the codes of 8 elements per lane as whole words: four lanes, STRIDE apart, hold 32 consecutive codes = BITS whole words
+// of the bit string, the first of them an element whose index is a multiple of 32 (q: which of the four this lane is).  Strings
+// of 3 bytes: word q is this lane's string and the next one's; of 5 to 7 bytes: a lane completes the word its string begins in with
+// the end of the string before, and adds the word that its own string may hold besides.  One shuffle and one or two coalesced
+// stores in place of BITS single bytes, each of which rewrote part of a sector in the L2.  The whole warp must call.
+template <int BITS, int STRIDE>
+__device__ __forceinline__ void store_code_words(uint32_t* pcodes, size_t eight, uint64_t str, uint32_t q, uint32_t lane) {
+    uint32_t* dst = pcodes + (eight >> 2) * (size_t)BITS;
+    if constexpr (BITS == 3) {
+        const uint32_t next = __shfl_sync(kFullMask, (uint32_t)str, (int)((lane + STRIDE) & 31u));
+        if (q < 3) dst[q] = __funnelshift_r((uint32_t)str | (next << 24), next >> 8, 8 * q);
+    } else if constexpr (BITS > 4 && BITS < 8) {
+        const uint32_t before = __shfl_sync(kFullMask, (uint32_t)(str >> (8 * BITS - 32)), (int)((lane - STRIDE) & 31u));
+        const uint32_t at = (8 * BITS * q) & 31u, k = (BITS * q) >> 2;      // where the string begins
+        dst[k] = __funnelshift_l(before, (uint32_t)str, at);
+        if (8 * BITS - 32 + at >= 32) dst[k + 1] = (uint32_t)(str >> (32u - at));
+    } else {
+        store_eight_codes(pcodes, eight, str, BITS);
+    }
 }
 
 // ---------------------------------------------------------------------------------------

@@ -633,7 +633,8 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
                         // elements, so the lanes of a pair are valid or not together, and a lane without a pack has
                         // nothing to say)
                         if constexpr (V > 1) {
-                            if (valid) store_code_bytes<V>(pcodes, (size_t)(e0 + k[j]), code_string, code_bits, threadIdx.x & 31);
+                            const uint32_t lanes = V == 4 ? __ballot_sync(kFullMask, valid) : 0u;
+                            if (valid) store_code_bytes<V>(pcodes, (size_t)(e0 + k[j]), code_string, code_bits, threadIdx.x & 31, lanes);
                         }
                     } else if (EXTRAS == 1 && (PACKONLY || pcodes)) {      // the warp's 32 * V codes are V * b whole words of the bit string
                         const uint32_t lane = threadIdx.x & 31;

@@ -218,7 +218,8 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
     DistAcc dacc;               // Table 2's sums over everything this thread quantizes (EXTRAS = 4)
     dacc.reset();
     const GroupParam one = s_par[0];
-    auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint32_t i) {
+    constexpr bool kPairs = V == 4 && (EXTRAS == 2 || EXTRAS == 3);      // written by neighbouring lanes together
+    auto emit = [&](const Pack<T>& px, const Pack<T>& pg, uint32_t i, uint32_t lanes) {
         Pack<T> py, pgx;
         uint32_t cb[V / 4], mb[V / 4];
         const int code_bits = EXTRAS == 3 ? a.code_bits : 8;
@@ -239,12 +240,12 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
         // masks and codes 8 elements at a time, a pair of fp32 units by the two lanes of a pair, the first of them by the even one: the
         // tensor is a multiple of 32 elements, a piece begins on a multiple of 8 units, and both walks give an even lane an even unit
         if constexpr (EXTRAS == 3) {
-            store_code_bytes<V>(a.pcodes, (size_t)(u0 + i) * V, code_string_of<V>(cb, code_bits), code_bits, lane);
+            store_code_bytes<V>(a.pcodes, (size_t)(u0 + i) * V, code_string_of<V>(cb, code_bits), code_bits, lane, lanes);
             return;
         }
         st_stream_16(yg + i, py.raw);
         if constexpr (kBwd) st_stream_16(gxg + i, pgx.raw);
-        if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, (size_t)(u0 + i) * V, mask_bits_of<V, EXTRAS>(mb), lane);
+        if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, (size_t)(u0 + i) * V, mask_bits_of<V, EXTRAS>(mb), lane, lanes);
         if constexpr (EXTRAS == 4) dacc.add(px, py);
     };
     // what did not stay, a block of units at a time from the end back; inside a block forward from an even unit (masks and codes:
@@ -264,7 +265,8 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
 #pragma unroll
             for (int k = 0; k < U; ++k) {
                 const uint32_t i = k * kHThreads + tid;
-                if (i < len) emit(px[k], pg[k], start + i);
+                const uint32_t lanes = kPairs ? __ballot_sync(kFullMask, i < len) : 0u;
+                if (i < len) emit(px[k], pg[k], start + i, lanes);
             }
             end = start;
         }
@@ -282,7 +284,8 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
 #pragma unroll
         for (int k = 0; k < U; ++k) {
             const uint32_t i = b + k * kHThreads + tid;
-            if (i < held) emit(px[k], pg[k], i);
+            const uint32_t lanes = kPairs ? __ballot_sync(kFullMask, i < held) : 0u;
+            if (i < held) emit(px[k], pg[k], i, lanes);
         }
     }
     if constexpr (EXTRAS == 4) dacc.flush(a.dist);

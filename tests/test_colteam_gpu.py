@@ -86,6 +86,25 @@ def test_two_channels_side_by_side_by_default(b, dtype, shape):
     assert int(zeroed.view(torch.int32).abs().sum().item()) == 0
 
 
+@pytest.mark.parametrize("shape", [(40, 290, 16, 20), (9, 310, 4, 8), (37, 300, 8, 12)], ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_strings_of_every_width(b, knobs, shape, dtype):
+    """Codes and mask bits that neighbouring lanes write together: planes of whole words of codes and others, lanes with four
+    units at a time, two, one, and warps whose first lanes alone have one more."""
+    x, _ = make_case(shape, seed=sum(shape), dtype=dtype)
+    xd = to_dev(x)
+    knobs(col_team=1)
+    assert b.team_geometry(b.BF16 if dtype == "bf16" else b.F32, shape, with_backward=False)["taken"] == 1
+    ws = b.make_workspace(xd, zeroed=True)
+    flags = b.FLAG_FORCE_COLWALK | b.FLAG_WORKSPACE_ZEROED
+    for bits in range(1, 9):
+        ref = orc.fused(x, bits)
+        got = b.granq_quantize_packed_fused(xd, bits, out=b.FakeQuantOut(workspace=ws), flags=flags)
+        assert_same_string(got.packed_codes, orc.pack_codes(ref.codes, bits))
+        got = b.granq_fakequant_fused_fwd_packmask(xd, bits, out=b.FakeQuantOut(workspace=ws), flags=flags)
+        assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+
+
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_waves_on_aligned_planes(b, knobs, shape, dtype):
