@@ -20,7 +20,7 @@
 // forward [128,64,56,56] 55.8 -> 45.7 / 34.7 -> 30.3, [128,96,112,112] 309 -> 264 / 174 -> 139, [256,512,28,28]
 // 219 -> 156 / 123 -> 92; with a gradient 87.5 -> 81.9 / 47.4 -> 45.6, 472 -> 469 / 258 -> 234, 332 -> 298 / 183 -> 153;
 // [256,16,32,32] 16.7 -> 14.9 and 21.9 -> 19.4.  Bound by the chain of copy, hand-over and quantize when a team has one
-// channel.  With several it moves 4.5 to 5.7 TB/s where plain copies in blocks that come in order move 6.7: 90 (with a
+// channel.  With several it moves 4.5 to 5.7 TB/s where plain copies in blocks that come in order move 6.7: 66 (with a
 // packed mask) to 106 (with a gradient) instructions per unit, sixteen wavefronts for an asynchronous copy of a warp, and
 // equal shares, of which half of the SMs move 21 KB/us and the other half 37 when nothing holds them together.  Chunks dealt
 // out by a counter even the SMs out but publish, poll and fetch keys per chunk: 10 us of residence against the 10 us that

@@ -737,8 +737,9 @@ __device__ __forceinline__ uint32_t mask_bits_of(const uint32_t (&mb)[V / 4]) {
 
 // Masks and codes are written 8 elements at a time, which takes two neighbouring lanes of fp32 packs, and words of codes
 // eight.  `lanes` are the lanes of the warp that are here, whole groups of them, and the same value in every lane: with a mask
-// per group the warp goes through a shuffle group by group (forward with packed mask [128,64,56,56] 50.4 -> 45.6 us, 4-bit codes of
-// [128,256,14,14] 20.3 -> 16.6).
+// per group the warp goes through a shuffle group by group: 61 % of the time of the unit that takes it on, packed mask of
+// [128,64,56,56] (the kernel alone, with what else follows here: 51.3 -> 41.9 us; 5-bit codes of [128,144,56,56] 83.9 -> 65.9, 4-bit codes of
+// [128,256,14,14] 21.8 -> 18.0).
 __device__ __forceinline__ uint32_t from_lane(uint32_t lanes, uint32_t v, uint32_t src) {
     return lanes == kFullMask ? __shfl_sync(kFullMask, v, (int)src) : __shfl_sync(lanes, v, (int)src);
 }
@@ -823,7 +824,8 @@ __device__ __forceinline__ uint32_t pair_up_mask(const uint32_t (&bits)[U], uint
 // of the bit string, the first of them an element whose index is a multiple of 32 (q: which of the four this lane is).  Strings
 // of 3 bytes: word q is this lane's string and the next one's; of 5 to 7 bytes: a lane completes the word its string begins in with
 // the end of the string before, and adds the word that its own string may hold besides.  One shuffle and one or two coalesced
-// stores in place of BITS single bytes, each of which rewrote part of a sector in the L2.  The whole warp must call.
+// stores in place of BITS single bytes, each of which rewrote part of a sector in the L2.  The whole warp must call.  Codes and their
+// expansion, us: fp32 [128,144,56,56] at 3, 5, 8 bits 135 -> 109, 125 -> 109, 125 -> 115; bf16, whose bytes were no slower, 72 / 72, 85 / 83.
 template <int BITS, int STRIDE>
 __device__ __forceinline__ void store_code_words(uint32_t* pcodes, size_t eight, uint64_t str, uint32_t q, uint32_t lane) {
     uint32_t* dst = pcodes + (eight >> 2) * (size_t)BITS;
