@@ -86,6 +86,14 @@ __device__ __forceinline__ uint64_t a_smem_desc(const void* tile) {
 __device__ __forceinline__ uint32_t a_instr_desc(uint32_t n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((uint32_t)(kABm >> 4) << 24);
 }
+// One lane of a converged warp, chosen in the way that the compiler knows to be one lane: behind a test of the thread's
+// number it wraps every tcgen05.mma in a loop over the lanes that may be there, 273 cycles each whatever its size where one
+// of 128 x 256 x 16 takes 128.
+__device__ __forceinline__ bool a_elected() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void a_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -143,9 +151,8 @@ __device__ __forceinline__ uint64_t a_codes8(const uint32_t* __restrict__ packed
     return keep >= 64 ? v : (v & ((1ull << keep) - 1ull));
 }
 
-// The same in two steps, so that the loads can be issued long before their words are needed: a_codes8_load() only
-// loads (up to three words, none beyond the end of the bit string) and returns the shift; a_codes8_finish() lines
-// the codes up at bit 0 and clears what lies above them.
+// The same without the lining up, so that the loads can be issued long before their words are needed: up to three words, none
+// beyond the end of the bit string; returns the shift.
 __device__ __forceinline__ uint32_t a_codes8_load(const uint32_t* __restrict__ packed, uint64_t bit, uint32_t nbits,
                                                   int64_t nwords, uint32_t& w0, uint32_t& w1, uint32_t& w2) {
     const int64_t w = (int64_t)(bit >> 5);
@@ -156,13 +163,20 @@ __device__ __forceinline__ uint32_t a_codes8_load(const uint32_t* __restrict__ p
     w2 = (need > 64 && w + 2 < nwords) ? __ldg(packed + w + 2) : 0u;
     return sh;
 }
-__device__ __forceinline__ uint64_t a_codes8_finish(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t sh, int keep_bits) {
-    const uint64_t v = ((uint64_t)__funnelshift_r(w1, w2, sh) << 32) | __funnelshift_r(w0, w1, sh);
-    return keep_bits >= 64 ? v : (v & ((1ull << keep_bits) - 1ull));
-}
-
 // two codes -> two bf16 in one word (the first in the low half), exact.  Codes below 128: 0x4300 | code is the
-// bf16 number 128 + code, and one packed subtraction of 128 gives the code; 8-bit codes go through fp32.
+// bf16 number 128 + code, and one packed subtraction of 128 gives the code; 8-bit codes go through fp32, as 2^23 + code.
+__device__ __forceinline__ uint32_t a_pair_narrow(uint32_t biased) {
+    const uint32_t bias = 0x43004300u;
+    const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&biased),
+                                     *reinterpret_cast<const __nv_bfloat162*>(&bias));
+    return *reinterpret_cast<const uint32_t*>(&d);
+}
+__device__ __forceinline__ uint32_t a_pair_wide(uint32_t biased0, uint32_t biased1) {
+    float f0, f1;
+    f2_split(f2_sub(f2(__uint_as_float(biased0), __uint_as_float(biased1)), f2(8388608.0f, 8388608.0f)), f0, f1);
+    const __nv_bfloat162 d = __floats2bfloat162_rn(f0, f1);
+    return *reinterpret_cast<const uint32_t*>(&d);
+}
 __device__ __forceinline__ uint32_t a_pair_bf16(uint32_t c0, uint32_t c1, bool wide) {
     if (!wide) {
         const uint32_t biased = c0 | (c1 << 16) | 0x43004300u, bias = 0x43004300u;
@@ -393,9 +407,8 @@ __device__ __forceinline__ void a_tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
 //   warps 17 .. 24 two groups of four warps take the finished accumulators in turn (a warp reads the 32 lanes of
 //                  its quarter, warp % 4, 16 columns of each half at a time), add the halves, subtract the bias and
 //                  store y; while one group stores, the other reads tensor memory.
-// Both weight halves sit one after the other in shared memory and are multiplied as ONE operand of 2 BN columns
-// (an MMA of 128 x 64 x 16 spends its time fetching the 128 x 16 code operand, not computing: with both halves
-// behind one fetch the tensor core is busy half as long); the epilogue adds the two column blocks.
+// Both weight halves sit one after the other in shared memory and are multiplied as ONE operand of 2 BN columns: half the
+// instructions and one fetch of the 128 x 16 codes for both.  The epilogue adds the two column blocks.
 // The CTA owns all 512 columns of its SM's tensor memory: 512 / (2 BN) accumulators in turn, so the MMAs run
 // tiles ahead of the epilogue (a hand-over from the tensor core to the epilogue and back costs about a
 // microsecond; with two accumulators that latency, not the work, set the pace).  Needs the weight halves of
@@ -409,14 +422,22 @@ constexpr int kPThreads = kPProducers + 32 + kPEpilogue;
 constexpr size_t kPWeightBytes = 128 * 1024;      // resident weight halves at most (channels-last: 16 KB less,
                                                   // which the epilogue's staging tiles take)
 
+constexpr int kPKBlocks = 8;               // K blocks whose weights can be resident
+
+struct PArgs : AArgs {
+    uint32_t VP;              // rows of one sample: P, or P rounded up to whole strings of 8 pixels
+    uint32_t vrows;           // rows of the whole batch
+    FastDiv div_vp;
+};
+
 struct PBars {
-    uint64_t a_full[kPStages], a_empty[kPStages], acc_full[8], acc_empty[8], b_full;
+    uint64_t a_full[kPStages], a_empty[kPStages], acc_full[8], acc_empty[8], b_full[kPKBlocks];
 };
 
 template <int BN, bool NHWC>
 __global__ void __launch_bounds__(kPThreads, 1)
 accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
-                             const AArgs a) {
+                             const PArgs a) {
     constexpr uint32_t kABytes = kABm * kABk * 2, kBBytes = BN * kABk * 2;
     constexpr int kAcc = kPTmemCols / (2 * BN);    // accumulators (each: BN columns for the hi half, BN for the lo half)
     static_assert(kAcc <= 8, "barriers for at most 8 accumulators");
@@ -435,10 +456,10 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
     unsigned char* ring = a_smem + ((1024u - (a_smem_u32(a_smem) & 1023u)) & 1023u);
     unsigned char* wts = ring + (size_t)kPStages * kABytes;          // per K block: hi half, lo half
     const int col0 = (int)blockIdx.y * BN;
-    const int64_t row_tiles = (a.rows + kABm - 1) / kABm;
+    const uint32_t row_tiles = (a.vrows + kABm - 1) / kABm;
     const int kblocks = a.kblocks;
     // this CTA's row tiles: blockIdx.x, blockIdx.x + gridDim.x, ...
-    const int my_tiles = (int)((row_tiles - (int64_t)blockIdx.x + gridDim.x - 1) / gridDim.x);
+    const int my_tiles = (int)((row_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x);
     const int my_iters = my_tiles * kblocks;
 
     if (tid == 0) {
@@ -450,7 +471,7 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
             a_mbar_init(&bars.acc_full[b], 1);
             a_mbar_init(&bars.acc_empty[b], 4);     // one arrival per warp of the epilogue group that reads it out
         }
-        a_mbar_init(&bars.b_full, 1);
+        for (int kb = 0; kb < kPKBlocks; ++kb) a_mbar_init(&bars.b_full[kb], 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -488,8 +509,7 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
         // ---- producers: group g takes the iterations (tile, K block) with it % kPGroups == g ----
         const uint32_t group = tid >> 7, pt = tid & 127;
         const int bits = a.bits;
-        const bool wide = bits == 8;
-        const uint32_t code_mask = (1u << bits) - 1u;
+        const uint32_t code_mask = ((1u << bits) - 1u) * 0x00010001u;      // of two codes
         const uint32_t cg = pt & 7, rq = pt >> 3;          // 8 channels of the stage's 64; row group
         // The eight code strings of this thread for iteration `it`, as loaded words (three per string) and shifts
         // (5 bits each).  NCHW: 8 channels x rows 8 rq .. 8 rq + 7 (code j of string i = channel i, row j);
@@ -497,13 +517,14 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
         struct Raw {
             uint32_t w0[8], w1[8], w2[8];
             uint64_t shifts;
-            int keep;                 // bits of a string that hold codes
         };
         // (pixel counts are below 2^31: 32-bit index arithmetic; only bit offsets need 64 bits)
-        const uint32_t rows32 = (uint32_t)a.rows, P32 = (uint32_t)a.P, C32 = (uint32_t)a.C;
-        // 4-bit codes and strings (8 codes) that are whole words of the bit string: planes (NCHW) or pixels'
-        // channel vectors (channels-last) of a multiple of 8 elements
-        const bool words4 = bits == 4 && ((NHWC ? C32 : P32) & 7u) == 0;
+        const uint32_t rows32 = a.vrows, P32 = (uint32_t)a.P, C32 = (uint32_t)a.C;
+        // channels-last: 4-bit codes of pixels' channel vectors of a multiple of 8 elements are whole words of the bit string
+        const bool words4 = NHWC && bits == 4 && (C32 & 7u) == 0;
+        // NCHW: a sample's rows are whole strings of 8 pixels (of the last one the rest is another channel's codes, in rows that are
+        // nobody's); planes below 8 pixels are not padded to that
+        const bool strings = !NHWC && (a.VP & 7u) == 0;
         auto fetch = [&](int it, Raw& r) {
             const int ti = it / kblocks, kb = it - ti * kblocks;
             const uint32_t row0 = (blockIdx.x + (uint32_t)ti * gridDim.x) * (uint32_t)kABm;
@@ -511,7 +532,6 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
             r.shifts = 0;
             if (words4) {
                 // 4-bit codes whose strings are whole, aligned words: one load per string, 32-bit arithmetic throughout
-                r.keep = 32;
                 if constexpr (NHWC) {
                     const uint32_t* src = a.packed + ((size_t)(row0 + rq) * (C32 >> 3) + (c0 >> 3));
                     const uint32_t stepw = 16u * (C32 >> 3);
@@ -520,62 +540,38 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
                         r.w0[i] = (row0 + rq + 16u * i < rows32 && c0 < C32) ? __ldg(src + (size_t)i * stepw) : 0u;
                         r.w1[i] = r.w2[i] = 0;
                     }
-                } else {
-                    const uint32_t gp0 = row0 + 8u * rq;
-                    const uint32_t n0 = gp0 / P32, p0 = gp0 - n0 * P32;
-                    const uint32_t* src = a.packed + ((((size_t)n0 * C32 + c0) * P32 + p0) >> 3);
-                    const uint32_t stepw = P32 >> 3;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        r.w0[i] = (gp0 < rows32 && c0 + i < C32) ? __ldg(src + (size_t)i * stepw) : 0u;
-                        r.w1[i] = r.w2[i] = 0;
-                    }
                 }
                 return;
             }
             if constexpr (NHWC) {
                 const uint32_t count = c0 < C32 ? min(8u, C32 - c0) : 0u;
-                r.keep = (int)count * bits;
+                const uint32_t held = count * (uint32_t)bits;
                 uint64_t bit = ((uint64_t)(row0 + rq) * C32 + c0) * (uint32_t)bits;
                 const uint64_t step = (uint64_t)16 * C32 * (uint32_t)bits;           // 16 rows on
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     r.w0[i] = r.w1[i] = r.w2[i] = 0;
                     if (row0 + rq + 16u * i < rows32 && count > 0)
-                        r.shifts |= (uint64_t)a_codes8_load(a.packed, bit, (uint32_t)r.keep, a.nwords, r.w0[i], r.w1[i], r.w2[i])
+                        r.shifts |= (uint64_t)a_codes8_load(a.packed, bit, held, a.nwords, r.w0[i], r.w1[i], r.w2[i])
                                     << (5 * i);
                     bit += step;
                 }
             } else {
                 const uint32_t gp0 = row0 + 8u * rq;
-                const uint32_t n0 = gp0 / P32, p0 = gp0 - n0 * P32;
-                const bool together = (p0 + 7 < P32) && (gp0 + 7 < rows32);
-                r.keep = 8 * bits;
-                uint64_t bit = (((uint64_t)n0 * C32 + c0) * P32 + p0) * (uint32_t)bits;
+                uint32_t n0, p0;
+                a.div_vp.divmod(gp0, n0, p0);
+                const size_t e0 = ((size_t)n0 * C32 + c0) * P32 + p0;
+                uint64_t bit = (uint64_t)e0 * (uint32_t)bits;
                 const uint64_t step = (uint64_t)P32 * (uint32_t)bits;                 // one channel on
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const uint32_t c = c0 + i;
                     r.w0[i] = r.w1[i] = r.w2[i] = 0;
                     if (c < C32 && gp0 < rows32) {
-                        if (together) {
-                            r.shifts |= (uint64_t)a_codes8_load(a.packed, bit, (uint32_t)r.keep, a.nwords, r.w0[i], r.w1[i],
+                        if (strings) {
+                            r.shifts |= (uint64_t)a_codes8_load(a.packed, bit, 8u * (uint32_t)bits, a.nwords, r.w0[i], r.w1[i],
                                                                 r.w2[i])
                                         << (5 * i);
-                        } else if (P32 >= 8) {
-                            // a sample boundary or the end of the batch inside: the rows up to the boundary are one run of
-                            // this channel's codes in sample n0, the rest the first codes of the channel in sample n0 + 1
-                            const uint32_t live = min(8u, rows32 - gp0), first = min(live, P32 - p0), rest = live - first;
-                            uint32_t x0, x1, x2;
-                            uint32_t sh = a_codes8_load(a.packed, bit, first * (uint32_t)bits, a.nwords, x0, x1, x2);
-                            uint64_t v = a_codes8_finish(x0, x1, x2, sh, (int)first * bits);
-                            if (rest) {
-                                const uint64_t bit2 = (((uint64_t)(n0 + 1) * C32 + c) * P32) * (uint32_t)bits;
-                                sh = a_codes8_load(a.packed, bit2, rest * (uint32_t)bits, a.nwords, x0, x1, x2);
-                                v |= a_codes8_finish(x0, x1, x2, sh, (int)rest * bits) << (first * (uint32_t)bits);
-                            }
-                            r.w0[i] = (uint32_t)v;
-                            r.w1[i] = (uint32_t)(v >> 32);
                         } else {                                 // planes of fewer than 8 pixels: code by code
                             uint64_t v = 0;
                             for (uint32_t j = 0; j < 8; ++j) {
@@ -593,81 +589,124 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
                 }
             }
         };
+        // 4-bit codes: a string is the 8 nibbles of one word.  Even and odd nibbles are spread to bytes with two masks, byte permutes
+        // put a pair of codes beside the constant 0x43 (0x43cc is the bf16 number 128 + cc), and one packed subtraction of 128
+        // leaves the two codes as bf16: 13 instructions for 8 codes.
+        auto two = [&](uint32_t x, uint32_t sel) -> uint32_t { return a_pair_narrow(__byte_perm(x, 0x43434343u, sel)); };
         auto store = [&](unsigned char* tile, const Raw& r) {
-            if (bits == 4) {
-                // 4-bit codes: a string is the 8 nibbles of one word.  Even and odd nibbles are spread to bytes with two
-                // masks, byte permutes put a pair of codes beside the constant 0x43 (0x43cc is the bf16 number 128 + cc),
-                // and one packed subtraction of 128 leaves the two codes as bf16: 13 instructions for 8 codes.
-                const uint32_t k43 = 0x43434343u, k128 = 0x43004300u;
-                auto two = [&](uint32_t x, uint32_t sel) -> uint32_t {
-                    const uint32_t biased = __byte_perm(x, k43, sel);
-                    const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&biased),
-                                                     *reinterpret_cast<const __nv_bfloat162*>(&k128));
-                    return *reinterpret_cast<const uint32_t*>(&d);
-                };
-                uint32_t u[8];
+            if (NHWC && bits == 4) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    u[i] = __funnelshift_r(r.w0[i], r.w1[i], (uint32_t)(r.shifts >> (5 * i)) & 31u);
-                    if (r.keep < 32) u[i] &= (1u << r.keep) - 1u;
-                }
-                if constexpr (NHWC) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {          // string i = row rq + 16 i, its nibbles = 8 channels
-                        const uint32_t lo = u[i] & 0x0F0F0F0Fu, hi = (u[i] >> 4) & 0x0F0F0F0Fu;
-                        const uint32_t x01 = __byte_perm(lo, hi, 0x5140), x23 = __byte_perm(lo, hi, 0x7362);
-                        const uint32_t w[4] = {two(x01, 0x4140), two(x01, 0x4342), two(x23, 0x4140), two(x23, 0x4342)};
-                        a_store_chunk(tile, rq + 16u * i, cg, w);
-                    }
-                } else {
-                    uint32_t w[8][4];                      // [row][pair of channels]
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {          // strings 2h, 2h + 1 = two channels, nibble j = row 8 rq + j
-                        const uint32_t alo = u[2 * h] & 0x0F0F0F0Fu, ahi = (u[2 * h] >> 4) & 0x0F0F0F0Fu;
-                        const uint32_t blo = u[2 * h + 1] & 0x0F0F0F0Fu, bhi = (u[2 * h + 1] >> 4) & 0x0F0F0F0Fu;
-                        const uint32_t e01 = __byte_perm(alo, blo, 0x5140), e23 = __byte_perm(alo, blo, 0x7362);    // rows 0 2 | 4 6
-                        const uint32_t o01 = __byte_perm(ahi, bhi, 0x5140), o23 = __byte_perm(ahi, bhi, 0x7362);    // rows 1 3 | 5 7
-                        w[0][h] = two(e01, 0x4140);
-                        w[2][h] = two(e01, 0x4342);
-                        w[4][h] = two(e23, 0x4140);
-                        w[6][h] = two(e23, 0x4342);
-                        w[1][h] = two(o01, 0x4140);
-                        w[3][h] = two(o01, 0x4342);
-                        w[5][h] = two(o23, 0x4140);
-                        w[7][h] = two(o23, 0x4342);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) a_store_chunk(tile, 8u * rq + j, cg, w[j]);
+                for (int i = 0; i < 8; ++i) {              // string i = row rq + 16 i, its nibbles = 8 channels
+                    const uint32_t u = __funnelshift_r(r.w0[i], r.w1[i], (uint32_t)(r.shifts >> (5 * i)) & 31u);
+                    const uint32_t lo = u & 0x0F0F0F0Fu, hi = (u >> 4) & 0x0F0F0F0Fu;
+                    const uint32_t x01 = __byte_perm(lo, hi, 0x5140), x23 = __byte_perm(lo, hi, 0x7362);
+                    const uint32_t w[4] = {two(x01, 0x4140), two(x01, 0x4342), two(x23, 0x4140), two(x23, 0x4342)};
+                    a_store_chunk(tile, rq + 16u * i, cg, w);
                 }
                 return;
             }
-            uint64_t v[8];
+            // codes 0 .. 3 and 4 .. 7 of every string, a word each (what lies above a code is masked out where it is used; codes beyond
+            // the last channel meet weights of 0)
+            uint32_t v[8][2];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                v[i] = a_codes8_finish(r.w0[i], r.w1[i], r.w2[i], (uint32_t)(r.shifts >> (5 * i)) & 31u, r.keep);
-            if constexpr (NHWC) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        const uint32_t e0 = (uint32_t)v[i] & code_mask;
-                        v[i] >>= bits;
-                        const uint32_t e1 = (uint32_t)v[i] & code_mask;
-                        v[i] >>= bits;
-                        w[h] = a_pair_bf16(e0, e1, wide);
-                    }
-                    a_store_chunk(tile, rq + 16u * i, cg, w);
-                }
-            } else {
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t sh = (uint32_t)(r.shifts >> (5 * i)) & 31u;
+                const uint32_t lo = __funnelshift_r(r.w0[i], r.w1[i], sh), hi = __funnelshift_r(r.w1[i], r.w2[i], sh);
+                v[i][0] = lo;
+                v[i][1] = bits == 8 ? hi : __funnelshift_r(lo, hi, 4u * (uint32_t)bits);
+            }
+            auto pairs = [&](auto pair) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     uint32_t w[4];
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
-                        w[h] = a_pair_bf16((uint32_t)v[2 * h] & code_mask, (uint32_t)v[2 * h + 1] & code_mask, wide);
-                        v[2 * h] >>= bits;
-                        v[2 * h + 1] >>= bits;
+                        if constexpr (NHWC) w[h] = pair(v[j][h >> 1] >> ((2 * h & 3) * bits), v[j][h >> 1] >> ((2 * h & 3) * bits + bits));
+                        else w[h] = pair(v[2 * h][j >> 2] >> ((j & 3) * bits), v[2 * h + 1][j >> 2] >> ((j & 3) * bits));
+                    }
+                    a_store_chunk(tile, NHWC ? rq + 16u * j : 8u * rq + j, cg, w);
+                }
+            };
+            if (bits == 8) {
+                pairs([&](uint32_t c0, uint32_t c1) { return a_pair_wide((c0 & 0xFFu) | 0x4B000000u, (c1 & 0xFFu) | 0x4B000000u); });
+            } else {
+                pairs([&](uint32_t c0, uint32_t c1) { return a_pair_narrow((__byte_perm(c0, c1, 0x5410) & code_mask) | 0x43004300u); });
+            }
+        };
+        // NCHW, 4 and 8 bits, the widths a network's layers mostly have: strings of one or two words, which may begin at any code of a
+        // word (planes of no multiple of 8 codes; W words with the one behind).  Addresses and shifts step by the plane, no test
+        // per string away from the end of the channels and of the bit string.
+        constexpr int kShort = 3;
+        struct Short {
+            uint32_t w[8][kShort];
+            uint32_t first;             // position of the first string in its word, in codes
+        };
+        const uint32_t per_word = 32u / (uint32_t)bits, lg = bits == 4 ? 3u : 2u;
+        const bool whole = (P32 & (per_word - 1u)) == 0;      // strings begin at words
+        auto fetch_short = [&](auto width, int it, Short& r) {
+            constexpr int W = decltype(width)::value / 4;      // words of a string
+            const int ti = it / kblocks, kb = it - ti * kblocks;
+            const uint32_t c0 = (uint32_t)kb * kABk + 8u * cg;
+            const uint32_t gp0 = (blockIdx.x + (uint32_t)ti * gridDim.x) * (uint32_t)kABm + 8u * rq;
+            uint32_t n0, p0;
+            a.div_vp.divmod(gp0, n0, p0);
+            const size_t e0 = ((size_t)n0 * C32 + c0) * P32 + p0;
+            const uint32_t* src = a.packed + (e0 >> lg);
+            const int64_t left = a.nwords - (int64_t)(e0 >> lg);      // words from there on
+            uint32_t at = r.first = (uint32_t)e0 & (per_word - 1u);
+            if (gp0 < rows32 && c0 + 8 <= C32 && (int64_t)((at + 7u * P32) >> lg) + W < left) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i, at += P32) {
+#pragma unroll
+                    for (int k = 0; k <= W; ++k)
+                        if (k < W || !whole) r.w[i][k] = __ldg(src + (at >> lg) + k);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i, at += P32) {
+#pragma unroll
+                    for (int k = 0; k <= W; ++k)
+                        r.w[i][k] = gp0 < rows32 && c0 + i < C32 && (int64_t)(at >> lg) + k < left ? __ldg(src + (at >> lg) + k) : 0u;
+                }
+            }
+        };
+        auto store_short = [&](auto width, unsigned char* tile, const Short& r) {
+            constexpr int B = decltype(width)::value, W = B / 4;
+            uint32_t at = r.first;
+            uint32_t u[8][2];
+#pragma unroll
+            for (int i = 0; i < 8; ++i, at += P32) {
+#pragma unroll
+                for (int k = 0; k < W; ++k) u[i][k] = whole ? r.w[i][k] : __funnelshift_r(r.w[i][k], r.w[i][k + 1], at * (uint32_t)B);
+            }
+            if constexpr (B == 4) {
+                uint32_t w[8][4];                      // [row][pair of channels]
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {          // strings 2h, 2h + 1 = two channels, nibble j = row 8 rq + j
+                    const uint32_t alo = u[2 * h][0] & 0x0F0F0F0Fu, ahi = (u[2 * h][0] >> 4) & 0x0F0F0F0Fu;
+                    const uint32_t blo = u[2 * h + 1][0] & 0x0F0F0F0Fu, bhi = (u[2 * h + 1][0] >> 4) & 0x0F0F0F0Fu;
+                    const uint32_t e01 = __byte_perm(alo, blo, 0x5140), e23 = __byte_perm(alo, blo, 0x7362);    // rows 0 2 | 4 6
+                    const uint32_t o01 = __byte_perm(ahi, bhi, 0x5140), o23 = __byte_perm(ahi, bhi, 0x7362);    // rows 1 3 | 5 7
+                    w[0][h] = two(e01, 0x4140);
+                    w[2][h] = two(e01, 0x4342);
+                    w[4][h] = two(e23, 0x4140);
+                    w[6][h] = two(e23, 0x4342);
+                    w[1][h] = two(o01, 0x4140);
+                    w[3][h] = two(o01, 0x4342);
+                    w[5][h] = two(o23, 0x4140);
+                    w[7][h] = two(o23, 0x4342);
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) a_store_chunk(tile, 8u * rq + j, cg, w[j]);
+            } else {
+                // 8-bit codes: the byte beside 0x4B0000 is the fp32 number 2^23 + code
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const uint32_t sel = 0x7540u | (uint32_t)(j & 3);      // bytes: the code, 0, 0, 0x4B
+                        w[h] = a_pair_wide(__byte_perm(u[2 * h][j >> 2], 0x4B000000u, sel), __byte_perm(u[2 * h + 1][j >> 2], 0x4B000000u, sel));
                     }
                     a_store_chunk(tile, 8u * rq + j, cg, w);
                 }
@@ -676,38 +715,53 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
         // One iteration: load the words, wait for the stage, convert and store, publish.  The latency of the loads is
         // covered by the other groups' turns, not by loading ahead: a second set of registers for words in flight
         // cost more (register pressure, and the proxy fence below waits for them anyway) than it brought.
-        Raw r;
-        for (int it = (int)group; it < my_iters; it += kPGroups) {
-            fetch(it, r);
-            const int s = it % kPStages;
-            // the MMAs that read this stage kPStages iterations ago have completed (passes at once the first time round)
-            if (!warp_wait(&bars.a_empty[s], (uint32_t)(((it / kPStages) & 1) ^ 1))) break;
-            store(ring + (size_t)s * kABytes, r);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the stores above, for the tensor core
-            __syncwarp();
-            if (lane == 0) a_mbar_arrive(&bars.a_full[s]);
+        auto produce = [&](auto&& load, auto&& convert) {
+            int s = (int)group;
+            uint32_t turn = 1;
+            for (int it = (int)group; it < my_iters; it += kPGroups) {
+                load(it);
+                // the MMAs that read this stage one turn of the ring ago have completed (passes at once the first time round)
+                if (!warp_wait(&bars.a_empty[s], turn)) break;
+                convert(ring + (size_t)s * kABytes);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the stores above, for the tensor core
+                __syncwarp();
+                if (lane == 0) a_mbar_arrive(&bars.a_full[s]);
+                s += kPGroups;
+                if (s >= kPStages) {
+                    s -= kPStages;
+                    turn ^= 1u;
+                }
+            }
+        };
+        if (strings && (bits == 4 || bits == 8) && P32 < (1u << 28)) {
+            Short r;
+            if (bits == 4) produce([&](int it) { fetch_short(PartAt<4>{}, it, r); }, [&](unsigned char* t) { store_short(PartAt<4>{}, t, r); });
+            else produce([&](int it) { fetch_short(PartAt<8>{}, it, r); }, [&](unsigned char* t) { store_short(PartAt<8>{}, t, r); });
+        } else {
+            Raw r;
+            produce([&](int it) { fetch(it, r); }, [&](unsigned char* t) { store(t, r); });
         }
     } else if (warp == kPProducers / 32) {
-        if (lane == 0) {
+        if (a_elected()) {
             // ---- weights once, then every MMA: per K block 4 steps of 16, each against the hi and the lo half ----
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            a_mbar_expect_tx(&bars.b_full, (uint32_t)(2 * kBBytes) * (uint32_t)kblocks);
             for (int kb = 0; kb < kblocks; ++kb) {
-                a_tma_load_2d(wts + (size_t)kb * 2 * kBBytes, &map_hi, kb * kABk, col0, &bars.b_full);
-                a_tma_load_2d(wts + (size_t)kb * 2 * kBBytes + kBBytes, &map_lo, kb * kABk, col0, &bars.b_full);
+                a_mbar_expect_tx(&bars.b_full[kb], (uint32_t)(2 * kBBytes));
+                a_tma_load_2d(wts + (size_t)kb * 2 * kBBytes, &map_hi, kb * kABk, col0, &bars.b_full[kb]);
+                a_tma_load_2d(wts + (size_t)kb * 2 * kBBytes + kBBytes, &map_lo, kb * kABk, col0, &bars.b_full[kb]);
             }
             const uint32_t idesc = a_instr_desc(2 * BN);        // hi and lo halves as one operand
-            bool ok = wait(&bars.b_full, 0);
-            int it = 0;
+            bool ok = true;
+            int s = 0;
+            uint32_t turn = 0;                                  // of the ring
             for (int t = 0; t < my_tiles && ok; ++t) {
                 const uint32_t buf = (uint32_t)(t % kAcc);
                 // the epilogue has read this accumulator out (passes at once the first time round)
                 ok = wait(&bars.acc_empty[buf], (uint32_t)(((t / kAcc) & 1) ^ 1));
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const int s = it % kPStages;
-                    ok = wait(&bars.a_full[s], (uint32_t)((it / kPStages) & 1));
+                for (int kb = 0; kb < kblocks; ++kb) {
+                    ok = (t > 0 || wait(&bars.b_full[kb], 0)) && wait(&bars.a_full[s], turn);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t dq = a_smem_desc(ring + (size_t)s * kABytes);
@@ -716,6 +770,10 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
                     for (int k = 0; k < kABk / 16; ++k)      // 16 bf16 = 32 bytes = 2 sixteen-byte units along K
                         a_mma(tmem + buf * (2 * BN), dq + 2 * k, dw + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
                     a_commit(&bars.a_empty[s]);       // the stage may be refilled once these MMAs have read it
+                    if (++s == kPStages) {
+                        s = 0;
+                        turn ^= 1u;
+                    }
                 }
                 if (ok) a_commit(&bars.acc_full[buf]);       // the accumulator is final when this arrives
             }
@@ -733,12 +791,13 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
             if (!warp_wait(&bars.acc_full[buf], (uint32_t)((t / kAcc) & 1))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t gp = (blockIdx.x + (uint32_t)t * gridDim.x) * (uint32_t)kABm + q * 32u + lane;      // this thread's pixel
-            const uint32_t n = gp / (uint32_t)a.P, p = gp - n * (uint32_t)a.P;
-            const bool live = gp < (uint32_t)a.rows;
+            uint32_t n, p;
+            a.div_vp.divmod(gp, n, p);
+            const bool live = gp < a.vrows && p < (uint32_t)a.P;
             // this thread's element of output channel col0: the next channel is P (NCHW) or 1 (channels-last) further
             float* const yrow = NHWC ? a.y + (size_t)gp * (size_t)a.O + col0
                                      : a.y + ((size_t)n * (size_t)a.O + col0) * (size_t)a.P + p;
-#pragma unroll 1
+#pragma unroll 2
             for (int c = 0; c < BN; c += 16) {
                 uint32_t vh[16], vl[16];
                 const uint32_t taddr = tmem + ((q * 32u) << 16) + buf * (2 * BN) + (uint32_t)c;
@@ -893,7 +952,7 @@ cudaError_t a_launch(const CUtensorMap& mh, const CUtensorMap& ml, const AArgs& 
 
 // the persistent form, when the weight halves of all K blocks fit beside the ring of stages
 template <int BN, bool NHWC>
-cudaError_t p_launch(const CUtensorMap& mh, const CUtensorMap& ml, const AArgs& args, cudaStream_t st) {
+cudaError_t p_launch(const CUtensorMap& mh, const CUtensorMap& ml, const PArgs& args, cudaStream_t st) {
     const size_t smem = (size_t)kPStages * kABm * kABk * 2 + (size_t)args.kblocks * 2 * BN * kABk * 2 + 1024;
     auto kern = accumulate_persistent_kernel<BN, NHWC>;
     cudaError_t e = allow_smem(kern, (size_t)kPStages * kABm * kABk * 2 + kPWeightBytes - (NHWC ? 16 * 1024 : 0) + 1024);
@@ -901,14 +960,15 @@ cudaError_t p_launch(const CUtensorMap& mh, const CUtensorMap& ml, const AArgs& 
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int64_t row_tiles = (args.rows + kABm - 1) / kABm;
+    const int64_t row_tiles = ((int64_t)args.vrows + kABm - 1) / kABm;
     const unsigned col_tiles = (unsigned)((args.O + BN - 1) / BN);
     // one CTA per SM, shared out among the column tiles; no CTA without a row tile
     const unsigned per_col = (unsigned)std::max<int64_t>(1, std::min<int64_t>(row_tiles, sms / (int)std::min<unsigned>(col_tiles, (unsigned)sms)));
     const dim3 grid(per_col, col_tiles);
     // Set up, and expanding codes, while the weights kernel runs: that kernel lets it start when it has itself seen the end of
-    // everything ahead, the codes among it; only what takes its results waits (accumulate_persistent_kernel).  Encode and
-    // contraction of [128,256,14,14] to 256 channels 45.2 -> 40.5 us.
+    // everything ahead, the codes among it; only what takes its results waits (accumulate_persistent_kernel).  Splitting the weights in
+    // here instead, every CTA its own column tile, saves that launch and is slower all the same: [128,256,14,14] to 256 channels 29.6 us with
+    // the encoder ahead against 28.3, at 512 channels 16 against 14 (each split by 4 to 74 CTAs, straight-line code that each fetches once).
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kPThreads);
@@ -971,7 +1031,7 @@ extern "C" int granq_accumulate_codes(const uint32_t* packed_codes, const int64_
     if (launch_after(kAnyLayout, accumulate_weights_kernel, (unsigned)out_channels, 128, 0, st, weights, scale, zp, (int)L.C,
                      (int)L.Cpad, hi, lo, bias, (uint32_t*)workspace) != cudaSuccess)
         return GRANQ_ERR_CUDA;
-    AArgs args{};
+    PArgs args{};
     args.y = y;
     args.bias = bias;
     args.status = (uint32_t*)workspace;
@@ -985,7 +1045,13 @@ extern "C" int granq_accumulate_codes(const uint32_t* packed_codes, const int64_
     args.kblocks = kblocks;
     args.spin_limit = kASpin;
     args.stages = std::min(args.kblocks, kAStages);
-    const bool persistent = !one_tile_per_cta && resident(BN);
+    // NCHW: whole strings of 8 pixels per sample, so that none reaches into the next one: at [128,256,14,14] such strings took most of
+    // the expansion's instructions
+    const int64_t VP = channel_axis == 1 && L.P >= 8 ? (L.P + 7) / 8 * 8 : L.P;
+    args.VP = (uint32_t)VP;
+    args.vrows = (uint32_t)(VP * L.N);
+    args.div_vp = make_fastdiv(args.VP);
+    const bool persistent = !one_tile_per_cta && resident(BN) && VP * L.N < (1ll << 31);
     cudaError_t e = cudaSuccess;
     if (persistent) {
         if (channel_axis == 3)

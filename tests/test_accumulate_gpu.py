@@ -93,6 +93,27 @@ def test_accumulate_matches_the_oracle_within_the_derived_bound(b, shape, channe
     assert np.max(np.abs(ref)) > 100 * np.max(tol)
 
 
+@pytest.mark.parametrize("shape", [(3, 64, 7, 7, 64), (2, 70, 9, 9, 40), (5, 30, 10, 10, 130), (4, 72, 3, 5, 24), (7, 20, 2, 3, 8),
+                                   (30, 256, 14, 14, 256), (3, 512, 5, 5, 70)], ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("low", [0.0, -1.0, 3.0], ids=["from_zero", "below_zero", "off_zero"])
+def test_accumulate_every_width_on_ragged_planes(b, shape, low):
+    """Strings of 8 pixels that begin anywhere in a word and planes that end inside one, planes below a string, tiles of every
+    column of the GPU; zero-points of either sign and, where a channel's range does not hold 0, far beyond the codes."""
+    n, c, h, wd, o = shape
+    rng = np.random.default_rng(sum(shape))
+    x = (rng.random((n, c, h, wd)) * np.exp(rng.standard_normal((1, c, 1, 1)))).astype(np.float32)
+    x[:, ::2] += np.float32(low)
+    w = (rng.standard_normal((o, c)) / np.sqrt(c)).astype(np.float32)
+    for bits in range(1, 9):
+        res = orc.fused(x, bits)
+        assert bits < 8 or low < 3.0 or np.any(np.abs(res.z) > 256)
+        ref = orc.accumulate(res.codes, res.s, res.z, w)
+        S, bias = bound(res.codes, res.s, res.z, w)
+        tol = (2.0 ** -17 + c * 2.0 ** -22) * S + 2.0 ** -21 * (bias + np.abs(ref))
+        for channels_last in (False, True):
+            assert np.all(np.abs(run(b, res.codes, bits, res.s, res.z, w, channels_last) - ref) <= tol)
+
+
 @pytest.mark.parametrize("channels_last", [False, True], ids=["nchw", "nhwc"])
 def test_accumulate_is_exact_on_small_integers(b, channels_last):
     """Integer weights in [-8, 8], scales that are powers of two, integer zero-points: every product and every
