@@ -14,6 +14,11 @@ from typing import Optional
 
 import torch
 
+try:
+    from . import _host as _host_calls          # granq_host.cpp: the plain case of the calls below in native code, see lib()
+except ImportError:              # not built: the same calls, marshalled here
+    _host_calls = None
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libgranq.so")
 
@@ -54,6 +59,7 @@ class GranqError(RuntimeError):
 
 
 _lib = None
+_native = None                   # that module once it knows the library's entry points
 
 
 class WeightDesc(ctypes.Structure):
@@ -75,7 +81,7 @@ class FusedDesc(ctypes.Structure):
 
 def lib() -> ctypes.CDLL:
     """The loaded shared library; raises if it has not been built."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -164,7 +170,16 @@ def lib() -> ctypes.CDLL:
         L.granq_fakequant_fused_fwd_packmask.argtypes = [vp, ci, i64p, ci, ci, ci, vp, vp, vp, vp, vp, vp, vp, sz,
                                                          u32, vp]
         _lib = L
+        if _host_calls is not None:
+            _host_calls.setup({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in EXPORTS}, FakeQuantOut, GranqError)
+            _native = _host_calls
     return _lib
+
+
+def _goes_native(stream) -> bool:
+    """The current stream, and outputs from the plain allocator.  The native calls answer None, having done nothing, where a tensor or
+    an argument is not of the plain kind; the call is then marshalled here, which also says what is wrong with it."""
+    return _native is not None and stream is None and _new is _plain_new
 
 
 def status_string(status: int) -> str:
@@ -374,6 +389,10 @@ class FakeQuantOut:
 def granq_range(x: torch.Tensor, channel_axis: int = 1, group: int = GROUP_CHANNEL, lo: torch.Tensor = None,
                 hi: torch.Tensor = None, workspace: torch.Tensor = None, flags: int = 0, stream=None):
     """Per-group (lo, hi) of x: Eq. 4."""
+    if _goes_native(stream):
+        r = _native.range_call(x, channel_axis, group, lo, hi, workspace, flags)
+        if r is not None:
+            return r
     G = num_groups(x.shape, channel_axis, group)
     lo = _new(G, torch.float32, x.device) if lo is None else lo
     hi = _new(G, torch.float32, x.device) if hi is None else hi
@@ -437,6 +456,10 @@ def granq_fakequant_fused(x: torch.Tensor, bits: int, gy: torch.Tensor = None, c
     `out` may carry preallocated tensors (y, gx, lo, hi, s, z, codes, mask, workspace);
     whatever is missing is allocated here.
     """
+    if not (want_codes or want_mask) and _goes_native(stream):
+        r = _native.fused_call(0, x, bits, gy, channel_axis, group, out, int(want_params), flags)
+        if r is not None:
+            return r
     if gy is not None and (gy.shape != x.shape or gy.dtype != x.dtype):
         raise ValueError("gy must match x")
     G = num_groups(x.shape, channel_axis, group)
@@ -486,6 +509,10 @@ def granq_fakequant_fwd_packmask(x: torch.Tensor, bits: int, lo: torch.Tensor, h
                                  packed_mask: torch.Tensor = None, want_params: bool = False, flags: int = 0,
                                  stream=None) -> FakeQuantOut:
     """Forward with a given range that also stores the STE mask at one bit per element (Section 2.1)."""
+    if _goes_native(stream):
+        r = _native.fwd_packmask_call(x, bits, lo, hi, channel_axis, group, y, packed_mask, int(want_params), flags)
+        if r is not None:
+            return r
     G = num_groups(x.shape, channel_axis, group)
     o = FakeQuantOut(lo=lo, hi=hi)
     o.y = _new_like(x) if y is None else y
@@ -503,6 +530,10 @@ def granq_fakequant_fwd_packmask(x: torch.Tensor, bits: int, lo: torch.Tensor, h
 def granq_fakequant_bwd_packmask(gy: torch.Tensor, packed_mask: torch.Tensor, gx: torch.Tensor = None,
                                  flags: int = 0, stream=None) -> torch.Tensor:
     """STE backward from the packed mask alone: gx = gy where the bit is set, else 0."""
+    if _goes_native(stream):
+        r = _native.bwd_packmask_call(gy, packed_mask, gx, flags)
+        if r is not None:
+            return r
     if packed_mask.numel() * packed_mask.element_size() < packmask_bytes(gy.shape):
         raise ValueError("packed mask too small for gy")
     gx = _new_like(gy) if gx is None else gx
@@ -566,6 +597,10 @@ def granq_fakequant_fused_fwd_packmask(x: torch.Tensor, bits: int, channel_axis:
                                        group: int = GROUP_CHANNEL, out: FakeQuantOut = None,
                                        want_params: bool = False, flags: int = 0, stream=None) -> FakeQuantOut:
     """Range of x itself -> scale / zero-point -> y and the packed STE mask, in one call."""
+    if _goes_native(stream):
+        r = _native.fused_call(1, x, bits, None, channel_axis, group, out, int(want_params), flags)
+        if r is not None:
+            return r
     G = num_groups(x.shape, channel_axis, group)
     o = out if out is not None else FakeQuantOut()
     dev = x.device
@@ -612,6 +647,10 @@ def granq_fakequant_fused_stats(x: torch.Tensor, bits: int, channel_axis: int = 
                                 out: FakeQuantOut = None, want_params: bool = False, flags: int = 0,
                                 stream=None) -> FakeQuantOut:
     """Range of x itself -> scale / zero-point -> y, gathering Table 2's sums in the same pass."""
+    if _goes_native(stream):
+        r = _native.fused_call(2, x, bits, None, channel_axis, group, out, int(want_params), flags)
+        if r is not None:
+            return r
     G = num_groups(x.shape, channel_axis, group)
     o = out if out is not None else FakeQuantOut()
     dev = x.device
@@ -716,6 +755,10 @@ def granq_dequantize_packed(packed_codes: torch.Tensor, shape, dtype: torch.dtyp
                             z: torch.Tensor, channel_axis: int = 1, group: int = GROUP_CHANNEL,
                             y: torch.Tensor = None, stream=None) -> torch.Tensor:
     """Eq. 6 from the packed codes: y = s * (code - z)."""
+    if _goes_native(stream):
+        r = _native.dequantize_call(packed_codes, shape, dtype, bits, s, z, channel_axis, group, y)
+        if r is not None:
+            return r
     y = _new(tuple(shape), dtype, packed_codes.device) if y is None else y
     _check(lib().granq_dequantize_packed(_dev(packed_codes, "packed_codes"), _dtype(y), _dims(shape), channel_axis,
                                          group, bits, _dev(s, "s"), _dev(z, "z"), _dev(y, "y"), 0, _stream(stream)),
@@ -732,6 +775,10 @@ def granq_quantize_packed_fused(x: torch.Tensor, bits: int, channel_axis: int = 
                                 stream=None) -> FakeQuantOut:
     """Range of x itself -> scale / zero-point -> integer codes as a bit string, in one call (lo, hi, s, z and
     packed_codes of the returned record are filled)."""
+    if packed_codes is None and _goes_native(stream):
+        r = _native.fused_call(3, x, bits, None, channel_axis, group, out, 0, flags)
+        if r is not None:
+            return r
     G = num_groups(x.shape, channel_axis, group)
     o = out if out is not None else FakeQuantOut()
     dev = x.device
@@ -758,6 +805,10 @@ def granq_accumulate_codes(packed_codes: torch.Tensor, shape, bits: int, s: torc
     tensor of `shape` (NCHW for channel_axis 1, N H W C for 3): y = sum_c w[o, c] * s_c * (code - z_c), fp32.
     Returns (y, workspace); the workspace's status word tells whether a bounded wait ran out.
     flags: FLAG_FORCE_TWO_PASS takes the kernel with one tile per CTA instead of the persistent one."""
+    if _goes_native(stream):
+        r = _native.accumulate_call(packed_codes, shape, bits, s, z, weights, channel_axis, y, workspace, flags)
+        if r is not None:
+            return r
     shape = tuple(int(d) for d in shape)
     if weights.dtype != torch.float32 or weights.dim() != 2 or weights.shape[1] != shape[channel_axis]:
         raise ValueError("weights must be float32 [out_channels, C]")

@@ -1,15 +1,20 @@
-"""In-tree build of the GranQ CUDA library for sm_100a (nvcc cross-compiles without a GPU)."""
+"""In-tree build of the GranQ CUDA library for sm_100a (nvcc cross-compiles without a GPU) and of the binding's native calls."""
 from __future__ import annotations
 
+import importlib.util
 import os
+import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libgranq.so")
+HOST = os.path.join(HERE, "_host.so")               # the binding's calls in native code, an extension module of this package
+HOST_SOURCE = os.path.join(CSRC, "granq_host.cpp")
 OBJ_DIR = os.path.join(HERE, "_build")
 SOURCES = ["granq_api.cu", "granq_flat.cu", "granq_staged.cu", "granq_l2wave.cu", "granq_colwalk.cu", "granq_colteam.cu",
            "granq_cluster.cu", "granq_hold.cu", "granq_accumulate.cu", "granq_rows.cu", "granq_weights.cu", "granq_selftest.cu", "granq_noalloc.cu"]
@@ -33,11 +38,39 @@ def _stale() -> bool:
     return any(_newer(d, t) for d in [os.path.join(CSRC, f) for f in SOURCES] + _deps())
 
 
+def _host_stale() -> bool:
+    return not os.path.exists(HOST) or any(_newer(d, os.path.getmtime(HOST)) for d in (HOST_SOURCE, os.path.join(INCLUDE, "granq.h")))
+
+
+def _build_host() -> None:
+    torch = os.path.dirname(importlib.util.find_spec("torch").origin)
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_which_nvcc()))), "include")
+    tmp = HOST + f".tmp{os.getpid()}"
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", HOST_SOURCE, "-o", tmp,
+                           f"-I{torch}/include", f"-I{torch}/include/torch/csrc/api/include", f"-I{cuda}",
+                           f"-I{sysconfig.get_paths()['include']}", f"-L{torch}/lib", "-ltorch", "-ltorch_cpu", "-ltorch_python",
+                           "-lc10", "-lc10_cuda"])
+    os.replace(tmp, HOST)
+
+
+def _which_nvcc() -> str:
+    nvcc = os.environ.get("NVCC", "nvcc")
+    return shutil.which(nvcc) or nvcc
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile csrc/*.cu (one object per source, in parallel) and link libgranq.so beside this file;
-    returns its path.  Objects are kept in _build/ and reused while their source and the headers are older."""
-    if not (force or _stale()):
-        return LIB
+    """Compile csrc/*.cu (one object per source, in parallel) and link libgranq.so beside this file, and _host.so with
+    it; returns the library's path.  Objects are kept in _build/ and reused while their source and the headers are older."""
+    with ThreadPoolExecutor(max_workers=1) as beside:
+        host = beside.submit(_build_host) if force or _host_stale() else None
+        if force or _stale():
+            _build_lib(force, verbose)
+        if host is not None:
+            host.result()
+    return LIB
+
+
+def _build_lib(force: bool, verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "nvcc")
     os.makedirs(OBJ_DIR, exist_ok=True)
 
@@ -60,7 +93,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.check_call([nvcc, "-shared", "-cudart", "static", "-gencode", "arch=compute_100a,code=sm_100a",
                            "-o", tmp] + objs)
     os.replace(tmp, LIB)
-    return LIB
 
 
 if __name__ == "__main__":

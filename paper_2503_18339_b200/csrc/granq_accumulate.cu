@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 
 namespace granq {
 
@@ -902,6 +903,21 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// The tile-load descriptors are made by the driver: its encoder, looked up once (no link-time dependency on the driver).
+EncodeTiledFn a_encoder() {
+    static std::atomic<EncodeTiledFn> known{nullptr};
+    EncodeTiledFn fn = known.load(std::memory_order_relaxed);
+    if (fn) return fn;
+    void* found = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &found, cudaEnableDefault, &qres) != cudaSuccess ||
+        qres != cudaDriverEntryPointSuccess)
+        return nullptr;
+    fn = (EncodeTiledFn)found;
+    known.store(fn, std::memory_order_relaxed);
+    return fn;
+}
+
 // bf16 matrix [rows, cols] (cols contiguous) cut into boxes of 64 columns x box_rows rows, 128-byte swizzle;
 // columns and rows beyond the matrix read as zero
 bool a_make_map(EncodeTiledFn encode, CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols,
@@ -1004,13 +1020,8 @@ extern "C" int granq_accumulate_codes(const uint32_t* packed_codes, const int64_
         return GRANQ_ERR_INVALID_ARG;
     if (!workspace || ((uintptr_t)workspace & 255) || workspace_bytes < L.total) return GRANQ_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // the tile-load descriptors are made by the driver: look its encoder up (no link-time dependency on the driver)
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess || !fn ||
-        qres != cudaDriverEntryPointSuccess)
-        return GRANQ_ERR_CUDA;
-    EncodeTiledFn encode = (EncodeTiledFn)fn;
+    const EncodeTiledFn encode = a_encoder();
+    if (!encode) return GRANQ_ERR_CUDA;
     char* ws = (char*)workspace;
     __nv_bfloat16* hi = (__nv_bfloat16*)(ws + L.off_hi);
     __nv_bfloat16* lo = (__nv_bfloat16*)(ws + L.off_lo);
