@@ -655,6 +655,115 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
     }
 }
 
+// ---- Eq. 1, clamp, Eq. 6 with a given range, column path -------------------------------------------
+// As range_cols_kernel: a thread keeps one unit column of the slabs and with it the parameters of its channel, or of the two that its
+// unit straddles, in registers, and walks a few slabs; y and, PMASK, the packed mask.  In the tile kernel above every pack of a short
+// or ragged plane costs a division, two table rows and a choice of parameters per element: 180 instructions a unit at [128,960,7,7] with a
+// mask, here about 50.  Tiles / columns, us, without and with a mask: fp32 [128,960,7,7] 9.6 / 7.7, 11.8 / 8.5; [128,256,14,14] 9.5 / 6.3,
+// 11.8 / 6.6; [32,64,56,56] 8.7 / 5.7, 11.1 / 6.0; [256,512,28,28], 392 MB, 122 / 122, 136 / 127; bf16 [128,96,33,33] 17.3 / 14.1, 21.0 / 16.5,
+// [256,1024,14,14] 62.6 / 49.4, 74.6 / 53.4.  Bound by the instructions of 16 bytes up to a few times the L2, then by HBM.  Eight of bf16 that
+// straddle planes keep two units in flight and four blocks per SM (four and three: small tensors 4 to 15 % slower).
+template <typename T, bool ALIGNED, bool PMASK>
+__global__ void __launch_bounds__(kThreads, 4) quant_cols_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, uint8_t* __restrict__ pmask,
+                                                                 uint32_t slab_units, uint32_t outer, uint32_t slabs, FastDiv div_ncol,
+                                                                 FastDiv div_plane, float qmax, const float* __restrict__ lo,
+                                                                 const float* __restrict__ hi) {
+    after_the_kernel_ahead();
+    constexpr int V = Pack<T>::V, U = V == 8 && !ALIGNED ? 2 : 4, EXTRAS = PMASK ? 2 : 0;
+    uint32_t chunk, col;
+    div_ncol.divmod(blockIdx.x, chunk, col);
+    const uint32_t n0 = chunk * slabs, n1 = min(outer, n0 + slabs), lane = threadIdx.x & 31;
+    const uint32_t u = col * kThreads + threadIdx.x;
+    const bool valid = u < slab_units;                        // lanes beyond the last column walk along, for the shuffles
+    const uint4* p = x + ((size_t)n0 * slab_units + u);
+    Pack<T> px[U];
+    auto fetch = [&](uint32_t n) {
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+            if (valid && n + j < n1) px[j].raw = ld_stream_16(p + (size_t)j * slab_units);
+    };
+    fetch(n0);                                                // under way while the parameters are made
+    uint32_t ch;
+    int ne = V;
+    if constexpr (ALIGNED) {
+        ch = div_plane.div(valid ? u : 0u);
+    } else {
+        uint32_t rem;
+        div_plane.divmod((valid ? u : 0u) * V, ch, rem);
+        ne = (int)min((uint32_t)V, div_plane.d - rem);
+    }
+    auto params = [&](uint32_t c) {
+        const QParam q = make_qparam(__fadd_rn(lo[c], 0.0f), __fadd_rn(hi[c], 0.0f), qmax);
+        const float r = div_is_safe(q.s, 0.0f, 0.0f) ? __frcp_rn(q.s) : 0.0f;
+        return GroupParam{q.s, q.z, r, tie_threshold(r, q.z, qmax)};
+    };
+    const GroupParam g1 = params(ch);
+    GroupParam g2 = g1;
+    if constexpr (!ALIGNED) {
+        if (ne < V) g2 = params(ch + 1);
+    }
+    // fp32: two elements to an instruction where nothing of a pack is clamped or close to a tie
+    const float thr = fminf(g1.thr, g2.thr), top = __fadd_rn(kRoundMagic, qmax);
+    const float mza = __fadd_rn(kRoundMagic, g1.z), mzb = __fadd_rn(kRoundMagic, g2.z);
+    F2 r2[2], mz2[2], ns2[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const bool a = ALIGNED || 2 * k < ne, b = ALIGNED || 2 * k + 1 < ne;
+        r2[k] = f2(a ? g1.r : g2.r, b ? g1.r : g2.r);
+        mz2[k] = f2(a ? mza : mzb, b ? mza : mzb);
+        ns2[k] = f2(a ? -g1.s : -g2.s, b ? -g1.s : -g2.s);
+    }
+    auto quantize = [&](const Pack<T>& q, Pack<T>& py, uint32_t& bits) {
+        uint32_t cb[V / 4], mb[V / 4];
+        if constexpr (V == 4) {
+            float m[4], yv[4], worst = 0.0f;
+            const F2 zero = {0};
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const F2 v = f2(q.get(2 * k), q.get(2 * k + 1)), w = f2_fma(v, r2[k], mz2[k]), e = f2_sub(mz2[k], w);
+                float d0, d1;
+                f2_split(f2_fma(v, r2[k], e), d0, d1);
+                worst = max_or_nan(max_or_nan(worst, fabsf(d0)), fabsf(d1));
+                f2_split(f2_fma(ns2[k], e, zero), yv[2 * k], yv[2 * k + 1]);
+                f2_split(w, m[2 * k], m[2 * k + 1]);
+            }
+            const float least = fminf(fminf(m[0], m[1]), fminf(m[2], m[3])), most = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+            if (worst < thr && least >= kRoundMagic && most <= top) {
+                py.set_all(yv);
+                bits = 15;
+                return;
+            }
+        }
+        quantize_pack<T, false, !ALIGNED, EXTRAS, false, true>(q, q, g1, g2, ne, qmax, py, py, cb, mb, 8);
+        if constexpr (PMASK) bits = mb[0];
+    };
+    uint4* out = y + ((size_t)n0 * slab_units + u);
+    uint32_t at = n0 * slab_units + u;                        // of the units of the tensor
+    for (uint32_t n = n0; n < n1; n += U) {
+        if (n > n0) fetch(n);
+        uint32_t bits[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            bits[j] = 0;
+            if (valid && n + j < n1) {
+                Pack<T> py;
+                quantize(px[j], py, bits[j]);
+                st_stream_16(out + (size_t)j * slab_units, py.raw);
+                if constexpr (PMASK && V == 8) pmask[at + j * slab_units] = (uint8_t)bits[j];
+            }
+        }
+        if constexpr (PMASK && V == 4) {
+            const uint32_t bytes = pair_up_mask<U>(bits, lane);
+#pragma unroll
+            for (int j = 0; j < U; j += 2)
+                if (valid && n + j + (lane & 1u) < n1) pmask[(at + (j + (lane & 1u)) * slab_units) >> 1] = (uint8_t)(bytes >> (4 * j));
+        }
+        p += (size_t)U * slab_units;
+        out += (size_t)U * slab_units;
+        at += U * slab_units;
+    }
+}
+
 // ---- the "conventional" per-channel scheme (Section 5.3.2): one group per launch ------------------
 template <typename T, bool IS_MAX>
 __global__ void __launch_bounds__(kThreads) naive_extreme_kernel(const T* __restrict__ x, Geom g, int64_t c,
@@ -1002,6 +1111,24 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
                             io.pmask, io.dist, io.pcodes, io.code_bits, f, qmax, lo, hi);
     };
     if constexpr (MODE == MODE_FWD) {
+        // columns: slabs of whole units (with a mask whole bytes of it, and whole words in all), at least a batch of them: faster for
+        // all planes, see the kernel.  A few slabs to a block, so that blocks start in the order of memory; as many as leave a
+        // small tensor one wave of blocks.
+        const bool plain = !io.codes && !io.mask && !io.dist && !io.pcodes && io.y;
+        if (plain && (vec || ragged) && g.E < (1ll << 31) && g.C < (1ll << 30) && (g.C * g.inner) % VF == 0 && g.outer >= 8 &&
+            (!io.pmask || ((g.C * g.inner) % 8 == 0 && g.E % 32 == 0))) {
+            const uint32_t slab_units = (uint32_t)(g.C * g.inner / VF), ncol = (slab_units + kThreads - 1) / kThreads, outer = (uint32_t)g.outer;
+            const uint32_t slots = (uint32_t)sm_count() * 4;
+            const uint32_t slabs = std::min<uint32_t>(16, std::max<uint32_t>(4, (uint32_t)(((uint64_t)outer * ncol + slots - 1) / slots)));
+            auto cols = [&](auto kern, uint32_t plane) {
+                return launch_after(sm_layout(0, (uint64_t)g.E * sizeof(T)), kern, ncol * ((outer + slabs - 1) / slabs), kThreads, 0, st,
+                                    (const uint4*)io.x, (uint4*)io.y, (uint8_t*)io.pmask, slab_units, outer, slabs, make_fastdiv(ncol),
+                                    make_fastdiv(plane), qmax, lo, hi);
+            };
+            const uint32_t plane = (uint32_t)(vec ? g.inner / VF : g.inner);
+            if (io.pmask) return vec ? cols(quant_cols_kernel<T, true, true>, plane) : cols(quant_cols_kernel<T, false, true>, plane);
+            return vec ? cols(quant_cols_kernel<T, true, false>, plane) : cols(quant_cols_kernel<T, false, false>, plane);
+        }
         const bool dist_only = io.dist != nullptr && io.y != nullptr && io.codes == nullptr && io.mask == nullptr &&
                                io.pmask == nullptr && io.pcodes == nullptr;
         if ((vec || ragged) && pack_only && g.E % 32 == 0)         // whole words of codes: the byte-wise writer
