@@ -89,12 +89,12 @@ __device__ __forceinline__ void t_cp_async_wait_all() { asm volatile("cp.async.w
 // U = units a thread handles together in the quantize walk
 // BITS = bits of a code (EXTRAS = 3 only: shifts and lanes of the code string are then constants)
 // At = index of a unit of the tensor: 32 bits below 64 GB
-template <typename T, int MODE, int EXTRAS, int U, int BITS, typename At>
-__global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
+template <typename T, int MODE, int EXTRAS, int U, int BITS, typename At, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) colteam_kernel(const TArgs a) {
     constexpr int V = Pack<T>::V;
     constexpr bool kBwd = (MODE & MODE_BWD) != 0;
     extern __shared__ __align__(16) uint4 t_smem[];
-    __shared__ uint32_t s_kmn[kTWarps], s_kmx[kTWarps];
+    __shared__ uint32_t s_kmn[(NT / 32)], s_kmx[(NT / 32)];
     __shared__ GroupParam s_par;
     __shared__ uint32_t s_ok;
     const uint32_t tid = threadIdx.x, lane = tid & 31;
@@ -104,13 +104,13 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     const uint32_t q0 = 8 * (uint32_t)(((uint64_t)rank * runs) / a.R);
     const uint32_t q1 = min(a.units, 8 * (uint32_t)(((uint64_t)(rank + 1) * runs) / a.R));
     const uint32_t n = q1 - q0;
-    const uint32_t cnt = tid < n ? (n - tid + kTThreads - 1) / kTThreads : 0u;      // units of this thread
-    // where they are: unit q lies in slab q / plane_units, and the next one of this thread is kTThreads units on
+    const uint32_t cnt = tid < n ? (n - tid + NT - 1) / NT : 0u;      // units of this thread
+    // where they are: unit q lies in slab q / plane_units, and the next one of this thread is NT units on
     uint32_t slab0, off0;
     a.div_plane.divmod(q0 + min(tid, n), slab0, off0);
     const At first = (At)slab0 * a.slab_units + off0;
     uint32_t dslab, doff;
-    a.div_plane.divmod((uint32_t)kTThreads, dslab, doff);
+    a.div_plane.divmod((uint32_t)NT, dslab, doff);
     const At dstep = (At)dslab * a.slab_units + doff, dwrap = a.slab_units - a.plane_units;
     auto advance = [&](At& at, uint32_t& off) {
         at += dstep;
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     const uint32_t whole = kPairs ? __shfl_sync(kFullMask, cnt, 31) : cnt;
     uint4* tile = t_smem + tid;
     uint4* tileg = t_smem + a.tile_units + tid;
-    const uint32_t gcnt = kBwd ? (tid < a.gy_units ? min(cnt, (a.gy_units - tid + kTThreads - 1) / kTThreads) : 0u) : 0u;
+    const uint32_t gcnt = kBwd ? (tid < a.gy_units ? min(cnt, (a.gy_units - tid + NT - 1) / NT) : 0u) : 0u;
     const uint4* xg = reinterpret_cast<const uint4*>(a.x);
     const uint4* gyg = reinterpret_cast<const uint4*>(a.gy);
     uint4* yg = reinterpret_cast<uint4*>(a.y);
@@ -140,8 +140,8 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
         At at = first + (At)team * a.plane_units;
         uint32_t off = off0;
         for (uint32_t i = 0; i < cnt; ++i) {
-            cp_async_16(tile + i * kTThreads, xg + at);
-            if (kBwd && i < gcnt) cp_async_16(tileg + i * kTThreads, gyg + at);
+            cp_async_16(tile + i * NT, xg + at);
+            if (kBwd && i < gcnt) cp_async_16(tileg + i * NT, gyg + at);
             advance(at, off);
         }
     }
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
         RangeFold<T> fold;
         for (uint32_t i = 0; i < cnt; ++i) {
             Pack<T> p;
-            p.raw = tile[i * kTThreads];
+            p.raw = tile[i * NT];
             fold.add(p);
         }
         float m0, m1;
@@ -166,8 +166,8 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
         }
         __syncthreads();
         if (tid < 32) {
-            ka = __reduce_max_sync(kFullMask, lane < kTWarps ? s_kmn[lane] : 0u);
-            kb = __reduce_max_sync(kFullMask, lane < kTWarps ? s_kmx[lane] : 0u);
+            ka = __reduce_max_sync(kFullMask, lane < (NT / 32) ? s_kmn[lane] : 0u);
+            kb = __reduce_max_sync(kFullMask, lane < (NT / 32) ? s_kmx[lane] : 0u);
             if (lane == 0) {
                 atomicMax(a.kmin + c, ka);
                 atomicMax(a.kmax + c, kb);
@@ -224,17 +224,17 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
             for (int j = 0; j < N; ++j) {
                 w[j] = at;
                 if constexpr (kBwd) {
-                    if (i + j < gcnt) pg[j].raw = tileg[(i + j) * kTThreads];
+                    if (i + j < gcnt) pg[j].raw = tileg[(i + j) * NT];
                     else pg[j].raw = ld_stream_16(gyg + at);
                 }
-                px[j].raw = tile[(i + j) * kTThreads];
+                px[j].raw = tile[(i + j) * NT];
                 advance(at, off);
             }
             if (more) {
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
-                    cp_async_16(tile + (i + j) * kTThreads, xg + (w[j] + ahead));
-                    if (kBwd && i + j < gcnt) cp_async_16(tileg + (i + j) * kTThreads, gyg + (w[j] + ahead));
+                    cp_async_16(tile + (i + j) * NT, xg + (w[j] + ahead));
+                    if (kBwd && i + j < gcnt) cp_async_16(tileg + (i + j) * NT, gyg + (w[j] + ahead));
                 }
             }
             i += N;
@@ -270,13 +270,13 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
         auto alone = [&](uint32_t lanes) {
             Pack<T> px, pg;
             if constexpr (kBwd) {
-                if (i < gcnt) pg.raw = tileg[i * kTThreads];
+                if (i < gcnt) pg.raw = tileg[i * NT];
                 else pg.raw = ld_stream_16(gyg + at);
             }
-            px.raw = tile[i * kTThreads];
+            px.raw = tile[i * NT];
             if (more) {
-                cp_async_16(tile + i * kTThreads, xg + (at + ahead));
-                if (kBwd && i < gcnt) cp_async_16(tileg + i * kTThreads, gyg + (at + ahead));
+                cp_async_16(tile + i * NT, xg + (at + ahead));
+                if (kBwd && i < gcnt) cp_async_16(tileg + i * NT, gyg + (at + ahead));
             }
             uint32_t cb[V / 4], mb[V / 4];
             quantize(px, pg, at, cb, mb);
@@ -305,11 +305,11 @@ __global__ void __launch_bounds__(kTThreads, 2) colteam_kernel(const TArgs a) {
     }
     __syncthreads();
     if (s_ok) {
-        for (uint32_t i = tid; i < a.C; i += kTThreads) {
+        for (uint32_t i = tid; i < a.C; i += NT) {
             a.kmin[i] = 0;
             a.kmax[i] = 0;
         }
-        for (uint32_t i = tid; i <= a.C; i += kTThreads) a.counters[i] = 0;
+        for (uint32_t i = tid; i <= a.C; i += NT) a.counters[i] = 0;
     }
 }
 
@@ -535,10 +535,13 @@ cudaError_t t_launch(const TArgs& args, const TeamPlan& p, const StagedTuning& t
         const cudaError_t e = allow_smem(kern, kTSmemUnits * 16);
         if (e != cudaSuccess) return e;
         void* params[] = {(void*)&args};
-        return launch_cooperative((const void*)kern, args.R * args.teams, kTThreads, params, p.smem_bytes, tune, st);
+        return launch_cooperative((const void*)kern, args.R * args.teams, p.threads, params, p.smem_bytes, tune, st);
     };
-    return (uint64_t)args.units * args.C < (1ull << 32) ? go(colteam_kernel<T, MODE, EXTRAS, U, BITS, uint32_t>)
-                                                        : go(colteam_kernel<T, MODE, EXTRAS, U, BITS, uint64_t>);
+    if constexpr (MODE == MODE_FWD) {
+        if (p.threads == kTThreads / 2) return go(colteam_kernel<T, MODE, EXTRAS, U, BITS, uint32_t, kTThreads / 2>);
+    }
+    return (uint64_t)args.units * args.C < (1ull << 32) ? go(colteam_kernel<T, MODE, EXTRAS, U, BITS, uint32_t, kTThreads>)
+                                                        : go(colteam_kernel<T, MODE, EXTRAS, U, BITS, uint64_t, kTThreads>);
 }
 
 template <typename T>
@@ -627,11 +630,49 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
         }
     }
     if (best == ~0ull) return p;
+    p.threads = kTThreads;
+    p.threads = kTThreads;
+    p.sm_count = (uint32_t)sm_count;
     p.gy_units = backward && !p.lag ? std::min(p.tile_units, kTSmemUnits - p.tile_units) : 0u;
     p.smem_bytes = 16u * ((p.lag ? 2 : 1) * p.tile_units + p.gy_units);
     p.ok = true;
     return p;
 }
+
+namespace {
+
+// Forward, four CTAs of half the threads and half the shared memory per SM: a finer cut, which is worth having where it saves a round
+// or more of several, and in bf16 also where it saves none (two / four, us: fp32 [87,240,56,56], 10 / 9 rounds, 111 / 102, with sums 109 / 103, codes
+// 123 / 120.5; [60,200,48,48], 5 / 4, 51.6 / 47.3; [49,608,56,56], 13 / 12, 141 / 137; bf16 [128,96,112,112], 12 / 10, 139 / 135, [256,512,28,28], 7 / 7,
+// 89.1 / 88.7; but fp32 [150,60,56,56], 4 / 4, 49.9 / 53.1, codes of [64,64,112,112], 8 / 8, 103.6 / 107.0, and anything of one or two
+// rounds).  The plan that was asked about stays that of two CTAs per SM.
+TeamPlan finer_cut(const TeamPlan& plan, const QuantIO& io, int dtype, const Geom& g, const StagedTuning& tune) {
+    const uint32_t C = (uint32_t)g.C, rounds = (C + plan.teams - 1) / plan.teams;
+    const uint64_t units = (uint64_t)g.outer * (uint64_t)(g.inner / (dtype == 0 ? 4 : 8));
+    if (rounds < 5 || tune.col_team == 1 || units * C >= (1ull << 32)) return plan;
+    const uint32_t ctas = 4u * plan.sm_count, runs = (uint32_t)((units + 7) / 8);
+    uint64_t best = ~0ull;
+    TeamPlan f = plan;
+    for (uint32_t R = 1; R <= ctas && R <= runs; ++R) {
+        const uint32_t share = 8 * ((runs + R - 1) / R);
+        if (share > kTSmemUnits / 2) continue;
+        const uint32_t teams = std::min(ctas / R, C);
+        const uint64_t cost = (uint64_t)((C + teams - 1) / teams) * (share + 1000);
+        if (cost < best) {
+            best = cost;
+            f.R = R;
+            f.teams = teams;
+            f.tile_units = share;
+        }
+    }
+    const uint32_t finer = (C + f.teams - 1) / f.teams;
+    if (best == ~0ull || f.tile_units < 2500 || !(finer < rounds || (finer == rounds && dtype == 1 && !io.dist && !io.pcodes))) return plan;
+    f.smem_bytes = 16u * f.tile_units;
+    f.threads = kTThreads / 2;
+    return f;
+}
+
+}  // namespace
 
 cudaError_t launch_colteam_list(const TeamPlan& plan, const TeamTensor* tensors, uint32_t n, int dtype, const Geom& g,
                                 const StagedTuning& tune, cudaStream_t st) {
@@ -658,14 +699,15 @@ cudaError_t launch_colteam_list(const TeamPlan& plan, const TeamTensor* tensors,
     return dtype == 0 ? t_launch_lag<float>(a, list, plan, tune, st) : t_launch_lag<__nv_bfloat16>(a, list, plan, tune, st);
 }
 
-cudaError_t launch_colteam(const TeamPlan& plan, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
+cudaError_t launch_colteam(const TeamPlan& asked, const QuantIO& io, int mode, int dtype, const Geom& g, int bits,
                            const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,
                            const StagedTuning& tune, cudaStream_t st) {
     const uint32_t V = dtype == 0 ? 4 : 8;
-    if (plan.lag) {
+    if (asked.lag) {
         const TeamTensor one{io, bits, ws, lo, hi, s_opt, z_opt};
-        return launch_colteam_list(plan, &one, 1, dtype, g, tune, st);
+        return launch_colteam_list(asked, &one, 1, dtype, g, tune, st);
     }
+    const TeamPlan plan = mode == MODE_FWD ? finer_cut(asked, io, dtype, g, tune) : asked;
     TArgs a{};
     a.x = io.x;
     a.gy = io.gy;

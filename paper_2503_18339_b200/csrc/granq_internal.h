@@ -243,6 +243,8 @@ struct TeamPlan {
     uint32_t tile_units;     // 16-byte units of x one CTA holds of each
     uint32_t gy_units;       // units of gy it holds beside them
     uint32_t smem_bytes;     // dynamic shared memory per CTA
+    uint32_t threads;        // of a CTA
+    uint32_t sm_count;       // planned for
 };
 // tensors: that many of these dims in one launch
 TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward, int sm_count, const StagedTuning& tune,

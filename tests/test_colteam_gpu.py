@@ -105,6 +105,33 @@ def test_strings_of_every_width(b, knobs, shape, dtype):
         assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
 
 
+@pytest.mark.parametrize("dtype,shape", [("f32", (8, 1500, 36, 36)), ("bf16", (16, 1500, 36, 36)), ("f32", (25, 480, 36, 40))],
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else v)
+def test_forward_with_a_finer_cut(b, dtype, shape):
+    """Half the threads and twice the CTAs, where that saves rounds: one CTA per channel and several, every output of the form."""
+    x, _ = make_case(shape, seed=sum(shape), dtype=dtype, relu=shape[0] % 2 == 0)
+    form = b.team_geometry(b.BF16 if dtype == "bf16" else b.F32, shape, with_backward=False)
+    assert form["taken"] == 1 and form["rounds"] >= 5
+    ref = orc.fused(x, 5)
+    xd = to_dev(x)
+    ws = b.make_workspace(xd, zeroed=True)
+    flags = b.FLAG_FORCE_COLWALK | b.FLAG_WORKSPACE_ZEROED
+    new = lambda: b.FakeQuantOut(workspace=ws)
+    clean = lambda: b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
+    assert_parity(b.granq_fakequant_fused(xd, 5, out=new(), flags=flags), ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    got = b.granq_fakequant_fused_fwd_packmask(xd, 5, out=new(), flags=flags)
+    assert clean()
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+    got = b.granq_quantize_packed_fused(xd, 5, out=new(), flags=flags)
+    assert_same_string(got.packed_codes, orc.pack_codes(ref.codes, 5))
+    got = b.granq_fakequant_fused_stats(xd, 5, out=new(), flags=flags)
+    assert clean()
+    assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+    # fp32 inside a pack, fp64 beyond: about 8 roundings of 2^-24 of a sum of same-signed terms
+    assert np.allclose(to_np(got.sums), orc.distortion_sums(x, ref.y), rtol=1e-6, atol=0)
+
+
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_waves_on_aligned_planes(b, knobs, shape, dtype):
