@@ -6,7 +6,9 @@
 // groups' keys with atomics; the grid hands over once (bounded), every CTA works out the parameters of its planes (Eq. 5) and
 // quantizes its piece from shared memory (Eq. 1, clamp, Eq. 6, STE).  Of one group over a larger tensor what does not stay is
 // read again, the last of it first, most of it from the L2.
-// Bound by the chain copy, fold, hand-over, quantize.  Against range pass and quantize pass (us, with gradient / forward / with
+// Bound by the chain copy, fold, hand-over, quantize; of the kept piece gy is brought into the L2 during the hand-over, when memory
+// is idle: with gradient, [200,33,33,33] fp32, 29 MB, 22.8 -> 21.2, one group [128,64,28,28] fp32 20.5 -> 18.7, [128,192,28,28] bf16
+// 30.6 -> 28.9 us.  Before that, against range pass and quantize pass (us, with gradient / forward / with
 // sums): [100,75,27,27] fp32, 21.9 MB, 37.9 / 31.6 / 36.7 -> 25.0 / 18.7 / 21.4; [200,301,7,7] bf16 38.5 / 34.0 / 37.9 -> 17.6 /
 // 16.6 / 19.8; one group: [128,128,28,28] fp32, 51 MB, sums 39.9 -> 29.2; [128,64,28,28] bf16, 13 MB, sums 24.5 -> 17.5.  Packed mask,
 // 4-bit and 5-bit codes of one group: [128,128,28,28] fp32, a third of it read again, 33.9 / 37.0 / 38.7 -> 32.3 / 32.9 / 33.6; [96,128,28,28]
@@ -179,6 +181,10 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
         }
     }
     // ---- the grid's hand-over (bounded) ----
+    if constexpr (kBwd) {
+        // what the kept piece meets is on its way to the L2 while the grid waits for its last CTA (half of it gives half as much)
+        if (tid == 0 && held > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gyg), "r"(held * 16u) : "memory");
+    }
     __threadfence();
     __syncthreads();
     if (tid == 0) {
