@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
     // ---- the grid's hand-over (bounded) ----
     if constexpr (kBwd) {
         // what the kept piece meets is on its way to the L2 while the grid waits for its last CTA (half of it gives half as much)
-        if (tid == 0 && held > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gyg), "r"(held * 16u) : "memory");
+        if (tid == 0 && held > 0) prefetch_l2(gyg, held * 16u);
     }
     __threadfence();
     __syncthreads();

@@ -32,6 +32,11 @@ template <typename T>
 constexpr int kRMaxThreads = Pack<T>::V == 4 ? 448 : 384;
 constexpr uint32_t kRMaxChannels = 4096;      // 64 slices at most
 constexpr uint32_t kRSmemBytes = 111u * 1024; // of one of two CTAs on an SM
+// From here on gy is sent for during the hand-over; a smaller one is most often still in the L2, and asking for it again costs
+// what it takes.  With gradient, us, gy in memory | gy in the L2: [32,28,28,128] fp32, 13 MB, 23.5 -> 21.4 | 14.8 -> 15.4;
+// [61,35,34,56] fp32, 16 MB, 25.6 -> 23.5 | 16.1 -> 16.6; [134,71,70,8] fp32, 21 MB, 28.4 -> 25.5 | 18.9 -> 18.8; [64,14,14,512]
+// fp32, 26 MB, 31.2 -> 29.7 | 22.4 -> 20.7; [17,14,14,2048] fp32, 27 MB, 31.7 -> 29.7 | 22.8 -> 20.9.
+constexpr uint64_t kRFetchBytes = 20ull << 20;
 constexpr uint32_t kRSpinLimit = 1u << 24;    // bounded wait on the grid (x ~32 ns)
 constexpr uint32_t kRStatusTimeout = 5;       // GRANQ_ERR_TIMEOUT
 
@@ -60,6 +65,7 @@ struct RArgs {
     uint32_t hold;       // blocks of rows a CTA keeps in shared memory
     uint32_t lost;       // of the others, those before this one are not expected to be in the L2 when they are read again
     uint32_t spin_limit, expected;
+    uint32_t fetch;      // what the kept blocks meet of gy is sent for during the hand-over
     uint32_t early;      // x may be read before the kernel ahead has completed: it only clears the workspace
     uint64_t rows;
 };
@@ -139,6 +145,16 @@ __global__ void __launch_bounds__(kRMaxThreads<T>, 2) rows_kernel(const RArgs a)
         }
     }
     // ---- the team's hand-over (bounded) ----
+    if constexpr (kBwd) {
+        if (a.fetch) {
+            if (a.slices == 1) {                           // a block of rows is one piece
+                const uint64_t row0 = ((uint64_t)rank + (uint64_t)tid * a.team) * L;
+                if (tid < a.hold && row0 < a.rows) prefetch_l2(reinterpret_cast<const uint4*>(a.gy) + row0 * a.ncol, (uint32_t)min((uint64_t)L, a.rows - row0) * a.ncol * 16u);
+            } else if (cin == 0) {
+                for (uint32_t k = 0; k < held; ++k) prefetch_l2(gyg + k * step, width * 16u);
+            }
+        }
+    }
     __threadfence();
     __syncthreads();
     if (tid == 0) {
@@ -363,6 +379,7 @@ cudaError_t launch_rows(const QuantIO& io, int mode, int dtype, const Geom& g, i
     // ([128,112,112,64] fp32 forward 217 -> 208 us)
     const double tail = 64e6 / ((double)a.rows * a.ncol * 16);
     a.lost = tail < 1.0 ? (uint32_t)((1.0 - tail) * (double)per_cta) : 0u;
+    a.fetch = (uint64_t)a.rows * a.ncol * 16 >= kRFetchBytes ? 1u : 0u;
     a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kRSpinLimit;
     a.expected = a.team + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
     a.early = ws.cleared ? 1u : 0u;
