@@ -920,7 +920,7 @@ int granq_hold_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
     const bool backward = with_backward != 0;
     const QuantIO io = aligned_io(backward, packed != 0);
     const HoldPlan p = plan_hold(dtype, g, io, sm_count);
-    if (!p.ok) return GRANQ_ERR_UNSUPPORTED;
+    if (!p.ok || !p.whole) return GRANQ_ERR_UNSUPPORTED;
     const int plan = packed ? (plan_cluster(dtype, g, io, false, g_tune).ok || plan_colwalk(dtype, g, io, g_tune).ok ? PLAN_COLWALK : PLAN_TWO_PASS)
                             : choose_plan(dtype, g, io, backward, 0, nullptr, nullptr, nullptr, nullptr);
     const bool taken = (plan == PLAN_TWO_PASS || plan == PLAN_L2WAVE) && hold_allowed(0);

@@ -13,7 +13,9 @@
 // 16.6 / 19.8; one group: [128,128,28,28] fp32, 51 MB, sums 39.9 -> 29.2; [128,64,28,28] bf16, 13 MB, sums 24.5 -> 17.5.  Packed mask,
 // 4-bit and 5-bit codes of one group: [128,128,28,28] fp32, a third of it read again, 33.9 / 37.0 / 38.7 -> 32.3 / 32.9 / 33.6; [96,128,28,28]
 // fp32 27.0 / 28.8 / 29.9 -> 26.6 / 26.5 / 27.2; bf16 20.8 / 22.3 / 22.6 -> 16.6 / 20.7 / 20.8.  Against the L2-resident waves, one group:
-// bf16 [128,192,28,28], 38.5 MB, 38.9 / 30.8 -> 35.4 / 24.7; fp32 [128,64,28,28] 26.6 / 18.8 -> 26.2 / 18.0.  There is no smallest size: a tensor
+// bf16 [128,192,28,28], 38.5 MB, 38.9 / 30.8 -> 35.4 / 24.7; fp32 [128,64,28,28] 26.6 / 18.8 -> 26.2 / 18.0.  What is left
+// behind the last whole unit, and the last word of a mask or of codes, is one thread's: two passes with scalar loads there (with gradient)
+// [60,301,7,7] bf16 41.2 -> 10.4, [150,75,27,27] bf16 138 -> 18.7, [5,75,27,27] fp32 30.5 -> 8.9.  There is no smallest size: a tensor
 // of 80 KB, [8,75,5,7], takes 5.8 us from a graph and 11.9 eagerly where two passes took 23.1 and 25.4, one group of 0.5 MB 6.0 and 9.9 where the
 // waves took 12.4 and 9.8.
 #include "granq_internal.h"
@@ -29,6 +31,7 @@ constexpr uint32_t kHWarps = kHThreads / 32;
 constexpr uint32_t kHSpinLimit = 1u << 24;              // bounded wait for the grid (x ~32 ns)
 constexpr uint32_t kHStatusTimeout = 5;                 // GRANQ_ERR_TIMEOUT
 constexpr uint32_t kHSmemBytes = 111u * 1024;           // two CTAs per SM
+constexpr uint32_t kHFetchUnits = 1024;                 // gy of a kept piece of 16 KB and more is sent for during the hand-over
 constexpr uint32_t kHPlaneBytes = 2 * sizeof(uint32_t) + sizeof(GroupParam);      // keys and parameters of one plane
 
 enum : int { H_ONE = 0, H_PLANES = 1, H_RAGGED = 2 };   // one group; planes of whole units; planes that are not
@@ -51,7 +54,8 @@ struct HArgs {
     float* s_out;
     float* z_out;
     float qmax;
-    uint32_t units;        // 16-byte units of the tensor
+    uint32_t units;        // whole 16-byte units of the tensor (with a mask or codes, an even number of fp32 ones)
+    uint32_t tail;         // elements behind them
     uint32_t share;        // of one CTA
     uint32_t held;         // of those, kept in shared memory
     uint32_t planes;       // room in the tables
@@ -62,8 +66,9 @@ struct HArgs {
     FastDiv div_inner, div_groups;
 };
 
-// U = units a thread handles together in the quantize walk
-template <typename T, int MODE, int EXTRAS, int KIND, int U>
+// END: elements are left behind the last whole unit, or mask or codes end inside a 32-bit word (a form of its own: the code for it
+// cost the others 0.3 us of 10).  U = units a thread handles together in the quantize walk
+template <typename T, int MODE, int EXTRAS, int KIND, bool END, int U>
 __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
     constexpr int V = Pack<T>::V;
     constexpr bool kBwd = (MODE & MODE_BWD) != 0;
@@ -81,6 +86,9 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
     uint4* yg = reinterpret_cast<uint4*>(a.y) + u0;
     uint4* gxg = reinterpret_cast<uint4*>(a.gx) + u0;
     const float qmax = a.qmax;
+    // elements behind the last whole unit, all of the last plane: the last CTA's, one thread handles them
+    const uint32_t tail = END && blockIdx.x == gridDim.x - 1 ? a.tail : 0u;
+    const T* xt = reinterpret_cast<const T*>(a.x) + (size_t)a.units * V;
     // planes of this piece: p0, p0 + 1, ..., the first of them from element rem0 on
     uint32_t p0 = 0, rem0 = 0, np = 1;
     if constexpr (KIND != H_ONE) {
@@ -115,6 +123,13 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
         }
         float m0, m1;
         fold.result(m0, m1);
+        if constexpr (END) {
+            for (uint32_t i = 0; tid == kHThreads - 1 && i < tail; ++i) {
+                const float v = load_scalar(xt + i);
+                m0 = fminf(m0, v);
+                m1 = fmaxf(m1, v);
+            }
+        }
         uint32_t ka = m0 <= m1 ? ~enc(m0) : 0u, kb = m0 <= m1 ? enc(m1) : 0u;
         ka = __reduce_max_sync(kFullMask, ka);
         kb = __reduce_max_sync(kFullMask, kb);
@@ -170,6 +185,15 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
             }
             flush();
         }
+        if constexpr (END) {
+            for (uint32_t i = 0; tid == kHThreads - 1 && i < tail; ++i) {
+                const float v = load_scalar(xt + i);
+                if (v == v) {
+                    atomicMax(s_kmn + np - 1, ~enc(v));
+                    atomicMax(s_kmx + np - 1, enc(v));
+                }
+            }
+        }
         if (a.early) after_the_kernel_ahead();
         __syncthreads();
         for (uint32_t t = tid; t < np; t += kHThreads) {
@@ -182,8 +206,9 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
     }
     // ---- the grid's hand-over (bounded) ----
     if constexpr (kBwd) {
-        // what the kept piece meets is on its way to the L2 while the grid waits for its last CTA (half of it gives half as much)
-        if (tid == 0 && held > 0) prefetch_l2(gyg, held * 16u);
+        // what the kept piece meets is on its way to the L2 while the grid waits for its last CTA (half of it gives half as much); a
+        // smaller one is most often still there ([20,75,27,27] fp32 10.1 -> 10.5)
+        if (tid == 0 && held >= kHFetchUnits) prefetch_l2(gyg, held * 16u);
     }
     __threadfence();
     __syncthreads();
@@ -244,7 +269,7 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
             }
         }
         // masks and codes 8 elements at a time, a pair of fp32 units by the two lanes of a pair, the first of them by the even one: the
-        // tensor is a multiple of 32 elements, a piece begins on a multiple of 8 units, and both walks give an even lane an even unit
+        // whole units are a multiple of 8 elements, a piece begins on a multiple of 8 units, and both walks give an even lane an even unit
         if constexpr (EXTRAS == 3) {
             store_code_bytes<V>(a.pcodes, (size_t)(u0 + i) * V, code_string_of<V>(cb, code_bits), code_bits, lane, lanes);
             return;
@@ -254,6 +279,39 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
         if constexpr (EXTRAS == 2) store_mask_byte<V>(a.pmask, (size_t)(u0 + i) * V, mask_bits_of<V, EXTRAS>(mb), lane, lanes);
         if constexpr (EXTRAS == 4) dacc.add(px, py);
     };
+    if constexpr (END) {
+        if (tid == kHThreads - 1 && blockIdx.x == gridDim.x - 1) {
+            const size_t e0 = (size_t)a.units * V;
+            const GroupParam gp = s_par[np - 1];
+            uint64_t str = 0;                   // masks and codes: of the tail, a whole number of bytes before it
+            for (uint32_t off = 0; off < tail; off += V) {
+                Pack<T> px, pg, py, pgx;
+                uint32_t cb[V / 4], mb[V / 4];
+                px.raw = pg.raw = make_uint4(0, 0, 0, 0);
+                for (uint32_t i = 0; i < (uint32_t)V; ++i)
+                    if (off + i < tail) {
+                        px.set(i, load_scalar(xt + off + i));
+                        if constexpr (kBwd) pg.set(i, load_scalar(reinterpret_cast<const T*>(a.gy) + e0 + off + i));
+                    }
+                quantize_own<T, kBwd, EXTRAS>(px, pg, gp, qmax, py, pgx, cb, mb, EXTRAS == 3 ? a.code_bits : 8);
+                for (uint32_t i = 0; i < (uint32_t)V; ++i)
+                    if (off + i < tail) {
+                        if constexpr (EXTRAS != 3) store_scalar(reinterpret_cast<T*>(a.y) + e0 + off + i, py.get(i));
+                        if constexpr (kBwd) store_scalar(reinterpret_cast<T*>(a.gx) + e0 + off + i, pgx.get(i));
+                        if constexpr (EXTRAS == 4) dacc.add_one(px.get(i), py.get(i));
+                    }
+                if constexpr (EXTRAS == 2) str |= (uint64_t)mask_bits_of<V, EXTRAS>(mb) << off;
+                if constexpr (EXTRAS == 3) str |= code_string_of<V>(cb, a.code_bits) << (off * a.code_bits);
+            }
+            if constexpr (EXTRAS == 2 || EXTRAS == 3) {                        // up to the end of the last word
+                const uint32_t width = EXTRAS == 3 ? a.code_bits : 1;
+                uint8_t* dst = reinterpret_cast<uint8_t*>(EXTRAS == 3 ? a.pcodes : a.pmask) + e0 / 8 * width;
+                const size_t bytes = ((e0 + tail) * width + 31) / 32 * 4 - e0 / 8 * width;
+                str &= (1ull << (tail * width)) - 1;                           // at most 7 codes: 56 bits
+                for (size_t i = 0; i < bytes; ++i) dst[i] = i < 8 ? (uint8_t)(str >> (8 * i)) : (uint8_t)0;
+            }
+        }
+    }
     // what did not stay, a block of units at a time from the end back; inside a block forward from an even unit (masks and codes:
     // n and held are even), so that the even lane of a pair has its first unit there too
     if constexpr (KIND == H_ONE) {
@@ -316,9 +374,12 @@ cudaError_t h_launch(const HArgs& a, const HoldPlan& p, int kind, const StagedTu
         void* params[] = {(void*)&a};
         return launch_cooperative((const void*)kern, p.ctas, kHThreads, params, p.held * 16 + p.planes * kHPlaneBytes, tune, st);
     };
-    if (kind == H_ONE) return go(hold_kernel<T, MODE, EXTRAS, H_ONE, U>);
-    if (kind == H_PLANES) return go(hold_kernel<T, MODE, EXTRAS, H_PLANES, U>);
-    return go(hold_kernel<T, MODE, EXTRAS, H_RAGGED, U>);
+    if (kind == H_ONE) return p.whole ? go(hold_kernel<T, MODE, EXTRAS, H_ONE, false, U>) : go(hold_kernel<T, MODE, EXTRAS, H_ONE, true, U>);
+    if (kind == H_RAGGED) return p.whole ? go(hold_kernel<T, MODE, EXTRAS, H_RAGGED, false, U>) : go(hold_kernel<T, MODE, EXTRAS, H_RAGGED, true, U>);
+    // planes of whole units leave nothing behind the last of them but for a mask or codes
+    if constexpr (EXTRAS == 2 || EXTRAS == 3)
+        if (!p.whole) return go(hold_kernel<T, MODE, EXTRAS, H_PLANES, true, U>);
+    return go(hold_kernel<T, MODE, EXTRAS, H_PLANES, false, U>);
 }
 
 }  // namespace
@@ -330,10 +391,14 @@ HoldPlan plan_hold(int dtype, const Geom& g, const QuantIO& io, int sm_count) {
     p.ok = false;
     const int64_t V = dtype == 0 ? 4 : 8;
     if (io.codes || io.mask) return p;
-    if ((io.pmask || io.pcodes) && (g.E % 32 != 0 || io.gy)) return p;
-    if (g.E % V != 0 || g.inner < V || g.E >= (1ll << 31) || g.C >= (1ll << 28)) return p;
+    const bool packed = io.pmask || io.pcodes;
+    if (packed && io.gy) return p;
+    const int64_t step = packed ? 8 : V;                  // the whole units: masks and codes whole bytes of them
+    p.tail = (uint32_t)(g.E % step);
+    p.whole = p.tail == 0 && !(packed && g.E % 32 != 0);
+    if (g.E < step || g.inner < V || (p.tail && g.inner < step) || g.E >= (1ll << 31) || g.C >= (1ll << 28)) return p;
     if (!h_aligned16(io.x) || !h_aligned16(io.gy) || !h_aligned16(io.y) || !h_aligned16(io.gx)) return p;
-    const uint64_t units = (uint64_t)(g.E / V), most = 2ull * (uint64_t)sm_count;
+    const uint64_t units = (uint64_t)((g.E - p.tail) / V), most = 2ull * (uint64_t)sm_count;
     p.share = (uint32_t)((std::max<uint64_t>((units + most - 1) / most, 64) + 7) / 8 * 8);
     p.ctas = (uint32_t)((units + p.share - 1) / p.share);
     const bool one = g.C == 1 && g.outer == 1;
@@ -369,7 +434,8 @@ cudaError_t launch_hold(const HoldPlan& plan, const QuantIO& io, int mode, int d
     a.s_out = s_opt;
     a.z_out = z_opt;
     a.qmax = (float)((1 << bits) - 1);
-    a.units = (uint32_t)(g.E / V);
+    a.units = (uint32_t)((g.E - plan.tail) / V);
+    a.tail = plan.tail;
     a.share = plan.share;
     a.held = plan.held;
     a.planes = plan.planes;

@@ -282,6 +282,8 @@ struct HoldPlan {
     bool ok;
     uint32_t ctas, share;    // CTAs, 16-byte units of one
     uint32_t held, planes;   // of those, kept in shared memory; planes it can cut through
+    uint32_t tail;           // elements behind the last whole unit (masks and codes: behind the last whole byte)
+    bool whole;              // nothing is left behind the units, or in the last word of a mask or of codes
 };
 HoldPlan plan_hold(int dtype, const Geom& g, const QuantIO& io, int sm_count);
 // may be refused: launch_cooperative()

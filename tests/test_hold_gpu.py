@@ -73,6 +73,55 @@ def test_held_tensor(b, shape, mode, dtype):
     assert_parity(b.granq_fakequant_fused(xd, bits, gy=gyd, group=mode, out=dirty), ref, shape, 1, mode, backward=True)
 
 
+@pytest.mark.parametrize("shape,mode", [
+    ((1, 1, 3, 3), 0),          # one unit of bf16 and one element
+    ((3, 5, 7, 7), 0),          # 7 elements behind the last whole byte of a mask
+    ((3, 2, 5, 9), 1),
+    ((33, 7, 2, 5), 0),         # planes of little more than a unit of bf16
+    ((3, 7, 5, 13), 2),
+    ((21, 379, 7, 7), 0),       # several planes to a thread
+    ((13, 13, 93, 93), 0),      # a plane over several pieces
+    ((5, 41, 97, 10), 1),       # whole units of bf16 and half a unit of fp32 more than whole bytes
+    ((7, 3, 2, 3), 0),          # planes shorter than what a thread handles: two passes
+    ((1, 1, 4999, 5001), 2),    # one group of which bf16 reads a part again
+], ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else f"g{v}")
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_elements_behind_the_last_whole_unit(b, shape, mode, dtype):
+    """The last elements, the top of their group's range in one call and not in the other; masks and codes up to the end of the
+    last word, in buffers that held something else; the workspace zero again; both kinds of call agree with two passes."""
+    x, gy = make_case(shape, seed=sum(shape), dtype=dtype)
+    for peak in (False, True):
+        if peak:
+            x.reshape(-1)[-1] = 0x42C8 if dtype == "bf16" else 100.0
+        xd, gyd = to_dev(x), to_dev(gy)
+        ws = b.make_workspace(xd, group=mode, zeroed=True)
+        new = lambda: b.FakeQuantOut(workspace=ws)
+        clean = lambda: b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
+        for bits in (4, 7) if x.size < 1 << 20 else (4,):
+            ref = orc.fused(x, bits, gy=gy, group_mode=mode)
+            got = b.granq_fakequant_fused(xd, bits, gy=gyd, group=mode, out=new(), want_params=True, flags=b.FLAG_WORKSPACE_ZEROED)
+            assert clean()
+            assert_parity(got, ref, shape, 1, mode, backward=True)
+            assert_parity(b.granq_fakequant_fused(xd, bits, group=mode), ref, shape, 1, mode, backward=False)
+            got = b.granq_fakequant_fused_stats(xd, bits, group=mode, out=new(), flags=b.FLAG_WORKSPACE_ZEROED)
+            assert clean()
+            assert_parity(got, ref, shape, 1, mode, backward=False)
+            # fp32 inside a pack, fp64 beyond: about 8 roundings of 2^-24 of a sum of same-signed terms
+            assert np.allclose(to_np(got.sums), orc.distortion_sums(x, ref.y), rtol=1e-6, atol=0)
+            out = new()
+            out.packed_mask = torch.full(((x.size + 31) // 32,), -1, dtype=torch.int32, device="cuda")
+            got = b.granq_fakequant_fused_fwd_packmask(xd, bits, group=mode, out=out, flags=b.FLAG_WORKSPACE_ZEROED)
+            assert clean()
+            assert_parity(got, ref, shape, 1, mode, backward=False)
+            assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+            for code_bits in (1, 3, 4, 7, 8) if bits == 4 else ():
+                out = new()
+                out.packed_codes = torch.full(((x.size * code_bits + 31) // 32,), -1, dtype=torch.int32, device="cuda")
+                got = b.granq_quantize_packed_fused(xd, code_bits, group=mode, out=out, flags=b.FLAG_WORKSPACE_ZEROED)
+                assert clean()
+                assert_same_string(got.packed_codes, orc.pack_codes(orc.fused(x, code_bits, group_mode=mode).codes, code_bits))
+
+
 @pytest.mark.parametrize("dtype,shape", [("f32", (96, 128, 28, 28)), ("bf16", (192, 128, 28, 28))])
 def test_one_group_beyond_what_stays_on_chip(b, dtype, shape):
     x, gy = make_case(shape, seed=3, dtype=dtype)
