@@ -162,9 +162,10 @@ __global__ void __launch_bounds__(kThreads, 8) range_flat_kernel(const T* __rest
 constexpr uint32_t kRangeSmemGroups = 1024;
 
 // ALIGNED: planes are whole packs (div_plane divides pack indices); otherwise a pack may straddle two
-// planes (div_plane divides element indices, `inner` >= V elements per plane).
+// planes (div_plane divides element indices, `inner` >= V elements per plane), and `tail` elements may be left behind
+// the last whole pack, all of them of the last plane.
 template <typename T, bool ALIGNED>
-__global__ void __launch_bounds__(kThreads) range_rows_kernel(const uint4* __restrict__ x, uint32_t n_units,
+__global__ void __launch_bounds__(kThreads) range_rows_kernel(const uint4* __restrict__ x, uint32_t n_units, uint32_t tail,
                                                               uint32_t inner, FastDiv div_plane, FastDiv div_C,
                                                               uint32_t groups, uint32_t* __restrict__ kmin,
                                                               uint32_t* __restrict__ kmax, RangeEnd end) {
@@ -248,7 +249,16 @@ __global__ void __launch_bounds__(kThreads) range_rows_kernel(const uint4* __res
         reduce(row + nwarps, pb);
     }
     run_flush(run, dmn, dmx);
-    if constexpr (!ALIGNED) run_flush(run2, dmn, dmx);
+    if constexpr (!ALIGNED) {
+        run_flush(run2, dmn, dmx);
+        if (blockIdx.x == gridDim.x - 1 && threadIdx.x < tail) {
+            const float v = load_scalar(reinterpret_cast<const T*>(x + n_units) + threadIdx.x);
+            if (v == v) {
+                atomicMax(dmn + groups - 1, ~enc(v));
+                atomicMax(dmx + groups - 1, enc(v));
+            }
+        }
+    }
     if (combine) {
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < groups; i += kThreads) {
@@ -457,7 +467,11 @@ constexpr int kFlatBlocks = !kFlatParts<V, MODE, EXTRAS, RAGGED> ? 0 : MODE == M
 // fp32 lane (every bf16 lane) with plain stores: no word assembly across the warp.
 // RAGGED: planes are not whole 16-byte packs (7x7 planes), so a pack may straddle two planes and takes the
 // parameters of both (planes of at least one pack: never more than two).
-template <typename T, int V, int MODE, int EXTRAS, bool PACKONLY = false, bool RAGGED = false>
+// END (RAGGED): the last pack is not whole; it is read and written element by element, the rest of it is +0 and says nothing.
+// Calls against the scalar form, us: bf16 forward of [31,1509,29,29], 79 MB, range and quantize 236 -> 105; fp32 with gradient
+// [51,79,69,69] 142 -> 93, sums [207,77,34,35] 121 -> 73; range, mask and the way back of bf16 [61,225,18,17] 82.5 -> 23.9, fp32
+// [22,193,95,95] 323 -> 188; codes and back of [31,157,23,22] bf16 22.8 -> 17.3 (the way back alone).
+template <typename T, int V, int MODE, int EXTRAS, bool PACKONLY = false, bool RAGGED = false, bool END = false>
 __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKONLY, RAGGED>))
                                             quant_flat_kernel(const T* __restrict__ x, const T* __restrict__ gy,
                                                               T* __restrict__ y, T* __restrict__ gx,
@@ -495,6 +509,15 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
                     if constexpr (V == 1) {
                         sx[j] = load_scalar(x + e0 + k[j]);
                         if constexpr (kBwd) sg[j] = load_scalar(gy + e0 + k[j]);
+                    } else if (END && k[j] + V > ne) {
+                        px[j].raw = make_uint4(0, 0, 0, 0);
+                        if constexpr (kBwd) pg[j].raw = make_uint4(0, 0, 0, 0);
+#pragma unroll
+                        for (int i = 0; i < V; ++i)
+                            if (k[j] + i < ne) {
+                                px[j].set(i, load_scalar(x + e0 + k[j] + i));
+                                if constexpr (kBwd) pg[j].set(i, load_scalar(gy + e0 + k[j] + i));
+                            }
                     } else {
                         px[j].raw = ld_stream_16(x + e0 + k[j]);
                         if constexpr (kBwd) pg[j].raw = ld_stream_16(gy + e0 + k[j]);
@@ -560,9 +583,10 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
                     GroupParam gp{p.s, p.z, rcp, tie_threshold(rcp, p.z, qmax)};
                     GroupParam gp2 = gp;
                     int n1 = V;
+                    const bool whole = !END || k[j] + V <= ne;
                     if constexpr (RAGGED) {
                         const uint32_t rem = (uint32_t)base.rem + k[j] - q * (uint32_t)g.inner;      // position inside plane q
-                        n1 = (int)min((uint32_t)V, (uint32_t)g.inner - rem);
+                        n1 = whole ? (int)min((uint32_t)V, (uint32_t)g.inner - rem) : V;
                         if (n1 < V) {                                                           // the rest lies in plane q + 1
                             if (tabled) {
                                 gp2.s = s_tab_s[q + 1];
@@ -580,6 +604,20 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
                         }
                     }
                     quantize_pack<T, kBwd, RAGGED, EXTRAS, false, kParts>(px[j], pg[j], gp, gp2, n1, qmax, py, pgx, cb, mb, EXTRAS == 3 ? code_bits : 8);
+                    if constexpr (END) {
+                        if (!whole) {
+#pragma unroll
+                            for (int i = 0; i < V; ++i)
+                                if (k[j] + i < ne) {
+                                    if constexpr (kFwd && !PACKONLY) store_scalar(y + e + i, py.get(i));
+                                    if constexpr (kBwd) store_scalar(gx + e + i, pgx.get(i));
+                                } else {
+                                    py.set(i, 0.0f);
+                                    if constexpr (EXTRAS == 1) cb[i / 4] &= ~(0xFFu << (8 * (i % 4)));
+                                    if constexpr (EXTRAS == 2) mb[0] &= ~(1u << i);
+                                }
+                        }
+                    }
                     if constexpr (EXTRAS == 3) {
                         code_string = code_string_of<V>(cb, code_bits);
                     } else if constexpr (EXTRAS != 0) {
@@ -594,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
                         }
                     }
                     if constexpr (kFwd && !PACKONLY) {
-                        if (EXTRAS != 1 || y) st_stream_16(y + e, py.raw);
+                        if ((EXTRAS != 1 || y) && whole) st_stream_16(y + e, py.raw);
                         if constexpr (EXTRAS == 1) {
                             if (codes) {
 #pragma unroll
@@ -603,7 +641,7 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
                         }
                     }
                     if constexpr (kBwd) {
-                        st_stream_16(gx + e, pgx.raw);
+                        if (whole) st_stream_16(gx + e, pgx.raw);
                         if constexpr (EXTRAS == 1) {
                             if (mask) {
 #pragma unroll
@@ -820,12 +858,17 @@ __global__ void __launch_bounds__(kThreads) naive_quant_kernel(const T* __restri
 // persistent grid).  The kernel behind is not let start beside it: that is mostly one that takes an SM's shared memory (the next
 // layer's), which a stream of a wave or two is slower beside (packed mask and backward, us, with / without: bf16 [128,960,7,7] 26.0 / 21.2,
 // fp32 [25,856,14,14] 21.6 / 19.2, [41,1896,15,16] 60.8 / 60.3; 26 shapes 0.98).
-// V = elements per thread and step: a 16-byte pack when E and the pointers allow it, else 1.
+// V = elements per thread and step: a 16-byte pack when the pointers allow it, else 1.  `tail` elements behind the E of whole
+// packs are the first threads' of the last block.
 template <typename T, int V>
 __global__ void __launch_bounds__(kThreads) bwd_packmask_kernel(const T* __restrict__ gy,
                                                                 const uint32_t* __restrict__ pmask,
-                                                                T* __restrict__ gx, int64_t E) {
+                                                                T* __restrict__ gx, int64_t E, uint32_t tail) {
     wait_for_the_kernel_ahead();      // and no word to the kernel behind
+    if (V > 1 && blockIdx.x == gridDim.x - 1 && threadIdx.x < tail) {
+        const int64_t at = E + threadIdx.x;
+        store_scalar(gx + at, (__ldg(pmask + (at >> 5)) >> (uint32_t)(at & 31)) & 1u ? load_scalar(gy + at) : 0.0f);
+    }
     const int64_t u0 = (int64_t)blockIdx.x * kThreads * kUnroll;
     int64_t e[kUnroll];
     Pack<T> pg[kUnroll];
@@ -894,17 +937,23 @@ __global__ void __launch_bounds__(kThreads) distortion_kernel(const T* __restric
 // Eight codes (BITS bytes of the bit string) per thread and step, two such strings in flight: two or three words of
 // codes, one pair of divisions for the channel, shifts that are constants, and 32 bytes of fp32 (16 of bf16) stored at
 // once.  Planes of at least 8 elements; where they are no multiple of 8 (RAGGED) a string may reach into the next
-// plane.  Bound by the stores: [128,144,56,56], 231 MB written from 36 MB of 5-bit codes, 92 -> 45 us
+// plane.  `tail` codes behind the last whole string, all of the last plane, are the first threads' of the last block.
+// Bound by the stores: [128,144,56,56], 231 MB written from 36 MB of 5-bit codes, 92 -> 45 us
 // (5.9 TB/s; a thread per 16 bytes with two 32-bit divisions took 171 instructions for 4 elements).  A block per 512
 // strings rather than a persistent grid, so that the stores go out in the order of memory: [128,96,112,112] 133 -> 110 us.
 template <typename T, int BITS, bool RAGGED>
 __global__ void __launch_bounds__(kThreads) dequant_strings_kernel(const uint32_t* __restrict__ pcodes, T* __restrict__ y,
-                                                                   uint32_t nstrings, uint32_t last_word, uint32_t inner,
+                                                                   uint32_t nstrings, uint32_t tail, uint32_t last_word, uint32_t inner,
                                                                    FastDiv div_inner, FastDiv div_C,
                                                                    const float* __restrict__ s, const float* __restrict__ z) {
     after_the_kernel_ahead();
     constexpr uint32_t kField = (1u << BITS) - 1u;
     constexpr int kFly = 2;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x < tail) {
+        const uint64_t bit = ((uint64_t)nstrings * 8 + threadIdx.x) * BITS;
+        const uint32_t w0 = (uint32_t)(bit >> 5), c = __funnelshift_r(__ldg(pcodes + w0), __ldg(pcodes + min(w0 + 1, last_word)), (uint32_t)bit & 31);
+        store_scalar(y + (size_t)nstrings * 8 + threadIdx.x, __fmul_rn(__ldg(s + div_C.d - 1), __fsub_rn((float)(c & kField), __ldg(z + div_C.d - 1))));
+    }
     const uint32_t t0 = blockIdx.x * (kThreads * kFly) + threadIdx.x;
     uint32_t w[kFly][3];
 #pragma unroll
@@ -1040,7 +1089,7 @@ cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t*
     constexpr int VF = Pack<T>::V;
     bool vec = aligned16(x) && (g.inner % VF == 0);
     int grid = flat_grid(f);
-    const bool rows_ok = aligned16(x) && g.E % VF == 0 && g.inner >= VF && g.E < (1ll << 31) &&
+    const bool rows_ok = aligned16(x) && g.inner >= VF && g.E < (1ll << 31) &&
                          g.C < (1ll << 30) && g.inner < (1ll << 30);
     // columns: slabs of whole units, at least a batch of them to walk, planes shorter than a row of the vector path or
     // not whole units
@@ -1062,7 +1111,7 @@ cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t*
         const int64_t cap = (int64_t)range_rows_ctas();                 // 4 resident CTAs per SM at 64 registers
         int rgrid = (int)(ctas < cap ? ctas : cap);
         auto by_rows = [&](auto kern, uint32_t plane) {
-            return launch_after(layout, kern, rgrid, kThreads, 0, st, (const uint4*)x, n_units, (uint32_t)g.inner, make_fastdiv(plane),
+            return launch_after(layout, kern, rgrid, kThreads, 0, st, (const uint4*)x, n_units, (uint32_t)(g.E % VF), (uint32_t)g.inner, make_fastdiv(plane),
                                 make_fastdiv((uint32_t)g.C), (uint32_t)g.C, kmin, kmax, end);
         };
         return vec ? by_rows(range_rows_kernel<T, true>, (uint32_t)(g.inner / VF)) : by_rows(range_rows_kernel<T, false>, (uint32_t)g.inner);
@@ -1091,20 +1140,24 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
     // forward with y and the packed mask as the only outputs: a leaner instantiation
     const bool pmask_only = io.pmask != nullptr && io.y != nullptr && io.codes == nullptr && io.mask == nullptr &&
                             io.dist == nullptr && io.pcodes == nullptr;
+    const bool dist_only = io.dist != nullptr && io.y != nullptr && io.codes == nullptr && io.mask == nullptr &&
+                           io.pmask == nullptr && io.pcodes == nullptr;
     const bool pack_only = io.pcodes != nullptr && io.y == nullptr && io.codes == nullptr && io.mask == nullptr &&
                            io.pmask == nullptr && io.dist == nullptr;
     // planes that are not whole packs, everything else in place for 16-byte accesses: the vector kernel with
     // packs that may straddle two planes
-    const bool ragged = !vec && g.inner >= VF && g.inner % VF != 0 && g.E % VF == 0 && !f.inner_big && aligned16(io.x) &&
+    const bool planes = !vec && g.inner >= VF && g.inner % VF != 0 && !f.inner_big && aligned16(io.x) &&
                         aligned16(io.gy) && aligned16(io.y) && aligned16(io.gx) && ((uintptr_t)io.codes % 4 == 0) &&
                         ((uintptr_t)io.mask % 4 == 0);
+    // ... and of those, where the last pack is not whole either: all outputs but codes and masks by the byte
+    const bool ragged = planes && g.E % VF == 0, end = planes && g.E % VF != 0 && (!extras || pmask_only || pack_only || dist_only);
     // Five blocks of a table each fill an SM.  The scalar form is bound by its instructions, and its grids of up to a wave - four blocks
     // to an SM or, backward, seven - are spread evenly only over an empty GPU: blocks that start before the kernel ahead has
     // ended crowd on the SMs that have room first, unless two grids leave SMs free.  Alone / set up early, us: backward f32 [75,31,41,41], 477
     // blocks, 24.8 / 31.5, of [33,41,51,51], 430, 22.8 / 20.5; fused call of bf16 [37,532,7,7], 118, 41.4 / 49.5, of [37,133,7,7], 30, 39.3 / 37.3;
     // forward [33,41,51,51] 22.8 / 24.1, [101,75,27,27], 674, 39.3 / 38.2.
     const int64_t sms = sm_count(), slots = sms * (MODE == MODE_BWD ? 7 : 4);
-    const bool crowded = !vec && !ragged && 2 * f.ntiles > sms && f.ntiles <= slots;
+    const bool crowded = !vec && !ragged && !end && 2 * f.ntiles > sms && f.ntiles <= slots;
     const int layout = crowded ? kAlone : sm_layout(100, (uint64_t)g.E * sizeof(T));
     auto go = [&](auto kern) {
         return launch_after(layout, kern, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask,
@@ -1129,8 +1182,6 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
             if (io.pmask) return vec ? cols(quant_cols_kernel<T, true, true>, plane) : cols(quant_cols_kernel<T, false, true>, plane);
             return vec ? cols(quant_cols_kernel<T, true, false>, plane) : cols(quant_cols_kernel<T, false, false>, plane);
         }
-        const bool dist_only = io.dist != nullptr && io.y != nullptr && io.codes == nullptr && io.mask == nullptr &&
-                               io.pmask == nullptr && io.pcodes == nullptr;
         if ((vec || ragged) && pack_only && g.E % 32 == 0)         // whole words of codes: the byte-wise writer
             return vec ? go(quant_flat_kernel<T, VF, MODE, 3, true>) : go(quant_flat_kernel<T, VF, MODE, 3, true, true>);
         if ((vec || ragged) && pack_only)
@@ -1139,6 +1190,14 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
             return vec ? go(quant_flat_kernel<T, VF, MODE, 4>) : go(quant_flat_kernel<T, VF, MODE, 4, false, true>);
         if ((vec || ragged) && pmask_only)
             return vec ? go(quant_flat_kernel<T, VF, MODE, 2>) : go(quant_flat_kernel<T, VF, MODE, 2, false, true>);
+    }
+    if (end) {
+        if constexpr (MODE == MODE_FWD) {
+            if (pack_only) return go(quant_flat_kernel<T, VF, MODE, 1, true, true, true>);
+            if (dist_only) return go(quant_flat_kernel<T, VF, MODE, 4, false, true, true>);
+            if (pmask_only) return go(quant_flat_kernel<T, VF, MODE, 2, false, true, true>);
+        }
+        return go(quant_flat_kernel<T, VF, MODE, 0, false, true, true>);
     }
     if (ragged) return extras ? go(quant_flat_kernel<T, VF, MODE, 1, false, true>) : go(quant_flat_kernel<T, VF, MODE, 0, false, true>);
     if (vec) return extras ? go(quant_flat_kernel<T, VF, MODE, 1>) : go(quant_flat_kernel<T, VF, MODE, 0>);
@@ -1172,7 +1231,7 @@ cudaError_t dequant_strings_bits(const uint32_t* pcodes, T* y, const Geom& g, co
     const uint32_t per_cta = kThreads * 2, grid = (n + per_cta - 1) / per_cta;
     const FastDiv di = make_fastdiv((uint32_t)g.inner), dc = make_fastdiv((uint32_t)g.C);
     auto go = [&](auto kern) {
-        return launch_after(sm_layout(0, (uint64_t)g.E * sizeof(T)), kern, grid, kThreads, 0, st, pcodes, y, n, last, (uint32_t)g.inner,
+        return launch_after(sm_layout(0, (uint64_t)g.E * sizeof(T)), kern, grid, kThreads, 0, st, pcodes, y, n, (uint32_t)(g.E % 8), last, (uint32_t)g.inner,
                             di, dc, s, z);
     };
     return g.inner % 8 == 0 ? go(dequant_strings_kernel<T, BITS, false>) : go(dequant_strings_kernel<T, BITS, true>);
@@ -1243,13 +1302,14 @@ cudaError_t launch_naive(const QuantIO& io, int mode, int dtype, const Geom& g, 
 cudaError_t launch_bwd_packmask(const void* gy, const uint32_t* pmask, void* gx, int dtype, int64_t E,
                                 cudaStream_t st) {
     const int VF = dtype == 0 ? 4 : 8;
-    const bool vec = aligned16(gy) && aligned16(gx) && (E % VF == 0);
+    const bool vec = aligned16(gy) && aligned16(gx) && E >= VF;
     const int64_t units = vec ? E / VF : E;
+    const uint32_t tail = vec ? (uint32_t)(E % VF) : 0u;
     const int64_t per_cta = (int64_t)kThreads * kUnroll;
     const unsigned grid = (unsigned)((units + per_cta - 1) / per_cta);
     auto go = [&](auto kern, auto zero) {
         using T = decltype(zero);
-        return launch_after(sm_layout(0, (uint64_t)E * sizeof(T)), kern, grid, kThreads, 0, st, (const T*)gy, pmask, (T*)gx, E);
+        return launch_after(sm_layout(0, (uint64_t)E * sizeof(T)), kern, grid, kThreads, 0, st, (const T*)gy, pmask, (T*)gx, E - tail, tail);
     };
     if (dtype == 0) return vec ? go(bwd_packmask_kernel<float, 4>, 0.0f) : go(bwd_packmask_kernel<float, 1>, 0.0f);
     const __nv_bfloat16 zero{};
@@ -1277,8 +1337,8 @@ cudaError_t launch_distortion(const void* x, const void* q, int dtype, int64_t E
 
 cudaError_t launch_dequant_packed(const uint32_t* pcodes, void* y, int dtype, const Geom& g, int bits,
                                   const float* s, const float* z, cudaStream_t st) {
-    // strings of 8 codes: planes of at least 8 elements, a whole number of strings, 32-byte (fp32) stores
-    if (g.E % 8 == 0 && g.E < (1ll << 31) && g.inner >= 8 && g.inner < (1ll << 30) && g.C < (1ll << 30) &&
+    // strings of 8 codes: planes of at least 8 elements, 32-byte (fp32) stores
+    if (g.E < (1ll << 31) && g.inner >= 8 && g.inner < (1ll << 30) && g.C < (1ll << 30) &&
         ((uintptr_t)y & (dtype == 0 ? 31 : 15)) == 0)
         return dtype == 0 ? dequant_strings<float>(pcodes, (float*)y, g, bits, s, z, st)
                           : dequant_strings<__nv_bfloat16>(pcodes, (__nv_bfloat16*)y, g, bits, s, z, st);
