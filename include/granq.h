@@ -420,7 +420,7 @@ int granq_host_arena_status(int dtype, const int64_t dims[4], int channel_axis, 
  * 4 = column walk, 5 = cluster-local, 6 = channels-last rows; negative = -status.  Plan 4 covers two kernels, the
  * resident form and the waves: granq_team_geometry() tells which.  The resident form also runs in place of plan 5
  * for x of 96 MB and more (128 MB for fp32 with a gradient) in channels of at least 256 KB.  Where granq_hold_geometry() says
- * so, plans 0 and 3 run as one launch that holds the tensor on chip piece by piece.
+ * so, plans 0, 3 and 5 run as one launch that holds the tensor on chip piece by piece.
  * `launches_out` (HOST, may be NULL) receives the number of kernel launches of that plan.
  */
 int granq_fused_plan(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward,

@@ -151,6 +151,27 @@ HoldPlan prefer_hold(int dtype, const Geom& g, const QuantIO& io, uint32_t flags
     return plan_hold(dtype, g, io, sms);
 }
 
+// In place of the cluster-local plan, where every group is one plane (a group per sample and channel, or a batch of one): a cluster then
+// has one slab to walk, and a thread that keeps a unit column works out its parameters for a single unit; pieces of equal size have tables of
+// them.  Cluster / piece by piece, us: bf16 whose planes are not whole units, forward [64,256,3,3] 49.5 / 13.5, [8,64,7,7] 20.1 / 10.6,
+// [64,64,13,13] 15.6 / 10.4, with gradient [16,784,14,14] 16.4 / 14.5, but [8,8,7,7], 3136 elements, 6.3 / 8.5, packed mask [8,64,7,7] 22.5 / 23.7; of whole units from 8 KB a
+// plane and 2 MB on, with gradient [16,64,112,112] 31.0 / 20.8, forward 24.0 / 18.8, but [64,256,24,24] 16.0 / 18.6, [16,64,56,56] 10.6 / 11.1; with the
+// sums from 0.5 KB on, [64,64,20,20] 13.2 / 11.2, [16,64,56,56] 13.7 / 12.5, packed mask 30.7 / 26.8, but [8,3,64,64] 12.9 / 19.7.  fp32 with the sums, planes of 1.6 KB, 12 MB: [64,200,20,20] 21.6 / 16.5,
+// [32,128,28,28] 14.4 / 13.2, [50,10,112,112] 20.6 / 16.6, but [64,300,14,14] 15.4 / 16.4; without sums a third slower or more.
+// Not in a list, whose cluster-local kernels run beside one another: eight bf16 [16,256,14,14] 34 / 82, [8,16,112,112] 39 / 82.
+HoldPlan hold_over_cluster(int dtype, const Geom& g, const QuantIO& io, uint32_t flags) {
+    HoldPlan none{};
+    const StagedTuning& t = g_tune;
+    if ((flags & (GRANQ_FLAG_FORCE_CLUSTER | GRANQ_FLAG_FORCE_COLWALK)) || t.cl_tile_kb || t.cl_r || t.cl_threads || t.cl_load || t.cl_prefetch ||
+        t.cl_kmul || t.cl_pdl || g.outer != 1 || g.C == 1)
+        return none;
+    const bool sums = io.dist != nullptr;
+    const bool pays = dtype == GRANQ_BF16 ? (g.inner % 8 != 0 ? g.E >= (io.pmask || io.pcodes ? 1 << 16 : 8192)
+                                                              : sums ? g.inner >= 256 : g.inner >= 4096 && g.E >= 1 << 20)
+                                          : sums && g.inner >= 400 && g.E >= 3'000'000;
+    return pays ? prefer_hold(dtype, g, io, flags) : none;
+}
+
 // The workspace set to zero ahead of one cooperative launch, or of range launches.  On the device the clearing kernel, which the launch
 // behind it need not wait for to read on, is 3 us shorter than a memset (with the launch behind it, from a graph, 1.1 / 4.1), but it
 // costs the host 1.5 us more (2.4 / 0.85).  So a call whose kernels take less time than the host needs to make it, and which is not
@@ -256,11 +277,11 @@ int granq_fakequant_bwd(const void* gy, const void* x, int dtype, const int64_t 
 }
 
 // granq_fakequant_fused(); independent: the call shares no memory with those ahead of it on the stream that were made
-// since one that was not (a cluster-local kernel then need not wait for theirs before it starts)
+// since one that was not (a cluster-local kernel then need not wait for theirs before it starts); listed: one of several
 static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_t dims[4], int channel_axis, int group,
                       int bits, void* y, void* gx_opt, float* min_out, float* max_out, uint8_t* codes_opt,
                       uint8_t* mask_opt, float* scale_opt, float* zp_opt, void* workspace, size_t workspace_bytes,
-                      uint32_t flags, void* cuda_stream, bool independent) {
+                      uint32_t flags, void* cuda_stream, bool independent, bool listed) {
     Geom g;
     int64_t G;
     if (!x || !y || !min_out || !max_out || bits < 1 || bits > 8 || !dtype_ok(dtype) ||
@@ -293,12 +314,14 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
     // true for the next call, clear after themselves.
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     kp.zero_status = !zeroed && kp.clears_status;
-    const HoldPlan hp = plan == PLAN_TWO_PASS || plan == PLAN_L2WAVE ? prefer_hold(dtype, g, io, flags) : HoldPlan{};
+    HoldPlan hp{};
+    if (plan == PLAN_TWO_PASS || plan == PLAN_L2WAVE) hp = prefer_hold(dtype, g, io, flags);
+    if (plan == PLAN_CLUSTER && !listed) hp = hold_over_cluster(dtype, g, io, flags);
     bool keeps_zero = plan == PLAN_COLWALK || plan == PLAN_CLUSTER || plan == PLAN_ROWS || hp.ok;
     TeamPlan tp{};
-    if (plan == PLAN_CLUSTER) tp = prefer_team(dtype, g, io, gy_opt != nullptr, flags);
+    if (plan == PLAN_CLUSTER && !hp.ok) tp = prefer_team(dtype, g, io, gy_opt != nullptr, flags);
     cudaError_t e = cudaSuccess;
-    if (plan == PLAN_CLUSTER && !tp.ok) {
+    if (plan == PLAN_CLUSTER && !tp.ok && !hp.ok) {
         if (!zeroed && !kp.clears_status) e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), st);      // the status word
     } else if (!zeroed) {
         e = clear_workspace(ws, g, plan == PLAN_ROWS || hp.ok ? kHostBoundHeld : 0, st);
@@ -309,7 +332,10 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
         cudaError_t r = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, ws.cleared, st);
         return r == cudaSuccess ? launch_quant_flat(io, mode, dtype, g, bits, min_out, max_out, st) : r;
     };
-    if (plan == PLAN_CLUSTER) {
+    if (hp.ok && (e = launch_hold(hp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st)) !=
+                     cudaErrorCooperativeLaunchTooLarge) {
+        // done
+    } else if (plan == PLAN_CLUSTER) {
         e = launch_held(tp, kp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st);
     } else if (plan == PLAN_ROWS) {
         e = launch_rows(io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
@@ -319,9 +345,6 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
         }
     } else if (plan == PLAN_STAGED) {
         e = launch_staged(sp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
-    } else if (hp.ok && (e = launch_hold(hp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st)) !=
-                            cudaErrorCooperativeLaunchTooLarge) {
-        // done
     } else if (plan == PLAN_L2WAVE) {
         keeps_zero = false;
         e = launch_l2wave(lp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
@@ -345,7 +368,7 @@ int granq_fakequant_fused(const void* x, const void* gy_opt, int dtype, const in
                           uint8_t* codes_opt, uint8_t* mask_opt, float* scale_opt, float* zp_opt, void* workspace,
                           size_t workspace_bytes, uint32_t flags, void* cuda_stream) {
     return fused_call(x, gy_opt, dtype, dims, channel_axis, group, bits, y, gx_opt, min_out, max_out, codes_opt, mask_opt,
-                      scale_opt, zp_opt, workspace, workspace_bytes, flags, cuda_stream, false);
+                      scale_opt, zp_opt, workspace, workspace_bytes, flags, cuda_stream, false, false);
 }
 
 size_t granq_packmask_bytes(const int64_t dims[4]) {
@@ -418,7 +441,17 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     kp.zero_status = !zeroed && kp.clears_status;
     cudaError_t e = cudaSuccess;
-    const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
+    HoldPlan hp{};
+    if (kp.ok) hp = hold_over_cluster(dtype, g, io, flags);
+    else if (!cp.ok) hp = prefer_hold(dtype, g, io, flags);
+    const TeamPlan tp = kp.ok && !hp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
+    if (hp.ok) {
+        if (!zeroed) e = clear_workspace(ws, g, kHostBoundHeld, st);
+        if (e != cudaSuccess) return GRANQ_ERR_CUDA;
+        e = launch_hold(hp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
+        if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_status(e);
+        e = cudaSuccess;
+    }
     if (kp.ok) {
         // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
         if (!zeroed && (tp.ok || !kp.clears_status))
@@ -429,13 +462,8 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
         return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     }
-    const HoldPlan hp = cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
-    if (!zeroed) e = clear_workspace(ws, g, hp.ok ? kHostBoundHeld : 0, st);
+    if (!zeroed && !hp.ok) e = clear_workspace(ws, g, 0, st);
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
-    if (hp.ok) {
-        e = launch_hold(hp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
-        if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_status(e);
-    }
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {
@@ -579,7 +607,7 @@ int granq_fakequant_fused_batch(const granq_fused_desc* descs, int n_tensors, in
         if (!independent) first = i;
         const int rc = fused_call(d.x, d.gy_opt, dtype, d.dims, channel_axis, group, d.bits, d.y, d.gx_opt, d.min_out,
                                   d.max_out, nullptr, nullptr, d.scale_opt, d.zp_opt, d.workspace, d.workspace_bytes, flags,
-                                  cuda_stream, independent);
+                                  cuda_stream, independent, n_tensors > 1);
         if (rc != GRANQ_OK) {
             if (failed_opt) *failed_opt = i;
             return rc;
@@ -639,20 +667,22 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
     Workspace ws = carve_workspace(workspace, G);
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     kp.zero_status = !zeroed && kp.clears_status;
-    const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
-    const HoldPlan hp = kp.ok || cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
+    HoldPlan hp{};
+    if (kp.ok) hp = hold_over_cluster(dtype, g, io, flags);
+    else if (!cp.ok) hp = prefer_hold(dtype, g, io, flags);
+    const TeamPlan tp = kp.ok && !hp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
     // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
-    const size_t clear = zeroed ? 0 : !kp.ok || tp.ok ? ws.clear_bytes : kp.clears_status ? 0 : sizeof(uint32_t);
+    const size_t clear = zeroed ? 0 : !kp.ok || tp.ok || hp.ok ? ws.clear_bytes : kp.clears_status ? 0 : sizeof(uint32_t);
     cudaError_t e = launch_clear(workspace, clear, sums_out, st);
     ws.cleared = true;
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
-    if (kp.ok)
-        return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     if (hp.ok) {
         e = launch_hold(hp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
         if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_status(e);
         e = cudaSuccess;
     }
+    if (kp.ok)
+        return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, st));
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {
@@ -718,7 +748,17 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
     const bool zeroed = (flags & GRANQ_FLAG_WORKSPACE_ZEROED) != 0;
     kp.zero_status = !zeroed && kp.clears_status;
     cudaError_t e = cudaSuccess;
-    const TeamPlan tp = kp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
+    HoldPlan hp{};
+    if (kp.ok) hp = hold_over_cluster(dtype, g, io, flags);
+    else if (!cp.ok) hp = prefer_hold(dtype, g, io, flags);
+    const TeamPlan tp = kp.ok && !hp.ok ? prefer_team(dtype, g, io, false, flags) : TeamPlan{};
+    if (hp.ok) {
+        if (!zeroed) e = clear_workspace(ws, g, kHostBoundHeld, st);
+        if (e != cudaSuccess) return GRANQ_ERR_CUDA;
+        e = launch_hold(hp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, g_tune, st);
+        if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_status(e);
+        e = cudaSuccess;
+    }
     if (kp.ok) {
         // the team form needs zeroed keys and counters; of the cluster kernel, the status word where it does not write it
         if (!zeroed && (tp.ok || !kp.clears_status))
@@ -727,13 +767,8 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
         if (e != cudaSuccess) return GRANQ_ERR_CUDA;
         return cuda_status(launch_held(tp, kp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, st));
     }
-    const HoldPlan hp = cp.ok ? HoldPlan{} : prefer_hold(dtype, g, io, flags);
-    if (!zeroed) e = clear_workspace(ws, g, hp.ok ? kHostBoundHeld : 0, st);
+    if (!zeroed && !hp.ok) e = clear_workspace(ws, g, 0, st);
     if (e != cudaSuccess) return GRANQ_ERR_CUDA;
-    if (hp.ok) {
-        e = launch_hold(hp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, g_tune, st);
-        if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_status(e);
-    }
     if (cp.ok) {
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, g_tune, st);
     } else {
@@ -921,9 +956,9 @@ int granq_hold_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
     const QuantIO io = aligned_io(backward, packed != 0);
     const HoldPlan p = plan_hold(dtype, g, io, sm_count);
     if (!p.ok || !p.whole) return GRANQ_ERR_UNSUPPORTED;
-    const int plan = packed ? (plan_cluster(dtype, g, io, false, g_tune).ok || plan_colwalk(dtype, g, io, g_tune).ok ? PLAN_COLWALK : PLAN_TWO_PASS)
+    const int plan = packed ? (plan_cluster(dtype, g, io, false, g_tune).ok ? PLAN_CLUSTER : plan_colwalk(dtype, g, io, g_tune).ok ? PLAN_COLWALK : PLAN_TWO_PASS)
                             : choose_plan(dtype, g, io, backward, 0, nullptr, nullptr, nullptr, nullptr);
-    const bool taken = (plan == PLAN_TWO_PASS || plan == PLAN_L2WAVE) && hold_allowed(0);
+    const bool taken = ((plan == PLAN_TWO_PASS || plan == PLAN_L2WAVE) && hold_allowed(0)) || (plan == PLAN_CLUSTER && hold_over_cluster(dtype, g, io, 0).ok);
     const int64_t v[4] = {p.ctas, p.share, p.held, taken ? 1 : 0};
     for (int i = 0; i < 4; ++i) out[i] = v[i];
     return GRANQ_OK;

@@ -122,6 +122,58 @@ def test_elements_behind_the_last_whole_unit(b, shape, mode, dtype):
                 assert_same_string(got.packed_codes, orc.pack_codes(orc.fused(x, code_bits, group_mode=mode).codes, code_bits))
 
 
+@pytest.mark.parametrize("dtype,shape,mode,calls", [
+    ("bf16", (8, 16, 8, 8), 1, ""),                      # planes of whole units, too short
+    ("bf16", (8, 8, 11, 12), 1, "fs"),                   # 8448 elements in planes that are not
+    ("bf16", (8, 7, 11, 12), 1, ""),                     # 7392
+    ("bf16", (64, 256, 3, 3), 1, "fsm"),                 # planes of little more than a unit
+    ("bf16", (1, 304, 21, 21), 0, "fsm"),                # a batch of one
+    ("bf16", (4, 5, 16, 16), 1, "s"),
+    ("bf16", (8, 3, 64, 64), 1, "s"),
+    ("bf16", (4, 17, 128, 128), 1, "fsm"),
+    ("f32", (8, 8, 11, 13), 1, ""),
+    ("f32", (60, 128, 20, 20), 1, "s"),
+    ("f32", (7, 1072, 20, 20), 1, "s"),
+], ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_groups_of_one_plane(b, dtype, shape, mode, calls):
+    """Where the launch that holds pieces stands in for the cluster-local one: f forward and with a gradient, s sums, m packed mask
+    and codes; both give the oracle's bits, also where the cooperative launch is refused."""
+    x, gy = make_case(shape, seed=sum(shape), dtype=dtype)
+    ref = orc.fused(x, 5, gy=gy, group_mode=mode)
+    xd, gyd = to_dev(x), to_dev(gy)
+    assert b.fused_plan(b.BF16 if dtype == "bf16" else b.F32, shape, group=mode)[0] == b.PLAN_CLUSTER
+    assert takes(b, dtype, shape, mode) == takes(b, dtype, shape, mode, with_backward=True) == ("f" in calls)
+    assert takes(b, dtype, shape, mode, packed=True) == ("m" in calls and x.size % 32 == 0)
+    ws = b.make_workspace(xd, group=mode, zeroed=True)
+    clean = lambda: b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
+    for flags in (0, b.FLAG_WORKSPACE_ZEROED, b.FLAG_FORCE_CLUSTER):
+        new = lambda: b.FakeQuantOut(workspace=ws) if flags == b.FLAG_WORKSPACE_ZEROED else b.FakeQuantOut()
+        got = b.granq_fakequant_fused(xd, 5, gy=gyd, group=mode, out=new(), want_params=True, flags=flags)
+        assert clean()
+        assert_parity(got, ref, shape, 1, mode, backward=True)
+        assert_parity(b.granq_fakequant_fused(xd, 5, group=mode, out=new(), flags=flags), ref, shape, 1, mode, backward=False)
+        got = b.granq_fakequant_fused_stats(xd, 5, group=mode, out=new(), flags=flags)
+        assert clean()
+        assert_parity(got, ref, shape, 1, mode, backward=False)
+        # fp32 inside a pack, fp64 beyond: about 8 roundings of 2^-24 of a sum of same-signed terms
+        assert np.allclose(to_np(got.sums), orc.distortion_sums(x, ref.y), rtol=1e-6, atol=0)
+        got = b.granq_fakequant_fused_fwd_packmask(xd, 5, group=mode, out=new(), flags=flags)
+        assert_parity(got, ref, shape, 1, mode, backward=False)
+        assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+        if not flags & b.FLAG_FORCE_CLUSTER:
+            got = b.granq_quantize_packed_fused(xd, 5, group=mode, out=new(), flags=flags)
+            assert clean()
+            assert_same_string(got.packed_codes, orc.pack_codes(ref.codes, 5))
+    try:
+        b.tune(b.KNOB_TEST_COOP_CTAS, 1)
+        assert_parity(b.granq_fakequant_fused(xd, 5, gy=gyd, group=mode), ref, shape, 1, mode, backward=True)
+        assert_parity(b.granq_fakequant_fused_stats(xd, 5, group=mode), ref, shape, 1, mode, backward=False)
+        assert_same_string(b.granq_fakequant_fused_fwd_packmask(xd, 5, group=mode).packed_mask, orc.pack_mask(ref.mask))
+        assert_same_string(b.granq_quantize_packed_fused(xd, 5, group=mode).packed_codes, orc.pack_codes(ref.codes, 5))
+    finally:
+        b.tune(b.KNOB_TEST_COOP_CTAS, 0)
+
+
 @pytest.mark.parametrize("dtype,shape", [("f32", (96, 128, 28, 28)), ("bf16", (192, 128, 28, 28))])
 def test_one_group_beyond_what_stays_on_chip(b, dtype, shape):
     x, gy = make_case(shape, seed=3, dtype=dtype)
