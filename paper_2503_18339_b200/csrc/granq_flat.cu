@@ -941,7 +941,8 @@ __global__ void __launch_bounds__(kThreads) distortion_kernel(const T* __restric
 // Bound by the stores: [128,144,56,56], 231 MB written from 36 MB of 5-bit codes, 92 -> 45 us
 // (5.9 TB/s; a thread per 16 bytes with two 32-bit divisions took 171 instructions for 4 elements).  A block per 512
 // strings rather than a persistent grid, so that the stores go out in the order of memory: [128,96,112,112] 133 -> 110 us.
-template <typename T, int BITS, bool RAGGED>
+// END: there is such a tail (in a form of its own: bf16 [26,920,45,44], 6 bits, 31.1 without, 31.8 with the test for it).
+template <typename T, int BITS, bool RAGGED, bool END>
 __global__ void __launch_bounds__(kThreads) dequant_strings_kernel(const uint32_t* __restrict__ pcodes, T* __restrict__ y,
                                                                    uint32_t nstrings, uint32_t tail, uint32_t last_word, uint32_t inner,
                                                                    FastDiv div_inner, FastDiv div_C,
@@ -949,7 +950,7 @@ __global__ void __launch_bounds__(kThreads) dequant_strings_kernel(const uint32_
     after_the_kernel_ahead();
     constexpr uint32_t kField = (1u << BITS) - 1u;
     constexpr int kFly = 2;
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x < tail) {
+    if (END && blockIdx.x == gridDim.x - 1 && threadIdx.x < tail) {
         const uint64_t bit = ((uint64_t)nstrings * 8 + threadIdx.x) * BITS;
         const uint32_t w0 = (uint32_t)(bit >> 5), c = __funnelshift_r(__ldg(pcodes + w0), __ldg(pcodes + min(w0 + 1, last_word)), (uint32_t)bit & 31);
         store_scalar(y + (size_t)nstrings * 8 + threadIdx.x, __fmul_rn(__ldg(s + div_C.d - 1), __fsub_rn((float)(c & kField), __ldg(z + div_C.d - 1))));
@@ -1234,7 +1235,8 @@ cudaError_t dequant_strings_bits(const uint32_t* pcodes, T* y, const Geom& g, co
         return launch_after(sm_layout(0, (uint64_t)g.E * sizeof(T)), kern, grid, kThreads, 0, st, pcodes, y, n, (uint32_t)(g.E % 8), last, (uint32_t)g.inner,
                             di, dc, s, z);
     };
-    return g.inner % 8 == 0 ? go(dequant_strings_kernel<T, BITS, false>) : go(dequant_strings_kernel<T, BITS, true>);
+    if (g.inner % 8 == 0) return go(dequant_strings_kernel<T, BITS, false, false>);
+    return g.E % 8 == 0 ? go(dequant_strings_kernel<T, BITS, true, false>) : go(dequant_strings_kernel<T, BITS, true, true>);
 }
 
 template <typename T>
