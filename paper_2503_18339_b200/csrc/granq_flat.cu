@@ -859,13 +859,13 @@ __global__ void __launch_bounds__(kThreads) naive_quant_kernel(const T* __restri
 // layer's), which a stream of a wave or two is slower beside (packed mask and backward, us, with / without: bf16 [128,960,7,7] 26.0 / 21.2,
 // fp32 [25,856,14,14] 21.6 / 19.2, [41,1896,15,16] 60.8 / 60.3; 26 shapes 0.98).
 // V = elements per thread and step: a 16-byte pack when the pointers allow it, else 1.  `tail` elements behind the E of whole
-// packs are the first threads' of the last block.
-template <typename T, int V>
+// packs are the first threads' of the last block, in a form of its own (END: the test for them took 0.1 us of 2.7).
+template <typename T, int V, bool END>
 __global__ void __launch_bounds__(kThreads) bwd_packmask_kernel(const T* __restrict__ gy,
                                                                 const uint32_t* __restrict__ pmask,
                                                                 T* __restrict__ gx, int64_t E, uint32_t tail) {
     wait_for_the_kernel_ahead();      // and no word to the kernel behind
-    if (V > 1 && blockIdx.x == gridDim.x - 1 && threadIdx.x < tail) {
+    if (END && blockIdx.x == gridDim.x - 1 && threadIdx.x < tail) {
         const int64_t at = E + threadIdx.x;
         store_scalar(gx + at, (__ldg(pmask + (at >> 5)) >> (uint32_t)(at & 31)) & 1u ? load_scalar(gy + at) : 0.0f);
     }
@@ -1313,9 +1313,12 @@ cudaError_t launch_bwd_packmask(const void* gy, const uint32_t* pmask, void* gx,
         using T = decltype(zero);
         return launch_after(sm_layout(0, (uint64_t)E * sizeof(T)), kern, grid, kThreads, 0, st, (const T*)gy, pmask, (T*)gx, E - tail, tail);
     };
-    if (dtype == 0) return vec ? go(bwd_packmask_kernel<float, 4>, 0.0f) : go(bwd_packmask_kernel<float, 1>, 0.0f);
-    const __nv_bfloat16 zero{};
-    return vec ? go(bwd_packmask_kernel<__nv_bfloat16, 8>, zero) : go(bwd_packmask_kernel<__nv_bfloat16, 1>, zero);
+    auto by_type = [&](auto zero) {
+        using T = decltype(zero);
+        if (!vec) return go(bwd_packmask_kernel<T, 1, false>, zero);
+        return tail ? go(bwd_packmask_kernel<T, Pack<T>::V, true>, zero) : go(bwd_packmask_kernel<T, Pack<T>::V, false>, zero);
+    };
+    return dtype == 0 ? by_type(0.0f) : by_type(__nv_bfloat16{});
 }
 
 cudaError_t launch_distortion(const void* x, const void* q, int dtype, int64_t E, double* sums, cudaStream_t st) {
