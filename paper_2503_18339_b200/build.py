@@ -60,13 +60,20 @@ def _which_nvcc() -> str:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile csrc/*.cu (one object per source, in parallel) and link libgranq.so beside this file, and _host.so with
-    it; returns the library's path.  Objects are kept in _build/ and reused while their source and the headers are older."""
+    it; returns the library's path.  Objects are kept in _build/ and reused while their source and the headers are older.
+    The library needs nvcc alone.  Where _host.so cannot be built (no C++ compiler, no torch, no Python headers) one line says
+    so and the binding marshals its calls in Python."""
     with ThreadPoolExecutor(max_workers=1) as beside:
         host = beside.submit(_build_host) if force or _host_stale() else None
         if force or _stale():
             _build_lib(force, verbose)
-        if host is not None:
-            host.result()
+        try:
+            if host is not None:
+                host.result()
+        except Exception as e:
+            if os.path.exists(HOST):
+                os.remove(HOST)          # of an older source, which may call the library otherwise than it is now
+            print(f"_host.so has not been built, the binding's calls are marshalled in Python: {type(e).__name__}: {e}", file=sys.stderr)
     return LIB
 
 
