@@ -9,15 +9,20 @@ from __future__ import annotations
 import ctypes
 import functools
 import os
+import warnings
 from dataclasses import dataclass
 from typing import Optional
 
 import torch
 
+from .build import host_record
+
 try:
     from . import _host as _host_calls          # granq_host.cpp: the plain case of the calls below in native code, see lib()
-except ImportError:              # not built: the same calls, marshalled here
+except ImportError as e:         # not built: the same calls, marshalled here
     _host_calls = None
+    if os.path.exists(os.path.join(os.path.dirname(os.path.abspath(__file__)), "_host.so")):
+        warnings.warn(f"_host.so cannot be loaded, calls are marshalled in Python: {e}")
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libgranq.so")
@@ -170,7 +175,10 @@ def lib() -> ctypes.CDLL:
         L.granq_fakequant_fused_fwd_packmask.argtypes = [vp, ci, i64p, ci, ci, ci, vp, vp, vp, vp, vp, vp, vp, sz,
                                                          u32, vp]
         _lib = L
-        if _host_calls is not None:
+        if _host_calls is not None and getattr(_host_calls, "built_for", None) != host_record():
+            warnings.warn(f"_host.so was built for {getattr(_host_calls, 'built_for', 'unknown versions')} and this is {host_record()}: "
+                          "calls are marshalled in Python until it is built again")
+        elif _host_calls is not None:
             _host_calls.setup({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in EXPORTS}, FakeQuantOut, GranqError)
             _native = _host_calls
     return _lib

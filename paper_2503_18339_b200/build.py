@@ -1,7 +1,6 @@
 """In-tree build of the GranQ CUDA library for sm_100a (nvcc cross-compiles without a GPU) and of the binding's native calls."""
 from __future__ import annotations
 
-import importlib.util
 import os
 import shutil
 import subprocess
@@ -16,6 +15,7 @@ LIB = os.path.join(HERE, "libgranq.so")
 HOST = os.path.join(HERE, "_host.so")               # the binding's calls in native code, an extension module of this package
 HOST_SOURCE = os.path.join(CSRC, "granq_host.cpp")
 OBJ_DIR = os.path.join(HERE, "_build")
+HOST_RECORD = os.path.join(OBJ_DIR, "host_record")  # host_record() of that module, which holds the same text
 SOURCES = ["granq_api.cu", "granq_flat.cu", "granq_staged.cu", "granq_l2wave.cu", "granq_colwalk.cu", "granq_colteam.cu",
            "granq_cluster.cu", "granq_hold.cu", "granq_accumulate.cu", "granq_rows.cu", "granq_weights.cu", "granq_selftest.cu", "granq_noalloc.cu"]
 HEADERS = ["granq_device.cuh", "granq_internal.h"]
@@ -38,19 +38,35 @@ def _stale() -> bool:
     return any(_newer(d, t) for d in [os.path.join(CSRC, f) for f in SOURCES] + _deps())
 
 
+def host_record() -> str:
+    """What _host.so depends on besides its source: it reads torch's objects and Python's in place."""
+    import torch
+    return f"torch {torch.__version__}, cxx11 abi {int(torch.compiled_with_cxx11_abi())}, python {sys.version_info[0]}.{sys.version_info[1]}"
+
+
 def _host_stale() -> bool:
-    return not os.path.exists(HOST) or any(_newer(d, os.path.getmtime(HOST)) for d in (HOST_SOURCE, os.path.join(INCLUDE, "granq.h")))
+    try:
+        with open(HOST_RECORD) as f:
+            same = f.read() == host_record()
+    except (OSError, ImportError):
+        same = False
+    return not same or not os.path.exists(HOST) or any(_newer(d, os.path.getmtime(HOST)) for d in (HOST_SOURCE, os.path.join(INCLUDE, "granq.h")))
 
 
 def _build_host() -> None:
-    torch = os.path.dirname(importlib.util.find_spec("torch").origin)
+    import torch
+    record, home = host_record(), os.path.dirname(torch.__file__)
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_which_nvcc()))), "include")
     tmp = HOST + f".tmp{os.getpid()}"
     subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", HOST_SOURCE, "-o", tmp,
-                           f"-I{torch}/include", f"-I{torch}/include/torch/csrc/api/include", f"-I{cuda}",
-                           f"-I{sysconfig.get_paths()['include']}", f"-L{torch}/lib", "-ltorch", "-ltorch_cpu", "-ltorch_python",
+                           f'-DGRANQ_HOST_RECORD="{record}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+                           f"-I{home}/include", f"-I{home}/include/torch/csrc/api/include", f"-I{cuda}",
+                           f"-I{sysconfig.get_paths()['include']}", f"-L{home}/lib", "-ltorch", "-ltorch_cpu", "-ltorch_python",
                            "-lc10", "-lc10_cuda"])
     os.replace(tmp, HOST)
+    os.makedirs(OBJ_DIR, exist_ok=True)
+    with open(HOST_RECORD, "w") as f:
+        f.write(record)
 
 
 def _which_nvcc() -> str:

@@ -383,4 +383,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_host", nullptr, -1, methods};
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__host() { return PyModule_Create(&module); }
+// built_for: the versions whose objects are taken apart here, which binding.py compares before it calls anything
+PyMODINIT_FUNC PyInit__host() {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", GRANQ_HOST_RECORD)) Py_CLEAR(m);
+    return m;
+}
