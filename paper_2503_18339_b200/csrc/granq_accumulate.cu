@@ -429,10 +429,11 @@ struct PArgs : AArgs {
     uint32_t VP;              // rows of one sample: P, or P rounded up to whole strings of 8 pixels
     uint32_t vrows;           // rows of the whole batch
     FastDiv div_vp;
+    uint32_t expected;        // arrivals that complete a stage of codes: the four warps of a producer group
 };
 
 struct PBars {
-    uint64_t a_full[kPStages], a_empty[kPStages], acc_full[8], acc_empty[8], b_full[kPKBlocks];
+    uint64_t a_full[kPStages], a_empty[kPStages], acc_full[8], acc_empty[8], b_full[kPKBlocks], drained;
 };
 
 template <int BN, bool NHWC>
@@ -465,7 +466,7 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
 
     if (tid == 0) {
         for (int s = 0; s < kPStages; ++s) {
-            a_mbar_init(&bars.a_full[s], 4);                 // one arrival per warp of a producer group
+            a_mbar_init(&bars.a_full[s], a.expected);        // one arrival per warp of a producer group
             a_mbar_init(&bars.a_empty[s], 1);
         }
         for (int b = 0; b < kAcc; ++b) {
@@ -473,6 +474,7 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
             a_mbar_init(&bars.acc_empty[b], 4);     // one arrival per warp of the epilogue group that reads it out
         }
         for (int kb = 0; kb < kPKBlocks; ++kb) a_mbar_init(&bars.b_full[kb], 1);
+        a_mbar_init(&bars.drained, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -778,6 +780,16 @@ accumulate_persistent_kernel(const __grid_constant__ CUtensorMap map_hi, const _
                 }
                 if (ok) a_commit(&bars.acc_full[buf]);       // the accumulator is final when this arrives
             }
+            if (!ok) {
+                // Given up: the weights may still be on their way into shared memory, and MMAs that were issued still read it and
+                // write tensor memory, which is freed below.  Both are waited for (bounded, the other threads' giving up aside).
+                auto settle = [&](uint64_t* bar) {
+                    for (uint32_t i = 0; i < kASpin && !a_mbar_try_wait(bar, 0); ++i) {}
+                };
+                a_commit(&bars.drained);
+                for (int kb = 0; kb < kblocks; ++kb) settle(&bars.b_full[kb]);
+                settle(&bars.drained);
+            }
         }
         __syncwarp();
     } else {
@@ -1054,7 +1066,8 @@ extern "C" int granq_accumulate_codes(const uint32_t* packed_codes, const int64_
     args.O = out_channels;
     args.bits = bits;
     args.kblocks = kblocks;
-    args.spin_limit = kASpin;
+    args.spin_limit = g_tune.spin_limit > 0 ? (uint32_t)g_tune.spin_limit : kASpin;
+    args.expected = 4 + (uint32_t)std::max(g_tune.extra_arrivals, 0);
     args.stages = std::min(args.kblocks, kAStages);
     // NCHW: whole strings of 8 pixels per sample, so that none reaches into the next one: at [128,256,14,14] such strings took most of
     // the expansion's instructions

@@ -8,9 +8,9 @@
 
 using namespace granq;
 
-namespace {
+StagedTuning granq::g_tune = {};
 
-StagedTuning g_tune = {};
+namespace {
 
 bool dtype_ok(int dtype) { return dtype == GRANQ_F32 || dtype == GRANQ_BF16; }
 size_t elt_size(int dtype) { return dtype == GRANQ_F32 ? 4 : 2; }

@@ -189,6 +189,7 @@ struct StagedTuning {
     int col_team;         // column-walk plan: 1 = resident form wherever it can, 2 = L2 waves only
     int coop_ctas;        // test hook: launch_cooperative() refuses more CTAs than this
 };
+extern StagedTuning g_tune;      // what granq_tune() sets
 // A cooperative launch that may be refused: every CTA has to be resident at once, and where the GPU is shared out (a
 // partition, a limit on the SMs of a process) fewer are than its attributes say.  cudaErrorCooperativeLaunchTooLarge,
 // with nothing enqueued and no error left behind, tells the caller to take a plan that needs no such launch.

@@ -155,6 +155,34 @@ def test_accumulate_from_the_library_s_own_packed_codes(b):
     assert np.all(np.abs(got.cpu().numpy().astype(np.float64) - ref) <= tol)
 
 
+@pytest.mark.parametrize("channels_last", [False, True], ids=["nchw", "nhwc"])
+@pytest.mark.parametrize("c", [64, 300, 512], ids=lambda c: f"{c}in")
+def test_accumulate_gives_up_and_works_again(b, c, channels_last):
+    """A stage of codes that is never complete: every wait runs out, with weights of the further K blocks (at most 5 of 5, 7 of 8)
+    still to be waited for, the status says so, and the next call on the same workspace is right."""
+    if channels_last and c > 448:
+        c = 448                                   # the most whose weights are resident beside the staging tiles
+    rng = np.random.default_rng(c)
+    codes = rng.integers(0, 16, (3, c, 9, 7)).astype(np.uint8)
+    src = np.ascontiguousarray(codes.transpose(0, 2, 3, 1)) if channels_last else codes
+    s, z = np.ones(c, np.float32), np.zeros(c, np.float32)
+    w = rng.integers(-3, 4, (40, c)).astype(np.float32)
+    args = (packed_words(src, 4), src.shape, 4, torch.from_numpy(s).cuda(), torch.from_numpy(z).cuda(), torch.from_numpy(w).cuda())
+    how = dict(channel_axis=3 if channels_last else 1)
+    try:
+        b.tune(b.KNOB_TEST_EXTRA_ARRIVALS, 1)
+        b.tune(b.KNOB_SPIN_LIMIT, 200)
+        _, ws = b.granq_accumulate_codes(*args, **how)
+        assert b.workspace_status(ws) == b.ERR_TIMEOUT
+    finally:
+        b.tune(b.KNOB_TEST_EXTRA_ARRIVALS, 0)
+        b.tune(b.KNOB_SPIN_LIMIT, 0)
+    y, ws = b.granq_accumulate_codes(*args, workspace=ws, **how)
+    assert b.workspace_status(ws) == b.OK
+    y = y.cpu().numpy().transpose(0, 3, 1, 2) if channels_last else y.cpu().numpy()
+    assert np.array_equal(y, np.einsum("oc,nchw->nohw", w, codes.astype(np.float32)))      # whole numbers below 2^24: exact
+
+
 def test_accumulate_argument_errors(b):
     x = torch.zeros(4, dtype=torch.int32, device="cuda")
     f = torch.zeros(8, device="cuda")
