@@ -1,5 +1,5 @@
 """The build on the CPU: the library does not depend on the binding's native calls, and those are not used with another torch or
-Python than they were built for."""
+Python than they were built for; what the binding hands to them."""
 import ctypes
 import os
 import sys
@@ -82,3 +82,19 @@ def test_native_calls_of_other_versions_are_built_again(elsewhere, monkeypatch):
     with open(build.HOST_RECORD, "w") as f:
         f.write(build.host_record())
     assert not build._host_stale()
+
+
+@pytest.mark.parametrize("want", [None, False, True, 0, 1, "yes"])
+def test_want_params_is_a_truth_value(monkeypatch, want):
+    import torch
+    asked = []
+    spy = lambda name: lambda *a: asked.append((name, a)) or "answered"
+    monkeypatch.setattr(binding, "_native", types.SimpleNamespace(fused_call=spy("fused"), fwd_packmask_call=spy("fwd_packmask")))
+    x, g = torch.zeros(1, 1, 2, 2), torch.zeros(1)
+    for call in (lambda: binding.granq_fakequant_fused(x, 4, want_params=want),
+                 lambda: binding.granq_fakequant_fused_fwd_packmask(x, 4, want_params=want),
+                 lambda: binding.granq_fakequant_fused_stats(x, 4, want_params=want),
+                 lambda: binding.granq_fakequant_fwd_packmask(x, 4, g, g, want_params=want)):
+        assert call() == "answered"
+    at = {"fused": 7, "fwd_packmask": 8}
+    assert [a[at[name]] for name, a in asked] == [int(bool(want))] * 4
