@@ -858,14 +858,16 @@ __global__ void __launch_bounds__(kThreads) naive_quant_kernel(const T* __restri
 // persistent grid).  The kernel behind is not let start beside it: that is mostly one that takes an SM's shared memory (the next
 // layer's), which a stream of a wave or two is slower beside (packed mask and backward, us, with / without: bf16 [128,960,7,7] 26.0 / 21.2,
 // fp32 [25,856,14,14] 21.6 / 19.2, [41,1896,15,16] 60.8 / 60.3; 26 shapes 0.98).
-// V = elements per thread and step: a 16-byte pack when the pointers allow it, else 1.  `tail` elements behind the E of whole
-// packs are the first threads' of the last block, in a form of its own (END: the test for them took 0.1 us of 2.7).
+// V = elements per thread and step: a 16-byte pack when the pointers allow it, else 1.  What is left behind the whole packs
+// is the first threads' of the last block, in a form of its own (END: the test for it took 0.1 us of 2.7).  Four arguments of
+// 8 bytes: with a fifth a launch cost the host 0.35 us more (calls one after another, 16 KB tensors: 2.73 -> 2.38 us).
 template <typename T, int V, bool END>
 __global__ void __launch_bounds__(kThreads) bwd_packmask_kernel(const T* __restrict__ gy,
                                                                 const uint32_t* __restrict__ pmask,
-                                                                T* __restrict__ gx, int64_t E, uint32_t tail) {
+                                                                T* __restrict__ gx, int64_t all) {
     wait_for_the_kernel_ahead();      // and no word to the kernel behind
-    if (END && blockIdx.x == gridDim.x - 1 && threadIdx.x < tail) {
+    const int64_t E = END ? all - all % V : all;
+    if (END && blockIdx.x == gridDim.x - 1 && threadIdx.x < (uint32_t)(all - E)) {
         const int64_t at = E + threadIdx.x;
         store_scalar(gx + at, (__ldg(pmask + (at >> 5)) >> (uint32_t)(at & 31)) & 1u ? load_scalar(gy + at) : 0.0f);
     }
@@ -1301,17 +1303,21 @@ cudaError_t launch_naive(const QuantIO& io, int mode, int dtype, const Geom& g, 
     return naive_t<__nv_bfloat16, MODE_BOTH>(io, g, bits, kmin, kmax, lo, hi, st, launches);
 }
 
+// With elements behind the last whole pack, scalar loads up to here: a small call ends sooner with more blocks of less each.
+// Scalar / packs, us from a graph: [3,31,25,25] 1.0 / 1.35; fp32 [9,301,15,15], 0.6 M, 1.5 / 1.7, [21,251,15,15], 1.2 M, 1.94 / 2.02,
+// [33,301,15,15], 2.2 M, 3.45 / 3.25; bf16 1.5 / 1.4, 1.9 / 1.6, 2.9 / 2.0.
+constexpr int64_t kTailElements[2] = {1'500'000, 500'000};
+
 cudaError_t launch_bwd_packmask(const void* gy, const uint32_t* pmask, void* gx, int dtype, int64_t E,
                                 cudaStream_t st) {
     const int VF = dtype == 0 ? 4 : 8;
-    const bool vec = aligned16(gy) && aligned16(gx) && E >= VF;
+    const bool tail = E % VF != 0, vec = aligned16(gy) && aligned16(gx) && (!tail || E >= kTailElements[dtype == 0 ? 0 : 1]);
     const int64_t units = vec ? E / VF : E;
-    const uint32_t tail = vec ? (uint32_t)(E % VF) : 0u;
     const int64_t per_cta = (int64_t)kThreads * kUnroll;
     const unsigned grid = (unsigned)((units + per_cta - 1) / per_cta);
     auto go = [&](auto kern, auto zero) {
         using T = decltype(zero);
-        return launch_after(sm_layout(0, (uint64_t)E * sizeof(T)), kern, grid, kThreads, 0, st, (const T*)gy, pmask, (T*)gx, E - tail, tail);
+        return launch_after(sm_layout(0, (uint64_t)E * sizeof(T)), kern, grid, kThreads, 0, st, (const T*)gy, pmask, (T*)gx, E);
     };
     auto by_type = [&](auto zero) {
         using T = decltype(zero);

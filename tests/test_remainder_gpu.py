@@ -20,7 +20,8 @@ SHAPES = [
     ((33, 7, 2, 5), 0),          # planes of little more than a unit
     ((9, 2001, 3, 3), 0),        # more groups, and planes of a tile, than the tables hold
     ((21, 379, 7, 7), 0),
-    ((13, 13, 93, 93), 0),
+    ((13, 13, 93, 93), 0),       # (of bf16, the way back from the mask by packs)
+    ((13, 14, 93, 97), 0),       # (of fp32 too)
     ((7, 3, 2, 3), 0),           # planes of less than a unit of bf16: the scalar forms
 ]
 
