@@ -1086,6 +1086,24 @@ int range_rows_ctas() {
     return sm_count() * 4;
 }
 
+// With elements behind the last whole pack: where scalar loads are faster than packs.  In planes of a few packs every pack of the
+// vector path straddles two planes, each lane of a warp with a group of its own, two updates a pack; scalars have one update an element,
+// and wait for one another's atomics when a group's elements are many.  Scalar / packs, us: bf16 [301,33,3,3] 29 / 60, 1101 of them 58 / 61,
+// 1684 86 / 61, [301,501,3,3] 38 / 62, [1746,509,3,3] 198 / 134; planes of 15 [451,33,3,5] 31 / 41, [701,33,3,5] 45 / 40, of 25 [301,33,5,5]
+// 25 / 27, [451,33,5,5] 37 / 28, of 49 no more; fp32 [301,33,1,5] 39 / 52, [1101,33,1,5] 61 / 52, [451,33,3,3] 30 / 32, [701,33,3,3] 42 / 32, of 15 25 / 23.
+// Of a few channels the lanes of a warp share groups again: bf16 [407,5,3,3] 27 / 16, [301,9,3,3] 29 / 25, [301,13,3,3] 29 / 33; fp32 29 / 17,
+// 27 / 23, 27 / 29.
+// Of a group per plane, whose atomics meet nobody: bf16 [1001,901,3,3] 82 / 137, fp32 83 / 117, planes of 25 125 / 134 and 126 / 153, but 126 K groups
+// fp32 of 15 to 25 as fast.  Of a few thousand elements in short planes [7,5,5,5] 5.2 / 9.5, [7,61,3,5] fp32 18 / 21.
+template <typename T>
+bool scalar_range(const Geom& g) {
+    const int64_t channel = g.outer * g.inner * (int64_t)sizeof(T);      // its bytes
+    const bool few = g.inner < (sizeof(T) == 4 ? 12 : 32);
+    if (g.E < (g.C < 12 ? 4096 : 8192) && g.inner < 64) return true;
+    if (g.outer == 1) return few || (g.inner < 32 && g.C > 200'000);
+    return few && g.C >= 12 && channel <= 18'432 && channel * g.C <= 1 << 22;
+}
+
 template <typename T>
 cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t* kmax, const RangeEnd& end, int layout, cudaStream_t st) {
     FlatGeom f = make_flat(g);
@@ -1093,7 +1111,7 @@ cudaError_t range_flat_t(const void* x, const Geom& g, uint32_t* kmin, uint32_t*
     bool vec = aligned16(x) && (g.inner % VF == 0);
     int grid = flat_grid(f);
     const bool rows_ok = aligned16(x) && g.inner >= VF && g.E < (1ll << 31) &&
-                         g.C < (1ll << 30) && g.inner < (1ll << 30);
+                         g.C < (1ll << 30) && g.inner < (1ll << 30) && (g.E % VF == 0 || !scalar_range<T>(g));
     // columns: slabs of whole units, at least a batch of them to walk, planes shorter than a row of the vector path or
     // not whole units
     if (rows_ok && (g.C * g.inner) % VF == 0 && g.outer >= 8 && (!vec || g.inner / VF < 128)) {

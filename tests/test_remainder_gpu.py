@@ -20,6 +20,9 @@ SHAPES = [
     ((33, 7, 2, 5), 0),          # planes of little more than a unit
     ((9, 2001, 3, 3), 0),        # more groups, and planes of a tile, than the tables hold
     ((21, 379, 7, 7), 0),
+    ((1291, 15, 3, 3), 0),       # short planes, whose range takes packs from here on
+    ((301, 33, 3, 3), 0),        # ... and scalars up to here
+    ((2, 1501, 7, 7), 0),        # packs again, more groups than a block keeps
     ((13, 13, 93, 93), 0),       # (of bf16, the way back from the mask by packs)
     ((13, 14, 93, 97), 0),       # (of fp32 too)
     ((7, 3, 2, 3), 0),           # planes of less than a unit of bf16: the scalar forms
