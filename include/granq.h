@@ -468,6 +468,14 @@ int granq_rows_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
                         int64_t out[4]);
 
 /*
+ * Host-only query: how granq_fakequant_fwd() and granq_fakequant_fwd_packmask() (`packed_mask` != 0) walk a tensor by columns on a
+ * device with `sm_count` SMs (no counterpart in the paper), 16-byte aligned and with no other outputs.
+ * out = { slabs side by side in a row, blocks of 256 16-byte units across it, rows, rows a block walks }.
+ * Returns GRANQ_ERR_UNSUPPORTED where those calls take tiles of the tensor instead.
+ */
+int granq_forward_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int packed_mask, int sm_count, int64_t out[4]);
+
+/*
  * Host-only query: how the launch that holds a tensor on chip piece by piece would cut this tensor on a device with `sm_count` SMs;
  * `packed`: for packed masks and packed codes (forward only) rather than for y and gx.
  * out = { CTAs, 16-byte units of one CTA, of those kept in shared memory (the others are read again), 1 if

@@ -52,7 +52,7 @@ EXPORTS = [
     "granq_quantize_packed", "granq_dequantize_packed", "granq_cluster_geometry", "granq_distortion_stats",
     "granq_accumulate_workspace_bytes", "granq_accumulate_codes", "granq_fakequant_fused_batch",
     "granq_quantize_packed_fused", "granq_rows_geometry", "granq_team_geometry", "granq_batch_geometry",
-    "granq_hold_geometry",
+    "granq_forward_geometry", "granq_hold_geometry",
 ]
 NOALLOC_MAX_GROUPS = 32768
 
@@ -137,6 +137,8 @@ def lib() -> ctypes.CDLL:
         L.granq_team_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, i64p]
         L.granq_hold_geometry.restype = ci
         L.granq_hold_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, ci, i64p]
+        L.granq_forward_geometry.restype = ci
+        L.granq_forward_geometry.argtypes = [ci, i64p, ci, ci, ci, ci, i64p]
         L.granq_batch_geometry.restype = ci
         L.granq_batch_geometry.argtypes = [ci, i64p, ci, ci, ci, ci]
         L.granq_rows_geometry.restype = ci
@@ -356,6 +358,17 @@ def rows_geometry(dtype: int, shape, channel_axis: int = 3, group: int = GROUP_C
         return None
     _check(rc, "granq_rows_geometry")
     return dict(zip(["columns", "slices", "lanes", "team"], [int(v) for v in out]))
+
+
+def forward_geometry(dtype: int, shape, channel_axis: int = 1, group: int = GROUP_CHANNEL, packed_mask: bool = False,
+                     sm_count: int = 148):
+    """Host-only: the walk of a forward with a given range by columns, or None where it takes tiles of the tensor."""
+    out = (ctypes.c_int64 * 4)()
+    rc = lib().granq_forward_geometry(dtype, _dims(shape), channel_axis, group, int(packed_mask), sm_count, out)
+    if rc == ERR_UNSUPPORTED:
+        return None
+    _check(rc, "granq_forward_geometry")
+    return dict(zip(["side", "columns", "rows", "walk"], [int(v) for v in out]))
 
 
 def hold_geometry(dtype: int, shape, channel_axis: int = 1, group: int = GROUP_CHANNEL, with_backward: bool = True,

@@ -946,6 +946,17 @@ int granq_team_geometry(int dtype, const int64_t dims[4], int channel_axis, int 
     return GRANQ_OK;
 }
 
+int granq_forward_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int packed_mask, int sm_count, int64_t out[4]) {
+    Geom g;
+    int64_t G;
+    if (!out || !dtype_ok(dtype) || sm_count < 1 || !make_geom(dims, channel_axis, group, g, G)) return GRANQ_ERR_INVALID_ARG;
+    ColsCut cut{};
+    if (!cut_cols(dtype, g, packed_mask != 0, sm_count, cut)) return GRANQ_ERR_UNSUPPORTED;
+    const int64_t v[4] = {cut.side, cut.ncol, cut.rows, cut.walk};
+    for (int i = 0; i < 4; ++i) out[i] = v[i];
+    return GRANQ_OK;
+}
+
 int granq_hold_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward, int packed, int sm_count,
                         int64_t out[4]) {
     Geom g;

@@ -694,42 +694,46 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
 }
 
 // ---- Eq. 1, clamp, Eq. 6 with a given range, column path -------------------------------------------
-// As range_cols_kernel: a thread keeps one unit column of the slabs and with it the parameters of its channel, or of the two that its
-// unit straddles, in registers, and walks a few slabs; y and, PMASK, the packed mask.  In the tile kernel above every pack of a short
+// As range_cols_kernel: a thread keeps one unit column of the slabs (of rows of several short ones) and with it the parameters of its channel, or
+// of the two that its unit straddles, in registers, and walks a few of them; y and, PMASK, the packed mask.  In the tile kernel above every pack of a short
 // or ragged plane costs a division, two table rows and a choice of parameters per element: 180 instructions a unit at [128,960,7,7] with a
 // mask, here about 50.  Tiles / columns, us, without and with a mask: fp32 [128,960,7,7] 9.6 / 7.7, 11.8 / 8.5; [128,256,14,14] 9.5 / 6.3,
-// 11.8 / 6.6; [32,64,56,56] 8.7 / 5.7, 11.1 / 6.0; [256,512,28,28], 392 MB, 122 / 122, 136 / 127; bf16 [128,96,33,33] 17.3 / 14.1, 21.0 / 16.5,
-// [256,1024,14,14] 62.6 / 49.4, 74.6 / 53.4.  Bound by the instructions of 16 bytes up to a few times the L2, then by HBM.  Eight of bf16 that
+// 11.8 / 6.6; [32,64,56,56] 8.7 / 5.7, 11.1 / 6.0; [256,512,28,28], 411 MB, 122 / 123, 134 / 127; bf16 [128,96,33,33] 17.3 / 14.1, 21.0 / 16.5,
+// [256,1024,14,14] 60.8 / 46.3, 72.3 / 52.3.  Bound by the instructions of 16 bytes up to a few times the L2, then by HBM.  Eight of bf16 that
 // straddle planes keep two units in flight and four blocks per SM (four and three: small tensors 4 to 15 % slower).
 template <typename T, bool ALIGNED, bool PMASK>
 __global__ void __launch_bounds__(kThreads, 4) quant_cols_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, uint8_t* __restrict__ pmask,
-                                                                 uint32_t slab_units, uint32_t outer, uint32_t slabs, FastDiv div_ncol,
-                                                                 FastDiv div_plane, float qmax, const float* __restrict__ lo,
-                                                                 const float* __restrict__ hi) {
+                                                                 ColsCut cut, FastDiv div_ncol, FastDiv div_plane, FastDiv div_C, float qmax,
+                                                                 const float* __restrict__ lo, const float* __restrict__ hi) {
     after_the_kernel_ahead();
     constexpr int V = Pack<T>::V, U = V == 8 && !ALIGNED ? 2 : 4, EXTRAS = PMASK ? 2 : 0;
+    const uint32_t row_units = cut.row_units;
     uint32_t chunk, col;
     div_ncol.divmod(blockIdx.x, chunk, col);
-    const uint32_t n0 = chunk * slabs, n1 = min(outer, n0 + slabs), lane = threadIdx.x & 31;
+    const uint32_t n0 = chunk * cut.walk, n1 = min(cut.rows, n0 + cut.walk), lane = threadIdx.x & 31;
     const uint32_t u = col * kThreads + threadIdx.x;
-    const bool valid = u < slab_units;                        // lanes beyond the last column walk along, for the shuffles
-    const uint4* p = x + ((size_t)n0 * slab_units + u);
+    // the rows this thread has a unit in: none beyond the last column, where lanes walk along for the shuffles, and the tensor may
+    // end inside the last row
+    const uint32_t end = u >= row_units ? n0 : n1 == cut.rows && u >= cut.last_units ? n1 - 1 : n1;
+    const uint4* p = x + ((size_t)n0 * row_units + u);
     Pack<T> px[U];
     auto fetch = [&](uint32_t n) {
 #pragma unroll
         for (int j = 0; j < U; ++j)
-            if (valid && n + j < n1) px[j].raw = ld_stream_16(p + (size_t)j * slab_units);
+            if (n + j < end) px[j].raw = ld_stream_16(p + (size_t)j * row_units);
     };
     fetch(n0);                                                // under way while the parameters are made
+    const uint32_t own = min(u, row_units - 1);
     uint32_t ch;
     int ne = V;
     if constexpr (ALIGNED) {
-        ch = div_plane.div(valid ? u : 0u);
+        ch = div_plane.div(own);
     } else {
         uint32_t rem;
-        div_plane.divmod((valid ? u : 0u) * V, ch, rem);
+        div_plane.divmod(own * V, ch, rem);
         ne = (int)min((uint32_t)V, div_plane.d - rem);
     }
+    if (cut.side > 1) ch -= div_C.div(ch) * div_C.d;          // (a unit that straddles planes lies in one slab)
     auto params = [&](uint32_t c) {
         const QParam q = make_qparam(__fadd_rn(lo[c], 0.0f), __fadd_rn(hi[c], 0.0f), qmax);
         const float r = div_is_safe(q.s, 0.0f, 0.0f) ? __frcp_rn(q.s) : 0.0f;
@@ -775,30 +779,30 @@ __global__ void __launch_bounds__(kThreads, 4) quant_cols_kernel(const uint4* __
         quantize_pack<T, false, !ALIGNED, EXTRAS, false, true>(q, q, g1, g2, ne, qmax, py, py, cb, mb, 8);
         if constexpr (PMASK) bits = mb[0];
     };
-    uint4* out = y + ((size_t)n0 * slab_units + u);
-    uint32_t at = n0 * slab_units + u;                        // of the units of the tensor
+    uint4* out = y + ((size_t)n0 * row_units + u);
+    uint32_t at = n0 * row_units + u;                        // of the units of the tensor
     for (uint32_t n = n0; n < n1; n += U) {
         if (n > n0) fetch(n);
         uint32_t bits[U];
 #pragma unroll
         for (int j = 0; j < U; ++j) {
             bits[j] = 0;
-            if (valid && n + j < n1) {
+            if (n + j < end) {
                 Pack<T> py;
                 quantize(px[j], py, bits[j]);
-                st_stream_16(out + (size_t)j * slab_units, py.raw);
-                if constexpr (PMASK && V == 8) pmask[at + j * slab_units] = (uint8_t)bits[j];
+                st_stream_16(out + (size_t)j * row_units, py.raw);
+                if constexpr (PMASK && V == 8) pmask[at + j * row_units] = (uint8_t)bits[j];
             }
         }
         if constexpr (PMASK && V == 4) {
             const uint32_t bytes = pair_up_mask<U>(bits, lane);
 #pragma unroll
             for (int j = 0; j < U; j += 2)
-                if (valid && n + j + (lane & 1u) < n1) pmask[(at + (j + (lane & 1u)) * slab_units) >> 1] = (uint8_t)(bytes >> (4 * j));
+                if (n + j + (lane & 1u) < end) pmask[(at + (j + (lane & 1u)) * row_units) >> 1] = (uint8_t)(bytes >> (4 * j));
         }
-        p += (size_t)U * slab_units;
-        out += (size_t)U * slab_units;
-        at += U * slab_units;
+        p += (size_t)U * row_units;
+        out += (size_t)U * row_units;
+        at += U * row_units;
     }
 }
 
@@ -1186,18 +1190,14 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
     };
     if constexpr (MODE == MODE_FWD) {
         // columns: slabs of whole units (with a mask whole bytes of it, and whole words in all), at least a batch of them: faster for
-        // all planes, see the kernel.  A few slabs to a block, so that blocks start in the order of memory; as many as leave a
-        // small tensor one wave of blocks.
+        // all planes, see the kernel
         const bool plain = !io.codes && !io.mask && !io.dist && !io.pcodes && io.y;
-        if (plain && (vec || ragged) && g.E < (1ll << 31) && g.C < (1ll << 30) && (g.C * g.inner) % VF == 0 && g.outer >= 8 &&
-            (!io.pmask || ((g.C * g.inner) % 8 == 0 && g.E % 32 == 0))) {
-            const uint32_t slab_units = (uint32_t)(g.C * g.inner / VF), ncol = (slab_units + kThreads - 1) / kThreads, outer = (uint32_t)g.outer;
-            const uint32_t slots = (uint32_t)sm_count() * 4;
-            const uint32_t slabs = std::min<uint32_t>(16, std::max<uint32_t>(4, (uint32_t)(((uint64_t)outer * ncol + slots - 1) / slots)));
+        ColsCut cut{};
+        if (plain && (vec || ragged) && cut_cols(VF == 4 ? 0 : 1, g, io.pmask != nullptr, (int)sms, cut)) {
             auto cols = [&](auto kern, uint32_t plane) {
-                return launch_after(sm_layout(0, (uint64_t)g.E * sizeof(T)), kern, ncol * ((outer + slabs - 1) / slabs), kThreads, 0, st,
-                                    (const uint4*)io.x, (uint4*)io.y, (uint8_t*)io.pmask, slab_units, outer, slabs, make_fastdiv(ncol),
-                                    make_fastdiv(plane), qmax, lo, hi);
+                return launch_after(sm_layout(0, (uint64_t)g.E * sizeof(T)), kern, cut.ncol * ((cut.rows + cut.walk - 1) / cut.walk), kThreads, 0, st,
+                                    (const uint4*)io.x, (uint4*)io.y, (uint8_t*)io.pmask, cut, make_fastdiv(cut.ncol), make_fastdiv(plane),
+                                    make_fastdiv((uint32_t)g.C), qmax, lo, hi);
             };
             const uint32_t plane = (uint32_t)(vec ? g.inner / VF : g.inner);
             if (io.pmask) return vec ? cols(quant_cols_kernel<T, true, true>, plane) : cols(quant_cols_kernel<T, false, true>, plane);
@@ -1319,6 +1319,31 @@ cudaError_t launch_naive(const QuantIO& io, int mode, int dtype, const Geom& g, 
     }
     if (mode == MODE_FWD) return naive_t<__nv_bfloat16, MODE_FWD>(io, g, bits, kmin, kmax, lo, hi, st, launches);
     return naive_t<__nv_bfloat16, MODE_BOTH>(io, g, bits, kmin, kmax, lo, hi, st, launches);
+}
+
+// Of a forward with a given range by columns (quant_cols_kernel).  A row is as many slabs side by side as fill the blocks across it to
+// 15/16, of 8192 units at most: with a slab to a row the lanes beyond a slab of 64 units were three of four ([65536,4,4,4] fp32
+// 22.3, by tiles 8.8, slabs side by side 7.2 us; bf16 34.7, 7.6, 7.0).  Four to sixteen rows to a block, so that blocks start in the order of
+// memory: as many as leave a small tensor one wave of blocks, and a larger one whole waves (bf16 [1178,11,40,40], a wave and an
+// eighth of 16 rows 22.2, by tiles 20.3, two waves of 9 19.2 us).
+bool cut_cols(int dtype, const Geom& g, bool packed_mask, int sms, ColsCut& cut) {
+    const int64_t V = dtype == 0 ? 4 : 8, slab = g.C * g.inner;
+    if (g.outer < 8 || g.inner < V || slab % V != 0 || g.E >= (1ll << 31) || g.C >= (1ll << 30)) return false;
+    if (packed_mask && (slab % 8 != 0 || g.E % 32 != 0)) return false;
+    const uint32_t units = (uint32_t)(slab / V), outer = (uint32_t)g.outer;
+    auto lanes = [&](uint32_t side) { return ((uint64_t)side * units + kThreads - 1) / kThreads * kThreads; };
+    cut.side = 1;
+    for (uint32_t side = 1; side <= outer && (side == 1 || (uint64_t)side * units <= 8192); ++side) {
+        if (lanes(side) * cut.side < lanes(cut.side) * side) cut.side = side;
+        if (15 * lanes(side) <= 16ull * side * units) break;
+    }
+    cut.row_units = cut.side * units;
+    cut.ncol = (cut.row_units + kThreads - 1) / kThreads;
+    cut.rows = (outer + cut.side - 1) / cut.side;
+    cut.last_units = (outer - (cut.rows - 1) * cut.side) * units;
+    const uint64_t slots = (uint64_t)sms * 4, each = ((uint64_t)cut.rows * cut.ncol + slots - 1) / slots, waves = (each + 15) / 16;
+    cut.walk = (uint32_t)std::max<uint64_t>(4, (each + waves - 1) / waves);
+    return true;
 }
 
 // With elements behind the last whole pack, scalar loads up to here: a small call ends sooner with more blocks of less each.

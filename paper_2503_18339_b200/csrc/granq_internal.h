@@ -278,6 +278,15 @@ cudaError_t launch_colwalk(const ColPlan& plan, const QuantIO& io, int mode, int
                            const Workspace& ws, float* lo, float* hi, float* s_opt, float* z_opt,
                            const StagedTuning& tune, cudaStream_t st);
 
+// forward with a given range by columns (granq_flat.cu)
+struct ColsCut {
+    uint32_t side;                   // slabs side by side in a row
+    uint32_t row_units, last_units;  // 16-byte units of a row, of the last row
+    uint32_t ncol;                   // blocks across a row
+    uint32_t rows, walk;             // rows, those a block walks
+};
+bool cut_cols(int dtype, const Geom& g, bool packed_mask, int sms, ColsCut& cut);
+
 // ---- range and quantization of a tensor held in shared memory piece by piece (granq_hold.cu) ----
 struct HoldPlan {
     bool ok;

@@ -395,3 +395,35 @@ def test_held_form_cuts_within_its_limits_and_leaves_the_waves_to_their_knobs(li
     finally:
         for k in range(b.N_KNOBS):
             b.tune(k, 0)
+
+
+def test_forward_by_columns_covers_the_tensor_and_fills_its_blocks(lib):
+    """Every 16-byte unit is walked once, by a thread that knows its channel, and the lanes of a row's blocks are units to 15 of 16
+    wherever some number of slabs side by side, up to 8192 units, makes them so."""
+    from paper_2503_18339_b200 import binding as b
+    rnd = random.Random(5)
+    shapes = [(65536, 4, 4, 4), (100000, 3, 8, 8), (60000, 1, 28, 28), (20000, 16, 2, 2), (5000, 8, 4, 8), (8, 1, 1, 4), (9, 3, 5, 5)]
+    shapes += [(rnd.choice([8, 9, 50, 333, 4001]), rnd.randint(1, 40), rnd.randint(1, 12), rnd.randint(1, 12)) for _ in range(200)]
+    seen = 0
+    for shape in shapes:
+        for dtype, v in ((b.F32, 4), (b.BF16, 8)):
+            n, c, inner = shape[0], shape[1], shape[2] * shape[3]
+            for packed in (False, True):
+                g = b.forward_geometry(dtype, shape, packed_mask=packed)
+                ok = inner >= v and c * inner % v == 0 and (not packed or (c * inner % 8 == 0 and n * c * inner % 32 == 0))
+                assert (g is not None) == ok
+                if not ok:
+                    continue
+                seen += 1
+                units, row = c * inner // v, g["side"] * (c * inner // v)
+                lanes = lambda side: -(-side * units // 256) * 256
+                assert g["columns"] * 256 == lanes(g["side"]) and 1 <= g["side"] <= n and (g["side"] == 1 or row <= 8192)
+                assert (g["rows"] - 1) * row < n * units <= g["rows"] * row and 4 <= g["walk"] <= 16
+                best = min(lanes(s) / (s * units) for s in range(1, max(1, min(n, 8192 // units)) + 1))
+                assert lanes(g["side"]) / row <= max(16 / 15, best)
+                # the thread of column u quantizes element u * v of a row, in channel (u * v // inner) % c
+                u = rnd.randrange(row)
+                at = rnd.randrange(g["rows"]) * row + u
+                if at < n * units:
+                    assert at * v // inner % c == u * v // inner % c
+    assert seen > 100

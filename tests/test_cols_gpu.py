@@ -4,6 +4,7 @@ import pytest
 
 from gpu_util import assert_parity, make_case, to_dev
 from oracle import granq_oracle as orc
+from paper_2503_18339_b200 import workloads as wl
 from test_parity_gpu import b  # noqa: F401
 from test_rounding_gpu import assert_same_string, hard_groups
 
@@ -18,6 +19,12 @@ SHAPES = [
     (11, 8, 1, 8),        # planes of one bf16 unit
     (8, 6, 3, 5),         # slabs that are no whole units: left to tiles
     (160, 1184, 5, 5),    # 16 slabs to a block, more than a wave of blocks
+    (1003, 3, 8, 8),      # several short slabs side by side in a row, the last row not full
+    (5001, 4, 4, 4),      # the same, rows of one and of several blocks
+    (2050, 8, 3, 3),      # ... with units that straddle planes
+    (333, 1, 28, 28),     # one channel
+    (70000, 1, 2, 4),     # slabs of a unit or two
+    (9, 1, 4, 4),         # fewer slabs than would fill a block
 ]
 
 
@@ -50,3 +57,21 @@ def test_ties_by_columns(b, plane, bits):
         got = b.granq_fakequant_fwd_packmask(to_dev(x), bits, to_dev(low), to_dev(high))
         assert_parity(got, ref, x.shape, 1, orc.GROUP_CHANNEL, backward=False)
         assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
+
+
+@pytest.mark.parametrize("plane", [(6, 6), (7, 7), (8, 4)], ids=["whole", "ragged", "long"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("bits", [1, 4, 8])
+def test_elements_up_to_the_largest_finite_value(b, plane, dtype, bits):
+    """Far outside the given range on both sides, up to where the quotient overflows, beside elements inside it."""
+    x = np.ascontiguousarray(np.moveaxis(hard_groups(8 * plane[0] * plane[1], bits, seed=3).reshape((16, 8) + plane), 0, 1))
+    lo, hi = orc.range_(np.clip(x, -0.8, 0.9))
+    for i, v in enumerate((3.0e38, -3.0e38, 3.3e38, -3.3e38, 1.0e20, -1.0e30)):
+        x[i, :, i % plane[0], (2 * i + 1) % plane[1]] = v
+    if dtype == "bf16":
+        x = wl.to_bf16_bits(x)
+    assert b.forward_geometry(b.BF16 if dtype == "bf16" else b.F32, x.shape, packed_mask=True) is not None
+    ref = orc.fakequant(x, bits, lo, hi, gy=x)
+    for got in (b.granq_fakequant_fwd(to_dev(x), bits, to_dev(lo), to_dev(hi)), b.granq_fakequant_fwd_packmask(to_dev(x), bits, to_dev(lo), to_dev(hi))):
+        assert_parity(got, ref, x.shape, 1, orc.GROUP_CHANNEL, backward=False)
+    assert_same_string(got.packed_mask, orc.pack_mask(ref.mask))
