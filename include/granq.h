@@ -480,8 +480,9 @@ int granq_forward_geometry(int dtype, const int64_t dims[4], int channel_axis, i
  * `packed`: for packed masks and packed codes (forward only) rather than for y and gx.
  * out = { CTAs, 16-byte units of one CTA, of those kept in shared memory (the others are read again), 1 if
  *         granq_fakequant_fused() / granq_fakequant_fused_fwd_packmask() and granq_quantize_packed_fused() take it by default }.
- * Returns GRANQ_ERR_UNSUPPORTED when the geometry does not qualify, and for what is held with a remainder: elements behind the last
- * 16-byte unit, masks and codes that end inside a 32-bit word.
+ * Returns GRANQ_ERR_UNSUPPORTED when the geometry does not qualify, and for a tensor with a remainder - elements behind the last
+ * 16-byte unit, masks and codes that end inside a 32-bit word - also where it is held: what granq_fused_plan() counts as one launch
+ * of plan 0 or 3 is.
  */
 int granq_hold_geometry(int dtype, const int64_t dims[4], int channel_axis, int group, int with_backward, int packed, int sm_count,
                         int64_t out[4]);

@@ -141,6 +141,17 @@ cudaError_t launch_held(const TeamPlan& tp, const ClusterPlan& kp, const QuantIO
 bool hold_allowed(uint32_t flags) {
     return !(flags & (GRANQ_FLAG_FORCE_TWO_PASS | GRANQ_FLAG_FORCE_L2WAVE)) && !g_tune.l2_wave_kb && !g_tune.l2_upl && !g_tune.l2_ctas_per_sm;
 }
+// Whether it pays for a tensor that leaves something behind its whole units, or whose codes end inside a 32-bit word.  A group's keys
+// come together by atomics, one per plane: two passes are faster for codes of whole packs in many short planes, and where planes
+// are groups, some hundred thousand of them.  Two passes / held, us: 5-bit codes of fp32 [3473,18,2,2] 17 / 23, [27779,18,2,4] 32 / 135, [701,150,2,4]
+// 16 / 19, [601,301,2,4] 17 / 18.5, but [415,301,2,4] 17 / 14.5, [1501,18,2,2] 15 / 14.5; bf16 [3473,18,2,4] 15 / 23, [701,150,2,4] 12 / 18, [415,301,4,4]
+// 13.7 / 14.7, [301,301,4,4] 12.3 / 12.7, but [209,301,2,4] 12 / 10; a group per plane, forward, fp32 [118,3767,3,3] 75 / 92, but [67,2133,7,7] 52 / 49;
+// bf16 [117,3761,5,5] 88 / 103, [67,2132,7,7] 39 / 48, but [83,2677,3,3] 48 / 49, from a graph 53 / 46, [71,2254,5,5] 44 / 43.
+bool remainder_held(int dtype, const Geom& g, const QuantIO& io) {
+    if (g.outer == 1) return g.C <= (dtype == GRANQ_F32 || g.E <= 5'000'000 ? 250'000 : 100'000);
+    if (!io.pcodes || g.E % (dtype == GRANQ_F32 ? 4 : 8) != 0) return true;
+    return g.outer * g.C + 110 * g.outer <= (dtype == GRANQ_F32 ? 180'000 : 88'000);
+}
 HoldPlan prefer_hold(int dtype, const Geom& g, const QuantIO& io, uint32_t flags) {
     HoldPlan none{};
     if (!hold_allowed(flags)) return none;
@@ -148,7 +159,8 @@ HoldPlan prefer_hold(int dtype, const Geom& g, const QuantIO& io, uint32_t flags
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return none;
-    return plan_hold(dtype, g, io, sms);
+    const HoldPlan p = plan_hold(dtype, g, io, sms);
+    return p.ok && !p.whole && !remainder_held(dtype, g, io) ? none : p;
 }
 
 // In place of the cluster-local plan, where every group is one plane (a group per sample and channel, or a batch of one): a cluster then

@@ -122,6 +122,31 @@ def test_elements_behind_the_last_whole_unit(b, shape, mode, dtype):
                 assert_same_string(got.packed_codes, orc.pack_codes(orc.fused(x, code_bits, group_mode=mode).codes, code_bits))
 
 
+@pytest.mark.parametrize("dtype,shape,mode,launches", [
+    ("f32", (101, 75, 27, 27), 0, 1),
+    ("bf16", (101, 75, 27, 27), 0, 1),
+    ("f32", (83, 2677, 3, 3), 1, 1),             # 222 191 groups of one plane
+    ("f32", (119, 3767, 3, 3), 1, 3),            # 448 273
+    ("bf16", (51, 1601, 7, 7), 1, 1),            # 81 651 groups, 4 M elements
+    ("bf16", (67, 2133, 7, 7), 1, 3),            # 142 911 groups, 7 M elements
+    ("f32", (1651, 18, 2, 2), 0, 1),             # plane after plane of few channels: codes by two passes
+    ("f32", (401, 31, 2, 2), 0, 1),              # ... and held
+], ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_many_groups_with_a_remainder(b, dtype, shape, mode, launches):
+    """Held or, with very many groups or codes of very many short planes, not: the same bits either way."""
+    x, _ = make_case(shape, seed=2, dtype=dtype)
+    xd = to_dev(x)
+    ref = orc.fused(x, 5, group_mode=mode)
+    plan, n = b.fused_plan(b.BF16 if dtype == "bf16" else b.F32, shape, group=mode, with_backward=False)
+    assert n == launches or plan != b.PLAN_TWO_PASS
+    ws = b.make_workspace(xd, group=mode, zeroed=True)
+    for kw in (dict(out=b.FakeQuantOut(workspace=ws), flags=b.FLAG_WORKSPACE_ZEROED), {}):
+        assert_parity(b.granq_fakequant_fused(xd, 5, group=mode, **kw), ref, shape, 1, mode, backward=False)
+        got = b.granq_quantize_packed_fused(xd, 5, group=mode, **kw)
+        assert_same_string(got.packed_codes, orc.pack_codes(ref.codes, 5))
+        assert b.workspace_status(ws) == b.OK and int(ws.view(torch.int32).abs().sum().item()) == 0
+
+
 @pytest.mark.parametrize("dtype,shape,mode,calls", [
     ("bf16", (8, 16, 8, 8), 1, ""),                      # planes of whole units, too short
     ("bf16", (8, 8, 11, 12), 1, "fs"),                   # 8448 elements in planes that are not
