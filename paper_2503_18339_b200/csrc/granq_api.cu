@@ -165,11 +165,17 @@ HoldPlan prefer_hold(int dtype, const Geom& g, const QuantIO& io, uint32_t flags
 
 // In place of the cluster-local plan, where every group is one plane (a group per sample and channel, or a batch of one): a cluster then
 // has one slab to walk, and a thread that keeps a unit column works out its parameters for a single unit; pieces of equal size have tables of
-// them.  Cluster / piece by piece, us: bf16 whose planes are not whole units, forward [64,256,3,3] 49.5 / 13.5, [8,64,7,7] 20.1 / 10.6,
-// [64,64,13,13] 15.6 / 10.4, with gradient [16,784,14,14] 16.4 / 14.5, but [8,8,7,7], 3136 elements, 6.3 / 8.5, packed mask [8,64,7,7] 22.5 / 23.7; of whole units from 8 KB a
-// plane and 2 MB on, with gradient [16,64,112,112] 31.0 / 20.8, forward 24.0 / 18.8, but [64,256,24,24] 16.0 / 18.6, [16,64,56,56] 10.6 / 11.1; with the
-// sums from 0.5 KB on, [64,64,20,20] 13.2 / 11.2, [16,64,56,56] 13.7 / 12.5, packed mask 30.7 / 26.8, but [8,3,64,64] 12.9 / 19.7.  fp32 with the sums, planes of 1.6 KB, 12 MB: [64,200,20,20] 21.6 / 16.5,
-// [32,128,28,28] 14.4 / 13.2, [50,10,112,112] 20.6 / 16.6, but [64,300,14,14] 15.4 / 16.4; without sums a third slower or more.
+// them.  Against that stand a clearing launch and a cooperative one instead of a plain launch, one after another 2 us of every call, and atomics of
+// every plane.  A wave of clusters holds 9 MB, up to where their time hardly grows and the pieces' does; a second one takes half as long
+// again.  Cluster / piece by piece, us, calls one after another:
+// bf16 whose planes are not whole units, forward [64,256,3,3] 49.0 / 13.4, [8,64,7,7] 19.5 / 10.3, [64,64,13,13] 15.4 / 10.3, with gradient [16,784,14,14]
+// 18.6 / 14.7, but [8,8,7,7], 3136 elements, 6.3 / 8.5, packed mask [8,64,7,7] 22.5 / 23.7; of many groups [79,2536,5,5] 51 / 49, [44,1408,9,9] 31 / 27, but
+// [132,4216,3,3] 63 / 99, [100,3200,5,5] 52 / 72, and beyond the wave [33,1080,15,15] 27 / 28, [31,984,19,19] 39 / 35, but [56,1764,9,9] 33 / 40, [44,1414,15,15] 40 / 46.
+// Of whole units with gradient [16,64,112,112] 36 / 25, [10,73,64,64] 13.3 / 12.4; forward [12,102,64,64], 10 MB, 15.4 / 14.4, [17,144,64,64] 23.6 / 20.1,
+// [4,40,112,112] 12.6 / 10.3, but [11,89,64,64], 8 MB, 10.7 / 12.5, [8,61,64,64] 9.4 / 10.3, [16,64,56,56] 10.6 / 11.1.
+// With the sums [22,178,16,16] 12.1 / 10.4, [16,122,32,32] 12.4 / 11.7, [12,102,64,64] 20.1 / 16.5, but [19,154,32,32], 6 MB, 13.0 / 13.9, [11,89,64,64] 13.5 / 14.5,
+// [61,480,16,16] 20.8 / 23.1; fp32 [31,242,20,20], 12 MB, 15.7 / 14.6, [40,312,20,20] 23.6 / 18.9, but [13,108,56,56], 18 MB, 16.0 / 16.5, [37,297,20,20] 16.7 / 18.5, [64,300,14,14]
+// 15.4 / 16.4; fp32 without sums a third slower or more.  From a graph the pieces are 2 us better throughout.
 // Not in a list, whose cluster-local kernels run beside one another: eight bf16 [16,256,14,14] 34 / 82, [8,16,112,112] 39 / 82.
 HoldPlan hold_over_cluster(int dtype, const Geom& g, const QuantIO& io, uint32_t flags) {
     HoldPlan none{};
@@ -177,10 +183,15 @@ HoldPlan hold_over_cluster(int dtype, const Geom& g, const QuantIO& io, uint32_t
     if ((flags & (GRANQ_FLAG_FORCE_CLUSTER | GRANQ_FLAG_FORCE_COLWALK)) || t.cl_tile_kb || t.cl_r || t.cl_threads || t.cl_load || t.cl_prefetch ||
         t.cl_kmul || t.cl_pdl || g.outer != 1 || g.C == 1)
         return none;
-    const bool sums = io.dist != nullptr;
-    const bool pays = dtype == GRANQ_BF16 ? (g.inner % 8 != 0 ? g.E >= (io.pmask || io.pcodes ? 1 << 16 : 8192)
-                                                              : sums ? g.inner >= 256 : g.inner >= 4096 && g.E >= 1 << 20)
-                                          : sums && g.inner >= 400 && g.E >= 3'000'000;
+    const bool bf16 = dtype == GRANQ_BF16, sums = io.dist != nullptr, beyond = g.E >= 4'800'000, long_planes = g.inner >= 8192;
+    bool pays;
+    if (bf16 && g.inner % 8 != 0)
+        pays = g.E >= (io.pmask || io.pcodes ? 1 << 16 : 8192) && g.C <= (g.E <= 6'000'000 ? 200'000 : 32'000);
+    else if (sums)
+        pays = g.inner >= (bf16 ? 256 : 400) && (bf16 || g.E >= 3'000'000) &&
+               (long_planes || g.E <= (bf16 ? 2'500'000 : 3'500'000) || (beyond && g.inner >= 400));
+    else
+        pays = bf16 && g.inner >= 4096 && g.E >= 1 << 20 && (io.gy || long_planes || beyond);
     return pays ? prefer_hold(dtype, g, io, flags) : none;
 }
 

@@ -159,6 +159,9 @@ def test_many_groups_with_a_remainder(b, dtype, shape, mode, launches):
     ("f32", (8, 8, 11, 13), 1, ""),
     ("f32", (60, 128, 20, 20), 1, "s"),
     ("f32", (7, 1072, 20, 20), 1, "s"),
+    ("bf16", (75, 2800, 3, 3), 1, ""),                   # 210 000 groups
+    ("bf16", (9, 72, 88, 88), 1, "fsm"),                 # beyond a wave of clusters
+    ("bf16", (33, 1080, 15, 15), 1, ""),                 # ... with 35 640 groups
 ], ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
 def test_groups_of_one_plane(b, dtype, shape, mode, calls):
     """Where the launch that holds pieces stands in for the cluster-local one: f forward and with a gradient, s sums, m packed mask
