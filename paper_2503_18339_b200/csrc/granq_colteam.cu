@@ -631,7 +631,6 @@ TeamPlan plan_colteam(int dtype, const Geom& g, const QuantIO& io, bool backward
     }
     if (best == ~0ull) return p;
     p.threads = kTThreads;
-    p.threads = kTThreads;
     p.sm_count = (uint32_t)sm_count;
     p.gy_units = backward && !p.lag ? std::min(p.tile_units, kTSmemUnits - p.tile_units) : 0u;
     p.smem_bytes = 16u * ((p.lag ? 2 : 1) * p.tile_units + p.gy_units);
@@ -707,7 +706,6 @@ cudaError_t launch_colteam(const TeamPlan& asked, const QuantIO& io, int mode, i
         const TeamTensor one{io, bits, ws, lo, hi, s_opt, z_opt};
         return launch_colteam_list(asked, &one, 1, dtype, g, tune, st);
     }
-    const TeamPlan plan = mode == MODE_FWD ? finer_cut(asked, io, dtype, g, tune) : asked;
     TArgs a{};
     a.x = io.x;
     a.gy = io.gy;
@@ -731,17 +729,23 @@ cudaError_t launch_colteam(const TeamPlan& asked, const QuantIO& io, int mode, i
     a.plane_units = (uint32_t)(g.inner / V);
     a.units = (uint32_t)((uint64_t)g.outer * a.plane_units);
     a.slab_units = (uint32_t)((uint64_t)a.C * a.plane_units);
-    a.R = plan.R;
-    a.teams = plan.teams;
-    a.tile_units = plan.tile_units;
-    a.gy_units = plan.gy_units;
     a.spin_limit = tune.spin_limit > 0 ? (uint32_t)tune.spin_limit : kTSpinLimit;
-    a.expected = plan.R + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
     a.early = ws.cleared ? 1u : 0u;
     a.div_plane = make_fastdiv(a.plane_units);
     const int extras = io.dist ? 4 : io.pmask ? 2 : io.pcodes ? 3 : 0;
-    return dtype == 0 ? t_launch_mode<float>(a, mode, extras, plan, tune, st)
-                      : t_launch_mode<__nv_bfloat16>(a, mode, extras, plan, tune, st);
+    auto go = [&](const TeamPlan& plan) -> cudaError_t {
+        a.R = plan.R;
+        a.teams = plan.teams;
+        a.tile_units = plan.tile_units;
+        a.gy_units = plan.gy_units;
+        a.expected = plan.R + (uint32_t)(tune.extra_arrivals > 0 ? tune.extra_arrivals : 0);
+        return dtype == 0 ? t_launch_mode<float>(a, mode, extras, plan, tune, st)
+                          : t_launch_mode<__nv_bfloat16>(a, mode, extras, plan, tune, st);
+    };
+    const TeamPlan plan = mode == MODE_FWD ? finer_cut(asked, io, dtype, g, tune) : asked;
+    const cudaError_t e = go(plan);
+    // where the GPU does not hold the finer cut's CTAs at once it may hold those asked for
+    return e == cudaErrorCooperativeLaunchTooLarge && plan.threads != asked.threads ? go(asked) : e;
 }
 
 }  // namespace granq

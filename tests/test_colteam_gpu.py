@@ -27,6 +27,32 @@ SHAPES = [
 SEVERAL_ROUNDS = [(8, 400, 8, 8), (13, 700, 2, 4), (33, 310, 4, 8), (64, 300, 20, 20)]
 
 
+@pytest.mark.parametrize("dtype,shape", [("f32", (8, 1500, 36, 36)), ("bf16", (16, 1500, 36, 36))],
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else v)
+def test_forward_whose_finer_cut_is_refused(b, dtype, shape):
+    """Where the GPU does not hold twice the CTAs at once the call takes the cut that was asked for, not another plan."""
+    x, _ = make_case(shape, seed=sum(shape), dtype=dtype)
+    form = b.team_geometry(b.BF16 if dtype == "bf16" else b.F32, shape, with_backward=False)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert form["taken"] == 1 and form["rounds"] >= 5
+    xd, ref = to_dev(x), orc.fused(x, 5)
+    ran = []
+    try:
+        for cap in (0, 2 * sms):         # the finer cut has 4 CTAs of 256 threads per SM, the other 2 of 512
+            b.tune(b.KNOB_TEST_COOP_CTAS, cap)
+            with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as p:
+                got = b.granq_fakequant_fused(xd, 5, flags=b.FLAG_FORCE_COLWALK)
+                torch.cuda.synchronize()
+            assert_parity(got, ref, shape, 1, orc.GROUP_CHANNEL, backward=False)
+            ran.append([e.key for e in p.key_averages() if "granq" in e.key])
+    finally:
+        b.tune(b.KNOB_TEST_COOP_CTAS, 0)
+    if not any(ran):
+        pytest.skip("the profiler shows no kernels on this machine")
+    for names, threads in zip(ran, (256, 512)):
+        assert any("colteam_kernel" in n and f", {threads}>" in n for n in names), names
+
+
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_resident_walk(b, knobs, shape, dtype):
