@@ -87,9 +87,8 @@ __device__ __forceinline__ uint64_t a_smem_desc(const void* tile) {
 __device__ __forceinline__ uint32_t a_instr_desc(uint32_t n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((uint32_t)(kABm >> 4) << 24);
 }
-// One lane of a converged warp, chosen in the way that the compiler knows to be one lane: behind a test of the thread's
-// number it wraps every tcgen05.mma in a loop over the lanes that may be there, 273 cycles each whatever its size where one
-// of 128 x 256 x 16 takes 128.
+// One lane of a converged warp: tcgen05.mma issued one after another by the lane that this chooses take 128 cycles each at
+// 128 x 256 x 16, by a lane chosen by a test of the thread's number 273, whatever their size.
 __device__ __forceinline__ bool a_elected() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
@@ -179,16 +178,7 @@ __device__ __forceinline__ uint32_t a_pair_wide(uint32_t biased0, uint32_t biase
     return *reinterpret_cast<const uint32_t*>(&d);
 }
 __device__ __forceinline__ uint32_t a_pair_bf16(uint32_t c0, uint32_t c1, bool wide) {
-    if (!wide) {
-        const uint32_t biased = c0 | (c1 << 16) | 0x43004300u, bias = 0x43004300u;
-        const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&biased),
-                                         *reinterpret_cast<const __nv_bfloat162*>(&bias));
-        return *reinterpret_cast<const uint32_t*>(&d);
-    }
-    const float f0 = __fsub_rn(__uint_as_float(0x4B000000u | c0), 8388608.0f);
-    const float f1 = __fsub_rn(__uint_as_float(0x4B000000u | c1), 8388608.0f);
-    const __nv_bfloat162 d = __floats2bfloat162_rn(f0, f1);
-    return *reinterpret_cast<const uint32_t*>(&d);
+    return wide ? a_pair_wide(c0 | 0x4B000000u, c1 | 0x4B000000u) : a_pair_narrow(c0 | (c1 << 16) | 0x43004300u);
 }
 
 // 16 bytes of an operand row: chunk `chunk` (8 bf16) of row `row` of a K-major tile with the 128-byte swizzle

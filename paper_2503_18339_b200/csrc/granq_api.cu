@@ -198,10 +198,12 @@ HoldPlan hold_over_cluster(int dtype, const Geom& g, const QuantIO& io, uint32_t
 // The workspace set to zero ahead of one cooperative launch, or of range launches.  On the device the clearing kernel, which the launch
 // behind it need not wait for to read on, is 3 us shorter than a memset (with the launch behind it, from a graph, 1.1 / 4.1), but it
 // costs the host 1.5 us more (2.4 / 0.85).  So a call whose kernels take less time than the host needs to make it, and which is not
-// being captured, takes the memset: up to `host_bound` elements, where the two cross.  Kernel / memset, us: channels-last fp32 of
-// 0.5 MB 10.8 / 9.5, 1.5 MB 10.8 / 10.5, 2 MB 11.3 / 12.3, bf16 of 0.5 MB 11.0 / 10.5, 1.5 MB 12.6 / 13.8; one group of 0.5 MB 10.9 / 9.9; range of
-// 4 MB fp32 14.3 / 13.6, ragged of 12 MB 14.8 / 16.5, of bf16 6 MB 14.7 / 16.6.
-constexpr int64_t kHostBoundHeld = 1 << 18, kHostBoundRange = 2'000'000;
+// being captured, takes the memset: up to `host_bound` elements, where the two cross for a call with everything to allocate, through the
+// binding's native calls.  Kernel / memset, us: range of 0.26 M elements 8.8 / 8.4, 1 M 8.7 / 8.4, 1.5 M 8.65 / 8.5, 2 M fp32 8.7 / 10.0; ahead of a
+// cooperative launch, fp32, channels-last of 0.12 M elements 11.5 / 10.8, 0.26 M 11.4 / 10.6, 1.5 M 11.2 / 12.4, bf16 0.5 M 12.4 / 12.7, 1 M 12.5 / 14.1, one
+// group with gradient of 0.26 M 12.6 / 12.0.  A call with its buffers at hand makes the host no match for the GPU and would be better off with
+// the kernel: range 5.6 / 7.4, 1 M 5.6 / 8.3, channels-last of 0.12 M 8.2 / 8.8, 0.26 M 8.4 / 9.6.
+constexpr int64_t kHostBoundHeld = 1 << 18, kHostBoundRange = 1'500'000;
 cudaError_t clear_workspace(Workspace& ws, const Geom& g, int64_t host_bound, cudaStream_t st) {
     if (g.E <= host_bound) {
         cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -256,7 +258,8 @@ int granq_range(const void* x, int dtype, const int64_t dims[4], int channel_axi
     if (int rc = check_workspace(workspace, workspace_bytes, G)) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     Workspace ws = carve_workspace(workspace, G);
-    // (tensors that are no whole 16-byte units keep the GPU longer than the host: [37,133,7,7] 21.9 by a memset, 19.2)
+    // (tensors that are no whole 16-byte units keep the GPU longer than the host, with everything to allocate too: [7,33,33,33] 8.8 by the
+    // kernel, 10.4 by a memset, [19,133,7,7] 12.7 / 15.4)
     cudaError_t e = clear_workspace(ws, g, g.E * (int64_t)elt_size(dtype) % 16 == 0 ? kHostBoundRange : 0, st);
     if (e == cudaSuccess)
         e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, 0, nullptr, nullptr, ws.cleared, st);
