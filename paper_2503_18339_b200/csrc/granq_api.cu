@@ -149,7 +149,7 @@ bool hold_allowed(uint32_t flags) {
 // bf16 [117,3761,5,5] 88 / 103, [67,2132,7,7] 39 / 48, but [83,2677,3,3] 48 / 49, from a graph 53 / 46, [71,2254,5,5] 44 / 43.
 bool remainder_held(int dtype, const Geom& g, const QuantIO& io) {
     if (g.outer == 1) return g.C <= (dtype == GRANQ_F32 || g.E <= 5'000'000 ? 250'000 : 100'000);
-    if (!io.pcodes || g.E % (dtype == GRANQ_F32 ? 4 : 8) != 0) return true;
+    if (!io.pcodes || g.inner % (dtype == GRANQ_F32 ? 4 : 8) != 0) return true;
     return g.outer * g.C + 110 * g.outer <= (dtype == GRANQ_F32 ? 180'000 : 88'000);
 }
 HoldPlan prefer_hold(int dtype, const Geom& g, const QuantIO& io, uint32_t flags) {
