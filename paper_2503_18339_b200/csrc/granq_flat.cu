@@ -1391,9 +1391,9 @@ cudaError_t launch_distortion(const void* x, const void* q, int dtype, int64_t E
 
 cudaError_t launch_dequant_packed(const uint32_t* pcodes, void* y, int dtype, const Geom& g, int bits,
                                   const float* s, const float* z, cudaStream_t st) {
-    // strings of 8 codes: planes of at least 8 elements, 32-byte (fp32) stores; with codes behind the last whole string from 64 K on (one by
-    // one / strings, us from a graph: fp32 [7,373,4,5], 52 K, 1.5 / 1.7, bf16 1.5 / 1.6, [165,52,3,3], 77 K, 1.5 / 1.55, 1.75 / 1.5)
-    if ((g.E % 8 == 0 || g.E >= 1 << 16) && g.E < (1ll << 31) && g.inner >= 8 && g.inner < (1ll << 30) && g.C < (1ll << 30) &&
+    // strings of 8 codes: planes of at least 8 elements, 32-byte (fp32) stores; with codes behind the last whole string from 64 K on, fp32
+    // 128 K (one by one / strings, us from a graph: [7,373,4,5], 52 K, bf16 1.5 / 1.6, fp32 1.5 / 1.7, [165,52,3,3], 77 K, 1.75 / 1.5, a group per plane fp32 1.5 / 1.75)
+    if ((g.E % 8 == 0 || g.E >= (dtype == 0 ? 1 << 17 : 1 << 16)) && g.E < (1ll << 31) && g.inner >= 8 && g.inner < (1ll << 30) && g.C < (1ll << 30) &&
         ((uintptr_t)y & (dtype == 0 ? 31 : 15)) == 0)
         return dtype == 0 ? dequant_strings<float>(pcodes, (float*)y, g, bits, s, z, st)
                           : dequant_strings<__nv_bfloat16>(pcodes, (__nv_bfloat16*)y, g, bits, s, z, st);

@@ -20,7 +20,8 @@ SHAPES = [
     ((33, 7, 2, 5), 0),          # planes of little more than a unit
     ((9, 2001, 3, 3), 0),        # more groups, and planes of a tile, than the tables hold
     ((21, 379, 7, 7), 0),
-    ((11, 111, 5, 11), 0),       # 67 155 elements: few more than decode by strings takes
+    ((11, 111, 5, 11), 0),       # 67 155 elements: few more than decode by strings takes of bf16
+    ((11, 219, 5, 11), 0),       # 132 495: ... of fp32
     ((1291, 15, 3, 3), 0),       # short planes, whose range takes packs from here on
     ((301, 33, 3, 3), 0),        # ... and scalars up to here
     ((2, 1501, 7, 7), 0),        # packs again, more groups than a block keeps
