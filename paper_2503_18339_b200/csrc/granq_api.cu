@@ -356,6 +356,7 @@ static int fused_call(const void* x, const void* gy_opt, int dtype, const int64_
     // two passes over x by ordinary launches: any geometry, any GPU
     auto two_pass = [&]() -> cudaError_t {
         cudaError_t r = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, ws.cleared, st);
+        io.behind_range = true;
         return r == cudaSuccess ? launch_quant_flat(io, mode, dtype, g, bits, min_out, max_out, st) : r;
     };
     if (hp.ok && (e = launch_hold(hp, io, mode, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st)) !=
@@ -494,6 +495,7 @@ int granq_fakequant_fused_fwd_packmask(const void* x, int dtype, const int64_t d
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {
         e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, ws.cleared, st);
+        io.behind_range = true;
         if (e == cudaSuccess) e = launch_quant_flat(io, MODE_FWD, dtype, g, bits, min_out, max_out, st);
         if (e == cudaSuccess && zeroed)
             e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);
@@ -713,6 +715,7 @@ int granq_fakequant_fused_stats(const void* x, int dtype, const int64_t dims[4],
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_opt, zp_opt, g_tune, st);
     } else {
         e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_opt, zp_opt, ws.cleared, st);
+        io.behind_range = true;
         if (e == cudaSuccess) e = launch_quant_flat(io, MODE_FWD, dtype, g, bits, min_out, max_out, st);
         if (e == cudaSuccess && zeroed)
             e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);
@@ -799,6 +802,7 @@ int granq_quantize_packed_fused(const void* x, int dtype, const int64_t dims[4],
         e = launch_colwalk(cp, io, MODE_FWD, dtype, g, bits, ws, min_out, max_out, scale_out, zp_out, g_tune, st);
     } else {
         e = launch_range(x, dtype, g, ws.kmin, ws.kmax, ws.counters, min_out, max_out, bits, scale_out, zp_out, ws.cleared, st);
+        io.behind_range = true;
         if (e == cudaSuccess) e = launch_quant_flat(io, MODE_FWD, dtype, g, bits, min_out, max_out, st);
         if (e == cudaSuccess && zeroed)
             e = cudaMemsetAsync((char*)workspace + sizeof(uint32_t), 0, ws.clear_bytes - sizeof(uint32_t), st);

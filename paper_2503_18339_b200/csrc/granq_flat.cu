@@ -1176,13 +1176,16 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
                         ((uintptr_t)io.mask % 4 == 0);
     // ... and of those, where the last pack is not whole either: all outputs but codes and masks by the byte
     const bool ragged = planes && g.E % VF == 0, end = planes && g.E % VF != 0 && (!extras || pmask_only || pack_only || dist_only);
-    // Five blocks of a table each fill an SM.  The scalar form is bound by its instructions, and its grids of up to a wave - four blocks
-    // to an SM or, backward, seven - are spread evenly only over an empty GPU: blocks that start before the kernel ahead has
-    // ended crowd on the SMs that have room first, unless two grids leave SMs free.  Alone / set up early, us: backward f32 [75,31,41,41], 477
-    // blocks, 24.8 / 31.5, of [33,41,51,51], 430, 22.8 / 20.5; fused call of bf16 [37,532,7,7], 118, 41.4 / 49.5, of [37,133,7,7], 30, 39.3 / 37.3;
-    // forward [33,41,51,51] 22.8 / 24.1, [101,75,27,27], 674, 39.3 / 38.2.
-    const int64_t sms = sm_count(), slots = sms * (MODE == MODE_BWD ? 7 : 4);
-    const bool crowded = !vec && !ragged && !end && 2 * f.ntiles > sms && f.ntiles <= slots;
+    // Five blocks of a table each fill an SM.  The scalar form is bound by its instructions, and its grids of up to a wave are spread evenly
+    // only over an empty GPU: blocks that start before the kernel ahead has ended crowd on the SMs that have room first, unless two grids
+    // leave SMs free.  Alone / set up early, us, by blocks: backward (seven to an SM) channels-last [60,30,30,75], 494, 22.7 / 28.3, bf16
+    // 24.8 / 31.8, [120,30,30,35], 461, 22.7 / 28.3, but [4001,201,1,3], 295, 16.7 / 15.3, [64,14,14,51], 79, 12.8 / 11.8; behind the range of the same call
+    // (four to an SM), whose last block ends late, both directions [4001,201,1,3] 381 / 387, bf16 [9001,50,2,2], 220, 377 / 382, codes [1916,672,2,1], 314, 222 / 227;
+    // forward with a given range 16.2 / 13.8 at 79 blocks, 24.8 / 23.4 at 494.
+    const int64_t sms = sm_count();
+    const bool scalar = !vec && !ragged && !end;
+    const bool crowded = scalar && (io.behind_range ? 2 * f.ntiles > sms && f.ntiles <= 4 * sms
+                                                    : MODE == MODE_BWD && f.ntiles > 3 * sms && f.ntiles <= 7 * sms);
     const int layout = crowded ? kAlone : sm_layout(100, (uint64_t)g.E * sizeof(T));
     auto go = [&](auto kern) {
         return launch_after(layout, kern, grid, kThreads, 0, st, (const T*)io.x, (const T*)io.gy, (T*)io.y, (T*)io.gx, io.codes, io.mask,

@@ -87,6 +87,7 @@ struct QuantIO {
     double* dist;     // optional: 4 running sums of Table 2's statistics, zero on entry (same plans)
     uint32_t* pcodes; // optional: the integer codes as a bit string, code_bits each (flat forward kernel; y may then be null)
     int code_bits;
+    bool behind_range;  // the flat kernels: the kernel ahead on the stream is this call's range
 };
 
 // Room for dynamic shared memory.  The attribute belongs to the kernel, not to the launch: every call states the same
