@@ -141,12 +141,13 @@ cudaError_t launch_held(const TeamPlan& tp, const ClusterPlan& kp, const QuantIO
 bool hold_allowed(uint32_t flags) {
     return !(flags & (GRANQ_FLAG_FORCE_TWO_PASS | GRANQ_FLAG_FORCE_L2WAVE)) && !g_tune.l2_wave_kb && !g_tune.l2_upl && !g_tune.l2_ctas_per_sm;
 }
-// Whether it pays for a tensor that leaves something behind its whole units, or whose codes end inside a 32-bit word.  A group's keys
-// come together by atomics, one per plane: two passes are faster for codes of whole packs in many short planes, and where planes
-// are groups, some hundred thousand of them.  Two passes / held, us: 5-bit codes of fp32 [3473,18,2,2] 17 / 23, [27779,18,2,4] 32 / 135, [701,150,2,4]
-// 16 / 19, [601,301,2,4] 17 / 18.5, but [415,301,2,4] 17 / 14.5, [1501,18,2,2] 15 / 14.5; bf16 [3473,18,2,4] 15 / 23, [701,150,2,4] 12 / 18, [415,301,4,4]
-// 13.7 / 14.7, [301,301,4,4] 12.3 / 12.7, but [209,301,2,4] 12 / 10; a group per plane, forward, fp32 [118,3767,3,3] 75 / 92, but [67,2133,7,7] 52 / 49;
-// bf16 [117,3761,5,5] 88 / 103, [67,2132,7,7] 39 / 48, but [83,2677,3,3] 48 / 49, from a graph 53 / 46, [71,2254,5,5] 44 / 43.
+// Whether it pays for a tensor that leaves something behind its whole units, or whose codes end inside a 32-bit word.  A group's keys come together
+// by atomics, one per plane: two passes are faster for codes of many short planes of whole packs (of planes that are none they cost more: 4-bit codes
+// of fp32 [5656,11,9,9] 39 / 33), and where planes are groups, some hundred thousand of them.  Two passes / held, us: 5-bit codes of fp32
+// [3473,18,2,2] 17 / 23, [27779,18,2,4] 32 / 135, [701,150,2,4] 16 / 19, [601,301,2,4] 17 / 18.5, but [415,301,2,4] 17 / 14.5, [1501,18,2,2] 15 /
+// 14.5; bf16 [3473,18,2,4] 15 / 23, [701,150,2,4] 12 / 18, [415,301,4,4] 13.7 / 14.7, [301,301,4,4] 12.3 / 12.7, but [209,301,2,4] 12 / 10; a group
+// per plane, forward, fp32 [118,3767,3,3] 75 / 92, but [67,2133,7,7] 52 / 49; bf16 [117,3761,5,5] 88 / 103, [67,2132,7,7] 39 / 48, but [83,2677,3,3]
+// 48 / 49, from a graph 53 / 46, [71,2254,5,5] 44 / 43.
 bool remainder_held(int dtype, const Geom& g, const QuantIO& io) {
     if (g.outer == 1) return g.C <= (dtype == GRANQ_F32 || g.E <= 5'000'000 ? 250'000 : 100'000);
     if (!io.pcodes || g.inner % (dtype == GRANQ_F32 ? 4 : 8) != 0) return true;
@@ -168,15 +169,16 @@ HoldPlan prefer_hold(int dtype, const Geom& g, const QuantIO& io, uint32_t flags
 // them.  Against that stand a clearing launch and a cooperative one instead of a plain launch, one after another 2 us of every call, and atomics of
 // every plane.  A wave of clusters holds 9 MB, up to where their time hardly grows and the pieces' does; a second one takes half as long
 // again.  Cluster / piece by piece, us, calls one after another:
-// bf16 whose planes are not whole units, forward [64,256,3,3] 49.0 / 13.4, [8,64,7,7] 19.5 / 10.3, [64,64,13,13] 15.4 / 10.3, with gradient [16,784,14,14]
-// 18.6 / 14.7, but [8,8,7,7], 3136 elements, 6.3 / 8.5, packed mask [8,64,7,7] 22.5 / 23.7; of many groups [79,2536,5,5] 51 / 49, [44,1408,9,9] 31 / 27, but
-// [132,4216,3,3] 63 / 99, [100,3200,5,5] 52 / 72, and beyond the wave [33,1080,15,15] 27 / 28, [31,984,19,19] 39 / 35, but [56,1764,9,9] 33 / 40, [44,1414,15,15] 40 / 46.
-// Of whole units with gradient [16,64,112,112] 36 / 25, [10,73,64,64] 13.3 / 12.4; forward [12,102,64,64], 10 MB, 15.4 / 14.4, [17,144,64,64] 23.6 / 20.1,
-// [4,40,112,112] 12.6 / 10.3, but [11,89,64,64], 8 MB, 10.7 / 12.5, [8,61,64,64] 9.4 / 10.3, [16,64,56,56] 10.6 / 11.1.
-// With the sums [22,178,16,16] 12.1 / 10.4, [16,122,32,32] 12.4 / 11.7, [12,102,64,64] 20.1 / 16.5, but [19,154,32,32], 6 MB, 13.0 / 13.9, [11,89,64,64] 13.5 / 14.5,
-// [61,480,16,16] 20.8 / 23.1; fp32 [31,242,20,20], 12 MB, 15.7 / 14.6, [40,312,20,20] 23.6 / 18.9, but [13,108,56,56], 18 MB, 16.0 / 16.5, [37,297,20,20] 16.7 / 18.5, [64,300,14,14]
-// 15.4 / 16.4; fp32 without sums a third slower or more.  From a graph the pieces are 2 us better throughout.
-// Not in a list, whose cluster-local kernels run beside one another: eight bf16 [16,256,14,14] 34 / 82, [8,16,112,112] 39 / 82.
+// bf16 whose planes are not whole units, forward [64,256,3,3] 49.0 / 13.4, [8,64,7,7] 19.5 / 10.3, [64,64,13,13] 15.4 / 10.3, with gradient
+// [16,784,14,14] 18.6 / 14.7, but [8,8,7,7], 3136 elements, 6.3 / 8.5, packed mask [8,64,7,7] 22.5 / 23.7; of many groups [79,2536,5,5] 51 / 49,
+// [44,1408,9,9] 31 / 27, but [132,4216,3,3] 63 / 99, [100,3200,5,5] 52 / 72, and beyond the wave [33,1080,15,15] 27 / 28, [31,984,19,19] 39 / 35, but
+// [56,1764,9,9] 33 / 40, [44,1414,15,15] 40 / 46. Of whole units with gradient [16,64,112,112] 36 / 25, [10,73,64,64] 13.3 / 12.4; forward
+// [12,102,64,64], 10 MB, 15.4 / 14.4, [17,144,64,64] 23.6 / 20.1, [4,40,112,112] 12.6 / 10.3, but [11,89,64,64], 8 MB, 10.7 / 12.5, [8,61,64,64] 9.4
+// / 10.3, [16,64,56,56] 10.6 / 11.1. With the sums [22,178,16,16] 12.1 / 10.4, [16,122,32,32] 12.4 / 11.7, [12,102,64,64] 20.1 / 16.5, but
+// [19,154,32,32], 6 MB, 13.0 / 13.9, [11,89,64,64] 13.5 / 14.5, [61,480,16,16] 20.8 / 23.1; fp32 [31,242,20,20], 12 MB, 15.7 / 14.6, [40,312,20,20]
+// 23.6 / 18.9, but [13,108,56,56], 18 MB, 16.0 / 16.5, [37,297,20,20] 16.7 / 18.5, [64,300,14,14] 15.4 / 16.4; fp32 without sums a third slower or
+// more.  From a graph the pieces are 2 us better throughout. Not in a list, whose cluster-local kernels run beside one another: eight bf16
+// [16,256,14,14] 34 / 82, [8,16,112,112] 39 / 82.
 HoldPlan hold_over_cluster(int dtype, const Geom& g, const QuantIO& io, uint32_t flags) {
     HoldPlan none{};
     const StagedTuning& t = g_tune;
@@ -200,9 +202,9 @@ HoldPlan hold_over_cluster(int dtype, const Geom& g, const QuantIO& io, uint32_t
 // costs the host 1.5 us more (2.4 / 0.85).  So a call whose kernels take less time than the host needs to make it, and which is not
 // being captured, takes the memset: up to `host_bound` elements, where the two cross for a call with everything to allocate, through the
 // binding's native calls.  Kernel / memset, us: range of 0.26 M elements 8.8 / 8.4, 1 M 8.7 / 8.4, 1.5 M 8.65 / 8.5, 2 M fp32 8.7 / 10.0; ahead of a
-// cooperative launch, fp32, channels-last of 0.12 M elements 11.5 / 10.8, 0.26 M 11.4 / 10.6, 1.5 M 11.2 / 12.4, bf16 0.5 M 12.4 / 12.7, 1 M 12.5 / 14.1, one
-// group with gradient of 0.26 M 12.6 / 12.0.  A call with its buffers at hand makes the host no match for the GPU and would be better off with
-// the kernel: range 5.6 / 7.4, 1 M 5.6 / 8.3, channels-last of 0.12 M 8.2 / 8.8, 0.26 M 8.4 / 9.6.
+// cooperative launch, fp32, channels-last of 0.12 M elements 11.5 / 10.8, 0.26 M 11.4 / 10.6, 1.5 M 11.2 / 12.4, bf16 0.5 M 12.4 / 12.7, 1 M 12.5 /
+// 14.1, one group with gradient of 0.26 M 12.6 / 12.0.  A call with its buffers at hand makes the host no match for the GPU and would be better off
+// with the kernel: range 5.6 / 7.4, 1 M 5.6 / 8.3, channels-last of 0.12 M 8.2 / 8.8, 0.26 M 8.4 / 9.6.
 constexpr int64_t kHostBoundHeld = 1 << 18, kHostBoundRange = 1'500'000;
 cudaError_t clear_workspace(Workspace& ws, const Geom& g, int64_t host_bound, cudaStream_t st) {
     if (g.E <= host_bound) {

@@ -644,10 +644,10 @@ namespace {
 // or more of several (two / four, us: fp32 [87,240,56,56], 10 / 9 rounds, 111 / 102, with sums 109 / 103, codes 123 / 120.5; [60,200,48,48], 5 / 4,
 // 51.6 / 47.3; [49,608,56,56], 13 / 12, 141 / 137; bf16 [128,96,112,112], 12 / 10, 139 / 135; but fp32 [150,60,56,56], 4 / 4, 49.9 / 53.1, codes of
 // [64,64,112,112], 8 / 8, 103.6 / 107.0, and anything of one or two rounds), and of y alone or with a packed mask in bf16 also at the same rounds in
-// teams of up to 16 CTAs: [200,300,40,40], teams of 13, 85.7 / 82.9 and 88.2 / 85.1; [87,240,56,56], 12, 63.0 / 62.1 and 67.0 / 64.5; [26,393,88,88], 10, 72.4 / 70.9 and
-// 75.0 / 73.7; [90,700,32,32], 4, 59.9 / 57.5 and 63.7 / 63.8; [256,512,28,28], 8, 87.6 / 87.6 and 93.0 / 94.1.  Larger teams wait for the last of more CTAs: [300,200,44,44],
-// 23, 101.0 / 102.4; [156,102,68,68], 28, 68.2 / 69.7 and 69.4 / 70.5; [246,99,52,52], 29, 62.4 / 64.0; [247,25,104,104], 98, packed mask 68.5 / 71.2.  The plan that
-// was asked about stays that of two CTAs per SM.
+// teams of up to 16 CTAs: [200,300,40,40], teams of 13, 85.7 / 82.9 and 88.2 / 85.1; [87,240,56,56], 12, 63.0 / 62.1 and 67.0 / 64.5; [26,393,88,88],
+// 10, 72.4 / 70.9 and 75.0 / 73.7; [90,700,32,32], 4, 59.9 / 57.5 and 63.7 / 63.8; [256,512,28,28], 8, 87.6 / 87.6 and 93.0 / 94.1.  Larger teams
+// wait for the last of more CTAs: [300,200,44,44], 23, 101.0 / 102.4; [156,102,68,68], 28, 68.2 / 69.7 and 69.4 / 70.5; [246,99,52,52], 29, 62.4 /
+// 64.0; [247,25,104,104], 98, packed mask 68.5 / 71.2.  The plan that was asked about stays that of two CTAs per SM.
 TeamPlan finer_cut(const TeamPlan& plan, const QuantIO& io, int dtype, const Geom& g, const StagedTuning& tune) {
     const uint32_t C = (uint32_t)g.C, rounds = (C + plan.teams - 1) / plan.teams;
     const uint64_t units = (uint64_t)g.outer * (uint64_t)(g.inner / (dtype == 0 ? 4 : 8));

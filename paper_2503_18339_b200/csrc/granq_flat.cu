@@ -695,10 +695,10 @@ __global__ void __launch_bounds__(kThreads, (kFlatBlocks<V, MODE, EXTRAS, PACKON
 
 // ---- Eq. 1, clamp, Eq. 6 with a given range, column path -------------------------------------------
 // As range_cols_kernel: a thread keeps one unit column of the slabs (of rows of several short ones) and with it the parameters of its channel, or
-// of the two that its unit straddles, in registers, and walks a few of them; y and, PMASK, the packed mask.  In the tile kernel above every pack of a short
-// or ragged plane costs a division, two table rows and a choice of parameters per element: 180 instructions a unit at [128,960,7,7] with a
-// mask, here about 50.  Tiles / columns, us, without and with a mask: fp32 [128,960,7,7] 9.6 / 7.7, 11.8 / 8.5; [128,256,14,14] 9.5 / 6.3,
-// 11.8 / 6.6; [32,64,56,56] 8.7 / 5.7, 11.1 / 6.0; [256,512,28,28], 411 MB, 122 / 123, 134 / 127; bf16 [128,96,33,33] 17.3 / 14.1, 21.0 / 16.5,
+// of the two that its unit straddles, in registers, and walks a few of them; y and, PMASK, the packed mask.  In the tile kernel above every pack of a
+// short or ragged plane costs a division, two table rows and a choice of parameters per element: 180 instructions a unit at [128,960,7,7] with a
+// mask, here about 50.  Tiles / columns, us, without and with a mask: fp32 [128,960,7,7] 9.6 / 7.7, 11.8 / 8.5; [128,256,14,14] 9.5 / 6.3, 11.8 /
+// 6.6; [32,64,56,56] 8.7 / 5.7, 11.1 / 6.0; [256,512,28,28], 411 MB, 122 / 123, 134 / 127; bf16 [128,96,33,33] 17.3 / 14.1, 21.0 / 16.5,
 // [256,1024,14,14] 60.8 / 46.3, 72.3 / 52.3.  Bound by the instructions of 16 bytes up to a few times the L2, then by HBM.  Eight of bf16 that
 // straddle planes keep two units in flight and four blocks per SM (four and three: small tensors 4 to 15 % slower).
 template <typename T, bool ALIGNED, bool PMASK>
@@ -1094,11 +1094,10 @@ int range_rows_ctas() {
 // vector path straddles two planes, each lane of a warp with a group of its own, two updates a pack; scalars have one update an element,
 // and wait for one another's atomics when a group's elements are many.  Scalar / packs, us: bf16 [301,33,3,3] 29 / 60, 1101 of them 58 / 61,
 // 1684 86 / 61, [301,501,3,3] 38 / 62, [1746,509,3,3] 198 / 134; planes of 15 [451,33,3,5] 31 / 41, [701,33,3,5] 45 / 40, of 25 [301,33,5,5]
-// 25 / 27, [451,33,5,5] 37 / 28, of 49 no more; fp32 [301,33,1,5] 39 / 52, [1101,33,1,5] 61 / 52, [451,33,3,3] 30 / 32, [701,33,3,3] 42 / 32, of 15 25 / 23.
-// Of a few channels the lanes of a warp share groups again: bf16 [407,5,3,3] 27 / 16, [301,9,3,3] 29 / 25, [301,13,3,3] 29 / 33; fp32 29 / 17,
-// 27 / 23, 27 / 29.
-// Of a group per plane, whose atomics meet nobody: bf16 [1001,901,3,3] 82 / 137, fp32 83 / 117, planes of 25 125 / 134 and 126 / 153, but 126 K groups
-// fp32 of 15 to 25 as fast.  Of a few thousand elements in short planes [7,5,5,5] 5.2 / 9.5, [7,61,3,5] fp32 18 / 21.
+// 25 / 27, [451,33,5,5] 37 / 28, of 49 no more; fp32 [301,33,1,5] 39 / 52, [1101,33,1,5] 61 / 52, [451,33,3,3] 30 / 32, [701,33,3,3] 42 / 32, of 15
+// 25 / 23. Of a few channels the lanes of a warp share groups again: bf16 [407,5,3,3] 27 / 16, [301,9,3,3] 29 / 25, [301,13,3,3] 29 / 33; fp32 29 /
+// 17, 27 / 23, 27 / 29. Of a group per plane, whose atomics meet nobody: bf16 [1001,901,3,3] 82 / 137, fp32 83 / 117, planes of 25 125 / 134 and 126
+// / 153, but 126 K groups fp32 of 15 to 25 as fast.  Of a few thousand elements in short planes [7,5,5,5] 5.2 / 9.5, [7,61,3,5] fp32 18 / 21.
 template <typename T>
 bool scalar_range(const Geom& g) {
     const int64_t channel = g.outer * g.inner * (int64_t)sizeof(T);      // its bytes
@@ -1179,9 +1178,9 @@ cudaError_t quant_flat_t(const QuantIO& io, const Geom& g, int bits, const float
     // Five blocks of a table each fill an SM.  The scalar form is bound by its instructions, and its grids of up to a wave are spread evenly
     // only over an empty GPU: blocks that start before the kernel ahead has ended crowd on the SMs that have room first, unless two grids
     // leave SMs free.  Alone / set up early, us, by blocks: backward (seven to an SM) channels-last [60,30,30,75], 494, 22.7 / 28.3, bf16
-    // 24.8 / 31.8, [120,30,30,35], 461, 22.7 / 28.3, but [4001,201,1,3], 295, 16.7 / 15.3, [64,14,14,51], 79, 12.8 / 11.8; behind the range of the same call
-    // (four to an SM), whose last block ends late, both directions [4001,201,1,3] 381 / 387, bf16 [9001,50,2,2], 220, 377 / 382, codes [1916,672,2,1], 314, 222 / 227;
-    // forward with a given range 16.2 / 13.8 at 79 blocks, 24.8 / 23.4 at 494.
+    // 24.8 / 31.8, [120,30,30,35], 461, 22.7 / 28.3, but [4001,201,1,3], 295, 16.7 / 15.3, [64,14,14,51], 79, 12.8 / 11.8; behind the range of the
+    // same call (four to an SM), whose last block ends late, both directions [4001,201,1,3] 381 / 387, bf16 [9001,50,2,2], 220, 377 / 382, codes
+    // [1916,672,2,1], 314, 222 / 227; forward with a given range 16.2 / 13.8 at 79 blocks, 24.8 / 23.4 at 494.
     const int64_t sms = sm_count();
     const bool scalar = !vec && !ragged && !end;
     const bool crowded = scalar && (io.behind_range ? 2 * f.ntiles > sms && f.ntiles <= 4 * sms
@@ -1395,7 +1394,8 @@ cudaError_t launch_distortion(const void* x, const void* q, int dtype, int64_t E
 cudaError_t launch_dequant_packed(const uint32_t* pcodes, void* y, int dtype, const Geom& g, int bits,
                                   const float* s, const float* z, cudaStream_t st) {
     // strings of 8 codes: planes of at least 8 elements, 32-byte (fp32) stores; with codes behind the last whole string from 64 K on, fp32
-    // 128 K (one by one / strings, us from a graph: [7,373,4,5], 52 K, bf16 1.5 / 1.6, fp32 1.5 / 1.7, [165,52,3,3], 77 K, 1.75 / 1.5, a group per plane fp32 1.5 / 1.75)
+    // 128 K (one by one / strings, us from a graph: [7,373,4,5], 52 K, bf16 1.5 / 1.6, fp32 1.5 / 1.7, [165,52,3,3], 77 K, 1.75 / 1.5, a group per
+    // plane fp32 1.5 / 1.75)
     if ((g.E % 8 == 0 || g.E >= (dtype == 0 ? 1 << 17 : 1 << 16)) && g.E < (1ll << 31) && g.inner >= 8 && g.inner < (1ll << 30) && g.C < (1ll << 30) &&
         ((uintptr_t)y & (dtype == 0 ? 31 : 15)) == 0)
         return dtype == 0 ? dequant_strings<float>(pcodes, (float*)y, g, bits, s, z, st)

@@ -5,6 +5,8 @@ import dataclasses
 import pytest
 import torch
 
+from gpu_util import Guarded
+
 pytestmark = pytest.mark.gpu
 
 
@@ -94,6 +96,42 @@ def test_what_was_passed_comes_back(b):
     acc, aws = b.granq_accumulate_codes(codes.packed_codes, x.shape, 4, codes.s, codes.z, w)
     again = b.granq_accumulate_codes(codes.packed_codes, x.shape, 4, codes.s, codes.z, w, y=acc, workspace=aws)
     assert again[0] is acc and again[1] is aws
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("shape,axis", [((3, 8, 5, 8), 1), ((9, 13, 7, 7), 1), ((40, 3, 4, 4), 1), ((4, 6, 6, 16), 3), ((1, 1, 1, 5), 1), ((5, 41, 27, 27), 1)])
+def test_nothing_is_written_beside_the_outputs(b, monkeypatch, dtype, shape, axis):
+    """Every output of every native call between guard bands, of the size that the binding would have made it."""
+    asked = []
+    native = b._native
+    spy = lambda name: lambda *a: asked.append(getattr(native, name)(*a)) or asked[-1]
+    monkeypatch.setattr(b, "_native", type("Spy", (), {n: staticmethod(spy(n)) for n in dir(native) if n.endswith("_call")}))
+    torch.manual_seed(sum(shape))
+    x, gy = torch.randn(shape, device="cuda").to(dtype), torch.randn(shape, device="cuda").to(dtype)
+    guard = Guarded()
+    for group in (b.GROUP_CHANNEL, b.GROUP_SAMPLE_CHANNEL, b.GROUP_TENSOR):
+        G, how = b.num_groups(shape, axis, group), dict(channel_axis=axis, group=group)
+        few = lambda: guard.empty((G,), torch.float32)
+        work = lambda: guard.empty((b.workspace_bytes(b.F32 if dtype == torch.float32 else b.BF16, shape, axis, group),), torch.uint8)
+        mask = lambda: guard.empty((b.packmask_bytes(shape) // 4,), torch.int32)
+        like = lambda: guard.empty(shape, dtype)
+        record = lambda **more: b.FakeQuantOut(lo=few(), hi=few(), s=few(), z=few(), workspace=work(), **more)
+        b.granq_fakequant_fused(x, 4, gy=gy, out=record(y=like(), gx=like()), want_params=True, **how)
+        b.granq_fakequant_fused(x, 4, out=record(y=like()), **how)
+        m = b.granq_fakequant_fused_fwd_packmask(x, 3, out=record(y=like(), packed_mask=mask()), **how).packed_mask
+        b.granq_fakequant_fused_stats(x, 5, out=record(y=like(), sums=guard.empty((4,), torch.float64)), **how)
+        lo, hi = b.granq_range(x, lo=few(), hi=few(), workspace=work(), **how)
+        b.granq_fakequant_fwd_packmask(x, 4, lo, hi, y=like(), packed_mask=mask(), **how)
+        b.granq_fakequant_bwd_packmask(gy, m, gx=like())
+        q = b.granq_quantize_packed_fused(x, 5, out=record(packed_codes=guard.empty((b.packed_codes_bytes(shape, 5) // 4,), torch.int32)), **how)
+        b.granq_dequantize_packed(q.packed_codes, shape, dtype, 5, q.s, q.z, y=like(), **how)
+        if group == b.GROUP_CHANNEL:
+            out = tuple(24 if i == axis else d for i, d in enumerate(shape))
+            b.granq_accumulate_codes(q.packed_codes, shape, 5, q.s, q.z, torch.randn(24, shape[axis], device="cuda"), channel_axis=axis,
+                                     y=guard.empty(out, torch.float32),
+                                     workspace=guard.empty((b.accumulate_workspace_bytes(shape, axis, 24),), torch.uint8))
+    assert len(asked) == 3 * 9 + 1 and all(r is not None for r in asked)
+    guard.check_and_release()
 
 
 def test_what_is_left_to_python(b, monkeypatch):
