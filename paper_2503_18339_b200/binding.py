@@ -478,7 +478,7 @@ def granq_fakequant_fused(x: torch.Tensor, bits: int, gy: torch.Tensor = None, c
     whatever is missing is allocated here.
     """
     if not (want_codes or want_mask) and _goes_native(stream):
-        r = _native.fused_call(0, x, bits, gy, channel_axis, group, out, int(bool(want_params)), flags)
+        r = _native.fused_call(0, x, bits, gy, channel_axis, group, out, 1 if want_params else 0, flags)
         if r is not None:
             return r
     if gy is not None and (gy.shape != x.shape or gy.dtype != x.dtype):
@@ -531,7 +531,7 @@ def granq_fakequant_fwd_packmask(x: torch.Tensor, bits: int, lo: torch.Tensor, h
                                  stream=None) -> FakeQuantOut:
     """Forward with a given range that also stores the STE mask at one bit per element (Section 2.1)."""
     if _goes_native(stream):
-        r = _native.fwd_packmask_call(x, bits, lo, hi, channel_axis, group, y, packed_mask, int(bool(want_params)), flags)
+        r = _native.fwd_packmask_call(x, bits, lo, hi, channel_axis, group, y, packed_mask, 1 if want_params else 0, flags)
         if r is not None:
             return r
     G = num_groups(x.shape, channel_axis, group)
@@ -619,7 +619,7 @@ def granq_fakequant_fused_fwd_packmask(x: torch.Tensor, bits: int, channel_axis:
                                        want_params: bool = False, flags: int = 0, stream=None) -> FakeQuantOut:
     """Range of x itself -> scale / zero-point -> y and the packed STE mask, in one call."""
     if _goes_native(stream):
-        r = _native.fused_call(1, x, bits, None, channel_axis, group, out, int(bool(want_params)), flags)
+        r = _native.fused_call(1, x, bits, None, channel_axis, group, out, 1 if want_params else 0, flags)
         if r is not None:
             return r
     G = num_groups(x.shape, channel_axis, group)
@@ -669,7 +669,7 @@ def granq_fakequant_fused_stats(x: torch.Tensor, bits: int, channel_axis: int = 
                                 stream=None) -> FakeQuantOut:
     """Range of x itself -> scale / zero-point -> y, gathering Table 2's sums in the same pass."""
     if _goes_native(stream):
-        r = _native.fused_call(2, x, bits, None, channel_axis, group, out, int(bool(want_params)), flags)
+        r = _native.fused_call(2, x, bits, None, channel_axis, group, out, 1 if want_params else 0, flags)
         if r is not None:
             return r
     G = num_groups(x.shape, channel_axis, group)
