@@ -31,7 +31,8 @@ constexpr uint32_t kHWarps = kHThreads / 32;
 constexpr uint32_t kHSpinLimit = 1u << 24;              // bounded wait for the grid (x ~32 ns)
 constexpr uint32_t kHStatusTimeout = 5;                 // GRANQ_ERR_TIMEOUT
 constexpr uint32_t kHSmemBytes = 111u * 1024;           // two CTAs per SM
-constexpr uint32_t kHFetchUnits = 1024;                 // gy of a kept piece of 16 KB and more is sent for during the hand-over
+constexpr uint32_t kHFetchUnits = 1024;                 // gy of a kept piece of 16 KB and more is sent for during the hand-over,
+constexpr uint32_t kHFetchPlane = 256;                  // of bf16 in planes of this many elements
 constexpr uint32_t kHPlaneBytes = 2 * sizeof(uint32_t) + sizeof(GroupParam);      // keys and parameters of one plane
 
 enum : int { H_ONE = 0, H_PLANES = 1, H_RAGGED = 2 };   // one group; planes of whole units; planes that are not
@@ -207,8 +208,9 @@ __global__ void __launch_bounds__(kHThreads, 2) hold_kernel(const HArgs a) {
     // ---- the grid's hand-over (bounded) ----
     if constexpr (kBwd) {
         // what the kept piece meets is on its way to the L2 while the grid waits for its last CTA (half of it gives half as much); a
-        // smaller one is most often still there ([20,75,27,27] fp32 10.1 -> 10.5)
-        if (tid == 0 && held >= kHFetchUnits) prefetch_l2(gyg, held * 16u);
+        // smaller one is most often still there ([20,75,27,27] fp32 10.1 -> 10.5), and CTAs that fold short planes of bf16 leave memory no idle
+        // time to use ([789,75,13,13] 31.3 -> 32.2, [5333,75,5,5] 81.2 -> 81.8, of 17 x 17 on 38.6 -> 37.5; fp32 [1361,75,7,7] 36.4 -> 34.0)
+        if (tid == 0 && held >= kHFetchUnits && (V == 4 || a.inner >= kHFetchPlane)) prefetch_l2(gyg, held * 16u);
     }
     __threadfence();
     __syncthreads();
